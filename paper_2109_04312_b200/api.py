@@ -1,4 +1,5 @@
-"""ctypes binding of libmate.so (same names as the C entry points; marshalling only)."""
+"""Binding of libmate.so (same names as the C entry points; marshalling only): ctypes for what is called
+once per plan, a native module (csrc/binding.cpp) for what is called once per layer."""
 import ctypes as C
 import os
 
@@ -74,6 +75,12 @@ def _load():
     lib.mate_cell_mean.argtypes = [vp, vp, vp, vp, vp, vp]
     lib.mate_attn_bwd_noalloc.restype = i32
     lib.mate_attn_bwd_noalloc.argtypes = [vp, vp, vp, vp, vp, vp, vp, i32, i32, f32, vp, vp, vp, vp]
+    try:
+        from . import _native
+    except ImportError as e:
+        raise ImportError("the native binding is not built: run `python -m paper_2109_04312_b200.build`") from e
+    _native.bind(*(C.cast(f, C.c_void_p).value for f in (lib.mate_attn_workspace_bytes, lib.mate_attn_fwd,
+                                                         lib.mate_attn_bwd, lib.mate_cell_mean)), MateError)
     _lib = lib
     return lib
 
@@ -111,13 +118,17 @@ def _dev(t, name):
 class Plan:
     """Owner of a mate_plan_t*: the pre-computed per-view order (see mate_plan)."""
 
-    def __init__(self, handle, B, N, P, H, max_row_id, max_col_id, device):
+    def __init__(self, handle, B, N, P, H, max_row_id, max_col_id, device, T=None):
         self._h = handle
         self.B, self.N, self.P, self.H = B, N, P, H
         self.max_id = (max_row_id, max_col_id)
         self.device = device
-        self.T = None          # packed plans: total number of tokens (tensors are [H, T, d])
-        self._ws = {}
+        self.T = T             # packed plans: total number of tokens (tensors are [H, T, d])
+        from . import _native
+        self._native = _native
+        # what the native calls need of the plan, and the workspaces they keep for it
+        self._info = _native.plan_info(handle.value, B, N, H, -1 if T is None else T, max_row_id + 1, max_col_id + 1,
+                                       device.index if device.index is not None else torch.cuda.current_device())
 
     def _split(self, Q):
         """Checks a tensor's shape against the plan; returns (d, shape of the row statistic)."""
@@ -152,7 +163,8 @@ class Plan:
 
     def destroy(self):
         if self._h is not None:
-            _load().mate_plan_destroy(self._h)
+            self._native.drop(self._info)
+            _lib.mate_plan_destroy(self._h)
             self._h = None
 
     def __del__(self):
@@ -190,9 +202,8 @@ def mate_plan_packed(row_ids, col_ids, cu_seqlens, prefix_lens, head_view, max_r
                                         pf.ctypes.data, hv.ctypes.data, int(hv.shape[0]), int(max_row_id),
                                         int(max_col_id), _stream(), C.byref(handle)), "mate_plan_packed")
     n_max = max(int(np.diff(cu).max()), 1)
-    plan = Plan(handle, B, n_max, pf.tolist(), int(hv.shape[0]), int(max_row_id), int(max_col_id), row_ids.device)
-    plan.T = int(cu[-1])
-    return plan
+    return Plan(handle, B, n_max, pf.tolist(), int(hv.shape[0]), int(max_row_id), int(max_col_id), row_ids.device,
+                T=int(cu[-1]))
 
 
 def mate_plan_varlen(row_ids, col_ids, prefix_lens, head_view, radius=0, max_row_id=None, max_col_id=None) -> Plan:
@@ -279,79 +290,24 @@ def mate_attn_workspace_bytes(plan, d, dtype, impl=IMPL_AUTO):
     return f.value, b.value
 
 
-def _workspace(plan, nbytes, key):
-    if nbytes == 0:
-        return None
-    ws = plan._ws.get(key)
-    if ws is None or ws.numel() < nbytes:
-        ws = torch.empty(nbytes, dtype=torch.uint8, device=plan.device)
-        plan._ws[key] = ws
-    return ws
-
-
 def mate_attn_fwd(plan, Q, K, V, scale=None, impl=IMPL_AUTO, out=None, lse=None, workspace=None):
     """Q, K, V: [B, H, N, d] CUDA tensors (bf16 or f32), or [H, T, d] for a packed plan.  Returns (O, LSE)
     in original token order."""
-    d, stat_shape = plan._split(Q)
-    if K.shape != Q.shape or V.shape != Q.shape:
-        raise ValueError("tensor shapes do not match the plan")
-    dt = _dtype_code(Q)
-    if scale is None:
-        scale = 1.0 / float(d) ** 0.5
-    O = torch.empty_like(Q) if out is None else out
-    LSE = torch.empty(stat_shape, dtype=torch.float32, device=Q.device) if lse is None else lse
-    need, _ = mate_attn_workspace_bytes(plan, d, dt, impl)
-    ws = workspace if workspace is not None else _workspace(plan, need, "fwd")
-    with torch.cuda.device(Q.device):
-        _check(_load().mate_attn_fwd(plan._h, _dev(Q, "Q"), _dev(K, "K"), _dev(V, "V"), d, dt,
-                                     float(scale), _dev(O, "O"), _dev(LSE, "LSE"),
-                                     C.c_void_p(ws.data_ptr()) if ws is not None else None,
-                                     ws.numel() if ws is not None else 0, impl, _stream()),
-               "mate_attn_fwd")
-    return O, LSE
+    return plan._native.attn_fwd(plan._info, Q, K, V, scale, impl, out, lse, workspace)
 
 
 def mate_attn_bwd(plan, Q, K, V, O, LSE, dO, scale=None, impl=IMPL_AUTO, workspace=None):
     """Returns (dQ, dK, dV)."""
-    d, _ = plan._split(Q)
-    for t in (K, V, O, dO):
-        if t.shape != Q.shape or t.dtype != Q.dtype:
-            raise ValueError("K, V, O, dO must match Q in shape and dtype")
-    dt = _dtype_code(Q)
-    if scale is None:
-        scale = 1.0 / float(d) ** 0.5
-    dQ, dK, dV = torch.empty_like(Q), torch.empty_like(Q), torch.empty_like(Q)
-    _, need = mate_attn_workspace_bytes(plan, d, dt, impl)
-    ws = workspace if workspace is not None else _workspace(plan, need, "bwd")
-    with torch.cuda.device(Q.device):
-        _check(_load().mate_attn_bwd(plan._h, _dev(Q, "Q"), _dev(K, "K"), _dev(V, "V"), _dev(O, "O"),
-                                     _dev(LSE, "LSE"), _dev(dO, "dO"), d, dt, float(scale),
-                                     _dev(dQ, "dQ"), _dev(dK, "dK"), _dev(dV, "dV"),
-                                     C.c_void_p(ws.data_ptr()) if ws is not None else None,
-                                     ws.numel() if ws is not None else 0, impl, _stream()),
-               "mate_attn_bwd")
-    return dQ, dK, dV
+    return plan._native.attn_bwd(plan._info, Q, K, V, O, LSE, dO, scale, impl, workspace)
 
 
 def mate_cell_mean(plan, logits, col_ids, want_count=True, out=None):
     """Mean of the token logits per table cell (see mate_cell_mean in mate.h).  logits: float32 [B, N];
     col_ids: the int32 [B, N] tensor the plan was made from.  Returns (mean, count) of shape
-    [B, max_row_id + 1, max_col_id + 1] (count is None when not wanted)."""
-    if logits.dtype != torch.float32 or tuple(logits.shape) != (plan.B, plan.N):
-        raise ValueError("logits must be a float32 [B, N] tensor")
-    if col_ids.dtype != torch.int32 or tuple(col_ids.shape) != (plan.B, plan.N):
-        raise ValueError("col_ids must be the int32 [B, N] tensor given to mate_plan")
-    shape = (plan.B, plan.max_id[0] + 1, plan.max_id[1] + 1)
-    if out is not None:  # (mean, count) tensors of an earlier call, written in place
-        mean, count = out
-        want_count = count is not None
-    else:
-        mean = torch.empty(shape, dtype=torch.float32, device=logits.device)
-        count = torch.empty(shape, dtype=torch.int32, device=logits.device) if want_count else None
-    with torch.cuda.device(logits.device):
-        _check(_load().mate_cell_mean(plan._h, _dev(logits, "logits"), _dev(col_ids, "col_ids"), _dev(mean, "mean"),
-                                      _dev(count, "count") if want_count else None, _stream()), "mate_cell_mean")
-    return mean, count
+    [B, max_row_id + 1, max_col_id + 1] (count is None when not wanted).  out: (mean, count) tensors of an
+    earlier call, written in place."""
+    mean, count = (None, None) if out is None else out
+    return plan._native.cell_mean(plan._info, logits, col_ids, want_count, mean, count)
 
 
 def mate_attn_bwd_noalloc(plan, Q, K, V, O, LSE, dO, dQ, dK, dV, scale=None):

@@ -7,6 +7,7 @@
 #include "mate_internal.h"
 
 using mate::FwdUnit;
+using mate::TileInfo;
 using mate::kTile;
 using mate::ViewPlan;
 
@@ -52,21 +53,6 @@ void carve(mate_plan_t *pl, char *base, size_t *total) {
     *total = align_up(c.off, 256);
 }
 
-// Work-list of the tensor-core forward, built on the host from the segment offsets, then spread
-// over the CTAs of a persistent kernel so that every CTA gets about the same amount of softmax
-// work (longest-processing-time-first: units by decreasing cost, each to the least loaded CTA).
-//
-// Cost model: the exponentials are the inner limit of the kernel, and a warp (32 query rows)
-// evaluates them 32 key columns at a time, so the cost of a unit is the number of (warp, 32-column
-// chunk) pairs it visits plus a constant per half for loading Q and storing O.
-constexpr int kChunk = 32;
-constexpr int kCostPerHalf = 12;
-
-struct UnitCost {
-    FwdUnit u;
-    int64_t cost;
-};
-
 // Column range of one table row (view position t) of one (example, view): its segment, clipped to the
 // three adjacent buckets when the plan is bucketed.  The same arithmetic as step 4 of the plan kernel.
 struct RowBounds {
@@ -74,8 +60,9 @@ struct RowBounds {
     int S, P, radius;  // P: length of the global block (bucket origin; no range reaches in front of it)
     int mode = mate::kBoundsOwn, group = 1;
     int seg_of(int t) const { return (int)(std::upper_bound(so, so + S, t) - so) - 1; }
-    int lo(int t) const {
-        const int id = seg_of(t);
+    int lo(int t) const { return lo(t, seg_of(t)); }
+    int hi(int t) const { return hi(t, seg_of(t)); }
+    int lo(int t, int id) const {
         int l = so[id];
         if (mode == mate::kBoundsBefore) l = so[id / group * group];
         if (mode == mate::kBoundsAfter) l = so[id + 1];
@@ -83,8 +70,7 @@ struct RowBounds {
         const int64_t bk = (t - P) / radius;
         return (int)std::max<int64_t>(std::max(l, P), P + (bk - 1) * radius);
     }
-    int hi(int t) const {
-        const int id = seg_of(t);
+    int hi(int t, int id) const {
         int h = so[id + 1];
         if (mode == mate::kBoundsBefore) h = so[id];
         if (mode == mate::kBoundsAfter) h = so[std::min((id / group + 1) * group, S - 1)];
@@ -92,148 +78,405 @@ struct RowBounds {
             const int64_t bk = (t - P) / radius;
             h = (int)std::min<int64_t>(h, P + (bk + 2) * radius);
         }
-        return std::max(h, lo(t));
+        return std::max(h, lo(t, id));
     }
 };
 
-int64_t half_cost(const FwdUnit &u, int h, const RowBounds &rb) {
-    const int rows = std::min(kTile, u.nq - h * kTile);
-    if (rows <= 0) return 0;
-    int64_t c = kCostPerHalf;
-    const int n_warps = ceil_div(rows, 32);
-    c += (int64_t)n_warps * ceil_div(std::max(u.kA_end - u.kA0, 0), kChunk);
-    if (u.kB_end > u.kB0) {
-        for (int w = 0; w < n_warps; ++w) {
-            const int t0 = u.q0 + h * kTile + w * 32;
-            const int t1 = std::min(t0 + 32, u.q0 + h * kTile + rows) - 1;
-            c += ceil_div(rb.hi(t1) - rb.lo(t0), kChunk) + 1;  // + 1: chunks are aligned to the tile, not to lo
+// ---------------------------------------------------------------------------- work-lists
+// Work-lists of the tensor-core kernels, built on the host from the segment offsets: the rows of every
+// (example, view) are cut into units (see FwdUnit), the same for all heads of the view, and the units are
+// dealt to the CTAs.
+constexpr int kChunk = 32;
+
+// Key ranges of the rows of one (example, view), by view position.
+struct RowRanges {
+    int P, nv;  // [0, P): rows of the global block; [P, nv): table rows with the keys [lo, hi) behind the block
+    std::vector<int32_t> lo, hi;
+};
+
+void fill_ranges(const mate_plan_t *pl, const std::vector<std::vector<int32_t>> &seg_off_host, int v, int b, RowRanges &rr) {
+    const int S = pl->view[v].max_id + 2;
+    const int32_t *so = seg_off_host[v].data() + (size_t)b * S;
+    const RowBounds rb{so, S, std::min(pl->global[b], pl->n_valid[b]), pl->radius, pl->bounds_mode, pl->group};
+    rr.P = rb.P;
+    rr.nv = pl->n_valid[b];
+    rr.lo.resize(rr.nv);
+    rr.hi.resize(rr.nv);
+    for (int id = 0; id + 1 < S; ++id)
+        for (int t = std::max(so[id], rb.P); t < so[id + 1]; ++t) {
+            rr.lo[t] = rb.lo(t, id);
+            rr.hi[t] = rb.hi(t, id);
         }
-    }
-    return c;
 }
 
-// Units of all (example, head) pairs.  share = 0: no unit is split (the backward's list: its work
-// items are halves of units per side, fine enough as they are).  share > 0 (a CTA's share of the
-// total cost): a prefix-row unit, whose columns are all valid positions, that costs more than 1.3
-// shares is cut along the columns into parts of about 0.75 shares, to be combined in the kernel.
-void make_units(mate_plan_t *pl, const std::vector<std::vector<int32_t>> &seg_off_host, int64_t share,
-                std::vector<UnitCost> &all, int *n_slots, size_t *ws_bytes, int64_t *total_cost) {
-    const int N = pl->N;
-    all.clear();
-    *n_slots = 0;
-    *ws_bytes = 0;
-    *total_cost = 0;
+// Estimated clocks of the forward kernel (fitted to its per-unit times): a half alone on a tile; both
+// halves on a tile together take 0.72 of the sum.  A unit costs its loads, set-up and epilogue; a part of a
+// split unit also writes its partial result and, in the end, somebody combines them.
+constexpr int kFullClk = 1800, kPartialClk = 900, kChunkClk = 350, kUnitClk = 3500, kPartClk = 3000;
+
+struct Proto {
+    FwdUnit u;
+    std::vector<int32_t> tile;  // estimated clocks of every tile
+    int64_t cost;               // of the whole unit
+};
+
+// Estimated clocks of a half on every tile of its unit (0: skipped).
+void half_tile_clks(const FwdUnit &u, int h, const RowRanges &rr, std::vector<int32_t> &clk) {
+    const int nA = u.tiles_a(), n_tiles = nA + u.tiles_b(), rows = u.rows_of(h), r0 = u.row0_of(h);
+    clk.assign(n_tiles, 0);
+    if (rows == 0) return;
+    for (int i = 0; i < n_tiles; ++i) {
+        const TileInfo t = mate::tile_info(u, i, nA);
+        int c0, c1;
+        mate::half_cols(u.lo[h], u.hi[h], t, c0, c1);
+        if (c1 <= c0) continue;
+        int chunks = ceil_div(t.w, kChunk);
+        bool full = t.w == kTile;
+        if (t.is_b) {
+            chunks = 0;
+            for (int r = 0; r < rows; r += 32) {  // the warps of the half
+                const int last = r0 + std::min(r + 32, rows) - 1;
+                const int a = std::max(rr.lo[r0 + r] - t.k0, 0), e = std::min(rr.hi[last] - t.k0, t.w);
+                chunks = std::max(chunks, e > a ? ceil_div(e, kChunk) - a / kChunk : 0);
+            }
+            full = full && rr.lo[r0 + rows - 1] <= t.k0 && rr.hi[r0] >= t.k0 + kTile;
+        }
+        clk[i] = full ? kFullClk : kPartialClk + kChunkClk * chunks;
+    }
+}
+
+void unit_cost(Proto &pr, const RowRanges &rr) {
+    std::vector<int32_t> other;
+    half_tile_clks(pr.u, 0, rr, pr.tile);
+    half_tile_clks(pr.u, 1, rr, other);
+    pr.cost = kUnitClk;
+    for (size_t i = 0; i < pr.tile.size(); ++i) {
+        pr.tile[i] = pr.tile[i] && other[i] ? (pr.tile[i] + other[i]) * 18 / 25 : std::max(pr.tile[i] + other[i], 100);
+        pr.cost += pr.tile[i];
+    }
+}
+
+// One unit of the halves [r0, r1) and [r1, r2) (the second one may be empty) of table rows.
+FwdUnit table_unit(const RowRanges &rr, int r0, int r1, int r2) {
+    FwdUnit u{};
+    u.q0 = r0;
+    u.rows = (r1 - r0) | (r2 - r1) << 16;
+    u.kA_end = rr.P;
+    u.lo[0] = rr.lo[r0];  // lo and hi do not decrease along the rows
+    u.hi[0] = rr.hi[r1 - 1];
+    u.lo[1] = r2 > r1 ? rr.lo[r1] : 0;
+    u.hi[1] = r2 > r1 ? rr.hi[r2 - 1] : 0;
+    u.kB0 = u.lo[0];
+    u.kB_end = rr.hi[r2 - 1];
+    u.tB = kTile;
+    // When the second half's keys begin at most a tile behind the first half's, tiles of that width give each
+    // half one tile of its own (short segments: the keys of a half are its own rows).
+    const int step = u.lo[1] - u.lo[0];
+    if (r2 > r1 && step > 0 && step <= kTile && u.hi[0] - u.lo[0] <= step && u.hi[1] - u.lo[1] <= step) u.tB = step;
+    u.parts = 1;
+    u.ctr = -1;
+    return u;
+}
+
+// Units of one (example, view), for any head of the view.  Padding rows are left out.  `pairs`: two halves
+// to a unit where they share most of their tiles.
+void proto_units(const RowRanges &rr, bool pairs, std::vector<FwdUnit> &proto) {
+    const int P = rr.P, nv = rr.nv;
+    proto.clear();
+    for (int q0 = 0; q0 < P;) {  // rows of the global block: every valid key
+        FwdUnit u{};
+        const int n0 = std::min(kTile, P - q0), n1 = pairs ? std::min(kTile, P - q0 - n0) : 0;
+        u.q0 = q0;
+        u.rows = n0 | n1 << 16;
+        u.kA_end = nv;
+        u.tB = kTile;
+        u.parts = 1;
+        u.ctr = -1;
+        proto.push_back(u);
+        q0 += n0 + n1;
+    }
+    // Halves of table rows: 128 rows, or fewer when ending where a segment begins saves tiles (a half that
+    // reaches into the next long segment visits the tiles of both; one that ends with a short segment needs
+    // one tile for its own keys instead of two).  Measure: tiles, and 1.5 for the half itself, per row.
+    std::vector<int> cuts(1, P);
+    const int tiles_a = ceil_div(P, kTile);
+    for (int q = P; q < nv;) {
+        int end = std::min(q + kTile, nv);
+        if (end < nv || rr.lo[end - 1] != rr.lo[q]) {
+            int cut = end;
+            while (cut > q + 1 && (cut >= nv || rr.lo[cut] == rr.lo[cut - 1])) --cut;  // the last row that begins a new range
+            const auto per_row = [&](int e) { return (3 + 2 * (tiles_a + ceil_div(rr.hi[e - 1] - rr.lo[q], kTile))) / (double)(e - q); };
+            if (cut > q + 1 && per_row(cut) < per_row(end)) end = cut;
+        }
+        cuts.push_back(end);
+        q = end;
+    }
+    for (size_t i = 0; i + 1 < cuts.size();) {
+        const int r0 = cuts[i], r1 = cuts[i + 1];
+        bool two = pairs && i + 2 < cuts.size();
+        if (two) {
+            const int r2 = cuts[i + 2];
+            const int n0 = ceil_div(rr.hi[r1 - 1] - rr.lo[r0], kTile), n1 = ceil_div(rr.hi[r2 - 1] - rr.lo[r1], kTile);
+            const int both = ceil_div(rr.hi[r2 - 1] - rr.lo[r0], kTile);
+            two = 4 * (tiles_a + both) <= 3 * (2 * tiles_a + n0 + n1) || tiles_a + both <= 4;
+        }
+        proto.push_back(table_unit(rr, r0, r1, two ? cuts[i + 2] : r1));
+        i += two ? 2 : 1;
+    }
+}
+
+// Backward: no unit is split; its work items are the halves of the units, once per side.
+void make_bwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges) {
+    std::vector<std::pair<int64_t, FwdUnit>> all;
+    std::vector<FwdUnit> proto;
+    std::vector<int32_t> clk;
     for (int v = 0; v < 2; ++v) {
-        const ViewPlan &vp = pl->view[v];
-        if (vp.n_heads == 0) continue;
-        const int S = vp.max_id + 2;
+        if (pl->view[v].n_heads == 0) continue;
         for (int b = 0; b < pl->B; ++b) {
-            const int32_t *so = seg_off_host[v].data() + (size_t)b * S;
-            const int nv = pl->n_valid[b];
-            const int P = std::min(pl->global[b], nv);  // rows and keys in front of it are global
-            const RowBounds rb{so, S, P, pl->radius, pl->bounds_mode, pl->group};
-            std::vector<UnitCost> proto;  // units of one (example, view); copied per head below
-            for (int q0 = 0; q0 < P; q0 += mate::kUnitRows) {  // prefix rows: every valid key
+            const RowRanges &rr = ranges[(size_t)v * pl->B + b];
+            proto_units(rr, true, proto);
+            for (int q0 = pl->n_valid[b]; q0 < pl->N; q0 += 2 * kTile) {  // padding rows: no key at all
                 FwdUnit u{};
                 u.q0 = q0;
-                u.nq = std::min(mate::kUnitRows, P - q0);
-                u.kA_end = nv;
-                const int n_tiles = ceil_div(nv, kTile);
-                const int64_t whole = half_cost(u, 0, rb) + half_cost(u, 1, rb);
-                int want = 1;
-                if (share > 0 && 10 * whole > 13 * share)
-                    want = (int)std::min<int64_t>(n_tiles, (4 * whole + 3 * share - 1) / (3 * share));
-                const int per = ceil_div(n_tiles, want);
-                const int n_parts = ceil_div(n_tiles, per);  // every part holds at least one tile
-                for (int part = 0; part < n_parts; ++part) {
-                    FwdUnit w = u;
-                    w.kA0 = part * per * kTile;
-                    w.kA_end = std::min(nv, (part + 1) * per * kTile);
-                    w.n_parts = n_parts;
-                    w.part = part;
-                    proto.push_back({w, 0});
-                }
+                u.rows = std::min(kTile, pl->N - q0) | std::min(kTile, std::max(pl->N - q0 - kTile, 0)) << 16;
+                u.tB = kTile;
+                proto.push_back(u);
             }
-            for (int q0 = P; q0 < nv; q0 += mate::kUnitRows) {  // table rows: prefix + own segments
-                FwdUnit u{};
-                u.q0 = q0;
-                u.nq = std::min(mate::kUnitRows, nv - q0);
-                u.kA0 = 0;
-                u.kA_end = P;
-                u.kB0 = rb.lo(q0);   // lo and hi do not decrease along the rows
-                u.kB_end = rb.hi(q0 + u.nq - 1);
+            for (FwdUnit &u : proto) {
+                int64_t cost = 0;
                 for (int h = 0; h < 2; ++h) {
-                    const int r0 = q0 + h * kTile, r1 = std::min(q0 + u.nq, r0 + kTile) - 1;
-                    if (r1 < r0) continue;
-                    u.lo[h] = rb.lo(r0);
-                    u.hi[h] = rb.hi(r1);
+                    half_tile_clks(u, h, rr, clk);
+                    for (int c : clk) cost += c;
                 }
-                u.n_parts = 1;
-                proto.push_back({u, 0});
-            }
-            for (int q0 = nv; q0 < N; q0 += mate::kUnitRows) {  // padding rows: no key at all
-                FwdUnit u{};
-                u.q0 = q0;
-                u.nq = std::min(mate::kUnitRows, N - q0);
-                u.n_parts = 1;
-                proto.push_back({u, 0});
-            }
-            for (auto &pc : proto) pc.cost = half_cost(pc.u, 0, rb) + half_cost(pc.u, 1, rb);
-            for (int h = 0; h < pl->H; ++h) {
-                if (pl->head_view[h] != v) continue;
-                int slot = -1;
-                for (UnitCost pc : proto) {
-                    pc.u.b = b;
-                    pc.u.h = h;
-                    pc.u.ctr = -1;
-                    if (pc.u.n_parts > 1) {
-                        if (pc.u.part == 0) slot = (*n_slots)++;
-                        pc.u.ctr = slot;
-                        pc.u.ws_off = (int32_t)((*ws_bytes + pc.u.part * mate::kPartialBytes) >> 10);
-                        if (pc.u.part == pc.u.n_parts - 1) *ws_bytes += pc.u.n_parts * mate::kPartialBytes;
-                    }
-                    *total_cost += pc.cost;
-                    all.push_back(pc);
+                u.b = b;
+                for (int h = 0; h < pl->H; ++h) {
+                    if (pl->head_view[h] != v) continue;
+                    u.h = h;
+                    all.push_back({cost, u});
                 }
             }
         }
     }
-    // longest first: the CTAs of the persistent kernels take work from the head of the list as they
+    // longest first: the CTAs of the persistent kernel take work from the head of the list as they
     // become free (a shared counter), so the order is the whole schedule
-    std::stable_sort(all.begin(), all.end(), [](const UnitCost &a, const UnitCost &b) { return a.cost > b.cost; });
+    std::stable_sort(all.begin(), all.end(), [](const std::pair<int64_t, FwdUnit> &a, const std::pair<int64_t, FwdUnit> &b) {
+        return a.first > b.first;
+    });
+    pl->bwd_units.clear();
+    for (const auto &uc : all) pl->bwd_units.push_back(uc.second);
+    pl->n_bwd_units = (int)pl->bwd_units.size();
+}
+
+// Tiles [i0, i1) of a unit as a unit of its own.
+FwdUnit slice_unit(const FwdUnit &u, int i0, int i1) {
+    const int nA = u.tiles_a();
+    FwdUnit w = u;
+    const int a0 = std::min(i0, nA), a1 = std::min(i1, nA), b0 = std::max(i0 - nA, 0), b1 = std::max(i1 - nA, 0);
+    w.kA0 = u.kA0 + a0 * kTile;
+    w.kA_end = a1 > a0 ? std::min(u.kA_end, u.kA0 + a1 * kTile) : w.kA0;
+    w.kB0 = u.kB0 + b0 * u.tB;
+    w.kB_end = b1 > b0 ? std::min(u.kB_end, u.kB0 + b1 * u.tB) : w.kB0;
+    return w;
+}
+
+// ---- forward schedule: which CTA does which units, decided here once
+struct Piece {
+    int unit;     // index into the instances
+    int i0, i1;   // its tiles
+    int cta;
+};
+struct Instance {
+    int proto, h;
+};
+
+// Units that cost more than `divisible` clocks may be cut between two tiles.  The others go, longest first,
+// to the CTA with the least work; the divisible ones then fill all CTAs up to a common level, one after
+// the other.  Returns the estimated time of the slowest CTA.
+int64_t balance(const std::vector<Proto> &protos, const std::vector<Instance> &inst, const std::vector<int> &order, int n_ctas,
+                int64_t divisible, std::vector<Piece> &pieces) {
+    pieces.clear();
+    std::vector<std::pair<int64_t, int>> heap;  // (load, CTA), least on top
+    const auto more = [](const std::pair<int64_t, int> &a, const std::pair<int64_t, int> &b) { return a > b; };
+    for (int c = 0; c < n_ctas; ++c) heap.push_back({0, c});
+    size_t n_div = 0;
+    int64_t div_clk = 0;
+    while (n_div < order.size() && protos[inst[order[n_div]].proto].cost > divisible) {
+        for (int c : protos[inst[order[n_div]].proto].tile) div_clk += c;
+        ++n_div;
+    }
+    for (size_t k = n_div; k < order.size(); ++k) {
+        const Proto &pr = protos[inst[order[k]].proto];
+        std::pop_heap(heap.begin(), heap.end(), more);
+        heap.back().first += pr.cost;
+        pieces.push_back({order[k], 0, (int)pr.tile.size(), heap.back().second});
+        std::push_heap(heap.begin(), heap.end(), more);
+    }
+    std::sort(heap.begin(), heap.end());
+    int64_t worst = heap.back().first;
+    if (n_div == 0) return worst;
+    // Level: the `used` least loaded CTAs take the divisible tiles, each with the cost of one more (partial)
+    // unit.  What rounding to tiles leaves over or takes too much is carried to the next CTA; every
+    // divisible unit begun inside a CTA costs one more partial unit.
+    const int64_t extra = kUnitClk + kPartClk;
+    int used = 0;
+    int64_t level = 0, sum = div_clk + (int64_t)n_div * extra;
+    for (used = 1; used <= n_ctas; ++used) {
+        sum += heap[used - 1].first + extra;
+        level = (sum + used - 1) / used;
+        if (used == n_ctas || level <= heap[used].first + extra + 2 * kFullClk) break;
+    }
+    size_t k = 0;
+    int i0 = 0;
+    int64_t carry = 0;
+    for (int c = 0; c < used && k < n_div; ++c) {
+        int64_t load = heap[c].first, room = level - load + carry;
+        const bool last = c + 1 == used;
+        while (k < n_div) {
+            const std::vector<int32_t> &tile = protos[inst[order[k]].proto].tile;
+            int64_t left = room - extra;
+            int i1 = i0;
+            while (i1 < (int)tile.size() && (last || left >= tile[i1] / 2)) left -= tile[i1++];
+            if (!last && i1 > i0 + 1 && i1 + 1 == (int)tile.size()) left += tile[--i1];  // leave no crumb
+            if (i1 == i0) break;
+            load += room - left;
+            room = left;
+            i0 = i1;
+            pieces.push_back({order[k], i1, i1, heap[c].second});
+            if (i1 < (int)tile.size()) break;
+            ++k;
+            i0 = 0;
+        }
+        carry = room;
+        worst = std::max(worst, load);
+    }
+    // pieces of divisible units carry their end only: fill in where each begins
+    int prev_unit = -1, prev_end = 0;
+    for (Piece &pc : pieces) {
+        if (protos[inst[pc.unit].proto].cost <= divisible) continue;
+        pc.i0 = pc.unit == prev_unit ? prev_end : 0;
+        prev_unit = pc.unit;
+        prev_end = pc.i1;
+    }
+    return worst;
+}
+
+void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges) {
+    const int n_ctas = std::max(pl->n_ctas, 1);
+    std::vector<Proto> protos;
+    std::vector<Instance> inst;
+    int64_t total = 0;
+    // Single halves when there are not enough pairs for half of the SMs: a CTA then works on one half only,
+    // which takes less than the time of both.
+    for (bool pairs = true;; pairs = false) {
+        protos.clear();
+        inst.clear();
+        total = 0;
+        std::vector<FwdUnit> proto;
+        for (int v = 0; v < 2; ++v) {
+            if (pl->view[v].n_heads == 0) continue;
+            for (int b = 0; b < pl->B; ++b) {
+                const RowRanges &rr = ranges[(size_t)v * pl->B + b];
+                proto_units(rr, pairs, proto);
+                for (FwdUnit &u : proto) {
+                    u.b = b;
+                    Proto pr{u, {}, 0};
+                    unit_cost(pr, rr);
+                    for (int h = 0; h < pl->H; ++h)
+                        if (pl->head_view[h] == v) inst.push_back({(int)protos.size(), h});
+                    total += pr.cost * pl->view[v].n_heads;
+                    protos.push_back(std::move(pr));
+                }
+            }
+        }
+        if (!pairs || 2 * (int)inst.size() > n_ctas) break;
+    }
+    std::vector<int> order(inst.size());
+    for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int a, int b) { return protos[inst[a].proto].cost > protos[inst[b].proto].cost; });
+    // How much is cut is decided by the estimate: nothing, units longer than a CTA's share, half of it, a quarter.
+    const int64_t share = total / n_ctas;
+    std::vector<Piece> best, pieces;
+    int64_t best_clk = -1;
+    for (const int64_t divisible : {INT64_MAX, share, share / 2, share / 4}) {
+        if (divisible < kUnitClk + 4 * kFullClk) break;
+        const int64_t clk = balance(protos, inst, order, n_ctas, divisible, pieces);
+        if (best_clk < 0 || clk < best_clk) {
+            best_clk = clk;
+            best.swap(pieces);
+        }
+    }
+    if (best_clk < 0) balance(protos, inst, order, n_ctas, INT64_MAX, best);
+
+    // records, split units with their place in the workspace; a CTA starts with its parts of split units, so
+    // that nobody waits for them in the end
+    std::vector<int> n_parts(inst.size(), 0), seen(inst.size(), 0), slot(inst.size(), -1);
+    std::vector<size_t> ws_off(inst.size(), 0);
+    for (const Piece &pc : best) ++n_parts[pc.unit];
+    size_t ws_bytes = 0;
+    pl->n_fwd_slots = 0;
+    for (size_t k = 0; k < inst.size(); ++k)
+        if (n_parts[k] > 1) {
+            slot[k] = pl->n_fwd_slots++;
+            ws_off[k] = ws_bytes;
+            ws_bytes += n_parts[k] * mate::kPartialBytes;
+        }
+    std::vector<std::vector<FwdUnit>> lists(n_ctas);
+    for (int pass = 0; pass < 2; ++pass)
+        for (const Piece &pc : best) {
+            if ((n_parts[pc.unit] > 1) != (pass == 0)) continue;
+            FwdUnit u = slice_unit(protos[inst[pc.unit].proto].u, pc.i0, pc.i1);
+            u.h = inst[pc.unit].h;
+            u.parts = n_parts[pc.unit] | seen[pc.unit]++ << 16;
+            u.ctr = slot[pc.unit];
+            u.ws_off = (int32_t)((ws_off[pc.unit] + u.part() * mate::kPartialBytes) >> 10);
+            lists[pc.cta].push_back(u);
+        }
+    pl->fwd_units.clear();
+    pl->fwd_cta_off.assign(1, 0);
+    for (int c = 0; c < n_ctas; ++c) {
+        pl->fwd_units.insert(pl->fwd_units.end(), lists[c].begin(), lists[c].end());
+        pl->fwd_cta_off.push_back((int32_t)pl->fwd_units.size());
+    }
+    pl->n_fwd_units = (int)pl->fwd_units.size();
+    pl->fwd_ws_bytes = ws_bytes;
+    // padding rows of every (example, head)
+    pl->pads.clear();
+    for (int b = 0; b < pl->B; ++b)
+        for (int t0 = pl->n_valid[b]; t0 < pl->N; t0 += mate::kPadRows)
+            for (int h = 0; h < pl->H; ++h) pl->pads.push_back({b, h, t0, std::min(mate::kPadRows, pl->N - t0)});
+    pl->n_pads = (int)pl->pads.size();
+    // CTAs without units are not launched (the list is filled from CTA 0 on only when there are fewer units
+    // than CTAs), unless there is padding to be spread
+    int grid = n_ctas;
+    if (pl->n_fwd_units < n_ctas) {
+        grid = std::min(n_ctas, std::max(pl->n_fwd_units, pl->n_pads));
+        for (int c = grid; c < n_ctas; ++c)
+            if (pl->fwd_cta_off[c + 1] > pl->fwd_cta_off[c]) grid = c + 1;
+    }
+    pl->fwd_grid = grid;
+    if (getenv("MATE_LOG"))
+        fprintf(stderr, "[mate] forward: %d units (%d of %d split), %d CTAs, estimated clocks: mean %lld, slowest %lld; "
+                        "workspace %zu bytes; %d chunks of padding\n",
+                pl->n_fwd_units, pl->n_fwd_slots, (int)inst.size(), pl->fwd_grid, (long long)share, (long long)best_clk,
+                pl->fwd_ws_bytes, pl->n_pads);
 }
 
 int build_units(mate_plan_t *pl, const std::vector<std::vector<int32_t>> &seg_off_host) {
     static_assert(mate::kPartialBytes % 1024 == 0, "ws_off counts KiB");
-    const int n_ctas = std::max(pl->n_ctas, 1);
-    std::vector<UnitCost> all;
-    int n_slots = 0;
-    size_t ws_bytes = 0;
-    int64_t total_cost = 0;
-    // backward: unsplit list; its total cost also gives the share of a CTA
-    make_units(pl, seg_off_host, 0, all, &n_slots, &ws_bytes, &total_cost);
-    pl->bwd_units.clear();
-    for (const UnitCost &uc : all) pl->bwd_units.push_back(uc.u);
-    pl->n_bwd_units = (int)pl->bwd_units.size();
-    // forward: long prefix units split; the forward kernel runs several CTAs per SM
-    const int64_t share = std::max<int64_t>(total_cost / ((int64_t)n_ctas * mate::tc_fwd_ctas_per_sm()), 1);
-    make_units(pl, seg_off_host, share, all, &n_slots, &ws_bytes, &total_cost);
-    pl->fwd_units.clear();
-    for (const UnitCost &uc : all) pl->fwd_units.push_back(uc.u);
-    pl->n_fwd_units = (int)pl->fwd_units.size();
-    pl->n_fwd_slots = n_slots;
-    pl->fwd_ws_bytes = ws_bytes;
-    if (getenv("MATE_LOG"))
-        fprintf(stderr, "[mate] work-lists: forward %d units (%d split), backward %d units, %d CTAs, cost total %lld "
-                        "(%.1f per CTA, largest forward unit %lld), forward workspace %zu bytes\n",
-                pl->n_fwd_units, pl->n_fwd_slots, pl->n_bwd_units, n_ctas, (long long)total_cost,
-                (double)total_cost / n_ctas, all.empty() ? 0ll : (long long)all.front().cost, pl->fwd_ws_bytes);
+    std::vector<RowRanges> ranges((size_t)2 * pl->B);
+    for (int v = 0; v < 2; ++v)
+        for (int b = 0; b < pl->B && pl->view[v].n_heads > 0; ++b) fill_ranges(pl, seg_off_host, v, b, ranges[(size_t)v * pl->B + b]);
+    make_bwd_units(pl, ranges);
+    make_fwd_units(pl, ranges);
 
-    // device copy: units, CTA offsets, arrival counters (zeroed once; the kernel resets them)
+    // device copy: units, CTA offsets, padding, arrival counters (zeroed once; the kernel resets them)
     Carver c(nullptr);
     c.take<FwdUnit>(pl->n_fwd_units);
     c.take<FwdUnit>(pl->n_bwd_units);
-    c.take<int32_t>(mate::kSchedWords + 8 * (size_t)pl->n_fwd_slots);
+    c.take<int32_t>(pl->fwd_cta_off.size());
+    c.take<mate::PadChunk>(pl->n_pads);
+    c.take<int32_t>(8 * (size_t)pl->n_fwd_slots);
     const size_t bytes = align_up(c.off, 256);
     if (cudaMalloc(&pl->work_block, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -242,7 +485,9 @@ int build_units(mate_plan_t *pl, const std::vector<std::vector<int32_t>> &seg_of
     Carver d((char *)pl->work_block);
     pl->fwd_units_dev = d.take<FwdUnit>(pl->n_fwd_units);
     pl->bwd_units_dev = d.take<FwdUnit>(pl->n_bwd_units);
-    pl->fwd_counters_dev = d.take<int32_t>(mate::kSchedWords + 8 * (size_t)pl->n_fwd_slots);
+    pl->fwd_cta_off_dev = d.take<int32_t>(pl->fwd_cta_off.size());
+    pl->pads_dev = d.take<mate::PadChunk>(pl->n_pads);
+    pl->fwd_counters_dev = d.take<int32_t>(8 * (size_t)pl->n_fwd_slots);
     return MATE_OK;
 }
 
@@ -507,8 +752,13 @@ static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int
         mate_plan_destroy(pl);
         return rc;
     }
-    bool up = cudaMemsetAsync(pl->fwd_counters_dev, 0,
-                              sizeof(int32_t) * (mate::kSchedWords + 8 * (size_t)pl->n_fwd_slots), st) == cudaSuccess;
+    bool up = cudaMemcpyAsync(pl->fwd_cta_off_dev, pl->fwd_cta_off.data(), sizeof(int32_t) * pl->fwd_cta_off.size(),
+                              cudaMemcpyHostToDevice, st) == cudaSuccess;
+    if (pl->n_fwd_slots > 0)
+        up = up && cudaMemsetAsync(pl->fwd_counters_dev, 0, sizeof(int32_t) * 8 * (size_t)pl->n_fwd_slots, st) == cudaSuccess;
+    if (pl->n_pads > 0)
+        up = up && cudaMemcpyAsync(pl->pads_dev, pl->pads.data(), sizeof(mate::PadChunk) * pl->n_pads, cudaMemcpyHostToDevice,
+                                   st) == cudaSuccess;
     if (pl->n_fwd_units > 0)
         up = up && cudaMemcpyAsync(pl->fwd_units_dev, pl->fwd_units.data(), sizeof(FwdUnit) * pl->n_fwd_units,
                                    cudaMemcpyHostToDevice, st) == cudaSuccess;
@@ -567,9 +817,8 @@ int mate_plan_status(const mate_plan_t *plan, void *stream) {
         if (getenv("MATE_LOG"))
             fprintf(stderr, "[mate] a bounded wait expired: barrier slot %d, parity %d, warp %d\n", (s[2] >> 8) & 0xff,
                     (s[2] >> 7) & 1, s[2] & 0x7f);
-        // a kernel that gave up may have left the scheduling and arrival counters half way
-        if (cudaMemsetAsync(plan->fwd_counters_dev, 0,
-                            sizeof(int32_t) * (mate::kSchedWords + 8 * (size_t)plan->n_fwd_slots), st) != cudaSuccess ||
+        // a kernel that gave up may have left the arrival counters half way
+        if (cudaMemsetAsync(plan->fwd_counters_dev, 0, sizeof(int32_t) * 8 * (size_t)plan->n_fwd_slots, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
             return MATE_ERR_CUDA;
         return MATE_ERR_TIMEOUT;

@@ -94,39 +94,6 @@ struct Params {
     int32_t *counter;      // next work item (zeroed before the launch)
 };
 
-struct TileInfo {
-    int k0, w;
-    bool is_b;
-};
-__device__ __forceinline__ int n_tiles_a(const FwdUnit &u) {
-    return u.kA_end > u.kA0 ? (u.kA_end - u.kA0 + kTile - 1) / kTile : 0;
-}
-__device__ __forceinline__ int n_tiles_b(const FwdUnit &u) {
-    return u.kB_end > u.kB0 ? (u.kB_end - u.kB0 + kTile - 1) / kTile : 0;
-}
-__device__ __forceinline__ TileInfo tile_info(const FwdUnit &u, int i, int nA) {
-    TileInfo t;
-    if (i < nA) {
-        t.k0 = u.kA0 + i * kTile;
-        t.w = min(kTile, u.kA_end - t.k0);
-        t.is_b = false;
-    } else {
-        t.k0 = u.kB0 + (i - nA) * kTile;
-        t.w = min(kTile, u.kB_end - t.k0);
-        t.is_b = true;
-    }
-    return t;
-}
-// Columns [c0, c1) of the tile (multiples of 16) needed by a half whose rows' segments span keys [lo, hi).
-__device__ __forceinline__ void half_cols(int lo, int hi, const TileInfo &t, int &c0, int &c1) {
-    if (!t.is_b) {
-        c0 = 0;
-        c1 = (t.w + 15) & ~15;
-    } else {
-        c0 = (max(lo, t.k0) - t.k0) & ~15;
-        c1 = (min(hi, t.k0 + t.w) - t.k0 + 15) & ~15;
-    }
-}
 __device__ __forceinline__ FwdUnit load_unit(const FwdUnit *p) {
     FwdUnit u;
     const int4 *s = reinterpret_cast<const int4 *>(p);
@@ -212,10 +179,10 @@ __device__ __forceinline__ Item make_item(const Params &p, int it) {
     x.un = load_unit(p.units + (it >> 2));
     x.h = it & 1;
     x.key_side = (it & 2) != 0;
-    x.nA = n_tiles_a(x.un);
-    x.n_tiles = x.nA + n_tiles_b(x.un);
-    x.rows_h = max(0, min(kTile, x.un.nq - x.h * kTile));
-    x.row0 = x.un.q0 + x.h * kTile;
+    x.nA = x.un.tiles_a();
+    x.n_tiles = x.nA + x.un.tiles_b();
+    x.rows_h = x.un.rows_of(x.h);
+    x.row0 = x.un.row0_of(x.h);
     x.lo = x.h ? x.un.lo[1] : x.un.lo[0];
     x.hi = x.h ? x.un.hi[1] : x.un.hi[0];
     return x;

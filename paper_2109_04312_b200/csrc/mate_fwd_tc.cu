@@ -1,29 +1,43 @@
 // Tensor-core forward of multi-view attention (head formula and pattern of Section 3) for bf16,
-// d = 64, on sm_100a.  One persistent, warp-specialised CTA per SM walks the units that
-// mate_plan assigned to it (see FwdUnit): 256 query rows of one (example, head) in the head's view
+// d = 64, on sm_100a.  One persistent, warp-specialised CTA per SM walks its list of units, which
+// mate_plan balanced over the CTAs (see FwdUnit): 256 query rows of one (example, head) in the head's view
 // order (Section 3.1: per-head traversal order) against the key tiles those rows may attend.
 //
 //   warps 0-3   softmax of half 0 (query rows 0..127 of the unit), one thread per row
 //   warps 4-7   softmax of half 1 (rows 128..255)
-//   warps 8, 9  one thread each issues the tcgen05.mma of half 0 / half 1
-//   warps 10-11 loaders: gather Q, K, V rows by view-order index into 128-byte swizzled shared
+//   warps 8, 9  issue the tcgen05.mma of half 0 / half 1 (one elected lane each)
+//   warps 10,11 padding rows
+//   warps 12-15 loaders: gather Q, K, V rows by view-order index into 128-byte swizzled shared
 //               memory with 16-byte cp.async (the gather of Section 3.1 fused into the loads); K/V
 //               tiles whose rows lie in place in the tensors come in by one bulk tensor copy each
 //
 // Per key tile and half:   S = Q K^T  (tcgen05.mma, M = 128, N <= 128, K = 64, accumulator in TMEM)
-//                          online softmax in the exp2 domain: P = exp2(S c - m), row sum.  P is
-//                          formed in one pass over S with the running max m (for a unit's first
-//                          tile: the max over its first 32 columns); the tile's own max is tracked
-//                          on the way and only a growth by more than 2^8 sends the tile through
-//                          the two-pass path (max, rescale O, exp)
+//                          P = exp2(S c - m), row sum
 //                          O += P V   (tcgen05.mma, M = 128, N = 64, P read from TMEM; O stays there)
-// S is released to the MMA issuer as soon as its last 32 columns sit in registers, so the Q K^T of
-// the half's next tile runs under the rest of the exponentials.
-// The two halves share every K/V tile and alternate on the tensor pipe, so the exponentials of
-// one half overlap the MMAs of the other.  Key tiles of range B are visited by a half only where
-// they meet the segments of its rows, and inside a tile a warp evaluates only the 32-column chunks
-// that meet the segments of its 32 rows.  The scatter back to the original token order is fused
-// into the epilogue (each thread stores its 128-byte row at the row's original position).
+//
+// The base m of a row.  The largest score of a row's first tile serves for the whole unit: powers of two
+// cost no precision (P is bf16 with fp32's exponent range, O and the row sum are fp32), so a later score may
+// exceed it by up to 2^60.  That is read off the row sum when the unit is done: a row whose sum has
+// left [2^-100, 2^60] sends the unit through once more, with the running max of online softmax (`exact`).
+// The common case therefore has no max, no rescaling and no wait between the scores and the exponentials.
+//
+// What bounds it: the exponentials (16 per clock and SM: 1024 clk per 128 x 128 half tile, against 512 clk
+// of tensor pipe), as far as everything else hides behind them.
+//   - A thread takes its whole row of S (128 columns) into registers in one go (setmaxnreg) and gives S
+//     back at once, so the Q K^T of the half's next tile runs under all of this tile's arithmetic.
+//   - On a scheduler one warp of each half shares the exponential unit.  Left alone the two fall into step
+//     and it idles through every wait and load; kept half a tile apart one half's loads run under the
+//     other's exponentials (a fifth faster on long rows of full tiles).  See s_stamp.
+//   - Two threads per row (four warps per scheduler) hide the latencies as well, but the control flow of twice
+//     the warps takes more issue slots than that gains.
+//   - The instruction cache is about 32 KB for all roles of the CTA; straight-line code that misses it issues
+//     at a third of the rate, from L2 at a sixth.  Rarely taken paths are rolled.
+// Key tiles of range B are visited by a half only where they meet the segments of its rows, and inside
+// a tile a warp evaluates only the 32-column chunks that meet the segments of its 32 rows.  The scatter
+// back to the original token order is fused into the epilogue.
+//
+// The unit's record and what the softmax threads need of its rows (original position, key range) travel
+// through shared memory with the unit's Q, so no role waits for global memory between two units.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -41,20 +55,30 @@ namespace {
 using namespace ptx;
 
 constexpr int kSoftmaxWarps = 8;
-constexpr int kMmaWarp = 8;   // warps 8 and 9: one MMA-issuing thread per half
+constexpr int kMmaWarp = kSoftmaxWarps;   // one MMA-issuing warp per half
 constexpr int kMmaWarps = 2;
-constexpr int kLoadWarp0 = 10;
-constexpr int kLoadWarps = 2;
+constexpr int kPadWarp0 = kMmaWarp + kMmaWarps;
+constexpr int kPadWarps = 2;
+constexpr int kLoadWarp0 = kPadWarp0 + kPadWarps;
+constexpr int kLoadWarps = 4;                // (two keep the softmax warps waiting on gathered tiles)
 constexpr int kLoadThreads = 32 * kLoadWarps;
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
-constexpr int kStages = 5;                   // K/V ring
+constexpr int kStages = 4;                   // K/V ring
 constexpr int kLag = 2;                      // loader: copy groups in flight behind the newest one
+// registers per thread after the roles have split: 256 x 200 + 256 x 56 = 65,536 = the 512 x 128 the CTA is
+// launched with
+constexpr int kRegsSoftmax = 200, kRegsOther = 56;
+constexpr uint32_t kApart = 1000;            // clocks between the exponentials of the two halves
 
+constexpr int kSchedDepth = 4;
 constexpr int kRowBytes = 128;                 // 64 bf16
 constexpr int kTileBytes = kTile * kRowBytes;  // 16 KB: 128 rows
 constexpr uint32_t kOffQ = 0;                                // [2 buffers][2 halves] x 16 KB
 constexpr uint32_t kOffKV = 4 * kTileBytes;                  // [kStages] x (K 16 KB, V 16 KB)
-constexpr uint32_t kOffBar = kOffKV + kStages * 2 * kTileBytes;
+constexpr uint32_t kOffMeta = kOffKV + kStages * 2 * kTileBytes;    // [2 buffers] x (perm, seg_lo, seg_hi) of 256 rows
+constexpr uint32_t kOffStage = kOffMeta + 2 * 3 * kUnitRows * 4;    // [softmax warps] x 32 rows x 64 bytes
+constexpr uint32_t kOffUnit = kOffStage + kSoftmaxWarps * 2048;     // [kSchedDepth] unit records
+constexpr uint32_t kOffBar = kOffUnit + kSchedDepth * sizeof(FwdUnit);
 constexpr uint32_t kSmemBytes = kOffBar + 512 + 1024;        // + slack for the 1024-byte alignment
 static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 // tensor memory: S of half h at column 128 h; O at 256 + 64 h; P (bf16 pairs) at 384 + 64 h
@@ -62,26 +86,26 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kTmemO = 256;
 constexpr uint32_t kTmemP = 384;
 constexpr uint32_t kWaitLimit = 4096;        // tries (up to 1 ms each) before a wait gives up
-constexpr float kRescaleThreshold = 8.f;     // log2 units
+constexpr float kRescale = 8.f;                              // exact units: log2 units before the base moves
+constexpr float kSumMin = 0x1p-100f, kSumMax = 0x1p60f;      // row sums outside: the unit is done once more, exactly
 
 // barrier slots (8 bytes each) behind kOffBar
 enum {
-    kBarQFull = 0,    // [2] loader -> MMA         (count: loader warps)
-    kBarQEmpty = 2,   // [2] MMA commit -> loader  (count 2: one per half)
-    kBarKVFull = 4,   // [kStages] loader -> MMA   (count: loader warps)
-    kBarKVEmpty = 9,  // [kStages] MMA -> loader   (count 2: one per half)
-    kBarSFull = 14,   // [2] MMA commit -> softmax (count 1)
-    kBarPFull = 16,   // [2] softmax -> MMA        (count 4: one per warp)
-    kBarPVDone = 18,  // [2] MMA commit -> softmax: the P V of a tile is complete (count 1)
+    kBarQFull = 0,        // [2] loaders -> MMA, softmax   (count: loader warps)
+    kBarQEmpty = 2,       // [2] MMA commits and softmax warps (row data read) -> loaders (count kMmaWarps + kSoftmaxWarps)
+    kBarKVFull = 4,       // [kStages] loaders -> MMA      (count: loader warps)
+    kBarKVEmpty = 8,      // [kStages] MMA -> loaders      (count 2: one per half)
+    kBarSFull = 12,       // [2] MMA commit -> softmax (count 1)
+    kBarSFree = 14,       // [2] softmax -> MMA: S of a tile has been read (count 4: one per warp)
+    kBarPFull = 16,       // [2] softmax -> MMA        (count 4: one per warp)
+    kBarPVDone = 18,      // [2] MMA commit -> softmax: the P V of a tile is complete (count 1)
     kBarFinal = 20,       // [2]
     kBarSchedFull = 22,   // [kSchedDepth] scheduler -> every warp that follows the unit list (count 1)
     kBarSchedEmpty = 26,  // [kSchedDepth] those warps -> scheduler (count kSchedReaders)
-    kBarSFree = 30,       // [2] softmax -> MMA: S of a tile has been read for the last time (count 4: one per warp)
-    kNumBars = 32
+    kNumBars = 30
 };
-constexpr int kSchedDepth = 4;
 constexpr int kSchedReaders = kSoftmaxWarps + kMmaWarps + kLoadWarps;
-static_assert(kStages <= 5, "barrier slots");
+static_assert(kStages == 4, "barrier slots");
 
 struct Params {
     // 2-D tensor maps over K and V seen as [B H N rows, 64 columns]: boxes of 128 rows, 128-byte swizzle
@@ -93,98 +117,54 @@ struct Params {
     float *LSE;
     ViewPlan rowv, colv;
     const uint8_t *head_view;
-    const FwdUnit *units;
-    int n_units;
+    const FwdUnit *units;      // by CTA; those of CTA c are [cta_off[c], cta_off[c + 1])
+    const int32_t *cta_off;
+    const PadChunk *pads;      // padding rows, which no unit covers
+    int n_pads;
     int N, H;
     TensorRows tr;     // where (example, head) starts in the tensors
     float scale_log2;  // scale * log2(e)
     int32_t *status;
-    int32_t *counters;
+    int32_t *counters;  // arrivals at the split units, 8 per unit
     uint8_t *ws;
 };
 
-struct TileInfo {
-    int k0, w;    // first key and number of keys (<= 128)
-    bool is_b;
-};
-
-__device__ __forceinline__ int n_tiles_a(const FwdUnit &u) {
-    return u.kA_end > u.kA0 ? (u.kA_end - u.kA0 + kTile - 1) / kTile : 0;
+// The loaders copy a tile of up to 128 rows (128 B each), warp w of the four the rows 32 w .. 32 w + 31.
+// Row rr of the tile comes from view position row0 + min(rr, clamp).  A lane looks up the original
+// position of one row (coalesced, one latency for the whole tile, and cheap enough to be done a tile
+// ahead); the copies then run four rows at a time, eight lanes per row, with the positions handed
+// around by shuffle.
+__device__ __forceinline__ int fetch_idx(const int32_t *perm, int row0, int clamp, int lw, int lane) {
+    const int t = row0 + min(32 * lw + lane, clamp);
+    return perm ? __ldg(perm + t) : t;  // no order given: the tensors are in view order
 }
-__device__ __forceinline__ int n_tiles_b(const FwdUnit &u) {
-    return u.kB_end > u.kB0 ? (u.kB_end - u.kB0 + kTile - 1) / kTile : 0;
-}
-__device__ __forceinline__ TileInfo tile_info(const FwdUnit &u, int i, int nA) {
-    TileInfo t;
-    if (i < nA) {
-        t.k0 = u.kA0 + i * kTile;
-        t.w = min(kTile, u.kA_end - t.k0);
-        t.is_b = false;
-    } else {
-        t.k0 = u.kB0 + (i - nA) * kTile;
-        t.w = min(kTile, u.kB_end - t.k0);
-        t.is_b = true;
-    }
-    return t;
-}
-__device__ __forceinline__ int rows_of_half(const FwdUnit &u, int h) {
-    return max(0, min(kTile, u.nq - h * kTile));
-}
-// Columns [c0, c1) of the tile (multiples of 16) needed by a half whose rows' segments span keys
-// [lo, hi); c1 <= c0 when it skips the tile.
-__device__ __forceinline__ void half_cols(int lo, int hi, const TileInfo &t, int &c0, int &c1) {
-    if (!t.is_b) {
-        c0 = 0;
-        c1 = (t.w + 15) & ~15;
-    } else {
-        c0 = (max(lo, t.k0) - t.k0) & ~15;
-        c1 = (min(hi, t.k0 + t.w) - t.k0 + 15) & ~15;
-    }
-}
-
-__device__ __forceinline__ FwdUnit load_unit(const FwdUnit *p) {
-    FwdUnit u;
-    const int4 *s = reinterpret_cast<const int4 *>(p);
-    int4 *d = reinterpret_cast<int4 *>(&u);
+// Rows [0, n_rows) of one tensor, or of two (`pair`; b_off: bytes from the first one's rows to the second's)
+// -> tiles at s_a and 16 KB behind it, 128-byte swizzle.
+__device__ __forceinline__ void gather_rows(uint32_t s_a, const uint8_t *a_bh, bool pair, int64_t b_off, int idx, int n_rows,
+                                            int lw, int lane) {
+    if (32 * lw >= n_rows) return;  // (rows past n_rows inside a group of 32 repeat a row that exists)
+    const int sub = lane >> 3;      // row of the group of four
+    a_bh += (lane & 7) * 16;
+    const uint32_t d = s_a + (32 * lw + sub) * kRowBytes + (((lane & 7) ^ sub) << 4);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) d[i] = __ldg(s + i);
-    return u;
-}
-
-// The loaders copy a tile of up to 128 rows (128 B each) in passes of kRowsPerPass rows, 8 threads
-// per row.  Row rr of the tile comes from view position row0 + min(rr, clamp); its original
-// position is looked up first for every pass (independent loads), then the 16-byte copies follow.
-constexpr int kRowsPerPass = kLoadThreads / 8;
-constexpr int kPasses = (kTile + kRowsPerPass - 1) / kRowsPerPass;
-
-__device__ __forceinline__ void load_indices(int (&idx)[kPasses], const int32_t *perm, int row0,
-                                             int n_rows, int clamp, int ltid) {
-#pragma unroll
-    for (int i = 0; i < kPasses; ++i) {
-        const int rr = (ltid >> 3) + kRowsPerPass * i;
-        const int t = row0 + min(rr, clamp);
-        idx[i] = rr < n_rows ? (perm ? __ldg(perm + t) : t) : -1;  // no order given: the tensors are in view order
-    }
-}
-__device__ __forceinline__ void copy_rows(uint32_t s_tile, const __nv_bfloat16 *src_bh,
-                                          const int (&idx)[kPasses], int ltid) {
-    const int chunk = ltid & 7;
-#pragma unroll
-    for (int i = 0; i < kPasses; ++i) {
-        const int rr = (ltid >> 3) + kRowsPerPass * i;
-        if (idx[i] >= 0)
-            cp_async16(s_tile + rr * kRowBytes + ((chunk ^ (rr & 7)) << 4),
-                       src_bh + (size_t)idx[i] * 64 + chunk * 8, 16u);
+    for (int i = 0; i < 8; ++i) {
+        const uint8_t *src = a_bh + (size_t)(uint32_t)__shfl_sync(0xffffffffu, idx, 4 * i + sub) * kRowBytes;
+        const uint32_t dst = (d ^ ((i & 1) << 6)) + 4 * i * kRowBytes;
+        cp_async16(dst, src);
+        if (pair) cp_async16(dst + kTileBytes, src + b_off);
     }
 }
 
 // A chunk is 32 scores of one row (tile-local columns cb .. cb + 31).  A column c counts for the row
-// iff r_lo <= c < r_lo + r_span; the scores of the other columns are replaced by -inf, which the row
-// max ignores and the exponential turns into an exact 0 (the scale is positive).
-__device__ __forceinline__ void chunk_mask(uint32_t (&v)[32], int cb, int r_lo, uint32_t r_span) {
+// iff r_lo <= c < r_hi; the scores of the other columns are replaced by -inf, which the row max
+// ignores and the exponential turns into an exact 0 (the scale is positive).
+__device__ __forceinline__ void chunk_mask(uint32_t (&v)[32], int cb, int r_lo, int r_hi) {
+    const int a = min(max(r_lo - cb, 0), 32), b = min(max(r_hi - cb, 0), 32);
+    const uint32_t below_b = b >= 32 ? 0xffffffffu : (1u << b) - 1u, below_a = a >= 32 ? 0xffffffffu : (1u << a) - 1u;
+    const uint32_t on = below_b & ~below_a;
 #pragma unroll
     for (int e = 0; e < 32; ++e)
-        if ((uint32_t)(cb + e - r_lo) >= r_span) v[e] = 0xff800000u;
+        if (!(on & (1u << e))) v[e] = 0xff800000u;
 }
 // Row max over one chunk, four partial maxima.
 __device__ __forceinline__ void chunk_max(const uint32_t (&v)[32], float (&tm)[4]) {
@@ -196,11 +176,11 @@ __device__ __forceinline__ void chunk_max(const uint32_t (&v)[32], float (&tm)[4
         tm[3] = fmax3(tm[3], __uint_as_float(v[e + 6]), __uint_as_float(v[e + 7]));
     }
 }
-// P of one chunk: exp2(s * scale_log2 + neg_m), packed as bf16 pairs (even column in the low half);
-// the row sums go to two packed pairs of partial sums.  The multiply-adds and the sums work on two
-// columns per instruction (packed fp32 pairs); only the exponential is per column.
-__device__ __forceinline__ void chunk_exp(const uint32_t (&v)[32], uint64_t scale2, uint64_t neg_m2,
-                                          uint32_t (&packed)[16], uint64_t &l01, uint64_t &l23) {
+// P of one chunk: exp2(s * scale_log2 + neg_m), packed as bf16 pairs (even column in the low half); the row
+// sums go to two packed pairs of partial sums.  The multiply-adds and the sums work on two columns per
+// instruction (packed fp32 pairs); only the exponential is per column.
+__device__ __forceinline__ void chunk_exp(const uint32_t (&v)[32], uint64_t scale2, uint64_t neg_m2, uint32_t (&packed)[16],
+                                          uint64_t &l01, uint64_t &l23) {
 #pragma unroll
     for (int e = 0; e < 32; e += 4) {
         float x0, x1, x2, x3;
@@ -209,9 +189,8 @@ __device__ __forceinline__ void chunk_exp(const uint32_t (&v)[32], uint64_t scal
         const float p0 = ex2(x0), p1 = ex2(x1), p2 = ex2(x2), p3 = ex2(x3);
         l01 = add_f32x2(l01, pack_f32x2(p0, p1));
         l23 = add_f32x2(l23, pack_f32x2(p2, p3));
-        __nv_bfloat162 b01 = __floats2bfloat162_rn(p0, p1), b23 = __floats2bfloat162_rn(p2, p3);
-        packed[e >> 1] = *reinterpret_cast<uint32_t *>(&b01);
-        packed[(e >> 1) + 1] = *reinterpret_cast<uint32_t *>(&b23);
+        packed[e >> 1] = cvt_bf16x2(p0, p1);
+        packed[(e >> 1) + 1] = cvt_bf16x2(p2, p3);
     }
 }
 __device__ __forceinline__ float sum_f32x2(uint64_t a, uint64_t b) {
@@ -229,18 +208,36 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     const uint32_t bars = base + kOffBar;
     volatile uint32_t *tmem_slot = (volatile uint32_t *)(sm + kOffBar + 8 * kNumBars);
     volatile int *s_abort = (volatile int *)(sm + kOffBar + 8 * kNumBars + 4);
-    volatile int *s_unit = (volatile int *)(sm + kOffBar + 8 * kNumBars + 8);  // [kSchedDepth] unit ids
+    volatile uint32_t *s_bad = (volatile uint32_t *)(sm + kOffBar + 8 * kNumBars + 16);  // [kSchedDepth] warps that need the unit once more
+    volatile uint32_t *s_stamp = s_bad + kSchedDepth;  // [softmax warps] when the warp began its exponentials
+    FwdUnit *s_unit = reinterpret_cast<FwdUnit *>(sm + kOffUnit);  // [kSchedDepth]; rows = 0 marks the end of the list
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = tid & 31;
+
+    // The first loader warp publishes the records of the CTA's units; its lanes 0-3 hold the next one ahead
+    // of its turn.
+    int u_next = 0, u_end = 0;
+    int4 rec = make_int4(0, 0, 0, 0);
+    auto fetch_record = [&]() {
+        rec = make_int4(0, 0, 0, 0);  // rows = 0: the list is exhausted
+        if (u_next < u_end && lane < 4) rec = __ldg(reinterpret_cast<const int4 *>(p.units + u_next) + lane);
+        ++u_next;
+    };
+    if (warp == kLoadWarp0) {  // requested before the set-up below, which takes as long
+        u_next = __ldg(p.cta_off + blockIdx.x);
+        u_end = __ldg(p.cta_off + blockIdx.x + 1);
+        fetch_record();
+    }
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
             mbar_init(bars + 8 * (kBarQFull + i), kLoadWarps);
-            mbar_init(bars + 8 * (kBarQEmpty + i), 2);
+            mbar_init(bars + 8 * (kBarQEmpty + i), kMmaWarps + kSoftmaxWarps);
             mbar_init(bars + 8 * (kBarSFull + i), 1);
-            mbar_init(bars + 8 * (kBarPFull + i), 4);
+            mbar_init(bars + 8 * (kBarSFree + i), kSoftmaxWarps / 2);
+            mbar_init(bars + 8 * (kBarPFull + i), kSoftmaxWarps / 2);
             mbar_init(bars + 8 * (kBarPVDone + i), 1);
-            mbar_init(bars + 8 * (kBarSFree + i), 4);
+            mbar_init(bars + 8 * (kBarFinal + i), 1);
         }
         for (int i = 0; i < kStages; ++i) {
             mbar_init(bars + 8 * (kBarKVFull + i), kLoadWarps);
@@ -250,9 +247,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             mbar_init(bars + 8 * (kBarSchedFull + i), 1);
             mbar_init(bars + 8 * (kBarSchedEmpty + i), kSchedReaders);
         }
-        mbar_init(bars + 8 * kBarFinal, 1);
-        mbar_init(bars + 8 * (kBarFinal + 1), 1);
         *s_abort = 0;
+        for (int i = 0; i < kSchedDepth; ++i) s_bad[i] = 0;
+        for (int i = 0; i < kSoftmaxWarps; ++i) s_stamp[i] = (uint32_t)clock() - 2 * kApart;
         fence_mbar_init();
     }
     if (warp == kMmaWarp) {
@@ -262,11 +259,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     // every wait is bounded; the first one to expire raises the abort flag, which ends all roles
     auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
         if (mbar_test_wait(bar, parity)) return true;  // already complete: no trip through the suspending form
+#pragma unroll 1
         for (uint32_t it = 0; it < kWaitLimit; ++it) {
             if (mbar_try_wait(bar, parity)) return true;
             if (*s_abort) return false;
@@ -280,489 +278,481 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     long long tr[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const long long tr_start = clock64();
 #endif
-    // The unit list is shared by all CTAs: lane 0 of the first loader warp takes the next index from
-    // a global counter and publishes it in a small ring; every warp that follows the list reads the
-    // n-th entry here (-1 = the list is exhausted) and frees the slot for the scheduler.
-    auto next_unit = [&](uint32_t n) -> int {
+    // The first loader warp publishes the records of the CTA's units in a small ring; every warp that
+    // follows the list reads the n-th entry here and frees the slot.  false = the list is exhausted.
+    auto next_unit = [&](uint32_t n, FwdUnit &u) -> bool {
         const int slot = n % kSchedDepth;
-        if (!wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) return -1;
-        const int u = s_unit[slot];
+        if (!wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) return false;
+        const int4 *src = reinterpret_cast<const int4 *>(s_unit + slot);
+        int4 *dst = reinterpret_cast<int4 *>(&u);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dst[i] = src[i];
         __syncwarp();
         if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
-        return u;
+        return u.rows != 0;
     };
 
     if (warp < kSoftmaxWarps) {
         // ------------------------------------------------------------------ softmax + epilogue
+        reg_alloc<kRegsSoftmax>();
         const int h = warp >> 2;
-        const int r = tid & 127;  // row of the half; TMEM lane
+        const int r = tid & 127;           // row of the half; TMEM lane
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tS = tmem + lane_base + h * kTile;
         const uint32_t tO = tmem + lane_base + kTmemO + h * 64;
         const uint32_t tP = tmem + lane_base + kTmemP + h * 64;
         const uint32_t bar_s = bars + 8 * (kBarSFull + h), bar_p = bars + 8 * (kBarPFull + h),
                        bar_pv = bars + 8 * (kBarPVDone + h), bar_sf = bars + 8 * (kBarSFree + h);
-        uint32_t ph_s = 0, ph_pv = 0;
+        uint8_t *stage = sm + kOffStage + warp * 2048;
+        const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
+        uint32_t ph_s = 0, ph_pv = 0, unit_cnt = 0;
         bool alive = true;
 
         for (uint32_t n = 0; alive; ++n) {
             TR_T0(t_nu);
-            const int u = next_unit(n);
+            const int slot = n % kSchedDepth;
+            if (!wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) break;
             TR_ADD(7, t_nu);
-            if (u < 0) break;
+            // The record and the row data stay in shared memory until the unit is done: what is needed of
+            // them is read where it is needed (registers are what this role is short of).
+            const FwdUnit &un = s_unit[slot];
+            if (un.rows == 0) break;
             TR_T0(t_setup);
-            const FwdUnit un = load_unit(p.units + u);
-            const int rows_h = rows_of_half(un, h);
-            if (rows_h == 0) continue;
-            const ViewPlan &vp = p.head_view[un.h] ? p.colv : p.rowv;
-            const int32_t *perm = vp.perm + (size_t)un.b * p.N;
-            const size_t bh = p.tr.base(un.b, un.h);
-            const bool row_valid = r < rows_h;
-            const int t_row = un.q0 + h * kTile + min(r, rows_h - 1);  // rows past the end shadow the last one
-            const int orig = p.view_order ? t_row : perm[t_row];
-            const int nA = n_tiles_a(un), nB = n_tiles_b(un), n_tiles = nA + nB;
-            const int h_lo = h ? un.lo[1] : un.lo[0], h_hi = h ? un.hi[1] : un.hi[0];  // segments of this half's rows
-
-            if (n_tiles == 0) {  // padding rows: O = 0, LSE = -inf
-                if (row_valid && p.tr.exists(un.b, orig)) {
-                    uint4 *dst = reinterpret_cast<uint4 *>(p.O + (bh + orig) * 64);
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) dst[c] = make_uint4(0, 0, 0, 0);
-                    p.LSE[bh + orig] = -INFINITY;
+            const int qb = unit_cnt & 1;
+            if (!(alive = wait(bars + 8 * (kBarQFull + qb), (unit_cnt >> 1) & 1))) break;
+            ++unit_cnt;
+            auto unit_done = [&]() {
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(bars + 8 * (kBarQEmpty + qb));
+                    mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
                 }
+            };
+            const int rows_h = un.rows_of(h);
+            if (rows_h == 0) {
+                unit_done();
                 continue;
             }
-
-            int my_lo = 0, my_hi = 0, w_lo_min = 0, w_lo_max = 0, w_hi_min = 0, w_hi_max = 0;
-            if (nB > 0) {
-                my_lo = vp.seg_lo[(size_t)un.b * p.N + t_row];
-                my_hi = vp.seg_hi[(size_t)un.b * p.N + t_row];
-                w_lo_min = w_lo_max = my_lo;
-                w_hi_min = w_hi_max = my_hi;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    w_lo_min = min(w_lo_min, __shfl_xor_sync(0xffffffffu, w_lo_min, o));
-                    w_lo_max = max(w_lo_max, __shfl_xor_sync(0xffffffffu, w_lo_max, o));
-                    w_hi_min = min(w_hi_min, __shfl_xor_sync(0xffffffffu, w_hi_min, o));
-                    w_hi_max = max(w_hi_max, __shfl_xor_sync(0xffffffffu, w_hi_max, o));
-                }
-            }
+            // this row's data: original position, key range (rows past the end shadow the last one)
+            const int32_t *meta = reinterpret_cast<const int32_t *>(sm + kOffMeta) + qb * 3 * kUnitRows + h * kTile + min(r, rows_h - 1);
+            // The tiles this half visits: those of range A, then those of range B that meet the key ranges of its
+            // rows, [k_lo, k_hi)
+            const int nA = un.tiles_a(), tB = un.tB & 0xff;
+            const int k_lo = max(un.lo[h], un.kB0), k_hi = min(un.hi[h], un.kB_end);
+            const int b0 = k_hi > k_lo ? (k_lo - un.kB0) / tB : 0, b1 = k_hi > k_lo ? (k_hi - un.kB0 - 1) / tB + 1 : 0;
+            const int n_visit = nA + b1 - b0;
+            const bool exact = (un.tB >> 8) != 0;
+            const int w_lo_max = __reduce_max_sync(0xffffffffu, meta[kUnitRows]), w_hi_min = __reduce_min_sync(0xffffffffu, meta[2 * kUnitRows]);
+            // tiles that count in full for every row of the warp: the first fa of range A, [fb0, fb1) of range B (by
+            // number of visit)
+            const int fa = max(un.kA_end - un.kA0, 0) / kTile;
+            const int fb0 = nA - b0 + (tB == kTile ? (max(w_lo_max - un.kB0, 0) + kTile - 1) / kTile : n_visit);
+            const int fb1 = nA - b0 + max(min(w_hi_min, k_hi) - un.kB0, 0) / kTile;
 
             TR_ADD(5, t_setup);
-            float m2 = -INFINITY, l = 0.f;  // running max (log2 domain, scaled) and row sum
-            bool first = true;
+            float m2 = -INFINITY;                // base of the row (log2 domain, scaled)
+            uint64_t l01 = 0ull, l23 = 0ull;     // row sum: packed pairs of partial sums
 
-            for (int i = 0; i < n_tiles && alive; ++i) {
-                const TileInfo t = tile_info(un, i, nA);
-                int c0, c1;
-                half_cols(h_lo, h_hi, t, c0, c1);
-                if (c1 <= c0) continue;
-
-                // this row's columns [r_lo, r_hi) and the warp's envelope, tile-local
-                int r_lo, r_hi, e_lo_min, e_lo_max, e_hi_min, e_hi_max;
-                if (!t.is_b) {
-                    r_lo = e_lo_min = e_lo_max = 0;
-                    r_hi = e_hi_min = e_hi_max = un.kA_end - t.k0;
-                } else {
-                    r_lo = my_lo - t.k0;
-                    r_hi = my_hi - t.k0;
-                    e_lo_min = w_lo_min - t.k0;
-                    e_lo_max = w_lo_max - t.k0;
-                    e_hi_min = w_hi_min - t.k0;
-                    e_hi_max = w_hi_max - t.k0;
-                }
-                const uint32_t r_span = (uint32_t)max(r_hi - r_lo, 0);
-                const int ch0 = c0 >> 5, ch1 = (c1 + 31) >> 5;
-
+#pragma unroll 1
+            for (int j = 0; j < n_visit; ++j) {
                 TR_T0(t_ws);
                 if (!(alive = wait(bar_s, ph_s))) break;
                 ph_s ^= 1;
                 tc_fence_after();
                 TR_ADD(0, t_ws);
-                // last chunk of the tile that this warp reads from tensor memory (-1: none): after it,
-                // S may be overwritten
-                int last_ld = -1;
-                for (int ch = ch0; ch < ch1; ++ch)
-                    if (!(ch * 32 + 32 <= e_lo_min || ch * 32 >= e_hi_max)) last_ld = ch;
-                auto release_s = [&]() {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_sf);
-                };
+                TR_T0(t_p2);
                 // P of the previous tile is still being read, and O written, until that tile's P V is done
-                bool pv_waited = first;
-                auto wait_pv = [&]() -> bool {
-                    if (pv_waited) return true;
+                bool p_free = j == 0;
+                auto wait_pv = [&]() {
+                    if (p_free) return;
                     TR_T0(t_wpv);
-                    if (!(alive = wait(bar_pv, ph_pv))) return false;
+                    alive = wait(bar_pv, ph_pv);
                     ph_pv ^= 1;
                     tc_fence_after();
-                    pv_waited = true;
+                    p_free = true;
                     TR_ADD(1, t_wpv);
-                    return true;
                 };
-
-                bool two_pass = first;
-                TR_T0(t_p2);
-                if (first) {
-                    // A unit's first tile has no running max yet.  The max over the first 32 columns in which
-                    // the warp has keys serves as the base when every row of the warp has a key there: the
-                    // one-pass path below then runs as for any other tile (and still falls back to two passes
-                    // when a row's max over the whole tile lies more than the threshold above that base).
-                    const int cq = max(ch0, e_lo_min > 0 ? e_lo_min >> 5 : 0);
-                    if (cq < ch1 && cq * 32 < e_hi_max) {
-                        float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                        uint32_t v[32];
-                        tmem_ld32(tS + cq * 32, v);
-                        tc_wait_ld();
-                        if (!(cq * 32 >= e_lo_max && cq * 32 + 32 <= e_hi_min)) chunk_mask(v, cq * 32, r_lo, r_span);
-                        chunk_max(v, tm);
-                        const float t = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2;
-                        if (__all_sync(0xffffffffu, t > -INFINITY)) {
-                            m2 = t;
-                            two_pass = false;
-                        }
+                // Base of the row from the max t2 of this tile (the whole warp takes part).
+                auto new_base = [&](float t2) {
+                    if (!exact) {
+                        m2 = t2 == -INFINITY ? 0.f : t2;
+                        return;
                     }
-                }
-                if (!two_pass) {
-                    // one pass with the running max; the tile's own max is known before S is given up
-                    float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                    const float neg_m = (m2 == -INFINITY) ? 0.f : -m2;
-                    const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2), neg_m2 = pack_f32x2(neg_m, neg_m);
-                    uint64_t lsum = 0ull, lsum1 = 0ull;  // packed pairs of partial row sums
-                    bool redo = false;
-#pragma unroll 1
-                    for (int ch = ch0; ch < ch1; ++ch) {
-                        const int cb = ch * 32;
-                        uint32_t packed[16];
-                        if (cb + 32 <= e_lo_min || cb >= e_hi_max) {
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) packed[e] = 0u;
-                        } else {
-                            uint32_t v[32];
-                            tmem_ld32(tS + cb, v);
-                            tc_wait_ld();
-                            if (!(cb >= e_lo_max && cb + 32 <= e_hi_min)) chunk_mask(v, cb, r_lo, r_span);
-                            chunk_max(v, tm);
-                            if (ch == last_ld) {
-                                const float t2 = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2;
-                                redo = __any_sync(0xffffffffu, t2 > m2 + kRescaleThreshold);
-                                if (redo) break;
-                                release_s();
-                            }
-                            chunk_exp(v, scale2, neg_m2, packed, lsum, lsum1);
-                        }
-                        if (!wait_pv()) break;
-                        tmem_st16(tP + ch * 16, packed);
-                    }
-                    if (!alive) break;
-                    if (!redo) {
-                        if (last_ld < 0) release_s();
-                        l += sum_f32x2(lsum, lsum1);
-                    }
-                    two_pass = redo;
-                }
-                if (two_pass) {
-                    // pass 1: row max of the raw scores, 32 columns at a time (chunks in which no row of
-                    // the warp has a key are not looked at)
-                    float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll 1
-                    for (int ch = ch0; ch < ch1; ++ch) {
-                        const int cb = ch * 32;
-                        if (cb + 32 <= e_lo_min || cb >= e_hi_max) continue;
-                        uint32_t v[32];
-                        tmem_ld32(tS + cb, v);
-                        tc_wait_ld();
-                        if (!(cb >= e_lo_max && cb + 32 <= e_hi_min)) chunk_mask(v, cb, r_lo, r_span);
-                        chunk_max(v, tm);
-                    }
-                    const float tmax = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3]));
-                    const float t2 = tmax * p.scale_log2;
-                    const bool grow = t2 > m2 + kRescaleThreshold;  // also true for the first finite max
+                    if (!__any_sync(0xffffffffu, t2 > m2 + kRescale)) return;
                     float alpha = 1.f;
-                    if (grow) {
+                    if (t2 > m2 + kRescale) {  // also the first finite max
                         alpha = ex2(m2 - t2);  // 0 when m2 = -inf
                         m2 = t2;
-                        l *= alpha;
                     }
-                    if (!wait_pv()) break;
-                    if (!first && __any_sync(0xffffffffu, grow)) {
-#pragma unroll
-                        for (int c2 = 0; c2 < 2; ++c2) {
-                            uint32_t o[32];
-                            tmem_ld32(tO + c2 * 32, o);
-                            tc_wait_ld();
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                            tmem_st32(tO + c2 * 32, o);
-                        }
-                        tc_wait_st();
-                    }
-                    const float neg_m = (m2 == -INFINITY) ? 0.f : -m2;
-
-                    // pass 2: P = exp2(s * scale_log2 - m) as bf16 pairs into the P columns, row sum
-                    const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2), neg_m2 = pack_f32x2(neg_m, neg_m);
-                    uint64_t lsum = 0ull, lsum1 = 0ull;
-                    if (last_ld < 0) release_s();
+                    if (j == 0) return;
+                    wait_pv();
+                    const uint64_t alpha2 = pack_f32x2(alpha, alpha);
+                    l01 = mul_f32x2(l01, alpha2);
+                    l23 = mul_f32x2(l23, alpha2);
 #pragma unroll 1
-                    for (int ch = ch0; ch < ch1; ++ch) {
-                        const int cb = ch * 32;
+                    for (int c2 = 0; c2 < 8; ++c2) {
+                        uint32_t o[8];
+                        tmem_ld8(tO + c2 * 8, o);
+                        tc_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                        tmem_st8(tO + c2 * 8, o);
+                    }
+                };
+                if (j < fa || (j >= fb0 && j < fb1)) {
+                    uint32_t v[4][32];
+#pragma unroll
+                    for (int ch = 0; ch < 4; ++ch) tmem_ld32(tS + ch * 32, v[ch]);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int ch = 0; ch < 4; ++ch) reg_fence(v[ch]);
+                    tc_fence_before();  // S may be overwritten
+                    if (lane == 0) mbar_arrive(bar_sf);
+                    if (j == 0 || exact) {
+                        // base of the row: the max over its first tile, or, exactly, over every tile
+                        float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                        for (int ch = 0; ch < 4; ++ch) chunk_max(v[ch], tm);
+                        new_base(fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2);
+                        // When the other half's warp on this scheduler has begun its exponentials a moment ago, let it
+                        // get ahead, at most kApart clocks; the distance then lasts.
+                        if (lane == 0) s_stamp[warp] = (uint32_t)clock();
+#pragma unroll 1
+                        for (int it = 0; it < 64 && h && (uint32_t)clock() - s_stamp[warp ^ 4] < kApart; ++it) {}
+                    }
+                    const uint64_t neg_m2 = pack_f32x2(-m2, -m2);
+#pragma unroll
+                    for (int ch = 0; ch < 4; ++ch) {
                         uint32_t packed[16];
-                        if (cb + 32 <= e_lo_min || cb >= e_hi_max) {
+                        chunk_exp(v[ch], scale2, neg_m2, packed, l01, l23);
+                        if (ch == 0) wait_pv();
+                        tmem_st16(tP + ch * 16, packed);
+                    }
+                } else {
+                    // the tile's keys start at k0; the half's MMAs touch the columns [c_begin, c1), this row counts
+                    // [r_lo, r_hi), and some row of the warp counts columns only within [e_lo, e_hi)
+                    const bool is_b = j >= nA;
+                    const int k0 = is_b ? un.kB0 + (b0 + j - nA) * tB : un.kA0 + j * kTile;
+                    const int t_end = min((is_b ? k_hi : un.kA_end) - k0, is_b ? tB : kTile);
+                    const int r_lo = is_b ? meta[kUnitRows] - k0 : 0, r_hi = is_b ? min(meta[2 * kUnitRows] - k0, t_end) : t_end;
+                    const int e_lo = __reduce_min_sync(0xffffffffu, r_lo), e_hi = __reduce_max_sync(0xffffffffu, r_hi);
+                    const int c_begin = is_b ? max(k_lo - k0, 0) & ~31 : 0, c1 = (t_end + 15) & ~15;
+                    uint32_t v[32];
+                    if (j == 0 || exact) {
+                        float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 1
+                        for (int cb = max(c_begin, e_lo & ~31); cb < e_hi; cb += 32) {
+                            tmem_ld32(tS + cb, v);
+                            tc_wait_ld();
+                            reg_fence(v);
+                            chunk_mask(v, cb, r_lo, r_hi);
+                            chunk_max(v, tm);
+                        }
+                        new_base(fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2);
+                    }
+                    const float neg_m = m2 == -INFINITY ? 0.f : -m2;
+                    const uint64_t neg_m2 = pack_f32x2(neg_m, neg_m);
+                    bool held = true;  // S has not been given up yet
+                    wait_pv();
+#pragma unroll 1
+                    for (int cb = c_begin; cb < c1; cb += 32) {
+                        uint32_t packed[16];
+                        if (cb + 32 <= e_lo || cb >= e_hi) {  // no row of the warp has a key here
 #pragma unroll
                             for (int e = 0; e < 16; ++e) packed[e] = 0u;
                         } else {
-                            uint32_t v[32];
                             tmem_ld32(tS + cb, v);
                             tc_wait_ld();
-                            if (ch == last_ld) release_s();
-                            if (!(cb >= e_lo_max && cb + 32 <= e_hi_min)) chunk_mask(v, cb, r_lo, r_span);
-                            chunk_exp(v, scale2, neg_m2, packed, lsum, lsum1);
+                            reg_fence(v);
+                            if (cb + 32 >= e_hi) {  // read for the last time
+                                tc_fence_before();
+                                if (lane == 0) mbar_arrive(bar_sf);
+                                held = false;
+                            }
+                            chunk_mask(v, cb, r_lo, r_hi);
+                            chunk_exp(v, scale2, neg_m2, packed, l01, l23);
                         }
-                        tmem_st16(tP + ch * 16, packed);
+                        tmem_st16(tP + (cb >> 1), packed);
                     }
-                    l += sum_f32x2(lsum, lsum1);
+                    if (held) {
+                        tc_fence_before();
+                        if (lane == 0) mbar_arrive(bar_sf);
+                    }
                 }
-                first = false;
-
+                if (!alive) break;
                 tc_wait_st();
                 tc_fence_before();
-                __syncwarp();
                 if (lane == 0) mbar_arrive(bar_p);
                 TR_ADD(3, t_p2);
                 TR_INC(4);
             }
             if (!alive) break;
 
-            // epilogue: wait for the last P V of this half
+            // epilogue: wait for the last P V of this half (a half may have visited no tile at all: in its part of
+            // a split unit, or when its rows have no key)
             TR_T0(t_ep);
-            if (!(alive = wait(bar_pv, ph_pv))) break;
-            ph_pv ^= 1;
-            tc_fence_after();
-            TR_ADD(1, t_ep);
-            uint32_t o0[32], o1[32];
-            tmem_ld32(tO, o0);
-            tmem_ld32(tO + 32, o1);
-            tc_wait_ld();
-
-            if (un.n_parts == 1) {
-                const float inv_l = l > 0.f ? 1.f / l : 0.f;  // a row without any key (possible in the passes of the
-                                                               // row-or-column pattern) gives O = 0, LSE = -inf
-                if (row_valid) {
-                    uint4 *dst = reinterpret_cast<uint4 *>(p.O + (bh + orig) * 64);
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint32_t *src = c < 4 ? o0 + 8 * c : o1 + 8 * (c - 4);
-                        uint32_t wv[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(src[2 * e]) * inv_l,
-                                                                      __uint_as_float(src[2 * e + 1]) * inv_l);
-                            wv[e] = *reinterpret_cast<uint32_t *>(&b2);
-                        }
-                        dst[c] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-                    }
-                    p.LSE[bh + orig] = (m2 + log2f(l)) * 0.6931471805599453f;
+            float l = sum_f32x2(l01, l23);
+            if (n_visit > 0) {
+                if (!(alive = wait(bar_pv, ph_pv))) break;
+                ph_pv ^= 1;
+                tc_fence_after();
+            }
+            bool write = true;
+            if (exact) {
+                write = ((un.tB >> 16) >> warp) & 1;  // the others were right the first time
+            } else if (n_visit > 0) {
+                const bool has_keys = nA > 0 || min(meta[2 * kUnitRows], k_hi) > max(meta[kUnitRows], k_lo);
+                if (__any_sync(0xffffffffu, !(l < kSumMax) || (l < kSumMin && has_keys))) {
+                    write = false;
+                    if (lane == 0) atomicOr((uint32_t *)s_bad + slot, 1u << warp);
                 }
-            } else {
-                // split unit: publish the un-normalised partial, the last part to arrive combines
-                float *part = reinterpret_cast<float *>(p.ws + ((size_t)un.ws_off << 10));
-                const int prow = h * kTile + r;
-                float4 *po = reinterpret_cast<float4 *>(part + (size_t)prow * 64);
+            }
+            const int n_parts = un.n_parts();
+            const float4 *parts = nullptr;  // this row's column groups (of four) in the first part
+            constexpr size_t kPartStride = kPartialBytes / sizeof(float4);
+            if (write && n_parts > 1) {
+                // Split unit: publish the un-normalised partial (groups of four columns by row, so that the
+                // lanes of a warp write and read consecutive 16-byte words).  Every warp owns its 32 rows: it
+                // counts the arrival, and the warp that comes last for these rows combines all parts (no wait
+                // on another CTA anywhere).
+                float4 *part = reinterpret_cast<float4 *>(p.ws + ((size_t)un.ws_off << 10)) + h * kTile + r;
+#pragma unroll 1
+                for (int c2 = 0; c2 < 4; ++c2) {
+                    uint32_t o[16];
+                    if (n_visit > 0) {
+                        tmem_ld16(tO + c2 * 16, o);
+                        tc_wait_ld();
+                    } else {
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    po[c] = make_float4(__uint_as_float(o0[4 * c]), __uint_as_float(o0[4 * c + 1]),
-                                        __uint_as_float(o0[4 * c + 2]), __uint_as_float(o0[4 * c + 3]));
+                        for (int e = 0; e < 16; ++e) o[e] = 0u;
+                    }
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    po[8 + c] = make_float4(__uint_as_float(o1[4 * c]), __uint_as_float(o1[4 * c + 1]),
-                                            __uint_as_float(o1[4 * c + 2]), __uint_as_float(o1[4 * c + 3]));
-                part[kUnitRows * 64 + prow] = m2;
-                part[kUnitRows * 64 + kUnitRows + prow] = l;
-                // every warp owns its 32 rows: publish, count the arrival, and the warp that comes
-                // last for these rows combines all parts (no wait on another CTA anywhere)
+                    for (int c = 0; c < 4; ++c)
+                        part[(c2 * 4 + c) * kUnitRows] = make_float4(__uint_as_float(o[4 * c]), __uint_as_float(o[4 * c + 1]),
+                                                                     __uint_as_float(o[4 * c + 2]), __uint_as_float(o[4 * c + 3]));
+                }
+                part[16 * kUnitRows] = make_float4(m2, l, 0.f, 0.f);
                 __threadfence();
                 __syncwarp();
                 int last = 0;
                 if (lane == 0) {
-                    int32_t *ctr = p.counters + kSchedWords + 8 * un.ctr + 4 * h + (warp & 3);
-                    last = atomicAdd(ctr, 1) == un.n_parts - 1;
+                    int32_t *ctr = p.counters + 8 * un.ctr + warp;
+                    last = atomicAdd(ctr, 1) == n_parts - 1;
                     if (last) *ctr = 0;  // ready for the next launch
                 }
-                last = __shfl_sync(0xffffffffu, last, 0);
-                if (last) {
-                    // The warp combines its 32 rows one row at a time with all lanes on the row's 64
-                    // columns (two per lane), so every load of a partial row is one coalesced 256-byte
-                    // request; a row's weights live in the lane of that row and travel by shuffle.
+                write = __shfl_sync(0xffffffffu, last, 0) != 0;
+                if (write) {
                     __threadfence();
-                    const float *first_part = reinterpret_cast<const float *>(
-                        p.ws + ((size_t)(un.ws_off - un.part * (int)(kPartialBytes >> 10)) << 10));
-                    const size_t stride = kPartialBytes / sizeof(float);
-                    const float *ml = first_part + kUnitRows * 64 + prow;  // this lane's row: max, then sum
-                    float M = -INFINITY;
-                    for (int q = 0; q < un.n_parts; ++q) M = fmaxf(M, __ldcg(ml + q * stride));
-                    float L = 0.f;
-                    for (int q = 0; q < un.n_parts; ++q)
-                        L = fmaf(__ldcg(ml + q * stride + kUnitRows), ex2(__ldcg(ml + q * stride) - M), L);
-                    const float inv_L = 1.f / L;
-                    float2 acc[32];
+                    parts = part - un.part() * kPartStride;
+                    m2 = -INFINITY;
+                    l = 0.f;
+#pragma unroll 4
+                    for (int q = 0; q < n_parts; ++q) {  // (a part in which the row has no key has the sum 0)
+                        const float4 s = __ldcg(parts + q * kPartStride + 16 * kUnitRows);
+                        m2 = fmaxf(m2, s.y > 0.f ? s.x : -INFINITY);
+                    }
+#pragma unroll 4
+                    for (int q = 0; q < n_parts; ++q) {
+                        const float4 s = __ldcg(parts + q * kPartStride + 16 * kUnitRows);
+                        l = s.y > 0.f ? fmaf(s.y, ex2(s.x - m2), l) : l;
+                    }
+                }
+            }
+            if (write) {
+                // a row without any key (possible in the passes of the row-or-column pattern) gives O = 0, LSE = -inf
+                const float inv_l = l > 0.f ? 1.f / l : 0.f;
+                const bool row_valid = r < rows_h;
+                const int orig = p.view_order ? un.row0_of(h) + r : meta[0], dst_row = row_valid ? orig : -1;
+                const size_t bh = p.tr.base(un.b, un.h);
+                if (row_valid) p.LSE[bh + orig] = (m2 + log2f(l)) * 0.6931471805599453f;
+                // rows go through the warp's staging area, 32 columns at a time, so that a store instruction
+                // writes 64 consecutive bytes of eight rows
+#pragma unroll 1
+                for (int c2 = 0; c2 < 2; ++c2) {
+                    uint32_t o[32];
+                    if (parts || n_visit == 0) {
 #pragma unroll
-                    for (int rr = 0; rr < 32; ++rr) acc[rr] = make_float2(0.f, 0.f);
-                    const int row0 = h * kTile + (warp & 3) * 32;  // first row of this warp in the partials
-                    for (int q = 0; q < un.n_parts; ++q) {
-                        const float wq = ex2(__ldcg(ml + q * stride) - M) * inv_L;
-                        const float2 *src = reinterpret_cast<const float2 *>(first_part + q * stride + (size_t)row0 * 64) + lane;
+                        for (int e = 0; e < 32; ++e) o[e] = 0u;
+#pragma unroll 2
+                        for (int q = 0; q < (parts ? n_parts : 0); ++q) {  // in the order of the parts, whoever comes last
+                            const float4 s = __ldcg(parts + q * kPartStride + 16 * kUnitRows);
+                            const float wq = s.y > 0.f ? ex2(s.x - m2) : 0.f;
 #pragma unroll
-                        for (int rr = 0; rr < 32; ++rr) {
-                            const float2 x = __ldcg(src + rr * 32);
-                            const float w = __shfl_sync(0xffffffffu, wq, rr);
-                            acc[rr].x = fmaf(x.x, w, acc[rr].x);
-                            acc[rr].y = fmaf(x.y, w, acc[rr].y);
+                            for (int c = 0; c < 8; ++c) {
+                                const float4 x = __ldcg(parts + q * kPartStride + (c2 * 8 + c) * kUnitRows);
+                                o[4 * c] = __float_as_uint(fmaf(x.x, wq, __uint_as_float(o[4 * c])));
+                                o[4 * c + 1] = __float_as_uint(fmaf(x.y, wq, __uint_as_float(o[4 * c + 1])));
+                                o[4 * c + 2] = __float_as_uint(fmaf(x.z, wq, __uint_as_float(o[4 * c + 2])));
+                                o[4 * c + 3] = __float_as_uint(fmaf(x.w, wq, __uint_as_float(o[4 * c + 3])));
+                            }
                         }
+                    } else {
+                        tmem_ld32(tO + c2 * 32, o);
+                        tc_wait_ld();
+                        reg_fence(o);
                     }
 #pragma unroll
-                    for (int rr = 0; rr < 32; ++rr) {
-                        const int dst_row = __shfl_sync(0xffffffffu, orig, rr);
-                        const bool ok = __shfl_sync(0xffffffffu, (int)row_valid, rr) != 0;
-                        if (ok) {
-                            __nv_bfloat162 b2 = __floats2bfloat162_rn(acc[rr].x, acc[rr].y);
-                            reinterpret_cast<__nv_bfloat162 *>(p.O + (bh + dst_row) * 64)[lane] = b2;
-                        }
+                    for (int j = 0; j < 4; ++j) {
+                        uint32_t w4[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            w4[e] = cvt_bf16x2(__uint_as_float(o[8 * j + 2 * e]) * inv_l, __uint_as_float(o[8 * j + 2 * e + 1]) * inv_l);
+                        *reinterpret_cast<uint4 *>(stage + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
+                            make_uint4(w4[0], w4[1], w4[2], w4[3]);
                     }
-                    if (row_valid) p.LSE[bh + orig] = (M + log2f(L)) * 0.6931471805599453f;
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int row = 8 * i + (lane >> 2), j = lane & 3;
+                        const int dr = __shfl_sync(0xffffffffu, dst_row, row);
+                        const uint4 x = *reinterpret_cast<const uint4 *>(stage + row * 64 + ((j ^ ((row >> 1) & 3)) << 4));
+                        if (dr >= 0) *reinterpret_cast<uint4 *>(p.O + (bh + dr) * 64 + c2 * 32 + j * 8) = x;
+                    }
+                    __syncwarp();
                 }
             }
             tc_fence_before();  // O was read; the next unit's first P V may overwrite it
+            unit_done();
             TR_ADD(6, t_ep);
         }
-    } else if (warp < kLoadWarp0) {
-        // ------------------------------------------------------------------ MMA issuers (one thread per half)
-        // Per half: Q K^T of a tile -> (softmax) -> when P arrives, the Q K^T of the half's next tile
-        // goes first (the softmax warps wait for it) and the P V of the finished tile behind it.  A
-        // tile's ring stage is released by both halves: by the commit behind the P V, or, for a
-        // tile the half skips, by a plain arrival once the tile has landed.
-        if (lane == 0) {
-            const int h = warp - kMmaWarp;
-            uint32_t kv_cnt = 0, unit_cnt = 0, ph_p = 0, ph_sf = 0;
-            bool alive = true;
-            const uint32_t idesc_pv = idesc_bf16(128, 64, 0, 1);
-            const uint32_t tSh0 = tmem + h * kTile, tOh = tmem + kTmemO + h * 64, tPh0 = tmem + kTmemP + h * 64;
-            const uint32_t bar_p = bars + 8 * (kBarPFull + h), bar_s = bars + 8 * (kBarSFull + h),
-                           bar_pv = bars + 8 * (kBarPVDone + h), bar_sf = bars + 8 * (kBarSFree + h);
+    } else if (warp < kPadWarp0) {
+        // ------------------------------------------------------------------ MMA issuers (one warp per half)
+        // Per half: Q K^T of a tile -> (softmax) -> as soon as S sits in registers the Q K^T of the
+        // half's next tile, and behind it the P V of the tile once its P has arrived.  A tile's ring
+        // stage is released by both halves: by the commit behind the P V, or, for a tile the half
+        // skips, by a plain arrival once the tile has landed.  The whole warp runs the control flow (the
+        // operands stay warp-uniform: 64 / 32 clk per Q K^T / P V step, the rate of the tensor pipe,
+        // against 51 clk per P V step when a single diverged thread computes them); one lane issues.
+        reg_dealloc<kRegsOther>();
+        const bool leader = elect_one();
+        const int h = warp - kMmaWarp;
+        uint32_t kv_cnt = 0, unit_cnt = 0, ph_p = 0, ph_sf = 0;
+        bool alive = true;
+        const uint32_t idesc_pv = idesc_bf16(128, 64, 0, 1);
+        const uint32_t tSh0 = tmem + h * kTile, tOh = tmem + kTmemO + h * 64, tPh0 = tmem + kTmemP + h * 64;
+        const uint32_t bar_p = bars + 8 * (kBarPFull + h), bar_s = bars + 8 * (kBarSFull + h),
+                       bar_pv = bars + 8 * (kBarPVDone + h), bar_sf = bars + 8 * (kBarSFree + h);
+        FwdUnit un;
 
-            for (uint32_t n = 0; alive; ++n) {
-                const int slot = n % kSchedDepth;
-                if (!(alive = wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1))) break;
-                const int u = s_unit[slot];
-                mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
-                if (u < 0) break;
-                const FwdUnit un = load_unit(p.units + u);
-                const int nA = n_tiles_a(un), nB = n_tiles_b(un), n_tiles = nA + nB;
-                const int h_lo = h ? un.lo[1] : un.lo[0], h_hi = h ? un.hi[1] : un.hi[0];  // segments of this half's rows
-                if (n_tiles == 0) continue;
-                const int qb = unit_cnt & 1;
-                TR_T0(t_qf);
-                if (!(alive = wait(bars + 8 * (kBarQFull + qb), (unit_cnt >> 1) & 1))) break;
+        for (uint32_t n = 0; alive; ++n) {
+            if (!next_unit(n, un)) break;
+            un.tB &= 0xff;
+            const int nA = un.tiles_a(), nB = un.tiles_b(), n_tiles = nA + nB;
+            const int qb = unit_cnt & 1;
+            TR_T0(t_qf);
+            if (!(alive = wait(bars + 8 * (kBarQFull + qb), (unit_cnt >> 1) & 1))) break;
+            tc_fence_after();
+            TR_ADD(0, t_qf);
+            const uint32_t q_lo = smem_desc_lo(base + kOffQ + (qb * 2 + h) * kTileBytes);
+            const bool has_rows = un.rows_of(h) > 0;
+
+            // `out`: a tile whose Q K^T has been issued and whose P V has not; one step more than there are tiles
+            int o_c0 = 0, o_c1 = 0, o_stage = 0;
+            bool out = false, acc = false;
+#pragma unroll 1
+            for (int i = 0; i <= n_tiles; ++i) {
+                const TileInfo t = tile_info(un, i, nA);
+                const uint32_t c = kv_cnt + i;
+                const int stage = c % kStages;
+                int c0 = 0, c1 = 0;
+                if (has_rows && i < n_tiles) half_cols(h ? un.lo[1] : un.lo[0], h ? un.hi[1] : un.hi[0], t, c0, c1);
+                const bool visit = c1 > c0;
+                if (out) {  // S of the outstanding tile has been read
+                    TR_T0(t_sf);
+                    if (!(alive = wait(bar_sf, ph_sf))) break;
+                    ph_sf ^= 1;
+                    TR_ADD(6, t_sf);
+                }
+                if (visit) {  // the tile has landed
+                    TR_T0(t_kv);
+                    if (!(alive = wait(bars + 8 * (kBarKVFull + stage), (c / kStages) & 1))) break;
+                    TR_ADD(5, t_kv);
+                }
                 tc_fence_after();
-                TR_ADD(0, t_qf);
-                const uint32_t q_lo = smem_desc_lo(base + kOffQ + (qb * 2 + h) * kTileBytes);
-                const bool has_rows = rows_of_half(un, h) > 0;
-
-                // `out`: a tile whose Q K^T has been issued and whose P V has not
-                int o_c0 = 0, o_c1 = 0, o_stage = 0;
-                bool out = false, acc = false;
-
-                auto issue_pv = [&]() -> bool {  // waits for the P of the outstanding tile, then O += P V
+                if (visit) {
+                    TR_T0(t_qk);
+                    const uint32_t idesc = idesc_bf16(128, c1 - c0, 0, 0);
+                    const uint32_t k_lo = smem_desc_lo(base + kOffKV + stage * 2 * kTileBytes + c0 * kRowBytes);
+                    const uint32_t tSh = tSh0 + c0;
+                    if (leader) {
+                        mma_ss_lean<0>(tSh, q_lo, k_lo, idesc);  // K = 64 as four steps of 16 (32 bytes)
+                        mma_ss_lean<1>(tSh, q_lo + 2, k_lo + 2, idesc);
+                        mma_ss_lean<1>(tSh, q_lo + 4, k_lo + 4, idesc);
+                        mma_ss_lean<1>(tSh, q_lo + 6, k_lo + 6, idesc);
+                        mma_commit(bar_s);
+                    }
+                    __syncwarp();
+                    TR_ADD(2, t_qk);
+                    TR_INC(4);
+                }
+                if (out) {  // P V of the previous tile, behind this tile's Q K^T: O += P V
                     TR_T0(t_wp);
-                    if (!wait(bar_p, ph_p)) return false;
+                    if (!(alive = wait(bar_p, ph_p))) break;
                     TR_ADD(1, t_wp);
                     ph_p ^= 1;
                     tc_fence_after();
                     TR_T0(t_pv);
                     const int ks0 = o_c0 >> 4, n_ks = (o_c1 - o_c0) >> 4;
                     // V rows 16 ks .. 16 ks + 15 (2 KB per step), P columns 8 ks .. 8 ks + 7
-                    uint32_t v_lo = smem_desc_lo(base + kOffKV + o_stage * 2 * kTileBytes + kTileBytes + ks0 * 16 * kRowBytes);
-                    uint32_t tPh = tPh0 + ks0 * 8;
-                    mma_ts_lean_flag(tOh, tPh, v_lo, idesc_pv, acc);
+                    const uint32_t v_lo = smem_desc_lo(base + kOffKV + o_stage * 2 * kTileBytes + kTileBytes + ks0 * 16 * kRowBytes);
+                    const uint32_t tPh = tPh0 + ks0 * 8;
+                    if (leader) {
+                        mma_ts_lean_flag(tOh, tPh, v_lo, idesc_pv, acc);
+                        if (n_ks == 8) {
+#pragma unroll
+                            for (int ks = 1; ks < 8; ++ks) mma_ts_lean<1>(tOh, tPh + 8 * ks, v_lo + ks * ((16 * kRowBytes) >> 4), idesc_pv);
+                        } else {
 #pragma unroll 1
-                    for (int ks = 1; ks < n_ks; ++ks) {
-                        v_lo += (16 * kRowBytes) >> 4;
-                        tPh += 8;
-                        mma_ts_lean<1>(tOh, tPh, v_lo, idesc_pv);
-                    }
-                    acc = true;
-                    out = false;
-                    mma_commit(bar_pv);
-                    mma_commit(bars + 8 * (kBarKVEmpty + o_stage));
-                    TR_ADD(3, t_pv);
-                    return true;
-                };
-                auto wait_s_free = [&]() -> bool {  // S of the outstanding tile has been read for the last time
-                    TR_T0(t_sf);
-                    if (!wait(bar_sf, ph_sf)) return false;
-                    ph_sf ^= 1;
-                    TR_ADD(6, t_sf);
-                    return true;
-                };
-
-                for (int i = 0; i < n_tiles && alive; ++i) {
-                    const TileInfo t = tile_info(un, i, nA);
-                    const uint32_t c = kv_cnt + i;
-                    const int stage = c % kStages;
-                    const uint32_t bar_kv = bars + 8 * (kBarKVFull + stage), par_kv = (c / kStages) & 1;
-                    int c0 = 0, c1 = 0;
-                    if (has_rows) half_cols(h_lo, h_hi, t, c0, c1);
-                    if (c1 <= c0) {  // this half skips the tile
-                        if (out) {  // nothing to issue ahead of the P V of the outstanding tile
-                            if (!(alive = wait_s_free())) break;
-                            if (!(alive = issue_pv())) break;
+                            for (int ks = 1; ks < n_ks; ++ks) mma_ts_lean<1>(tOh, tPh + 8 * ks, v_lo + ks * ((16 * kRowBytes) >> 4), idesc_pv);
                         }
-                        TR_T0(t_kv);
-                        if (!(alive = wait(bar_kv, par_kv))) break;
-                        TR_ADD(5, t_kv);
-                        mbar_arrive(bars + 8 * (kBarKVEmpty + stage));
-                        continue;
+                        mma_commit(bar_pv);
+                        mma_commit(bars + 8 * (kBarKVEmpty + o_stage));
                     }
-                    if (out && !(alive = wait_s_free())) break;
-                    TR_T0(t_kv);
-                    if (!(alive = wait(bar_kv, par_kv))) break;
-                    TR_ADD(5, t_kv);
-                    tc_fence_after();
-                    {
-                        TR_T0(t_qk);
-                        const uint32_t idesc = idesc_bf16(128, c1 - c0, 0, 0);
-                        const uint32_t k_lo = smem_desc_lo(base + kOffKV + stage * 2 * kTileBytes + c0 * kRowBytes);
-                        const uint32_t tSh = tSh0 + c0;
-                        mma_ss_lean<0>(tSh, q_lo, k_lo, idesc);  // K = 64 as four steps of 16 (32 bytes)
-                        mma_ss_lean<1>(tSh, q_lo + 2, k_lo + 2, idesc);
-                        mma_ss_lean<1>(tSh, q_lo + 4, k_lo + 4, idesc);
-                        mma_ss_lean<1>(tSh, q_lo + 6, k_lo + 6, idesc);
-                        mma_commit(bar_s);
-                        TR_ADD(2, t_qk);
-                        TR_INC(4);
-                    }
-                    if (out && !(alive = issue_pv())) break;  // P V of the previous tile, behind this tile's Q K^T
-                    out = true;
-                    o_c0 = c0;
-                    o_c1 = c1;
-                    o_stage = stage;
+                    __syncwarp();
+                    acc = true;
+                    TR_ADD(3, t_pv);
                 }
-                if (alive && out) {
-                    if ((alive = wait_s_free())) alive = issue_pv();
+                if (!visit && i < n_tiles) {  // released by a plain arrival, but not before it has landed
+                    if (!(alive = wait(bars + 8 * (kBarKVFull + stage), (c / kStages) & 1))) break;
+                    if (lane == 0) mbar_arrive(bars + 8 * (kBarKVEmpty + stage));
                 }
-                kv_cnt += n_tiles;
-                if (!alive) break;
-                mma_commit(bars + 8 * (kBarQEmpty + qb));
-                ++unit_cnt;
+                out = visit;
+                o_c0 = c0;
+                o_c1 = c1;
+                o_stage = stage;
             }
-            // nothing of this CTA may still run on the tensor pipe when TMEM is freed
-            mma_commit(bars + 8 * (kBarFinal + h));
-            mbar_wait_bounded(bars + 8 * (kBarFinal + h), 0, kWaitLimit);
+            kv_cnt += n_tiles;
+            if (!alive) break;
+            if (leader) mma_commit(bars + 8 * (kBarQEmpty + qb));
+            __syncwarp();
+            ++unit_cnt;
         }
+        // nothing of this CTA may still run on the tensor pipe when TMEM is freed
+        if (leader) mma_commit(bars + 8 * (kBarFinal + h));
         __syncwarp();
+        mbar_wait_bounded(bars + 8 * (kBarFinal + h), 0, kWaitLimit);
+    } else if (warp < kLoadWarp0) {
+        // ------------------------------------------------------------------ padding rows: O = 0, LSE = -inf
+        reg_dealloc<kRegsOther>();
+#pragma unroll 1
+        for (int c = blockIdx.x; c < p.n_pads; c += gridDim.x) {
+            const PadChunk pc = p.pads[c];
+            const ViewPlan &vp = p.head_view[pc.h] ? p.colv : p.rowv;
+#pragma unroll 4
+            for (int i = (warp - kPadWarp0) * 4 + (lane >> 3); i < pc.n; i += 4 * kPadWarps) {  // eight lanes per row
+                const int t = pc.t0 + i;
+                const int orig = p.view_order ? t : __ldg(vp.perm + (size_t)pc.b * p.N + t);
+                if (p.tr.exists(pc.b, orig)) {
+                    const size_t row = p.tr.base(pc.b, pc.h) + orig;
+                    reinterpret_cast<uint4 *>(p.O + row * 64)[lane & 7] = make_uint4(0, 0, 0, 0);
+                    if ((lane & 7) == 0) p.LSE[row] = -INFINITY;
+                }
+            }
+        }
     } else {
         // ------------------------------------------------------------------ loaders
-        const int ltid = tid - 32 * kLoadWarp0;
+        reg_dealloc<kRegsOther>();
+        const int ltid = tid - 32 * kLoadWarp0, lw = warp - kLoadWarp0;
         uint32_t kv_cnt = 0, unit_cnt = 0;
         uint32_t pend[kLag];
 #pragma unroll
@@ -816,58 +806,50 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             return ok;
         };
 
-        // scheduler state (lane 0 of the first loader warp only)
-        uint32_t produced = 0;
-        bool list_done = false;
-        auto produce = [&]() -> bool {  // publishes one more entry; false = gave up
-            const int slot = produced % kSchedDepth;
-            if (produced >= (uint32_t)kSchedDepth) {
-                const uint32_t par = ((produced / kSchedDepth) & 1) ^ 1;
-                const uint32_t bar = bars + 8 * (kBarSchedEmpty + slot);
-                if (!wait(bar, par)) return false;
-            }
-            // the first unit of a CTA is its own index; later ones come from the shared counter
-            const int u = produced == 0 ? (int)blockIdx.x : atomicAdd(p.counters, 1) + (int)gridDim.x;
-            const int val = u < p.n_units ? u : -1;
-            s_unit[slot] = val;
-            mbar_arrive(bars + 8 * (kBarSchedFull + slot));  // release: the store above is visible to the readers
-            ++produced;
-            if (val < 0) list_done = true;
-            return true;
-        };
+        FwdUnit un;
+        uint32_t checked = 0;  // entries of the list that are known to be done
+        int4 held_back = make_int4(0, 0, 0, 0);
+        auto rec_rows = [&]() { return __shfl_sync(0xffffffffu, rec.w, 0); };  // FwdUnit::rows
 
         for (uint32_t n = 0; alive; ++n) {
-            // Entry n is taken only now, when the loaders are about to start on it (they run a few key
-            // tiles ahead of the other warps): taking units earlier would hand them out before it is
-            // known which CTA becomes free first.  Before a loader warp blocks here it signals its
-            // pending copy groups: the warps it would wait for may need exactly those tiles.
-            {
-                const int slot = n % kSchedDepth;
-                bool must_wait;
-                if (warp == kLoadWarp0) {  // the scheduler's warp: blocks only if the ring slot is still being read
-                    must_wait = produced >= (uint32_t)kSchedDepth &&
-                                !mbar_test_wait(bars + 8 * (kBarSchedEmpty + slot), ((produced / kSchedDepth) & 1) ^ 1);
-                    must_wait = __shfl_sync(0xffffffffu, (int)must_wait, 0) != 0;
-                } else {
-                    must_wait = !__all_sync(0xffffffffu, mbar_test_wait(bars + 8 * (kBarSchedFull + slot),
-                                                                       (n / kSchedDepth) & 1));
+            const int slot = n % kSchedDepth;
+            if (warp == kLoadWarp0) {
+                // Before the n-th entry goes out, the entries up to n - kSchedDepth have to be done (their slots are
+                // used again), and before the end of the list all of them: one that came out with a row sum out of
+                // range goes out once more, as an exact unit for the warps concerned.
+                const uint32_t done_to = rec_rows() ? n - min(n, (uint32_t)kSchedDepth - 1) : n;
+                bool again = false;
+                for (; checked < done_to && !again; ++checked) {
+                    const int sc = checked % kSchedDepth;
+                    if (!(alive = wait_free(bars + 8 * (kBarSchedEmpty + sc), (checked / kSchedDepth) & 1))) break;
+                    const uint32_t bad = s_bad[sc];
+                    if (bad) {
+                        again = true;
+                        held_back = rec;  // the record that was next comes after it
+                        if (lane < 4) rec = reinterpret_cast<const int4 *>(s_unit + sc)[lane];
+                        if (lane == 3) rec.x = (rec.x & 0xff) | 0x100 | bad << 16;
+                        __syncwarp();
+                        if (lane == 0) s_bad[sc] = 0;
+                    }
                 }
-                if (must_wait) flush();
+                if (!alive) break;
+                if (lane < 4) reinterpret_cast<int4 *>(s_unit + slot)[lane] = rec;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedFull + slot));  // release: the record is visible to the readers
+                if (again) rec = held_back;
+                else fetch_record();
+            } else if (!wait_free(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) {
+                break;
             }
-            if (ltid == 0) {
-                while (!list_done && produced <= n)
-                    if (!produce()) break;
-            }
-            __syncwarp();
-            const int u = next_unit(n);
-            if (u < 0) break;
-            const FwdUnit un = load_unit(p.units + u);
-            const int nA = n_tiles_a(un), nB = n_tiles_b(un), n_tiles = nA + nB;
-            if (n_tiles == 0) continue;
+            if (!next_unit(n, un)) break;
+            un.tB &= 0xff;
+            const int nA = un.tiles_a(), nB = un.tiles_b(), n_tiles = nA + nB;
             const ViewPlan &vp = p.head_view[un.h] ? p.colv : p.rowv;
-            const int32_t *perm = p.view_order ? nullptr : vp.perm + (size_t)un.b * p.N;
+            const size_t bn = (size_t)un.b * p.N;
+            const int32_t *perm = p.view_order ? nullptr : vp.perm + bn;
             const size_t bh = p.tr.base(un.b, un.h);
-            const __nv_bfloat16 *Qbh = p.Q + bh * 64, *Kbh = p.K + bh * 64, *Vbh = p.V + bh * 64;
+            const uint8_t *Qbh = reinterpret_cast<const uint8_t *>(p.Q + bh * 64), *Kbh = reinterpret_cast<const uint8_t *>(p.K + bh * 64);
+            const int64_t v_off = reinterpret_cast<const uint8_t *>(p.V) - reinterpret_cast<const uint8_t *>(p.K);
             // Rows of the order that sit in place in the tensors ([0, ident)): a full K/V tile inside that
             // range is one contiguous [128, 64] box and comes in by one bulk tensor copy per matrix
             // (issued by one thread, completing on the tile's barrier by byte count) instead of 2 x 1024
@@ -876,44 +858,58 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             const int ident = !p.use_tma ? 0 : p.view_order ? p.N : __ldg(vp.ident + un.b);
 
             const int qb = unit_cnt & 1;
-            if (!(alive = wait_free(bars + 8 * (kBarQEmpty + qb), ((unit_cnt >> 1) & 1) ^ 1))) break;
-            // (Q tiles are always gathered: fetching them with bulk copies as well measured slower.)
-            for (int h = 0; h < 2; ++h) {
-                const int rows_h = rows_of_half(un, h);
-                if (rows_h > 0) {
-                    int idx[kPasses];
-                    load_indices(idx, perm, un.q0 + h * kTile, kTile, rows_h - 1, ltid);
-                    copy_rows(base + kOffQ + (qb * 2 + h) * kTileBytes, Qbh, idx, ltid);
-                }
-            }
-            commit_and_signal(bars + 8 * (kBarQFull + qb));
-            ++unit_cnt;
-
-            for (int i = 0; i < n_tiles; ++i) {
-                const TileInfo t = tile_info(un, i, nA);
+            // steps -2, -1: the two Q halves (and the row data of the unit); steps 0 ..: the key tiles
+            auto step_idx = [&](int i) {
+                const TileInfo t = tile_info(un, max(i, 0), nA);
+                const int row0 = i < 0 ? un.row0_of(i + 2) : t.k0, rows = i < 0 ? un.rows_of(i + 2) : t.w;
+                return rows > 0 ? fetch_idx(perm, row0, rows - 1, lw, lane) : 0;
+            };
+            int next = step_idx(-2);
+#pragma unroll 1
+            for (int i = -2; i < n_tiles; ++i) {
+                const int now = next;
+                if (i + 1 < n_tiles) next = step_idx(i + 1);
+                const TileInfo t = tile_info(un, max(i, 0), nA);
                 const int stage = kv_cnt % kStages;
-                const bool bulk = t.w == kTile && t.k0 + kTile <= ident;
-                int idx[kPasses];
-                if (!bulk) load_indices(idx, perm, t.k0, (t.w + 15) & ~15, t.w - 1, ltid);
-                if (!(alive = wait_free(bars + 8 * (kBarKVEmpty + stage), ((kv_cnt / kStages) & 1) ^ 1))) break;
-                const uint32_t sK = base + kOffKV + stage * 2 * kTileBytes;
-                const uint32_t bar_kv = bars + 8 * (kBarKVFull + stage);
+                if (i != -1) {
+                    const uint32_t bar = i < 0 ? kBarQEmpty + qb : kBarKVEmpty + stage;
+                    if (!(alive = wait_free(bars + 8 * bar, ((i < 0 ? unit_cnt >> 1 : kv_cnt / kStages) & 1) ^ 1))) break;
+                }
+                const uint32_t dst = base + (i < 0 ? kOffQ + (qb * 2 + i + 2) * kTileBytes : kOffKV + stage * 2 * kTileBytes);
+                const uint32_t bar_full = bars + 8 * (i < 0 ? kBarQFull + qb : kBarKVFull + stage);
+                // (Q tiles are always gathered: fetching them with bulk copies as well measured slower.)
+                const bool bulk = i >= 0 && t.k0 + kTile <= ident;  // (rows behind the tile's own come along)
                 TR_T0(t_cp);
                 if (bulk) {
                     if (ltid == 0) {
-                        mbar_expect_tx(bar_kv, 2 * kTileBytes);
-                        tma_load_2d(sK, &p.tmK, 0, (int)bh + t.k0, bar_kv);
-                        tma_load_2d(sK + kTileBytes, &p.tmV, 0, (int)bh + t.k0, bar_kv);
+                        mbar_expect_tx(bar_full, 2 * kTileBytes);
+                        tma_load_2d(dst, &p.tmK, 0, (int)bh + t.k0, bar_full);
+                        tma_load_2d(dst + kTileBytes, &p.tmV, 0, (int)bh + t.k0, bar_full);
                     }
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_kv);
-                } else {
-                    copy_rows(sK, Kbh, idx, ltid);
-                    copy_rows(sK + kTileBytes, Vbh, idx, ltid);
+                    if (lane == 0) mbar_arrive(bar_full);
+                } else if (i >= 0 || un.rows_of(i + 2) > 0) {
+                    gather_rows(dst, i < 0 ? Qbh : Kbh, i >= 0, v_off, now, i < 0 ? kTile : (t.w + 15) & ~15, lw, lane);
                     TR_ADD(2, t_cp);
-                    TR_T0(t_cs);
-                    commit_and_signal(bar_kv);
-                    TR_ADD(3, t_cs);
+                }
+                if (i == -2) {  // row data for the softmax threads: original position and key range
+                    const uint32_t meta = base + kOffMeta + qb * 3 * kUnitRows * 4;
+#pragma unroll 1
+                    for (int rr = ltid; rr < kUnitRows; rr += kLoadThreads) {
+                        const int half = rr / kTile;
+                        if (rr - half * kTile < un.rows_of(half)) {
+                            const size_t at = bn + un.row0_of(half) + rr - half * kTile;
+                            cp_async4(meta + rr * 4, vp.perm + at);
+                            cp_async4(meta + (kUnitRows + rr) * 4, vp.seg_lo + at);
+                            cp_async4(meta + (2 * kUnitRows + rr) * 4, vp.seg_hi + at);
+                        }
+                    }
+                    continue;
+                }
+                if (!bulk) commit_and_signal(bar_full);
+                if (i < 0) {
+                    ++unit_cnt;
+                    continue;
                 }
                 // The very first tile of the CTA: the other warps are waiting for it, so it (and Q) are
                 // signalled as soon as they have landed, not two tiles later.
@@ -927,7 +923,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
 
 #ifdef MATE_TRACE
     if (lane == 0 && (warp == 0 || warp == 4 || warp == kMmaWarp || warp == kLoadWarp0) &&
-        blockIdx.x < kTraceCtas) {  // MMA: half 0's thread
+        blockIdx.x < kTraceCtas) {  // MMA: half 0's warp
         const int role = warp == 0 ? 0 : warp == 4 ? 1 : warp == kMmaWarp ? 2 : 3;
         long long *o = g_trace + blockIdx.x * 32 + role * 8;
         for (int i = 0; i < 7; ++i) o[i] = tr[i];
@@ -937,15 +933,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tmem, kTmemCols);
-    if (tid == 0) {
-        // the CTA that finishes last puts the scheduling counters back to zero for the next launch
-        // (every CTA has taken its last index by the time it counts itself as finished)
-        __threadfence();
-        if (atomicAdd(p.counters + 1, 1) == (int)gridDim.x - 1) {
-            p.counters[0] = 0;
-            p.counters[1] = 0;
-        }
-    }
 }
 
 SmemAttrOnce g_smem_attr;
@@ -984,14 +971,12 @@ bool make_row_map(CUtensorMap *map, const void *base, size_t rows) {
 
 bool tc_supported(int d, int dtype) { return d == 64 && dtype == MATE_BF16; }
 
-int tc_fwd_ctas_per_sm() { return 1; }
-
 size_t tc_fwd_workspace(const mate_plan_t *plan, int) { return plan->fwd_ws_bytes; }
 
 int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, float scale, void *O,
            float *LSE, void *workspace, unsigned flags, cudaStream_t stream) {
     if (!(scale > 0.f)) return MATE_ERR_UNSUPPORTED;  // the row max is taken before scaling (the caller falls back)
-    if (plan->n_fwd_units == 0) return MATE_OK;
+    if (plan->fwd_grid == 0) return MATE_OK;
     if (g_smem_attr.ensure((const void *)tc_fwd_kernel, (int)kSmemBytes, plan->device) != MATE_OK) return MATE_ERR_CUDA;
     Params p;
     const size_t rows = plan->n_rows();
@@ -1011,7 +996,9 @@ int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.colv = plan->view[1];
     p.head_view = plan->head_view_dev;
     p.units = plan->fwd_units_dev;
-    p.n_units = plan->n_fwd_units;
+    p.cta_off = plan->fwd_cta_off_dev;
+    p.pads = plan->pads_dev;
+    p.n_pads = plan->n_pads;
     p.N = plan->N;
     p.H = plan->H;
     p.tr = plan->rows();
@@ -1019,7 +1006,7 @@ int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.status = plan->status_dev;
     p.counters = plan->fwd_counters_dev;
     p.ws = (uint8_t *)workspace;
-    tc_fwd_kernel<<<plan->n_ctas, kThreads, kSmemBytes, stream>>>(p);
+    tc_fwd_kernel<<<plan->fwd_grid, kThreads, kSmemBytes, stream>>>(p);
     return cudaGetLastError() == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }
 

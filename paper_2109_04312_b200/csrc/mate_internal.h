@@ -11,35 +11,73 @@
 namespace mate {
 
 constexpr int kTile = 128;       // key columns per tile and query rows per half of a unit
-constexpr int kSchedWords = 8;   // scheduling counters in front of the split-unit counters
 constexpr int kUnitRows = 256;   // query rows per unit of the tensor-core kernels (two halves)
 // what the key range of a table row is made of (plan kernel step 4 and its host twin)
 enum { kBoundsOwn = 0, kBoundsBefore = 1, kBoundsAfter = 2 };
 constexpr int kTraceCtas = 256;  // CTAs whose cycle counters a -DMATE_TRACE build keeps
 
-// One unit of work of the tensor-core forward: up to 256 consecutive query rows (view order) of one
-// (example, head) -- half 0 = the first 128 rows, half 1 = the rest -- and the key tiles (128 wide)
-// they visit, in this order:
-//   range A = keys [kA0, kA_end): the prefix block for table rows ([0, P)), a slice of all valid
-//             keys for prefix rows.  Key j counts for every row iff j < kA_end.
-//   range B = keys [kB0, kB_end): the union of the segments the rows belong to (table rows only).
-//             Key j counts for a row iff seg_lo[row] <= j < seg_hi[row]; half h touches only the
-//             tiles that meet [lo[h], hi[h]) (min seg_lo / max seg_hi over its rows).
-// Prefix rows whose key range is long are split along the keys into n_parts units; each writes an
-// un-normalised partial result to the workspace at ws_off (KiB); per group of 32 rows the part
-// that finishes last (counted in counters[kSchedWords + 8 * ctr + row / 32]) combines them.
-struct FwdUnit {
+// One unit of work of the tensor-core kernels: up to 256 consecutive rows (view order) of one (example, head)
+// in two halves of up to 128 -- half 0 = the first n0 rows, half 1 = the n1 rows behind them -- and the
+// column tiles they visit, in this order:
+//   range A = columns [kA0, kA_end) in tiles of 128: the global block for table rows ([0, P)), all valid
+//             positions for rows of the global block.  Column j counts for every row iff j < kA_end.
+//   range B = columns [kB0, kB_end) in tiles of tB <= 128: the union of the key ranges of the rows (table
+//             rows only).  Column j counts for a row iff seg_lo[row] <= j < seg_hi[row]; half h touches only
+//             the tiles that meet [lo[h], hi[h]) (min seg_lo / max seg_hi over its rows).
+// A unit of the forward may be split along its tiles into n_parts units; each writes an un-normalised
+// partial result to the workspace at ws_off (KiB); per group of 32 rows the part that finishes
+// last (counted in counters[8 * ctr + row / 32]) combines them.
+struct alignas(16) FwdUnit {  // (copied as four 16-byte words)
     int32_t b, h;
-    int32_t q0, nq;
+    int32_t q0, rows;          // rows = n0 | n1 << 16; 0 ends a list
     int32_t kA0, kA_end;
     int32_t kB0, kB_end;
     int32_t lo[2], hi[2];
-    int32_t n_parts, part;
+    int32_t tB, parts;         // parts = n_parts | part << 16 (tB: the forward keeps flags above bit 7 on its way)
     int32_t ws_off, ctr;
+
+    __host__ __device__ int rows_of(int half) const { return half ? rows >> 16 : rows & 0xffff; }
+    __host__ __device__ int row0_of(int half) const { return half ? q0 + (rows & 0xffff) : q0; }
+    __host__ __device__ int n_parts() const { return parts & 0xffff; }
+    __host__ __device__ int part() const { return parts >> 16; }
+    __host__ __device__ int tiles_a() const { return kA_end > kA0 ? (kA_end - kA0 + kTile - 1) / kTile : 0; }
+    __host__ __device__ int tiles_b() const { return kB_end > kB0 ? (kB_end - kB0 + tB - 1) / tB : 0; }
 };
 static_assert(sizeof(FwdUnit) == 64, "FwdUnit is read as four 16-byte words");
-// bytes of one partial result: 256 rows x (64 fp32 + running max + row sum)
-constexpr size_t kPartialBytes = (size_t)kUnitRows * (64 + 2) * sizeof(float);
+
+// Tile i of a unit (nA = its tiles of range A): first column and number of columns (<= 128).
+struct TileInfo {
+    int k0, w;
+    bool is_b;
+};
+__host__ __device__ inline TileInfo tile_info(const FwdUnit &u, int i, int nA) {
+    TileInfo t;
+    t.is_b = i >= nA;
+    t.k0 = t.is_b ? u.kB0 + (i - nA) * u.tB : u.kA0 + i * kTile;
+    const int left = (t.is_b ? u.kB_end : u.kA_end) - t.k0, most = t.is_b ? u.tB : kTile;
+    t.w = left < most ? left : most;
+    return t;
+}
+// Columns [c0, c1) of the tile (multiples of 16) needed by a half whose rows' key ranges span [lo, hi);
+// c1 <= c0 when it skips the tile.
+__host__ __device__ inline void half_cols(int lo, int hi, const TileInfo &t, int &c0, int &c1) {
+    c0 = 0;
+    c1 = (t.w + 15) & ~15;
+    if (t.is_b) {
+        const int a = lo > t.k0 ? lo - t.k0 : 0, b = hi < t.k0 + t.w ? hi - t.k0 : t.w;
+        c0 = a & ~15;
+        c1 = a < b ? (b + 15) & ~15 : c0;
+    }
+}
+// bytes of one partial result: 256 rows x (64 fp32 + base, row sum, two unused)
+constexpr size_t kPartialBytes = (size_t)kUnitRows * (64 + 4) * sizeof(float);
+
+// Up to kPadRows padding rows (view positions t0 ..) of one (example, head); zeroed by the forward
+// kernel before its first unit.
+constexpr int kPadRows = 64;
+struct PadChunk {
+    int32_t b, h, t0, n;
+};
 
 // Where the rows of example b, head h start in the caller's tensors (in rows of d elements), and how
 // far an example reaches.  Padded layout [B, H, N, d]: (b H + h) N, every example N positions long.
@@ -111,18 +149,22 @@ struct mate_plan_s {
     int32_t *status_dev = nullptr;       // device status word(s): [0] = id validation, [1] = kernel timeouts
     void *dev_block = nullptr;           // one allocation backing all device arrays above
     void *work_block = nullptr;          // one allocation backing the work-lists below
-    // tensor-core forward work-list: units by decreasing cost; the CTAs of the persistent kernel
-    // take them in this order through a shared counter
+    // tensor-core forward work-list: the units of CTA c are [fwd_cta_off[c], fwd_cta_off[c + 1])
     mate::FwdUnit *fwd_units_dev = nullptr;
-    // [kSchedWords + 8 * n_fwd_slots]: [0] next unit, [1] CTAs finished, then the arrival counters of
-    // the split units.  Zero between launches (the kernel resets what it counted), which is why
-    // two forward calls on one plan must not overlap on the GPU.
+    int32_t *fwd_cta_off_dev = nullptr;
+    mate::PadChunk *pads_dev = nullptr;
+    // [8 * n_fwd_slots]: arrival counters of the split units.  Zero between launches (the kernel resets
+    // what it counted), which is why two forward calls on one plan must not overlap on the GPU.
     int32_t *fwd_counters_dev = nullptr;
     int n_fwd_units = 0;
-    int n_fwd_slots = 0;                  // split units (prefix rows cut along the keys)
+    int n_pads = 0;
+    int fwd_grid = 0;                     // CTAs of a forward launch
+    int n_fwd_slots = 0;                  // split units
     int n_ctas = 0;                       // CTAs of the persistent kernel (SMs of the plan's device)
     size_t fwd_ws_bytes = 0;              // partial results of the split units
-    std::vector<mate::FwdUnit> fwd_units; // host copy
+    std::vector<mate::FwdUnit> fwd_units; // host copies
+    std::vector<int32_t> fwd_cta_off;
+    std::vector<mate::PadChunk> pads;
     // tensor-core backward work-list: the same units with no prefix unit split
     mate::FwdUnit *bwd_units_dev = nullptr;
     int n_bwd_units = 0;
@@ -175,7 +217,6 @@ int simt_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *
 
 // tensor-core kernels (mate_fwd_tc.cu / mate_bwd_tc.cu)
 bool tc_supported(int d, int dtype);
-int tc_fwd_ctas_per_sm();  // CTAs of the forward kernel per SM (the grid is this times the plan's SM count)
 size_t tc_fwd_workspace(const mate_plan_t *plan, int d);
 size_t tc_bwd_workspace(const mate_plan_t *plan);
 int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, const void *O,

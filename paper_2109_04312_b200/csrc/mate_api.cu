@@ -225,7 +225,7 @@ void proto_units(const RowRanges &rr, bool pairs, std::vector<FwdUnit> &proto) {
     }
 }
 
-// Backward: no unit is split; its work items are the halves of the units, once per side.
+// Backward: single halves, none split; its work items are the units, once per side.
 void make_bwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges) {
     std::vector<std::pair<int64_t, FwdUnit>> all;
     std::vector<FwdUnit> proto;
@@ -234,20 +234,11 @@ void make_bwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges) {
         if (pl->view[v].n_heads == 0) continue;
         for (int b = 0; b < pl->B; ++b) {
             const RowRanges &rr = ranges[(size_t)v * pl->B + b];
-            proto_units(rr, true, proto);
-            for (int q0 = pl->n_valid[b]; q0 < pl->N; q0 += 2 * kTile) {  // padding rows: no key at all
-                FwdUnit u{};
-                u.q0 = q0;
-                u.rows = std::min(kTile, pl->N - q0) | std::min(kTile, std::max(pl->N - q0 - kTile, 0)) << 16;
-                u.tB = kTile;
-                proto.push_back(u);
-            }
+            proto_units(rr, false, proto);
             for (FwdUnit &u : proto) {
                 int64_t cost = 0;
-                for (int h = 0; h < 2; ++h) {
-                    half_tile_clks(u, h, rr, clk);
-                    for (int c : clk) cost += c;
-                }
+                half_tile_clks(u, 0, rr, clk);
+                for (int c : clk) cost += c;
                 u.b = b;
                 for (int h = 0; h < pl->H; ++h) {
                     if (pl->head_view[h] != v) continue;
@@ -265,6 +256,7 @@ void make_bwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges) {
     pl->bwd_units.clear();
     for (const auto &uc : all) pl->bwd_units.push_back(uc.second);
     pl->n_bwd_units = (int)pl->bwd_units.size();
+    pl->bwd_grid = std::min(std::max(pl->n_ctas, 1), std::max(2 * pl->n_bwd_units, pl->n_pads));
 }
 
 // Tiles [i0, i1) of a unit as a unit of its own.
@@ -467,8 +459,8 @@ int build_units(mate_plan_t *pl, const std::vector<std::vector<int32_t>> &seg_of
     std::vector<RowRanges> ranges((size_t)2 * pl->B);
     for (int v = 0; v < 2; ++v)
         for (int b = 0; b < pl->B && pl->view[v].n_heads > 0; ++b) fill_ranges(pl, seg_off_host, v, b, ranges[(size_t)v * pl->B + b]);
-    make_bwd_units(pl, ranges);
     make_fwd_units(pl, ranges);
+    make_bwd_units(pl, ranges);
 
     // device copy: units, CTA offsets, padding, arrival counters (zeroed once; the kernel resets them)
     Carver c(nullptr);
@@ -926,8 +918,8 @@ int mate_attn_fwd(const mate_plan_t *plan, const void *Q, const void *K, const v
 
 static int bwd_pass(const mate_plan_t *plan, bool use_tc, const void *Q, const void *K, const void *V, const void *O,
                     const float *LSE, const void *dO, int d, int dtype, float scale, void *dQ, void *dK, void *dV, void *ws,
-                    cudaStream_t st) {
-    if (use_tc) return mate::tc_bwd(plan, Q, K, V, O, LSE, dO, scale, dQ, dK, dV, ws, st);
+                    int pass, cudaStream_t st) {
+    if (use_tc) return mate::tc_bwd(plan, Q, K, V, O, LSE, dO, scale, dQ, dK, dV, ws, pass, st);
     return mate::simt_bwd(plan, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, ws, st);
 }
 
@@ -949,7 +941,7 @@ int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const v
     if (!workspace || workspace_bytes < need) return MATE_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MATE_ERR_ALIGNMENT;
     cudaStream_t st = (cudaStream_t)stream;
-    rc = bwd_pass(plan, use_tc, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, workspace, st);
+    rc = bwd_pass(plan, use_tc, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, workspace, 0, st);
     if (rc != MATE_OK || !plan->sub[0]) return rc;
     // Row-or-column pattern.  With the final O and LSE every pass computes the gradient of its own
     // pairs.  The two column passes are each other's transpose (keys in front of / behind the own
@@ -961,7 +953,7 @@ int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const v
     void *g[2][3];
     for (int s = 0; s < 2; ++s) {
         for (int i = 0; i < 3; ++i, w += g_bytes) g[s][i] = w;
-        rc = bwd_pass(plan->sub[s], use_tc, Q, K, V, O, LSE, dO, d, dtype, scale, g[s][0], g[s][1], g[s][2], workspace, st);
+        rc = bwd_pass(plan->sub[s], use_tc, Q, K, V, O, LSE, dO, d, dtype, scale, g[s][0], g[s][1], g[s][2], workspace, 1 + s, st);
         if (rc != MATE_OK) return rc;
     }
     void *outs[3] = {dQ, dK, dV};

@@ -43,6 +43,7 @@
 
 #include "mate_internal.h"
 #include "sm100_ptx.cuh"
+#include "tc_tiles.cuh"
 
 namespace mate {
 
@@ -71,8 +72,6 @@ constexpr int kRegsSoftmax = 200, kRegsOther = 56;
 constexpr uint32_t kApart = 1000;            // clocks between the exponentials of the two halves
 
 constexpr int kSchedDepth = 4;
-constexpr int kRowBytes = 128;                 // 64 bf16
-constexpr int kTileBytes = kTile * kRowBytes;  // 16 KB: 128 rows
 constexpr uint32_t kOffQ = 0;                                // [2 buffers][2 halves] x 16 KB
 constexpr uint32_t kOffKV = 4 * kTileBytes;                  // [kStages] x (K 16 KB, V 16 KB)
 constexpr uint32_t kOffMeta = kOffKV + kStages * 2 * kTileBytes;    // [2 buffers] x (perm, seg_lo, seg_hi) of 256 rows
@@ -128,32 +127,6 @@ struct Params {
     int32_t *counters;  // arrivals at the split units, 8 per unit
     uint8_t *ws;
 };
-
-// The loaders copy a tile of up to 128 rows (128 B each), warp w of the four the rows 32 w .. 32 w + 31.
-// Row rr of the tile comes from view position row0 + min(rr, clamp).  A lane looks up the original
-// position of one row (coalesced, one latency for the whole tile, and cheap enough to be done a tile
-// ahead); the copies then run four rows at a time, eight lanes per row, with the positions handed
-// around by shuffle.
-__device__ __forceinline__ int fetch_idx(const int32_t *perm, int row0, int clamp, int lw, int lane) {
-    const int t = row0 + min(32 * lw + lane, clamp);
-    return perm ? __ldg(perm + t) : t;  // no order given: the tensors are in view order
-}
-// Rows [0, n_rows) of one tensor, or of two (`pair`; b_off: bytes from the first one's rows to the second's)
-// -> tiles at s_a and 16 KB behind it, 128-byte swizzle.
-__device__ __forceinline__ void gather_rows(uint32_t s_a, const uint8_t *a_bh, bool pair, int64_t b_off, int idx, int n_rows,
-                                            int lw, int lane) {
-    if (32 * lw >= n_rows) return;  // (rows past n_rows inside a group of 32 repeat a row that exists)
-    const int sub = lane >> 3;      // row of the group of four
-    a_bh += (lane & 7) * 16;
-    const uint32_t d = s_a + (32 * lw + sub) * kRowBytes + (((lane & 7) ^ sub) << 4);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint8_t *src = a_bh + (size_t)(uint32_t)__shfl_sync(0xffffffffu, idx, 4 * i + sub) * kRowBytes;
-        const uint32_t dst = (d ^ ((i & 1) << 6)) + 4 * i * kRowBytes;
-        cp_async16(dst, src);
-        if (pair) cp_async16(dst + kTileBytes, src + b_off);
-    }
-}
 
 // A chunk is 32 scores of one row (tile-local columns cb .. cb + 31).  A column c counts for the row
 // iff r_lo <= c < r_hi; the scores of the other columns are replaced by -inf, which the row max
@@ -953,6 +926,8 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
+}  // namespace
+
 // Map over a [rows, 64] bf16 matrix (row = 128 bytes): boxes of 128 rows, written to shared memory in
 // the 128-byte swizzle the tensor-core descriptors expect (16-byte chunk index XOR row & 7).
 bool make_row_map(CUtensorMap *map, const void *base, size_t rows) {
@@ -966,8 +941,6 @@ bool make_row_map(CUtensorMap *map, const void *base, size_t rows) {
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-
-}  // namespace
 
 bool tc_supported(int d, int dtype) { return d == 64 && dtype == MATE_BF16; }
 

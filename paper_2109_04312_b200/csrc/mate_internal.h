@@ -165,9 +165,10 @@ struct mate_plan_s {
     std::vector<mate::FwdUnit> fwd_units; // host copies
     std::vector<int32_t> fwd_cta_off;
     std::vector<mate::PadChunk> pads;
-    // tensor-core backward work-list: the same units with no prefix unit split
+    // tensor-core backward work-list: single halves by decreasing cost; every one is done once per side
     mate::FwdUnit *bwd_units_dev = nullptr;
     int n_bwd_units = 0;
+    int bwd_grid = 0;                     // CTAs of a backward launch
     std::vector<mate::FwdUnit> bwd_units;
 };
 
@@ -190,6 +191,23 @@ struct SmemAttrOnce {
         return MATE_OK;
     }
 };
+
+// Launches a kernel that may start before the one in front of it in the stream is complete; it waits for that
+// itself (griddepcontrol.wait) before it touches what that one writes.
+template <typename Params>
+cudaError_t launch_after(void (*kernel)(const Params), int grid, int threads, size_t smem, cudaStream_t stream, const Params &p) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, p);
+}
 
 // plan kernels (mate_plan_kernels.cu)
 cudaError_t launch_plan_kernels(const int32_t *row_ids, const int32_t *col_ids, int B, int N,
@@ -220,7 +238,7 @@ bool tc_supported(int d, int dtype);
 size_t tc_fwd_workspace(const mate_plan_t *plan, int d);
 size_t tc_bwd_workspace(const mate_plan_t *plan);
 int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, const void *O,
-           const float *LSE, const void *dO, float scale, void *dQ, void *dK, void *dV, void *workspace,
+           const float *LSE, const void *dO, float scale, void *dQ, void *dK, void *dV, void *workspace, int pass,
            cudaStream_t stream);
 int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, float scale, void *O,
            float *LSE, void *workspace, unsigned flags, cudaStream_t stream);

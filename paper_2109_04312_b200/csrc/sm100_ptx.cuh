@@ -305,6 +305,10 @@ template <int kRegs>
 __device__ __forceinline__ void reg_dealloc() {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs));
 }
+// Programmatic dependent launch: lets the next kernel of the stream start (if it was launched so) / waits
+// until the kernel before this one is complete and its writes are visible.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // True in exactly one lane of the (converged) warp.  Code that one lane issues on behalf of the warp
 // is written as `if (elect_one())` inside warp-uniform control flow, so that its operands stay
 // warp-uniform values.

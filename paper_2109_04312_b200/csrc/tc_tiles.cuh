@@ -1,0 +1,43 @@
+// What the tensor-core forward and backward share: tiles of 128 rows of 64 bf16 in shared memory (128-byte
+// swizzle), gathered by view-order position or fetched whole by a bulk tensor copy.
+#pragma once
+#include <cuda.h>
+
+#include "mate_internal.h"
+#include "sm100_ptx.cuh"
+
+namespace mate {
+
+constexpr int kRowBytes = 128;                 // 64 bf16
+constexpr int kTileBytes = kTile * kRowBytes;  // 16 KB: 128 rows
+
+// Tensor map over a [rows, 64] bf16 matrix in boxes of 128 rows (false: no tensor maps to be had).
+bool make_row_map(CUtensorMap *map, const void *base, size_t rows);
+
+// The loaders copy a tile of up to 128 rows (128 B each), warp w of the four the rows 32 w .. 32 w + 31.
+// Row rr of the tile comes from view position row0 + min(rr, clamp).  A lane looks up the original
+// position of one row (coalesced, one latency for the whole tile, and cheap enough to be done a tile
+// ahead); the copies then run four rows at a time, eight lanes per row, with the positions handed
+// around by shuffle.
+__device__ __forceinline__ int fetch_idx(const int32_t *perm, int row0, int clamp, int lw, int lane) {
+    const int t = row0 + min(32 * lw + lane, clamp);
+    return perm ? __ldg(perm + t) : t;  // no order given: the tensors are in view order
+}
+// Rows [0, n_rows) of one tensor, or of two (`pair`; b_off: bytes from the first one's rows to the second's)
+// -> tiles at s_a and 16 KB behind it, 128-byte swizzle.
+__device__ __forceinline__ void gather_rows(uint32_t s_a, const uint8_t *a_bh, bool pair, int64_t b_off, int idx, int n_rows,
+                                            int lw, int lane) {
+    if (32 * lw >= n_rows) return;  // (rows past n_rows inside a group of 32 repeat a row that exists)
+    const int sub = lane >> 3;      // row of the group of four
+    a_bh += (lane & 7) * 16;
+    const uint32_t d = s_a + (32 * lw + sub) * kRowBytes + (((lane & 7) ^ sub) << 4);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint8_t *src = a_bh + (size_t)(uint32_t)__shfl_sync(0xffffffffu, idx, 4 * i + sub) * kRowBytes;
+        const uint32_t dst = (d ^ ((i & 1) << 6)) + 4 * i * kRowBytes;
+        ptx::cp_async16(dst, src);
+        if (pair) ptx::cp_async16(dst + kTileBytes, src + b_off);
+    }
+}
+
+}  // namespace mate

@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <new>
 
 #include "mate_internal.h"
@@ -31,26 +32,37 @@ struct Carver {
     }
 };
 
-void carve(mate_plan_t *pl, char *base, size_t *total) {
+// What is copied in before the plan kernel (prefix, global, head_view) and out behind it (segment offsets,
+// numbers of valid positions, status) lies together, so that each is one copy.
+struct PlanLayout {
+    size_t total, in_off, in_bytes, out_off, out_bytes;
+};
+PlanLayout carve(mate_plan_t *pl, char *base) {
     Carver c(base);
+    PlanLayout L;
     const size_t BN = (size_t)pl->B * pl->N;
     for (int v = 0; v < 2; ++v) {
         ViewPlan &vp = pl->view[v];
-        const size_t S = (size_t)pl->B * (vp.max_id + 2);
         vp.perm = c.take<int32_t>(BN);
         vp.inv_perm = c.take<int32_t>(BN);
         vp.seg_lo = c.take<int32_t>(BN);
         vp.seg_hi = c.take<int32_t>(BN);
-        vp.seg_off = c.take<int32_t>(S);
-        vp.cursor = c.take<int32_t>(S);
+        vp.cursor = c.take<int32_t>((size_t)pl->B * (vp.max_id + 2));
         vp.ident = c.take<int32_t>(pl->B);
     }
-    pl->n_valid_dev = c.take<int32_t>(pl->B);
+    L.in_off = c.off = align_up(c.off, 256);
     pl->prefix_dev = c.take<int32_t>(pl->B);
     pl->global_dev = c.take<int32_t>(pl->B);
-    pl->status_dev = c.take<int32_t>(4);
     pl->head_view_dev = c.take<uint8_t>(pl->H);
-    *total = align_up(c.off, 256);
+    c.off = align_up(c.off, 256);
+    pl->status_dev = c.take<int32_t>(4);  // in both: comes in as zeros
+    L.in_bytes = c.off - L.in_off;
+    L.out_off = c.off - 4 * sizeof(int32_t);
+    pl->n_valid_dev = c.take<int32_t>(pl->B);
+    for (int v = 0; v < 2; ++v) pl->view[v].seg_off = c.take<int32_t>((size_t)pl->B * (pl->view[v].max_id + 2));
+    L.out_bytes = c.off - L.out_off;
+    L.total = align_up(c.off, 256);
+    return L;
 }
 
 // Column range of one table row (view position t) of one (example, view): its segment, clipped to the
@@ -94,9 +106,9 @@ struct RowRanges {
     std::vector<int32_t> lo, hi;
 };
 
-void fill_ranges(const mate_plan_t *pl, const std::vector<std::vector<int32_t>> &seg_off_host, int v, int b, RowRanges &rr) {
+void fill_ranges(const mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], int v, int b, RowRanges &rr) {
     const int S = pl->view[v].max_id + 2;
-    const int32_t *so = seg_off_host[v].data() + (size_t)b * S;
+    const int32_t *so = seg_off_host[v] + (size_t)b * S;
     const RowBounds rb{so, S, std::min(pl->global[b], pl->n_valid[b]), pl->radius, pl->bounds_mode, pl->group};
     rr.P = rb.P;
     rr.nv = pl->n_valid[b];
@@ -454,7 +466,7 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges) {
                 pl->fwd_ws_bytes, pl->n_pads);
 }
 
-int build_units(mate_plan_t *pl, const std::vector<std::vector<int32_t>> &seg_off_host) {
+int build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], cudaStream_t st) {
     static_assert(mate::kPartialBytes % 1024 == 0, "ws_off counts KiB");
     std::vector<RowRanges> ranges((size_t)2 * pl->B);
     for (int v = 0; v < 2; ++v)
@@ -462,24 +474,35 @@ int build_units(mate_plan_t *pl, const std::vector<std::vector<int32_t>> &seg_of
     make_fwd_units(pl, ranges);
     make_bwd_units(pl, ranges);
 
-    // device copy: units, CTA offsets, padding, arrival counters (zeroed once; the kernel resets them)
-    Carver c(nullptr);
-    c.take<FwdUnit>(pl->n_fwd_units);
-    c.take<FwdUnit>(pl->n_bwd_units);
-    c.take<int32_t>(pl->fwd_cta_off.size());
-    c.take<mate::PadChunk>(pl->n_pads);
-    c.take<int32_t>(8 * (size_t)pl->n_fwd_slots);
-    const size_t bytes = align_up(c.off, 256);
-    if (cudaMalloc(&pl->work_block, bytes) != cudaSuccess) {
-        cudaGetLastError();
+    // device copy, in one piece: units, CTA offsets, padding, arrival counters (zeros; the kernel resets them)
+    const auto lay_out = [pl](char *base) {
+        Carver c(base);
+        pl->fwd_units_dev = c.take<FwdUnit>(pl->n_fwd_units);
+        pl->bwd_units_dev = c.take<FwdUnit>(pl->n_bwd_units);
+        pl->fwd_cta_off_dev = c.take<int32_t>(pl->fwd_cta_off.size());
+        pl->pads_dev = c.take<mate::PadChunk>(pl->n_pads);
+        pl->fwd_counters_dev = c.take<int32_t>(8 * (size_t)pl->n_fwd_slots);
+        return align_up(c.off, 256);
+    };
+    const size_t bytes = lay_out(nullptr);
+    mate::Staging host;
+    if (!mate::staging_take(bytes, pl->device, &host)) return MATE_ERR_NOMEM;
+    if (!mate::pool_take(bytes, st, pl->device, &pl->work_block)) {
+        mate::staging_give(host, st);
         return MATE_ERR_NOMEM;
     }
-    Carver d((char *)pl->work_block);
-    pl->fwd_units_dev = d.take<FwdUnit>(pl->n_fwd_units);
-    pl->bwd_units_dev = d.take<FwdUnit>(pl->n_bwd_units);
-    pl->fwd_cta_off_dev = d.take<int32_t>(pl->fwd_cta_off.size());
-    pl->pads_dev = d.take<mate::PadChunk>(pl->n_pads);
-    pl->fwd_counters_dev = d.take<int32_t>(8 * (size_t)pl->n_fwd_slots);
+    lay_out((char *)host.ptr);
+    std::copy(pl->fwd_units.begin(), pl->fwd_units.end(), pl->fwd_units_dev);
+    std::copy(pl->bwd_units.begin(), pl->bwd_units.end(), pl->bwd_units_dev);
+    std::copy(pl->fwd_cta_off.begin(), pl->fwd_cta_off.end(), pl->fwd_cta_off_dev);
+    std::copy(pl->pads.begin(), pl->pads.end(), pl->pads_dev);
+    std::fill_n(pl->fwd_counters_dev, 8 * (size_t)pl->n_fwd_slots, 0);
+    lay_out((char *)pl->work_block.ptr);
+    bool ok = cudaMemcpyAsync(pl->work_block.ptr, host.ptr, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    mate::staging_give(host, st);
+    ok = ok && cudaEventCreateWithFlags(&pl->ready, cudaEventDisableTiming) == cudaSuccess &&
+         cudaEventRecord(pl->ready, st) == cudaSuccess;
+    if (!ok) return MATE_ERR_CUDA;
     return MATE_OK;
 }
 
@@ -505,10 +528,11 @@ const char *mate_status_string(int status) {
 int mate_plan_destroy(mate_plan_t *plan) {
     if (!plan) return MATE_OK;
     for (int s = 0; s < 2; ++s) mate_plan_destroy(plan->sub[s]);
-    if (plan->pair_ids_dev) cudaFree(plan->pair_ids_dev);
-    if (plan->tok_off_dev) cudaFree(plan->tok_off_dev);
-    if (plan->dev_block) cudaFree(plan->dev_block);
-    if (plan->work_block) cudaFree(plan->work_block);
+    const uint64_t stream = plan->elsewhere ? 0 : plan->stream;
+    mate::pool_give(plan->extra_block, stream);
+    mate::pool_give(plan->dev_block, stream);
+    mate::pool_give(plan->work_block, stream);
+    if (plan->ready) cudaEventDestroy(plan->ready);
     delete plan;
     return MATE_OK;
 }
@@ -573,24 +597,32 @@ int mate_plan_packed(const int32_t *row_ids, const int32_t *col_ids, int B, cons
     }
     const int T = cu_seqlens[B];
     cudaStream_t st = (cudaStream_t)stream;
-    int32_t *off_dev = nullptr, *ids = nullptr;
     const size_t BN = (size_t)B * n_max;
-    if (cudaMalloc(&off_dev, sizeof(int32_t) * 2 * B) != cudaSuccess || cudaMalloc(&ids, sizeof(int32_t) * 2 * BN) != cudaSuccess) {
-        cudaGetLastError();
-        if (off_dev) cudaFree(off_dev);
-        return MATE_ERR_NOMEM;
-    }
-    bool ok = cudaMemcpyAsync(off_dev, off_len.data(), sizeof(int32_t) * 2 * B, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    ok = ok && mate::launch_unpack_ids(row_ids, col_ids, B, n_max, off_dev, off_dev + B, ids, ids + BN, st) == cudaSuccess;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return MATE_ERR_CUDA;
+    mate::Block offs, ids;
+    mate::Staging host;
+    bool ok = mate::staging_take(sizeof(int32_t) * 2 * B, dev, &host) && mate::pool_take(sizeof(int32_t) * 2 * B, st, dev, &offs) &&
+              mate::pool_take(sizeof(int32_t) * 2 * BN, st, dev, &ids);
+    int rc = ok ? MATE_OK : MATE_ERR_NOMEM;
     mate_plan_t *pl = nullptr;
-    int rc = ok ? build_plan(ids, ids + BN, B, n_max, prefix_len, nullptr, head_view, H, max_row_id, max_col_id, 0,
+    const uint64_t id = mate::stream_id(st);
+    int32_t *off_dev = (int32_t *)offs.ptr, *ids_dev = (int32_t *)ids.ptr;
+    if (ok) {
+        std::copy(off_len.begin(), off_len.end(), (int32_t *)host.ptr);
+        ok = cudaMemcpyAsync(off_dev, host.ptr, sizeof(int32_t) * 2 * B, cudaMemcpyHostToDevice, st) == cudaSuccess &&
+             mate::launch_unpack_ids(row_ids, col_ids, B, n_max, off_dev, off_dev + B, ids_dev, ids_dev + BN, st) == cudaSuccess;
+        rc = ok ? build_plan(ids_dev, ids_dev + BN, B, n_max, prefix_len, nullptr, head_view, H, max_row_id, max_col_id, 0,
                              mate::kBoundsOwn, 1, stream, &pl)
                 : MATE_ERR_CUDA;
-    cudaFree(ids);  // build_plan has waited for its kernels
+    }
+    mate::staging_give(host, st);
+    mate::pool_give(ids, id);
     if (rc != MATE_OK) {
-        cudaFree(off_dev);
+        mate::pool_give(offs, id);
         return rc;
     }
+    pl->extra_block = offs;
     pl->T = T;
     pl->tok_off_dev = off_dev;
     pl->len_dev = off_dev + B;
@@ -618,7 +650,8 @@ int mate_plan_sat(const int32_t *row_ids, const int32_t *col_ids, int B, int N, 
     if (rc != MATE_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     const int n_row_ids = max_row_id + 1, max_pair = n_row_ids * (max_col_id + 1) - 1;
-    bool ok = cudaMalloc(&pl->pair_ids_dev, sizeof(int32_t) * (size_t)B * N) == cudaSuccess;
+    bool ok = mate::pool_take(sizeof(int32_t) * (size_t)B * N, st, pl->device, &pl->extra_block);
+    pl->pair_ids_dev = (int32_t *)pl->extra_block.ptr;
     ok = ok && mate::launch_pair_ids(row_ids, col_ids, B, N, pl->prefix_dev, n_row_ids, pl->pair_ids_dev, st) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -677,45 +710,38 @@ static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int
         }
         pl->device = dev;
     }
-    size_t total = 0;
-    carve(pl, nullptr, &total);
-    if (cudaMalloc(&pl->dev_block, total) != cudaSuccess) {
-        cudaGetLastError();
-        delete pl;
+    pl->stream = mate::stream_id(st);
+    if (pl->stream == 0) pl->elsewhere = true;
+    const PlanLayout L = carve(pl, nullptr);
+    mate::Staging host;
+    if (!mate::staging_take(std::max(L.in_bytes, L.out_bytes), pl->device, &host) ||
+        !mate::pool_take(L.total, st, pl->device, &pl->dev_block)) {
+        mate::staging_give(host, st);
+        mate_plan_destroy(pl);
         return MATE_ERR_NOMEM;
     }
-    carve(pl, (char *)pl->dev_block, &total);
-
-    int rc = MATE_OK;
-    int32_t status_host[4] = {0, 0, 0, 0};
-    std::vector<std::vector<int32_t>> seg_off_host(2);
-    pl->n_valid.resize(B);
-    bool ok = cudaMemsetAsync(pl->status_dev, 0, 4 * sizeof(int32_t), st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(pl->head_view_dev, pl->head_view.data(), H, cudaMemcpyHostToDevice,
-                               st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(pl->prefix_dev, pl->prefix.data(), B * sizeof(int32_t), cudaMemcpyHostToDevice,
-                               st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(pl->global_dev, pl->global.data(), B * sizeof(int32_t), cudaMemcpyHostToDevice,
-                               st) == cudaSuccess;
-    ok = ok && mate::launch_plan_kernels(row_ids, col_ids, B, N, pl->prefix_dev, pl->global_dev, radius, bounds_mode, pl->group, pl->view[0], pl->view[1],
-                                         pl->n_valid_dev, pl->status_dev, st) == cudaSuccess;
-    for (int v = 0; v < 2 && ok; ++v) {
-        seg_off_host[v].resize((size_t)B * (pl->view[v].max_id + 2));
-        ok = cudaMemcpyAsync(seg_off_host[v].data(), pl->view[v].seg_off,
-                             seg_off_host[v].size() * sizeof(int32_t), cudaMemcpyDeviceToHost,
-                             st) == cudaSuccess;
-    }
-    ok = ok && cudaMemcpyAsync(pl->n_valid.data(), pl->n_valid_dev, B * sizeof(int32_t),
-                               cudaMemcpyDeviceToHost, st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(status_host, pl->status_dev, sizeof(status_host),
-                               cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    char *dev_base = (char *)pl->dev_block.ptr, *host_base = (char *)host.ptr;
+    carve(pl, dev_base);
+    const auto in_host = [&](const void *dev) { return host_base + ((const char *)dev - dev_base - L.in_off); };
+    memset(host_base, 0, L.in_bytes);
+    memcpy(in_host(pl->prefix_dev), pl->prefix.data(), B * sizeof(int32_t));
+    memcpy(in_host(pl->global_dev), pl->global.data(), B * sizeof(int32_t));
+    memcpy(in_host(pl->head_view_dev), pl->head_view.data(), H);
+    bool ok = cudaMemcpyAsync(dev_base + L.in_off, host_base, L.in_bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    ok = ok && mate::launch_plan_kernels(row_ids, col_ids, B, N, pl->prefix_dev, pl->global_dev, radius, bounds_mode, pl->group,
+                                         pl->view[0], pl->view[1], pl->n_valid_dev, pl->status_dev, st) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(host_base, dev_base + L.out_off, L.out_bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess;
     ok = ok && cudaStreamSynchronize(st) == cudaSuccess;
-    if (!ok) rc = MATE_ERR_CUDA;
-    if (rc == MATE_OK && status_host[0] != 0) rc = MATE_ERR_INVALID_ARG;
+    int rc = ok ? MATE_OK : MATE_ERR_CUDA;
+    const auto out_host = [&](const void *dev) { return (const int32_t *)(host_base + ((const char *)dev - dev_base - L.out_off)); };
+    if (rc == MATE_OK && out_host(pl->status_dev)[0] != 0) rc = MATE_ERR_INVALID_ARG;
     if (rc != MATE_OK) {
+        mate::staging_give(host, st);
         mate_plan_destroy(pl);
         return rc;
     }
+    pl->n_valid.assign(out_host(pl->n_valid_dev), out_host(pl->n_valid_dev) + B);
+    const int32_t *seg_off_host[2] = {out_host(pl->view[0].seg_off), out_host(pl->view[1].seg_off)};
 
     // unmasked pairs per (example, view): P * n_valid + sum_s L_s (L_s + P); a bucketed plan counts,
     // row by row, the prefix and the clipped part of the segment
@@ -723,7 +749,7 @@ static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int
     for (int v = 0; v < 2; ++v) {
         const int S = pl->view[v].max_id + 2;
         for (int b = 0; b < B; ++b) {
-            const int32_t *so = seg_off_host[v].data() + (size_t)b * S;
+            const int32_t *so = seg_off_host[v] + (size_t)b * S;
             const int P = std::min(pl->global[b], pl->n_valid[b]);
             int64_t c = (int64_t)P * pl->n_valid[b];
             if (radius > 0 || pl->bounds_mode != mate::kBoundsOwn || P != pl->prefix[b]) {
@@ -739,28 +765,11 @@ static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int
         }
     }
 
-    rc = build_units(pl, seg_off_host);
+    rc = build_units(pl, seg_off_host, st);
+    mate::staging_give(host, st);
     if (rc != MATE_OK) {
         mate_plan_destroy(pl);
         return rc;
-    }
-    bool up = cudaMemcpyAsync(pl->fwd_cta_off_dev, pl->fwd_cta_off.data(), sizeof(int32_t) * pl->fwd_cta_off.size(),
-                              cudaMemcpyHostToDevice, st) == cudaSuccess;
-    if (pl->n_fwd_slots > 0)
-        up = up && cudaMemsetAsync(pl->fwd_counters_dev, 0, sizeof(int32_t) * 8 * (size_t)pl->n_fwd_slots, st) == cudaSuccess;
-    if (pl->n_pads > 0)
-        up = up && cudaMemcpyAsync(pl->pads_dev, pl->pads.data(), sizeof(mate::PadChunk) * pl->n_pads, cudaMemcpyHostToDevice,
-                                   st) == cudaSuccess;
-    if (pl->n_fwd_units > 0)
-        up = up && cudaMemcpyAsync(pl->fwd_units_dev, pl->fwd_units.data(), sizeof(FwdUnit) * pl->n_fwd_units,
-                                   cudaMemcpyHostToDevice, st) == cudaSuccess;
-    if (pl->n_bwd_units > 0)
-        up = up && cudaMemcpyAsync(pl->bwd_units_dev, pl->bwd_units.data(), sizeof(FwdUnit) * pl->n_bwd_units,
-                                   cudaMemcpyHostToDevice, st) == cudaSuccess;
-    up = up && cudaStreamSynchronize(st) == cudaSuccess;
-    if (!up) {
-        mate_plan_destroy(pl);
-        return MATE_ERR_CUDA;
     }
     *out = pl;
     return MATE_OK;
@@ -800,6 +809,7 @@ int mate_plan_status(const mate_plan_t *plan, void *stream) {
             if (rc != MATE_OK) return rc;
         }
     cudaStream_t st = (cudaStream_t)stream;
+    if (mate::use_plan(plan, st) != cudaSuccess) return MATE_ERR_CUDA;
     int32_t s[4] = {0, 0, 0, 0};
     if (cudaMemcpyAsync(s, plan->status_dev, sizeof(s), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaMemsetAsync(plan->status_dev + 1, 0, 2 * sizeof(int32_t), st) != cudaSuccess ||
@@ -870,6 +880,13 @@ int mate_attn_workspace_bytes(const mate_plan_t *plan, int d, int dtype, unsigne
     return MATE_OK;
 }
 
+static cudaError_t use_plans(const mate_plan_t *plan, cudaStream_t st) {
+    cudaError_t rc = mate::use_plan(plan, st);
+    for (int s = 0; s < 2 && rc == cudaSuccess; ++s)
+        if (plan->sub[s]) rc = mate::use_plan(plan->sub[s], st);
+    return rc;
+}
+
 static int fwd_pass(const mate_plan_t *plan, bool use_tc, const void *Q, const void *K, const void *V, int d, int dtype,
                     float scale, void *O, float *LSE, void *ws, unsigned flags, cudaStream_t st) {
     if (use_tc) return mate::tc_fwd(plan, Q, K, V, scale, O, LSE, ws, flags, st);
@@ -897,6 +914,7 @@ int mate_attn_fwd(const mate_plan_t *plan, const void *Q, const void *K, const v
     if (need > 0 && (!workspace || workspace_bytes < need)) return MATE_ERR_WORKSPACE;
     if (need > 0 && (reinterpret_cast<uintptr_t>(workspace) & 255u)) return MATE_ERR_ALIGNMENT;
     if ((flags & MATE_FLAG_VIEW_ORDER) && (plan->sub[0] || plan->T)) return MATE_ERR_UNSUPPORTED;
+    if (use_plans(plan, st) != cudaSuccess) return MATE_ERR_CUDA;
     rc = fwd_pass(plan, use_tc, Q, K, V, d, dtype, scale, O, LSE, workspace, flags, st);
     if (rc != MATE_OK || !plan->sub[0]) return rc;
     // row-or-column pattern: the two passes over the rest of the column, then the merge
@@ -941,6 +959,7 @@ int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const v
     if (!workspace || workspace_bytes < need) return MATE_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MATE_ERR_ALIGNMENT;
     cudaStream_t st = (cudaStream_t)stream;
+    if (use_plans(plan, st) != cudaSuccess) return MATE_ERR_CUDA;
     rc = bwd_pass(plan, use_tc, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, workspace, 0, st);
     if (rc != MATE_OK || !plan->sub[0]) return rc;
     // Row-or-column pattern.  With the final O and LSE every pass computes the gradient of its own

@@ -21,6 +21,7 @@ __global__ void expire_wait_kernel(int32_t *status) {
 
 extern "C" int mate_debug_expire_wait(const mate_plan_t *plan, void *stream) {
     if (!plan) return MATE_ERR_INVALID_ARG;
+    if (mate::use_plan(plan, (cudaStream_t)stream) != cudaSuccess) return MATE_ERR_CUDA;
     mate::expire_wait_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(plan->status_dev);
     return cudaGetLastError() == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -96,6 +97,25 @@ struct TensorRows {
 #endif
 };
 
+// ---- memory pool (mate_pool.cu)
+struct Block {              // device memory
+    void *ptr = nullptr;
+    size_t bytes = 0;
+    int device = 0;
+    uint64_t stream = 0;    // stream_id of the only stream that uses it (0: unknown or several)
+};
+struct Staging {            // host memory, pinned when `event` is set
+    void *ptr = nullptr;
+    size_t bytes = 0;
+    int device = 0;
+    cudaEvent_t event = nullptr;
+};
+uint64_t stream_id(cudaStream_t st);  // unique over the process's life, 0 = not to be had
+bool pool_take(size_t bytes, cudaStream_t st, int device, Block *out);
+void pool_give(Block &b, uint64_t stream);
+bool staging_take(size_t bytes, int device, Staging *out);
+void staging_give(Staging &s, cudaStream_t st);
+
 struct ViewPlan {
     int32_t *perm = nullptr;      // [B, N]   view position -> original position
     int32_t *inv_perm = nullptr;  // [B, N]
@@ -126,10 +146,10 @@ struct mate_plan_s {
     // row-or-column pattern (mate_plan_sat): this plan is the row pass; sub[0] / sub[1] are the passes
     // over the rest of the token's column in front of / behind its own cell
     mate_plan_s *sub[2] = {nullptr, nullptr};
-    int32_t *pair_ids_dev = nullptr;     // ids of the sub-plans (owned by the main plan)
+    int32_t *pair_ids_dev = nullptr;     // ids of the sub-plans (in extra_block)
     // packed layout (mate_plan_packed): start and length of every example on the common token axis
     int T = 0;                           // total tokens; 0 = padded layout
-    int32_t *tok_off_dev = nullptr, *len_dev = nullptr;  // [B] each (one allocation, owned by the plan)
+    int32_t *tok_off_dev = nullptr, *len_dev = nullptr;  // [B] each (in extra_block)
     mate::TensorRows rows() const {
         mate::TensorRows r;
         r.tok_off = tok_off_dev;
@@ -147,8 +167,15 @@ struct mate_plan_s {
     std::vector<int32_t> n_valid;        // host copy
     std::vector<int64_t> pairs;          // [B, 2] unmasked pairs per example and view
     int32_t *status_dev = nullptr;       // device status word(s): [0] = id validation, [1] = kernel timeouts
-    void *dev_block = nullptr;           // one allocation backing all device arrays above
-    void *work_block = nullptr;          // one allocation backing the work-lists below
+    // device memory behind the arrays above / the work-lists below / pair_ids_dev, tok_off_dev and len_dev
+    mate::Block dev_block, work_block, extra_block;
+    // The stream the plan was made on, and whether it has been used on another one (or in a graph) since.  The
+    // work-lists are still on their way when mate_plan returns: uses on the same stream are ordered behind the
+    // copy, the first use elsewhere waits for it.
+    uint64_t stream = 0;
+    mutable std::atomic<bool> elsewhere{false};
+    mutable std::mutex ready_mu;
+    mutable cudaEvent_t ready = nullptr;  // recorded behind the copy; null once it has been waited for
     // tensor-core forward work-list: the units of CTA c are [fwd_cta_off[c], fwd_cta_off[c + 1])
     mate::FwdUnit *fwd_units_dev = nullptr;
     int32_t *fwd_cta_off_dev = nullptr;
@@ -208,6 +235,9 @@ cudaError_t launch_after(void (*kernel)(const Params), int grid, int threads, si
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, p);
 }
+
+// To be called before work that uses the plan is put on `st`.
+cudaError_t use_plan(const mate_plan_t *plan, cudaStream_t st);
 
 // plan kernels (mate_plan_kernels.cu)
 cudaError_t launch_plan_kernels(const int32_t *row_ids, const int32_t *col_ids, int B, int N,

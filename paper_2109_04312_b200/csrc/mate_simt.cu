@@ -323,6 +323,7 @@ extern "C" int mate_attn_bwd_noalloc(const mate_plan_t *plan, const void *Q, con
     const size_t rows = (size_t)plan->B * plan->H * plan->N;
     if (rows > mate::kNoAllocMaxRows) return MATE_ERR_TOO_LARGE;
 
+    if (mate::use_plan(plan, (cudaStream_t)stream) != cudaSuccess) return MATE_ERR_CUDA;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return MATE_ERR_CUDA;
     if (dev < 0 || dev >= kMaxDevices) return MATE_ERR_UNSUPPORTED;

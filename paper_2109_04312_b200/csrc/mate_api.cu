@@ -71,27 +71,16 @@ struct RowBounds {
     const int32_t *so;
     int S, P, radius;  // P: length of the global block (bucket origin; no range reaches in front of it)
     int mode = mate::kBoundsOwn, group = 1;
-    int seg_of(int t) const { return (int)(std::upper_bound(so, so + S, t) - so) - 1; }
-    int lo(int t) const { return lo(t, seg_of(t)); }
-    int hi(int t) const { return hi(t, seg_of(t)); }
-    int lo(int t, int id) const {
-        int l = so[id];
-        if (mode == mate::kBoundsBefore) l = so[id / group * group];
-        if (mode == mate::kBoundsAfter) l = so[id + 1];
-        if (radius <= 0) return std::max(l, P);
-        const int64_t bk = (t - P) / radius;
-        return (int)std::max<int64_t>(std::max(l, P), P + (bk - 1) * radius);
+    // range of the positions of segment `id`, without the buckets
+    int own_lo(int id) const {
+        return std::max(mode == mate::kBoundsBefore ? so[id / group * group] : mode == mate::kBoundsAfter ? so[id + 1] : so[id], P);
     }
-    int hi(int t, int id) const {
-        int h = so[id + 1];
-        if (mode == mate::kBoundsBefore) h = so[id];
-        if (mode == mate::kBoundsAfter) h = so[std::min((id / group + 1) * group, S - 1)];
-        if (radius > 0) {
-            const int64_t bk = (t - P) / radius;
-            h = (int)std::min<int64_t>(h, P + (bk + 2) * radius);
-        }
-        return std::max(h, lo(t, id));
+    int own_hi(int id) const {
+        return mode == mate::kBoundsBefore ? so[id] : mode == mate::kBoundsAfter ? so[std::min((id / group + 1) * group, S - 1)] : so[id + 1];
     }
+    // the three adjacent buckets of position t (never beyond 2^31: positions are below 2^30)
+    int bucket_lo(int t) const { return (int)std::max<int64_t>(P + (int64_t)((t - P) / radius - 1) * radius, P); }
+    int bucket_hi(int t) const { return (int)std::min<int64_t>(P + (int64_t)((t - P) / radius + 2) * radius, INT32_MAX); }
 };
 
 // ---------------------------------------------------------------------------- work-lists
@@ -114,11 +103,23 @@ void fill_ranges(const mate_plan_t *pl, const int32_t *const (&seg_off_host)[2],
     rr.nv = pl->n_valid[b];
     rr.lo.resize(rr.nv);
     rr.hi.resize(rr.nv);
-    for (int id = 0; id + 1 < S; ++id)
-        for (int t = std::max(so[id], rb.P); t < so[id + 1]; ++t) {
-            rr.lo[t] = rb.lo(t, id);
-            rr.hi[t] = rb.hi(t, id);
+    for (int id = 0; id + 1 < S; ++id) {
+        const int t0 = std::max(so[id], rb.P), t1 = so[id + 1];
+        if (t1 <= t0) continue;
+        const int l = rb.own_lo(id), h = std::max(rb.own_hi(id), l);
+        if (pl->radius <= 0) {
+            std::fill(rr.lo.begin() + t0, rr.lo.begin() + t1, l);
+            std::fill(rr.hi.begin() + t0, rr.hi.begin() + t1, h);
+            continue;
         }
+        for (int t = t0; t < t1;) {  // bucket by bucket
+            const int end = (int)std::min<int64_t>(t1, rb.P + (int64_t)((t - rb.P) / pl->radius + 1) * pl->radius);
+            const int lo = std::max(l, rb.bucket_lo(t)), hi = std::max(std::min(h, rb.bucket_hi(t)), lo);
+            std::fill(rr.lo.begin() + t, rr.lo.begin() + end, lo);
+            std::fill(rr.hi.begin() + t, rr.hi.begin() + end, hi);
+            t = end;
+        }
+    }
 }
 
 // Estimated clocks of the forward kernel (fitted to its per-unit times): a half alone on a tile; both
@@ -128,45 +129,66 @@ constexpr int kFullClk = 1800, kPartialClk = 900, kChunkClk = 350, kUnitClk = 35
 
 struct Proto {
     FwdUnit u;
-    std::vector<int32_t> tile;  // estimated clocks of every tile
-    int64_t cost;               // of the whole unit
+    int view;
+    int tile0, n_tiles;  // estimated clocks of its tiles: tiles[tile0 ..] of the list
+    int64_t cost;        // of the whole unit
+};
+struct ProtoList {
+    std::vector<Proto> protos;
+    std::vector<int32_t> tiles;
 };
 
-// Estimated clocks of a half on every tile of its unit (0: skipped).
-void half_tile_clks(const FwdUnit &u, int h, const RowRanges &rr, std::vector<int32_t> &clk) {
+// Adds the estimated clocks of half h on every tile of its unit to clk (none where it skips the tile).
+void half_tile_clks(const FwdUnit &u, int h, const RowRanges &rr, int32_t *clk) {
     const int nA = u.tiles_a(), n_tiles = nA + u.tiles_b(), rows = u.rows_of(h), r0 = u.row0_of(h);
-    clk.assign(n_tiles, 0);
     if (rows == 0) return;
-    for (int i = 0; i < n_tiles; ++i) {
+    for (int i = 0; i < nA; ++i) {
+        const int w = std::min(kTile, u.kA_end - u.kA0 - i * kTile);
+        clk[i] = w == kTile ? kFullClk : kPartialClk + kChunkClk * ceil_div(w, kChunk);
+    }
+    for (int i = nA; i < n_tiles; ++i) {
         const TileInfo t = mate::tile_info(u, i, nA);
         int c0, c1;
         mate::half_cols(u.lo[h], u.hi[h], t, c0, c1);
         if (c1 <= c0) continue;
-        int chunks = ceil_div(t.w, kChunk);
-        bool full = t.w == kTile;
-        if (t.is_b) {
-            chunks = 0;
-            for (int r = 0; r < rows; r += 32) {  // the warps of the half
-                const int last = r0 + std::min(r + 32, rows) - 1;
-                const int a = std::max(rr.lo[r0 + r] - t.k0, 0), e = std::min(rr.hi[last] - t.k0, t.w);
-                chunks = std::max(chunks, e > a ? ceil_div(e, kChunk) - a / kChunk : 0);
-            }
-            full = full && rr.lo[r0 + rows - 1] <= t.k0 && rr.hi[r0] >= t.k0 + kTile;
+        if (t.w == kTile && rr.lo[r0 + rows - 1] <= t.k0 && rr.hi[r0] >= t.k0 + kTile) {
+            clk[i] = kFullClk;
+            continue;
         }
-        clk[i] = full ? kFullClk : kPartialClk + kChunkClk * chunks;
+        int chunks = 0;
+        for (int r = 0; r < rows; r += 32) {  // the warps of the half
+            const int last = r0 + std::min(r + 32, rows) - 1;
+            const int a = std::max(rr.lo[r0 + r] - t.k0, 0), e = std::min(rr.hi[last] - t.k0, t.w);
+            chunks = std::max(chunks, e > a ? ceil_div(e, kChunk) - a / kChunk : 0);
+        }
+        clk[i] = kPartialClk + kChunkClk * chunks;
     }
 }
 
-void unit_cost(Proto &pr, const RowRanges &rr) {
-    std::vector<int32_t> other;
-    half_tile_clks(pr.u, 0, rr, pr.tile);
-    half_tile_clks(pr.u, 1, rr, other);
-    pr.cost = kUnitClk;
-    for (size_t i = 0; i < pr.tile.size(); ++i) {
-        pr.tile[i] = pr.tile[i] && other[i] ? (pr.tile[i] + other[i]) * 18 / 25 : std::max(pr.tile[i] + other[i], 100);
-        pr.cost += pr.tile[i];
+void add_proto(ProtoList &pl, const FwdUnit &u, int view, const RowRanges &rr) {
+    Proto pr{u, view, (int)pl.tiles.size(), u.tiles_a() + u.tiles_b(), kUnitClk};
+    pl.tiles.resize(pr.tile0 + 2 * pr.n_tiles, 0);
+    int32_t *a = pl.tiles.data() + pr.tile0, *b = a + pr.n_tiles;
+    half_tile_clks(u, 0, rr, a);
+    half_tile_clks(u, 1, rr, b);
+    for (int i = 0; i < pr.n_tiles; ++i) {
+        a[i] = a[i] && b[i] ? (a[i] + b[i]) * 18 / 25 : std::max(a[i] + b[i], 100);
+        pr.cost += a[i];
     }
+    pl.tiles.resize(pr.tile0 + pr.n_tiles);
+    pl.protos.push_back(pr);
 }
+
+// Longest first; the heads of a view repeat its units.
+void sort_protos(ProtoList &pl) {
+    std::stable_sort(pl.protos.begin(), pl.protos.end(), [](const Proto &a, const Proto &b) { return a.cost > b.cost; });
+}
+struct HeadLists {
+    std::vector<int> heads[2];
+    explicit HeadLists(const mate_plan_t *pl) {
+        for (int h = 0; h < pl->H; ++h) heads[pl->head_view[h]].push_back(h);
+    }
+};
 
 // One unit of the halves [r0, r1) and [r1, r2) (the second one may be empty) of table rows.
 FwdUnit table_unit(const RowRanges &rr, int r0, int r1, int r2) {
@@ -192,9 +214,12 @@ FwdUnit table_unit(const RowRanges &rr, int r0, int r1, int r2) {
 
 // Units of one (example, view), for any head of the view.  Padding rows are left out.  `pairs`: two halves
 // to a unit where they share most of their tiles.
-void proto_units(const RowRanges &rr, bool pairs, std::vector<FwdUnit> &proto) {
+void add_units(const RowRanges &rr, int b, int view, bool pairs, ProtoList &out) {
+    const auto add = [&](FwdUnit &u) {
+        u.b = b;
+        add_proto(out, u, view, rr);
+    };
     const int P = rr.P, nv = rr.nv;
-    proto.clear();
     for (int q0 = 0; q0 < P;) {  // rows of the global block: every valid key
         FwdUnit u{};
         const int n0 = std::min(kTile, P - q0), n1 = pairs ? std::min(kTile, P - q0 - n0) : 0;
@@ -204,7 +229,7 @@ void proto_units(const RowRanges &rr, bool pairs, std::vector<FwdUnit> &proto) {
         u.tB = kTile;
         u.parts = 1;
         u.ctr = -1;
-        proto.push_back(u);
+        add(u);
         q0 += n0 + n1;
     }
     // Halves of table rows: 128 rows, or fewer when ending where a segment begins saves tiles (a half that
@@ -232,41 +257,30 @@ void proto_units(const RowRanges &rr, bool pairs, std::vector<FwdUnit> &proto) {
             const int both = ceil_div(rr.hi[r2 - 1] - rr.lo[r0], kTile);
             two = 4 * (tiles_a + both) <= 3 * (2 * tiles_a + n0 + n1) || tiles_a + both <= 4;
         }
-        proto.push_back(table_unit(rr, r0, r1, two ? cuts[i + 2] : r1));
+        FwdUnit u = table_unit(rr, r0, r1, two ? cuts[i + 2] : r1);
+        add(u);
         i += two ? 2 : 1;
     }
 }
 
-// Backward: single halves, none split; its work items are the units, once per side.
-void make_bwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges) {
-    std::vector<std::pair<int64_t, FwdUnit>> all;
-    std::vector<FwdUnit> proto;
-    std::vector<int32_t> clk;
-    for (int v = 0; v < 2; ++v) {
-        if (pl->view[v].n_heads == 0) continue;
-        for (int b = 0; b < pl->B; ++b) {
-            const RowRanges &rr = ranges[(size_t)v * pl->B + b];
-            proto_units(rr, false, proto);
-            for (FwdUnit &u : proto) {
-                int64_t cost = 0;
-                half_tile_clks(u, 0, rr, clk);
-                for (int c : clk) cost += c;
-                u.b = b;
-                for (int h = 0; h < pl->H; ++h) {
-                    if (pl->head_view[h] != v) continue;
-                    u.h = h;
-                    all.push_back({cost, u});
-                }
-            }
-        }
-    }
-    // longest first: the CTAs of the persistent kernel take work from the head of the list as they
-    // become free (a shared counter), so the order is the whole schedule
-    std::stable_sort(all.begin(), all.end(), [](const std::pair<int64_t, FwdUnit> &a, const std::pair<int64_t, FwdUnit> &b) {
-        return a.first > b.first;
-    });
+void list_units(const mate_plan_t *pl, const std::vector<RowRanges> &ranges, bool pairs, ProtoList &out) {
+    out.protos.clear();
+    out.tiles.clear();
+    for (int v = 0; v < 2; ++v)
+        for (int b = 0; b < pl->B && pl->view[v].n_heads > 0; ++b) add_units(ranges[(size_t)v * pl->B + b], b, v, pairs, out);
+    sort_protos(out);
+}
+
+// Backward: single halves, none split; its work items are the units, once per side.  Longest first: the CTAs of
+// the persistent kernel take work from the head of the list as they become free (a shared counter), so the
+// order is the whole schedule.
+void make_bwd_units(mate_plan_t *pl, const ProtoList &singles, const HeadLists &heads) {
     pl->bwd_units.clear();
-    for (const auto &uc : all) pl->bwd_units.push_back(uc.second);
+    for (const Proto &pr : singles.protos)
+        for (int h : heads.heads[pr.view]) {
+            pl->bwd_units.push_back(pr.u);
+            pl->bwd_units.back().h = h;
+        }
     pl->n_bwd_units = (int)pl->bwd_units.size();
     pl->bwd_grid = std::min(std::max(pl->n_ctas, 1), std::max(2 * pl->n_bwd_units, pl->n_pads));
 }
@@ -293,29 +307,35 @@ struct Instance {
     int proto, h;
 };
 
-// Units that cost more than `divisible` clocks may be cut between two tiles.  The others go, longest first,
-// to the CTA with the least work; the divisible ones then fill all CTAs up to a common level, one after
+// Units (longest first) that cost more than `divisible` clocks may be cut between two tiles.  The others go to
+// the CTA with the least work; the divisible ones then fill all CTAs up to a common level, one after
 // the other.  Returns the estimated time of the slowest CTA.
-int64_t balance(const std::vector<Proto> &protos, const std::vector<Instance> &inst, const std::vector<int> &order, int n_ctas,
-                int64_t divisible, std::vector<Piece> &pieces) {
+int64_t balance(const ProtoList &list, const std::vector<Instance> &inst, int n_ctas, int64_t divisible, std::vector<Piece> &pieces) {
+    const std::vector<Proto> &protos = list.protos;
     pieces.clear();
-    std::vector<std::pair<int64_t, int>> heap;  // (load, CTA), least on top
-    const auto more = [](const std::pair<int64_t, int> &a, const std::pair<int64_t, int> &b) { return a > b; };
-    for (int c = 0; c < n_ctas; ++c) heap.push_back({0, c});
     size_t n_div = 0;
     int64_t div_clk = 0;
-    while (n_div < order.size() && protos[inst[order[n_div]].proto].cost > divisible) {
-        for (int c : protos[inst[order[n_div]].proto].tile) div_clk += c;
-        ++n_div;
+    for (; n_div < inst.size() && protos[inst[n_div].proto].cost > divisible; ++n_div) div_clk += protos[inst[n_div].proto].cost - kUnitClk;
+    // heap of (load, CTA) in one word, least on top
+    std::vector<int64_t> loads(n_ctas);
+    for (int c = 0; c < n_ctas; ++c) loads[c] = c;
+    for (size_t k = n_div; k < inst.size(); ++k) {
+        const Proto &pr = protos[inst[k].proto];
+        const int64_t top = loads[0];
+        pieces.push_back({(int)k, 0, pr.n_tiles, (int)(top & 0xffff)});
+        const int64_t key = top + (pr.cost << 16);
+        size_t i = 0;  // sift down
+        for (size_t c = 1; c < loads.size(); c = 2 * i + 1) {
+            if (c + 1 < loads.size() && loads[c + 1] < loads[c]) ++c;
+            if (loads[c] >= key) break;
+            loads[i] = loads[c];
+            i = c;
+        }
+        loads[i] = key;
     }
-    for (size_t k = n_div; k < order.size(); ++k) {
-        const Proto &pr = protos[inst[order[k]].proto];
-        std::pop_heap(heap.begin(), heap.end(), more);
-        heap.back().first += pr.cost;
-        pieces.push_back({order[k], 0, (int)pr.tile.size(), heap.back().second});
-        std::push_heap(heap.begin(), heap.end(), more);
-    }
-    std::sort(heap.begin(), heap.end());
+    std::sort(loads.begin(), loads.end());
+    std::vector<std::pair<int64_t, int>> heap(n_ctas);
+    for (int c = 0; c < n_ctas; ++c) heap[c] = {loads[c] >> 16, (int)(loads[c] & 0xffff)};
     int64_t worst = heap.back().first;
     if (n_div == 0) return worst;
     // Level: the `used` least loaded CTAs take the divisible tiles, each with the cost of one more (partial)
@@ -336,17 +356,18 @@ int64_t balance(const std::vector<Proto> &protos, const std::vector<Instance> &i
         int64_t load = heap[c].first, room = level - load + carry;
         const bool last = c + 1 == used;
         while (k < n_div) {
-            const std::vector<int32_t> &tile = protos[inst[order[k]].proto].tile;
+            const int32_t *tile = list.tiles.data() + protos[inst[k].proto].tile0;
+            const int n_tiles = protos[inst[k].proto].n_tiles;
             int64_t left = room - extra;
             int i1 = i0;
-            while (i1 < (int)tile.size() && (last || left >= tile[i1] / 2)) left -= tile[i1++];
-            if (!last && i1 > i0 + 1 && i1 + 1 == (int)tile.size()) left += tile[--i1];  // leave no crumb
+            while (i1 < n_tiles && (last || left >= tile[i1] / 2)) left -= tile[i1++];
+            if (!last && i1 > i0 + 1 && i1 + 1 == n_tiles) left += tile[--i1];  // leave no crumb
             if (i1 == i0) break;
             load += room - left;
             room = left;
             i0 = i1;
-            pieces.push_back({order[k], i1, i1, heap[c].second});
-            if (i1 < (int)tile.size()) break;
+            pieces.push_back({(int)k, i1, i1, heap[c].second});
+            if (i1 < n_tiles) break;
             ++k;
             i0 = 0;
         }
@@ -364,53 +385,36 @@ int64_t balance(const std::vector<Proto> &protos, const std::vector<Instance> &i
     return worst;
 }
 
-void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges) {
-    const int n_ctas = std::max(pl->n_ctas, 1);
-    std::vector<Proto> protos;
-    std::vector<Instance> inst;
-    int64_t total = 0;
+void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const ProtoList &singles, const HeadLists &heads) {
+    const int n_ctas = std::min(std::max(pl->n_ctas, 1), 0xffff);
+    ProtoList paired;
+    list_units(pl, ranges, true, paired);
+    size_t n_inst = 0;
+    for (const Proto &pr : paired.protos) n_inst += heads.heads[pr.view].size();
     // Single halves when there are not enough pairs for half of the SMs: a CTA then works on one half only,
     // which takes less than the time of both.
-    for (bool pairs = true;; pairs = false) {
-        protos.clear();
-        inst.clear();
-        total = 0;
-        std::vector<FwdUnit> proto;
-        for (int v = 0; v < 2; ++v) {
-            if (pl->view[v].n_heads == 0) continue;
-            for (int b = 0; b < pl->B; ++b) {
-                const RowRanges &rr = ranges[(size_t)v * pl->B + b];
-                proto_units(rr, pairs, proto);
-                for (FwdUnit &u : proto) {
-                    u.b = b;
-                    Proto pr{u, {}, 0};
-                    unit_cost(pr, rr);
-                    for (int h = 0; h < pl->H; ++h)
-                        if (pl->head_view[h] == v) inst.push_back({(int)protos.size(), h});
-                    total += pr.cost * pl->view[v].n_heads;
-                    protos.push_back(std::move(pr));
-                }
-            }
-        }
-        if (!pairs || 2 * (int)inst.size() > n_ctas) break;
+    const ProtoList &list = 2 * (int)n_inst > n_ctas ? paired : singles;
+    const std::vector<Proto> &protos = list.protos;
+    std::vector<Instance> inst;
+    inst.reserve(n_inst);
+    int64_t total = 0;
+    for (size_t k = 0; k < protos.size(); ++k) {
+        for (int h : heads.heads[protos[k].view]) inst.push_back({(int)k, h});
+        total += protos[k].cost * (int64_t)heads.heads[protos[k].view].size();
     }
-    std::vector<int> order(inst.size());
-    for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int a, int b) { return protos[inst[a].proto].cost > protos[inst[b].proto].cost; });
     // How much is cut is decided by the estimate: nothing, units longer than a CTA's share, half of it, a quarter.
     const int64_t share = total / n_ctas;
     std::vector<Piece> best, pieces;
-    int64_t best_clk = -1;
-    for (const int64_t divisible : {INT64_MAX, share, share / 2, share / 4}) {
-        if (divisible < kUnitClk + 4 * kFullClk) break;
-        const int64_t clk = balance(protos, inst, order, n_ctas, divisible, pieces);
-        if (best_clk < 0 || clk < best_clk) {
+    best.reserve(inst.size());
+    int64_t best_clk = balance(list, inst, n_ctas, INT64_MAX, best);
+    for (const int64_t divisible : {share, share / 2, share / 4}) {
+        if (divisible < kUnitClk + 4 * kFullClk || 100 * best_clk <= 106 * share) break;
+        const int64_t clk = balance(list, inst, n_ctas, divisible, pieces);
+        if (clk < best_clk) {
             best_clk = clk;
             best.swap(pieces);
         }
     }
-    if (best_clk < 0) balance(protos, inst, order, n_ctas, INT64_MAX, best);
 
     // records, split units with their place in the workspace; a CTA starts with its parts of split units, so
     // that nobody waits for them in the end
@@ -425,23 +429,25 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges) {
             ws_off[k] = ws_bytes;
             ws_bytes += n_parts[k] * mate::kPartialBytes;
         }
-    std::vector<std::vector<FwdUnit>> lists(n_ctas);
-    for (int pass = 0; pass < 2; ++pass)
+    pl->fwd_cta_off.assign(n_ctas + 1, 0);
+    for (const Piece &pc : best) ++pl->fwd_cta_off[pc.cta + 1];
+    for (int c = 0; c < n_ctas; ++c) pl->fwd_cta_off[c + 1] += pl->fwd_cta_off[c];
+    pl->fwd_units.resize(best.size());
+    std::vector<int32_t> at(pl->fwd_cta_off.begin(), pl->fwd_cta_off.end() - 1);
+    for (int pass = pl->n_fwd_slots > 0 ? 0 : 1; pass < 2; ++pass)
         for (const Piece &pc : best) {
             if ((n_parts[pc.unit] > 1) != (pass == 0)) continue;
-            FwdUnit u = slice_unit(protos[inst[pc.unit].proto].u, pc.i0, pc.i1);
+            const Proto &pr = protos[inst[pc.unit].proto];
+            FwdUnit &u = pl->fwd_units[at[pc.cta]++];
+            u = pr.u;
+            if (n_parts[pc.unit] > 1) {
+                u = slice_unit(pr.u, pc.i0, pc.i1);
+                u.parts = n_parts[pc.unit] | seen[pc.unit]++ << 16;
+                u.ctr = slot[pc.unit];
+                u.ws_off = (int32_t)((ws_off[pc.unit] + u.part() * mate::kPartialBytes) >> 10);
+            }
             u.h = inst[pc.unit].h;
-            u.parts = n_parts[pc.unit] | seen[pc.unit]++ << 16;
-            u.ctr = slot[pc.unit];
-            u.ws_off = (int32_t)((ws_off[pc.unit] + u.part() * mate::kPartialBytes) >> 10);
-            lists[pc.cta].push_back(u);
         }
-    pl->fwd_units.clear();
-    pl->fwd_cta_off.assign(1, 0);
-    for (int c = 0; c < n_ctas; ++c) {
-        pl->fwd_units.insert(pl->fwd_units.end(), lists[c].begin(), lists[c].end());
-        pl->fwd_cta_off.push_back((int32_t)pl->fwd_units.size());
-    }
     pl->n_fwd_units = (int)pl->fwd_units.size();
     pl->fwd_ws_bytes = ws_bytes;
     // padding rows of every (example, head)
@@ -471,8 +477,22 @@ int build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], cudaSt
     std::vector<RowRanges> ranges((size_t)2 * pl->B);
     for (int v = 0; v < 2; ++v)
         for (int b = 0; b < pl->B && pl->view[v].n_heads > 0; ++b) fill_ranges(pl, seg_off_host, v, b, ranges[(size_t)v * pl->B + b]);
-    make_fwd_units(pl, ranges);
-    make_bwd_units(pl, ranges);
+    // unmasked pairs per (example, view): the global block with everything, every table row with the block and
+    // its own range
+    pl->pairs.assign((size_t)pl->B * 2, 0);
+    for (int v = 0; v < 2; ++v)
+        for (int b = 0; b < pl->B && pl->view[v].n_heads > 0; ++b) {
+            const RowRanges &rr = ranges[(size_t)v * pl->B + b];
+            int64_t c = (int64_t)rr.P * rr.nv + (int64_t)rr.P * (rr.nv - rr.P);
+            for (int t = rr.P; t < rr.nv; ++t) c += rr.hi[t] - rr.lo[t];
+            pl->pairs[(size_t)b * 2 + v] = c;
+        }
+
+    const HeadLists heads(pl);
+    ProtoList singles;
+    list_units(pl, ranges, false, singles);
+    make_fwd_units(pl, ranges, singles, heads);
+    make_bwd_units(pl, singles, heads);
 
     // device copy, in one piece: units, CTA offsets, padding, arrival counters (zeros; the kernel resets them)
     const auto lay_out = [pl](char *base) {
@@ -743,28 +763,6 @@ static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int
     pl->n_valid.assign(out_host(pl->n_valid_dev), out_host(pl->n_valid_dev) + B);
     const int32_t *seg_off_host[2] = {out_host(pl->view[0].seg_off), out_host(pl->view[1].seg_off)};
 
-    // unmasked pairs per (example, view): P * n_valid + sum_s L_s (L_s + P); a bucketed plan counts,
-    // row by row, the prefix and the clipped part of the segment
-    pl->pairs.assign((size_t)B * 2, 0);
-    for (int v = 0; v < 2; ++v) {
-        const int S = pl->view[v].max_id + 2;
-        for (int b = 0; b < B; ++b) {
-            const int32_t *so = seg_off_host[v] + (size_t)b * S;
-            const int P = std::min(pl->global[b], pl->n_valid[b]);
-            int64_t c = (int64_t)P * pl->n_valid[b];
-            if (radius > 0 || pl->bounds_mode != mate::kBoundsOwn || P != pl->prefix[b]) {
-                const RowBounds rb{so, S, P, radius, pl->bounds_mode, pl->group};
-                for (int t = P; t < pl->n_valid[b]; ++t) c += P + rb.hi(t) - rb.lo(t);
-            } else {
-                for (int s = 0; s + 1 < S; ++s) {
-                    const int64_t L = so[s + 1] - so[s];
-                    c += L * (L + P);
-                }
-            }
-            pl->pairs[(size_t)b * 2 + v] = c;
-        }
-    }
-
     rc = build_units(pl, seg_off_host, st);
     mate::staging_give(host, st);
     if (rc != MATE_OK) {
@@ -938,7 +936,7 @@ static int bwd_pass(const mate_plan_t *plan, bool use_tc, const void *Q, const v
                     const float *LSE, const void *dO, int d, int dtype, float scale, void *dQ, void *dK, void *dV, void *ws,
                     int pass, cudaStream_t st) {
     if (use_tc) return mate::tc_bwd(plan, Q, K, V, O, LSE, dO, scale, dQ, dK, dV, ws, pass, st);
-    return mate::simt_bwd(plan, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, ws, st);
+    return mate::simt_bwd(plan, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, ws, pass, st);
 }
 
 int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,

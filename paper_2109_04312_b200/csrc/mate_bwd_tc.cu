@@ -756,7 +756,7 @@ int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
         rowdot_kernel<<<(unsigned)((rows + kRowdotRows - 1) / kRowdotRows), 256, 0, stream>>>(
             (const __nv_bfloat16 *)dO, (const __nv_bfloat16 *)O, LSE, D, nlse, rows, (int32_t *)ws);
     // started while the kernel before drains: its set-up and first records overlap with that
-    return launch_after(tc_bwd_kernel, plan->bwd_grid, kThreads, kSmemBytes, stream, p) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
+    return launch_after(tc_bwd_kernel, dim3((unsigned)plan->bwd_grid), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }
 
 }  // namespace mate

@@ -222,9 +222,9 @@ struct SmemAttrOnce {
 // Launches a kernel that may start before the one in front of it in the stream is complete; it waits for that
 // itself (griddepcontrol.wait) before it touches what that one writes.
 template <typename Params>
-cudaError_t launch_after(void (*kernel)(const Params), int grid, int threads, size_t smem, cudaStream_t stream, const Params &p) {
+cudaError_t launch_after(void (*kernel)(const Params), dim3 grid, int threads, size_t smem, cudaStream_t stream, const Params &p) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -261,7 +261,7 @@ int simt_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *
 size_t simt_bwd_workspace(const mate_plan_t *plan);
 int simt_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, const void *O,
              const float *LSE, const void *dO, int d, int dtype, float scale, void *dQ, void *dK,
-             void *dV, void *workspace, cudaStream_t stream);
+             void *dV, void *workspace, int pass, cudaStream_t stream);
 
 // tensor-core kernels (mate_fwd_tc.cu / mate_bwd_tc.cu)
 bool tc_supported(int d, int dtype);

@@ -1,17 +1,27 @@
-// SIMT (no tensor core) kernels: one warp per query row (forward, dQ) or per key row (dK/dV).
-// fp32 arithmetic whatever the storage type; this is the debug / any-head-dim path and the
-// reference the tensor-core kernels were brought up against on the device.
+// Kernels without tensor cores: fp32 arithmetic whatever the storage type, any head size up to 128.  They serve
+// fp32 tensors and head sizes other than 64, and are the reference the tensor-core kernels were brought up
+// against on the device.
 //
 // In a head's view order (see mate_plan) the keys of query row t are
 //     [0, P)  u  [max(seg_lo[t], P), seg_hi[t])
 // which is the attention pattern A of Section 3 for both table rows (own segment plus prefix) and
 // prefix rows (seg_lo = 0, seg_hi = n_valid).  The pattern is symmetric, so the queries that
 // attend to key t are the same two ranges; dK/dV therefore need no atomics.
+//
+// A block takes 32 rows of the order against tiles of 64 columns: [0, P), then the union of the rows' other
+// ranges.  256 threads; a thread forms 2 x 4 scores, the 16 lanes of a half warp share two rows from the scores
+// to the results, so only the loads of a tile need the whole block to meet.  The next tile travels to
+// registers under the arithmetic of this one.  Bound by fp32 multiply-adds fed from shared memory (6 to 8
+// 16-byte reads per 32 of them) and, on small tables, by the latency of a handful of tiles.  One warp per
+// row with global reads of every key took 463 us for the forward and 1540 us for the backward of 2 x 512
+// tokens, 12 heads of 64.
 #include <cuda_bf16.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "mate_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace mate {
 
@@ -23,281 +33,480 @@ namespace {
 constexpr size_t kNoAllocMaxRows = size_t(1) << 20;
 static __device__ __align__(256) float g_noalloc_rowdot[kNoAllocMaxRows];
 
-constexpr int kWarpsPerBlock = 4;
 constexpr int kMaxD = 128;
-constexpr int kAccPerLane = kMaxD / 32;
+constexpr int kRows = 32, kCols = 64, kThreads = 256;
+constexpr int kPStride = kCols + 4;
 
-__device__ __forceinline__ float to_f(float x) { return x; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
+__device__ __forceinline__ float4 load4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16 *p) {
+    const uint2 x = __ldg(reinterpret_cast<const uint2 *>(p));
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x.x));
+    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
 __device__ __forceinline__ void from_f(float &dst, float x) { dst = x; }
 __device__ __forceinline__ void from_f(__nv_bfloat16 &dst, float x) { dst = __float2bfloat16_rn(x); }
 
-__device__ __forceinline__ float warp_max(float v) {
+// reductions over the 16 lanes of a half warp
+__device__ __forceinline__ float half_max(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
-__device__ __forceinline__ float warp_sum(float v) {
+__device__ __forceinline__ float half_sum(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
-template <typename T>
-__device__ __forceinline__ float dot_row(const float *__restrict__ a_smem, const T *__restrict__ row,
-                                         int d) {
-    float acc = 0.f;
-    for (int e = 0; e < d; ++e) acc = fmaf(a_smem[e], to_f(row[e]), acc);
-    return acc;
-}
-
-struct RowCtx {
-    const int32_t *perm, *seg_lo, *seg_hi;
-    int n_valid, view;
+struct Common {
+    ViewPlan rowv, colv;
+    const uint8_t *head_view;
+    const int32_t *n_valid, *prefix;  // prefix: length of the global block
+    int N, d, view_order;
+    float scale;
+    TensorRows tr;
 };
 
-__device__ __forceinline__ RowCtx row_ctx(const ViewPlan &rowv, const ViewPlan &colv,
-                                          const uint8_t *head_view, const int32_t *n_valid, int b,
-                                          int h, int N) {
-    RowCtx c;
-    c.view = head_view[h];
-    const ViewPlan &vp = c.view ? colv : rowv;
-    c.perm = vp.perm + (size_t)b * N;
-    c.seg_lo = vp.seg_lo + (size_t)b * N;
-    c.seg_hi = vp.seg_hi + (size_t)b * N;
-    c.n_valid = n_valid[b];
-    return c;
+// The rows of a block and the column tiles they meet.
+struct RowBlock {
+    const int32_t *perm;
+    size_t bh;
+    int t0, n, P, b_lo, b_hi, n_a, n_tiles, lo[2], hi[2];  // lo, hi: behind the global block, of this thread's two rows
+    __device__ __forceinline__ int orig(int t) const { return perm ? __ldg(perm + t) : t; }
+    __device__ __forceinline__ void tile(int i, int &c0, int &w) const {
+        c0 = i < n_a ? i * kCols : b_lo + (i - n_a) * kCols;
+        w = min(kCols, (i < n_a ? P : b_hi) - c0);
+    }
+    // does column c (of range A or B) count for row j of this thread?
+    __device__ __forceinline__ bool counts(int i, int c, int w_end, int j) const {
+        return c < w_end && (i < n_a || (c >= lo[j] && c < hi[j]));
+    }
+};
+__device__ __forceinline__ RowBlock row_block(const Common &c, int b, int h, int blk, int *s_range) {
+    const ViewPlan &vp = c.head_view[h] ? c.colv : c.rowv;
+    RowBlock r;
+    r.perm = c.view_order ? nullptr : vp.perm + (size_t)b * c.N;
+    r.bh = c.tr.base(b, h);
+    r.t0 = blk * kRows;
+    const int nv = c.n_valid[b];
+    r.n = min(kRows, nv - r.t0);  // valid rows of the block (<= 0: padding only)
+    r.P = min(c.prefix[b], nv);
+    const int32_t *slo = vp.seg_lo + (size_t)b * c.N + r.t0, *shi = vp.seg_hi + (size_t)b * c.N + r.t0;
+    if (threadIdx.x < 32) {  // union of the rows' ranges behind the global block
+        const bool on = (int)threadIdx.x < r.n;
+        const int l = on ? max(slo[threadIdx.x], r.P) : 0x7fffffff, u = on ? shi[threadIdx.x] : 0;
+        const int lmin = __reduce_min_sync(0xffffffffu, u > l ? l : 0x7fffffff), umax = __reduce_max_sync(0xffffffffu, u > l ? u : 0);
+        if (threadIdx.x == 0) {
+            s_range[0] = lmin;
+            s_range[1] = umax;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int row = min((int)(threadIdx.x >> 4) * 2 + j, max(r.n - 1, 0));
+        r.lo[j] = r.n > 0 ? max(slo[row], r.P) : 0;
+        r.hi[j] = r.n > 0 ? shi[row] : 0;
+    }
+    __syncthreads();
+    r.b_lo = s_range[0];
+    r.b_hi = s_range[1];
+    r.n_a = (r.P + kCols - 1) / kCols;
+    r.n_tiles = r.n_a + (r.b_hi > r.b_lo ? (r.b_hi - r.b_lo + kCols - 1) / kCols : 0);
+    return r;
+}
+
+// kN rows of a tensor in registers (float4 chunks dealt over the threads), on their way to shared memory.
+template <int kN, int DP>
+struct Chunks {
+    static constexpr int kPer = kN * DP / 4 / kThreads > 0 ? kN * DP / 4 / kThreads : 1;
+    float4 v[kPer];
+    template <typename T>
+    __device__ __forceinline__ void load(const T *base, const RowBlock &r, int c0, int n, int d) {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int c = threadIdx.x + i * kThreads, row = c / (DP / 4), ch = c % (DP / 4);
+            v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row < kN && ch * 4 < d) v[i] = load4(base + (size_t)r.orig(c0 + min(row, n - 1)) * d + ch * 4);  // rows past n repeat the last
+        }
+    }
+    __device__ __forceinline__ void store(float *s) const {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int c = threadIdx.x + i * kThreads, row = c / (DP / 4), ch = c % (DP / 4);
+            if (row < kN) *reinterpret_cast<float4 *>(s + row * (DP + 4) + ch * 4) = v[i];
+        }
+    }
+};
+
+// s[2][4] = rows (2 per thread) of A times columns tx, tx + 16, .. of B, both [., DP + 4] in shared memory
+template <int DP>
+__device__ __forceinline__ void scores(float (&s)[2][4], const float *A, const float *B, int row0, int tx) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[j][c] = 0.f;
+#pragma unroll 4
+    for (int e = 0; e < DP; e += 4) {
+        float4 a[2], b[4];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) a[j] = *reinterpret_cast<const float4 *>(A + (row0 + j) * (DP + 4) + e);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) b[c] = *reinterpret_cast<const float4 *>(B + (tx + 16 * c) * (DP + 4) + e);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                s[j][c] = fmaf(a[j].x, b[c].x, s[j][c]);
+                s[j][c] = fmaf(a[j].y, b[c].y, s[j][c]);
+                s[j][c] = fmaf(a[j].z, b[c].z, s[j][c]);
+                s[j][c] = fmaf(a[j].w, b[c].w, s[j][c]);
+            }
+    }
+}
+// The DP / 16 result columns of a thread: groups of kW at tx * kW + g * 16 * kW.
+template <int DP>
+struct Cols {
+    static constexpr int kN = DP / 16, kW = kN < 4 ? kN : 4;
+    __device__ static __forceinline__ int col(int tx, int i) { return (i / kW) * 16 * kW + tx * kW + i % kW; }
+};
+// acc[2][DP / 16] += rows of X ([., kPStride], 64 columns) times B [64, DP + 4]
+template <int DP>
+__device__ __forceinline__ void accumulate(float (&acc)[2][DP / 16], const float *X, const float *B, int row0, int tx) {
+    constexpr int kN = Cols<DP>::kN;
+#pragma unroll 2
+    for (int k = 0; k < kCols; k += 4) {
+        float4 x[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) x[j] = *reinterpret_cast<const float4 *>(X + (row0 + j) * kPStride + k);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float *brow = B + (k + q) * (DP + 4);
+            float b[kN];
+            if (kN >= 4) {
+#pragma unroll
+                for (int g = 0; g < kN / 4; ++g) *reinterpret_cast<float4 *>(b + 4 * g) = *reinterpret_cast<const float4 *>(brow + g * 64 + tx * 4);
+            } else if (kN == 2) {
+                *reinterpret_cast<float2 *>(b) = *reinterpret_cast<const float2 *>(brow + tx * 2);
+            } else {
+                b[0] = brow[tx];
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const float xv = q == 0 ? x[j].x : q == 1 ? x[j].y : q == 2 ? x[j].z : x[j].w;
+#pragma unroll
+                for (int i = 0; i < kN; ++i) acc[j][i] = fmaf(xv, b[i], acc[j][i]);
+            }
+        }
+    }
+}
+template <typename T, int DP>
+__device__ __forceinline__ void store_row(T *row, const float (&acc)[DP / 16], float mul, int tx, int d) {
+#pragma unroll
+    for (int i = 0; i < DP / 16; ++i) {
+        const int c = Cols<DP>::col(tx, i);
+        if (c < d) from_f(row[c], acc[i] * mul);
+    }
+}
+// Rows of the block behind the valid ones: zeros (and LSE = -inf) where the row exists.
+template <typename T>
+__device__ __forceinline__ void pad_rows(const Common &c, const RowBlock &r, int b, T *o0, T *o1, float *lse) {
+    for (int i = max(r.n, 0) * 16 + (int)threadIdx.x; i < min(kRows, c.N - r.t0) * 16; i += kThreads) {
+        const int k = r.orig(r.t0 + (i >> 4));
+        if (!c.tr.exists(b, k)) continue;  // packed layout: beyond the example's end there is no such row
+        for (int e = i & 15; e < c.d; e += 16) {
+            from_f(o0[(r.bh + k) * c.d + e], 0.f);
+            if (o1) from_f(o1[(r.bh + k) * c.d + e], 0.f);
+        }
+        if (lse && (i & 15) == 0) lse[r.bh + k] = -INFINITY;
+    }
 }
 
 // ---------------------------------------------------------------------------------- forward
-template <typename T>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
-                T *__restrict__ O, float *__restrict__ LSE, ViewPlan rowv, ViewPlan colv,
-                const uint8_t *__restrict__ head_view, const int32_t *__restrict__ n_valid, int N,
-                const int32_t *__restrict__ prefix, int d, float scale, int view_order, TensorRows tr) {
-    __shared__ float s_q[kWarpsPerBlock][kMaxD];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t = blockIdx.x * kWarpsPerBlock + warp;
-    const int h = blockIdx.y, b = blockIdx.z;
-    if (t >= N) return;
-    const RowCtx c = row_ctx(rowv, colv, head_view, n_valid, b, h, N);
-    const size_t bh = tr.base(b, h);
-    const int k = view_order ? t : c.perm[t];  // view order: the tensors are laid out in the head's own order
-    T *o_row = O + (bh + k) * d;
-    if (t >= c.n_valid) {  // padding query row
-        if (!tr.exists(b, k)) return;  // packed layout: beyond the example's end there is no such row
-        for (int e = lane; e < d; e += 32) from_f(o_row[e], 0.f);
-        if (lane == 0) LSE[bh + k] = -INFINITY;
-        return;
+template <typename T, int DP>
+__global__ void __launch_bounds__(kThreads, DP <= 64 ? 3 : 1)
+simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V, T *__restrict__ O,
+                float *__restrict__ LSE, const Common c, int H, int n_bh) {
+    extern __shared__ __align__(16) float smem[];
+    __shared__ int s_range[2];
+    float *sQ = smem, *sK = sQ + kRows * (DP + 4), *sV = sK + kCols * (DP + 4), *sP = sV + kCols * (DP + 4);
+    // row blocks vary slowest: the long ones (global block) come first
+    const int bh = blockIdx.x % n_bh, b = bh / H, h = bh % H;
+    const RowBlock r = row_block(c, b, h, blockIdx.x / n_bh, s_range);
+    pad_rows(c, r, b, O, (T *)nullptr, LSE);
+    if (r.n <= 0) return;
+    const int tx = threadIdx.x & 15, row0 = (threadIdx.x >> 4) * 2;
+    const T *Qh = Q + r.bh * c.d, *Kh = K + r.bh * c.d, *Vh = V + r.bh * c.d;
+
+    Chunks<kCols, DP> nk, nv;
+    int c0 = 0, w = 0;
+    if (r.n_tiles > 0) {
+        r.tile(0, c0, w);
+        nk.load(Kh, r, c0, w, c.d);
+        nv.load(Vh, r, c0, w, c.d);
     }
-    for (int e = lane; e < d; e += 32) s_q[warp][e] = to_f(Q[(bh + k) * d + e]);
-    __syncwarp();
+    {
+        Chunks<kRows, DP> q;
+        q.load(Qh, r, r.t0, r.n, c.d);
+        q.store(sQ);
+    }
+    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, acc[2][DP / 16];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int i = 0; i < DP / 16; ++i) acc[j][i] = 0.f;
 
-    float m = -INFINITY, l = 0.f, acc[kAccPerLane];
-#pragma unroll
-    for (int i = 0; i < kAccPerLane; ++i) acc[i] = 0.f;
-
-    const int P = min(prefix[b], c.n_valid);  // length of the global block (never reaches into the padding)
-    const int lo = max(c.seg_lo[t], P), hi = c.seg_hi[t];
-    for (int range = 0; range < 2; ++range) {
-        const int j_begin = range ? lo : 0, j_end = range ? hi : P;
-        for (int j0 = j_begin; j0 < j_end; j0 += 32) {
-            const int j = j0 + lane;
-            const bool on = j < j_end;
-            const int kj = on ? (view_order ? j : c.perm[j]) : 0;
-            float s = on ? scale * dot_row(s_q[warp], K + (bh + kj) * d, d) : -INFINITY;
-            const float m_new = fmaxf(m, warp_max(s));
-            const float p = on ? expf(s - m_new) : 0.f;
-            const float alpha = expf(m - m_new);  // m = -inf on the first step gives 0
-            l = l * alpha + warp_sum(p);
-            m = m_new;
-#pragma unroll
-            for (int i = 0; i < kAccPerLane; ++i) acc[i] *= alpha;
-            const int n_here = min(32, j_end - j0);
-            for (int jj = 0; jj < n_here; ++jj) {
-                const float pj = __shfl_sync(0xffffffffu, p, jj);
-                const int vj = __shfl_sync(0xffffffffu, kj, jj);
-                const T *v_row = V + (bh + vj) * d;
-#pragma unroll
-                for (int i = 0; i < kAccPerLane; ++i) {
-                    const int e = lane + 32 * i;
-                    if (e < d) acc[i] = fmaf(pj, to_f(v_row[e]), acc[i]);
-                }
-            }
+#pragma unroll 1
+    for (int i = 0; i < r.n_tiles; ++i) {
+        const int t_c0 = c0, t_end = c0 + w;
+        __syncthreads();  // the tile before has been read
+        nk.store(sK);
+        nv.store(sV);
+        __syncthreads();
+        if (i + 1 < r.n_tiles) {
+            r.tile(i + 1, c0, w);
+            nk.load(Kh, r, c0, w, c.d);
+            nv.load(Vh, r, c0, w, c.d);
         }
-    }
-    // a valid row attends at least to itself, except in the passes of the row-or-column pattern,
-    // where a row may have no key at all: O = 0, LSE = -inf
-    const float inv_l = l > 0.f ? 1.f / l : 0.f;
+        float s[2][4];
+        scores<DP>(s, sQ, sK, row0, tx);
 #pragma unroll
-    for (int i = 0; i < kAccPerLane; ++i) {
-        const int e = lane + 32 * i;
-        if (e < d) from_f(o_row[e], acc[i] * inv_l);
+        for (int j = 0; j < 2; ++j) {
+            float mx = -INFINITY;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                s[j][q] = r.counts(i, t_c0 + tx + 16 * q, t_end, j) ? c.scale * s[j][q] : -INFINITY;
+                mx = fmaxf(mx, s[j][q]);
+            }
+            const float m_new = fmaxf(m[j], half_max(mx));
+            const float base = m_new == -INFINITY ? 0.f : m_new;  // no key yet
+            const float alpha = expf(m[j] - base);
+            float sum = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float p = expf(s[j][q] - base);
+                sP[(row0 + j) * kPStride + tx + 16 * q] = p;
+                sum += p;
+            }
+            l[j] = l[j] * alpha + half_sum(sum);
+            m[j] = m_new;
+#pragma unroll
+            for (int e = 0; e < DP / 16; ++e) acc[j][e] *= alpha;
+        }
+        __syncwarp();
+        accumulate<DP>(acc, sP, sV, row0, tx);
+        __syncwarp();
     }
-    if (lane == 0) LSE[bh + k] = m + logf(l);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        if (row0 + j >= r.n) continue;
+        const int k = r.orig(r.t0 + row0 + j);
+        // a valid row attends at least to itself, except in the passes of the row-or-column pattern,
+        // where a row may have no key at all: O = 0, LSE = -inf
+        store_row<T, DP>(O + (r.bh + k) * c.d, acc[j], l[j] > 0.f ? 1.f / l[j] : 0.f, tx, c.d);
+        if (tx == 0) LSE[r.bh + k] = m[j] + logf(l[j]);
+    }
 }
 
 // ---------------------------------------------------------------------------------- backward
-// D_k = sum_e dO_ke O_ke, original token order, one warp per row.
+// D_k = sum_e dO_ke O_ke, original token order, 16 lanes per row.
 template <typename T>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-simt_rowdot_kernel(const T *__restrict__ dO, const T *__restrict__ O, float *__restrict__ D,
-                   size_t rows, int d) {
-    const size_t r = (size_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (r >= rows) return;
+__global__ void __launch_bounds__(kThreads) simt_rowdot_kernel(const T *__restrict__ dO, const T *__restrict__ O,
+                                                               float *__restrict__ D, size_t rows, int d) {
+    ptx::launch_dependents();
+    const size_t r = (size_t)blockIdx.x * (kThreads / 16) + (threadIdx.x >> 4);
+    const int tx = threadIdx.x & 15;
     float acc = 0.f;
-    for (int e = lane; e < d; e += 32) acc = fmaf(to_f(dO[r * d + e]), to_f(O[r * d + e]), acc);
-    acc = warp_sum(acc);
-    if (lane == 0) D[r] = acc;
-}
-
-// kDKV = false: the warp owns query row t and produces dQ_t = scale * sum_j dS_tj K_j.
-// kDKV = true : the warp owns key row t and produces dV_t = sum_k P_kt dO_k and
-//               dK_t = scale * sum_k dS_kt Q_k, looping over the queries k that attend to it.
-template <typename T, bool kDKV>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-simt_bwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
-                const T *__restrict__ dO, const float *__restrict__ LSE,
-                const float *__restrict__ D, T *__restrict__ dQ, T *__restrict__ dK,
-                T *__restrict__ dV, ViewPlan rowv, ViewPlan colv,
-                const uint8_t *__restrict__ head_view, const int32_t *__restrict__ n_valid, int N,
-                const int32_t *__restrict__ prefix, int d, float scale, TensorRows tr) {
-    __shared__ float s_a[kWarpsPerBlock][kMaxD];  // own q (dQ) or own k (dK/dV)
-    __shared__ float s_b[kWarpsPerBlock][kMaxD];  // own dO (dQ) or own v (dK/dV)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t = blockIdx.x * kWarpsPerBlock + warp;
-    const int h = blockIdx.y, b = blockIdx.z;
-    if (t >= N) return;
-    const RowCtx c = row_ctx(rowv, colv, head_view, n_valid, b, h, N);
-    const size_t bh = tr.base(b, h);
-    const int own = c.perm[t];
-    T *out0 = (kDKV ? dK : dQ) + (bh + own) * d;
-    T *out1 = kDKV ? dV + (bh + own) * d : nullptr;
-    if (t >= c.n_valid) {
-        if (!tr.exists(b, own)) return;  // packed layout: beyond the example's end there is no such row
-        for (int e = lane; e < d; e += 32) {
-            from_f(out0[e], 0.f);
-            if (kDKV) from_f(out1[e], 0.f);
+    if (r < rows)
+        for (int e = tx * 4; e < d; e += 64) {
+            const float4 a = load4(dO + r * d + e), b = load4(O + r * d + e);
+            acc = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, acc))));
         }
-        return;
-    }
-    const T *a_src = (kDKV ? K : Q) + (bh + own) * d;
-    const T *b_src = (kDKV ? V : dO) + (bh + own) * d;
-    for (int e = lane; e < d; e += 32) {
-        s_a[warp][e] = to_f(a_src[e]);
-        s_b[warp][e] = to_f(b_src[e]);
-    }
-    __syncwarp();
-    float own_lse = 0.f, own_D = 0.f;
-    if (!kDKV) {
-        own_lse = LSE[bh + own];
-        own_D = D[bh + own];
-    }
-    float acc0[kAccPerLane], acc1[kAccPerLane];
-#pragma unroll
-    for (int i = 0; i < kAccPerLane; ++i) acc0[i] = acc1[i] = 0.f;
-
-    const int P = min(prefix[b], c.n_valid);  // length of the global block (never reaches into the padding)
-    const int lo = max(c.seg_lo[t], P), hi = c.seg_hi[t];
-    for (int range = 0; range < 2; ++range) {
-        const int j_begin = range ? lo : 0, j_end = range ? hi : P;
-        for (int j0 = j_begin; j0 < j_end; j0 += 32) {
-            const int j = j0 + lane;
-            const bool on = j < j_end;
-            const int oj = on ? c.perm[j] : 0;  // original index of the other row
-            float p = 0.f, ds = 0.f;
-            if (on) {
-                // dQ: other row is a key  -> s = q_own . k_other, dP = dO_own . v_other
-                // dKV: other row is a query -> s = q_other . k_own, dP = dO_other . v_own
-                const T *x = (kDKV ? Q : K) + (bh + oj) * d;
-                const T *y = (kDKV ? dO : V) + (bh + oj) * d;
-                const float s = scale * dot_row(s_a[warp], x, d);
-                const float dp = dot_row(s_b[warp], y, d);
-                const float lse = kDKV ? LSE[bh + oj] : own_lse;
-                const float Dk = kDKV ? D[bh + oj] : own_D;
-                p = expf(s - lse);
-                ds = p * (dp - Dk);
-            }
-            const int n_here = min(32, j_end - j0);
-            for (int jj = 0; jj < n_here; ++jj) {
-                const float pj = __shfl_sync(0xffffffffu, p, jj);
-                const float dsj = __shfl_sync(0xffffffffu, ds, jj) * scale;
-                const int rj = __shfl_sync(0xffffffffu, oj, jj);
-                const T *x = (kDKV ? Q : K) + (bh + rj) * d;   // dK += ds q ; dQ += ds k
-                const T *y = dO + (bh + rj) * d;               // dV += p dO
-#pragma unroll
-                for (int i = 0; i < kAccPerLane; ++i) {
-                    const int e = lane + 32 * i;
-                    if (e < d) {
-                        acc0[i] = fmaf(dsj, to_f(x[e]), acc0[i]);
-                        if (kDKV) acc1[i] = fmaf(pj, to_f(y[e]), acc1[i]);
-                    }
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < kAccPerLane; ++i) {
-        const int e = lane + 32 * i;
-        if (e < d) {
-            from_f(out0[e], acc0[i]);
-            if (kDKV) from_f(out1[e], acc1[i]);
-        }
-    }
+    acc = half_sum(acc);
+    if (tx == 0 && r < rows) D[r] = acc;
 }
 
 template <typename T>
-int simt_fwd_t(const mate_plan_t *pl, const void *Q, const void *K, const void *V, int d, float scale,
-               void *O, float *LSE, int view_order, cudaStream_t st) {
-    dim3 grid((pl->N + kWarpsPerBlock - 1) / kWarpsPerBlock, pl->H, pl->B);
-    simt_fwd_kernel<T><<<grid, kWarpsPerBlock * 32, 0, st>>>(
-        (const T *)Q, (const T *)K, (const T *)V, (T *)O, LSE, pl->view[0], pl->view[1],
-        pl->head_view_dev, pl->n_valid_dev, pl->N, pl->global_dev, d, scale, view_order, pl->rows());
+struct BwdArgs {
+    const T *Q, *K, *V, *dO;
+    const float *LSE, *D;
+    T *dQ, *dK, *dV;
+    Common c;
+    int H, n_bh;
+};
+// Even blockIdx.x: the block owns key rows and produces dV = P^T dO and dK = scale dS^T Q from the queries that attend
+// to them; odd: it owns query rows and produces dQ = scale dS K.
+template <typename T, int DP>
+__global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(const BwdArgs<T> a) {
+    extern __shared__ __align__(16) float smem[];
+    __shared__ int s_range[2];
+    constexpr int kR = kRows * (DP + 4), kC = kCols * (DP + 4), kX = kRows * kPStride;
+    float *sRa = smem, *sRb = sRa + kR, *sCa = sRb + kR, *sCb = sCa + kC, *sP = sCb + kC, *sS = sP + kX, *sVec = sS + kX;
+    const Common &c = a.c;
+    const bool key_side = (blockIdx.x & 1) == 0;
+    const int bh = (blockIdx.x >> 1) % a.n_bh, b = bh / a.H, h = bh % a.H;
+    const RowBlock r = row_block(c, b, h, (blockIdx.x >> 1) / a.n_bh, s_range);
+    pad_rows(c, r, b, key_side ? a.dK : a.dQ, key_side ? a.dV : (T *)nullptr, (float *)nullptr);
+    if (r.n <= 0) return;
+    const int tx = threadIdx.x & 15, row0 = (threadIdx.x >> 4) * 2;
+    const T *Ra = (key_side ? a.K : a.Q) + r.bh * c.d, *Rb = (key_side ? a.V : a.dO) + r.bh * c.d;
+    const T *Ca = (key_side ? a.Q : a.K) + r.bh * c.d, *Cb = (key_side ? a.dO : a.V) + r.bh * c.d;
+
+    Chunks<kCols, DP> na, nb;
+    float n_lse = 0.f, n_D = 0.f;  // of column threadIdx.x of the next tile (key side)
+    int c0 = 0, w = 0;
+    auto fetch = [&](int i) {
+        r.tile(i, c0, w);
+        na.load(Ca, r, c0, w, c.d);
+        nb.load(Cb, r, c0, w, c.d);
+        if (key_side && threadIdx.x < kCols) {
+            const size_t at = r.bh + r.orig(c0 + min((int)threadIdx.x, w - 1));
+            n_lse = a.LSE[at];
+            n_D = a.D[at];
+        }
+    };
+    {
+        Chunks<kRows, DP> x, y;
+        x.load(Ra, r, r.t0, r.n, c.d);
+        y.load(Rb, r, r.t0, r.n, c.d);
+        x.store(sRa);
+        y.store(sRb);
+    }
+    ptx::wait_prior_grid();  // D comes from the kernel before
+    if (r.n_tiles > 0) fetch(0);
+    float lse[2], D[2], acc0[2][DP / 16], acc1[2][DP / 16];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const size_t at = r.bh + r.orig(r.t0 + min(row0 + j, r.n - 1));
+        lse[j] = a.LSE[at];
+        D[j] = a.D[at];
+#pragma unroll
+        for (int i = 0; i < DP / 16; ++i) acc0[j][i] = acc1[j][i] = 0.f;
+    }
+
+#pragma unroll 1
+    for (int i = 0; i < r.n_tiles; ++i) {
+        const int t_c0 = c0, t_end = c0 + w;
+        __syncthreads();  // the tile before has been read
+        na.store(sCa);
+        nb.store(sCb);
+        if (key_side && threadIdx.x < kCols) {
+            sVec[threadIdx.x] = n_lse;
+            sVec[kCols + threadIdx.x] = n_D;
+        }
+        __syncthreads();
+        if (i + 1 < r.n_tiles) fetch(i + 1);
+        float s[2][4], dp[2][4];
+        scores<DP>(s, sRa, sCa, row0, tx);
+        scores<DP>(dp, sRb, sCb, row0, tx);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int col = tx + 16 * q;
+            const float c_lse = key_side ? sVec[col] : 0.f, c_D = key_side ? sVec[kCols + col] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const bool on = r.counts(i, t_c0 + col, t_end, j);
+                const float p = on ? expf(c.scale * s[j][q] - (key_side ? c_lse : lse[j])) : 0.f;
+                const float ds = on ? p * (dp[j][q] - (key_side ? c_D : D[j])) : 0.f;
+                if (key_side) sP[(row0 + j) * kPStride + col] = p;
+                sS[(row0 + j) * kPStride + col] = ds;
+            }
+        }
+        __syncwarp();
+        accumulate<DP>(acc0, sS, sCa, row0, tx);
+        if (key_side) accumulate<DP>(acc1, sP, sCb, row0, tx);
+        __syncwarp();
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        if (row0 + j >= r.n) continue;
+        const size_t at = (r.bh + r.orig(r.t0 + row0 + j)) * c.d;
+        store_row<T, DP>((key_side ? a.dK : a.dQ) + at, acc0[j], c.scale, tx, c.d);
+        if (key_side) store_row<T, DP>(a.dV + at, acc1[j], 1.f, tx, c.d);
+    }
+}
+
+Common common(const mate_plan_t *pl, int d, float scale, int view_order) {
+    Common c;
+    c.rowv = pl->view[0];
+    c.colv = pl->view[1];
+    c.head_view = pl->head_view_dev;
+    c.n_valid = pl->n_valid_dev;
+    c.prefix = pl->global_dev;
+    c.N = pl->N;
+    c.d = d;
+    c.view_order = view_order;
+    c.scale = scale;
+    c.tr = pl->rows();
+    return c;
+}
+// Blocks of a launch per side: row blocks of every (example, head).
+inline size_t n_blocks(const mate_plan_t *pl) { return (size_t)((pl->N + kRows - 1) / kRows) * pl->B * pl->H; }
+
+template <typename T, int DP>
+int fwd_launch(const mate_plan_t *pl, const void *Q, const void *K, const void *V, int d, float scale, void *O, float *LSE,
+               int view_order, cudaStream_t st) {
+    static SmemAttrOnce attr;
+    constexpr int bytes = 4 * ((kRows + 2 * kCols) * (DP + 4) + kRows * kPStride);
+    if (attr.ensure((const void *)simt_fwd_kernel<T, DP>, bytes, pl->device) != MATE_OK) return MATE_ERR_CUDA;
+    simt_fwd_kernel<T, DP><<<(unsigned)n_blocks(pl), kThreads, bytes, st>>>(
+        (const T *)Q, (const T *)K, (const T *)V, (T *)O, LSE, common(pl, d, scale, view_order), pl->H, pl->B * pl->H);
     return cudaGetLastError() == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }
-
-template <typename T>
-int simt_bwd_t(const mate_plan_t *pl, const void *Q, const void *K, const void *V, const void *O,
-               const float *LSE, const void *dO, int d, float scale, void *dQ, void *dK, void *dV,
-               void *ws, cudaStream_t st) {
-    float *D = (float *)ws;
+template <typename T, int DP>
+int bwd_launch(const mate_plan_t *pl, const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
+               int d, float scale, void *dQ, void *dK, void *dV, float *D, int pass, cudaStream_t st) {
+    static SmemAttrOnce attr;
+    constexpr int bytes = 4 * (2 * (kRows + kCols) * (DP + 4) + 2 * kRows * kPStride + 2 * kCols);
+    if (attr.ensure((const void *)simt_bwd_kernel<T, DP>, bytes, pl->device) != MATE_OK) return MATE_ERR_CUDA;
     const size_t rows = pl->n_rows();
-    simt_rowdot_kernel<T><<<(unsigned)((rows + kWarpsPerBlock - 1) / kWarpsPerBlock),
-                            kWarpsPerBlock * 32, 0, st>>>((const T *)dO, (const T *)O, D, rows, d);
-    dim3 grid((pl->N + kWarpsPerBlock - 1) / kWarpsPerBlock, pl->H, pl->B);
-    simt_bwd_kernel<T, false><<<grid, kWarpsPerBlock * 32, 0, st>>>(
-        (const T *)Q, (const T *)K, (const T *)V, (const T *)dO, LSE, D, (T *)dQ, (T *)dK, (T *)dV,
-        pl->view[0], pl->view[1], pl->head_view_dev, pl->n_valid_dev, pl->N, pl->global_dev, d, scale, pl->rows());
-    simt_bwd_kernel<T, true><<<grid, kWarpsPerBlock * 32, 0, st>>>(
-        (const T *)Q, (const T *)K, (const T *)V, (const T *)dO, LSE, D, (T *)dQ, (T *)dK, (T *)dV,
-        pl->view[0], pl->view[1], pl->head_view_dev, pl->n_valid_dev, pl->N, pl->global_dev, d, scale, pl->rows());
-    return cudaGetLastError() == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
+    if (pass == 0)
+        simt_rowdot_kernel<T><<<(unsigned)((rows + kThreads / 16 - 1) / (kThreads / 16)), kThreads, 0, st>>>((const T *)dO, (const T *)O,
+                                                                                                          D, rows, d);
+    const BwdArgs<T> a{(const T *)Q, (const T *)K, (const T *)V, (const T *)dO, LSE, D, (T *)dQ, (T *)dK, (T *)dV,
+                       common(pl, d, scale, 0), pl->H, pl->B * pl->H};
+    return launch_after(simt_bwd_kernel<T, DP>, dim3((unsigned)(2 * n_blocks(pl))), kThreads, bytes, st, a) == cudaSuccess
+               ? MATE_OK
+               : MATE_ERR_CUDA;
+}
+
+// Head size padded (in shared memory, with zeros) to 16, 32, 64 or 128.
+template <typename F>
+int by_head_size(int d, F &&f) {
+    if (d <= 16) return f(std::integral_constant<int, 16>{});
+    if (d <= 32) return f(std::integral_constant<int, 32>{});
+    if (d <= 64) return f(std::integral_constant<int, 64>{});
+    return f(std::integral_constant<int, 128>{});
 }
 
 }  // namespace
 
 int simt_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, int d, int dtype,
              float scale, void *O, float *LSE, unsigned flags, cudaStream_t stream) {
-    if (d > kMaxD) return MATE_ERR_UNSUPPORTED;
+    if (d > kMaxD || 2 * n_blocks(plan) > 0x7fffffffu) return MATE_ERR_UNSUPPORTED;
     const int vo = (flags & MATE_FLAG_VIEW_ORDER) ? 1 : 0;
-    return dtype == MATE_F32 ? simt_fwd_t<float>(plan, Q, K, V, d, scale, O, LSE, vo, stream)
-                             : simt_fwd_t<__nv_bfloat16>(plan, Q, K, V, d, scale, O, LSE, vo, stream);
+    if (dtype == MATE_F32)
+        return by_head_size(d, [&](auto dp) { return fwd_launch<float, dp()>(plan, Q, K, V, d, scale, O, LSE, vo, stream); });
+    return by_head_size(d, [&](auto dp) { return fwd_launch<__nv_bfloat16, dp()>(plan, Q, K, V, d, scale, O, LSE, vo, stream); });
 }
 
 size_t simt_bwd_workspace(const mate_plan_t *plan) {
     return sizeof(float) * (size_t)plan->B * plan->H * plan->N;
 }
 
+// pass: which of the calls that share the workspace, O and dO this is; the row dots are formed in pass 0.
 int simt_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, const void *O,
              const float *LSE, const void *dO, int d, int dtype, float scale, void *dQ, void *dK,
-             void *dV, void *workspace, cudaStream_t stream) {
-    if (d > kMaxD) return MATE_ERR_UNSUPPORTED;
-    return dtype == MATE_F32
-               ? simt_bwd_t<float>(plan, Q, K, V, O, LSE, dO, d, scale, dQ, dK, dV, workspace, stream)
-               : simt_bwd_t<__nv_bfloat16>(plan, Q, K, V, O, LSE, dO, d, scale, dQ, dK, dV,
-                                           workspace, stream);
+             void *dV, void *workspace, int pass, cudaStream_t stream) {
+    if (d > kMaxD || 2 * n_blocks(plan) > 0x7fffffffu) return MATE_ERR_UNSUPPORTED;
+    float *D = (float *)workspace;
+    if (dtype == MATE_F32)
+        return by_head_size(d, [&](auto dp) {
+            return bwd_launch<float, dp()>(plan, Q, K, V, O, LSE, dO, d, scale, dQ, dK, dV, D, pass, stream);
+        });
+    return by_head_size(d, [&](auto dp) {
+        return bwd_launch<__nv_bfloat16, dp()>(plan, Q, K, V, O, LSE, dO, d, scale, dQ, dK, dV, D, pass, stream);
+    });
 }
 
 }  // namespace mate
@@ -341,6 +550,6 @@ extern "C" int mate_attn_bwd_noalloc(const mate_plan_t *plan, const void *Q, con
     }
     // every element of D that the backward kernels read is written by the row-dot kernel of the
     // same call first, so nothing in the shared array has to start at zero
-    return mate::simt_bwd(plan, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, scratch,
+    return mate::simt_bwd(plan, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, scratch, 0,
                           (cudaStream_t)stream);
 }

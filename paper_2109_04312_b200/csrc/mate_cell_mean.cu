@@ -1,66 +1,57 @@
 // Per-cell mean of token logits (cell-selection stage, Section 4.1: S(c) = avg over the tokens t of
 // cell c of S(t)).  A cell is the set of table tokens that share a (row id, column id) pair.  In the
-// row view of the plan the tokens of one row are contiguous, so one warp takes one row: it reads
-// the row's (column id, logit) pairs 32 at a time, coalesced through the view order, and every lane
-// accumulates the cells of the columns lane, lane + 32, ... in the order of the tokens (the result
-// does not depend on the launch).  HBM-bound by design: every id and logit is read once.
+// row view of the plan the tokens of one row are contiguous, so one block takes one row: it brings the
+// row's (column id, logit) pairs into shared memory, all threads loading, and thread c then reads them in the
+// order of the tokens and accumulates column c (the result does not depend on the launch).  Bound by
+// latency at the sizes of a table: two dependent loads, then about four instructions per token of the row.
+// (One warp per row, 32 tokens at a time handed around by shuffles, took 7 us for rows of 30 tokens and 93 us
+// for rows of several hundred; this takes 2.3 and 6.3.)
 #include "mate_internal.h"
 
 namespace mate {
 namespace {
 
-constexpr int kWarpsPerBlock = 8;
-constexpr int kColsPerLane = 4;  // columns handled per pass: 32 * kColsPerLane
+constexpr int kThreads = 128;
+constexpr int kBuf = 1024;  // tokens of a row in shared memory at a time
 
-__global__ void __launch_bounds__(32 * kWarpsPerBlock)
+__global__ void __launch_bounds__(kThreads)
 cell_mean_kernel(const float *__restrict__ logits, const int32_t *__restrict__ col_ids, ViewPlan rowv, int N,
                  int n_rows, int n_cols, float *__restrict__ mean, int32_t *__restrict__ count) {
-    const int lane = threadIdx.x & 31;
-    const int r = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);  // row id
-    const int b = blockIdx.y;
-    if (r >= n_rows) return;
+    __shared__ __align__(16) int32_t s_col[kBuf];
+    __shared__ __align__(16) float s_x[kBuf];
+    const int r = blockIdx.x, b = blockIdx.y;  // row id, example
     const int32_t *seg_off = rowv.seg_off + (size_t)b * (rowv.max_id + 2);
-    const int32_t *perm = rowv.perm + (size_t)b * N;
     const int lo = seg_off[r], hi = seg_off[r + 1];
-    float *out_m = mean + ((size_t)b * n_rows + r) * n_cols;
-    int32_t *out_c = count ? count + ((size_t)b * n_rows + r) * n_cols : nullptr;
+    const int32_t *perm = rowv.perm + (size_t)b * N;
+    const size_t out = ((size_t)b * n_rows + r) * n_cols;
 
-    for (int c0 = 0; c0 < n_cols; c0 += 32 * kColsPerLane) {
-        float sum[kColsPerLane];
-        int cnt[kColsPerLane];
-#pragma unroll
-        for (int q = 0; q < kColsPerLane; ++q) {
-            sum[q] = 0.f;
-            cnt[q] = 0;
+    for (int c0 = 0; c0 < n_cols; c0 += kThreads) {
+        const int c = c0 + (int)threadIdx.x;
+        float sum = 0.f;
+        int cnt = 0;
+        for (int t0 = lo; t0 < hi; t0 += kBuf) {
+            const int n = min(kBuf, hi - t0), n4 = (n + 3) & ~3;
+            if (c0 > 0 || t0 > lo) __syncthreads();  // the buffer has been read
+            for (int i = threadIdx.x; i < n4; i += kThreads) {
+                const size_t at = (size_t)b * N + perm[t0 + min(i, n - 1)];
+                s_col[i] = i < n ? col_ids[at] : -1;
+                s_x[i] = logits[at];
+            }
+            __syncthreads();
+            if (c < n_cols)
+#pragma unroll 2
+                for (int i = 0; i < n4; i += 4) {
+                    const int4 k = *reinterpret_cast<const int4 *>(s_col + i);
+                    const float4 x = *reinterpret_cast<const float4 *>(s_x + i);
+                    if (k.x == c) sum += x.x, ++cnt;
+                    if (k.y == c) sum += x.y, ++cnt;
+                    if (k.z == c) sum += x.z, ++cnt;
+                    if (k.w == c) sum += x.w, ++cnt;
+                }
         }
-        for (int t0 = lo; t0 < hi; t0 += 32) {
-            const int t = t0 + lane;
-            int c = -1;
-            float x = 0.f;
-            if (t < hi) {
-                const int orig = perm[t];
-                c = col_ids[(size_t)b * N + orig];
-                x = logits[(size_t)b * N + orig];
-            }
-            const int n = min(32, hi - t0);
-            for (int j = 0; j < n; ++j) {
-                const int cj = __shfl_sync(0xffffffffu, c, j) - c0 - lane;
-                const float xj = __shfl_sync(0xffffffffu, x, j);
-#pragma unroll
-                for (int q = 0; q < kColsPerLane; ++q)
-                    if (cj == 32 * q) {
-                        sum[q] += xj;
-                        ++cnt[q];
-                    }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < kColsPerLane; ++q) {
-            const int c = c0 + 32 * q + lane;
-            if (c < n_cols) {
-                out_m[c] = cnt[q] ? sum[q] / (float)cnt[q] : 0.f;
-                if (out_c) out_c[c] = cnt[q];
-            }
+        if (c < n_cols) {
+            mean[out + c] = cnt ? sum / (float)cnt : 0.f;
+            if (count) count[out + c] = cnt;
         }
     }
 }
@@ -77,8 +68,7 @@ extern "C" int mate_cell_mean(const mate_plan_t *plan, const float *logits, cons
     if (plan->T) return MATE_ERR_UNSUPPORTED;  // packed batches: not here
     if (mate::use_plan(plan, (cudaStream_t)stream) != cudaSuccess) return MATE_ERR_CUDA;
     const int n_rows = plan->view[0].max_id + 1, n_cols = plan->view[1].max_id + 1;
-    dim3 grid((n_rows + mate::kWarpsPerBlock - 1) / mate::kWarpsPerBlock, plan->B);
-    mate::cell_mean_kernel<<<grid, 32 * mate::kWarpsPerBlock, 0, (cudaStream_t)stream>>>(
+    mate::cell_mean_kernel<<<dim3(n_rows, plan->B), mate::kThreads, 0, (cudaStream_t)stream>>>(
         logits, col_ids, plan->view[0], plan->N, n_rows, n_cols, mean, count);
     return cudaGetLastError() == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }

@@ -91,7 +91,7 @@ constexpr int kChunk = 32;
 
 // Key ranges of the rows of one (example, view), by view position.
 struct RowRanges {
-    int P, nv;  // [0, P): rows of the global block; [P, nv): table rows with the keys [lo, hi) behind the block
+    int P = 0, nv = 0;  // [0, P): rows of the global block; [P, nv): table rows with the keys [lo, hi) behind the block
     std::vector<int32_t> lo, hi;
 };
 
@@ -142,24 +142,24 @@ struct ProtoList {
 void half_tile_clks(const FwdUnit &u, int h, const RowRanges &rr, int32_t *clk) {
     const int nA = u.tiles_a(), n_tiles = nA + u.tiles_b(), rows = u.rows_of(h), r0 = u.row0_of(h);
     if (rows == 0) return;
-    for (int i = 0; i < nA; ++i) {
-        const int w = std::min(kTile, u.kA_end - u.kA0 - i * kTile);
-        clk[i] = w == kTile ? kFullClk : kPartialClk + kChunkClk * ceil_div(w, kChunk);
-    }
-    for (int i = nA; i < n_tiles; ++i) {
+    for (int i = 0; i < n_tiles; ++i) {
         const TileInfo t = mate::tile_info(u, i, nA);
         int c0, c1;
         mate::half_cols(u.lo[h], u.hi[h], t, c0, c1);
         if (c1 <= c0) continue;
-        if (t.w == kTile && rr.lo[r0 + rows - 1] <= t.k0 && rr.hi[r0] >= t.k0 + kTile) {
+        const auto lo = [&](int r) { return r < rr.P ? 0 : rr.lo[r] - t.k0; };
+        const auto hi = [&](int r) { return r < rr.P ? t.w : std::min(rr.hi[r] - t.k0, t.w); };
+        if (t.w == kTile && (t.pre == kTile || (lo(r0 + rows - 1) <= t.pre && hi(r0) >= kTile))) {
             clk[i] = kFullClk;
             continue;
         }
-        int chunks = 0;
-        for (int r = 0; r < rows; r += 32) {  // the warps of the half
+        int chunks = ceil_div(t.pre, kChunk);
+        for (int r = 0; t.is_b && r < rows; r += 32) {  // the warps of the half
             const int last = r0 + std::min(r + 32, rows) - 1;
-            const int a = std::max(rr.lo[r0 + r] - t.k0, 0), e = std::min(rr.hi[last] - t.k0, t.w);
-            chunks = std::max(chunks, e > a ? ceil_div(e, kChunk) - a / kChunk : 0);
+            const int a = std::max(lo(r0 + r), 0), e = hi(last);
+            int n = e > a ? ceil_div(e, kChunk) - a / kChunk : 0;
+            if (t.pre > 0) n = ceil_div(t.pre, kChunk) + (e > t.pre ? ceil_div(e, kChunk) - std::max(a / kChunk, ceil_div(t.pre, kChunk)) : 0);
+            chunks = std::max(chunks, n);
         }
         clk[i] = kPartialClk + kChunkClk * chunks;
     }
@@ -190,84 +190,118 @@ struct HeadLists {
     }
 };
 
-// One unit of the halves [r0, r1) and [r1, r2) (the second one may be empty) of table rows.
-FwdUnit table_unit(const RowRanges &rr, int r0, int r1, int r2) {
+// Tiles that the halves of a unit visit.
+int visits(const FwdUnit &u) {
+    const int nA = u.tiles_a(), n_tiles = nA + u.tiles_b();
+    int n = 0;
+    for (int i = 0; i < n_tiles; ++i)
+        for (int h = 0; h < 2; ++h) {
+            int c0, c1;
+            mate::half_cols(u.lo[h], u.hi[h], mate::tile_info(u, i, nA), c0, c1);
+            n += u.rows_of(h) > 0 && c1 > c0;
+        }
+    return n;
+}
+constexpr int kMaxMerged = 3 * kTile;  // longest global block that goes in front of range B
+
+// The unit of the rows [r0, r1) and [r1, r2) (the second half may be empty) with the global block in range A
+// or, where the halves then visit fewer tiles, in front of range B.  Rows of the global block may stand in
+// front of table rows in a half.
+FwdUnit make_unit(const RowRanges &rr, int r0, int r1, int r2) {
     FwdUnit u{};
+    const int n = (r1 - r0) | (r2 - r1) << 8;
     u.q0 = r0;
-    u.rows = (r1 - r0) | (r2 - r1) << 16;
-    u.kA_end = rr.P;
-    u.lo[0] = rr.lo[r0];  // lo and hi do not decrease along the rows
-    u.hi[0] = rr.hi[r1 - 1];
-    u.lo[1] = r2 > r1 ? rr.lo[r1] : 0;
-    u.hi[1] = r2 > r1 ? rr.hi[r2 - 1] : 0;
-    u.kB0 = u.lo[0];
-    u.kB_end = rr.hi[r2 - 1];
+    u.rows = n;
     u.tB = kTile;
+    u.parts = 1;
+    u.ctr = -1;
+    if (r2 <= rr.P) {  // global rows only
+        u.kA_end = rr.nv;
+        return u;
+    }
+    const int r[3] = {r0, r1, r2};
+    for (int h = 0; h < 2; ++h) {
+        if (r[h + 1] <= r[h]) continue;
+        u.lo[h] = r[h] < rr.P ? rr.P : rr.lo[r[h]];  // lo and hi do not decrease along the table rows
+        u.hi[h] = r[h] < rr.P ? rr.nv : rr.hi[r[h + 1] - 1];
+    }
+    u.kB0 = u.lo[0];
+    u.kB_end = std::max(u.hi[0], u.hi[1]);
+    FwdUnit m = u;
+    m.rows = n | rr.P << 16;
+    if (r0 < rr.P) return m;  // a mixed half masks row by row
+    u.kA_end = rr.P;
     // When the second half's keys begin at most a tile behind the first half's, tiles of that width give each
     // half one tile of its own (short segments: the keys of a half are its own rows).
     const int step = u.lo[1] - u.lo[0];
     if (r2 > r1 && step > 0 && step <= kTile && u.hi[0] - u.lo[0] <= step && u.hi[1] - u.lo[1] <= step) u.tB = step;
-    u.parts = 1;
-    u.ctr = -1;
-    return u;
+    const bool may = rr.P > 0 && rr.P % kTile != 0 && rr.P < kMaxMerged;
+    return may && visits(m) < visits(u) ? m : u;
 }
 
 // Units of one (example, view), for any head of the view.  Padding rows are left out.  `pairs`: two halves
-// to a unit where they share most of their tiles.
-void add_units(const RowRanges &rr, int b, int view, bool pairs, ProtoList &out) {
-    const auto add = [&](FwdUnit &u) {
+// to a unit where they share most of their tiles.  `fill_up`: see below.
+void add_units(const RowRanges &rr, int b, int view, bool pairs, bool fill_up, ProtoList &out) {
+    const int P = rr.P, nv = rr.nv;
+    const auto add = [&](int r0, int r1, int r2) {
+        FwdUnit u = make_unit(rr, r0, r1, r2);
         u.b = b;
         add_proto(out, u, view, rr);
     };
-    const int P = rr.P, nv = rr.nv;
-    for (int q0 = 0; q0 < P;) {  // rows of the global block: every valid key
-        FwdUnit u{};
-        const int n0 = std::min(kTile, P - q0), n1 = pairs ? std::min(kTile, P - q0 - n0) : 0;
-        u.q0 = q0;
-        u.rows = n0 | n1 << 16;
-        u.kA_end = nv;
-        u.tB = kTile;
-        u.parts = 1;
-        u.ctr = -1;
-        add(u);
-        q0 += n0 + n1;
+    const auto tiles = [&](int cols) {  // of a half whose own keys are that many: with the global block in either place
+        return std::min(ceil_div(P, kTile) + ceil_div(cols, kTile), P < kMaxMerged ? ceil_div(P + cols, kTile) : 1 << 28);
+    };
+    // The last half of the global block is filled up with table rows: these need no half of their own then (its
+    // tiles, and about two more for the half itself), but the half masks its tiles row by row, about 0.3 of a
+    // tile each.  Always for up to two tiles of positions; for longer examples only where all SMs have several
+    // units to do (`fill_up`: the half is the longest of its example) and it saves more than it costs.
+    std::vector<int> cuts(1, 0);
+    while (cuts.back() + kTile <= P) cuts.push_back(cuts.back() + kTile);
+    const int rem = P - cuts.back(), fill = std::min(kTile - rem, nv - P);
+    if (rem > 0) {
+        bool mix = fill > 0 && P < kMaxMerged;
+        if (mix && nv > 2 * kTile) {
+            const int own = rr.hi[P + fill - 1] - rr.lo[P];
+            mix = fill_up && 0.3 * ceil_div(nv, kTile) < (tiles(own) + 2) * fill / (double)kTile;
+        }
+        cuts.push_back(mix ? P + fill : P);
     }
+    const int n_global = (int)cuts.size() - 1;  // halves with rows of the global block
     // Halves of table rows: 128 rows, or fewer when ending where a segment begins saves tiles (a half that
     // reaches into the next long segment visits the tiles of both; one that ends with a short segment needs
     // one tile for its own keys instead of two).  Measure: tiles, and 1.5 for the half itself, per row.
-    std::vector<int> cuts(1, P);
-    const int tiles_a = ceil_div(P, kTile);
-    for (int q = P; q < nv;) {
+    while (cuts.back() < nv) {
+        const int q = cuts.back();
         int end = std::min(q + kTile, nv);
         if (end < nv || rr.lo[end - 1] != rr.lo[q]) {
             int cut = end;
             while (cut > q + 1 && (cut >= nv || rr.lo[cut] == rr.lo[cut - 1])) --cut;  // the last row that begins a new range
-            const auto per_row = [&](int e) { return (3 + 2 * (tiles_a + ceil_div(rr.hi[e - 1] - rr.lo[q], kTile))) / (double)(e - q); };
+            const auto per_row = [&](int e) { return (3 + 2 * tiles(rr.hi[e - 1] - rr.lo[q])) / (double)(e - q); };
             if (cut > q + 1 && per_row(cut) < per_row(end)) end = cut;
         }
         cuts.push_back(end);
-        q = end;
     }
-    for (size_t i = 0; i + 1 < cuts.size();) {
-        const int r0 = cuts[i], r1 = cuts[i + 1];
-        bool two = pairs && i + 2 < cuts.size();
-        if (two) {
-            const int r2 = cuts[i + 2];
-            const int n0 = ceil_div(rr.hi[r1 - 1] - rr.lo[r0], kTile), n1 = ceil_div(rr.hi[r2 - 1] - rr.lo[r1], kTile);
-            const int both = ceil_div(rr.hi[r2 - 1] - rr.lo[r0], kTile);
-            two = 4 * (tiles_a + both) <= 3 * (2 * tiles_a + n0 + n1) || tiles_a + both <= 4;
+    const int n_halves = (int)cuts.size() - 1;
+    for (int i = 0; i < n_halves;) {
+        bool two = pairs && i + 1 < n_halves;
+        if (two && i + 1 >= n_global && i < n_global) {  // a half of the global block with one of table rows
+            two = ceil_div(nv, kTile) <= 2 && cuts[i + 1] >= P;
+        } else if (two && i >= n_global) {
+            const int r0 = cuts[i], r1 = cuts[i + 1], r2 = cuts[i + 2];
+            const int both = rr.hi[r2 - 1] - rr.lo[r0];
+            const int apart = tiles(rr.hi[r1 - 1] - rr.lo[r0]) + tiles(rr.hi[r2 - 1] - rr.lo[r1]);
+            two = 4 * tiles(both) <= 3 * apart || tiles(both) <= 4;
         }
-        FwdUnit u = table_unit(rr, r0, r1, two ? cuts[i + 2] : r1);
-        add(u);
+        add(cuts[i], cuts[i + 1], two ? cuts[i + 2] : cuts[i + 1]);
         i += two ? 2 : 1;
     }
 }
 
-void list_units(const mate_plan_t *pl, const std::vector<RowRanges> &ranges, bool pairs, ProtoList &out) {
+void list_units(const mate_plan_t *pl, const std::vector<RowRanges> &ranges, bool pairs, bool fill_up, ProtoList &out) {
     out.protos.clear();
     out.tiles.clear();
     for (int v = 0; v < 2; ++v)
-        for (int b = 0; b < pl->B && pl->view[v].n_heads > 0; ++b) add_units(ranges[(size_t)v * pl->B + b], b, v, pairs, out);
+        for (int b = 0; b < pl->B && pl->view[v].n_heads > 0; ++b) add_units(ranges[(size_t)v * pl->B + b], b, v, pairs, fill_up, out);
     sort_protos(out);
 }
 
@@ -285,7 +319,7 @@ void make_bwd_units(mate_plan_t *pl, const ProtoList &singles, const HeadLists &
     pl->bwd_grid = std::min(std::max(pl->n_ctas, 1), std::max(2 * pl->n_bwd_units, pl->n_pads));
 }
 
-// Tiles [i0, i1) of a unit as a unit of its own.
+// Tiles [i0, i1) of a unit (kP = 0) as a unit of its own.
 FwdUnit slice_unit(const FwdUnit &u, int i0, int i1) {
     const int nA = u.tiles_a();
     FwdUnit w = u;
@@ -307,19 +341,29 @@ struct Instance {
     int proto, h;
 };
 
-// Units (longest first) that cost more than `divisible` clocks may be cut between two tiles.  The others go to
+// Units (longest first) that cost more than `divisible` clocks (and have kP = 0) may be cut between two tiles.  The others go to
 // the CTA with the least work; the divisible ones then fill all CTAs up to a common level, one after
 // the other.  Returns the estimated time of the slowest CTA.
 int64_t balance(const ProtoList &list, const std::vector<Instance> &inst, int n_ctas, int64_t divisible, std::vector<Piece> &pieces) {
     const std::vector<Proto> &protos = list.protos;
     pieces.clear();
-    size_t n_div = 0;
+    const auto divide = [&](size_t k) {
+        const Proto &pr = protos[inst[k].proto];
+        return pr.cost > divisible && pr.u.kP() == 0;
+    };
+    std::vector<int> div;
     int64_t div_clk = 0;
-    for (; n_div < inst.size() && protos[inst[n_div].proto].cost > divisible; ++n_div) div_clk += protos[inst[n_div].proto].cost - kUnitClk;
+    for (size_t k = 0; k < inst.size() && protos[inst[k].proto].cost > divisible; ++k)
+        if (divide(k)) {
+            div.push_back((int)k);
+            div_clk += protos[inst[k].proto].cost - kUnitClk;
+        }
+    const size_t n_div = div.size();
     // heap of (load, CTA) in one word, least on top
     std::vector<int64_t> loads(n_ctas);
     for (int c = 0; c < n_ctas; ++c) loads[c] = c;
-    for (size_t k = n_div; k < inst.size(); ++k) {
+    for (size_t k = 0; k < inst.size(); ++k) {
+        if (divide(k)) continue;
         const Proto &pr = protos[inst[k].proto];
         const int64_t top = loads[0];
         pieces.push_back({(int)k, 0, pr.n_tiles, (int)(top & 0xffff)});
@@ -356,8 +400,8 @@ int64_t balance(const ProtoList &list, const std::vector<Instance> &inst, int n_
         int64_t load = heap[c].first, room = level - load + carry;
         const bool last = c + 1 == used;
         while (k < n_div) {
-            const int32_t *tile = list.tiles.data() + protos[inst[k].proto].tile0;
-            const int n_tiles = protos[inst[k].proto].n_tiles;
+            const int32_t *tile = list.tiles.data() + protos[inst[div[k]].proto].tile0;
+            const int n_tiles = protos[inst[div[k]].proto].n_tiles;
             int64_t left = room - extra;
             int i1 = i0;
             while (i1 < n_tiles && (last || left >= tile[i1] / 2)) left -= tile[i1++];
@@ -366,7 +410,7 @@ int64_t balance(const ProtoList &list, const std::vector<Instance> &inst, int n_
             load += room - left;
             room = left;
             i0 = i1;
-            pieces.push_back({(int)k, i1, i1, heap[c].second});
+            pieces.push_back({div[k], i1, i1, heap[c].second});
             if (i1 < n_tiles) break;
             ++k;
             i0 = 0;
@@ -377,7 +421,7 @@ int64_t balance(const ProtoList &list, const std::vector<Instance> &inst, int n_
     // pieces of divisible units carry their end only: fill in where each begins
     int prev_unit = -1, prev_end = 0;
     for (Piece &pc : pieces) {
-        if (protos[inst[pc.unit].proto].cost <= divisible) continue;
+        if (!divide(pc.unit)) continue;
         pc.i0 = pc.unit == prev_unit ? prev_end : 0;
         prev_unit = pc.unit;
         prev_end = pc.i1;
@@ -385,15 +429,15 @@ int64_t balance(const ProtoList &list, const std::vector<Instance> &inst, int n_
     return worst;
 }
 
-void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const ProtoList &singles, const HeadLists &heads) {
+void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const HeadLists &heads) {
     const int n_ctas = std::min(std::max(pl->n_ctas, 1), 0xffff);
-    ProtoList paired;
-    list_units(pl, ranges, true, paired);
+    ProtoList list;
+    list_units(pl, ranges, true, false, list);
     size_t n_inst = 0;
-    for (const Proto &pr : paired.protos) n_inst += heads.heads[pr.view].size();
+    for (const Proto &pr : list.protos) n_inst += heads.heads[pr.view].size();
     // Single halves when there are not enough pairs for half of the SMs: a CTA then works on one half only,
     // which takes less than the time of both.
-    const ProtoList &list = 2 * (int)n_inst > n_ctas ? paired : singles;
+    if (2 * (int)n_inst <= n_ctas) list_units(pl, ranges, false, false, list);
     const std::vector<Proto> &protos = list.protos;
     std::vector<Instance> inst;
     inst.reserve(n_inst);
@@ -489,9 +533,12 @@ int build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], cudaSt
         }
 
     const HeadLists heads(pl);
+    make_fwd_units(pl, ranges, heads);
+    size_t n_halves = 0;
+    for (int v = 0; v < 2; ++v)
+        for (int b = 0; b < pl->B; ++b) n_halves += heads.heads[v].size() * ceil_div(ranges[(size_t)v * pl->B + b].nv, kTile);
     ProtoList singles;
-    list_units(pl, ranges, false, singles);
-    make_fwd_units(pl, ranges, singles, heads);
+    list_units(pl, ranges, false, n_halves > (size_t)std::max(pl->n_ctas, 1), singles);
     make_bwd_units(pl, singles, heads);
 
     // device copy, in one piece: units, CTA offsets, padding, arrival counters (zeros; the kernel resets them)

@@ -53,9 +53,9 @@ constexpr int kPadWarps = 3;
 constexpr int kLoadWarp0 = kPadWarp0 + kPadWarps;
 constexpr int kLoadWarps = 4;
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
-// registers per thread after the roles have split: 256 x 200 + 256 x 56 = 65,536 = the 512 x 128 the CTA is
+// registers per thread after the roles have split: 256 x 168 + 256 x 88 = 65,536 = the 512 x 128 the CTA is
 // launched with
-constexpr int kRegsCompute = 200, kRegsOther = 56;
+constexpr int kRegsCompute = 168, kRegsOther = 88;
 constexpr int kStages = 4;  // ring of column tiles
 constexpr int kLag = 2;     // loader: copy groups in flight behind the newest one
 constexpr int kSchedDepth = 4;
@@ -181,12 +181,7 @@ __device__ __forceinline__ void math32(const uint32_t (&sv)[32], const uint32_t 
         }
     }
 }
-// Bits r_lo - cb .. r_hi - cb - 1 of a chunk of 32 columns.
-__device__ __forceinline__ uint32_t chunk_bits(int cb, int r_lo, int r_hi) {
-    const int a = min(max(r_lo - cb, 0), 32), b = min(max(r_hi - cb, 0), 32);
-    const uint32_t below_b = b >= 32 ? 0xffffffffu : (1u << b) - 1u, below_a = a >= 32 ? 0xffffffffu : (1u << a) - 1u;
-    return below_b & ~below_a;
-}
+__device__ __forceinline__ uint32_t bits_below(int n) { return n <= 0 ? 0u : n >= 32 ? 0xffffffffu : (1u << n) - 1u; }
 
 __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_constant__ Params p) {
     extern __shared__ uint8_t smem_raw[];
@@ -313,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
 #pragma unroll 1
                 for (int i = 0; i < n_tiles; ++i, ++c_cnt) {
                     const TileInfo t = tile_info(un, i, nA);
-                    const bool full = t.w == kTile && (!t.is_b || (w_lo_max <= t.k0 && w_hi_min >= t.k0 + kTile));
+                    const bool full = t.w == kTile && (t.pre == kTile || (w_lo_max - t.k0 <= t.pre && w_hi_min - t.k0 >= kTile));
                     const float4 *vec = reinterpret_cast<const float4 *>(sm + kOffVec + (c_cnt % kStages) * 1024);
                     TR_T0(t_ws);
                     if (!(alive = wait(bars + 8 * kBarSFull, ph_s))) break;
@@ -359,12 +354,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                             tmem_st16(tm + (kKeySide ? kTmA2 : kTmA1) + (cb >> 1), pk_ds);
                         }
                     } else {
-                        const int r_lo = t.is_b ? my_lo - t.k0 : 0, r_hi = t.is_b ? min(my_hi - t.k0, t.w) : t.w;
+                        // this row counts the columns [0, pre) and [r_lo, r_hi); some row of the warp counts columns only
+                        // there and within [e_lo, e_hi)
+                        const int r_lo = t.is_b ? my_lo - t.k0 : 0, r_hi = t.is_b ? min(my_hi - t.k0, t.w) : 0;
                         const int e_lo = __reduce_min_sync(0xffffffffu, r_lo), e_hi = __reduce_max_sync(0xffffffffu, r_hi);
+                        const int e_end = max(t.pre, e_hi > e_lo ? e_hi : 0);
                         bool held = true;
 #pragma unroll 1
                         for (int cb = cq * 32; cb < t.w; cb += 64) {
-                            if (cb + 32 <= e_lo || cb >= e_hi) {  // no row of the warp has a pair here
+                            if (cb >= t.pre && (cb + 32 <= e_lo || cb >= e_hi)) {  // no row of the warp has a pair here
 #pragma unroll
                                 for (int e = 0; e < 16; ++e) pk_p[e] = pk_ds[e] = 0u;
                             } else {
@@ -374,12 +372,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                                 tc_wait_ld();
                                 reg_fence(sv);
                                 reg_fence(tv);
-                                if (cb + 64 >= min(e_hi, t.w)) {  // read for the last time
+                                if (cb + 64 >= e_end) {  // read for the last time
                                     release_st();
                                     held = false;
                                 }
                                 math32<kKeySide, true>(sv, tv, scale2, row_nlse2, row_D2, vec + (cb >> 2), vec + 32 + (cb >> 2),
-                                                       chunk_bits(cb, r_lo, r_hi), pk_p, pk_ds);
+                                                       bits_below(t.pre - cb) | (bits_below(r_hi - cb) & ~bits_below(r_lo - cb)), pk_p, pk_ds);
                             }
                             wait_a();
                             if (kKeySide) tmem_st16(tm + kTmA1 + (cb >> 1), pk_p);
@@ -468,19 +466,23 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             int g_ks = 0;  // 16-column steps of the tile whose gradient MMAs are outstanding; one round more than tiles
 #pragma unroll 1
             for (int i = 0; i <= n_tiles; ++i) {
+                int ks = 0;
+                uint32_t idesc = 0, ca = 0;
+                if (i < n_tiles) {  // the tile has landed
+                    const int st = c_cnt % kStages;
+                    const TileInfo t = tile_info(un, i, nA);
+                    ks = (t.w + 15) >> 4;
+                    idesc = idesc_bf16(128, ks * 16, 0, 0);
+                    ca = smem_desc_lo(base + kOffC + st * 2 * kTileBytes);
+                    if (!(alive = wait(bars + 8 * (kBarCFull + st), (c_cnt / kStages) & 1))) break;
+                }
                 if (i > 0) {  // S and dP are free again once the previous tile's values are in registers
                     if (!(alive = wait(bars + 8 * kBarSTFree, ph_st))) break;
                     ph_st ^= 1;
                 }
-                int ks = 0;
+                tc_fence_after();
                 if (i < n_tiles) {
-                    const int st = c_cnt % kStages;
-                    if (!(alive = wait(bars + 8 * (kBarCFull + st), (c_cnt / kStages) & 1))) break;
-                    tc_fence_after();
-                    const TileInfo t = tile_info(un, i, nA);
-                    ks = (t.w + 15) >> 4;
-                    const uint32_t idesc = idesc_bf16(128, ks * 16, 0, 0);
-                    const uint32_t ca = smem_desc_lo(base + kOffC + st * 2 * kTileBytes), cb = ca + (kTileBytes >> 4);
+                    const uint32_t cb = ca + (kTileBytes >> 4);
                     if (leader) {
                         mma_ss_lean<0>(tmem + kTmS, ra, ca, idesc);  // S = Ra Ca^T, K = 64 as four steps of 16
                         mma_ss_lean<1>(tmem + kTmS, ra + 2, ca + 2, idesc);
@@ -632,10 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             const int ident = p.use_tma ? __ldg(vp.ident + un.b) : 0;
 
             // step -1: the row operands and row data; steps 0 ..: the column tiles
-            auto step_idx = [&](int i) {
-                const TileInfo t = tile_info(un, max(i, 0), nA);
-                return fetch_idx(perm, i < 0 ? un.q0 : t.k0, (i < 0 ? rows_h : t.w) - 1, lw, lane);
-            };
+            auto step_idx = [&](int i) { return fetch_idx(perm, i < 0 ? row_tile(un.q0, rows_h) : tile_info(un, i, nA), lw, lane); };
             int next = step_idx(-1);
 #pragma unroll 1
             for (int i = -1; i < n_tiles; ++i) {
@@ -647,12 +646,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                 const uint32_t bar_e = i < 0 ? kBarREmpty + rb : kBarCEmpty + st, bar_full = bars + 8 * (i < 0 ? kBarRFull + rb : kBarCFull + st);
                 if (!(alive = wait_free(bars + 8 * bar_e, ((i < 0 ? item_cnt >> 1 : c_cnt / kStages) & 1) ^ 1))) break;
                 const uint32_t dst = base + (i < 0 ? kOffR + rb * 2 * kTileBytes : kOffC + st * 2 * kTileBytes);
-                const bool bulk = i >= 0 && t.k0 + kTile <= ident;  // (rows behind the tile's own come along)
+                const bool bulk = i >= 0 && t.contiguous() && t.first() + kTile <= ident;  // (rows behind the tile's own come along)
                 if (bulk) {
                     if (lw == 0 && lane == 0) {
                         mbar_expect_tx(bar_full, 2 * kTileBytes);
-                        tma_load_2d(dst, key_side ? &p.tmQ : &p.tmK, 0, (int)bh + t.k0, bar_full);
-                        tma_load_2d(dst + kTileBytes, key_side ? &p.tmdO : &p.tmV, 0, (int)bh + t.k0, bar_full);
+                        tma_load_2d(dst, key_side ? &p.tmQ : &p.tmK, 0, (int)bh + t.first(), bar_full);
+                        tma_load_2d(dst + kTileBytes, key_side ? &p.tmdO : &p.tmV, 0, (int)bh + t.first(), bar_full);
                     }
                     __syncwarp();
                 } else {

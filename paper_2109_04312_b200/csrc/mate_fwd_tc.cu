@@ -66,9 +66,9 @@ constexpr int kLoadThreads = 32 * kLoadWarps;
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
 constexpr int kStages = 4;                   // K/V ring
 constexpr int kLag = 2;                      // loader: copy groups in flight behind the newest one
-// registers per thread after the roles have split: 256 x 200 + 256 x 56 = 65,536 = the 512 x 128 the CTA is
+// registers per thread after the roles have split: 256 x 176 + 256 x 80 = 65,536 = the 512 x 128 the CTA is
 // launched with
-constexpr int kRegsSoftmax = 200, kRegsOther = 56;
+constexpr int kRegsSoftmax = 176, kRegsOther = 80;
 constexpr uint32_t kApart = 1000;            // clocks between the exponentials of the two halves
 
 constexpr int kSchedDepth = 4;
@@ -129,12 +129,11 @@ struct Params {
 };
 
 // A chunk is 32 scores of one row (tile-local columns cb .. cb + 31).  A column c counts for the row
-// iff r_lo <= c < r_hi; the scores of the other columns are replaced by -inf, which the row max
+// iff c < pre or r_lo <= c < r_hi; the scores of the other columns are replaced by -inf, which the row max
 // ignores and the exponential turns into an exact 0 (the scale is positive).
-__device__ __forceinline__ void chunk_mask(uint32_t (&v)[32], int cb, int r_lo, int r_hi) {
-    const int a = min(max(r_lo - cb, 0), 32), b = min(max(r_hi - cb, 0), 32);
-    const uint32_t below_b = b >= 32 ? 0xffffffffu : (1u << b) - 1u, below_a = a >= 32 ? 0xffffffffu : (1u << a) - 1u;
-    const uint32_t on = below_b & ~below_a;
+__device__ __forceinline__ uint32_t bits_below(int n) { return n <= 0 ? 0u : n >= 32 ? 0xffffffffu : (1u << n) - 1u; }
+__device__ __forceinline__ void chunk_mask(uint32_t (&v)[32], int cb, int pre, int r_lo, int r_hi) {
+    const uint32_t on = bits_below(pre - cb) | (bits_below(r_hi - cb) & ~bits_below(r_lo - cb));
 #pragma unroll
     for (int e = 0; e < 32; ++e)
         if (!(on & (1u << e))) v[e] = 0xff800000u;
@@ -308,19 +307,22 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             }
             // this row's data: original position, key range (rows past the end shadow the last one)
             const int32_t *meta = reinterpret_cast<const int32_t *>(sm + kOffMeta) + qb * 3 * kUnitRows + h * kTile + min(r, rows_h - 1);
-            // The tiles this half visits: those of range A, then those of range B that meet the key ranges of its
-            // rows, [k_lo, k_hi)
-            const int nA = un.tiles_a(), tB = un.tB & 0xff;
+            // The tiles this half visits: those with positions that count for every row, then those that meet the
+            // key ranges of its rows
+            const int nA = un.tiles_a(), tB = un.tB & 0xff, kP = un.kP();
             const int k_lo = max(un.lo[h], un.kB0), k_hi = min(un.hi[h], un.kB_end);
-            const int b0 = k_hi > k_lo ? (k_lo - un.kB0) / tB : 0, b1 = k_hi > k_lo ? (k_hi - un.kB0 - 1) / tB + 1 : 0;
-            const int n_visit = nA + b1 - b0;
+            const int n_pre = nA + (kP + tB - 1) / tB;
+            const int b0 = max(n_pre, nA + (kP + k_lo - un.kB0) / tB);
+            const int n_visit = n_pre + (k_hi > k_lo ? max(nA + (kP + k_hi - un.kB0 - 1) / tB + 1 - b0, 0) : 0);
             const bool exact = (un.tB >> 8) != 0;
             const int w_lo_max = __reduce_max_sync(0xffffffffu, meta[kUnitRows]), w_hi_min = __reduce_min_sync(0xffffffffu, meta[2 * kUnitRows]);
-            // tiles that count in full for every row of the warp: the first fa of range A, [fb0, fb1) of range B (by
-            // number of visit)
-            const int fa = max(un.kA_end - un.kA0, 0) / kTile;
-            const int fb0 = nA - b0 + (tB == kTile ? (max(w_lo_max - un.kB0, 0) + kTile - 1) / kTile : n_visit);
-            const int fb1 = nA - b0 + max(min(w_hi_min, k_hi) - un.kB0, 0) / kTile;
+            // The visits whose tile counts in full for every row of the warp: [0, fa) and [fb0, fb1).  (In columns of
+            // range B, with the positions that count for every row in front, the rows' common range is [x_lo, x_hi).)
+            const int shift = kP - un.kB0, x_lo = w_lo_max + shift, x_hi = min(w_hi_min, k_hi) + shift;
+            const int fa = kP == 0 ? max(un.kA_end - un.kA0, 0) / kTile
+                                   : kP / kTile + (x_lo <= kP && x_hi >= (kP / kTile + 1) * kTile);
+            const int fb0 = tB == kTile ? n_pre + max((max(x_lo, 0) + kTile - 1) / kTile + nA - b0, 0) : n_visit;
+            const int fb1 = n_pre + max(x_hi, 0) / kTile + nA - b0;
 
             TR_ADD(5, t_setup);
             float m2 = -INFINITY;                // base of the row (log2 domain, scaled)
@@ -402,23 +404,28 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                         tmem_st16(tP + ch * 16, packed);
                     }
                 } else {
-                    // the tile's keys start at k0; the half's MMAs touch the columns [c_begin, c1), this row counts
-                    // [r_lo, r_hi), and some row of the warp counts columns only within [e_lo, e_hi)
-                    const bool is_b = j >= nA;
-                    const int k0 = is_b ? un.kB0 + (b0 + j - nA) * tB : un.kA0 + j * kTile;
-                    const int t_end = min((is_b ? k_hi : un.kA_end) - k0, is_b ? tB : kTile);
-                    const int r_lo = is_b ? meta[kUnitRows] - k0 : 0, r_hi = is_b ? min(meta[2 * kUnitRows] - k0, t_end) : t_end;
+                    // the half's MMAs touch the columns [c_begin, c1); this row counts [0, pre) and [r_lo, r_hi), and some row
+                    // of the warp counts columns only there and within [e_lo, e_hi)
+                    FwdUnit u = un;
+                    u.tB = tB;
+                    const TileInfo t = tile_info(u, j < n_pre ? j : b0 + j - n_pre, nA);
+                    int c_begin, c1;
+                    half_cols(un.lo[h], un.hi[h], t, c_begin, c1);
+                    c_begin &= ~31;
+                    const int r_lo = t.is_b ? meta[kUnitRows] - t.k0 : 0, r_hi = t.is_b ? min(meta[2 * kUnitRows] - t.k0, t.w) : 0;
                     const int e_lo = __reduce_min_sync(0xffffffffu, r_lo), e_hi = __reduce_max_sync(0xffffffffu, r_hi);
-                    const int c_begin = is_b ? max(k_lo - k0, 0) & ~31 : 0, c1 = (t_end + 15) & ~15;
+                    const int e_end = max(t.pre, e_hi > e_lo ? e_hi : 0);
+                    auto off = [&](int cb) { return cb >= t.pre && (cb + 32 <= e_lo || cb >= e_hi); };
                     uint32_t v[32];
                     if (j == 0 || exact) {
                         float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll 1
-                        for (int cb = max(c_begin, e_lo & ~31); cb < e_hi; cb += 32) {
+                        for (int cb = c_begin; cb < e_end; cb += 32) {
+                            if (off(cb)) continue;
                             tmem_ld32(tS + cb, v);
                             tc_wait_ld();
                             reg_fence(v);
-                            chunk_mask(v, cb, r_lo, r_hi);
+                            chunk_mask(v, cb, t.pre, r_lo, r_hi);
                             chunk_max(v, tm);
                         }
                         new_base(fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2);
@@ -430,19 +437,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
 #pragma unroll 1
                     for (int cb = c_begin; cb < c1; cb += 32) {
                         uint32_t packed[16];
-                        if (cb + 32 <= e_lo || cb >= e_hi) {  // no row of the warp has a key here
+                        if (off(cb)) {  // no row of the warp has a key here
 #pragma unroll
                             for (int e = 0; e < 16; ++e) packed[e] = 0u;
                         } else {
                             tmem_ld32(tS + cb, v);
                             tc_wait_ld();
                             reg_fence(v);
-                            if (cb + 32 >= e_hi) {  // read for the last time
+                            if (cb + 32 >= e_end) {  // read for the last time
                                 tc_fence_before();
                                 if (lane == 0) mbar_arrive(bar_sf);
                                 held = false;
                             }
-                            chunk_mask(v, cb, r_lo, r_hi);
+                            chunk_mask(v, cb, t.pre, r_lo, r_hi);
                             chunk_exp(v, scale2, neg_m2, packed, l01, l23);
                         }
                         tmem_st16(tP + (cb >> 1), packed);
@@ -474,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             if (exact) {
                 write = ((un.tB >> 16) >> warp) & 1;  // the others were right the first time
             } else if (n_visit > 0) {
-                const bool has_keys = nA > 0 || min(meta[2 * kUnitRows], k_hi) > max(meta[kUnitRows], k_lo);
+                const bool has_keys = n_pre > 0 || min(meta[2 * kUnitRows], k_hi) > max(meta[kUnitRows], k_lo);
                 if (__any_sync(0xffffffffu, !(l < kSumMax) || (l < kSumMin && has_keys))) {
                     write = false;
                     if (lane == 0) atomicOr((uint32_t *)s_bad + slot, 1u << warp);
@@ -630,16 +637,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 int c0 = 0, c1 = 0;
                 if (has_rows && i < n_tiles) half_cols(h ? un.lo[1] : un.lo[0], h ? un.hi[1] : un.hi[0], t, c0, c1);
                 const bool visit = c1 > c0;
+                if (visit) {  // the tile has landed
+                    TR_T0(t_kv);
+                    if (!(alive = wait(bars + 8 * (kBarKVFull + stage), (c / kStages) & 1))) break;
+                    TR_ADD(5, t_kv);
+                }
                 if (out) {  // S of the outstanding tile has been read
                     TR_T0(t_sf);
                     if (!(alive = wait(bar_sf, ph_sf))) break;
                     ph_sf ^= 1;
                     TR_ADD(6, t_sf);
-                }
-                if (visit) {  // the tile has landed
-                    TR_T0(t_kv);
-                    if (!(alive = wait(bars + 8 * (kBarKVFull + stage), (c / kStages) & 1))) break;
-                    TR_ADD(5, t_kv);
                 }
                 tc_fence_after();
                 if (visit) {
@@ -833,9 +840,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             const int qb = unit_cnt & 1;
             // steps -2, -1: the two Q halves (and the row data of the unit); steps 0 ..: the key tiles
             auto step_idx = [&](int i) {
-                const TileInfo t = tile_info(un, max(i, 0), nA);
-                const int row0 = i < 0 ? un.row0_of(i + 2) : t.k0, rows = i < 0 ? un.rows_of(i + 2) : t.w;
-                return rows > 0 ? fetch_idx(perm, row0, rows - 1, lw, lane) : 0;
+                const TileInfo t = i < 0 ? row_tile(un.row0_of(i + 2), un.rows_of(i + 2)) : tile_info(un, i, nA);
+                return t.w > 0 ? fetch_idx(perm, t, lw, lane) : 0;
             };
             int next = step_idx(-2);
 #pragma unroll 1
@@ -851,13 +857,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 const uint32_t dst = base + (i < 0 ? kOffQ + (qb * 2 + i + 2) * kTileBytes : kOffKV + stage * 2 * kTileBytes);
                 const uint32_t bar_full = bars + 8 * (i < 0 ? kBarQFull + qb : kBarKVFull + stage);
                 // (Q tiles are always gathered: fetching them with bulk copies as well measured slower.)
-                const bool bulk = i >= 0 && t.k0 + kTile <= ident;  // (rows behind the tile's own come along)
+                const bool bulk = i >= 0 && t.contiguous() && t.first() + kTile <= ident;  // (rows behind the tile's own come along)
                 TR_T0(t_cp);
                 if (bulk) {
                     if (ltid == 0) {
                         mbar_expect_tx(bar_full, 2 * kTileBytes);
-                        tma_load_2d(dst, &p.tmK, 0, (int)bh + t.k0, bar_full);
-                        tma_load_2d(dst + kTileBytes, &p.tmV, 0, (int)bh + t.k0, bar_full);
+                        tma_load_2d(dst, &p.tmK, 0, (int)bh + t.first(), bar_full);
+                        tma_load_2d(dst + kTileBytes, &p.tmV, 0, (int)bh + t.first(), bar_full);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar_full);

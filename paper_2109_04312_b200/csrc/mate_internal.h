@@ -20,55 +20,62 @@ constexpr int kTraceCtas = 256;  // CTAs whose cycle counters a -DMATE_TRACE bui
 // One unit of work of the tensor-core kernels: up to 256 consecutive rows (view order) of one (example, head)
 // in two halves of up to 128 -- half 0 = the first n0 rows, half 1 = the n1 rows behind them -- and the
 // column tiles they visit, in this order:
-//   range A = columns [kA0, kA_end) in tiles of 128: the global block for table rows ([0, P)), all valid
-//             positions for rows of the global block.  Column j counts for every row iff j < kA_end.
-//   range B = columns [kB0, kB_end) in tiles of tB <= 128: the union of the key ranges of the rows (table
-//             rows only).  Column j counts for a row iff seg_lo[row] <= j < seg_hi[row]; half h touches only
-//             the tiles that meet [lo[h], hi[h]) (min seg_lo / max seg_hi over its rows).
-// A unit of the forward may be split along its tiles into n_parts units; each writes an un-normalised
+//   range A = columns [kA0, kA_end) in tiles of 128, all of which count for every row: the global block
+//             ([0, P)) for table rows, all valid positions for rows of the global block.
+//   range B = the first kP positions of the order (which count for every row), then [kB0, kB_end) = the union of
+//             the key ranges of the rows, in tiles of tB <= 128.  Position j of the latter counts for a row
+//             iff seg_lo[row] <= j < seg_hi[row]; half h touches only the tiles that meet the first kP
+//             positions or [lo[h], hi[h]) (min seg_lo / max seg_hi over its rows).
+// The global block is in range A, or in front of range B (kP = P) where that takes fewer tiles.
+// A unit of the forward may be split along its tiles (kP = 0) into n_parts units; each writes an un-normalised
 // partial result to the workspace at ws_off (KiB); per group of 32 rows the part that finishes
 // last (counted in counters[8 * ctr + row / 32]) combines them.
 struct alignas(16) FwdUnit {  // (copied as four 16-byte words)
     int32_t b, h;
-    int32_t q0, rows;          // rows = n0 | n1 << 16; 0 ends a list
+    int32_t q0, rows;          // rows = n0 | n1 << 8 | kP << 16; 0 ends a list
     int32_t kA0, kA_end;
     int32_t kB0, kB_end;
     int32_t lo[2], hi[2];
     int32_t tB, parts;         // parts = n_parts | part << 16 (tB: the forward keeps flags above bit 7 on its way)
     int32_t ws_off, ctr;
 
-    __host__ __device__ int rows_of(int half) const { return half ? rows >> 16 : rows & 0xffff; }
-    __host__ __device__ int row0_of(int half) const { return half ? q0 + (rows & 0xffff) : q0; }
+    __host__ __device__ int rows_of(int half) const { return half ? (rows >> 8) & 0xff : rows & 0xff; }
+    __host__ __device__ int row0_of(int half) const { return half ? q0 + (rows & 0xff) : q0; }
+    __host__ __device__ int kP() const { return rows >> 16; }
     __host__ __device__ int n_parts() const { return parts & 0xffff; }
     __host__ __device__ int part() const { return parts >> 16; }
     __host__ __device__ int tiles_a() const { return kA_end > kA0 ? (kA_end - kA0 + kTile - 1) / kTile : 0; }
-    __host__ __device__ int tiles_b() const { return kB_end > kB0 ? (kB_end - kB0 + tB - 1) / tB : 0; }
+    __host__ __device__ int tiles_b() const { return kB_end > kB0 || kP() > 0 ? (kP() + kB_end - kB0 + tB - 1) / tB : 0; }
 };
 static_assert(sizeof(FwdUnit) == 64, "FwdUnit is read as four 16-byte words");
 
-// Tile i of a unit (nA = its tiles of range A): first column and number of columns (<= 128).
+// Tile i of a unit (nA = its tiles of range A): w columns (<= 128).  Column c stands for position x0 + c if c < pre
+// -- these count for every row -- and for position k0 + c otherwise.
 struct TileInfo {
-    int k0, w;
+    int x0, k0, w, pre;
     bool is_b;
+    __host__ __device__ int pos(int c) const { return c < pre ? x0 + c : k0 + c; }
+    // one run of positions, starting at first()
+    __host__ __device__ bool contiguous() const { return pre == 0 || pre == w || k0 == x0; }
+    __host__ __device__ int first() const { return pre > 0 ? x0 : k0; }
 };
 __host__ __device__ inline TileInfo tile_info(const FwdUnit &u, int i, int nA) {
     TileInfo t;
     t.is_b = i >= nA;
-    t.k0 = t.is_b ? u.kB0 + (i - nA) * u.tB : u.kA0 + i * kTile;
-    const int left = (t.is_b ? u.kB_end : u.kA_end) - t.k0, most = t.is_b ? u.tB : kTile;
+    t.x0 = t.is_b ? (i - nA) * u.tB : u.kA0 + i * kTile;
+    const int kP = u.kP(), left = (t.is_b ? kP + u.kB_end - u.kB0 : u.kA_end) - t.x0, most = t.is_b ? u.tB : kTile;
     t.w = left < most ? left : most;
+    t.k0 = t.is_b ? t.x0 + u.kB0 - kP : t.x0;
+    t.pre = !t.is_b ? t.w : kP <= t.x0 ? 0 : kP - t.x0 < t.w ? kP - t.x0 : t.w;
     return t;
 }
 // Columns [c0, c1) of the tile (multiples of 16) needed by a half whose rows' key ranges span [lo, hi);
 // c1 <= c0 when it skips the tile.
 __host__ __device__ inline void half_cols(int lo, int hi, const TileInfo &t, int &c0, int &c1) {
-    c0 = 0;
-    c1 = (t.w + 15) & ~15;
-    if (t.is_b) {
-        const int a = lo > t.k0 ? lo - t.k0 : 0, b = hi < t.k0 + t.w ? hi - t.k0 : t.w;
-        c0 = a & ~15;
-        c1 = a < b ? (b + 15) & ~15 : c0;
-    }
+    const int a = lo > t.k0 ? lo - t.k0 : 0, b = hi < t.k0 + t.w ? hi - t.k0 : t.w;
+    const bool meets = t.is_b && a < b;
+    c0 = t.pre > 0 ? 0 : a & ~15;
+    c1 = meets && b > t.pre ? (b + 15) & ~15 : t.pre > 0 ? (t.pre + 15) & ~15 : c0;
 }
 // bytes of one partial result: 256 rows x (64 fp32 + base, row sum, two unused)
 constexpr size_t kPartialBytes = (size_t)kUnitRows * (64 + 4) * sizeof(float);

@@ -15,13 +15,20 @@ constexpr int kTileBytes = kTile * kRowBytes;  // 16 KB: 128 rows
 bool make_row_map(CUtensorMap *map, const void *base, size_t rows);
 
 // The loaders copy a tile of up to 128 rows (128 B each), warp w of the four the rows 32 w .. 32 w + 31.
-// Row rr of the tile comes from view position row0 + min(rr, clamp).  A lane looks up the original
-// position of one row (coalesced, one latency for the whole tile, and cheap enough to be done a tile
-// ahead); the copies then run four rows at a time, eight lanes per row, with the positions handed
-// around by shuffle.
-__device__ __forceinline__ int fetch_idx(const int32_t *perm, int row0, int clamp, int lw, int lane) {
-    const int t = row0 + min(32 * lw + lane, clamp);
-    return perm ? __ldg(perm + t) : t;  // no order given: the tensors are in view order
+// A lane looks up the original position of one row (coalesced, one latency for the whole tile, and cheap
+// enough to be done a tile ahead); the copies then run four rows at a time, eight lanes per row, with the
+// positions handed around by shuffle.  Rows behind the last one repeat it.
+__device__ __forceinline__ int fetch_idx(const int32_t *perm, const TileInfo &t, int lw, int lane) {
+    const int at = t.pos(min(32 * lw + lane, t.w - 1));
+    return perm ? __ldg(perm + at) : at;  // no order given: the tensors are in view order
+}
+// n rows from view position q0 on, as a tile
+__device__ __forceinline__ TileInfo row_tile(int q0, int n) {
+    TileInfo t;
+    t.x0 = t.k0 = q0;
+    t.w = t.pre = n;
+    t.is_b = false;
+    return t;
 }
 // Rows [0, n_rows) of one tensor, or of two (`pair`; b_off: bytes from the first one's rows to the second's)
 // -> tiles at s_a and 16 KB behind it, 128-byte swizzle.

@@ -1021,9 +1021,7 @@ int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const v
         if (rc != MATE_OK) return rc;
     }
     void *outs[3] = {dQ, dK, dV};
-    for (int i = 0; i < 3; ++i)
-        if (mate::launch_add3(outs[i], g[0][i], g[1][i], n, dtype, st) != cudaSuccess) return MATE_ERR_CUDA;
-    return MATE_OK;
+    return mate::launch_add3(outs, g[0], g[1], n, dtype, st) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(256) rowdot_kernel(const __nv_bfloat16 *__rest
                                                      const float *__restrict__ LSE, float *__restrict__ D,
                                                      float *__restrict__ nlse, size_t rows, int32_t *counter) {
     launch_dependents();
+    wait_prior_grid();
     if (blockIdx.x == 0 && threadIdx.x < 64) counter[threadIdx.x] = 0;
     const int part = threadIdx.x & 7;
     const size_t r0 = (size_t)blockIdx.x * kRowdotRows + (threadIdx.x >> 3);
@@ -184,6 +185,7 @@ __device__ __forceinline__ void math32(const uint32_t (&sv)[32], const uint32_t 
 __device__ __forceinline__ uint32_t bits_below(int n) { return n <= 0 ? 0u : n >= 32 ? 0xffffffffu : (1u << n) - 1u; }
 
 __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_constant__ Params p) {
+    launch_dependents();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -536,6 +538,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
     } else if (warp < kLoadWarp0) {
         // ------------------------------------------------------------------ padding rows: zero gradients
         reg_dealloc<kRegsOther>();
+        wait_prior_grid();
 #pragma unroll 1
         for (int c = blockIdx.x; c < p.n_pads; c += gridDim.x) {
             const PadChunk pc = p.pads[c];
@@ -751,10 +754,9 @@ int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.status = plan->status_dev;
     p.counter = (int32_t *)ws + 8 * pass;
 
-    if (pass == 0)
-        rowdot_kernel<<<(unsigned)((rows + kRowdotRows - 1) / kRowdotRows), 256, 0, stream>>>(
-            (const __nv_bfloat16 *)dO, (const __nv_bfloat16 *)O, LSE, D, nlse, rows, (int32_t *)ws);
-    // started while the kernel before drains: its set-up and first records overlap with that
+    if (pass == 0 && launch_after(rowdot_kernel, dim3((unsigned)((rows + kRowdotRows - 1) / kRowdotRows)), 256, 0, stream, p.dO,
+                                  (const __nv_bfloat16 *)O, LSE, D, nlse, rows, (int32_t *)ws) != cudaSuccess)
+        return MATE_ERR_CUDA;
     return launch_after(tc_bwd_kernel, dim3((unsigned)plan->bwd_grid), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }
 

@@ -7,6 +7,7 @@
 // (One warp per row, 32 tokens at a time handed around by shuffles, took 7 us for rows of 30 tokens and 93 us
 // for rows of several hundred; this takes 2.3 and 6.3.)
 #include "mate_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace mate {
 namespace {
@@ -19,6 +20,8 @@ cell_mean_kernel(const float *__restrict__ logits, const int32_t *__restrict__ c
                  int n_rows, int n_cols, float *__restrict__ mean, int32_t *__restrict__ count) {
     __shared__ __align__(16) int32_t s_col[kBuf];
     __shared__ __align__(16) float s_x[kBuf];
+    ptx::launch_dependents();
+    ptx::wait_prior_grid();
     const int r = blockIdx.x, b = blockIdx.y;  // row id, example
     const int32_t *seg_off = rowv.seg_off + (size_t)b * (rowv.max_id + 2);
     const int lo = seg_off[r], hi = seg_off[r + 1];
@@ -68,7 +71,8 @@ extern "C" int mate_cell_mean(const mate_plan_t *plan, const float *logits, cons
     if (plan->T) return MATE_ERR_UNSUPPORTED;  // packed batches: not here
     if (mate::use_plan(plan, (cudaStream_t)stream) != cudaSuccess) return MATE_ERR_CUDA;
     const int n_rows = plan->view[0].max_id + 1, n_cols = plan->view[1].max_id + 1;
-    mate::cell_mean_kernel<<<dim3(n_rows, plan->B), mate::kThreads, 0, (cudaStream_t)stream>>>(
-        logits, col_ids, plan->view[0], plan->N, n_rows, n_cols, mean, count);
-    return cudaGetLastError() == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
+    return mate::launch_after(mate::cell_mean_kernel, dim3(n_rows, plan->B), mate::kThreads, 0, (cudaStream_t)stream, logits, col_ids,
+                              plan->view[0], plan->N, n_rows, n_cols, mean, count) == cudaSuccess
+               ? MATE_OK
+               : MATE_ERR_CUDA;
 }

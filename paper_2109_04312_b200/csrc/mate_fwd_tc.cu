@@ -173,6 +173,7 @@ __device__ __forceinline__ float sum_f32x2(uint64_t a, uint64_t b) {
 }
 
 __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_constant__ Params p) {
+    launch_dependents();
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -714,6 +715,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     } else if (warp < kLoadWarp0) {
         // ------------------------------------------------------------------ padding rows: O = 0, LSE = -inf
         reg_dealloc<kRegsOther>();
+        wait_prior_grid();
 #pragma unroll 1
         for (int c = blockIdx.x; c < p.n_pads; c += gridDim.x) {
             const PadChunk pc = p.pads[c];
@@ -732,6 +734,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     } else {
         // ------------------------------------------------------------------ loaders
         reg_dealloc<kRegsOther>();
+        wait_prior_grid();  // (the other roles touch global memory only behind data from here)
         const int ltid = tid - 32 * kLoadWarp0, lw = warp - kLoadWarp0;
         uint32_t kv_cnt = 0, unit_cnt = 0;
         uint32_t pend[kLag];
@@ -985,8 +988,8 @@ int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.status = plan->status_dev;
     p.counters = plan->fwd_counters_dev;
     p.ws = (uint8_t *)workspace;
-    tc_fwd_kernel<<<plan->fwd_grid, kThreads, kSmemBytes, stream>>>(p);
-    return cudaGetLastError() == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
+    return launch_after(tc_fwd_kernel, dim3((unsigned)plan->fwd_grid), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MATE_OK
+                                                                                                                      : MATE_ERR_CUDA;
 }
 
 }  // namespace mate

@@ -226,10 +226,12 @@ struct SmemAttrOnce {
     }
 };
 
-// Launches a kernel that may start before the one in front of it in the stream is complete; it waits for that
-// itself (griddepcontrol.wait) before it touches what that one writes.
-template <typename Params>
-cudaError_t launch_after(void (*kernel)(const Params), dim3 grid, int threads, size_t smem, cudaStream_t stream, const Params &p) {
+// Launches a kernel that may start while the one in front of it in the stream drains: all kernels that are launched so
+// let the next one start (griddepcontrol.launch_dependents) and wait for the one before (griddepcontrol.wait)
+// before they read or write anything that another kernel writes or reads.  Takes the launch gap (about 2 us)
+// and the set-up of the tensor-core kernels out of a layer's time.
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
@@ -240,7 +242,7 @@ cudaError_t launch_after(void (*kernel)(const Params), dim3 grid, int threads, s
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p);
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 // To be called before work that uses the plan is put on `st`.
@@ -260,7 +262,7 @@ cudaError_t launch_pair_ids(const int32_t *row_ids, const int32_t *col_ids, int 
 // row-or-column pattern (mate_sat.cu): merge of the passes' outputs, sum of their gradients
 cudaError_t launch_merge_passes(void *O, float *LSE, const void *O1, const float *LSE1, const void *O2, const float *LSE2,
                                 size_t rows, int d, int dtype, cudaStream_t stream);
-cudaError_t launch_add3(void *a, const void *b, const void *c, size_t n, int dtype, cudaStream_t stream);
+cudaError_t launch_add3(void *const (&a)[3], void *const (&b)[3], void *const (&c)[3], size_t n, int dtype, cudaStream_t stream);
 
 // SIMT kernels (mate_simt.cu)
 int simt_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, int d, int dtype,

@@ -224,11 +224,12 @@ __device__ __forceinline__ void pad_rows(const Common &c, const RowBlock &r, int
 
 // ---------------------------------------------------------------------------------- forward
 template <typename T, int DP>
-__global__ void __launch_bounds__(kThreads, DP <= 64 ? 3 : 1)
+__global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1)
 simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V, T *__restrict__ O,
                 float *__restrict__ LSE, const Common c, int H, int n_bh) {
     extern __shared__ __align__(16) float smem[];
     __shared__ int s_range[2];
+    ptx::wait_prior_grid();
     float *sQ = smem, *sK = sQ + kRows * (DP + 4), *sV = sK + kCols * (DP + 4), *sP = sV + kCols * (DP + 4);
     // row blocks vary slowest: the long ones (global block) come first
     const int bh = blockIdx.x % n_bh, b = bh / H, h = bh % H;
@@ -313,7 +314,7 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
 template <typename T>
 __global__ void __launch_bounds__(kThreads) simt_rowdot_kernel(const T *__restrict__ dO, const T *__restrict__ O,
                                                                float *__restrict__ D, size_t rows, int d) {
-    ptx::launch_dependents();
+    ptx::wait_prior_grid();
     const size_t r = (size_t)blockIdx.x * (kThreads / 16) + (threadIdx.x >> 4);
     const int tx = threadIdx.x & 15;
     float acc = 0.f;
@@ -346,6 +347,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
     const bool key_side = (blockIdx.x & 1) == 0;
     const int bh = (blockIdx.x >> 1) % a.n_bh, b = bh / a.H, h = bh % a.H;
     const RowBlock r = row_block(c, b, h, (blockIdx.x >> 1) / a.n_bh, s_range);
+    ptx::wait_prior_grid();
     pad_rows(c, r, b, key_side ? a.dK : a.dQ, key_side ? a.dV : (T *)nullptr, (float *)nullptr);
     if (r.n <= 0) return;
     const int tx = threadIdx.x & 15, row0 = (threadIdx.x >> 4) * 2;
@@ -372,7 +374,6 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
         x.store(sRa);
         y.store(sRb);
     }
-    ptx::wait_prior_grid();  // D comes from the kernel before
     if (r.n_tiles > 0) fetch(0);
     float lse[2], D[2], acc0[2][DP / 16], acc1[2][DP / 16];
 #pragma unroll
@@ -449,9 +450,10 @@ int fwd_launch(const mate_plan_t *pl, const void *Q, const void *K, const void *
     static SmemAttrOnce attr;
     constexpr int bytes = 4 * ((kRows + 2 * kCols) * (DP + 4) + kRows * kPStride);
     if (attr.ensure((const void *)simt_fwd_kernel<T, DP>, bytes, pl->device) != MATE_OK) return MATE_ERR_CUDA;
-    simt_fwd_kernel<T, DP><<<(unsigned)n_blocks(pl), kThreads, bytes, st>>>(
-        (const T *)Q, (const T *)K, (const T *)V, (T *)O, LSE, common(pl, d, scale, view_order), pl->H, pl->B * pl->H);
-    return cudaGetLastError() == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
+    return launch_after(simt_fwd_kernel<T, DP>, dim3((unsigned)n_blocks(pl)), kThreads, bytes, st, (const T *)Q, (const T *)K, (const T *)V,
+                        (T *)O, LSE, common(pl, d, scale, view_order), pl->H, pl->B * pl->H) == cudaSuccess
+               ? MATE_OK
+               : MATE_ERR_CUDA;
 }
 template <typename T, int DP>
 int bwd_launch(const mate_plan_t *pl, const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
@@ -460,9 +462,9 @@ int bwd_launch(const mate_plan_t *pl, const void *Q, const void *K, const void *
     constexpr int bytes = 4 * (2 * (kRows + kCols) * (DP + 4) + 2 * kRows * kPStride + 2 * kCols);
     if (attr.ensure((const void *)simt_bwd_kernel<T, DP>, bytes, pl->device) != MATE_OK) return MATE_ERR_CUDA;
     const size_t rows = pl->n_rows();
-    if (pass == 0)
-        simt_rowdot_kernel<T><<<(unsigned)((rows + kThreads / 16 - 1) / (kThreads / 16)), kThreads, 0, st>>>((const T *)dO, (const T *)O,
-                                                                                                          D, rows, d);
+    if (pass == 0 && launch_after(simt_rowdot_kernel<T>, dim3((unsigned)((rows + kThreads / 16 - 1) / (kThreads / 16))), kThreads, 0, st,
+                                  (const T *)dO, (const T *)O, D, rows, d) != cudaSuccess)
+        return MATE_ERR_CUDA;
     const BwdArgs<T> a{(const T *)Q, (const T *)K, (const T *)V, (const T *)dO, LSE, D, (T *)dQ, (T *)dK, (T *)dV,
                        common(pl, d, scale, 0), pl->H, pl->B * pl->H};
     return launch_after(simt_bwd_kernel<T, DP>, dim3((unsigned)(2 * n_blocks(pl))), kThreads, bytes, st, a) == cudaSuccess

@@ -331,106 +331,10 @@ FwdUnit slice_unit(const FwdUnit &u, int i0, int i1) {
     return w;
 }
 
-// ---- forward schedule: which CTA does which units, decided here once
-struct Piece {
-    int unit;     // index into the instances
-    int i0, i1;   // its tiles
-    int cta;
-};
-struct Instance {
-    int proto, h;
-};
-
-// Units (longest first) that cost more than `divisible` clocks (and have kP = 0) may be cut between two tiles.  The others go to
-// the CTA with the least work; the divisible ones then fill all CTAs up to a common level, one after
-// the other.  Returns the estimated time of the slowest CTA.
-int64_t balance(const ProtoList &list, const std::vector<Instance> &inst, int n_ctas, int64_t divisible, std::vector<Piece> &pieces) {
-    const std::vector<Proto> &protos = list.protos;
-    pieces.clear();
-    const auto divide = [&](size_t k) {
-        const Proto &pr = protos[inst[k].proto];
-        return pr.cost > divisible && pr.u.kP() == 0;
-    };
-    std::vector<int> div;
-    int64_t div_clk = 0;
-    for (size_t k = 0; k < inst.size() && protos[inst[k].proto].cost > divisible; ++k)
-        if (divide(k)) {
-            div.push_back((int)k);
-            div_clk += protos[inst[k].proto].cost - kUnitClk;
-        }
-    const size_t n_div = div.size();
-    // heap of (load, CTA) in one word, least on top
-    std::vector<int64_t> loads(n_ctas);
-    for (int c = 0; c < n_ctas; ++c) loads[c] = c;
-    for (size_t k = 0; k < inst.size(); ++k) {
-        if (divide(k)) continue;
-        const Proto &pr = protos[inst[k].proto];
-        const int64_t top = loads[0];
-        pieces.push_back({(int)k, 0, pr.n_tiles, (int)(top & 0xffff)});
-        const int64_t key = top + (pr.cost << 16);
-        size_t i = 0;  // sift down
-        for (size_t c = 1; c < loads.size(); c = 2 * i + 1) {
-            if (c + 1 < loads.size() && loads[c + 1] < loads[c]) ++c;
-            if (loads[c] >= key) break;
-            loads[i] = loads[c];
-            i = c;
-        }
-        loads[i] = key;
-    }
-    std::sort(loads.begin(), loads.end());
-    std::vector<std::pair<int64_t, int>> heap(n_ctas);
-    for (int c = 0; c < n_ctas; ++c) heap[c] = {loads[c] >> 16, (int)(loads[c] & 0xffff)};
-    int64_t worst = heap.back().first;
-    if (n_div == 0) return worst;
-    // Level: the `used` least loaded CTAs take the divisible tiles, each with the cost of one more (partial)
-    // unit.  What rounding to tiles leaves over or takes too much is carried to the next CTA; every
-    // divisible unit begun inside a CTA costs one more partial unit.
-    const int64_t extra = kUnitClk + kPartClk;
-    int used = 0;
-    int64_t level = 0, sum = div_clk + (int64_t)n_div * extra;
-    for (used = 1; used <= n_ctas; ++used) {
-        sum += heap[used - 1].first + extra;
-        level = (sum + used - 1) / used;
-        if (used == n_ctas || level <= heap[used].first + extra + 2 * kFullClk) break;
-    }
-    size_t k = 0;
-    int i0 = 0;
-    int64_t carry = 0;
-    for (int c = 0; c < used && k < n_div; ++c) {
-        int64_t load = heap[c].first, room = level - load + carry;
-        const bool last = c + 1 == used;
-        while (k < n_div) {
-            const int32_t *tile = list.tiles.data() + protos[inst[div[k]].proto].tile0;
-            const int n_tiles = protos[inst[div[k]].proto].n_tiles;
-            int64_t left = room - extra;
-            int i1 = i0;
-            while (i1 < n_tiles && (last || left >= tile[i1] / 2)) left -= tile[i1++];
-            if (!last && i1 > i0 + 1 && i1 + 1 == n_tiles) left += tile[--i1];  // leave no crumb
-            if (i1 == i0) break;
-            load += room - left;
-            room = left;
-            i0 = i1;
-            pieces.push_back({div[k], i1, i1, heap[c].second});
-            if (i1 < n_tiles) break;
-            ++k;
-            i0 = 0;
-        }
-        carry = room;
-        worst = std::max(worst, load);
-    }
-    // pieces of divisible units carry their end only: fill in where each begins
-    int prev_unit = -1, prev_end = 0;
-    for (Piece &pc : pieces) {
-        if (!divide(pc.unit)) continue;
-        pc.i0 = pc.unit == prev_unit ? prev_end : 0;
-        prev_unit = pc.unit;
-        prev_end = pc.i1;
-    }
-    return worst;
-}
-
+// Forward.  A unit of more than 1.3 of a CTA's share of the clocks is cut between tiles into parts of about
+// 0.75 of it (never less than four tiles), to be combined in the kernel; longest first, as for the backward.
 void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const HeadLists &heads) {
-    const int n_ctas = std::min(std::max(pl->n_ctas, 1), 0xffff);
+    const int n_ctas = std::max(pl->n_ctas, 1);
     ProtoList list;
     list_units(pl, ranges, true, false, list);
     size_t n_inst = 0;
@@ -438,60 +342,59 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
     // Single halves when there are not enough pairs for half of the SMs: a CTA then works on one half only,
     // which takes less than the time of both.
     if (2 * (int)n_inst <= n_ctas) list_units(pl, ranges, false, false, list);
-    const std::vector<Proto> &protos = list.protos;
-    std::vector<Instance> inst;
-    inst.reserve(n_inst);
     int64_t total = 0;
-    for (size_t k = 0; k < protos.size(); ++k) {
-        for (int h : heads.heads[protos[k].view]) inst.push_back({(int)k, h});
-        total += protos[k].cost * (int64_t)heads.heads[protos[k].view].size();
-    }
-    // How much is cut is decided by the estimate: nothing, units longer than a CTA's share, half of it, a quarter.
-    const int64_t share = total / n_ctas;
-    std::vector<Piece> best, pieces;
-    best.reserve(inst.size());
-    int64_t best_clk = balance(list, inst, n_ctas, INT64_MAX, best);
-    for (const int64_t divisible : {share, share / 2, share / 4}) {
-        if (divisible < kUnitClk + 4 * kFullClk || 100 * best_clk <= 106 * share) break;
-        const int64_t clk = balance(list, inst, n_ctas, divisible, pieces);
-        if (clk < best_clk) {
-            best_clk = clk;
-            best.swap(pieces);
-        }
-    }
+    for (const Proto &pr : list.protos) total += pr.cost * (int64_t)heads.heads[pr.view].size();
+    const int64_t share = std::max<int64_t>(total / n_ctas, 1);
 
-    // records, split units with their place in the workspace; a CTA starts with its parts of split units, so
-    // that nobody waits for them in the end
-    std::vector<int> n_parts(inst.size(), 0), seen(inst.size(), 0), slot(inst.size(), -1);
-    std::vector<size_t> ws_off(inst.size(), 0);
-    for (const Piece &pc : best) ++n_parts[pc.unit];
+    struct Entry {
+        FwdUnit u;
+        int view;
+        int64_t cost;
+    };
+    std::vector<Entry> entries;
+    entries.reserve(list.protos.size());
     size_t ws_bytes = 0;
     pl->n_fwd_slots = 0;
-    for (size_t k = 0; k < inst.size(); ++k)
-        if (n_parts[k] > 1) {
-            slot[k] = pl->n_fwd_slots++;
-            ws_off[k] = ws_bytes;
-            ws_bytes += n_parts[k] * mate::kPartialBytes;
-        }
-    pl->fwd_cta_off.assign(n_ctas + 1, 0);
-    for (const Piece &pc : best) ++pl->fwd_cta_off[pc.cta + 1];
-    for (int c = 0; c < n_ctas; ++c) pl->fwd_cta_off[c + 1] += pl->fwd_cta_off[c];
-    pl->fwd_units.resize(best.size());
-    std::vector<int32_t> at(pl->fwd_cta_off.begin(), pl->fwd_cta_off.end() - 1);
-    for (int pass = pl->n_fwd_slots > 0 ? 0 : 1; pass < 2; ++pass)
-        for (const Piece &pc : best) {
-            if ((n_parts[pc.unit] > 1) != (pass == 0)) continue;
-            const Proto &pr = protos[inst[pc.unit].proto];
-            FwdUnit &u = pl->fwd_units[at[pc.cta]++];
-            u = pr.u;
-            if (n_parts[pc.unit] > 1) {
-                u = slice_unit(pr.u, pc.i0, pc.i1);
-                u.parts = n_parts[pc.unit] | seen[pc.unit]++ << 16;
-                u.ctr = slot[pc.unit];
-                u.ws_off = (int32_t)((ws_off[pc.unit] + u.part() * mate::kPartialBytes) >> 10);
+    size_t n_units = 0;
+    for (const Proto &pr : list.protos) {
+        const size_t n_heads = heads.heads[pr.view].size();
+        int parts = 1;
+        if (pr.u.kP() == 0 && 10 * pr.cost > 13 * share)
+            parts = (int)std::max<int64_t>(1, std::min<int64_t>(pr.n_tiles / 4, (4 * pr.cost + 3 * share - 1) / (3 * share)));
+        if (parts == 1) {
+            entries.push_back({pr.u, pr.view, pr.cost});
+        } else {
+            const int32_t *tile = list.tiles.data() + pr.tile0;
+            for (int part = 0; part < parts; ++part) {
+                const int i0 = (int)((int64_t)pr.n_tiles * part / parts), i1 = (int)((int64_t)pr.n_tiles * (part + 1) / parts);
+                Entry e{slice_unit(pr.u, i0, i1), pr.view, kUnitClk + kPartClk};
+                for (int i = i0; i < i1; ++i) e.cost += tile[i];
+                e.u.parts = parts | part << 16;
+                e.u.ctr = pl->n_fwd_slots;  // of the first head; the others follow
+                e.u.ws_off = (int32_t)((ws_bytes + part * mate::kPartialBytes) >> 10);
+                entries.push_back(e);
             }
-            u.h = inst[pc.unit].h;
+            pl->n_fwd_slots += (int)n_heads;
+            ws_bytes += n_heads * parts * mate::kPartialBytes;
         }
+        n_units += n_heads * parts;
+    }
+    std::stable_sort(entries.begin(), entries.end(), [](const Entry &a, const Entry &b) { return a.cost > b.cost; });
+    pl->fwd_units.clear();
+    pl->fwd_units.reserve(n_units);
+    for (const Entry &e : entries) {
+        int k = 0;
+        for (int h : heads.heads[e.view]) {
+            pl->fwd_units.push_back(e.u);
+            FwdUnit &u = pl->fwd_units.back();
+            u.h = h;
+            if (u.n_parts() > 1) {
+                u.ctr += k;
+                u.ws_off += (int32_t)((k * u.n_parts() * mate::kPartialBytes) >> 10);
+            }
+            ++k;
+        }
+    }
     pl->n_fwd_units = (int)pl->fwd_units.size();
     pl->fwd_ws_bytes = ws_bytes;
     // padding rows of every (example, head)
@@ -500,20 +403,12 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
         for (int t0 = pl->n_valid[b]; t0 < pl->N; t0 += mate::kPadRows)
             for (int h = 0; h < pl->H; ++h) pl->pads.push_back({b, h, t0, std::min(mate::kPadRows, pl->N - t0)});
     pl->n_pads = (int)pl->pads.size();
-    // CTAs without units are not launched (the list is filled from CTA 0 on only when there are fewer units
-    // than CTAs), unless there is padding to be spread
-    int grid = n_ctas;
-    if (pl->n_fwd_units < n_ctas) {
-        grid = std::min(n_ctas, std::max(pl->n_fwd_units, pl->n_pads));
-        for (int c = grid; c < n_ctas; ++c)
-            if (pl->fwd_cta_off[c + 1] > pl->fwd_cta_off[c]) grid = c + 1;
-    }
-    pl->fwd_grid = grid;
+    pl->fwd_grid = std::min(n_ctas, std::max(pl->n_fwd_units, pl->n_pads));
     if (getenv("MATE_LOG"))
-        fprintf(stderr, "[mate] forward: %d units (%d of %d split), %d CTAs, estimated clocks: mean %lld, slowest %lld; "
-                        "workspace %zu bytes; %d chunks of padding\n",
-                pl->n_fwd_units, pl->n_fwd_slots, (int)inst.size(), pl->fwd_grid, (long long)share, (long long)best_clk,
-                pl->fwd_ws_bytes, pl->n_pads);
+        fprintf(stderr, "[mate] forward: %d units (%d split), %d CTAs, estimated clocks per CTA %lld, largest unit %lld; workspace %zu "
+                        "bytes; %d chunks of padding\n",
+                pl->n_fwd_units, pl->n_fwd_slots, pl->fwd_grid, (long long)share,
+                entries.empty() ? 0ll : (long long)entries.front().cost, pl->fwd_ws_bytes, pl->n_pads);
 }
 
 int build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], cudaStream_t st) {
@@ -541,14 +436,13 @@ int build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], cudaSt
     list_units(pl, ranges, false, n_halves > (size_t)std::max(pl->n_ctas, 1), singles);
     make_bwd_units(pl, singles, heads);
 
-    // device copy, in one piece: units, CTA offsets, padding, arrival counters (zeros; the kernel resets them)
+    // device copy, in one piece: units, padding, arrival counters (zeros; the kernel resets them)
     const auto lay_out = [pl](char *base) {
         Carver c(base);
         pl->fwd_units_dev = c.take<FwdUnit>(pl->n_fwd_units);
         pl->bwd_units_dev = c.take<FwdUnit>(pl->n_bwd_units);
-        pl->fwd_cta_off_dev = c.take<int32_t>(pl->fwd_cta_off.size());
         pl->pads_dev = c.take<mate::PadChunk>(pl->n_pads);
-        pl->fwd_counters_dev = c.take<int32_t>(8 * (size_t)pl->n_fwd_slots);
+        pl->fwd_counters_dev = c.take<int32_t>(mate::kSchedWords + 8 * (size_t)pl->n_fwd_slots);
         return align_up(c.off, 256);
     };
     const size_t bytes = lay_out(nullptr);
@@ -561,9 +455,8 @@ int build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], cudaSt
     lay_out((char *)host.ptr);
     std::copy(pl->fwd_units.begin(), pl->fwd_units.end(), pl->fwd_units_dev);
     std::copy(pl->bwd_units.begin(), pl->bwd_units.end(), pl->bwd_units_dev);
-    std::copy(pl->fwd_cta_off.begin(), pl->fwd_cta_off.end(), pl->fwd_cta_off_dev);
     std::copy(pl->pads.begin(), pl->pads.end(), pl->pads_dev);
-    std::fill_n(pl->fwd_counters_dev, 8 * (size_t)pl->n_fwd_slots, 0);
+    std::fill_n(pl->fwd_counters_dev, mate::kSchedWords + 8 * (size_t)pl->n_fwd_slots, 0);
     lay_out((char *)pl->work_block.ptr);
     bool ok = cudaMemcpyAsync(pl->work_block.ptr, host.ptr, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
     mate::staging_give(host, st);
@@ -865,7 +758,7 @@ int mate_plan_status(const mate_plan_t *plan, void *stream) {
             fprintf(stderr, "[mate] a bounded wait expired: barrier slot %d, parity %d, warp %d\n", (s[2] >> 8) & 0xff,
                     (s[2] >> 7) & 1, s[2] & 0x7f);
         // a kernel that gave up may have left the arrival counters half way
-        if (cudaMemsetAsync(plan->fwd_counters_dev, 0, sizeof(int32_t) * 8 * (size_t)plan->n_fwd_slots, st) != cudaSuccess ||
+        if (cudaMemsetAsync(plan->fwd_counters_dev, 0, sizeof(int32_t) * (mate::kSchedWords + 8 * (size_t)plan->n_fwd_slots), st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
             return MATE_ERR_CUDA;
         return MATE_ERR_TIMEOUT;

@@ -200,21 +200,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
     // The first loader warp hands out the items; its lanes 0-3 hold the record of the next one.  The first item
     // of a CTA is its own index, later ones come from the shared counter.
     int4 rec = make_int4(0, 0, 0, 0);
-    bool list_done = false;
-    auto claim = [&](bool first_item) {
-        int it = blockIdx.x;
-        if (!first_item) {
-            if (lane == 0) it = atomicAdd(p.counter, 1) + (int)gridDim.x;
-            it = __shfl_sync(0xffffffffu, it, 0);
-        }
-        rec = make_int4(0, 0, 0, 0);
-        list_done = it >= 2 * p.n_units;
-        if (!list_done && lane < 4) {
+    int it_next = blockIdx.x;  // lane 0
+    auto claim = [&]() {
+        if (lane == 0) it_next = atomicAdd(p.counter, 1) + (int)gridDim.x;
+    };
+    auto fetch_record = [&]() {
+        const int it = __shfl_sync(0xffffffffu, it_next, 0);
+        rec = make_int4(0, 0, 0, 0);  // rows = 0: the list is exhausted
+        if (it < 2 * p.n_units && lane < 4) {
             rec = __ldg(reinterpret_cast<const int4 *>(p.units + (it >> 1)) + lane);
             if (lane == 3) rec.z = it & 1;
         }
     };
-    if (warp == kLoadWarp0) claim(true);
+    if (warp == kLoadWarp0) fetch_record();
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -643,7 +641,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             for (int i = -1; i < n_tiles; ++i) {
                 const int now = next;
                 if (i + 1 < n_tiles) next = step_idx(i + 1);
-                else if (warp == kLoadWarp0 && !list_done) claim(false);
+                else if (warp == kLoadWarp0) claim();  // the number and then the record travel under the copies
                 const TileInfo t = tile_info(un, max(i, 0), nA);
                 const int st = c_cnt % kStages, rb = item_cnt & 1;
                 const uint32_t bar_e = i < 0 ? kBarREmpty + rb : kBarCEmpty + st, bar_full = bars + 8 * (i < 0 ? kBarRFull + rb : kBarCFull + st);
@@ -681,6 +679,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                 }
                 if (!bulk || key_side) commit_and_signal(bar_full);
                 else if (lane == 0) mbar_arrive(bar_full);
+                if (i + 1 == n_tiles && warp == kLoadWarp0) fetch_record();
                 if (i < 0) {
                     ++item_cnt;
                 } else {

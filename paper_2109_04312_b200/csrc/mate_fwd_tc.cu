@@ -1,6 +1,6 @@
 // Tensor-core forward of multi-view attention (head formula and pattern of Section 3) for bf16,
-// d = 64, on sm_100a.  One persistent, warp-specialised CTA per SM walks its list of units, which
-// mate_plan balanced over the CTAs (see FwdUnit): 256 query rows of one (example, head) in the head's view
+// d = 64, on sm_100a.  One persistent, warp-specialised CTA per SM takes units (see FwdUnit), longest first, from
+// a shared counter: 256 query rows of one (example, head) in the head's view
 // order (Section 3.1: per-head traversal order) against the key tiles those rows may attend.
 //
 //   warps 0-3   softmax of half 0 (query rows 0..127 of the unit), one thread per row
@@ -116,15 +116,15 @@ struct Params {
     float *LSE;
     ViewPlan rowv, colv;
     const uint8_t *head_view;
-    const FwdUnit *units;      // by CTA; those of CTA c are [cta_off[c], cta_off[c + 1])
-    const int32_t *cta_off;
+    const FwdUnit *units;      // longest first
+    int n_units;
     const PadChunk *pads;      // padding rows, which no unit covers
     int n_pads;
     int N, H;
     TensorRows tr;     // where (example, head) starts in the tensors
     float scale_log2;  // scale * log2(e)
     int32_t *status;
-    int32_t *counters;  // arrivals at the split units, 8 per unit
+    int32_t *counters;  // [0] next unit, from kSchedWords on arrivals at the split units, 8 per unit
     uint8_t *ws;
 };
 
@@ -187,20 +187,25 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = tid & 31;
 
-    // The first loader warp publishes the records of the CTA's units; its lanes 0-3 hold the next one ahead
-    // of its turn.
-    int u_next = 0, u_end = 0;
+    // The first loader warp hands out the units; its lanes 0-3 hold the record of the next one.  The first unit of
+    // a CTA is its own index, later ones come from the shared counter, each claimed when the loaders
+    // reach the last tile of the unit before it; the number and then the record travel under the copies.  Every CTA's last claim fails, so the claims of a
+    // launch number n_units: the one that draws the last number puts the counter back to zero for the next launch.
     int4 rec = make_int4(0, 0, 0, 0);
-    auto fetch_record = [&]() {
-        rec = make_int4(0, 0, 0, 0);  // rows = 0: the list is exhausted
-        if (u_next < u_end && lane < 4) rec = __ldg(reinterpret_cast<const int4 *>(p.units + u_next) + lane);
-        ++u_next;
+    int u_next = blockIdx.x;  // lane 0
+    auto claim = [&]() {
+        if (lane == 0) u_next = atomicAdd(p.counters, 1);
     };
-    if (warp == kLoadWarp0) {  // requested before the set-up below, which takes as long
-        u_next = __ldg(p.cta_off + blockIdx.x);
-        u_end = __ldg(p.cta_off + blockIdx.x + 1);
-        fetch_record();
-    }
+    auto fetch_record = [&](bool claimed) {
+        if (claimed && lane == 0) {
+            if (u_next == p.n_units - 1) *p.counters = 0;
+            u_next += (int)gridDim.x;
+        }
+        const int u = __shfl_sync(0xffffffffu, u_next, 0);
+        rec = make_int4(0, 0, 0, 0);  // rows = 0: the list is exhausted
+        if (u < p.n_units && lane < 4) rec = __ldg(reinterpret_cast<const int4 *>(p.units + u) + lane);
+    };
+    if (warp == kLoadWarp0) fetch_record(false);  // requested before the set-up below, which takes as long
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -517,7 +522,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 __syncwarp();
                 int last = 0;
                 if (lane == 0) {
-                    int32_t *ctr = p.counters + 8 * un.ctr + warp;
+                    int32_t *ctr = p.counters + kSchedWords + 8 * un.ctr + warp;
                     last = atomicAdd(ctr, 1) == n_parts - 1;
                     if (last) *ctr = 0;  // ready for the next launch
                 }
@@ -792,6 +797,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         FwdUnit un;
         uint32_t checked = 0;  // entries of the list that are known to be done
         int4 held_back = make_int4(0, 0, 0, 0);
+        bool redo = false;     // the entry being loaded is one that is done once more
         auto rec_rows = [&]() { return __shfl_sync(0xffffffffu, rec.w, 0); };  // FwdUnit::rows
 
         for (uint32_t n = 0; alive; ++n) {
@@ -819,8 +825,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 if (lane < 4) reinterpret_cast<int4 *>(s_unit + slot)[lane] = rec;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedFull + slot));  // release: the record is visible to the readers
-                if (again) rec = held_back;
-                else fetch_record();
+                redo = again;
             } else if (!wait_free(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) {
                 break;
             }
@@ -851,6 +856,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             for (int i = -2; i < n_tiles; ++i) {
                 const int now = next;
                 if (i + 1 < n_tiles) next = step_idx(i + 1);
+                else if (warp == kLoadWarp0 && !redo) claim();
                 const TileInfo t = tile_info(un, max(i, 0), nA);
                 const int stage = kv_cnt % kStages;
                 if (i != -1) {
@@ -889,6 +895,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                     continue;
                 }
                 if (!bulk) commit_and_signal(bar_full);
+                if (i + 1 == n_tiles && warp == kLoadWarp0) {
+                    if (redo) rec = held_back;
+                    else fetch_record(true);
+                }
                 if (i < 0) {
                     ++unit_cnt;
                     continue;
@@ -978,7 +988,7 @@ int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.colv = plan->view[1];
     p.head_view = plan->head_view_dev;
     p.units = plan->fwd_units_dev;
-    p.cta_off = plan->fwd_cta_off_dev;
+    p.n_units = plan->n_fwd_units;
     p.pads = plan->pads_dev;
     p.n_pads = plan->n_pads;
     p.N = plan->N;

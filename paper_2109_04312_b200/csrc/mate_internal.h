@@ -12,6 +12,7 @@
 namespace mate {
 
 constexpr int kTile = 128;       // key columns per tile and query rows per half of a unit
+constexpr int kSchedWords = 8;   // scheduling counters of the forward, in front of the split-unit counters
 constexpr int kUnitRows = 256;   // query rows per unit of the tensor-core kernels (two halves)
 // what the key range of a table row is made of (plan kernel step 4 and its host twin)
 enum { kBoundsOwn = 0, kBoundsBefore = 1, kBoundsAfter = 2 };
@@ -29,7 +30,7 @@ constexpr int kTraceCtas = 256;  // CTAs whose cycle counters a -DMATE_TRACE bui
 // The global block is in range A, or in front of range B (kP = P) where that takes fewer tiles.
 // A unit of the forward may be split along its tiles (kP = 0) into n_parts units; each writes an un-normalised
 // partial result to the workspace at ws_off (KiB); per group of 32 rows the part that finishes
-// last (counted in counters[8 * ctr + row / 32]) combines them.
+// last (counted in counters[kSchedWords + 8 * ctr + row / 32]) combines them.
 struct alignas(16) FwdUnit {  // (copied as four 16-byte words)
     int32_t b, h;
     int32_t q0, rows;          // rows = n0 | n1 << 8 | kP << 16; 0 ends a list
@@ -183,12 +184,12 @@ struct mate_plan_s {
     mutable std::atomic<bool> elsewhere{false};
     mutable std::mutex ready_mu;
     mutable cudaEvent_t ready = nullptr;  // recorded behind the copy; null once it has been waited for
-    // tensor-core forward work-list: the units of CTA c are [fwd_cta_off[c], fwd_cta_off[c + 1])
+    // tensor-core forward work-list, longest first; the CTAs of the persistent kernel take units through a counter
     mate::FwdUnit *fwd_units_dev = nullptr;
-    int32_t *fwd_cta_off_dev = nullptr;
     mate::PadChunk *pads_dev = nullptr;
-    // [8 * n_fwd_slots]: arrival counters of the split units.  Zero between launches (the kernel resets
-    // what it counted), which is why two forward calls on one plan must not overlap on the GPU.
+    // [kSchedWords + 8 * n_fwd_slots]: [0] next unit, then the arrival counters of the split units.
+    // Zero between launches (the kernel resets what it counted), which is why two forward calls on one
+    // plan must not overlap on the GPU.
     int32_t *fwd_counters_dev = nullptr;
     int n_fwd_units = 0;
     int n_pads = 0;
@@ -197,7 +198,6 @@ struct mate_plan_s {
     int n_ctas = 0;                       // CTAs of the persistent kernel (SMs of the plan's device)
     size_t fwd_ws_bytes = 0;              // partial results of the split units
     std::vector<mate::FwdUnit> fwd_units; // host copies
-    std::vector<int32_t> fwd_cta_off;
     std::vector<mate::PadChunk> pads;
     // tensor-core backward work-list: single halves by decreasing cost; every one is done once per side
     mate::FwdUnit *bwd_units_dev = nullptr;

@@ -1,0 +1,118 @@
+"""Sizes at which the kernels take another branch or a tile is partly filled: work units of the tensor-core
+kernels (global block in front of the own keys, halves filled up with table rows, units cut along their
+tiles), the tiled fp32 kernels, the cell mean's buffers, and plan memory reused between streams."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from tests import helpers as hp
+from workloads import tables
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(rows, cols, P, hv, d, dtype, seed, pad=0):
+    import paper_2109_04312_b200 as m
+    if pad:
+        rows, cols = (np.concatenate([x, np.full((x.shape[0], pad), -1, np.int32)], 1) for x in (rows, cols))
+    B, N = rows.shape
+    rng = np.random.default_rng(seed)
+    vals = {n: (rng.standard_normal((B, len(hv), N, d)) * 0.5).astype(np.float32) for n in ("Q", "K", "V", "dO")}
+    if dtype == "bf16":
+        vals = {n: tables.round_to_bf16(v) for n, v in vals.items()}
+    plan = m.mate_plan(torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda(), P, hv)
+    Q, K, V, dO = (hp.to_dev(vals[n], dtype) for n in ("Q", "K", "V", "dO"))
+    scale = 1.0 / np.sqrt(d)
+    O, LSE = m.mate_attn_fwd(plan, Q, K, V)
+    grads = m.mate_attn_bwd(plan, Q, K, V, O, LSE, dO)
+    torch.cuda.synchronize()
+    plan.status()
+    hv = np.asarray(hv, np.uint8)
+    oO, oL = oracle.fwd(vals["Q"], vals["K"], vals["V"], rows, cols, P, hv, scale)
+    og = oracle.bwd(vals["Q"], vals["K"], vals["V"], vals["dO"], rows, cols, P, hv, scale)
+    assert np.array_equal(plan.useful_pairs(), oracle.useful_pairs(rows, cols, P, hv))
+    atol, rtol = hp.tol(dtype)
+    valid = np.broadcast_to((rows >= 0)[:, None, :], oL.shape)
+    hp.assert_close(hp.to_np(O), oO, atol, rtol, "O")
+    hp.assert_close(hp.to_np(LSE)[valid], oL[valid], atol, rtol, "LSE")
+    for name, g, o in zip(("dQ", "dK", "dV"), grads, og):
+        hp.assert_close(hp.to_np(g), o, atol, rtol, name)
+
+
+def _structure(P, n_table, row_len, n_cols, seed):
+    """P prefix tokens, then n_table table tokens: rows of about row_len tokens, columns drawn at random."""
+    rng = np.random.default_rng(seed)
+    r = np.concatenate([np.zeros(P, np.int32), 1 + np.arange(n_table, dtype=np.int32) // row_len])
+    c = np.concatenate([np.zeros(P, np.int32), rng.integers(1, n_cols + 1, n_table).astype(np.int32)])
+    return r[None, :].astype(np.int32), c[None, :].astype(np.int32)
+
+
+@pytest.mark.parametrize("P,n_table,row_len,n_cols,pad", [
+    (1, 0, 1, 1, 0), (0, 1, 1, 1, 3), (20, 107, 9, 4, 1), (20, 108, 9, 4, 0), (20, 109, 9, 4, 0),   # around 128 positions
+    (100, 155, 40, 3, 0), (100, 156, 40, 3, 0), (100, 157, 40, 3, 0),                                # around 256
+    (64, 300, 64, 2, 5), (116, 400, 12, 5, 0), (127, 260, 130, 2, 0), (128, 256, 128, 2, 0), (129, 255, 17, 2, 0),
+    (383, 129, 33, 3, 0), (384, 200, 33, 3, 0), (16, 2500, 700, 2, 0)])
+def test_tensor_core_unit_edges(P, n_table, row_len, n_cols, pad):
+    rows, cols = _structure(P, n_table, row_len, n_cols, P + n_table)
+    _check(rows, cols, P, [0, 1, 1], 64, "bf16", 7, pad)
+
+
+def test_tensor_core_units_that_are_cut_and_a_busy_grid():
+    rows, cols = _structure(130, 2900, 40, 3, 5)    # few heads: the global rows' units are cut along their tiles
+    _check(rows, cols, 130, [0, 1], 64, "bf16", 8)
+    rows, cols = _structure(70, 330, 25, 4, 6)      # many heads: halves of the global block filled up with table rows
+    rows, cols = np.repeat(rows, 3, 0), np.repeat(cols, 3, 0)
+    _check(rows, cols, 70, [0, 1] * 26, 64, "bf16", 9)
+
+
+@pytest.mark.parametrize("d,dtype", [(8, "f32"), (16, "f32"), (24, "bf16"), (40, "f32"), (64, "f32"), (72, "bf16"), (128, "f32")])
+@pytest.mark.parametrize("P,n_table", [(0, 33), (31, 66), (64, 129), (65, 31)])
+def test_tiled_fp32_kernels(P, n_table, d, dtype):
+    rows, cols = _structure(P, n_table, 11, 3, d)
+    _check(rows, cols, P, [0, 1], d, dtype, d, pad=2)
+
+
+@pytest.mark.parametrize("row_len,n_cols", [(1, 1), (1023, 5), (1025, 129), (2100, 300)])
+def test_cell_mean_buffers(row_len, n_cols):
+    import paper_2109_04312_b200 as m
+    rows, cols = _structure(7, 2 * row_len + 3, row_len, n_cols, row_len)
+    x = np.random.default_rng(3).standard_normal(rows.shape).astype(np.float32)
+    r, c = torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda()
+    plan = m.mate_plan(r, c, 7, [0, 1])
+    mean, count = m.mate_cell_mean(plan, torch.from_numpy(x).cuda(), c)
+    n = np.zeros(tuple(mean.shape[1:]), np.int64)
+    s = np.zeros(n.shape)
+    np.add.at(n, (rows[0, 7:], cols[0, 7:]), 1)
+    np.add.at(s, (rows[0, 7:], cols[0, 7:]), x[0, 7:])
+    assert np.array_equal(count[0].cpu().numpy(), n)
+    hp.assert_close(mean[0].cpu().numpy(), s / np.maximum(n, 1), 1e-5, 1e-5, "mean")
+
+
+def test_plan_memory_is_reused_safely_across_streams_and_in_graphs():
+    import paper_2109_04312_b200 as m
+    rows, cols = _structure(40, 700, 21, 4, 2)
+    r, c = torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda()
+    Q, K, V = ((torch.randn(1, 2, 740, 64, device="cuda") * 0.5).bfloat16() for _ in range(3))
+    torch.cuda.synchronize()
+    want = m.mate_attn_fwd(m.mate_plan(r, c, 40, [0, 1]), Q, K, V)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    got = []
+    for i in range(12):                       # plans made on one stream, used on the next, dropped while in flight
+        with torch.cuda.stream(streams[i % 3]):
+            plan = m.mate_plan(r, c, 40, [0, 1])
+        with torch.cuda.stream(streams[(i + 1 + i // 6) % 3]):
+            got.append(m.mate_attn_fwd(plan, Q, K, V))
+        del plan
+    torch.cuda.synchronize()
+    plan = m.mate_plan(r, c, 40, [0, 1])      # captured before anything else has used it
+    ws = torch.empty(max(m.mate_attn_workspace_bytes(plan, 64, 0)[0], 256), dtype=torch.uint8, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got.append(m.mate_attn_fwd(plan, Q, K, V, workspace=ws))
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    for O, LSE in got:
+        assert torch.equal(O, want[0]) and torch.equal(LSE, want[1])
+    plan.status()

@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         for (uint32_t n = 0; alive; ++n) {
             if (!next_item(n, un)) break;
             const bool key_side = un.ws_off == 0;
-            const int nA = un.tiles_a(), n_tiles = nA + un.tiles_b(), rows_h = un.rows_of(0);
+            const int nA = un.tiles_a(), n_tiles = nA + ((un.kP() + un.kB_end - un.kB0 + kTile - 1) / kTile), rows_h = un.rows_of(0);
             const int rb = item_cnt & 1;
             if (!(alive = wait(bars + 8 * (kBarRFull + rb), (item_cnt >> 1) & 1))) break;
             ++item_cnt;
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         for (uint32_t n = 0; alive; ++n) {
             if (!next_item(n, un)) break;
             const bool key_side = un.ws_off == 0;
-            const int nA = un.tiles_a(), n_tiles = nA + un.tiles_b();
+            const int nA = un.tiles_a(), n_tiles = nA + ((un.kP() + un.kB_end - un.kB0 + kTile - 1) / kTile);
             const int rb = item_cnt & 1;
             if (!(alive = wait(bars + 8 * (kBarRFull + rb), (item_cnt >> 1) & 1))) break;
             tc_fence_after();
@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             }
             if (!next_item(n, un)) break;
             const bool key_side = un.ws_off == 0;
-            const int nA = un.tiles_a(), n_tiles = nA + un.tiles_b(), rows_h = un.rows_of(0);
+            const int nA = un.tiles_a(), n_tiles = nA + ((un.kP() + un.kB_end - un.kB0 + kTile - 1) / kTile), rows_h = un.rows_of(0);
             const ViewPlan &vp = p.head_view[un.h] ? p.colv : p.rowv;
             const size_t bn = (size_t)un.b * p.N;
             const int32_t *perm = vp.perm + bn;

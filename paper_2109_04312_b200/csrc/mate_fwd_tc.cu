@@ -317,9 +317,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             // key ranges of its rows
             const int nA = un.tiles_a(), tB = un.tB & 0xff, kP = un.kP();
             const int k_lo = max(un.lo[h], un.kB0), k_hi = min(un.hi[h], un.kB_end);
-            const int n_pre = nA + (kP + tB - 1) / tB;
-            const int b0 = max(n_pre, nA + (kP + k_lo - un.kB0) / tB);
-            const int n_visit = n_pre + (k_hi > k_lo ? max(nA + (kP + k_hi - un.kB0 - 1) / tB + 1 - b0, 0) : 0);
+            const int n_pre = nA + div_tile(kP + tB - 1, tB);
+            const int b0 = max(n_pre, nA + div_tile(kP + k_lo - un.kB0, tB));
+            const int n_visit = n_pre + (k_hi > k_lo ? max(nA + div_tile(kP + k_hi - un.kB0 - 1, tB) + 1 - b0, 0) : 0);
             const bool exact = (un.tB >> 8) != 0;
             const int w_lo_max = __reduce_max_sync(0xffffffffu, meta[kUnitRows]), w_hi_min = __reduce_min_sync(0xffffffffu, meta[2 * kUnitRows]);
             // The visits whose tile counts in full for every row of the warp: [0, fa) and [fb0, fb1).  (In columns of

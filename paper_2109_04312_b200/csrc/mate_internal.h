@@ -18,6 +18,10 @@ constexpr int kUnitRows = 256;   // query rows per unit of the tensor-core kerne
 enum { kBoundsOwn = 0, kBoundsBefore = 1, kBoundsAfter = 2 };
 constexpr int kTraceCtas = 256;  // CTAs whose cycle counters a -DMATE_TRACE build keeps
 
+// x / tB for tiles of tB columns (x >= 0); nearly always a shift.
+__host__ __device__ inline int div_tile(int x, int tB) { return tB == kTile ? x >> 7 : x / tB; }
+static_assert(kTile == 128, "div_tile");
+
 // One unit of work of the tensor-core kernels: up to 256 consecutive rows (view order) of one (example, head)
 // in two halves of up to 128 -- half 0 = the first n0 rows, half 1 = the n1 rows behind them -- and the
 // column tiles they visit, in this order:
@@ -46,7 +50,7 @@ struct alignas(16) FwdUnit {  // (copied as four 16-byte words)
     __host__ __device__ int n_parts() const { return parts & 0xffff; }
     __host__ __device__ int part() const { return parts >> 16; }
     __host__ __device__ int tiles_a() const { return kA_end > kA0 ? (kA_end - kA0 + kTile - 1) / kTile : 0; }
-    __host__ __device__ int tiles_b() const { return kB_end > kB0 || kP() > 0 ? (kP() + kB_end - kB0 + tB - 1) / tB : 0; }
+    __host__ __device__ int tiles_b() const { return kB_end > kB0 || kP() > 0 ? div_tile(kP() + kB_end - kB0 + tB - 1, tB) : 0; }
 };
 static_assert(sizeof(FwdUnit) == 64, "FwdUnit is read as four 16-byte words");
 

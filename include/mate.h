@@ -56,7 +56,7 @@ enum { MATE_VIEW_ROW = 0, MATE_VIEW_COL = 1 }; /* entries of head_view          
 
 /* flags for mate_attn_fwd / mate_attn_bwd: which implementation runs.
  *   AUTO     tensor-core (tcgen05) kernels when dtype = bf16 and d = 64, otherwise the SIMT kernels
- *   SIMT     one-warp-per-row fp32-arithmetic kernels (any dtype, d <= 128): the debug path
+ *   SIMT     fp32-arithmetic kernels without tensor cores (any dtype, d <= 128)
  *   TCGEN05  tensor-core kernels or MATE_ERR_UNSUPPORTED */
 enum { MATE_IMPL_AUTO = 0, MATE_IMPL_SIMT = 1, MATE_IMPL_TCGEN05 = 2 };
 

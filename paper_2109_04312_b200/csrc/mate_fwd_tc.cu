@@ -25,9 +25,9 @@
 // of tensor pipe), as far as everything else hides behind them.
 //   - A thread takes its whole row of S (128 columns) into registers in one go (setmaxnreg) and gives S
 //     back at once, so the Q K^T of the half's next tile runs under all of this tile's arithmetic.
-//   - On a scheduler one warp of each half shares the exponential unit.  Left alone the two fall into step
-//     and it idles through every wait and load; kept half a tile apart one half's loads run under the
-//     other's exponentials (a fifth faster on long rows of full tiles).  See s_stamp.
+//   - On a scheduler one warp of each half shares the exponential unit.  Holding one half back, so that its loads
+//     fall under the other's exponentials, is not worth its instructions: 37 heads of 8192 dense positions 787 us
+//     with it against 790 without, table batches of 4 x 2048 to 2 x 4096 tokens 0.3 us slower with it.
 //   - Two threads per row (four warps per scheduler) hide the latencies as well, but the control flow of twice
 //     the warps takes more issue slots than that gains.
 //   - The instruction cache is about 32 KB for all roles of the CTA; straight-line code that misses it issues
@@ -69,7 +69,6 @@ constexpr int kLag = 2;                      // loader: copy groups in flight be
 // registers per thread after the roles have split: 256 x 176 + 256 x 80 = 65,536 = the 512 x 128 the CTA is
 // launched with
 constexpr int kRegsSoftmax = 176, kRegsOther = 80;
-constexpr uint32_t kApart = 1000;            // clocks between the exponentials of the two halves
 
 constexpr int kSchedDepth = 4;
 constexpr uint32_t kOffQ = 0;                                // [2 buffers][2 halves] x 16 KB
@@ -182,7 +181,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     volatile uint32_t *tmem_slot = (volatile uint32_t *)(sm + kOffBar + 8 * kNumBars);
     volatile int *s_abort = (volatile int *)(sm + kOffBar + 8 * kNumBars + 4);
     volatile uint32_t *s_bad = (volatile uint32_t *)(sm + kOffBar + 8 * kNumBars + 16);  // [kSchedDepth] warps that need the unit once more
-    volatile uint32_t *s_stamp = s_bad + kSchedDepth;  // [softmax warps] when the warp began its exponentials
     FwdUnit *s_unit = reinterpret_cast<FwdUnit *>(sm + kOffUnit);  // [kSchedDepth]; rows = 0 marks the end of the list
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = tid & 31;
@@ -227,7 +225,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         }
         *s_abort = 0;
         for (int i = 0; i < kSchedDepth; ++i) s_bad[i] = 0;
-        for (int i = 0; i < kSoftmaxWarps; ++i) s_stamp[i] = (uint32_t)clock() - 2 * kApart;
         fence_mbar_init();
     }
     if (warp == kMmaWarp) {
@@ -395,11 +392,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
 #pragma unroll
                         for (int ch = 0; ch < 4; ++ch) chunk_max(v[ch], tm);
                         new_base(fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2);
-                        // When the other half's warp on this scheduler has begun its exponentials a moment ago, let it
-                        // get ahead, at most kApart clocks; the distance then lasts.
-                        if (lane == 0) s_stamp[warp] = (uint32_t)clock();
-#pragma unroll 1
-                        for (int it = 0; it < 64 && h && (uint32_t)clock() - s_stamp[warp ^ 4] < kApart; ++it) {}
                     }
                     const uint64_t neg_m2 = pack_f32x2(-m2, -m2);
 #pragma unroll

@@ -72,25 +72,14 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const void *tmap,
 }
 
 // ------------------------------------------------------------------------------- cp.async
-// 16-byte asynchronous copy global -> shared; src_bytes = 0 writes zeros and reads nothing.
-__device__ __forceinline__ void cp_async16(uint32_t dst_smem, const void *src, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst_smem), "l"(src),
-                 "r"(src_bytes)
-                 : "memory");
-}
+// 16-byte asynchronous copy global -> shared
 __device__ __forceinline__ void cp_async16(uint32_t dst_smem, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async4(uint32_t dst_smem, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst_smem), "l"(src) : "memory");
 }
-// Makes the mbarrier receive one arrival (already counted in its expected count) once all copies
-// this thread has issued so far have landed: the issuing thread does not wait for its own copies.
-__device__ __forceinline__ void cp_async_arrive_noinc(uint32_t bar) {
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 // waits until at most N of this thread's most recent copy groups are still in flight
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() {
@@ -123,33 +112,15 @@ __device__ __forceinline__ void tc_fence_after() {
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate; issued by ONE thread.
-__device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                            uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :
-        : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem]: the A operand (M = 128 rows = lanes, K bf16 elements packed two
-// per 32-bit column, even k in the low half) is read from tensor memory.
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                            uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        :
-        : "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
 // Lean forms for the MMA-issuing thread, whose own instruction count limits the MMA rate: the
 // caller keeps only the low word of each shared-memory descriptor (address >> 4 plus the constant
 // leading-offset field; advancing an operand is one 32-bit add), the constant high word is an
 // immediate, and so is the accumulate flag.
+// Descriptor: 128-byte swizzle, for tiles whose rows are 128 bytes (64 bf16) stored row after row with the 16-byte
+// chunk index XOR-ed with (row & 7); the tile base must be 1024-byte aligned.  Start address >> 4 at bit 0, leading
+// byte offset >> 4 at bit 16, stride byte offset >> 4 at bit 32 (1024 bytes between groups of eight rows), version 1
+// at bit 46, layout type 2 at bit 61.  The same form serves a K-major operand (rows = M or N index, the 64 columns =
+// K) and an MN-major operand (rows = K index, columns = N).
 constexpr uint32_t kDescHiSw128 = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr) {
     return ((saddr & 0x3FFFFu) >> 4) | (1u << 16);
@@ -209,19 +180,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
         : "r"(taddr)
         : "memory");
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-        :
-        : "r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
-          "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]),
-          "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]),
-          "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]),
-          "r"(v[29]), "r"(v[30]), "r"(v[31])
-        : "memory");
-}
 
 // Compiler-level fence for the destination registers of an asynchronous tensor-memory load: an empty
 // statement that "rewrites" them, placed right behind tc_wait_ld().  The values are only valid after
@@ -273,18 +231,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
           "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]),
           "r"(v[15])
         : "memory");
-}
-
-// ------------------------------------------------------------------------------- descriptors
-// Shared-memory operand descriptor, 128-byte swizzle, for tiles whose rows are 128 bytes (64 bf16)
-// stored row after row with the 16-byte chunk index XOR-ed with (row & 7); the tile base must be
-// 1024-byte aligned.  Fields: start address >> 4 at bit 0, leading byte offset >> 4 at bit 16,
-// stride byte offset >> 4 at bit 32 (1024 bytes between groups of eight rows), version 1 at bit
-// 46, layout type 2 (128-byte swizzle) at bit 61.  The same form serves a K-major operand (rows =
-// M or N index, the 64 columns = K) and an MN-major operand (rows = K index, columns = N).
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           (1ull << 46) | (2ull << 61);
 }
 
 // Instruction descriptor for kind::f16 with bf16 A and B and fp32 D: D format (bits 4-5) = 1,

@@ -445,7 +445,7 @@ def run_mate(args, cfg):
         bwd_tflops = fb / (bwd_med * 1e-3) / 1e12
         # Roofline of the dominant kernel, tc_bwd_kernel (one launch = the whole backward of one
         # rank).  Its duration is taken as that of the mate_attn_bwd call, which also holds the
-        # small row-dot kernel (about 5% by the ncu launch list), so `achieved` is a lower bound
+        # small row-dot kernel (5.7% of the two by the ncu launch list), so `achieved` is a lower bound
         # for the kernel itself.
         fwd_tflops_rank = f_fwd / (float(np.mean(fwd_ms)) * 1e-3) / 1e12
         bwd_tflops_rank = f_bwd / (float(np.mean(bwd_ms)) * 1e-3) / 1e12
@@ -467,7 +467,7 @@ def run_mate(args, cfg):
             "tokens_per_s_padded": world * cfg.B * N / (ms_per_step * 1e-3),
             "plan": {"wall_ms": plan_wall_ms, "stream_ms": plan_dev_ms,
                      "note": "mate_plan, pre-computed once per table, outside the timed step: wall time of the call "
-                             "(two allocations, plan kernel, work-lists built on the host) and time between two "
+                             "(pooled memory, plan kernel, work-lists built on the host) and time between two "
                              "events on its stream; plan_kernel alone is in the ncu launch list under profiles/"},
             "cell_mean": None if not cell_ms else {
                 "ms": cell_ms, "gbs": cell_bytes / (cell_ms * 1e-3) / 1e9, "peak_gbs": peaks["hbm_gbs"],

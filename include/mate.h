@@ -68,10 +68,10 @@ enum { MATE_IMPL_AUTO = 0, MATE_IMPL_SIMT = 1, MATE_IMPL_TCGEN05 = 2 };
  *                reordering can be folded into the neighbouring steps).  No gather, no scatter; the
  *                tensor-core kernel then fetches every full K/V tile with bulk tensor copies.  Not for
  *                mate_plan_sat plans and not for mate_attn_bwd (MATE_ERR_UNSUPPORTED).
- *   BULK_TILES   the tensor-core forward fetches the K/V tiles that are contiguous in the tensors -- the
- *                prefix block of every head and, for a row-major table, every tile of the row view --
- *                with bulk tensor copies (one per tile and matrix) instead of row-by-row gathers.  Same
- *                results bit for bit.  This is the default wherever the driver provides tensor maps,
+ *   BULK_TILES   the tensor-core forward fetches the full K/V tiles (and those of a multiple of 16
+ *                columns) that are contiguous in the tensors -- of the prefix block of every head and, for
+ *                a row-major table, of the row view -- with bulk tensor copies (one per tile and matrix)
+ *                instead of row-by-row gathers.  Same results bit for bit.  This is the default wherever the driver provides tensor maps,
  *                so the bit only states it.
  *   GATHER_TILES every K/V tile is gathered row by row.  (Timed back to back on sequences of 512 to
  *                8192 positions, bulk copies are 2-3 % faster on two workloads, equal on one and

@@ -631,7 +631,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             const uint8_t *col_a = reinterpret_cast<const uint8_t *>((key_side ? p.Q : p.K) + bh * 64);
             const int64_t kv = reinterpret_cast<const uint8_t *>(p.V) - reinterpret_cast<const uint8_t *>(p.K),
                           qdo = reinterpret_cast<const uint8_t *>(p.dO) - reinterpret_cast<const uint8_t *>(p.Q);
-            // full column tiles inside [0, ident) of the order are contiguous in the tensors
+            // column tiles inside [0, ident) of the order are contiguous in the tensors (see bulk_tile)
             const int ident = p.use_tma ? __ldg(vp.ident + un.b) : 0;
 
             // step -1: the row operands and row data; steps 0 ..: the column tiles
@@ -647,7 +647,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                 const uint32_t bar_e = i < 0 ? kBarREmpty + rb : kBarCEmpty + st, bar_full = bars + 8 * (i < 0 ? kBarRFull + rb : kBarCFull + st);
                 if (!(alive = wait_free(bars + 8 * bar_e, ((i < 0 ? item_cnt >> 1 : c_cnt / kStages) & 1) ^ 1))) break;
                 const uint32_t dst = base + (i < 0 ? kOffR + rb * 2 * kTileBytes : kOffC + st * 2 * kTileBytes);
-                const bool bulk = i >= 0 && t.contiguous() && t.first() + kTile <= ident;  // (rows behind the tile's own come along)
+                const bool bulk = i >= 0 && bulk_tile(t, ident);
                 if (bulk) {
                     if (lw == 0 && lane == 0) {
                         mbar_expect_tx(bar_full, 2 * kTileBytes);

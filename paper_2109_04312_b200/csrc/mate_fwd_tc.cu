@@ -830,11 +830,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             const size_t bh = p.tr.base(un.b, un.h);
             const uint8_t *Qbh = reinterpret_cast<const uint8_t *>(p.Q + bh * 64), *Kbh = reinterpret_cast<const uint8_t *>(p.K + bh * 64);
             const int64_t v_off = reinterpret_cast<const uint8_t *>(p.V) - reinterpret_cast<const uint8_t *>(p.K);
-            // Rows of the order that sit in place in the tensors ([0, ident)): a full K/V tile inside that
-            // range is one contiguous [128, 64] box and comes in by one bulk tensor copy per matrix
-            // (issued by one thread, completing on the tile's barrier by byte count) instead of 2 x 1024
-            // gathered 16-byte copies.  That is the prefix block of every unit and, for a row-major
-            // table, every tile of the row view.
+            // Rows of the order that sit in place in the tensors ([0, ident)): a K/V tile inside that range
+            // (see bulk_tile) is one contiguous [128, 64] box and comes in by one bulk tensor copy per matrix
+            // (issued by one thread, completing on the tile's barrier by byte count) instead of up to 2 x 1024
+            // gathered 16-byte copies.  That is the prefix block's full tiles in every unit and, for a
+            // row-major table, those of the row view.
             const int ident = !p.use_tma ? 0 : p.view_order ? p.N : __ldg(vp.ident + un.b);
 
             const int qb = unit_cnt & 1;
@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 const uint32_t dst = base + (i < 0 ? kOffQ + (qb * 2 + i + 2) * kTileBytes : kOffKV + stage * 2 * kTileBytes);
                 const uint32_t bar_full = bars + 8 * (i < 0 ? kBarQFull + qb : kBarKVFull + stage);
                 // (Q tiles are always gathered: fetching them with bulk copies as well measured slower.)
-                const bool bulk = i >= 0 && t.contiguous() && t.first() + kTile <= ident;  // (rows behind the tile's own come along)
+                const bool bulk = i >= 0 && bulk_tile(t, ident);
                 TR_T0(t_cp);
                 if (bulk) {
                     if (ltid == 0) {

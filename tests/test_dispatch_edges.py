@@ -66,6 +66,75 @@ def test_tensor_core_units_that_are_cut_and_a_busy_grid():
     _check(rows, cols, 70, [0, 1] * 26, 64, "bf16", 9)
 
 
+def _poisoned(t, where):
+    """A copy of t whose rows `where` (a mask over its rows) hold NaN, Inf and -Inf in turn."""
+    x = t.clone().view(-1, t.shape[-1])
+    i = torch.nonzero(where.reshape(-1)).flatten()
+    x[i] = torch.tensor([float("nan"), float("inf"), -float("inf")], dtype=t.dtype, device=t.device)[i % 3][:, None]
+    return x.view(t.shape)
+
+
+def _fwd_bwd(m, plan, impl, Q, K, V, dO):
+    O, LSE = m.mate_attn_fwd(plan, Q, K, V, None, impl)
+    return (O, LSE) + m.mate_attn_bwd(plan, Q, K, V, O, LSE, dO, None, impl)
+
+
+# The order's rows lie in place in the row view (bulk copies) and not in the column view (gathers); the valid
+# positions end inside a group of 16 (the unit of the matrix instructions), with a whole box of padding behind.
+@pytest.mark.parametrize("kind", ["exact", "bucketed", "sat"])
+@pytest.mark.parametrize("P,n_table,row_len,n_cols", [(64, 136, 150, 2), (20, 301, 9, 4), (100, 157, 40, 3), (128, 259, 259, 1),
+                                                      (31, 0, 1, 1), (130, 1000, 17, 3)])
+def test_values_at_padding_are_ignored(kind, P, n_table, row_len, n_cols):
+    import paper_2109_04312_b200 as m
+    rows, cols = _structure(P, n_table, row_len, n_cols, P + n_table)
+    nv = rows.shape[1]
+    assert nv % 16 != 0
+    rows, cols = (np.concatenate([np.concatenate([x, np.full((1, 160), -1, np.int32)], 1)] * 2) for x in (rows, cols))
+    r, c = torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda()
+    if kind == "sat":
+        plan = m.mate_plan_sat(r, c, P, 3)
+    else:
+        plan = m.mate_plan(r, c, P, [0, 1, 0], radius=24 if kind == "bucketed" else 0)
+    gen = torch.Generator(device="cuda").manual_seed(P)
+    clean = [(torch.randn(2, 3, nv + 160, 64, device="cuda", generator=gen) * 0.5).bfloat16() for _ in range(4)]
+    pad = (r < 0)[:, None, :].expand(2, 3, nv + 160)
+    dirty = [_poisoned(x, pad) for x in clean]
+    for impl in (m.IMPL_TCGEN05, m.IMPL_SIMT):
+        want, got = _fwd_bwd(m, plan, impl, *clean), _fwd_bwd(m, plan, impl, *dirty)
+        for name, w, g in zip(("O", "LSE", "dQ", "dK", "dV"), want, got):
+            assert torch.equal(w, g), (name, impl)
+            assert torch.isfinite(g[~pad]).all(), (name, impl)
+    if kind != "sat":  # in view order every whole box inside the tensors may come by bulk copy
+        perm = torch.from_numpy(np.stack([plan.get(v)[0] for v in (0, 1, 0)], 1).astype(np.int64)).cuda()
+        a, b = ([x.gather(2, perm[..., None].expand(x.shape)) for x in t[:3]] for t in (clean, dirty))
+        flags = m.IMPL_TCGEN05 | m.FLAG_VIEW_ORDER
+        for w, g in zip(m.mate_attn_fwd(plan, *a, None, flags), m.mate_attn_fwd(plan, *b, None, flags)):
+            assert torch.equal(w, g)
+    plan.status()
+
+
+def test_a_packed_example_does_not_reach_its_neighbours():
+    import paper_2109_04312_b200 as m
+    rng = np.random.default_rng(11)
+    prefix, lengths = [64, 20, 40, 7], [200, 421, 61, 333]
+    rows, cols = zip(*((np.concatenate([np.zeros(P, np.int32), 1 + np.arange(L - P, dtype=np.int32) // 90]),
+                        np.concatenate([np.zeros(P, np.int32), rng.integers(1, 4, L - P).astype(np.int32)]))
+                       for P, L in zip(prefix, lengths)))
+    cu = np.concatenate([[0], np.cumsum(lengths)])
+    r, c = (torch.from_numpy(np.concatenate(x)).cuda() for x in (rows, cols))
+    plan = m.mate_plan_packed(r, c, cu, prefix, [0, 1, 0])
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    clean = [(torch.randn(3, int(cu[-1]), 64, device="cuda", generator=gen) * 0.5).bfloat16() for _ in range(4)]
+    for bad in range(4):
+        where = torch.zeros(3, int(cu[-1]), dtype=torch.bool, device="cuda")
+        where[:, cu[bad]:cu[bad + 1]] = True
+        dirty = [_poisoned(x, where) for x in clean]
+        for impl in (m.IMPL_TCGEN05, m.IMPL_SIMT):
+            for name, w, g in zip(("O", "LSE", "dQ", "dK", "dV"), _fwd_bwd(m, plan, impl, *clean), _fwd_bwd(m, plan, impl, *dirty)):
+                assert torch.isfinite(w).all() and torch.equal(w[~where], g[~where]), (name, impl, bad)
+    plan.status()
+
+
 @pytest.mark.parametrize("d,dtype", [(8, "f32"), (16, "f32"), (24, "bf16"), (40, "f32"), (64, "f32"), (72, "bf16"), (128, "f32")])
 @pytest.mark.parametrize("P,n_table", [(0, 33), (31, 66), (64, 129), (65, 31)])
 def test_tiled_fp32_kernels(P, n_table, d, dtype):

@@ -244,6 +244,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
+    // The set-up, here and in every role, may run while the kernel before still does.  Each role then waits for its end
+    // (wait_prior_grid), in front of its first bounded wait: those count this kernel's own time only, and what
+    // they guard comes from that kernel.
+
 #ifdef MATE_TRACE
     long long tr[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const long long tr_start = clock64();
@@ -284,6 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         uint32_t ph_s = 0, ph_g = 0, c_cnt = 0, item_cnt = 0;
         bool alive = true;
         FwdUnit un;
+        wait_prior_grid();
 
 #pragma unroll 1
         for (uint32_t n = 0; alive; ++n) {
@@ -454,6 +459,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         constexpr uint32_t kStep = (16 * kRowBytes) >> 4;    // 16 rows of the column tile
         const uint32_t tA1 = tmem + kTmA1, tA2 = tmem + kTmA2, tG1 = tmem + kTmAcc1, tG2 = tmem + kTmAcc2;
         FwdUnit un;
+        wait_prior_grid();
 #pragma unroll 1
         for (uint32_t n = 0; alive; ++n) {
             if (!next_item(n, un)) break;
@@ -555,7 +561,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
     } else {
         // ------------------------------------------------------------------ loaders
         reg_dealloc<kRegsOther>();
-        wait_prior_grid();  // D, -LSE log2 e and the item counter come from the kernel before
+        wait_prior_grid();
         const int lw = warp - kLoadWarp0;
         uint32_t c_cnt = 0, item_cnt = 0;
         uint32_t pend[kLag];

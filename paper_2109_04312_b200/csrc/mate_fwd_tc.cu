@@ -236,6 +236,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
+    // The set-up, here and in every role, may run while the kernel before still does.  Each role then waits for its end
+    // (wait_prior_grid), in front of its first bounded wait: those count this kernel's own time only, and what
+    // they guard comes from that kernel.
+
     // every wait is bounded; the first one to expire raises the abort flag, which ends all roles
     auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
         if (mbar_test_wait(bar, parity)) return true;  // already complete: no trip through the suspending form
@@ -282,6 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
         uint32_t ph_s = 0, ph_pv = 0, unit_cnt = 0;
         bool alive = true;
+        wait_prior_grid();
 
         for (uint32_t n = 0; alive; ++n) {
             TR_T0(t_nu);
@@ -611,6 +616,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         const uint32_t bar_p = bars + 8 * (kBarPFull + h), bar_s = bars + 8 * (kBarSFull + h),
                        bar_pv = bars + 8 * (kBarPVDone + h), bar_sf = bars + 8 * (kBarSFree + h);
         FwdUnit un;
+        wait_prior_grid();
 
         for (uint32_t n = 0; alive; ++n) {
             if (!next_unit(n, un)) break;
@@ -731,7 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     } else {
         // ------------------------------------------------------------------ loaders
         reg_dealloc<kRegsOther>();
-        wait_prior_grid();  // (the other roles touch global memory only behind data from here)
+        wait_prior_grid();
         const int ltid = tid - 32 * kLoadWarp0, lw = warp - kLoadWarp0;
         uint32_t kv_cnt = 0, unit_cnt = 0;
         uint32_t pend[kLag];

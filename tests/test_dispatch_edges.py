@@ -185,3 +185,33 @@ def test_plan_memory_is_reused_safely_across_streams_and_in_graphs():
     for O, LSE in got:
         assert torch.equal(O, want[0]) and torch.equal(LSE, want[1])
     plan.status()
+
+
+def test_the_kernel_before_does_not_count_against_the_bounded_waits():
+    # A kernel that lets its successor start at once and then keeps one SM busy for about 75 ms: the attention
+    # kernels are resident all that time, several times as long as one of their waits may take.
+    import paper_2109_04312_b200 as m
+    hold = torch.cuda._compile_kernel("""extern "C" __global__ void hold(int kclocks) {
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        const long long t0 = clock64();
+        while (clock64() - t0 < 1000ll * kclocks) {}
+    }""", "hold")
+    rows, cols = _structure(40, 700, 21, 4, 2)
+    plan = m.mate_plan(torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda(), 40, [0, 1])
+    Q, K, V, dO = ((torch.randn(1, 2, 740, 64, device="cuda") * 0.5).bfloat16() for _ in range(4))
+    fwd = lambda: m.mate_attn_fwd(plan, Q, K, V)  # noqa: E731
+    O, LSE = fwd()
+    bwd = lambda: m.mate_attn_bwd(plan, Q, K, V, O, LSE, dO)  # noqa: E731
+    for call in (fwd, bwd):
+        want = call()
+        torch.cuda.synchronize()
+        begin, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        begin.record()
+        hold(grid=(1, 1, 1), block=(1, 1, 1), args=[150000])
+        got = call()
+        end.record()
+        torch.cuda.synchronize()
+        plan.status()
+        assert begin.elapsed_time(end) > 60
+        for w, g in zip(want, got):
+            assert torch.equal(w, g)

@@ -41,6 +41,15 @@ const char kCapsule[] = "mate_plan_info";
 
 struct Raised {};  // a Python exception is set
 
+// Other Python threads run while a call may wait: the allocator for memory to become free, a launch for room in
+// the queue, the first use of a plan on another stream for its upload.
+struct NoGil {
+    PyThreadState *state = PyEval_SaveThread();
+    NoGil() = default;
+    NoGil(const NoGil &) = delete;
+    ~NoGil() { PyEval_RestoreThread(state); }
+};
+
 [[noreturn]] void fail(PyObject *type, const char *msg) {
     PyErr_SetString(type, msg);
     throw Raised();
@@ -107,16 +116,23 @@ at::Tensor empty(c10::IntArrayRef size, at::ScalarType type, c10::Device device)
 struct Workspace {
     void *ptr = nullptr;
     size_t bytes = 0;
+    at::Tensor keep;  // the plan's own: another thread may put a larger one in its place during the call
     Workspace(PyObject *given, PlanInfo &pi, int which, size_t need) {
         if (given != Py_None) {
             const at::Tensor &t = tensor(given, "workspace");
             ptr = t.data_ptr();
             bytes = (size_t)t.numel();
         } else if (need > 0) {
-            at::Tensor &w = pi.ws[which];
-            if (!w.defined() || (size_t)w.numel() < need) w = empty({(int64_t)need}, at::kByte, c10::Device(c10::kCUDA, pi.device));
-            ptr = w.data_ptr();
-            bytes = (size_t)w.numel();
+            keep = pi.ws[which];
+            if (!keep.defined() || (size_t)keep.numel() < need) {
+                {
+                    const NoGil no_gil;
+                    keep = empty({(int64_t)need}, at::kByte, c10::Device(c10::kCUDA, pi.device));
+                }
+                pi.ws[which] = keep;
+            }
+            ptr = keep.data_ptr();
+            bytes = (size_t)keep.numel();
         }
     }
 };
@@ -148,14 +164,22 @@ PyObject *attn_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         const c10::cuda::OptionalCUDAGuard guard(Q.device().index() != c10::cuda::current_device()
                                                      ? std::optional<c10::Device>(Q.device())
                                                      : std::nullopt);
-        const at::Tensor O = a[6] == Py_None ? empty(Q.sizes(), Q.scalar_type(), Q.device()) : tensor(a[6], "O");
-        const at::Tensor LSE = a[7] == Py_None ? empty(Q.sizes().slice(0, Q.dim() - 1), at::kFloat, Q.device()) : tensor(a[7], "LSE");
+        at::Tensor O = a[6] == Py_None ? at::Tensor() : tensor(a[6], "O");
+        at::Tensor LSE = a[7] == Py_None ? at::Tensor() : tensor(a[7], "LSE");
+        void *o = O.defined() ? dev(O, "O") : nullptr, *l = LSE.defined() ? dev(LSE, "LSE") : nullptr;
         size_t need = 0;
         check(lib.workspace_bytes(pi.handle, (int)d, dt, impl, &need, nullptr), "mate_attn_workspace_bytes");
         const Workspace ws(a[8], pi, 0, need);
-        check(lib.fwd(pi.handle, q, k, v, (int)d, dt, scale, dev(O, "O"), (float *)dev(LSE, "LSE"), ws.ptr, ws.bytes, impl,
-                      c10::cuda::getCurrentCUDAStream(Q.device().index()).stream()),
-              "mate_attn_fwd");
+        const mate_plan_t *plan = pi.handle;
+        int status;
+        {
+            const NoGil no_gil;
+            if (!o) O = empty(Q.sizes(), Q.scalar_type(), Q.device()), o = O.data_ptr();
+            if (!l) LSE = empty(Q.sizes().slice(0, Q.dim() - 1), at::kFloat, Q.device()), l = LSE.data_ptr();
+            status = lib.fwd(plan, q, k, v, (int)d, dt, scale, o, (float *)l, ws.ptr, ws.bytes, impl,
+                             c10::cuda::getCurrentCUDAStream(Q.device().index()).stream());
+        }
+        check(status, "mate_attn_fwd");
         PyObject *po = a[6] == Py_None ? THPVariable_Wrap(O) : Py_NewRef(a[6]);
         PyObject *pl = a[7] == Py_None ? THPVariable_Wrap(LSE) : Py_NewRef(a[7]);
         PyObject *r = po && pl ? PyTuple_Pack(2, po, pl) : nullptr;
@@ -186,15 +210,20 @@ PyObject *attn_bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         const c10::cuda::OptionalCUDAGuard guard(Q.device().index() != c10::cuda::current_device()
                                                      ? std::optional<c10::Device>(Q.device())
                                                      : std::nullopt);
-        at::Tensor g[3];
-        for (at::Tensor &x : g) x = empty(Q.sizes(), Q.scalar_type(), Q.device());
         size_t need = 0;
         check(lib.workspace_bytes(pi.handle, (int)d, dt, impl, nullptr, &need), "mate_attn_workspace_bytes");
         const Workspace ws(a[9], pi, 1, need);
-        check(lib.bwd(pi.handle, ptr[0], ptr[1], ptr[2], ptr[3], (const float *)ptr[4], ptr[5], (int)d, dt, scale, g[0].data_ptr(),
-                      g[1].data_ptr(), g[2].data_ptr(), ws.ptr, ws.bytes, impl,
-                      c10::cuda::getCurrentCUDAStream(Q.device().index()).stream()),
-              "mate_attn_bwd");
+        const mate_plan_t *plan = pi.handle;
+        at::Tensor g[3];
+        int status;
+        {
+            const NoGil no_gil;
+            for (at::Tensor &x : g) x = empty(Q.sizes(), Q.scalar_type(), Q.device());
+            status = lib.bwd(plan, ptr[0], ptr[1], ptr[2], ptr[3], (const float *)ptr[4], ptr[5], (int)d, dt, scale, g[0].data_ptr(),
+                             g[1].data_ptr(), g[2].data_ptr(), ws.ptr, ws.bytes, impl,
+                             c10::cuda::getCurrentCUDAStream(Q.device().index()).stream());
+        }
+        check(status, "mate_attn_bwd");
         PyObject *r = PyTuple_New(3);
         for (int i = 0; r && i < 3; ++i) {
             PyObject *o = THPVariable_Wrap(g[i]);
@@ -225,12 +254,18 @@ PyObject *cell_mean(PyObject *, PyObject *const *a, Py_ssize_t n) {
                                                      ? std::optional<c10::Device>(x.device())
                                                      : std::nullopt);
         const int64_t shape[3] = {pi.B, pi.n_rows, pi.n_cols};
-        const at::Tensor mean = given ? tensor(a[4], "mean") : empty(shape, at::kFloat, x.device());
-        const at::Tensor count = !want ? at::Tensor() : given ? tensor(a[5], "count") : empty(shape, at::kInt, x.device());
-        check(lib.cell_mean(pi.handle, (const float *)px, (const int32_t *)pc, (float *)dev(mean, "mean"),
-                            want ? (int32_t *)dev(count, "count") : nullptr,
-                            c10::cuda::getCurrentCUDAStream(x.device().index()).stream()),
-              "mate_cell_mean");
+        at::Tensor mean = given ? tensor(a[4], "mean") : at::Tensor(), count = given && want ? tensor(a[5], "count") : at::Tensor();
+        void *pm_out = given ? dev(mean, "mean") : nullptr, *pn_out = given && want ? dev(count, "count") : nullptr;
+        const mate_plan_t *plan = pi.handle;
+        int status;
+        {
+            const NoGil no_gil;
+            if (!given) mean = empty(shape, at::kFloat, x.device()), pm_out = mean.data_ptr();
+            if (!given && want) count = empty(shape, at::kInt, x.device()), pn_out = count.data_ptr();
+            status = lib.cell_mean(plan, (const float *)px, (const int32_t *)pc, (float *)pm_out, (int32_t *)pn_out,
+                                   c10::cuda::getCurrentCUDAStream(x.device().index()).stream());
+        }
+        check(status, "mate_cell_mean");
         PyObject *pm = given ? Py_NewRef(a[4]) : THPVariable_Wrap(mean);
         PyObject *po = !want ? Py_NewRef(Py_None) : given ? Py_NewRef(a[5]) : THPVariable_Wrap(count);
         PyObject *r = pm && po ? PyTuple_Pack(2, pm, po) : nullptr;

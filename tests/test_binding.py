@@ -1,0 +1,49 @@
+"""The native binding of the per-layer calls: what it lets other threads do, and what it refuses."""
+import ctypes
+import threading
+import time
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def test_other_threads_run_while_a_call_waits():
+    # libc's usleep stands in for the three entry points that may wait: their first argument, the plan's address, is
+    # what it takes for its microseconds, and it returns 0 (MATE_OK)
+    import paper_2109_04312_b200 as m
+    lib = m.api._load()
+    from paper_2109_04312_b200 import _native
+    address = lambda f: ctypes.cast(f, ctypes.c_void_p).value  # noqa: E731
+    nothing = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_uint, ctypes.c_void_p,
+                               ctypes.c_void_p)(lambda *a: 0)
+    usleep = address(ctypes.CDLL(None).usleep)
+    info = _native.plan_info(200000, 1, 16, 2, -1, 1, 1, torch.cuda.current_device())
+    t, lse = torch.zeros(1, 2, 16, 64, device="cuda"), torch.zeros(1, 2, 16, device="cuda")
+    logits, ids = torch.zeros(1, 16, device="cuda"), torch.zeros(1, 16, dtype=torch.int32, device="cuda")
+    ticks, stop = [0], threading.Event()
+
+    def tick():
+        while not stop.is_set():
+            time.sleep(0.001)
+            ticks[0] += 1
+
+    thread = threading.Thread(target=tick)
+    _native.bind(address(nothing), usleep, usleep, usleep, m.MateError)
+    try:
+        thread.start()
+        for call in (lambda: _native.attn_fwd(info, t, t, t, None, 0, None, None, None),
+                     lambda: _native.attn_fwd(info, t, t, t, None, 0, t, lse, None),
+                     lambda: _native.attn_bwd(info, t, t, t, t, lse, t, None, 0, None),
+                     lambda: _native.cell_mean(info, logits, ids, True, None, None),
+                     lambda: _native.cell_mean(info, logits, ids, False, logits, None)):
+            before, begin = ticks[0], time.monotonic()
+            call()
+            assert time.monotonic() - begin > 0.19
+            assert ticks[0] - before > 20
+    finally:
+        stop.set()
+        thread.join()
+        _native.bind(*(address(f) for f in (lib.mate_attn_workspace_bytes, lib.mate_attn_fwd, lib.mate_attn_bwd,
+                                            lib.mate_cell_mean)), m.MateError)

@@ -57,6 +57,7 @@ bool pool_take(size_t bytes, cudaStream_t st, int device, Block *out) {
             if (out->stream != id || id == 0) {
                 if (cudaDeviceSynchronize() != cudaSuccess) {
                     cudaFree(out->ptr);
+                    *out = Block{};  // nothing for the caller to give back
                     return false;
                 }
             }

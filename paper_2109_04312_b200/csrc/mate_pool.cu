@@ -158,7 +158,7 @@ cudaError_t use_plan(const mate_plan_t *plan, cudaStream_t st) {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaError_t rc = cudaStreamIsCapturing(st, &capture);
     if (rc != cudaSuccess) return rc;
-    if (capture == cudaStreamCaptureStatusNone && stream_id(st) == plan->stream) return cudaSuccess;
+    if (capture == cudaStreamCaptureStatusNone && plan->stream != 0 && stream_id(st) == plan->stream) return cudaSuccess;
     plan->elsewhere = true;
     std::lock_guard<std::mutex> lock(plan->ready_mu);
     if (!plan->ready) return cudaSuccess;

@@ -53,3 +53,10 @@ def test_a_block_whose_wait_fails_is_gone(pool):
     for i in (2, 3):
         pool.pool_give(i, 2)
     assert pool.fake_bad_frees() == 0
+
+
+def test_a_plan_is_waited_for_on_any_stream_but_its_own(pool):
+    assert pool.plan_waits(1, 1) == 0
+    assert pool.plan_waits(1, 2) == 1
+    assert pool.plan_waits(0, 1) == 1 and pool.plan_waits(1, 0) == 1
+    assert pool.plan_waits(0, 0) == 1                 # two unknown streams are not one

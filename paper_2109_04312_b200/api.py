@@ -319,6 +319,8 @@ def mate_attn_bwd_noalloc(plan, Q, K, V, O, LSE, dO, dQ, dK, dV, scale=None):
     for t in (K, V, O, dO, dQ, dK, dV):
         if t.shape != Q.shape or t.dtype != Q.dtype:
             raise ValueError("K, V, O, dO, dQ, dK, dV must match Q in shape and dtype")
+    if LSE.dtype != torch.float32 or LSE.numel() * d < Q.numel():
+        raise ValueError("LSE must be a float32 tensor with one element per row")
     if scale is None:
         scale = 1.0 / float(d) ** 0.5
     with torch.cuda.device(Q.device):

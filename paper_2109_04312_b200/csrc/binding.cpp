@@ -112,6 +112,13 @@ at::Tensor empty(c10::IntArrayRef size, at::ScalarType type, c10::Device device)
     return at::Tensor(at::detail::empty_cuda(size, type, device, std::nullopt));
 }
 
+// A tensor that is read or written as `n` elements of a type has that type, and at least as many.
+void holds(const at::Tensor &t, at::ScalarType type, int64_t n, const char *name) {
+    if (t.scalar_type() == type && t.numel() >= n) return;
+    PyErr_Format(PyExc_ValueError, "%s must be a %s tensor of %lld elements", name, c10::toString(type), (long long)n);
+    throw Raised();
+}
+
 // The caller's workspace, or the plan's own (allocated at the first call, kept afterwards).
 struct Workspace {
     void *ptr = nullptr;
@@ -158,14 +165,18 @@ PyObject *attn_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         const int64_t d = split(pi, Q);
         if (K.sizes() != Q.sizes() || V.sizes() != Q.sizes()) fail(PyExc_ValueError, "tensor shapes do not match the plan");
         const int dt = dtype_code(Q);
+        for (const at::Tensor *t : {&K, &V})
+            if (t->scalar_type() != Q.scalar_type()) fail(PyExc_ValueError, "K and V must match Q in dtype");
+        at::Tensor O = a[6] == Py_None ? at::Tensor() : tensor(a[6], "O");
+        at::Tensor LSE = a[7] == Py_None ? at::Tensor() : tensor(a[7], "LSE");
+        if (O.defined()) holds(O, Q.scalar_type(), Q.numel(), "O");
+        if (LSE.defined()) holds(LSE, at::kFloat, d > 0 ? Q.numel() / d : 0, "LSE");
         const float scale = scale_of(a[4], d);
         const unsigned impl = flags_of(a[5]);
         void *q = dev(Q, "Q"), *k = dev(K, "K"), *v = dev(V, "V");
         const c10::cuda::OptionalCUDAGuard guard(Q.device().index() != c10::cuda::current_device()
                                                      ? std::optional<c10::Device>(Q.device())
                                                      : std::nullopt);
-        at::Tensor O = a[6] == Py_None ? at::Tensor() : tensor(a[6], "O");
-        at::Tensor LSE = a[7] == Py_None ? at::Tensor() : tensor(a[7], "LSE");
         void *o = O.defined() ? dev(O, "O") : nullptr, *l = LSE.defined() ? dev(LSE, "LSE") : nullptr;
         size_t need = 0;
         check(lib.workspace_bytes(pi.handle, (int)d, dt, impl, &need, nullptr), "mate_attn_workspace_bytes");
@@ -203,6 +214,7 @@ PyObject *attn_bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
             if (t[i]->sizes() != Q.sizes() || t[i]->scalar_type() != Q.scalar_type())
                 fail(PyExc_ValueError, "K, V, O, dO must match Q in shape and dtype");
         const int dt = dtype_code(Q);
+        holds(*t[4], at::kFloat, d > 0 ? Q.numel() / d : 0, "LSE");
         const float scale = scale_of(a[7], d);
         const unsigned impl = flags_of(a[8]);
         void *ptr[6];
@@ -249,12 +261,14 @@ PyObject *cell_mean(PyObject *, PyObject *const *a, Py_ssize_t n) {
             fail(PyExc_ValueError, "col_ids must be the int32 [B, N] tensor given to mate_plan");
         const bool given = a[4] != Py_None;  // (mean, count) tensors of an earlier call, written in place
         const bool want = given ? a[5] != Py_None : PyObject_IsTrue(a[3]) == 1;
+        at::Tensor mean = given ? tensor(a[4], "mean") : at::Tensor(), count = given && want ? tensor(a[5], "count") : at::Tensor();
+        if (given) holds(mean, at::kFloat, pi.B * pi.n_rows * pi.n_cols, "mean");
+        if (given && want) holds(count, at::kInt, pi.B * pi.n_rows * pi.n_cols, "count");
         void *px = dev(x, "logits"), *pc = dev(ids, "col_ids");
         const c10::cuda::OptionalCUDAGuard guard(x.device().index() != c10::cuda::current_device()
                                                      ? std::optional<c10::Device>(x.device())
                                                      : std::nullopt);
         const int64_t shape[3] = {pi.B, pi.n_rows, pi.n_cols};
-        at::Tensor mean = given ? tensor(a[4], "mean") : at::Tensor(), count = given && want ? tensor(a[5], "count") : at::Tensor();
         void *pm_out = given ? dev(mean, "mean") : nullptr, *pn_out = given && want ? dev(count, "count") : nullptr;
         const mate_plan_t *plan = pi.handle;
         int status;

@@ -6,9 +6,8 @@ import time
 import pytest
 import torch
 
-pytestmark = pytest.mark.gpu
 
-
+@pytest.mark.gpu
 def test_other_threads_run_while_a_call_waits():
     # libc's usleep stands in for the three entry points that may wait: their first argument, the plan's address, is
     # what it takes for its microseconds, and it returns 0 (MATE_OK)
@@ -47,3 +46,42 @@ def test_other_threads_run_while_a_call_waits():
         thread.join()
         _native.bind(*(address(f) for f in (lib.mate_attn_workspace_bytes, lib.mate_attn_fwd, lib.mate_attn_bwd,
                                             lib.mate_cell_mean)), m.MateError)
+
+
+def test_types_and_sizes_are_checked_before_anything_is_launched():
+    # host tensors: what is refused here is refused for its type or size; what passes stops at the next check,
+    # that the tensors are on a GPU
+    import paper_2109_04312_b200 as m
+    m.api._load()
+    from paper_2109_04312_b200 import _native
+    info = _native.plan_info(0, 1, 16, 2, -1, 3, 5, 0)
+    q, h = torch.zeros(1, 2, 16, 64), torch.zeros(1, 2, 16, 64, dtype=torch.bfloat16)
+    stat, ids = torch.zeros(1, 2, 16), torch.zeros(1, 16, dtype=torch.int32)
+
+    def fwd(k=q, v=q, out=None, lse=None):
+        _native.attn_fwd(info, q, k, v, None, 0, out, lse, None)
+
+    def bwd(lse):
+        _native.attn_bwd(info, q, q, q, q, lse, q, None, 0, None)
+
+    def cells(mean, count):
+        _native.cell_mean(info, torch.zeros(1, 16), ids, True, mean, count)
+
+    def noalloc(lse):
+        plan = m.Plan.__new__(m.Plan)
+        plan._h, plan.B, plan.H, plan.N, plan.T = None, 1, 2, 16, None
+        m.mate_attn_bwd_noalloc(plan, q, q, q, q, lse, q, q, q, q)
+
+    for what, call in (("K and V", lambda: fwd(k=h)), ("K and V", lambda: fwd(v=h)), ("O", lambda: fwd(out=h)),
+                       ("O", lambda: fwd(out=q[..., :32])), ("LSE", lambda: fwd(lse=stat.bfloat16())),
+                       ("LSE", lambda: fwd(lse=stat[..., 1:])), ("LSE", lambda: bwd(stat.bfloat16())), ("LSE", lambda: bwd(stat[..., 1:])),
+                       ("mean", lambda: cells(torch.zeros(1, 3, 5).half(), torch.zeros(1, 3, 5, dtype=torch.int32))),
+                       ("mean", lambda: cells(torch.zeros(1, 3, 4), torch.zeros(1, 3, 5, dtype=torch.int32))),
+                       ("count", lambda: cells(torch.zeros(1, 3, 5), torch.zeros(1, 3, 5, dtype=torch.int16))),
+                       ("LSE", lambda: noalloc(stat.bfloat16())), ("LSE", lambda: noalloc(stat[..., 1:]))):
+        with pytest.raises(ValueError, match="^%s must (match|be a )(?!contiguous)" % what):
+            call()
+    for call in (lambda: fwd(out=q, lse=stat), lambda: fwd(out=q.flatten(), lse=torch.zeros(40)), lambda: bwd(stat),
+                 lambda: cells(torch.zeros(1, 3, 5), torch.zeros(1, 3, 5, dtype=torch.int32))):
+        with pytest.raises(ValueError, match="contiguous CUDA tensor"):
+            call()

@@ -17,7 +17,8 @@
  *   - Q is the first prefix_len positions; their row and column ids must be 0.
  *   - a negative id marks padding (both arrays must agree).  Padding keys are never attended;
  *     padding query rows return O = 0, LSE = -inf and zero gradients; values stored at padding
- *     positions are ignored.
+ *     positions are ignored, whatever they are.  (A NaN or Inf at a valid position may also reach rows
+ *     of its example that do not attend it: tiles are multiplied whole, masked pairs with weight 0.)
  *   - a table token whose id is 0 is an ordinary table token (segment 0).
  *   - masking removes a key from the softmax support; `scale` multiplies q.k before the softmax.
  *   - LSE is the natural-log logsumexp of the scaled scores over A.
@@ -71,11 +72,11 @@ enum { MATE_IMPL_AUTO = 0, MATE_IMPL_SIMT = 1, MATE_IMPL_TCGEN05 = 2 };
  *   BULK_TILES   the tensor-core forward fetches the full K/V tiles (and those of a multiple of 16
  *                columns) that are contiguous in the tensors -- of the prefix block of every head and, for
  *                a row-major table, of the row view -- with bulk tensor copies (one per tile and matrix)
- *                instead of row-by-row gathers.  Same results bit for bit.  This is the default wherever the driver provides tensor maps,
- *                so the bit only states it.
+ *                instead of row-by-row gathers.  Same results bit for bit.  This is the default wherever
+ *                the driver provides tensor maps, so the bit only states it.
  *   GATHER_TILES every K/V tile is gathered row by row.  (Timed back to back on sequences of 512 to
- *                8192 positions, bulk copies are 2-3 % faster on two workloads, equal on one and
- *                0.6 % slower on one.)  Both bits together: MATE_ERR_INVALID_ARG. */
+ *                8192 positions, bulk copies are 1 % faster on one workload and within 0.6 % on the
+ *                others.)  Both bits together: MATE_ERR_INVALID_ARG. */
 enum { MATE_FLAG_VIEW_ORDER = 4, MATE_FLAG_BULK_TILES = 8, MATE_FLAG_GATHER_TILES = 16 };
 
 const char *mate_status_string(int status);

@@ -85,8 +85,8 @@ struct RowBounds {
 
 // ---------------------------------------------------------------------------- work-lists
 // Work-lists of the tensor-core kernels, built on the host from the segment offsets: the rows of every
-// (example, view) are cut into units (see FwdUnit), the same for all heads of the view, and the units are
-// dealt to the CTAs.
+// (example, view) are cut into units (see FwdUnit), the same for all heads of the view, and listed by
+// decreasing cost; the CTAs take them from the head of the list through a counter.
 constexpr int kChunk = 32;
 
 // Key ranges of the rows of one (example, view), by view position.

@@ -86,7 +86,7 @@ enum {
 constexpr int kSchedReaders = kComputeWarps + 1 + kLoadWarps;
 // tensor memory columns
 constexpr uint32_t kTmS = 0, kTmT = 128, kTmA1 = 256, kTmA2 = 320, kTmAcc1 = 384, kTmAcc2 = 448;
-constexpr uint32_t kWaitLimit = 4096;  // tries (up to 1 ms each) before a wait gives up
+constexpr uint32_t kWaitLimit = 4096;  // tries (about 5 us each) before a wait gives up
 
 struct Params {
     CUtensorMap tmQ, tmK, tmV, tmdO;  // boxes of 128 rows, 128-byte swizzle

@@ -26,8 +26,8 @@
 //   - A thread takes its whole row of S (128 columns) into registers in one go (setmaxnreg) and gives S
 //     back at once, so the Q K^T of the half's next tile runs under all of this tile's arithmetic.
 //   - On a scheduler one warp of each half shares the exponential unit.  Holding one half back, so that its loads
-//     fall under the other's exponentials, is not worth its instructions: 37 heads of 8192 dense positions 787 us
-//     with it against 790 without, table batches of 4 x 2048 to 2 x 4096 tokens 0.3 us slower with it.
+//     fall under the other's exponentials, is not worth its instructions: 37 heads of 8192 dense positions 840 us
+//     with it against 845 without, table batches of 4 x 2048 to 2 x 4096 tokens 0.3 us slower with it.
 //   - Two threads per row (four warps per scheduler) hide the latencies as well, but the control flow of twice
 //     the warps takes more issue slots than that gains.
 //   - The instruction cache is about 32 KB for all roles of the CTA; straight-line code that misses it issues
@@ -83,7 +83,7 @@ static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kTmemO = 256;
 constexpr uint32_t kTmemP = 384;
-constexpr uint32_t kWaitLimit = 4096;        // tries (up to 1 ms each) before a wait gives up
+constexpr uint32_t kWaitLimit = 4096;        // tries (about 5 us each) before a wait gives up
 constexpr float kRescale = 8.f;                              // exact units: log2 units before the base moves
 constexpr float kSumMin = 0x1p-100f, kSumMax = 0x1p60f;      // row sums outside: the unit is done once more, exactly
 
@@ -863,7 +863,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 }
                 const uint32_t dst = base + (i < 0 ? kOffQ + (qb * 2 + i + 2) * kTileBytes : kOffKV + stage * 2 * kTileBytes);
                 const uint32_t bar_full = bars + 8 * (i < 0 ? kBarQFull + qb : kBarKVFull + stage);
-                // (Q tiles are always gathered: fetching them with bulk copies as well measured slower.)
+                // (Q tiles are always gathered: their rows past the half's own repeat one of them.)
                 const bool bulk = i >= 0 && bulk_tile(t, ident);
                 TR_T0(t_cp);
                 if (bulk) {
@@ -970,10 +970,10 @@ int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     if (g_smem_attr.ensure((const void *)tc_fwd_kernel, (int)kSmemBytes, plan->device) != MATE_OK) return MATE_ERR_CUDA;
     Params p;
     const size_t rows = plan->n_rows();
-    // Bulk tensor copies for the K/V tiles that are contiguous in the caller's tensors, unless the caller
-    // asks for gathers (back to back the bulk copies measured 2-3 % faster on two workloads, equal on one,
-    // 0.6 % slower on one); tensors in view order always take them.  When the driver entry point for
-    // tensor maps is missing every tile is gathered.
+    // Bulk tensor copies for the K/V tiles that are contiguous in the caller's tensors (see bulk_tile), unless the
+    // caller asks for gathers; tensors in view order always take them.  Bulk copies against gathers, back to back:
+    // 4 x 2048 tokens 32.3 us against 32.7, 8 x 512 17.9 and 17.9, 2 x 4096 55.5 and 55.4, 1 x 8192 54.8 and 54.5.
+    // When the driver entry point for tensor maps is missing every tile is gathered.
     const bool want_bulk = !(flags & MATE_FLAG_GATHER_TILES) || (flags & MATE_FLAG_VIEW_ORDER);
     p.use_tma = want_bulk && rows < (size_t(1) << 31) && make_row_map(&p.tmK, K, rows) && make_row_map(&p.tmV, V, rows);
     p.view_order = (flags & MATE_FLAG_VIEW_ORDER) ? 1 : 0;

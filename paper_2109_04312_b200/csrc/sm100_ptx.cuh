@@ -19,8 +19,9 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void fence_mbar_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
-// One try: the thread may be suspended by the hardware until the phase completes or the time hint
-// (nanoseconds) runs out, so a waiting warp takes no issue slots from the warps that compute.
+// One try: the thread may be suspended by the hardware until the phase completes or a time runs out, so a
+// waiting warp takes no issue slots from the warps that compute.  The hint (nanoseconds) is an upper bound: a
+// try that fails takes about 5 us on this GPU.
 constexpr uint32_t kTryWaitHintNs = 1000000u;
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;

@@ -36,6 +36,7 @@ struct PlanInfo {
     int64_t n_rows, n_cols;  // ids per view (cell mean)
     c10::DeviceIndex device;
     at::Tensor ws[2];    // workspaces of forward and backward, kept from call to call
+    c10::StreamId ws_stream[2];  // the streams they were allocated on
 };
 const char kCapsule[] = "mate_plan_info";
 
@@ -124,7 +125,7 @@ struct Workspace {
     void *ptr = nullptr;
     size_t bytes = 0;
     at::Tensor keep;  // the plan's own: another thread may put a larger one in its place during the call
-    Workspace(PyObject *given, PlanInfo &pi, int which, size_t need) {
+    Workspace(PyObject *given, PlanInfo &pi, int which, size_t need, const c10::cuda::CUDAStream &stream) {
         if (given != Py_None) {
             const at::Tensor &t = tensor(given, "workspace");
             ptr = t.data_ptr();
@@ -137,6 +138,9 @@ struct Workspace {
                     keep = empty({(int64_t)need}, at::kByte, c10::Device(c10::kCUDA, pi.device));
                 }
                 pi.ws[which] = keep;
+                pi.ws_stream[which] = stream.id();
+            } else if (stream.id() != pi.ws_stream[which]) {
+                keep.record_stream(stream);  // not to be handed out again before this call's kernels are done
             }
             ptr = keep.data_ptr();
             bytes = (size_t)keep.numel();
@@ -180,15 +184,15 @@ PyObject *attn_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         void *o = O.defined() ? dev(O, "O") : nullptr, *l = LSE.defined() ? dev(LSE, "LSE") : nullptr;
         size_t need = 0;
         check(lib.workspace_bytes(pi.handle, (int)d, dt, impl, &need, nullptr), "mate_attn_workspace_bytes");
-        const Workspace ws(a[8], pi, 0, need);
+        const c10::cuda::CUDAStream stream = c10::cuda::getCurrentCUDAStream(Q.device().index());
+        const Workspace ws(a[8], pi, 0, need, stream);
         const mate_plan_t *plan = pi.handle;
         int status;
         {
             const NoGil no_gil;
             if (!o) O = empty(Q.sizes(), Q.scalar_type(), Q.device()), o = O.data_ptr();
             if (!l) LSE = empty(Q.sizes().slice(0, Q.dim() - 1), at::kFloat, Q.device()), l = LSE.data_ptr();
-            status = lib.fwd(plan, q, k, v, (int)d, dt, scale, o, (float *)l, ws.ptr, ws.bytes, impl,
-                             c10::cuda::getCurrentCUDAStream(Q.device().index()).stream());
+            status = lib.fwd(plan, q, k, v, (int)d, dt, scale, o, (float *)l, ws.ptr, ws.bytes, impl, stream.stream());
         }
         check(status, "mate_attn_fwd");
         PyObject *po = a[6] == Py_None ? THPVariable_Wrap(O) : Py_NewRef(a[6]);
@@ -224,7 +228,8 @@ PyObject *attn_bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
                                                      : std::nullopt);
         size_t need = 0;
         check(lib.workspace_bytes(pi.handle, (int)d, dt, impl, nullptr, &need), "mate_attn_workspace_bytes");
-        const Workspace ws(a[9], pi, 1, need);
+        const c10::cuda::CUDAStream stream = c10::cuda::getCurrentCUDAStream(Q.device().index());
+        const Workspace ws(a[9], pi, 1, need, stream);
         const mate_plan_t *plan = pi.handle;
         at::Tensor g[3];
         int status;
@@ -232,8 +237,7 @@ PyObject *attn_bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
             const NoGil no_gil;
             for (at::Tensor &x : g) x = empty(Q.sizes(), Q.scalar_type(), Q.device());
             status = lib.bwd(plan, ptr[0], ptr[1], ptr[2], ptr[3], (const float *)ptr[4], ptr[5], (int)d, dt, scale, g[0].data_ptr(),
-                             g[1].data_ptr(), g[2].data_ptr(), ws.ptr, ws.bytes, impl,
-                             c10::cuda::getCurrentCUDAStream(Q.device().index()).stream());
+                             g[1].data_ptr(), g[2].data_ptr(), ws.ptr, ws.bytes, impl, stream.stream());
         }
         check(status, "mate_attn_bwd");
         PyObject *r = PyTuple_New(3);
@@ -295,7 +299,7 @@ PyObject *new_plan_info(PyObject *, PyObject *args) {
     long long B, N, H, T, nr, nc;
     int device;
     if (!PyArg_ParseTuple(args, "KLLLLLLi", &h, &B, &N, &H, &T, &nr, &nc, &device)) return nullptr;
-    PlanInfo *pi = new PlanInfo{reinterpret_cast<const mate_plan_t *>(h), B, N, H, T, nr, nc, (c10::DeviceIndex)device, {}};
+    PlanInfo *pi = new PlanInfo{reinterpret_cast<const mate_plan_t *>(h), B, N, H, T, nr, nc, (c10::DeviceIndex)device, {}, {}};
     return PyCapsule_New(pi, kCapsule, [](PyObject *c) { delete static_cast<PlanInfo *>(PyCapsule_GetPointer(c, kCapsule)); });
 }
 // drop(info): the plan has been destroyed; later calls report a null plan

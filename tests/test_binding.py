@@ -48,6 +48,32 @@ def test_other_threads_run_while_a_call_waits():
                                             lib.mate_cell_mean)), m.MateError)
 
 
+@pytest.mark.gpu
+def test_a_plans_workspace_outlives_it_on_every_stream():
+    # The workspace is allocated by the first call and used by one on another stream, which is still to run when
+    # the plan goes: the memory must not be handed out on the first stream until then.
+    import paper_2109_04312_b200 as m
+    ids = torch.ones(1, 4096, dtype=torch.int32, device="cuda")
+    Q, K, V, dO = ((torch.randn(1, 2, 4096, 64, device="cuda") * 0.5).bfloat16() for _ in range(4))
+    plan = m.mate_plan(ids, ids, 0, [0, 1])
+    need = m.mate_attn_workspace_bytes(plan, 64, 0)
+    assert min(need) > 0                              # (few heads: units are cut, and their parts go through it)
+    O, LSE = m.mate_attn_fwd(plan, Q, K, V)
+    want = (O, LSE) + m.mate_attn_bwd(plan, Q, K, V, O, LSE, dO)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(50_000_000)
+        o, l = m.mate_attn_fwd(plan, Q, K, V)
+        got = (o, l) + m.mate_attn_bwd(plan, Q, K, V, o, l, dO)
+    plan.destroy()
+    junk = [torch.full((n,), 255, dtype=torch.uint8, device="cuda") for n in need * 4]   # NaN, whatever is read there
+    torch.cuda.synchronize()
+    for w, g in zip(want, got):
+        assert torch.equal(w, g)
+    del junk
+
+
 def test_types_and_sizes_are_checked_before_anything_is_launched():
     # host tensors: what is refused here is refused for its type or size; what passes stops at the next check,
     # that the tensors are on a GPU

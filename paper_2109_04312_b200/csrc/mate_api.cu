@@ -3,6 +3,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
 #include <new>
 
 #include "mate_internal.h"
@@ -17,6 +18,17 @@ namespace {
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
+
+// The entry points that make plans hold lists as long as their inputs: memory that is not to be had is a status
+// there, never an exception across the C boundary.
+template <typename F>
+int no_throw(F &&f) {
+    try {
+        return f();
+    } catch (const std::exception &) {
+        return MATE_ERR_NOMEM;
+    }
+}
 
 // Carves the plan's device arrays out of one allocation.
 struct Carver {
@@ -509,9 +521,11 @@ int mate_plan_bucketed(const int32_t *row_ids, const int32_t *col_ids, int B, in
                        void *stream, mate_plan_t **out) {
     if (out) *out = nullptr;
     if (B <= 0) return MATE_ERR_INVALID_ARG;
-    const std::vector<int32_t> prefix((size_t)B, prefix_len);
-    return mate_plan_varlen(row_ids, col_ids, B, N, prefix.data(), head_view, H, max_row_id, max_col_id, radius,
-                            stream, out);
+    return no_throw([&]() {
+        const std::vector<int32_t> prefix((size_t)B, prefix_len);
+        return mate_plan_varlen(row_ids, col_ids, B, N, prefix.data(), head_view, H, max_row_id, max_col_id, radius,
+                                stream, out);
+    });
 }
 
 static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int N, const int32_t *prefix_len,
@@ -539,10 +553,9 @@ int mate_plan_bucketed_global(const int32_t *row_ids, const int32_t *col_ids, in
 /* Packed batches: the examples lie one behind the other on a common token axis.  The plan itself is the
  * padded one over N = the longest example (small integer arrays); what changes is where the kernels
  * find an example's rows in the tensors, and that positions behind an example's end do not exist. */
-int mate_plan_packed(const int32_t *row_ids, const int32_t *col_ids, int B, const int32_t *cu_seqlens,
-                     const int32_t *prefix_len, const uint8_t *head_view, int H, int max_row_id, int max_col_id,
-                     void *stream, mate_plan_t **out) {
-    if (out) *out = nullptr;
+static int plan_packed(const int32_t *row_ids, const int32_t *col_ids, int B, const int32_t *cu_seqlens,
+                       const int32_t *prefix_len, const uint8_t *head_view, int H, int max_row_id, int max_col_id,
+                       void *stream, mate_plan_t **out) {
     if (!row_ids || !col_ids || !cu_seqlens || !prefix_len || !head_view || !out || B <= 0 || H <= 0)
         return MATE_ERR_INVALID_ARG;
     if (cu_seqlens[0] != 0) return MATE_ERR_INVALID_ARG;
@@ -590,6 +603,15 @@ int mate_plan_packed(const int32_t *row_ids, const int32_t *col_ids, int B, cons
     return MATE_OK;
 }
 
+int mate_plan_packed(const int32_t *row_ids, const int32_t *col_ids, int B, const int32_t *cu_seqlens,
+                     const int32_t *prefix_len, const uint8_t *head_view, int H, int max_row_id, int max_col_id,
+                     void *stream, mate_plan_t **out) {
+    if (out) *out = nullptr;
+    return no_throw([&]() {
+        return plan_packed(row_ids, col_ids, B, cu_seqlens, prefix_len, head_view, H, max_row_id, max_col_id, stream, out);
+    });
+}
+
 /* The head-independent pattern: three passes over plans the ordinary kernels can run (see mate.h).
  *   main plan  every head a row head: prefix rows against everything, table rows against the prefix
  *              and their own row (which holds their own cell)
@@ -597,9 +619,8 @@ int mate_plan_packed(const int32_t *row_ids, const int32_t *col_ids, int B, cons
  *              the cells of their column in front of their own cell
  *   sub[1]     the same behind their own cell
  * The three key sets of a row are disjoint and their union is the pattern. */
-int mate_plan_sat(const int32_t *row_ids, const int32_t *col_ids, int B, int N, int prefix_len, int H,
-                  int max_row_id, int max_col_id, void *stream, mate_plan_t **out) {
-    if (out) *out = nullptr;
+static int plan_sat(const int32_t *row_ids, const int32_t *col_ids, int B, int N, int prefix_len, int H,
+                    int max_row_id, int max_col_id, void *stream, mate_plan_t **out) {
     if (!out || B <= 0 || H <= 0 || max_row_id < 0 || max_col_id < 0) return MATE_ERR_INVALID_ARG;
     if ((long long)(max_row_id + 1) * (max_col_id + 1) > (1ll << 28)) return MATE_ERR_UNSUPPORTED;
     const std::vector<int32_t> prefix((size_t)B, prefix_len), zero((size_t)B, 0);
@@ -629,6 +650,63 @@ int mate_plan_sat(const int32_t *row_ids, const int32_t *col_ids, int B, int N, 
     return MATE_OK;
 }
 
+int mate_plan_sat(const int32_t *row_ids, const int32_t *col_ids, int B, int N, int prefix_len, int H,
+                  int max_row_id, int max_col_id, void *stream, mate_plan_t **out) {
+    if (out) *out = nullptr;
+    return no_throw([&]() { return plan_sat(row_ids, col_ids, B, N, prefix_len, H, max_row_id, max_col_id, stream, out); });
+}
+
+// Fills an empty plan from checked arguments; the caller owns the plan and the staging buffer whatever comes of it.
+static int fill_plan(mate_plan_t *pl, mate::Staging &host, const int32_t *row_ids, const int32_t *col_ids, int B, int N,
+                     const int32_t *prefix_len, const int32_t *global_len, const uint8_t *head_view, int H, int max_row_id,
+                     int max_col_id, int radius, int bounds_mode, int group, cudaStream_t st) {
+    pl->B = B;
+    pl->N = N;
+    pl->prefix.assign(prefix_len, prefix_len + B);
+    if (global_len) pl->global.assign(global_len, global_len + B);
+    else pl->global = pl->prefix;
+    pl->H = H;
+    pl->radius = radius;
+    pl->bounds_mode = bounds_mode;
+    pl->group = std::max(group, 1);
+    pl->head_view.assign(head_view, head_view + H);
+    pl->view[0].max_id = max_row_id;
+    pl->view[1].max_id = max_col_id;
+    for (int h = 0; h < H; ++h) pl->view[head_view[h]].n_heads++;
+
+    {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&pl->n_ctas, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return MATE_ERR_CUDA;
+        pl->device = dev;
+    }
+    pl->stream = mate::stream_id(st);
+    if (pl->stream == 0) pl->elsewhere = true;
+    const PlanLayout L = carve(pl, nullptr);
+    if (!mate::staging_take(std::max(L.in_bytes, L.out_bytes), pl->device, &host) ||
+        !mate::pool_take(L.total, st, pl->device, &pl->dev_block))
+        return MATE_ERR_NOMEM;
+    char *dev_base = (char *)pl->dev_block.ptr, *host_base = (char *)host.ptr;
+    carve(pl, dev_base);
+    const auto in_host = [&](const void *dev) { return host_base + ((const char *)dev - dev_base - L.in_off); };
+    memset(host_base, 0, L.in_bytes);
+    memcpy(in_host(pl->prefix_dev), pl->prefix.data(), B * sizeof(int32_t));
+    memcpy(in_host(pl->global_dev), pl->global.data(), B * sizeof(int32_t));
+    memcpy(in_host(pl->head_view_dev), pl->head_view.data(), H);
+    bool ok = cudaMemcpyAsync(dev_base + L.in_off, host_base, L.in_bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    ok = ok && mate::launch_plan_kernels(row_ids, col_ids, B, N, pl->prefix_dev, pl->global_dev, radius, bounds_mode, pl->group,
+                                         pl->view[0], pl->view[1], pl->n_valid_dev, pl->status_dev, st) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(host_base, dev_base + L.out_off, L.out_bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    ok = ok && cudaStreamSynchronize(st) == cudaSuccess;
+    if (!ok) return MATE_ERR_CUDA;
+    const auto out_host = [&](const void *dev) { return (const int32_t *)(host_base + ((const char *)dev - dev_base - L.out_off)); };
+    if (out_host(pl->status_dev)[0] != 0) return MATE_ERR_INVALID_ARG;
+    pl->n_valid.assign(out_host(pl->n_valid_dev), out_host(pl->n_valid_dev) + B);
+    const int32_t *seg_off_host[2] = {out_host(pl->view[0].seg_off), out_host(pl->view[1].seg_off)};
+    return build_units(pl, seg_off_host, st);
+}
+
 static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int N, const int32_t *prefix_len,
                       const int32_t *global_len, const uint8_t *head_view, int H, int max_row_id, int max_col_id,
                       int radius, int bounds_mode, int group, void *stream, mate_plan_t **out) {
@@ -647,63 +725,11 @@ static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int
     cudaStream_t st = (cudaStream_t)stream;
     mate_plan_t *pl = new (std::nothrow) mate_plan_t();
     if (!pl) return MATE_ERR_NOMEM;
-    pl->B = B;
-    pl->N = N;
-    pl->prefix.assign(prefix_len, prefix_len + B);
-    if (global_len) pl->global.assign(global_len, global_len + B);
-    else pl->global = pl->prefix;
-    pl->H = H;
-    pl->radius = radius;
-    pl->bounds_mode = bounds_mode;
-    pl->group = std::max(group, 1);
-    pl->head_view.assign(head_view, head_view + H);
-    pl->view[0].max_id = max_row_id;
-    pl->view[1].max_id = max_col_id;
-    for (int h = 0; h < H; ++h) pl->view[head_view[h]].n_heads++;
-
-    {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&pl->n_ctas, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-            delete pl;
-            return MATE_ERR_CUDA;
-        }
-        pl->device = dev;
-    }
-    pl->stream = mate::stream_id(st);
-    if (pl->stream == 0) pl->elsewhere = true;
-    const PlanLayout L = carve(pl, nullptr);
     mate::Staging host;
-    if (!mate::staging_take(std::max(L.in_bytes, L.out_bytes), pl->device, &host) ||
-        !mate::pool_take(L.total, st, pl->device, &pl->dev_block)) {
-        mate::staging_give(host, st);
-        mate_plan_destroy(pl);
-        return MATE_ERR_NOMEM;
-    }
-    char *dev_base = (char *)pl->dev_block.ptr, *host_base = (char *)host.ptr;
-    carve(pl, dev_base);
-    const auto in_host = [&](const void *dev) { return host_base + ((const char *)dev - dev_base - L.in_off); };
-    memset(host_base, 0, L.in_bytes);
-    memcpy(in_host(pl->prefix_dev), pl->prefix.data(), B * sizeof(int32_t));
-    memcpy(in_host(pl->global_dev), pl->global.data(), B * sizeof(int32_t));
-    memcpy(in_host(pl->head_view_dev), pl->head_view.data(), H);
-    bool ok = cudaMemcpyAsync(dev_base + L.in_off, host_base, L.in_bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    ok = ok && mate::launch_plan_kernels(row_ids, col_ids, B, N, pl->prefix_dev, pl->global_dev, radius, bounds_mode, pl->group,
-                                         pl->view[0], pl->view[1], pl->n_valid_dev, pl->status_dev, st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(host_base, dev_base + L.out_off, L.out_bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess;
-    ok = ok && cudaStreamSynchronize(st) == cudaSuccess;
-    int rc = ok ? MATE_OK : MATE_ERR_CUDA;
-    const auto out_host = [&](const void *dev) { return (const int32_t *)(host_base + ((const char *)dev - dev_base - L.out_off)); };
-    if (rc == MATE_OK && out_host(pl->status_dev)[0] != 0) rc = MATE_ERR_INVALID_ARG;
-    if (rc != MATE_OK) {
-        mate::staging_give(host, st);
-        mate_plan_destroy(pl);
-        return rc;
-    }
-    pl->n_valid.assign(out_host(pl->n_valid_dev), out_host(pl->n_valid_dev) + B);
-    const int32_t *seg_off_host[2] = {out_host(pl->view[0].seg_off), out_host(pl->view[1].seg_off)};
-
-    rc = build_units(pl, seg_off_host, st);
+    const int rc = no_throw([&]() {
+        return fill_plan(pl, host, row_ids, col_ids, B, N, prefix_len, global_len, head_view, H, max_row_id, max_col_id, radius,
+                         bounds_mode, group, st);
+    });
     mate::staging_give(host, st);
     if (rc != MATE_OK) {
         mate_plan_destroy(pl);

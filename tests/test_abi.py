@@ -2,6 +2,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -60,3 +62,27 @@ def test_binding_fails_loudly_without_the_library(monkeypatch):
     monkeypatch.setattr(api, "_LIB_PATH", os.path.join(ROOT, "no_such_dir", "libmate.so"))
     with pytest.raises(ImportError):
         api._load()
+
+
+def test_memory_that_is_not_to_be_had_is_a_status(lib):
+    # lists as long as the (absurd) inputs do not fit the process's address space: in the entry point, and in the plan
+    code = """
+import ctypes, mmap, resource, sys
+lib = ctypes.CDLL(sys.argv[1])
+held = int(open("/proc/self/statm").read().split()[0]) * mmap.PAGESIZE
+buf = (ctypes.c_ubyte * 64)()
+out = ctypes.c_void_p()
+arg = lambda x: ctypes.c_void_p(ctypes.addressof(x))
+B = 1 << 26
+zeros = mmap.mmap(-1, 4 * B, prot=mmap.PROT_READ | mmap.PROT_WRITE)
+prefix = (ctypes.c_ubyte * 1).from_buffer(zeros)
+resource.setrlimit(resource.RLIMIT_AS, (held + 4 * B + (128 << 20), resource.RLIM_INFINITY))
+big = 2 ** 31 - 1
+rc = [lib.mate_plan(arg(buf), arg(buf), big, 1, 0, arg(buf), 1, 1, 1, None, ctypes.byref(out)),
+      lib.mate_plan_sat(arg(buf), arg(buf), big, 1, 0, 1, 1, 1, None, ctypes.byref(out)),
+      lib.mate_plan_packed(arg(buf), arg(buf), B, arg(prefix), arg(prefix), arg(buf), 1, 1, 1, None, ctypes.byref(out)),
+      lib.mate_plan_varlen(arg(buf), arg(buf), B, 1, arg(prefix), arg(buf), 1, 1, 1, 0, None, ctypes.byref(out))]
+print(rc, out.value)
+"""
+    r = subprocess.run([sys.executable, "-c", code, lib._name], capture_output=True, text=True)
+    assert (r.returncode, r.stdout.strip()) == (0, "[-6, -6, -6, -6] None"), r.stderr

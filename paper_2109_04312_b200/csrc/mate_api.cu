@@ -780,9 +780,7 @@ int mate_plan_status(const mate_plan_t *plan, void *stream) {
         cudaStreamSynchronize(st) != cudaSuccess)
         return MATE_ERR_CUDA;
     if (s[1] != 0) {
-        if (getenv("MATE_LOG"))
-            fprintf(stderr, "[mate] a bounded wait expired: barrier slot %d, parity %d, warp %d\n", (s[2] >> 8) & 0xff,
-                    (s[2] >> 7) & 1, s[2] & 0x7f);
+        if (getenv("MATE_LOG")) fprintf(stderr, "[mate] a bounded wait expired\n");
         // a kernel that gave up may have left the arrival counters half way
         if (cudaMemsetAsync(plan->fwd_counters_dev, 0, sizeof(int32_t) * (mate::kSchedWords + 8 * (size_t)plan->n_fwd_slots), st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)

@@ -1,6 +1,7 @@
 """Sizes at which the kernels take another branch or a tile is partly filled: work units of the tensor-core
 kernels (global block in front of the own keys, halves filled up with table rows, units cut along their
-tiles), the tiled fp32 kernels, the cell mean's buffers, and plan memory reused between streams."""
+tiles), the tiled fp32 kernels, the cell mean's buffers, plan memory reused between streams; what must not
+reach a result: values at padding and of a packed neighbour, and the time of the kernel before."""
 import numpy as np
 import pytest
 import torch

@@ -513,13 +513,10 @@ FWD_TRACE_LABELS = {
                        "total"],
 }
 BWD_TRACE_LABELS = {
-    "arithmetic warp 0": ["wait S/dP", "wait previous gradient MMAs", "arithmetic", "epilogue", "tensor-memory loads", "total",
+    "arithmetic warp 0": ["wait S/dP", "wait previous gradient MMAs", "arithmetic", None, "tensor-memory loads", "total",
                           "signal operands", "tiles"],
-    "arithmetic warp 4": ["wait S/dP", "wait previous gradient MMAs", "arithmetic", "epilogue", "tensor-memory loads", None,
+    "arithmetic warp 4": ["wait S/dP", "wait previous gradient MMAs", "arithmetic", None, "tensor-memory loads", None,
                           "signal operands", "tiles"],
-    "MMA thread": ["wait row operands", "wait column tile", "wait operands from the warps", "issue gradient MMAs", "issue S/dP",
-                   "wait S/dP read", None, "tiles"],
-    "loader warp": ["wait for a free buffer", None, None, None, None, None, None, None],
 }
 
 

@@ -10,23 +10,37 @@
 //               -> P^T, dS^T -> dV += P^T dO, dK += dS^T Q
 // so no gradient is accumulated across CTAs and the result does not depend on the schedule.
 //
-// One persistent, warp-specialised CTA per SM (16 warps); work items (unit, side) are handed out through a
-// counter, longest first.
+// One persistent, warp-specialised CTA per SM (18 of 20 warps in use); work items (unit, side) are handed out through
+// a counter, longest first.
 //   warps 0-7   arithmetic: two threads (r, r + 128) share row r of the 128-row tile, the lane of
 //               tensor memory; each takes every other chunk of 32 columns.  S and dP (fp32) come out of
 //               tensor memory, P / dS (bf16 pairs) go back into it as MMA operands.
-//   warp  8     issues every tcgen05.mma (one elected lane): S and dP of tile n + 1 as soon as those of
-//               tile n sit in registers, ahead of the gradient MMAs of tile n
-//   warps 9-11  zero gradients of the padding rows
-//   warps 12-15 loaders: gather rows by view-order index with 16-byte cp.async into 128-byte swizzled
-//               shared memory, or fetch a column tile whose rows lie in place in the tensors by one bulk
-//               tensor copy per matrix (row operands double buffered, column tiles in a ring of 4)
-// What bounds it: the exponentials, 1024 clk per 128 x 128 tile and side (16 per clock and SM), as far as the
-// rest hides behind them.  A tile that counts in full is taken into registers whole (64 columns of S and of
-// dP per thread), which frees S and dP for the next tile's MMAs before the arithmetic begins; the
-// operand columns are waited for behind the first chunk's arithmetic.  Waits and rare paths are rolled (the
-// instruction cache holds about 32 KB).  The gradients accumulate in tensor memory and are scattered to the
-// rows' original positions in the epilogue, through a staging area so that stores cover whole sectors.
+//   warps 8-11  gradients of a finished item: tensor memory -> the rows' original positions, through a staging area so that
+//               a store covers whole rows; before the first item they zero the gradients of the padding rows
+//   warps 12,13 issue the tcgen05.mma (one elected lane each): S and dP of the tiles / the gradient MMAs, each as soon as
+//               what it needs is there
+//   warps 16-19 loaders, in two teams of two that take the loads (row operands, column tiles) in turn: rows by view-order
+//               index, four to a tensor copy (gather4), or a column tile whose rows lie in place in the tensors by one
+//               bulk tensor copy per matrix, into 128-byte swizzled shared memory (row operands double buffered,
+//               column tiles in a ring of 4)
+// What bounds it.  The exponentials take 1024 clk per 128 x 128 tile and side (16 per clock and SM); what is left is the
+// chain S complete -> registers -> arithmetic -> operands -> next S, about 2050 clk per tile when all pairs count, and on
+// tables the loads and the cost per item.  Hence:
+//   - A tile that counts in full is taken into registers whole (64 columns of S and of dP per thread), which frees S
+//     and dP for the next tile's MMAs before the arithmetic begins; the operand columns are waited for behind the
+//     first chunk's arithmetic.
+//   - The arithmetic warps have no part in an item's end: the store warps wait for its last gradient MMAs (700 clk
+//     behind the last operands) and take the gradients out of tensor memory under the next item's first tile.
+//   - A load costs a warp about 1700 clk of look-up, waiting and issuing (its instructions queue behind the exponentials),
+//     with a position's latency in it; two teams keep two loads under way.  The copies complete on the
+//     tile's barrier by themselves, so no warp waits for them to signal.
+//   - All roles share an instruction cache of about 32 KB: waits and rare paths are rolled, gathers are a loop of 15
+//     instructions.  (With the gathers and waits unrolled, 68 KB of code instead of 54, the same kernel takes 92 us for
+//     4 x 2048 tokens: a warp waits for instructions 3.9 times as long as it issues, instead of 0.7.)
+//   - The tensor maps are fetched ahead of the first copy (4 x 2048 tokens, forward and backward, 99.4 us without, 98.0 with).
+// With one warp for all MMAs, cp.async gathers by four warps and the epilogue in the arithmetic warps, forward and backward
+// back to back took 47.7 us for 8 x 512 tokens, 101.8 for 4 x 2048, 176.0 for 1 x 8192 and 172.9 for 2 x 4096; with this form
+// 46.4, 98.1, 165.6 and 162.7.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -47,51 +61,55 @@ namespace {
 using namespace ptx;
 
 constexpr int kComputeWarps = 8;
-constexpr int kMmaWarp = kComputeWarps;
-constexpr int kPadWarp0 = kMmaWarp + 1;
-constexpr int kPadWarps = 3;
-constexpr int kLoadWarp0 = kPadWarp0 + kPadWarps;
+constexpr int kStoreWarp0 = kComputeWarps;
+constexpr int kStoreWarps = 4;
+constexpr int kMmaWarp = kStoreWarp0 + kStoreWarps;
+constexpr int kMmaWarps = 2;  // one for S and dP, one for the gradients
+constexpr int kLoadWarp0 = kMmaWarp + 4;  // (two warps of the MMA warps' group of four have nothing to do)
 constexpr int kLoadWarps = 4;
+constexpr int kTeams = 2;                           // of loader warps, which take the steps in turn
+constexpr int kTeamWarps = kLoadWarps / kTeams;
+constexpr int kLoadRows = kTile / kTeamWarps;       // rows of a tile a loader warp fetches
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
-// registers per thread after the roles have split: 256 x 168 + 256 x 88 = 65,536 = the 512 x 128 the CTA is
-// launched with
-constexpr int kRegsCompute = 168, kRegsOther = 88;
+// registers per thread after the roles have split: 256 x 168 + 128 x 48 + 128 x 40 + 128 x 56 = 61,440 = the 640 x 96 the
+// CTA is launched with
+constexpr int kRegsCompute = 168, kRegsStore = 48, kRegsMma = 40, kRegsLoad = 56;
 constexpr int kStages = 4;  // ring of column tiles
-constexpr int kLag = 2;     // loader: copy groups in flight behind the newest one
 constexpr int kSchedDepth = 4;
 constexpr uint32_t kOffR = 0;                                    // [2 buffers] x (Ra: Q or K, Rb: dO or V), 16 KB each
 constexpr uint32_t kOffC = 4 * kTileBytes;                       // [kStages] x (Ca 16 KB, Cb 16 KB)
 constexpr uint32_t kOffVec = kOffC + kStages * 2 * kTileBytes;   // [kStages] x 128 x (-LSE log2 e), 128 x D
 constexpr uint32_t kOffMeta = kOffVec + kStages * 1024;          // [2 buffers] x (perm, seg_lo, seg_hi, -LSE log2 e, D) of 128 rows
-constexpr uint32_t kOffStage = kOffMeta + 2 * 5 * kTile * 4;     // [arithmetic warps] x 32 rows x 64 bytes
-constexpr uint32_t kOffItem = kOffStage + kComputeWarps * 2048;  // [kSchedDepth] unit records
+constexpr uint32_t kOffStage = kOffMeta + 2 * 5 * kTile * 4;     // [store warps] x 32 rows x 128 bytes
+constexpr uint32_t kOffItem = kOffStage + kStoreWarps * 4096;    // [kSchedDepth] unit records
 constexpr uint32_t kOffBar = kOffItem + kSchedDepth * sizeof(FwdUnit);
 constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024;            // + slack for the 1024-byte alignment
 static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 // barrier slots (8 bytes each) behind kOffBar
 enum {
-    kBarRFull = 0,    // [2] loaders -> MMA, arithmetic      (count: loader warps)
-    kBarREmpty = 2,   // [2] MMA commit and arithmetic warps (row data read) -> loaders (count 1 + kComputeWarps)
-    kBarCFull = 4,    // [kStages] loaders -> MMA            (count: loader warps)
+    kBarRFull = 0,    // [2] loaders -> MMA, arithmetic      (count: warps of a team)
+    kBarREmpty = 2,   // [2] MMA commit and arithmetic warps (row data read) -> loaders (count 1 + kComputeWarps + kStoreWarps)
+    kBarCFull = 4,    // [kStages] loaders -> MMA            (count: warps of a team)
     kBarCEmpty = 8,   // [kStages] MMA commit -> loaders     (count 1)
     kBarSFull = 12,   // MMA commit -> arithmetic: S and dP of a tile are complete (count 1)
     kBarAFull = 13,   // arithmetic -> MMA: the bf16 operands of a tile are written (count: one per warp)
     kBarGDone = 14,   // MMA commit -> arithmetic: the gradient MMAs of a tile are complete (count 1)
-    kBarFinal = 15,
     kBarSchedFull = 16,   // [kSchedDepth] scheduler -> every warp (count 1)
     kBarSchedEmpty = 20,  // [kSchedDepth] every warp -> scheduler (count kSchedReaders)
     kBarSTFree = 24,      // arithmetic -> MMA: S and dP of a tile are in registers (count: one per warp)
-    kNumBars = 25
+    kBarItemDone = 25,    // MMA commit -> store warps: every gradient MMA of an item is complete (count 1)
+    kBarAccFree = 26,     // store warps -> MMA: the gradients of an item are in registers (count: one per warp)
+    kBarFinal = 27,       // [2]
+    kNumBars = 29
 };
-constexpr int kSchedReaders = kComputeWarps + 1 + kLoadWarps;
+constexpr int kSchedReaders = kComputeWarps + kMmaWarps + kStoreWarps + kLoadWarps;
 // tensor memory columns
 constexpr uint32_t kTmS = 0, kTmT = 128, kTmA1 = 256, kTmA2 = 320, kTmAcc1 = 384, kTmAcc2 = 448;
 constexpr uint32_t kWaitLimit = 4096;  // tries (about 5 us each) before a wait gives up
 
 struct Params {
-    CUtensorMap tmQ, tmK, tmV, tmdO;  // boxes of 128 rows, 128-byte swizzle
-    int use_tma;                      // 0: every tile is gathered row by row
-    const __nv_bfloat16 *Q, *K, *V, *dO;
+    CUtensorMap tmQ, tmK, tmV, tmdO;      // boxes of 128 rows, 128-byte swizzle
+    CUtensorMap tmQ1, tmK1, tmV1, tmdO1;  // of one row, for the gathers
     const float *nlse, *D;  // per row, original order: -LSE log2 e, D
     __nv_bfloat16 *dQ, *dK, *dV;
     ViewPlan rowv, colv;
@@ -150,17 +168,17 @@ __global__ void __launch_bounds__(256) rowdot_kernel(const __nv_bfloat16 *__rest
 }
 
 // P and dS of 32 columns, as bf16 pairs (even column in the low half): p = exp2(s * scale2 + nlse), dS = p (dP - D).
-// kKeySide: nlse and D are per column (two arrays of shared memory), otherwise per row.  Columns whose bit of
+// kKeySide: nlse and D are per column (in shared memory at vec and 512 bytes behind), otherwise per row.  Columns whose bit of
 // `on` is clear do not count (kMask).  Two columns per instruction except for the exponential.
 template <bool kKeySide, bool kMask>
 __device__ __forceinline__ void math32(const uint32_t (&sv)[32], const uint32_t (&tv)[32], uint64_t scale2, uint64_t row_nlse2,
-                                       uint64_t row_D2, const float4 *vec_nlse, const float4 *vec_D, uint32_t on,
+                                       uint64_t row_D2, uint32_t vec, uint32_t on,
                                        uint32_t (&pk_p)[16], uint32_t (&pk_ds)[16]) {
 #pragma unroll
     for (int e = 0; e < 32; e += 4) {
         uint64_t nl[2] = {row_nlse2, row_nlse2}, Dv[2] = {row_D2, row_D2};
         if (kKeySide) {
-            const float4 a = vec_nlse[e >> 2], d4 = vec_D[e >> 2];
+            const float4 a = ld_shared_f4(vec + 4 * e), d4 = ld_shared_f4(vec + 512 + 4 * e);
             nl[0] = pack_f32x2(a.x, a.y);
             nl[1] = pack_f32x2(a.z, a.w);
             Dv[0] = pack_f32x2(d4.x, d4.y);
@@ -182,6 +200,29 @@ __device__ __forceinline__ void math32(const uint32_t (&sv)[32], const uint32_t 
         }
     }
 }
+// Tiles of an item: nA of range A, then those of range B (all of them kTile columns wide but for the last of either).
+struct ItemTiles {
+    int kA0, len_a, kB0, len_b, kP, nA, n;
+    __device__ __forceinline__ explicit ItemTiles(const FwdUnit &u) {
+        kA0 = u.kA0;
+        kB0 = u.kB0;
+        kP = u.kP();
+        len_a = max(u.kA_end - kA0, 0);
+        len_b = kP + u.kB_end - kB0;
+        nA = (len_a + kTile - 1) / kTile;
+        n = nA + (len_b + kTile - 1) / kTile;
+    }
+    __device__ __forceinline__ TileInfo tile(int i) const {  // = tile_info
+        TileInfo t;
+        t.is_b = i >= nA;
+        const int off = (t.is_b ? i - nA : i) * kTile;
+        t.w = min((t.is_b ? len_b : len_a) - off, kTile);
+        t.x0 = t.is_b ? off : kA0 + off;
+        t.k0 = t.is_b ? off + kB0 - kP : t.x0;
+        t.pre = t.is_b ? min(max(kP - off, 0), t.w) : t.w;
+        return t;
+    }
+};
 __device__ __forceinline__ uint32_t bits_below(int n) { return n <= 0 ? 0u : n >= 32 ? 0xffffffffu : (1u << n) - 1u; }
 
 __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_constant__ Params p) {
@@ -202,32 +243,35 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
     int4 rec = make_int4(0, 0, 0, 0);
     int it_next = blockIdx.x;  // lane 0
     auto claim = [&]() {
-        if (lane == 0) it_next = atomicAdd(p.counter, 1) + (int)gridDim.x;
+        if (lane == 0) it_next = atomicAdd(p.counter, 1);
     };
-    auto fetch_record = [&]() {
-        const int it = __shfl_sync(0xffffffffu, it_next, 0);
+    auto fetch_record = [&](bool claimed = true) {
+        const int it = __shfl_sync(0xffffffffu, it_next, 0) + (claimed ? (int)gridDim.x : 0);
         rec = make_int4(0, 0, 0, 0);  // rows = 0: the list is exhausted
         if (it < 2 * p.n_units && lane < 4) {
             rec = __ldg(reinterpret_cast<const int4 *>(p.units + (it >> 1)) + lane);
             if (lane == 3) rec.z = it & 1;
         }
     };
-    if (warp == kLoadWarp0) fetch_record();
+    if (warp == kLoadWarp0) fetch_record(false);
+    if (warp == kLoadWarp0 + 1 && lane < 8) prefetch_tmap(&p.tmQ + lane);  // all eight of them
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bars + 8 * (kBarRFull + i), kLoadWarps);
-            mbar_init(bars + 8 * (kBarREmpty + i), 1 + kComputeWarps);
+            mbar_init(bars + 8 * (kBarRFull + i), kTeamWarps);
+            mbar_init(bars + 8 * (kBarREmpty + i), 1 + kComputeWarps + kStoreWarps);
         }
         for (int i = 0; i < kStages; ++i) {
-            mbar_init(bars + 8 * (kBarCFull + i), kLoadWarps);
+            mbar_init(bars + 8 * (kBarCFull + i), kTeamWarps);
             mbar_init(bars + 8 * (kBarCEmpty + i), 1);
         }
         mbar_init(bars + 8 * kBarSFull, 1);
         mbar_init(bars + 8 * kBarAFull, kComputeWarps);
         mbar_init(bars + 8 * kBarSTFree, kComputeWarps);
         mbar_init(bars + 8 * kBarGDone, 1);
-        mbar_init(bars + 8 * kBarFinal, 1);
+        mbar_init(bars + 8 * kBarItemDone, 1);
+        mbar_init(bars + 8 * kBarAccFree, kStoreWarps);
+        for (int i = 0; i < kMmaWarps; ++i) mbar_init(bars + 8 * (kBarFinal + i), 1);
         for (int i = 0; i < kSchedDepth; ++i) {
             mbar_init(bars + 8 * (kBarSchedFull + i), 1);
             mbar_init(bars + 8 * (kBarSchedEmpty + i), kSchedReaders);
@@ -254,82 +298,64 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
 #endif
     // every wait is bounded; the first one to expire raises the abort flag, which ends all roles
     auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
-        if (mbar_test_wait(bar, parity)) return true;  // already complete: no trip through the suspending form
 #pragma unroll 1
         for (uint32_t it = 0; it < kWaitLimit; ++it) {
             if (mbar_try_wait(bar, parity)) return true;
             if (*s_abort) return false;
         }
-        *s_abort = 1;
-        atomicOr(p.status + 1, 1);
+        *s_abort = 1;  // (the status word is set when the CTA ends)
         return false;
     };
-    // n-th entry of the item list of this CTA; false = the list is exhausted
-    auto next_item = [&](uint32_t n, FwdUnit &u) -> bool {
-        const int slot = n % kSchedDepth;
-        if (!wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) return false;
-        const int4 *src = reinterpret_cast<const int4 *>(s_item + slot);
-        int4 *dst = reinterpret_cast<int4 *>(&u);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) dst[i] = src[i];
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
-        return u.rows != 0;
-    };
-
     if (warp < kComputeWarps) {
         // ------------------------------------------------------------------ arithmetic + epilogue
         reg_alloc<kRegsCompute>();
         const int r = tid & 127;   // row of the tile = lane of tensor memory
         const int cq = warp >> 2;  // takes the chunks cq and cq + 2 of a column tile
         const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        uint8_t *stage = sm + kOffStage + warp * 2048;
         const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
-        uint32_t ph_s = 0, ph_g = 0, c_cnt = 0, item_cnt = 0;
+        uint32_t c_cnt = 0;  // tiles so far
         bool alive = true;
-        FwdUnit un;
         wait_prior_grid();
+        auto gradients_done = [&]() {  // of every tile so far (at once when there is none)
+            alive = wait(bars + 8 * kBarGDone, (c_cnt - 1) & 1);
+            tc_fence_after();
+        };
 
 #pragma unroll 1
         for (uint32_t n = 0; alive; ++n) {
-            if (!next_item(n, un)) break;
+            const int slot = n % kSchedDepth, rb = n & 1;
+            if (!wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) break;
+            // The record and the row data stay in shared memory until the item's last tile: what is needed of them is
+            // read where it is needed (registers are what this role is short of).
+            const FwdUnit &un = s_item[slot];
+            if (un.rows == 0) break;
             const bool key_side = un.ws_off == 0;
-            const int nA = un.tiles_a(), n_tiles = nA + ((un.kP() + un.kB_end - un.kB0 + kTile - 1) / kTile), rows_h = un.rows_of(0);
-            const int rb = item_cnt & 1;
-            if (!(alive = wait(bars + 8 * (kBarRFull + rb), (item_cnt >> 1) & 1))) break;
-            ++item_cnt;
+            const ItemTiles tiles(un);
+            if (!(alive = wait(bars + 8 * (kBarRFull + rb), (n >> 1) & 1))) break;
             // this row's data (rows past the end shadow the last one)
-            const int32_t *meta = reinterpret_cast<const int32_t *>(sm + kOffMeta) + rb * 5 * kTile + min(r, rows_h - 1);
-            const int dst_row = r < rows_h ? meta[0] : -1, my_lo = meta[kTile], my_hi = meta[2 * kTile];
-            const float row_nlse = __int_as_float(meta[3 * kTile]), row_D = __int_as_float(meta[4 * kTile]);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bars + 8 * (kBarREmpty + rb));
-            const int w_lo_max = __reduce_max_sync(0xffffffffu, my_lo), w_hi_min = __reduce_min_sync(0xffffffffu, my_hi);
+            const uint32_t meta = base + kOffMeta + (rb * 5 * kTile + min(r, un.rows_of(0) - 1)) * 4;
+            const int w_lo_max = __reduce_max_sync(0xffffffffu, ld_shared_s32(meta + kTile * 4)),
+                      w_hi_min = __reduce_min_sync(0xffffffffu, ld_shared_s32(meta + 2 * kTile * 4));
 
             // the tile loop is compiled once per side
             auto tile_loop = [&](auto side) {
                 constexpr bool kKeySide = decltype(side)::value;
-                const uint64_t row_nlse2 = pack_f32x2(row_nlse, row_nlse), row_D2 = pack_f32x2(row_D, row_D);
+                uint64_t row_nlse2 = 0ull, row_D2 = 0ull;
+                if (!kKeySide) {
+                    const float nlse = __int_as_float(ld_shared_s32(meta + 3 * kTile * 4)), D = __int_as_float(ld_shared_s32(meta + 4 * kTile * 4));
+                    row_nlse2 = pack_f32x2(nlse, nlse);
+                    row_D2 = pack_f32x2(D, D);
+                }
+                TileInfo t = tiles.tile(0);
 #pragma unroll 1
-                for (int i = 0; i < n_tiles; ++i, ++c_cnt) {
-                    const TileInfo t = tile_info(un, i, nA);
+                for (int i = 0; i < tiles.n; ++i) {
                     const bool full = t.w == kTile && (t.pre == kTile || (w_lo_max - t.k0 <= t.pre && w_hi_min - t.k0 >= kTile));
-                    const float4 *vec = reinterpret_cast<const float4 *>(sm + kOffVec + (c_cnt % kStages) * 1024);
+                    const uint32_t vec = base + kOffVec + (c_cnt % kStages) * 1024;
                     TR_T0(t_ws);
-                    if (!(alive = wait(bars + 8 * kBarSFull, ph_s))) break;
-                    ph_s ^= 1;
+                    if (!(alive = wait(bars + 8 * kBarSFull, c_cnt & 1))) break;
                     tc_fence_after();
                     TR_ADD(0, t_ws);
                     TR_T0(t_cmp);
-                    // the operand columns are free once the gradient MMAs of the previous tile are done
-                    bool a_free = i == 0;
-                    auto wait_a = [&]() {
-                        if (a_free) return;
-                        alive = wait(bars + 8 * kBarGDone, ph_g);
-                        ph_g ^= 1;
-                        tc_fence_after();
-                        a_free = true;
-                    };
                     auto release_st = [&]() {  // S and dP may be overwritten
                         tc_fence_before();
                         if (lane == 0) mbar_arrive(bars + 8 * kBarSTFree);
@@ -349,22 +375,23 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                             reg_fence(tv[cc]);
                         }
                         release_st();
-#pragma unroll
-                        for (int cc = 0; cc < 2; ++cc) {
-                            const int cb = cq * 32 + cc * 64;
-                            math32<kKeySide, false>(sv[cc], tv[cc], scale2, row_nlse2, row_D2, vec + (cb >> 2), vec + 32 + (cb >> 2),
-                                                    0u, pk_p, pk_ds);
-                            if (cc == 0) wait_a();
-                            if (kKeySide) tmem_st16(tm + kTmA1 + (cb >> 1), pk_p);
-                            tmem_st16(tm + (kKeySide ? kTmA2 : kTmA1) + (cb >> 1), pk_ds);
-                        }
+                        TR_ADD(4, t_cmp);
+                        math32<kKeySide, false>(sv[0], tv[0], scale2, row_nlse2, row_D2, vec + cq * 128, 0u, pk_p, pk_ds);
+                        TR_T0(t_wa);
+                        gradients_done();  // of the tile before: the operand columns are free
+                        TR_ADD(1, t_wa);
+                        if (kKeySide) tmem_st16(tm + kTmA1 + cq * 16, pk_p);
+                        tmem_st16(tm + (kKeySide ? kTmA2 : kTmA1) + cq * 16, pk_ds);
+                        math32<kKeySide, false>(sv[1], tv[1], scale2, row_nlse2, row_D2, vec + 256 + cq * 128, 0u, pk_p, pk_ds);
+                        if (kKeySide) tmem_st16(tm + kTmA1 + cq * 16 + 32, pk_p);
+                        tmem_st16(tm + (kKeySide ? kTmA2 : kTmA1) + cq * 16 + 32, pk_ds);
                     } else {
                         // this row counts the columns [0, pre) and [r_lo, r_hi); some row of the warp counts columns only
                         // there and within [e_lo, e_hi)
-                        const int r_lo = t.is_b ? my_lo - t.k0 : 0, r_hi = t.is_b ? min(my_hi - t.k0, t.w) : 0;
+                        const int r_lo = t.is_b ? ld_shared_s32(meta + kTile * 4) - t.k0 : 0, r_hi = t.is_b ? min(ld_shared_s32(meta + 2 * kTile * 4) - t.k0, t.w) : 0;
                         const int e_lo = __reduce_min_sync(0xffffffffu, r_lo), e_hi = __reduce_max_sync(0xffffffffu, r_hi);
                         const int e_end = max(t.pre, e_hi > e_lo ? e_hi : 0);
-                        bool held = true;
+                        bool held = true, a_free = false;
 #pragma unroll 1
                         for (int cb = cq * 32; cb < t.w; cb += 64) {
                             if (cb >= t.pre && (cb + 32 <= e_lo || cb >= e_hi)) {  // no row of the warp has a pair here
@@ -381,174 +408,56 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                                     release_st();
                                     held = false;
                                 }
-                                math32<kKeySide, true>(sv, tv, scale2, row_nlse2, row_D2, vec + (cb >> 2), vec + 32 + (cb >> 2),
+                                math32<kKeySide, true>(sv, tv, scale2, row_nlse2, row_D2, vec + 4 * cb,
                                                        bits_below(t.pre - cb) | (bits_below(r_hi - cb) & ~bits_below(r_lo - cb)), pk_p, pk_ds);
                             }
-                            wait_a();
+                            if (!a_free) gradients_done();
+                            a_free = true;
                             if (kKeySide) tmem_st16(tm + kTmA1 + (cb >> 1), pk_p);
                             tmem_st16(tm + (kKeySide ? kTmA2 : kTmA1) + (cb >> 1), pk_ds);
                         }
                         if (held) release_st();
                         // Also when nothing was written: keeps this warp's arrival below out of the barrier phase of the
                         // previous tile, which a slower warp may not have reached yet.
-                        wait_a();
+                        if (!a_free) gradients_done();
                     }
                     if (!alive) break;
+                    ++c_cnt;
+                    TR_T0(t_st);
                     tc_wait_st();
                     tc_fence_before();
                     if (lane == 0) mbar_arrive(bars + 8 * kBarAFull);
+                    TR_ADD(6, t_st);
                     TR_ADD(2, t_cmp);
                     TR_INC(7);
+                    t = tiles.tile(i + 1);
                 }
             };
             if (key_side) tile_loop(std::true_type{});
             else tile_loop(std::false_type{});
             if (!alive) break;
-
-            // epilogue: wait for the last gradient MMAs, then scatter the rows to their original positions.  Key side:
-            // one column group of the arithmetic warps stores dV, the other dK; query side: 32 columns of dQ each.
-            TR_T0(t_ep);
-            if (n_tiles > 0) {
-                if (!(alive = wait(bars + 8 * kBarGDone, ph_g))) break;
-                ph_g ^= 1;
-                tc_fence_after();
-            }
-            __nv_bfloat16 *out = (key_side ? (cq ? p.dK : p.dV) : p.dQ + cq * 32) + p.tr.base(un.b, un.h) * 64;
-            const uint32_t acc = tm + (key_side ? (cq ? kTmAcc2 : kTmAcc1) : kTmAcc1 + cq * 32);
-            const float mul = key_side && cq == 0 ? 1.f : p.scale;
-#pragma unroll 1
-            for (int c2 = 0; c2 < (key_side ? 2 : 1); ++c2) {
-                uint32_t o[32];
-                if (n_tiles > 0) {
-                    tmem_ld32(acc + c2 * 32, o);
-                    tc_wait_ld();
-                    reg_fence(o);
-                } else {  // rows without any pair (possible in the passes of the row-or-column pattern)
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) o[e] = 0u;
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    uint32_t w4[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        w4[e] = cvt_bf16x2(__uint_as_float(o[8 * j + 2 * e]) * mul, __uint_as_float(o[8 * j + 2 * e + 1]) * mul);
-                    *reinterpret_cast<uint4 *>(stage + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-                }
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int row = 8 * i + (lane >> 2), j = lane & 3;
-                    const int dr = __shfl_sync(0xffffffffu, dst_row, row);
-                    const uint4 x = *reinterpret_cast<const uint4 *>(stage + row * 64 + ((j ^ ((row >> 1) & 3)) << 4));
-                    if (dr >= 0) *reinterpret_cast<uint4 *>(out + (size_t)dr * 64 + c2 * 32 + j * 8) = x;
-                }
-                __syncwarp();
-            }
-            tc_fence_before();  // the accumulators were read; the next item may overwrite them
-            TR_ADD(3, t_ep);
-        }
-    } else if (warp == kMmaWarp) {
-        // ------------------------------------------------------------------ MMA issuer
-        // The whole warp runs the control flow (operands stay warp-uniform), one lane issues.
-        reg_dealloc<kRegsOther>();
-        const bool leader = elect_one();
-        uint32_t c_cnt = 0, item_cnt = 0, ph_a = 0, ph_st = 0;
-        bool alive = true;
-        const uint32_t idesc_g = idesc_bf16(128, 64, 0, 1);  // B = 16 rows of the column tile x 64, MN-major
-        constexpr uint32_t kStep = (16 * kRowBytes) >> 4;    // 16 rows of the column tile
-        const uint32_t tA1 = tmem + kTmA1, tA2 = tmem + kTmA2, tG1 = tmem + kTmAcc1, tG2 = tmem + kTmAcc2;
-        FwdUnit un;
-        wait_prior_grid();
-#pragma unroll 1
-        for (uint32_t n = 0; alive; ++n) {
-            if (!next_item(n, un)) break;
-            const bool key_side = un.ws_off == 0;
-            const int nA = un.tiles_a(), n_tiles = nA + ((un.kP() + un.kB_end - un.kB0 + kTile - 1) / kTile);
-            const int rb = item_cnt & 1;
-            if (!(alive = wait(bars + 8 * (kBarRFull + rb), (item_cnt >> 1) & 1))) break;
-            tc_fence_after();
-            const uint32_t ra = smem_desc_lo(base + kOffR + rb * 2 * kTileBytes), rbb = ra + (kTileBytes >> 4);
-            int g_ks = 0;  // 16-column steps of the tile whose gradient MMAs are outstanding; one round more than tiles
-#pragma unroll 1
-            for (int i = 0; i <= n_tiles; ++i) {
-                int ks = 0;
-                uint32_t idesc = 0, ca = 0;
-                if (i < n_tiles) {  // the tile has landed
-                    const int st = c_cnt % kStages;
-                    const TileInfo t = tile_info(un, i, nA);
-                    ks = (t.w + 15) >> 4;
-                    idesc = idesc_bf16(128, ks * 16, 0, 0);
-                    ca = smem_desc_lo(base + kOffC + st * 2 * kTileBytes);
-                    if (!(alive = wait(bars + 8 * (kBarCFull + st), (c_cnt / kStages) & 1))) break;
-                }
-                if (i > 0) {  // S and dP are free again once the previous tile's values are in registers
-                    if (!(alive = wait(bars + 8 * kBarSTFree, ph_st))) break;
-                    ph_st ^= 1;
-                }
-                tc_fence_after();
-                if (i < n_tiles) {
-                    const uint32_t cb = ca + (kTileBytes >> 4);
-                    if (leader) {
-                        mma_ss_lean<0>(tmem + kTmS, ra, ca, idesc);  // S = Ra Ca^T, K = 64 as four steps of 16
-                        mma_ss_lean<1>(tmem + kTmS, ra + 2, ca + 2, idesc);
-                        mma_ss_lean<1>(tmem + kTmS, ra + 4, ca + 4, idesc);
-                        mma_ss_lean<1>(tmem + kTmS, ra + 6, ca + 6, idesc);
-                        mma_ss_lean<0>(tmem + kTmT, rbb, cb, idesc);  // dP = Rb Cb^T
-                        mma_ss_lean<1>(tmem + kTmT, rbb + 2, cb + 2, idesc);
-                        mma_ss_lean<1>(tmem + kTmT, rbb + 4, cb + 4, idesc);
-                        mma_ss_lean<1>(tmem + kTmT, rbb + 6, cb + 6, idesc);
-                        mma_commit(bars + 8 * kBarSFull);
-                    }
-                    __syncwarp();
-                    ++c_cnt;
-                }
-                if (i > 0) {  // gradient MMAs of the previous tile, behind this tile's S and dP
-                    if (!(alive = wait(bars + 8 * kBarAFull, ph_a))) break;
-                    ph_a ^= 1;
-                    tc_fence_after();
-                    const int g_st = (c_cnt - (i < n_tiles ? 2 : 1)) % kStages;
-                    const uint32_t a_lo = smem_desc_lo(base + kOffC + g_st * 2 * kTileBytes), b_lo = a_lo + (kTileBytes >> 4);
-                    if (leader) {
-                        if (key_side) {
-                            mma_ts_lean_flag(tG1, tA1, b_lo, idesc_g, i > 1);  // dV += P^T dO
-                            mma_ts_lean_flag(tG2, tA2, a_lo, idesc_g, i > 1);  // dK += dS^T Q
-#pragma unroll 1
-                            for (int k = 1; k < g_ks; ++k) {
-                                mma_ts_lean<1>(tG1, tA1 + 8 * k, b_lo + k * kStep, idesc_g);
-                                mma_ts_lean<1>(tG2, tA2 + 8 * k, a_lo + k * kStep, idesc_g);
-                            }
-                        } else {
-                            mma_ts_lean_flag(tG1, tA1, a_lo, idesc_g, i > 1);  // dQ += dS K
-#pragma unroll 1
-                            for (int k = 1; k < g_ks; ++k) mma_ts_lean<1>(tG1, tA1 + 8 * k, a_lo + k * kStep, idesc_g);
-                        }
-                        mma_commit(bars + 8 * kBarGDone);
-                        mma_commit(bars + 8 * (kBarCEmpty + g_st));
-                    }
-                    __syncwarp();
-                }
-                g_ks = ks;
-            }
-            if (!alive) break;
-            if (leader) mma_commit(bars + 8 * (kBarREmpty + rb));
             __syncwarp();
-            ++item_cnt;
+            if (lane == 0) {
+                mbar_arrive(bars + 8 * (kBarREmpty + rb));
+                mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
+            }
         }
-        // nothing of this CTA may still run on the tensor pipe when tensor memory is freed
-        if (leader) mma_commit(bars + 8 * kBarFinal);
-        __syncwarp();
-        mbar_wait_bounded(bars + 8 * kBarFinal, 0, kWaitLimit);
-    } else if (warp < kLoadWarp0) {
-        // ------------------------------------------------------------------ padding rows: zero gradients
-        reg_dealloc<kRegsOther>();
+    } else if (warp < kMmaWarp) {
+        // ------------------------------------------------------------------ gradients: tensor memory -> original positions
+        reg_dealloc<kRegsStore>();
+        const int q4 = warp - kStoreWarp0;  // rows 32 q4 .. of the tile = lanes of tensor memory this warp can read
+        static_assert(kStoreWarp0 % 4 == 0, "warp w reads the lanes 32 (w % 4) ..");
+        const uint32_t acc = tmem + ((uint32_t)(q4 * 32) << 16) + kTmAcc1;
+        uint8_t *stage = sm + kOffStage + q4 * 4096;
+        uint32_t units = 0;
         wait_prior_grid();
+        // padding rows: zero gradients
 #pragma unroll 1
         for (int c = blockIdx.x; c < p.n_pads; c += gridDim.x) {
             const PadChunk pc = p.pads[c];
             const ViewPlan &vp = p.head_view[pc.h] ? p.colv : p.rowv;
 #pragma unroll 2
-            for (int i = (warp - kPadWarp0) * 4 + (lane >> 3); i < pc.n; i += 4 * kPadWarps) {  // eight lanes per row
+            for (int i = q4 * 4 + (lane >> 3); i < pc.n; i += 4 * kStoreWarps) {  // eight lanes per row
                 const int orig = __ldg(vp.perm + (size_t)pc.b * p.N + pc.t0 + i);
                 if (p.tr.exists(pc.b, orig)) {
                     const size_t at = (p.tr.base(pc.b, pc.h) + orig) * 64 + (lane & 7) * 8;
@@ -558,144 +467,268 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                 }
             }
         }
+#pragma unroll 1
+        for (uint32_t n = 0;; ++n) {
+            const int slot = n % kSchedDepth, rb = n & 1;
+            if (!wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) break;
+            const FwdUnit &un = s_item[slot];
+            if (un.rows == 0) break;
+            const bool key_side = un.ws_off == 0, any = ItemTiles(un).n > 0;
+            const int rows_h = un.rows_of(0);
+            const size_t at = p.tr.base(un.b, un.h) * 64;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
+            if (!wait(bars + 8 * (kBarRFull + rb), (n >> 1) & 1)) break;
+            const int r = q4 * 32 + lane;
+            const int dst_row = r < rows_h ? (reinterpret_cast<const int32_t *>(sm + kOffMeta) + rb * 5 * kTile)[r] : -1;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bars + 8 * (kBarREmpty + rb));
+            if (any) {
+                if (!wait(bars + 8 * kBarItemDone, units++ & 1)) break;
+                tc_fence_after();
+            }
+            // key side: dV, dK; query side: dQ.  64 columns at a time through the staging area, so that a store writes
+            // whole rows of 128 bytes.
+#pragma unroll 1
+            for (int c = 0; c < (key_side ? 2 : 1); ++c) {
+                const float mul = key_side && c == 0 ? 1.f : p.scale;
+#pragma unroll 1
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t o[32];
+                    if (any) {
+                        tmem_ld32(acc + c * 64 + half * 32, o);
+                        tc_wait_ld();
+                        reg_fence(o);
+                    } else {  // rows without any pair (possible in the passes of the row-or-column pattern)
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) o[e] = 0u;
+                    }
+                    if (any && half == 1 && c == (key_side ? 1 : 0)) {  // read for the last time
+                        tc_fence_before();
+                        if (lane == 0) mbar_arrive(bars + 8 * kBarAccFree);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        uint32_t w4[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            w4[e] = cvt_bf16x2(__uint_as_float(o[8 * j + 2 * e]) * mul, __uint_as_float(o[8 * j + 2 * e + 1]) * mul);
+                        *reinterpret_cast<uint4 *>(stage + lane * 128 + (((half * 4 + j) ^ (lane & 7)) << 4)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+                    }
+                }
+                __syncwarp();
+                __nv_bfloat16 *out = (key_side ? (c ? p.dK : p.dV) : p.dQ) + at;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int row = 4 * i + (lane >> 3), j = lane & 7;
+                    const int dr = __shfl_sync(0xffffffffu, dst_row, row);
+                    const uint4 x = *reinterpret_cast<const uint4 *>(stage + row * 128 + ((j ^ (row & 7)) << 4));
+                    if (dr >= 0) *reinterpret_cast<uint4 *>(out + (size_t)dr * 64 + j * 8) = x;
+                }
+                __syncwarp();
+            }
+        }
+    } else if (warp < kLoadWarp0) {
+        // ------------------------------------------------------------------ MMA issuers
+        // One warp issues S and dP of the tiles, the other the gradient MMAs, each as soon as what it needs is there.  The
+        // whole warp runs the control flow and one lane issues; votes and shuffles keep conditions and operands
+        // warp-uniform (an MMA with other operands takes 51 clk to issue, more than a gradient MMA takes to run).
+        reg_dealloc<kRegsMma>();
+        if (warp < kMmaWarp + kMmaWarps) {
+            const bool leader = elect_one();
+            const bool grad = warp != kMmaWarp;
+            uint32_t c_cnt = 0, units = 0;  // tiles, items with a tile
+            wait_prior_grid();
+            auto wait_u = [&](uint32_t bar, uint32_t parity) -> bool {
+#pragma unroll 1
+                for (uint32_t it = 0; it < kWaitLimit; ++it) {
+                    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+                    if (__any_sync(0xffffffffu, *s_abort)) return false;
+                }
+                *s_abort = 1;
+                return false;
+            };
+            bool alive = true;
+#pragma unroll 1
+            for (uint32_t n = 0; alive; ++n) {
+                const int slot = n % kSchedDepth, rb = n & 1;
+                if (!wait_u(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) break;
+                const FwdUnit &un = s_item[slot];
+                auto uniform = [&](int x) { return __shfl_sync(0xffffffffu, x, 0); };
+                const int rows = uniform(un.rows), len_a = uniform(max(un.kA_end - un.kA0, 0)), len_b = uniform(un.kP() + un.kB_end - un.kB0);
+                const bool key_side = uniform(un.ws_off) == 0;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
+                if (rows == 0) break;
+                const int nA = (len_a + kTile - 1) / kTile, n_tiles = nA + (len_b + kTile - 1) / kTile;
+                auto steps = [&](int i) { return (min(i < nA ? len_a - i * kTile : len_b - (i - nA) * kTile, kTile) + 15) >> 4; };  // of 16 columns
+                if (!grad) {
+                    if (!(alive = wait_u(bars + 8 * (kBarRFull + rb), (n >> 1) & 1))) break;
+                    const uint32_t ra = smem_desc_lo(base + kOffR) + rb * ((2 * kTileBytes) >> 4), rbb = ra + (kTileBytes >> 4);
+#pragma unroll 1
+                    for (int i = 0; i < n_tiles; ++i, ++c_cnt) {
+                        const uint32_t st = c_cnt % kStages;
+                        const uint32_t idesc = idesc_bf16(128, 0, 0, 0) | (uint32_t)steps(i) << 18;  // N = 16 columns per step
+                        const uint32_t ca = smem_desc_lo(base + kOffC) + st * ((2 * kTileBytes) >> 4), cb = ca + (kTileBytes >> 4);
+                        const uint32_t tS = tmem + kTmS, tT = tmem + kTmT;
+                        if (!(alive = wait_u(bars + 8 * (kBarCFull + st), (c_cnt / kStages) & 1))) break;  // the tile has landed
+                        // the tile before sits in registers (parity 1 of a barrier without a phase behind it: at once)
+                        if (!(alive = wait_u(bars + 8 * kBarSTFree, (c_cnt - 1) & 1))) break;
+                        tc_fence_after();
+                        if (leader) {
+                            mma_ss_lean<0>(tS, ra, ca, idesc);  // S = Ra Ca^T, K = 64 as four steps of 16
+                            mma_ss_lean<1>(tS, ra + 2, ca + 2, idesc);
+                            mma_ss_lean<1>(tS, ra + 4, ca + 4, idesc);
+                            mma_ss_lean<1>(tS, ra + 6, ca + 6, idesc);
+                            mma_ss_lean<0>(tT, rbb, cb, idesc);  // dP = Rb Cb^T
+                            mma_ss_lean<1>(tT, rbb + 2, cb + 2, idesc);
+                            mma_ss_lean<1>(tT, rbb + 4, cb + 4, idesc);
+                            mma_ss_lean<1>(tT, rbb + 6, cb + 6, idesc);
+                            mma_commit(bars + 8 * kBarSFull);
+                        }
+                        __syncwarp();
+                    }
+                    if (!alive) break;
+                    if (leader) mma_commit(bars + 8 * (kBarREmpty + rb));  // the row operands are free once these MMAs are done
+                    __syncwarp();
+                } else {
+                    constexpr uint32_t idesc = idesc_bf16(128, 64, 0, 1);  // B = 16 rows of the column tile x 64, MN-major
+                    constexpr uint32_t kStep = (16 * kRowBytes) >> 4;      // 16 rows of the column tile
+                    // the accumulators are free once the gradients of the item before are in the store warps' registers
+                    if (n_tiles > 0 && !(alive = wait_u(bars + 8 * kBarAccFree, (units++ - 1) & 1))) break;
+                    const uint32_t tA1 = tmem + kTmA1, tA2 = tmem + kTmA2, tG1 = tmem + kTmAcc1, tG2 = tmem + kTmAcc2;
+#pragma unroll 1
+                    for (int i = 0; i < n_tiles; ++i, ++c_cnt) {
+                        const uint32_t st = c_cnt % kStages;
+                        const int ks = steps(i);
+                        const uint32_t a_lo = smem_desc_lo(base + kOffC) + st * ((2 * kTileBytes) >> 4), b_lo = a_lo + (kTileBytes >> 4);
+                        if (!(alive = wait_u(bars + 8 * kBarAFull, c_cnt & 1))) break;
+                        tc_fence_after();
+                        if (leader) {
+                            if (key_side) {
+                                mma_ts_lean_flag(tG1, tA1, b_lo, idesc, i > 0);  // dV += P^T dO
+                                mma_ts_lean_flag(tG2, tA2, a_lo, idesc, i > 0);  // dK += dS^T Q
+#pragma unroll 1
+                                for (int k = 1; k < ks; ++k) {
+                                    mma_ts_lean<1>(tG1, tA1 + 8 * k, b_lo + k * kStep, idesc);
+                                    mma_ts_lean<1>(tG2, tA2 + 8 * k, a_lo + k * kStep, idesc);
+                                }
+                            } else {
+                                mma_ts_lean_flag(tG1, tA1, a_lo, idesc, i > 0);  // dQ += dS K
+#pragma unroll 1
+                                for (int k = 1; k < ks; ++k) mma_ts_lean<1>(tG1, tA1 + 8 * k, a_lo + k * kStep, idesc);
+                            }
+                            mma_commit(bars + 8 * kBarGDone);
+                            mma_commit(bars + 8 * (kBarCEmpty + st));
+                            if (i + 1 == n_tiles) mma_commit(bars + 8 * kBarItemDone);
+                        }
+                        __syncwarp();
+                    }
+                }
+            }
+            // nothing of this CTA may still run on the tensor pipe when tensor memory is freed
+            if (leader) mma_commit(bars + 8 * (kBarFinal + grad));
+            __syncwarp();
+            mbar_wait_bounded(bars + 8 * (kBarFinal + grad), 0, kWaitLimit);
+        }
     } else {
         // ------------------------------------------------------------------ loaders
-        reg_dealloc<kRegsOther>();
+        reg_dealloc<kRegsLoad>();
         wait_prior_grid();
-        const int lw = warp - kLoadWarp0;
-        uint32_t c_cnt = 0, item_cnt = 0;
-        uint32_t pend[kLag];
-#pragma unroll
-        for (int i = 0; i < kLag; ++i) pend[i] = 0;
+        const int team = (warp - kLoadWarp0) / kTeamWarps, lw = (warp - kLoadWarp0) % kTeamWarps;
+        uint32_t step = 0;
+        const bool leader = elect_one();
+        uint32_t c_cnt = 0;
         bool alive = true;
-
-        // Commits the copies issued so far as one group and signals the barrier of the group that
-        // was committed kLag groups earlier (its copies have landed by then).
-        auto commit_and_signal = [&](uint32_t bar) {
-            cp_async_commit();
-            const uint32_t oldest = pend[0];
-#pragma unroll
-            for (int i = 0; i + 1 < kLag; ++i) pend[i] = pend[i + 1];
-            pend[kLag - 1] = bar;
-            if (oldest) {
-                cp_async_wait_group<kLag>();
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(oldest);
-            }
-        };
-        // Signals every group still pending, oldest first and each as soon as its own copies have
-        // landed (an older group is not held back by the latency of a newer one).  Called before
-        // this warp blocks on a buffer that is not free yet: the consumers may need exactly those
-        // groups to free it.
-        auto flush = [&]() {
-            static_assert(kLag == 2, "written out for two pending groups");
-            if (pend[0]) {
-                cp_async_wait_group<1>();
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(pend[0]);
-                pend[0] = 0;
-            }
-            if (pend[1]) {
-                cp_async_wait_group<0>();
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(pend[1]);
-                pend[1] = 0;
-            }
-        };
-        auto wait_free = [&](uint32_t bar, uint32_t parity) -> bool {
-            if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
-            flush();
-            TR_T0(t_wf);
-            const bool ok = wait(bar, parity);
-            TR_ADD(0, t_wf);
-            return ok;
-        };
-
-        FwdUnit un;
 #pragma unroll 1
         for (uint32_t n = 0; alive; ++n) {
-            const int slot = n % kSchedDepth;
+            const int slot = n % kSchedDepth, rb = n & 1;
             if (warp == kLoadWarp0) {
-                if (n >= (uint32_t)kSchedDepth && !wait_free(bars + 8 * (kBarSchedEmpty + slot), ((n / kSchedDepth) & 1) ^ 1)) break;
+                if (!wait(bars + 8 * (kBarSchedEmpty + slot), ((n / kSchedDepth) & 1) ^ 1)) break;
                 if (lane < 4) reinterpret_cast<int4 *>(s_item + slot)[lane] = rec;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedFull + slot));  // release: the record is visible to the readers
-            } else if (!wait_free(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) {
-                break;
             }
-            if (!next_item(n, un)) break;
+            if (!wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) break;
+            const FwdUnit un = s_item[slot];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
+            if (un.rows == 0) break;
             const bool key_side = un.ws_off == 0;
-            const int nA = un.tiles_a(), n_tiles = nA + ((un.kP() + un.kB_end - un.kB0 + kTile - 1) / kTile), rows_h = un.rows_of(0);
+            const ItemTiles tiles(un);
+            const int rows_h = un.rows_of(0);
             const ViewPlan &vp = p.head_view[un.h] ? p.colv : p.rowv;
             const size_t bn = (size_t)un.b * p.N;
             const int32_t *perm = vp.perm + bn;
             const size_t bh = p.tr.base(un.b, un.h);
-            const uint8_t *row_a = reinterpret_cast<const uint8_t *>((key_side ? p.K : p.Q) + bh * 64);
-            const uint8_t *col_a = reinterpret_cast<const uint8_t *>((key_side ? p.Q : p.K) + bh * 64);
-            const int64_t kv = reinterpret_cast<const uint8_t *>(p.V) - reinterpret_cast<const uint8_t *>(p.K),
-                          qdo = reinterpret_cast<const uint8_t *>(p.dO) - reinterpret_cast<const uint8_t *>(p.Q);
             // column tiles inside [0, ident) of the order are contiguous in the tensors (see bulk_tile)
-            const int ident = p.use_tma ? __ldg(vp.ident + un.b) : 0;
+            const int ident = __ldg(vp.ident + un.b);
+            const int r0 = kLoadRows * lw + lane;  // this lane's rows of a tile: r0, r0 + 32, .. (rows behind the last one repeat it)
 
             // step -1: the row operands and row data; steps 0 ..: the column tiles
-            auto step_idx = [&](int i) { return fetch_idx(perm, i < 0 ? row_tile(un.q0, rows_h) : tile_info(un, i, nA), lw, lane); };
-            int next = step_idx(-1);
+            constexpr int kPer = kLoadRows / 32;
+            const int first = (int)((step + team) & 1) - 1;  // of this team's steps
 #pragma unroll 1
-            for (int i = -1; i < n_tiles; ++i) {
-                const int now = next;
-                if (i + 1 < n_tiles) next = step_idx(i + 1);
-                else if (warp == kLoadWarp0) claim();  // the number and then the record travel under the copies
-                const TileInfo t = tile_info(un, max(i, 0), nA);
-                const int st = c_cnt % kStages, rb = item_cnt & 1;
-                const uint32_t bar_e = i < 0 ? kBarREmpty + rb : kBarCEmpty + st, bar_full = bars + 8 * (i < 0 ? kBarRFull + rb : kBarCFull + st);
-                if (!(alive = wait_free(bars + 8 * bar_e, ((i < 0 ? item_cnt >> 1 : c_cnt / kStages) & 1) ^ 1))) break;
-                const uint32_t dst = base + (i < 0 ? kOffR + rb * 2 * kTileBytes : kOffC + st * 2 * kTileBytes);
-                const bool bulk = i >= 0 && bulk_tile(t, ident);
-                if (bulk) {
-                    if (lw == 0 && lane == 0) {
-                        mbar_expect_tx(bar_full, 2 * kTileBytes);
-                        tma_load_2d(dst, key_side ? &p.tmQ : &p.tmK, 0, (int)bh + t.first(), bar_full);
-                        tma_load_2d(dst + kTileBytes, key_side ? &p.tmdO : &p.tmV, 0, (int)bh + t.first(), bar_full);
-                    }
-                    __syncwarp();
-                } else {
-                    const bool kv_pair = (i < 0) == key_side;
-                    gather_rows(dst, i < 0 ? row_a : col_a, true, kv_pair ? kv : qdo, now, i < 0 ? kTile : (t.w + 15) & ~15, lw, lane);
-                }
-                const int rr = 32 * lw + lane;
+            for (int i = -1; i < tiles.n; ++i) {
+                // the next item's number and then its record travel under the copies
+                if (warp == kLoadWarp0 && i == max(tiles.n - 2, -1)) claim();
+                if (warp == kLoadWarp0 && i + 1 == tiles.n) fetch_record();
+                if ((i ^ first) & 1) continue;
+                const TileInfo t = tiles.tile(max(i, 0));
+                int now[kPer];  // rows of the tensors
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) now[k] = (int)bh + __ldg(perm + (i < 0 ? un.q0 + min(r0 + 32 * k, rows_h - 1) : t.pos(min(r0 + 32 * k, t.w - 1))));
+                const uint32_t c = c_cnt + max(i, 0), st = c % kStages;
+                const uint32_t bar_e = bars + 8 * (i < 0 ? kBarREmpty + rb : kBarCEmpty + st), bar_full = bars + 8 * (i < 0 ? kBarRFull + rb : kBarCFull + st);
+                if (!(alive = wait(bar_e, ((i < 0 ? n >> 1 : c / kStages) & 1) ^ 1))) break;
                 if (i < 0) {  // row data for the arithmetic threads
-                    const uint32_t meta = base + kOffMeta + rb * 5 * kTile * 4 + rr * 4;
-                    if (rr < rows_h) {
-                        const size_t at = bn + un.q0 + rr;
-                        cp_async4(meta, vp.perm + at);
-                        cp_async4(meta + kTile * 4, vp.seg_lo + at);
-                        cp_async4(meta + 2 * kTile * 4, vp.seg_hi + at);
-                        if (!key_side) {
-                            cp_async4(meta + 3 * kTile * 4, p.nlse + bh + now);
-                            cp_async4(meta + 4 * kTile * 4, p.D + bh + now);
+#pragma unroll
+                    for (int k = 0; k < kPer; ++k) {
+                        const int rr = r0 + 32 * k;
+                        const uint32_t meta = base + kOffMeta + rb * 5 * kTile * 4 + rr * 4;
+                        if (rr < rows_h) {
+                            const size_t at = bn + un.q0 + rr;
+                            cp_async4(meta, vp.perm + at);
+                            cp_async4(meta + kTile * 4, vp.seg_lo + at);
+                            cp_async4(meta + 2 * kTile * 4, vp.seg_hi + at);
+                            if (!key_side) {
+                                cp_async4(meta + 3 * kTile * 4, p.nlse + now[k]);
+                                cp_async4(meta + 4 * kTile * 4, p.D + now[k]);
+                            }
                         }
                     }
+                    cp_async_arrive(bar_full);
                 } else if (key_side) {  // column data
-                    const uint32_t vec = base + kOffVec + st * 1024 + rr * 4;
-                    cp_async4(vec, p.nlse + bh + now);
-                    cp_async4(vec + 512, p.D + bh + now);
+#pragma unroll
+                    for (int k = 0; k < kPer; ++k) {
+                        const uint32_t vec = base + kOffVec + st * 1024 + (r0 + 32 * k) * 4;
+                        cp_async4(vec, p.nlse + now[k]);
+                        cp_async4(vec + 512, p.D + now[k]);
+                    }
+                    cp_async_arrive(bar_full);
                 }
-                if (!bulk || key_side) commit_and_signal(bar_full);
-                else if (lane == 0) mbar_arrive(bar_full);
-                if (i + 1 == n_tiles && warp == kLoadWarp0) fetch_record();
-                if (i < 0) {
-                    ++item_cnt;
+                __syncwarp();
+                const uint32_t dst = base + (i < 0 ? kOffR + rb * 2 * kTileBytes : kOffC + st * 2 * kTileBytes);
+                const bool kv = (i < 0) == key_side;  // K and V, or Q and dO
+                if (i >= 0 && bulk_tile(t, ident)) {
+                    if (leader) {
+                        mbar_arrive_expect_tx(bar_full, lw == 0 ? 2 * kTileBytes : 0);
+                        if (lw == 0) {
+                            tma_load_2d(dst, kv ? &p.tmK : &p.tmQ, 0, (int)bh + t.first(), bar_full);
+                            tma_load_2d(dst + kTileBytes, kv ? &p.tmV : &p.tmdO, 0, (int)bh + t.first(), bar_full);
+                        }
+                    }
                 } else {
-                    // the very first tile of the CTA is signalled as soon as it has landed
-                    if (c_cnt == 0) flush();
-                    ++c_cnt;
+                    // (the row operands' rows past the last one are never looked at: their results are not stored)
+                    const int n_rows = min(max((i < 0 ? rows_h : (t.w + 15) & ~15) - kLoadRows * lw, 0), kLoadRows);
+                    if (leader) mbar_arrive_expect_tx(bar_full, 2 * gather_bytes(n_rows));
+                    gather_rows4(dst, kv ? &p.tmK1 : &p.tmQ1, kv ? &p.tmV1 : &p.tmdO1, now, r0 - lane, n_rows, leader, bar_full);
                 }
+                __syncwarp();
             }
+            c_cnt += tiles.n;
+            step += 1 + tiles.n;
         }
-        flush();  // drain: signal the groups still pending
     }
 
 #ifdef MATE_TRACE
@@ -706,8 +739,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         if (role == 0) o[5] = clock64() - tr_start;
     }
 #endif
+    if (*s_abort)  // copies may still be on their way to shared memory: they take a few microseconds
+        for (int i = 0; i < 50; ++i) __nanosleep(1000);
     tc_fence_before();
     __syncthreads();
+    if (tid == 0 && *s_abort) atomicOr(p.status + 1, 1);
     if (warp == kMmaWarp) tmem_dealloc(tmem, 512);
 }
 
@@ -733,12 +769,13 @@ int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     float *D = (float *)(ws + 256);
     float *nlse = D + align256((size_t)plan->B * plan->H * plan->N * sizeof(float)) / sizeof(float);
     Params p;
-    p.use_tma = rows < (size_t(1) << 31) && make_row_map(&p.tmQ, Q, rows) && make_row_map(&p.tmK, K, rows) &&
-                make_row_map(&p.tmV, V, rows) && make_row_map(&p.tmdO, dO, rows);
-    p.Q = (const __nv_bfloat16 *)Q;
-    p.K = (const __nv_bfloat16 *)K;
-    p.V = (const __nv_bfloat16 *)V;
-    p.dO = (const __nv_bfloat16 *)dO;
+    struct {
+        CUtensorMap *box, *row;
+        const void *x;
+    } maps[] = {{&p.tmQ, &p.tmQ1, Q}, {&p.tmK, &p.tmK1, K}, {&p.tmV, &p.tmV1, V}, {&p.tmdO, &p.tmdO1, dO}};
+    if (rows >= (size_t(1) << 31)) return MATE_ERR_UNSUPPORTED;
+    for (const auto &m : maps)
+        if (!make_row_map(m.box, m.x, rows) || !make_row_map(m.row, m.x, rows, 1)) return MATE_ERR_CUDA;
     p.nlse = nlse;
     p.D = D;
     p.dQ = (__nv_bfloat16 *)dQ;
@@ -759,7 +796,7 @@ int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.status = plan->status_dev;
     p.counter = (int32_t *)ws + 8 * pass;
 
-    if (pass == 0 && launch_after(rowdot_kernel, dim3((unsigned)((rows + kRowdotRows - 1) / kRowdotRows)), 256, 0, stream, p.dO,
+    if (pass == 0 && launch_after(rowdot_kernel, dim3((unsigned)((rows + kRowdotRows - 1) / kRowdotRows)), 256, 0, stream, (const __nv_bfloat16 *)dO,
                                   (const __nv_bfloat16 *)O, LSE, D, nlse, rows, (int32_t *)ws) != cudaSuccess)
         return MATE_ERR_CUDA;
     return launch_after(tc_bwd_kernel, dim3((unsigned)plan->bwd_grid), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;

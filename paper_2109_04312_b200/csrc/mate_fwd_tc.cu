@@ -945,14 +945,14 @@ EncodeTiledFn encode_tiled_fn() {
 
 }  // namespace
 
-// Map over a [rows, 64] bf16 matrix (row = 128 bytes): boxes of 128 rows, written to shared memory in
+// Map over a [rows, 64] bf16 matrix (row = 128 bytes): boxes of box_rows rows, written to shared memory in
 // the 128-byte swizzle the tensor-core descriptors expect (16-byte chunk index XOR row & 7).
-bool make_row_map(CUtensorMap *map, const void *base, size_t rows) {
+bool make_row_map(CUtensorMap *map, const void *base, size_t rows, int box_rows) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {64, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {kRowBytes};
-    const cuuint32_t box[2] = {64, (cuuint32_t)kTile};
+    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     const cuuint32_t elem[2] = {1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, elem,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,

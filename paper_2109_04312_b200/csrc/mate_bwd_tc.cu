@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                     // (the row operands' rows past the last one are never looked at: their results are not stored)
                     const int n_rows = min(max((i < 0 ? rows_h : (t.w + 15) & ~15) - kLoadRows * lw, 0), kLoadRows);
                     if (leader) mbar_arrive_expect_tx(bar_full, 2 * gather_bytes(n_rows));
-                    gather_rows4(dst, kv ? &p.tmK1 : &p.tmQ1, kv ? &p.tmV1 : &p.tmdO1, now, r0 - lane, n_rows, leader, bar_full);
+                    gather_rows4<2>(dst, kv ? &p.tmK1 : &p.tmQ1, kv ? &p.tmV1 : &p.tmdO1, now, r0 - lane, n_rows, leader, bar_full);
                 }
                 __syncwarp();
             }

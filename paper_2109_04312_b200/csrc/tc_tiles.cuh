@@ -60,10 +60,11 @@ __device__ __forceinline__ void gather_rows(uint32_t s_a, const uint8_t *a_bh, b
 // behind it, 128-byte swizzle, four rows per copy.  idx: the tensors' rows for tile rows r0 + lane and r0 + 32 + lane.  The
 // whole warp takes part, its leader issues; the copies count on `bar` (gather_bytes per tensor).
 __device__ __forceinline__ uint32_t gather_bytes(int n_rows) { return (uint32_t)((n_rows + 3) >> 2) * 4 * kRowBytes; }
+template <int kUnroll>
 __device__ __forceinline__ void gather_rows4(uint32_t s_a, const CUtensorMap *map_a, const CUtensorMap *map_b, const int (&idx)[2], int r0,
                                              int n_rows, bool leader, uint32_t bar) {
     s_a += r0 * kRowBytes;
-#pragma unroll 1
+#pragma unroll kUnroll
     for (int g = 0; 4 * g < n_rows; ++g, s_a += 4 * kRowBytes) {
         const int v = g < 8 ? idx[0] : idx[1], l = 4 * (g & 7);
         const int y0 = __shfl_sync(0xffffffffu, v, l), y1 = __shfl_sync(0xffffffffu, v, l + 1), y2 = __shfl_sync(0xffffffffu, v, l + 2),

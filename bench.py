@@ -509,8 +509,7 @@ FWD_TRACE_LABELS = {
     "softmax warp 4 (half 1)": ["wait S", "wait previous P V", None, "tile: S seen to P handed over", "tiles", "unit set-up",
                                "epilogue", "total"],
     "MMA thread of half 0": ["wait Q", "wait P", "issue Q K^T", "issue P V", "tiles", "wait K/V tile", "wait S free", "total"],
-    "loader warp 10": ["wait for a free buffer", "flush pending copies", "issue copies", "commit and signal", "tiles", None, None,
-                       "total"],
+    "loader warp 12": [None, None, "issue copies", None, "loads", None, None, "total"],
 }
 BWD_TRACE_LABELS = {
     "arithmetic warp 0": ["wait S/dP", "wait previous gradient MMAs", "arithmetic", None, "tensor-memory loads", "total",

@@ -7,9 +7,12 @@
 //   warps 4-7   softmax of half 1 (rows 128..255)
 //   warps 8, 9  issue the tcgen05.mma of half 0 / half 1 (one elected lane each)
 //   warps 10,11 padding rows
-//   warps 12-15 loaders: gather Q, K, V rows by view-order index into 128-byte swizzled shared
-//               memory with 16-byte cp.async (the gather of Section 3.1 fused into the loads); K/V
-//               tiles whose rows lie in place in the tensors come in by one bulk tensor copy each
+//   warps 12-15 loaders, in two teams of two that take the loads (Q, key tiles) in turn: rows by view-order index
+//               (the gather of Section 3.1 fused into the loads), four to a tensor copy (gather4), into 128-byte swizzled
+//               shared memory; K/V tiles whose rows lie in place in the tensors come in by one bulk tensor copy each.
+//               The copies complete on the tile's barrier by themselves.  (Four warps with 16-byte cp.async copies of every
+//               tile, in line with waits for them to signal: 80 KB of code instead of 69, and forward and backward together
+//               44.7 us for 8 x 512 tokens, 96.0 for 4 x 2048, 161.8 for 2 x 4096; with this form 43.7, 94.0, 158.6.)
 //
 // Per key tile and half:   S = Q K^T  (tcgen05.mma, M = 128, N <= 128, K = 64, accumulator in TMEM)
 //                          P = exp2(S c - m), row sum
@@ -61,11 +64,12 @@ constexpr int kMmaWarps = 2;
 constexpr int kPadWarp0 = kMmaWarp + kMmaWarps;
 constexpr int kPadWarps = 2;
 constexpr int kLoadWarp0 = kPadWarp0 + kPadWarps;
-constexpr int kLoadWarps = 4;                // (two keep the softmax warps waiting on gathered tiles)
-constexpr int kLoadThreads = 32 * kLoadWarps;
+constexpr int kLoadWarps = 4;
+constexpr int kTeams = 2;                    // of loader warps, which take the steps in turn
+constexpr int kTeamWarps = kLoadWarps / kTeams;
+constexpr int kLoadRows = kTile / kTeamWarps;  // rows of a tile a loader warp fetches
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
 constexpr int kStages = 4;                   // K/V ring
-constexpr int kLag = 2;                      // loader: copy groups in flight behind the newest one
 // registers per thread after the roles have split: 256 x 176 + 256 x 80 = 65,536 = the 512 x 128 the CTA is
 // launched with
 constexpr int kRegsSoftmax = 176, kRegsOther = 80;
@@ -89,9 +93,9 @@ constexpr float kSumMin = 0x1p-100f, kSumMax = 0x1p60f;      // row sums outside
 
 // barrier slots (8 bytes each) behind kOffBar
 enum {
-    kBarQFull = 0,        // [2] loaders -> MMA, softmax   (count: loader warps)
+    kBarQFull = 0,        // [2] loaders -> MMA, softmax   (count: warps of a team)
     kBarQEmpty = 2,       // [2] MMA commits and softmax warps (row data read) -> loaders (count kMmaWarps + kSoftmaxWarps)
-    kBarKVFull = 4,       // [kStages] loaders -> MMA      (count: loader warps)
+    kBarKVFull = 4,       // [kStages] loaders -> MMA      (count: warps of a team)
     kBarKVEmpty = 8,      // [kStages] MMA -> loaders      (count 2: one per half)
     kBarSFull = 12,       // [2] MMA commit -> softmax (count 1)
     kBarSFree = 14,       // [2] softmax -> MMA: S of a tile has been read (count 4: one per warp)
@@ -106,11 +110,11 @@ constexpr int kSchedReaders = kSoftmaxWarps + kMmaWarps + kLoadWarps;
 static_assert(kStages == 4, "barrier slots");
 
 struct Params {
-    // 2-D tensor maps over K and V seen as [B H N rows, 64 columns]: boxes of 128 rows, 128-byte swizzle
-    CUtensorMap tmK, tmV;
-    int use_tma;     // 0: every tile is gathered row by row
+    // 2-D tensor maps over the tensors seen as [B H N rows, 64 columns], 128-byte swizzle: boxes of 128 rows, and of one row
+    // for the gathers
+    CUtensorMap tmK, tmV, tmQ1, tmK1, tmV1;
+    int bulk;        // 0: every tile is gathered row by row
     int view_order;  // 1: Q, K, V, O and LSE are laid out in each head's own order (no gather, no scatter)
-    const __nv_bfloat16 *Q, *K, *V;
     __nv_bfloat16 *O;
     float *LSE;
     ViewPlan rowv, colv;
@@ -203,11 +207,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         rec = make_int4(0, 0, 0, 0);  // rows = 0: the list is exhausted
         if (u < p.n_units && lane < 4) rec = __ldg(reinterpret_cast<const int4 *>(p.units + u) + lane);
     };
+    if (warp == kLoadWarp0 + 1 && lane < 5) prefetch_tmap(&p.tmK + lane);  // all five of them
     if (warp == kLoadWarp0) fetch_record(false);  // requested before the set-up below, which takes as long
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bars + 8 * (kBarQFull + i), kLoadWarps);
+            mbar_init(bars + 8 * (kBarQFull + i), kTeamWarps);
             mbar_init(bars + 8 * (kBarQEmpty + i), kMmaWarps + kSoftmaxWarps);
             mbar_init(bars + 8 * (kBarSFull + i), 1);
             mbar_init(bars + 8 * (kBarSFree + i), kSoftmaxWarps / 2);
@@ -216,7 +221,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             mbar_init(bars + 8 * (kBarFinal + i), 1);
         }
         for (int i = 0; i < kStages; ++i) {
-            mbar_init(bars + 8 * (kBarKVFull + i), kLoadWarps);
+            mbar_init(bars + 8 * (kBarKVFull + i), kTeamWarps);
             mbar_init(bars + 8 * (kBarKVEmpty + i), 2);
         }
         for (int i = 0; i < kSchedDepth; ++i) {
@@ -242,14 +247,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
 
     // every wait is bounded; the first one to expire raises the abort flag, which ends all roles
     auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
-        if (mbar_test_wait(bar, parity)) return true;  // already complete: no trip through the suspending form
 #pragma unroll 1
         for (uint32_t it = 0; it < kWaitLimit; ++it) {
             if (mbar_try_wait(bar, parity)) return true;
             if (*s_abort) return false;
         }
-        *s_abort = 1;
-        atomicOr(p.status + 1, 1);
+        *s_abort = 1;  // (the status word is set when the CTA ends)
         return false;
     };
 
@@ -485,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 write = ((un.tB >> 16) >> warp) & 1;  // the others were right the first time
             } else if (n_visit > 0) {
                 const bool has_keys = n_pre > 0 || min(meta[2 * kUnitRows], k_hi) > max(meta[kUnitRows], k_lo);
-                if (__any_sync(0xffffffffu, !(l < kSumMax) || (l < kSumMin && has_keys))) {
+                if (__any_sync(0xffffffffu, r < rows_h && (!(l < kSumMax) || (l < kSumMin && has_keys)))) {
                     write = false;
                     if (lane == 0) atomicOr((uint32_t *)s_bad + slot, 1u << warp);
                 }
@@ -738,60 +741,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         // ------------------------------------------------------------------ loaders
         reg_dealloc<kRegsOther>();
         wait_prior_grid();
-        const int ltid = tid - 32 * kLoadWarp0, lw = warp - kLoadWarp0;
-        uint32_t kv_cnt = 0, unit_cnt = 0;
-        uint32_t pend[kLag];
-#pragma unroll
-        for (int i = 0; i < kLag; ++i) pend[i] = 0;
+        const int team = (warp - kLoadWarp0) / kTeamWarps, lw = (warp - kLoadWarp0) % kTeamWarps;
+        const bool leader = elect_one();
+        uint32_t kv_cnt = 0, unit_cnt = 0, step = 0;
         bool alive = true;
-
-        // Commits the copies issued so far as one group and signals the barrier of the group that
-        // was committed kLag groups earlier (its copies have landed by then).
-        auto commit_and_signal = [&](uint32_t bar) {
-            cp_async_commit();
-            const uint32_t oldest = pend[0];
-#pragma unroll
-            for (int i = 0; i + 1 < kLag; ++i) pend[i] = pend[i + 1];
-            pend[kLag - 1] = bar;
-            if (oldest) {
-                cp_async_wait_group<kLag>();
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(oldest);
-            }
-        };
-        // Signals every group still pending, oldest first and each as soon as its own copies have
-        // landed (an older group is not held back by the latency of a newer one).  Called before
-        // this warp blocks on a buffer that is not free yet: the consumers may need exactly those
-        // groups to free it.
-        auto flush = [&]() {
-            static_assert(kLag == 2, "written out for two pending groups");
-            if (pend[0]) {
-                cp_async_wait_group<1>();
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(pend[0]);
-                pend[0] = 0;
-            }
-            if (pend[1]) {
-                cp_async_wait_group<0>();
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(pend[1]);
-                pend[1] = 0;
-            }
-        };
-        auto wait_free = [&](uint32_t bar, uint32_t parity) -> bool {
-            if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
-            TR_T0(t_fl);
-            flush();
-            TR_ADD(1, t_fl);
-            TR_T0(t_wf);
-            const bool ok = wait(bar, parity);
-            TR_ADD(0, t_wf);
-            return ok;
-        };
-
         FwdUnit un;
         uint32_t checked = 0;  // entries of the list that are known to be done
         int4 held_back = make_int4(0, 0, 0, 0);
@@ -808,7 +761,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 bool again = false;
                 for (; checked < done_to && !again; ++checked) {
                     const int sc = checked % kSchedDepth;
-                    if (!(alive = wait_free(bars + 8 * (kBarSchedEmpty + sc), (checked / kSchedDepth) & 1))) break;
+                    if (!(alive = wait(bars + 8 * (kBarSchedEmpty + sc), (checked / kSchedDepth) & 1))) break;
                     const uint32_t bad = s_bad[sc];
                     if (bad) {
                         again = true;
@@ -824,8 +777,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedFull + slot));  // release: the record is visible to the readers
                 redo = again;
-            } else if (!wait_free(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) {
-                break;
             }
             if (!next_unit(n, un)) break;
             un.tB &= 0xff;
@@ -834,81 +785,88 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             const size_t bn = (size_t)un.b * p.N;
             const int32_t *perm = p.view_order ? nullptr : vp.perm + bn;
             const size_t bh = p.tr.base(un.b, un.h);
-            const uint8_t *Qbh = reinterpret_cast<const uint8_t *>(p.Q + bh * 64), *Kbh = reinterpret_cast<const uint8_t *>(p.K + bh * 64);
-            const int64_t v_off = reinterpret_cast<const uint8_t *>(p.V) - reinterpret_cast<const uint8_t *>(p.K);
             // Rows of the order that sit in place in the tensors ([0, ident)): a K/V tile inside that range
             // (see bulk_tile) is one contiguous [128, 64] box and comes in by one bulk tensor copy per matrix
-            // (issued by one thread, completing on the tile's barrier by byte count) instead of up to 2 x 1024
-            // gathered 16-byte copies.  That is the prefix block's full tiles in every unit and, for a
+            // instead of 2 x 32 gathers of four rows.  That is the prefix block's full tiles in every unit and, for a
             // row-major table, those of the row view.
-            const int ident = !p.use_tma ? 0 : p.view_order ? p.N : __ldg(vp.ident + un.b);
-
-            const int qb = unit_cnt & 1;
-            // steps -2, -1: the two Q halves (and the row data of the unit); steps 0 ..: the key tiles
-            auto step_idx = [&](int i) {
-                const TileInfo t = i < 0 ? row_tile(un.row0_of(i + 2), un.rows_of(i + 2)) : tile_info(un, i, nA);
-                return t.w > 0 ? fetch_idx(perm, t, lw, lane) : 0;
+            const int ident = !p.bulk ? 0 : p.view_order ? p.N : __ldg(vp.ident + un.b);
+            const int qb = unit_cnt & 1, r0 = kLoadRows * lw;
+            // This lane's rows r0 + lane and r0 + 32 + lane of a tile, as rows of the tensors (rows behind the last one repeat it).
+            int idx[2];
+            static_assert(kLoadRows == 64, "rows per lane");
+            auto look_up = [&](const TileInfo &t) {
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const int at = t.pos(min(r0 + 32 * k + lane, t.w - 1));
+                    idx[k] = (int)bh + (perm ? __ldg(perm + at) : at);  // no order given: the tensors are in view order
+                }
             };
-            int next = step_idx(-2);
+            const int first = (int)((step + team) & 1) - 1;  // of this team's steps
+            // step -1: the two Q halves and the row data of the unit; steps 0 ..: the key tiles
 #pragma unroll 1
-            for (int i = -2; i < n_tiles; ++i) {
-                const int now = next;
-                if (i + 1 < n_tiles) next = step_idx(i + 1);
-                else if (warp == kLoadWarp0 && !redo) claim();
-                const TileInfo t = tile_info(un, max(i, 0), nA);
-                const int stage = kv_cnt % kStages;
-                if (i != -1) {
-                    const uint32_t bar = i < 0 ? kBarQEmpty + qb : kBarKVEmpty + stage;
-                    if (!(alive = wait_free(bars + 8 * bar, ((i < 0 ? unit_cnt >> 1 : kv_cnt / kStages) & 1) ^ 1))) break;
-                }
-                const uint32_t dst = base + (i < 0 ? kOffQ + (qb * 2 + i + 2) * kTileBytes : kOffKV + stage * 2 * kTileBytes);
+            for (int i = -1; i < n_tiles; ++i) {
+                // The number of the next unit travels under the copies.  Claimed in front of the last tile but one of a long
+                // unit, of the last one of a short one: there a claim more tiles ahead ties units to CTAs that are
+                // not the next to be free (4 x 2048 tokens: 33.5 us, 35.1 with all claims early; 1 x 8192: 55.0, 55.9 with
+                // all of them late).
+                if (warp == kLoadWarp0 && i == (n_tiles <= 6 ? n_tiles - 1 : n_tiles - 2) && !redo) claim();
+                if ((i ^ first) & 1) continue;
+                const uint32_t c = kv_cnt + max(i, 0), stage = c % kStages;
                 const uint32_t bar_full = bars + 8 * (i < 0 ? kBarQFull + qb : kBarKVFull + stage);
-                // (Q tiles are always gathered: their rows past the half's own repeat one of them.)
-                const bool bulk = i >= 0 && bulk_tile(t, ident);
+                if (!(alive = wait(bars + 8 * (i < 0 ? kBarQEmpty + qb : kBarKVEmpty + stage), ((i < 0 ? unit_cnt >> 1 : c / kStages) & 1) ^ 1))) break;
                 TR_T0(t_cp);
-                if (bulk) {
-                    if (ltid == 0) {
-                        mbar_expect_tx(bar_full, 2 * kTileBytes);
-                        tma_load_2d(dst, &p.tmK, 0, (int)bh + t.first(), bar_full);
-                        tma_load_2d(dst + kTileBytes, &p.tmV, 0, (int)bh + t.first(), bar_full);
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_full);
-                } else if (i >= 0 || un.rows_of(i + 2) > 0) {
-                    gather_rows(dst, i < 0 ? Qbh : Kbh, i >= 0, v_off, now, i < 0 ? kTile : (t.w + 15) & ~15, lw, lane);
-                    TR_ADD(2, t_cp);
-                }
-                if (i == -2) {  // row data for the softmax threads: original position and key range
-                    const uint32_t meta = base + kOffMeta + qb * 3 * kUnitRows * 4;
+                if (i < 0) {
+                    // row data for the softmax threads: original position and key range
 #pragma unroll 1
-                    for (int rr = ltid; rr < kUnitRows; rr += kLoadThreads) {
-                        const int half = rr / kTile;
-                        if (rr - half * kTile < un.rows_of(half)) {
-                            const size_t at = bn + un.row0_of(half) + rr - half * kTile;
-                            cp_async4(meta + rr * 4, vp.perm + at);
-                            cp_async4(meta + (kUnitRows + rr) * 4, vp.seg_lo + at);
-                            cp_async4(meta + (2 * kUnitRows + rr) * 4, vp.seg_hi + at);
+                    for (int k = 0; k < 4; ++k) {
+                        const int half = k >> 1, rr = r0 + (k & 1) * 32 + lane;
+                        if (rr < un.rows_of(half)) {
+                            const size_t at = bn + un.row0_of(half) + rr;
+                            const uint32_t meta = base + kOffMeta + (qb * 3 * kUnitRows + half * kTile + rr) * 4;
+                            cp_async4(meta, vp.perm + at);
+                            cp_async4(meta + kUnitRows * 4, vp.seg_lo + at);
+                            cp_async4(meta + 2 * kUnitRows * 4, vp.seg_hi + at);
                         }
                     }
-                    continue;
+                    cp_async_arrive(bar_full);
                 }
-                if (!bulk) commit_and_signal(bar_full);
-                if (i + 1 == n_tiles && warp == kLoadWarp0) {
-                    if (redo) rec = held_back;
-                    else fetch_record(true);
+                __syncwarp();
+                const TileInfo t = tile_info(un, max(i, 0), nA);
+                if (i >= 0 && bulk_tile(t, ident)) {
+                    if (leader) {
+                        mbar_arrive_expect_tx(bar_full, lw == 0 ? 2 * kTileBytes : 0);
+                        if (lw == 0) {
+                            const uint32_t dst = base + kOffKV + stage * 2 * kTileBytes;
+                            tma_load_2d(dst, &p.tmK, 0, (int)bh + t.first(), bar_full);
+                            tma_load_2d(dst + kTileBytes, &p.tmV, 0, (int)bh + t.first(), bar_full);
+                        }
+                    }
+                } else {
+                    // (rows of a Q half past its last one are never looked at: their results are not stored)
+                    const auto mine = [&](int rows) { return min(max(rows - r0, 0), kLoadRows); };
+                    const int rows_a = mine(i < 0 ? un.rows_of(0) : (t.w + 15) & ~15), rows_b = i < 0 ? mine(un.rows_of(1)) : rows_a;
+                    if (leader) mbar_arrive_expect_tx(bar_full, gather_bytes(rows_a) + gather_bytes(rows_b));
+#pragma unroll 1
+                    for (int half = 0; half < (i < 0 ? 2 : 1); ++half) {
+                        const int rows = half ? rows_b : rows_a;
+                        if (rows == 0) continue;
+                        look_up(i < 0 ? row_tile(un.row0_of(half), un.rows_of(half)) : t);
+                        gather_rows4<1>(base + (i < 0 ? kOffQ + (qb * 2 + half) * kTileBytes : kOffKV + stage * 2 * kTileBytes),
+                                     i < 0 ? &p.tmQ1 : &p.tmK1, i < 0 ? nullptr : &p.tmV1, idx, r0, rows, leader, bar_full);
+                    }
                 }
-                if (i < 0) {
-                    ++unit_cnt;
-                    continue;
-                }
-                // The very first tile of the CTA: the other warps are waiting for it, so it (and Q) are
-                // signalled as soon as they have landed, not two tiles later.
-                if (kv_cnt == 0) flush();
+                __syncwarp();
+                TR_ADD(2, t_cp);
                 TR_INC(4);
-                ++kv_cnt;
             }
+            if (warp == kLoadWarp0 && alive) {
+                if (redo) rec = held_back;
+                else fetch_record(true);
+            }
+            kv_cnt += n_tiles;
+            ++unit_cnt;
+            step += 1 + n_tiles;
         }
-        flush();  // drain: signal the groups still pending
     }
 
 #ifdef MATE_TRACE
@@ -920,8 +878,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         o[7] = clock64() - tr_start;
     }
 #endif
+    if (*s_abort)  // copies may still be on their way to shared memory: they take a few microseconds
+        for (int i = 0; i < 50; ++i) __nanosleep(1000);
     tc_fence_before();
     __syncthreads();
+    if (tid == 0 && *s_abort) atomicOr(p.status + 1, 1);
     if (warp == kMmaWarp) tmem_dealloc(tmem, kTmemCols);
 }
 
@@ -973,13 +934,13 @@ int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     // Bulk tensor copies for the K/V tiles that are contiguous in the caller's tensors (see bulk_tile), unless the
     // caller asks for gathers; tensors in view order always take them.  Bulk copies against gathers, back to back:
     // 4 x 2048 tokens 32.3 us against 32.7, 8 x 512 17.9 and 17.9, 2 x 4096 55.5 and 55.4, 1 x 8192 54.8 and 54.5.
-    // When the driver entry point for tensor maps is missing every tile is gathered.
     const bool want_bulk = !(flags & MATE_FLAG_GATHER_TILES) || (flags & MATE_FLAG_VIEW_ORDER);
-    p.use_tma = want_bulk && rows < (size_t(1) << 31) && make_row_map(&p.tmK, K, rows) && make_row_map(&p.tmV, V, rows);
+    p.bulk = want_bulk ? 1 : 0;
+    if (rows >= (size_t(1) << 31)) return MATE_ERR_UNSUPPORTED;
+    if (!make_row_map(&p.tmK, K, rows) || !make_row_map(&p.tmV, V, rows) || !make_row_map(&p.tmQ1, Q, rows, 1) ||
+        !make_row_map(&p.tmK1, K, rows, 1) || !make_row_map(&p.tmV1, V, rows, 1))
+        return MATE_ERR_CUDA;
     p.view_order = (flags & MATE_FLAG_VIEW_ORDER) ? 1 : 0;
-    p.Q = (const __nv_bfloat16 *)Q;
-    p.K = (const __nv_bfloat16 *)K;
-    p.V = (const __nv_bfloat16 *)V;
     p.O = (__nv_bfloat16 *)O;
     p.LSE = LSE;
     p.rowv = plan->view[0];

@@ -325,7 +325,7 @@ void make_bwd_units(mate_plan_t *pl, const ProtoList &singles, const HeadLists &
     for (const Proto &pr : singles.protos)
         for (int h : heads.heads[pr.view]) {
             pl->bwd_units.push_back(pr.u);
-            pl->bwd_units.back().h = h;
+            pl->bwd_units.back().hv = h | pr.view << mate::kViewShift;
         }
     pl->n_bwd_units = (int)pl->bwd_units.size();
     pl->bwd_grid = std::min(std::max(pl->n_ctas, 1), std::max(2 * pl->n_bwd_units, pl->n_pads));
@@ -399,7 +399,7 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
         for (int h : heads.heads[e.view]) {
             pl->fwd_units.push_back(e.u);
             FwdUnit &u = pl->fwd_units.back();
-            u.h = h;
+            u.hv = h | e.view << mate::kViewShift;
             if (u.n_parts() > 1) {
                 u.ctr += k;
                 u.ws_off += (int32_t)((k * u.n_parts() * mate::kPartialBytes) >> 10);
@@ -413,7 +413,7 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
     pl->pads.clear();
     for (int b = 0; b < pl->B; ++b)
         for (int t0 = pl->n_valid[b]; t0 < pl->N; t0 += mate::kPadRows)
-            for (int h = 0; h < pl->H; ++h) pl->pads.push_back({b, h, t0, std::min(mate::kPadRows, pl->N - t0)});
+            for (int h = 0; h < pl->H; ++h) pl->pads.push_back({b, h | pl->head_view[h] << mate::kViewShift, t0, std::min(mate::kPadRows, pl->N - t0)});
     pl->n_pads = (int)pl->pads.size();
     pl->fwd_grid = std::min(n_ctas, std::max(pl->n_fwd_units, pl->n_pads));
     if (getenv("MATE_LOG"))
@@ -717,7 +717,7 @@ static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int
     for (int b = 0; b < B; ++b)
         if (prefix_len[b] < 0 || prefix_len[b] > N) return MATE_ERR_INVALID_ARG;
     if (max_row_id < 0 || max_col_id < 0) return MATE_ERR_INVALID_ARG;
-    if ((long long)B * N > (1ll << 30) || max_row_id > (1 << 28) || max_col_id > (1 << 28))
+    if ((long long)B * N > (1ll << 30) || max_row_id > (1 << 28) || max_col_id > (1 << 28) || H >= 1 << mate::kViewShift)
         return MATE_ERR_UNSUPPORTED;
     for (int h = 0; h < H; ++h)
         if (head_view[h] > 1) return MATE_ERR_INVALID_ARG;

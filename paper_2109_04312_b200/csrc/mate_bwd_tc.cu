@@ -112,8 +112,7 @@ struct Params {
     CUtensorMap tmQ1, tmK1, tmV1, tmdO1;  // of one row, for the gathers
     const float *nlse, *D;  // per row, original order: -LSE log2 e, D
     __nv_bfloat16 *dQ, *dK, *dV;
-    ViewPlan rowv, colv;
-    const uint8_t *head_view;
+    ViewPlan view[2];
     const FwdUnit *units;  // one half each; item = 2 unit + (0 key side, 1 query side)
     int n_units, N, H;
     const PadChunk *pads;
@@ -455,12 +454,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
 #pragma unroll 1
         for (int c = blockIdx.x; c < p.n_pads; c += gridDim.x) {
             const PadChunk pc = p.pads[c];
-            const ViewPlan &vp = p.head_view[pc.h] ? p.colv : p.rowv;
+            const ViewPlan &vp = p.view[pc.view()];
 #pragma unroll 2
             for (int i = q4 * 4 + (lane >> 3); i < pc.n; i += 4 * kStoreWarps) {  // eight lanes per row
                 const int orig = __ldg(vp.perm + (size_t)pc.b * p.N + pc.t0 + i);
                 if (p.tr.exists(pc.b, orig)) {
-                    const size_t at = (p.tr.base(pc.b, pc.h) + orig) * 64 + (lane & 7) * 8;
+                    const size_t at = (p.tr.base(pc.b, pc.head()) + orig) * 64 + (lane & 7) * 8;
                     *reinterpret_cast<uint4 *>(p.dQ + at) = make_uint4(0, 0, 0, 0);
                     *reinterpret_cast<uint4 *>(p.dK + at) = make_uint4(0, 0, 0, 0);
                     *reinterpret_cast<uint4 *>(p.dV + at) = make_uint4(0, 0, 0, 0);
@@ -475,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             if (un.rows == 0) break;
             const bool key_side = un.ws_off == 0, any = ItemTiles(un).n > 0;
             const int rows_h = un.rows_of(0);
-            const size_t at = p.tr.base(un.b, un.h) * 64;
+            const size_t at = p.tr.base(un.b, un.head()) * 64;
             __syncwarp();
             if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
             if (!wait(bars + 8 * (kBarRFull + rb), (n >> 1) & 1)) break;
@@ -657,10 +656,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             const bool key_side = un.ws_off == 0;
             const ItemTiles tiles(un);
             const int rows_h = un.rows_of(0);
-            const ViewPlan &vp = p.head_view[un.h] ? p.colv : p.rowv;
+            const ViewPlan &vp = p.view[un.view()];
             const size_t bn = (size_t)un.b * p.N;
             const int32_t *perm = vp.perm + bn;
-            const size_t bh = p.tr.base(un.b, un.h);
+            const size_t bh = p.tr.base(un.b, un.head());
             // column tiles inside [0, ident) of the order are contiguous in the tensors (see bulk_tile)
             const int ident = __ldg(vp.ident + un.b);
             const int r0 = kLoadRows * lw + lane;  // this lane's rows of a tile: r0, r0 + 32, .. (rows behind the last one repeat it)
@@ -781,9 +780,7 @@ int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.dQ = (__nv_bfloat16 *)dQ;
     p.dK = (__nv_bfloat16 *)dK;
     p.dV = (__nv_bfloat16 *)dV;
-    p.rowv = plan->view[0];
-    p.colv = plan->view[1];
-    p.head_view = plan->head_view_dev;
+    for (int v = 0; v < 2; ++v) p.view[v] = plan->view[v];
     p.units = plan->bwd_units_dev;
     p.n_units = plan->n_bwd_units;
     p.N = plan->N;

@@ -117,8 +117,7 @@ struct Params {
     int view_order;  // 1: Q, K, V, O and LSE are laid out in each head's own order (no gather, no scatter)
     __nv_bfloat16 *O;
     float *LSE;
-    ViewPlan rowv, colv;
-    const uint8_t *head_view;
+    ViewPlan view[2];
     const FwdUnit *units;      // longest first
     int n_units;
     const PadChunk *pads;      // padding rows, which no unit covers
@@ -549,7 +548,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 const float inv_l = l > 0.f ? 1.f / l : 0.f;
                 const bool row_valid = r < rows_h;
                 const int orig = p.view_order ? un.row0_of(h) + r : meta[0], dst_row = row_valid ? orig : -1;
-                const size_t bh = p.tr.base(un.b, un.h);
+                const size_t bh = p.tr.base(un.b, un.head());
                 if (row_valid) p.LSE[bh + orig] = (m2 + log2f(l)) * 0.6931471805599453f;
                 // rows go through the warp's staging area, 32 columns at a time, so that a store instruction
                 // writes 64 consecutive bytes of eight rows
@@ -725,13 +724,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
 #pragma unroll 1
         for (int c = blockIdx.x; c < p.n_pads; c += gridDim.x) {
             const PadChunk pc = p.pads[c];
-            const ViewPlan &vp = p.head_view[pc.h] ? p.colv : p.rowv;
+            const ViewPlan &vp = p.view[pc.view()];
 #pragma unroll 4
             for (int i = (warp - kPadWarp0) * 4 + (lane >> 3); i < pc.n; i += 4 * kPadWarps) {  // eight lanes per row
                 const int t = pc.t0 + i;
                 const int orig = p.view_order ? t : __ldg(vp.perm + (size_t)pc.b * p.N + t);
                 if (p.tr.exists(pc.b, orig)) {
-                    const size_t row = p.tr.base(pc.b, pc.h) + orig;
+                    const size_t row = p.tr.base(pc.b, pc.head()) + orig;
                     reinterpret_cast<uint4 *>(p.O + row * 64)[lane & 7] = make_uint4(0, 0, 0, 0);
                     if ((lane & 7) == 0) p.LSE[row] = -INFINITY;
                 }
@@ -781,10 +780,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             if (!next_unit(n, un)) break;
             un.tB &= 0xff;
             const int nA = un.tiles_a(), nB = un.tiles_b(), n_tiles = nA + nB;
-            const ViewPlan &vp = p.head_view[un.h] ? p.colv : p.rowv;
+            const ViewPlan &vp = p.view[un.view()];
             const size_t bn = (size_t)un.b * p.N;
             const int32_t *perm = p.view_order ? nullptr : vp.perm + bn;
-            const size_t bh = p.tr.base(un.b, un.h);
+            const size_t bh = p.tr.base(un.b, un.head());
             // Rows of the order that sit in place in the tensors ([0, ident)): a K/V tile inside that range
             // (see bulk_tile) is one contiguous [128, 64] box and comes in by one bulk tensor copy per matrix
             // instead of 2 x 32 gathers of four rows.  That is the prefix block's full tiles in every unit and, for a
@@ -943,9 +942,7 @@ int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.view_order = (flags & MATE_FLAG_VIEW_ORDER) ? 1 : 0;
     p.O = (__nv_bfloat16 *)O;
     p.LSE = LSE;
-    p.rowv = plan->view[0];
-    p.colv = plan->view[1];
-    p.head_view = plan->head_view_dev;
+    for (int v = 0; v < 2; ++v) p.view[v] = plan->view[v];
     p.units = plan->fwd_units_dev;
     p.n_units = plan->n_fwd_units;
     p.pads = plan->pads_dev;

@@ -22,6 +22,8 @@ constexpr int kTraceCtas = 256;  // CTAs whose cycle counters a -DMATE_TRACE bui
 __host__ __device__ inline int div_tile(int x, int tB) { return tB == kTile ? x >> 7 : x / tB; }
 static_assert(kTile == 128, "div_tile");
 
+constexpr int kViewShift = 28;   // of the view (row or column) in a record's head: no look-up in front of a unit's first loads
+
 // One unit of work of the tensor-core kernels: up to 256 consecutive rows (view order) of one (example, head)
 // in two halves of up to 128 -- half 0 = the first n0 rows, half 1 = the n1 rows behind them -- and the
 // column tiles they visit, in this order:
@@ -36,7 +38,7 @@ static_assert(kTile == 128, "div_tile");
 // partial result to the workspace at ws_off (KiB); per group of 32 rows the part that finishes
 // last (counted in counters[kSchedWords + 8 * ctr + row / 32]) combines them.
 struct alignas(16) FwdUnit {  // (copied as four 16-byte words)
-    int32_t b, h;
+    int32_t b, hv;             // hv = head | view << kViewShift
     int32_t q0, rows;          // rows = n0 | n1 << 8 | kP << 16; 0 ends a list
     int32_t kA0, kA_end;
     int32_t kB0, kB_end;
@@ -44,6 +46,8 @@ struct alignas(16) FwdUnit {  // (copied as four 16-byte words)
     int32_t tB, parts;         // parts = n_parts | part << 16 (tB: the forward keeps flags above bit 7 on its way)
     int32_t ws_off, ctr;
 
+    __host__ __device__ int head() const { return hv & ((1 << kViewShift) - 1); }
+    __host__ __device__ int view() const { return hv >> kViewShift; }
     __host__ __device__ int rows_of(int half) const { return half ? (rows >> 8) & 0xff : rows & 0xff; }
     __host__ __device__ int row0_of(int half) const { return half ? q0 + (rows & 0xff) : q0; }
     __host__ __device__ int kP() const { return rows >> 16; }
@@ -89,7 +93,9 @@ constexpr size_t kPartialBytes = (size_t)kUnitRows * (64 + 4) * sizeof(float);
 // kernel before its first unit.
 constexpr int kPadRows = 64;
 struct PadChunk {
-    int32_t b, h, t0, n;
+    int32_t b, hv, t0, n;
+    __host__ __device__ int head() const { return hv & ((1 << kViewShift) - 1); }
+    __host__ __device__ int view() const { return hv >> kViewShift; }
 };
 
 // Where the rows of example b, head h start in the caller's tensors (in rows of d elements), and how

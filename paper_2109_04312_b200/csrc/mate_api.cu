@@ -322,8 +322,10 @@ void list_units(const mate_plan_t *pl, const std::vector<RowRanges> &ranges, boo
 // order is the whole schedule.
 void make_bwd_units(mate_plan_t *pl, const ProtoList &singles, const HeadLists &heads) {
     pl->bwd_units.clear();
+    pl->bwd_costs.clear();
     for (const Proto &pr : singles.protos)
         for (int h : heads.heads[pr.view]) {
+            pl->bwd_costs.push_back(pr.cost);
             pl->bwd_units.push_back(pr.u);
             pl->bwd_units.back().hv = h | pr.view << mate::kViewShift;
         }
@@ -394,9 +396,11 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
     std::stable_sort(entries.begin(), entries.end(), [](const Entry &a, const Entry &b) { return a.cost > b.cost; });
     pl->fwd_units.clear();
     pl->fwd_units.reserve(n_units);
+    pl->fwd_costs.clear();
     for (const Entry &e : entries) {
         int k = 0;
         for (int h : heads.heads[e.view]) {
+            pl->fwd_costs.push_back(e.cost);
             pl->fwd_units.push_back(e.u);
             FwdUnit &u = pl->fwd_units.back();
             u.hv = h | e.view << mate::kViewShift;
@@ -423,7 +427,7 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
                 entries.empty() ? 0ll : (long long)entries.front().cost, pl->fwd_ws_bytes, pl->n_pads);
 }
 
-int build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], cudaStream_t st) {
+void build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2]) {
     static_assert(mate::kPartialBytes % 1024 == 0, "ws_off counts KiB");
     std::vector<RowRanges> ranges((size_t)2 * pl->B);
     for (int v = 0; v < 2; ++v)
@@ -447,8 +451,62 @@ int build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], cudaSt
     ProtoList singles;
     list_units(pl, ranges, false, n_halves > (size_t)std::max(pl->n_ctas, 1), singles);
     make_bwd_units(pl, singles, heads);
+}
 
-    // device copy, in one piece: units, padding, arrival counters (zeros; the kernel resets them)
+// Row-or-column plan: the lists of the two further passes join this plan's, longest first again, so that one launch
+// does all three (they are independent until their results are merged).
+void join_units(mate_plan_t *pl) {
+    int slots = pl->n_fwd_slots;
+    const auto by_cost = [](std::vector<FwdUnit> &units, std::vector<int64_t> &costs) {
+        std::vector<int> order(units.size());
+        for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return costs[a] > costs[b]; });
+        std::vector<FwdUnit> u(units.size());
+        std::vector<int64_t> c(units.size());
+        for (size_t i = 0; i < order.size(); ++i) {
+            u[i] = units[order[i]];
+            c[i] = costs[order[i]];
+        }
+        units.swap(u);
+        costs.swap(c);
+    };
+    for (int s = 0; s < 2; ++s) {
+        mate_plan_t *sub = pl->sub[s];
+        const auto view = [s](int hv) { return (hv & ((1 << mate::kViewShift) - 1)) | (2 + s) << mate::kViewShift; };
+        for (FwdUnit u : sub->fwd_units) {
+            u.hv = view(u.hv);
+            if (u.n_parts() > 1) {
+                u.ctr += slots;
+                u.ws_off += (int32_t)(pl->fwd_ws_bytes >> 10);
+            }
+            pl->fwd_units.push_back(u);
+        }
+        for (FwdUnit u : sub->bwd_units) {
+            u.hv = view(u.hv);
+            pl->bwd_units.push_back(u);
+        }
+        for (mate::PadChunk c : sub->pads) {
+            c.hv = view(c.hv);
+            pl->pads.push_back(c);
+        }
+        pl->fwd_costs.insert(pl->fwd_costs.end(), sub->fwd_costs.begin(), sub->fwd_costs.end());
+        pl->bwd_costs.insert(pl->bwd_costs.end(), sub->bwd_costs.begin(), sub->bwd_costs.end());
+        slots += sub->n_fwd_slots;
+        pl->fwd_ws_bytes += sub->fwd_ws_bytes;
+    }
+    by_cost(pl->fwd_units, pl->fwd_costs);
+    by_cost(pl->bwd_units, pl->bwd_costs);
+    pl->n_fwd_slots = slots;
+    pl->n_fwd_units = (int)pl->fwd_units.size();
+    pl->n_bwd_units = (int)pl->bwd_units.size();
+    pl->n_pads = (int)pl->pads.size();
+    const int n_ctas = std::max(pl->n_ctas, 1);
+    pl->fwd_grid = std::min(n_ctas, std::max(pl->n_fwd_units, pl->n_pads));
+    pl->bwd_grid = std::min(n_ctas, std::max(2 * pl->n_bwd_units, pl->n_pads));
+}
+
+// Device copy of the lists, in one piece: units, padding, arrival counters (zeros; the kernel resets them).
+int upload_units(mate_plan_t *pl, cudaStream_t st) {
     const auto lay_out = [pl](char *base) {
         Carver c(base);
         pl->fwd_units_dev = c.take<FwdUnit>(pl->n_fwd_units);
@@ -530,13 +588,13 @@ int mate_plan_bucketed(const int32_t *row_ids, const int32_t *col_ids, int B, in
 
 static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int N, const int32_t *prefix_len,
                       const int32_t *global_len, const uint8_t *head_view, int H, int max_row_id, int max_col_id,
-                      int radius, int bounds_mode, int group, void *stream, mate_plan_t **out);
+                      int radius, int bounds_mode, int group, bool upload, void *stream, mate_plan_t **out);
 
 int mate_plan_varlen(const int32_t *row_ids, const int32_t *col_ids, int B, int N, const int32_t *prefix_len,
                      const uint8_t *head_view, int H, int max_row_id, int max_col_id, int radius,
                      void *stream, mate_plan_t **out) {
     return build_plan(row_ids, col_ids, B, N, prefix_len, nullptr, head_view, H, max_row_id, max_col_id, radius,
-                      mate::kBoundsOwn, 1, stream, out);
+                      mate::kBoundsOwn, 1, true, stream, out);
 }
 
 int mate_plan_bucketed_global(const int32_t *row_ids, const int32_t *col_ids, int B, int N, const int32_t *prefix_len,
@@ -547,7 +605,7 @@ int mate_plan_bucketed_global(const int32_t *row_ids, const int32_t *col_ids, in
     for (int b = 0; b < B; ++b)
         if (global_len[b] < prefix_len[b] || global_len[b] > N) return MATE_ERR_INVALID_ARG;
     return build_plan(row_ids, col_ids, B, N, prefix_len, global_len, head_view, H, max_row_id, max_col_id, radius,
-                      mate::kBoundsOwn, 1, stream, out);
+                      mate::kBoundsOwn, 1, true, stream, out);
 }
 
 /* Packed batches: the examples lie one behind the other on a common token axis.  The plan itself is the
@@ -586,7 +644,7 @@ static int plan_packed(const int32_t *row_ids, const int32_t *col_ids, int B, co
         ok = cudaMemcpyAsync(off_dev, host.ptr, sizeof(int32_t) * 2 * B, cudaMemcpyHostToDevice, st) == cudaSuccess &&
              mate::launch_unpack_ids(row_ids, col_ids, B, n_max, off_dev, off_dev + B, ids_dev, ids_dev + BN, st) == cudaSuccess;
         rc = ok ? build_plan(ids_dev, ids_dev + BN, B, n_max, prefix_len, nullptr, head_view, H, max_row_id, max_col_id, 0,
-                             mate::kBoundsOwn, 1, stream, &pl)
+                             mate::kBoundsOwn, 1, true, stream, &pl)
                 : MATE_ERR_CUDA;
     }
     mate::staging_give(host, st);
@@ -627,7 +685,7 @@ static int plan_sat(const int32_t *row_ids, const int32_t *col_ids, int B, int N
     const std::vector<uint8_t> rows_only((size_t)H, 0), cols_only((size_t)H, 1);
     mate_plan_t *pl = nullptr;
     int rc = build_plan(row_ids, col_ids, B, N, prefix.data(), nullptr, rows_only.data(), H, max_row_id, max_col_id, 0,
-                        mate::kBoundsOwn, 1, stream, &pl);
+                        mate::kBoundsOwn, 1, false, stream, &pl);
     if (rc != MATE_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     const int n_row_ids = max_row_id + 1, max_pair = n_row_ids * (max_col_id + 1) - 1;
@@ -641,7 +699,12 @@ static int plan_sat(const int32_t *row_ids, const int32_t *col_ids, int B, int N
     }
     for (int s = 0; s < 2 && rc == MATE_OK; ++s)
         rc = build_plan(pl->pair_ids_dev, pl->pair_ids_dev, B, N, zero.data(), nullptr, cols_only.data(), H, max_pair, max_pair, 0,
-                        s == 0 ? mate::kBoundsBefore : mate::kBoundsAfter, n_row_ids, stream, &pl->sub[s]);
+                        s == 0 ? mate::kBoundsBefore : mate::kBoundsAfter, n_row_ids, false, stream, &pl->sub[s]);
+    if (rc == MATE_OK)
+        rc = no_throw([&]() {
+            join_units(pl);
+            return upload_units(pl, st);
+        });
     if (rc != MATE_OK) {
         mate_plan_destroy(pl);
         return rc;
@@ -659,7 +722,7 @@ int mate_plan_sat(const int32_t *row_ids, const int32_t *col_ids, int B, int N, 
 // Fills an empty plan from checked arguments; the caller owns the plan and the staging buffer whatever comes of it.
 static int fill_plan(mate_plan_t *pl, mate::Staging &host, const int32_t *row_ids, const int32_t *col_ids, int B, int N,
                      const int32_t *prefix_len, const int32_t *global_len, const uint8_t *head_view, int H, int max_row_id,
-                     int max_col_id, int radius, int bounds_mode, int group, cudaStream_t st) {
+                     int max_col_id, int radius, int bounds_mode, int group, bool upload, cudaStream_t st) {
     pl->B = B;
     pl->N = N;
     pl->prefix.assign(prefix_len, prefix_len + B);
@@ -704,12 +767,13 @@ static int fill_plan(mate_plan_t *pl, mate::Staging &host, const int32_t *row_id
     if (out_host(pl->status_dev)[0] != 0) return MATE_ERR_INVALID_ARG;
     pl->n_valid.assign(out_host(pl->n_valid_dev), out_host(pl->n_valid_dev) + B);
     const int32_t *seg_off_host[2] = {out_host(pl->view[0].seg_off), out_host(pl->view[1].seg_off)};
-    return build_units(pl, seg_off_host, st);
+    build_units(pl, seg_off_host);
+    return upload ? upload_units(pl, st) : MATE_OK;
 }
 
 static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int N, const int32_t *prefix_len,
                       const int32_t *global_len, const uint8_t *head_view, int H, int max_row_id, int max_col_id,
-                      int radius, int bounds_mode, int group, void *stream, mate_plan_t **out) {
+                      int radius, int bounds_mode, int group, bool upload, void *stream, mate_plan_t **out) {
     if (out) *out = nullptr;
     if (radius < 0) return MATE_ERR_INVALID_ARG;
     if (!row_ids || !col_ids || !head_view || !out || !prefix_len) return MATE_ERR_INVALID_ARG;
@@ -728,7 +792,7 @@ static int build_plan(const int32_t *row_ids, const int32_t *col_ids, int B, int
     mate::Staging host;
     const int rc = no_throw([&]() {
         return fill_plan(pl, host, row_ids, col_ids, B, N, prefix_len, global_len, head_view, H, max_row_id, max_col_id, radius,
-                         bounds_mode, group, st);
+                         bounds_mode, group, upload, st);
     });
     mate::staging_give(host, st);
     if (rc != MATE_OK) {
@@ -782,8 +846,10 @@ int mate_plan_status(const mate_plan_t *plan, void *stream) {
     if (s[1] != 0) {
         if (getenv("MATE_LOG")) fprintf(stderr, "[mate] a bounded wait expired\n");
         // a kernel that gave up may have left the arrival counters half way
-        if (cudaMemsetAsync(plan->fwd_counters_dev, 0, sizeof(int32_t) * (mate::kSchedWords + 8 * (size_t)plan->n_fwd_slots), st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
+        // (the passes of a row-or-column plan have none of their own)
+        if (plan->fwd_counters_dev &&
+            (cudaMemsetAsync(plan->fwd_counters_dev, 0, sizeof(int32_t) * (mate::kSchedWords + 8 * (size_t)plan->n_fwd_slots), st) != cudaSuccess ||
+             cudaStreamSynchronize(st) != cudaSuccess))
             return MATE_ERR_CUDA;
         return MATE_ERR_TIMEOUT;
     }
@@ -812,14 +878,11 @@ static int check_common(const mate_plan_t *plan, int d, int dtype, unsigned flag
     return MATE_OK;
 }
 
-// Scratch of one pass (the ordinary kernels) and of a whole call.  For a row-or-column plan the call
-// holds, behind the passes' own scratch (the passes run one after the other and share it), the
-// outputs of the two extra passes: forward 2 x (O + LSE), backward 2 x (dQ, dK, dV).
+// Scratch of the ordinary kernels and of a whole call.  For a row-or-column plan the call holds, behind the kernels'
+// own scratch (the tensor-core kernels do the three passes in one launch; without tensor cores they run one after
+// the other and share it), the outputs of the two extra passes: forward 2 x (O + LSE), backward 2 x (dQ, dK, dV).
 static size_t pass_fwd_bytes(const mate_plan_t *plan, int d, bool use_tc) {
-    size_t n = use_tc ? mate::tc_fwd_workspace(plan, d) : 0;
-    for (int s = 0; s < 2; ++s)
-        if (plan->sub[s]) n = std::max(n, use_tc ? mate::tc_fwd_workspace(plan->sub[s], d) : (size_t)0);
-    return align_up(n, 256);
+    return align_up(use_tc ? mate::tc_fwd_workspace(plan, d) : 0, 256);
 }
 static size_t pass_bwd_bytes(const mate_plan_t *plan, bool use_tc) {
     return align_up(use_tc ? mate::tc_bwd_workspace(plan) : mate::simt_bwd_workspace(plan), 256);
@@ -849,12 +912,6 @@ static cudaError_t use_plans(const mate_plan_t *plan, cudaStream_t st) {
     return rc;
 }
 
-static int fwd_pass(const mate_plan_t *plan, bool use_tc, const void *Q, const void *K, const void *V, int d, int dtype,
-                    float scale, void *O, float *LSE, void *ws, unsigned flags, cudaStream_t st) {
-    if (use_tc) return mate::tc_fwd(plan, Q, K, V, scale, O, LSE, ws, flags, st);
-    return mate::simt_fwd(plan, Q, K, V, d, dtype, scale, O, LSE, flags, st);
-}
-
 int mate_attn_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, int d,
                   int dtype, float scale, void *O, float *LSE, void *workspace,
                   size_t workspace_bytes, unsigned flags, void *stream) {
@@ -877,30 +934,26 @@ int mate_attn_fwd(const mate_plan_t *plan, const void *Q, const void *K, const v
     if (need > 0 && (reinterpret_cast<uintptr_t>(workspace) & 255u)) return MATE_ERR_ALIGNMENT;
     if ((flags & MATE_FLAG_VIEW_ORDER) && (plan->sub[0] || plan->T)) return MATE_ERR_UNSUPPORTED;
     if (use_plans(plan, st) != cudaSuccess) return MATE_ERR_CUDA;
-    rc = fwd_pass(plan, use_tc, Q, K, V, d, dtype, scale, O, LSE, workspace, flags, st);
-    if (rc != MATE_OK || !plan->sub[0]) return rc;
-    // row-or-column pattern: the two passes over the rest of the column, then the merge
+    // Row-or-column pattern: the two passes over the rest of the column, and then the merge.
     const size_t rows = plan->n_rows();
     const size_t o_bytes = align_up(rows * d * elem_bytes(dtype), 256), l_bytes = align_up(rows * sizeof(float), 256);
     char *w = (char *)workspace + pass_fwd_bytes(plan, d, use_tc);
-    void *Os[2];
-    float *Ls[2];
-    for (int s = 0; s < 2; ++s) {
-        Os[s] = w;
-        Ls[s] = (float *)(w + o_bytes);
-        w += o_bytes + l_bytes;
-        rc = fwd_pass(plan->sub[s], use_tc, Q, K, V, d, dtype, scale, Os[s], Ls[s], workspace, flags, st);
-        if (rc != MATE_OK) return rc;
+    void *Os[mate::kPasses] = {O, nullptr, nullptr};
+    float *Ls[mate::kPasses] = {LSE, nullptr, nullptr};
+    for (int i = 1; i < mate::kPasses && plan->sub[0]; ++i, w += o_bytes + l_bytes) {
+        Os[i] = w;
+        Ls[i] = (float *)(w + o_bytes);
     }
-    return mate::launch_merge_passes(O, LSE, Os[0], Ls[0], Os[1], Ls[1], rows, d, dtype, st) == cudaSuccess ? MATE_OK
+    if (use_tc) {  // all passes at once
+        rc = mate::tc_fwd(plan, Q, K, V, scale, Os, Ls, workspace, flags, st);
+    } else {
+        for (int i = 0; i < mate::kPasses && rc == MATE_OK; ++i)
+            if (const mate_plan_t *pass = i ? plan->sub[i - 1] : plan)
+                rc = mate::simt_fwd(pass, Q, K, V, d, dtype, scale, Os[i], Ls[i], flags, st);
+    }
+    if (rc != MATE_OK || !plan->sub[0]) return rc;
+    return mate::launch_merge_passes(O, LSE, Os[1], Ls[1], Os[2], Ls[2], rows, d, dtype, st) == cudaSuccess ? MATE_OK
                                                                                                            : MATE_ERR_CUDA;
-}
-
-static int bwd_pass(const mate_plan_t *plan, bool use_tc, const void *Q, const void *K, const void *V, const void *O,
-                    const float *LSE, const void *dO, int d, int dtype, float scale, void *dQ, void *dK, void *dV, void *ws,
-                    int pass, cudaStream_t st) {
-    if (use_tc) return mate::tc_bwd(plan, Q, K, V, O, LSE, dO, scale, dQ, dK, dV, ws, pass, st);
-    return mate::simt_bwd(plan, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, ws, pass, st);
 }
 
 int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
@@ -922,8 +975,6 @@ int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const v
     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MATE_ERR_ALIGNMENT;
     cudaStream_t st = (cudaStream_t)stream;
     if (use_plans(plan, st) != cudaSuccess) return MATE_ERR_CUDA;
-    rc = bwd_pass(plan, use_tc, Q, K, V, O, LSE, dO, d, dtype, scale, dQ, dK, dV, workspace, 0, st);
-    if (rc != MATE_OK || !plan->sub[0]) return rc;
     // Row-or-column pattern.  With the final O and LSE every pass computes the gradient of its own
     // pairs.  The two column passes are each other's transpose (keys in front of / behind the own
     // cell), and the kernels take a plan's key ranges for the query side and for the key side alike;
@@ -931,14 +982,20 @@ int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const v
     const size_t n = plan->n_rows() * d;
     const size_t g_bytes = align_up(n * elem_bytes(dtype), 256);
     char *w = (char *)workspace + pass_bwd_bytes(plan, use_tc);
-    void *g[2][3];
-    for (int s = 0; s < 2; ++s) {
-        for (int i = 0; i < 3; ++i, w += g_bytes) g[s][i] = w;
-        rc = bwd_pass(plan->sub[s], use_tc, Q, K, V, O, LSE, dO, d, dtype, scale, g[s][0], g[s][1], g[s][2], workspace, 1 + s, st);
-        if (rc != MATE_OK) return rc;
+    void *g[3][mate::kPasses] = {{dQ}, {dK}, {dV}};  // of every pass
+    for (int i = 1; i < mate::kPasses && plan->sub[0]; ++i)
+        for (int t = 0; t < 3; ++t, w += g_bytes) g[t][i] = w;
+    if (use_tc) {  // all passes at once
+        rc = mate::tc_bwd(plan, Q, K, V, O, LSE, dO, scale, g[0], g[1], g[2], workspace, st);
+    } else {
+        for (int i = 0; i < mate::kPasses && rc == MATE_OK; ++i)
+            if (const mate_plan_t *pass = i ? plan->sub[i - 1] : plan)
+                rc = mate::simt_bwd(pass, Q, K, V, O, LSE, dO, d, dtype, scale, g[0][i], g[1][i], g[2][i], workspace, i, st);
     }
+    if (rc != MATE_OK || !plan->sub[0]) return rc;
+    void *second[3] = {g[0][1], g[1][1], g[2][1]}, *third[3] = {g[0][2], g[1][2], g[2][2]};
     void *outs[3] = {dQ, dK, dV};
-    return mate::launch_add3(outs, g[0], g[1], n, dtype, st) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
+    return mate::launch_add3(outs, second, third, n, dtype, st) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }
 
 }  // extern "C"

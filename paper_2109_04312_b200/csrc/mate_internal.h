@@ -22,7 +22,10 @@ constexpr int kTraceCtas = 256;  // CTAs whose cycle counters a -DMATE_TRACE bui
 __host__ __device__ inline int div_tile(int x, int tB) { return tB == kTile ? x >> 7 : x / tB; }
 static_assert(kTile == 128, "div_tile");
 
-constexpr int kViewShift = 28;   // of the view (row or column) in a record's head: no look-up in front of a unit's first loads
+constexpr int kViewShift = 28;   // of the view in a record's head: no look-up in front of a unit's first loads
+// Views of a work-list: row, column, and the two further passes of a row-or-column plan, which have outputs of their own.
+constexpr int kViews = 4, kPasses = 3;
+__host__ __device__ inline int pass_of(int view) { return view < 2 ? 0 : view - 1; }
 
 // One unit of work of the tensor-core kernels: up to 256 consecutive rows (view order) of one (example, head)
 // in two halves of up to 128 -- half 0 = the first n0 rows, half 1 = the n1 rows behind them -- and the
@@ -162,7 +165,8 @@ struct mate_plan_s {
     int radius = 0;                      // > 0: bucketed pattern (Section 3.1), buckets of this many positions
     int bounds_mode = 0, group = 1;      // key range of a table row (kBounds*), ids per group
     // row-or-column pattern (mate_plan_sat): this plan is the row pass; sub[0] / sub[1] are the passes
-    // over the rest of the token's column in front of / behind its own cell
+    // over the rest of the token's column in front of / behind its own cell.  The work-lists of all three are in
+    // this plan's, so that the tensor-core kernels do them in one launch.
     mate_plan_s *sub[2] = {nullptr, nullptr};
     int32_t *pair_ids_dev = nullptr;     // ids of the sub-plans (in extra_block)
     // packed layout (mate_plan_packed): start and length of every example on the common token axis
@@ -214,6 +218,8 @@ struct mate_plan_s {
     int n_bwd_units = 0;
     int bwd_grid = 0;                     // CTAs of a backward launch
     std::vector<mate::FwdUnit> bwd_units;
+    std::vector<int64_t> fwd_costs, bwd_costs;  // estimated clocks of the units
+    const mate::ViewPlan &work_view(int v) const { return v < 2 || !sub[0] ? view[v & 1] : sub[v - 2]->view[1]; }
 };
 
 namespace mate {
@@ -286,11 +292,12 @@ int simt_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *
 bool tc_supported(int d, int dtype);
 size_t tc_fwd_workspace(const mate_plan_t *plan, int d);
 size_t tc_bwd_workspace(const mate_plan_t *plan);
+// (outputs: one set per pass; an ordinary plan has one)
 int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, const void *O,
-           const float *LSE, const void *dO, float scale, void *dQ, void *dK, void *dV, void *workspace, int pass,
-           cudaStream_t stream);
-int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, float scale, void *O,
-           float *LSE, void *workspace, unsigned flags, cudaStream_t stream);
+           const float *LSE, const void *dO, float scale, void *const (&dQ)[kPasses], void *const (&dK)[kPasses],
+           void *const (&dV)[kPasses], void *workspace, cudaStream_t stream);
+int tc_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, float scale, void *const (&O)[kPasses],
+           float *const (&LSE)[kPasses], void *workspace, unsigned flags, cudaStream_t stream);
 
 }  // namespace mate
 

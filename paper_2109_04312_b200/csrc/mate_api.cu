@@ -4,6 +4,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <exception>
+#include <memory>
 #include <new>
 
 #include "mate_internal.h"
@@ -104,7 +105,13 @@ constexpr int kChunk = 32;
 // Key ranges of the rows of one (example, view), by view position.
 struct RowRanges {
     int P = 0, nv = 0;  // [0, P): rows of the global block; [P, nv): table rows with the keys [lo, hi) behind the block
-    std::vector<int32_t> lo, hi;
+    int64_t own = 0;    // pairs of table rows and the keys of their own ranges
+    std::unique_ptr<int32_t[]> both;  // (not cleared: the segments fill what is read of it)
+    int32_t *lo = nullptr, *hi = nullptr;
+    std::vector<int32_t> starts;      // table rows whose lo differs from the one before (ascending)
+    void begin(int t, int l) {
+        if (starts.empty() || lo[t - 1] != l) starts.push_back(t);
+    }
 };
 
 void fill_ranges(const mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], int v, int b, RowRanges &rr) {
@@ -113,22 +120,29 @@ void fill_ranges(const mate_plan_t *pl, const int32_t *const (&seg_off_host)[2],
     const RowBounds rb{so, S, std::min(pl->global[b], pl->n_valid[b]), pl->radius, pl->bounds_mode, pl->group};
     rr.P = rb.P;
     rr.nv = pl->n_valid[b];
-    rr.lo.resize(rr.nv);
-    rr.hi.resize(rr.nv);
+    rr.both.reset(new int32_t[2 * (size_t)rr.nv + 1]);
+    rr.lo = rr.both.get();
+    rr.hi = rr.lo + rr.nv;
+    rr.starts.clear();
+    rr.starts.reserve(256);
     for (int id = 0; id + 1 < S; ++id) {
         const int t0 = std::max(so[id], rb.P), t1 = so[id + 1];
         if (t1 <= t0) continue;
         const int l = rb.own_lo(id), h = std::max(rb.own_hi(id), l);
         if (pl->radius <= 0) {
-            std::fill(rr.lo.begin() + t0, rr.lo.begin() + t1, l);
-            std::fill(rr.hi.begin() + t0, rr.hi.begin() + t1, h);
+            rr.begin(t0, l);
+            std::fill(rr.lo + t0, rr.lo + t1, l);
+            std::fill(rr.hi + t0, rr.hi + t1, h);
+            rr.own += (int64_t)(t1 - t0) * (h - l);
             continue;
         }
         for (int t = t0; t < t1;) {  // bucket by bucket
             const int end = (int)std::min<int64_t>(t1, rb.P + (int64_t)((t - rb.P) / pl->radius + 1) * pl->radius);
             const int lo = std::max(l, rb.bucket_lo(t)), hi = std::max(std::min(h, rb.bucket_hi(t)), lo);
-            std::fill(rr.lo.begin() + t, rr.lo.begin() + end, lo);
-            std::fill(rr.hi.begin() + t, rr.hi.begin() + end, hi);
+            rr.begin(t, lo);
+            std::fill(rr.lo + t, rr.lo + end, lo);
+            std::fill(rr.hi + t, rr.hi + end, hi);
+            rr.own += (int64_t)(end - t) * (hi - lo);
             t = end;
         }
     }
@@ -154,7 +168,11 @@ struct ProtoList {
 void half_tile_clks(const FwdUnit &u, int h, const RowRanges &rr, int32_t *clk) {
     const int nA = u.tiles_a(), n_tiles = nA + u.tiles_b(), rows = u.rows_of(h), r0 = u.row0_of(h);
     if (rows == 0) return;
-    for (int i = 0; i < n_tiles; ++i) {
+    for (int i = 0; i < nA; ++i) {  // every row counts every column
+        const int w = std::min(u.kA_end - u.kA0 - i * kTile, kTile);
+        clk[i] = w == kTile ? kFullClk : kPartialClk + kChunkClk * ceil_div(w, kChunk);
+    }
+    for (int i = nA; i < n_tiles; ++i) {
         const TileInfo t = mate::tile_info(u, i, nA);
         int c0, c1;
         mate::half_cols(u.lo[h], u.hi[h], t, c0, c1);
@@ -193,7 +211,13 @@ void add_proto(ProtoList &pl, const FwdUnit &u, int view, const RowRanges &rr) {
 
 // Longest first; the heads of a view repeat its units.
 void sort_protos(ProtoList &pl) {
-    std::stable_sort(pl.protos.begin(), pl.protos.end(), [](const Proto &a, const Proto &b) { return a.cost > b.cost; });
+    std::vector<std::pair<int64_t, int>> order(pl.protos.size());  // (the records are moved once)
+    for (size_t i = 0; i < order.size(); ++i) order[i] = {-pl.protos[i].cost, (int)i};
+    std::sort(order.begin(), order.end());
+    std::vector<Proto> sorted;
+    sorted.reserve(order.size());
+    for (const auto &o : order) sorted.push_back(pl.protos[o.second]);
+    pl.protos.swap(sorted);
 }
 struct HeadLists {
     std::vector<int> heads[2];
@@ -205,8 +229,8 @@ struct HeadLists {
 // Tiles that the halves of a unit visit.
 int visits(const FwdUnit &u) {
     const int nA = u.tiles_a(), n_tiles = nA + u.tiles_b();
-    int n = 0;
-    for (int i = 0; i < n_tiles; ++i)
+    int n = nA * ((u.rows_of(0) > 0) + (u.rows_of(1) > 0));
+    for (int i = nA; i < n_tiles; ++i)
         for (int h = 0; h < 2; ++h) {
             int c0, c1;
             mate::half_cols(u.lo[h], u.hi[h], mate::tile_info(u, i, nA), c0, c1);
@@ -282,12 +306,13 @@ void add_units(const RowRanges &rr, int b, int view, bool pairs, bool fill_up, P
     // Halves of table rows: 128 rows, or fewer when ending where a segment begins saves tiles (a half that
     // reaches into the next long segment visits the tiles of both; one that ends with a short segment needs
     // one tile for its own keys instead of two).  Measure: tiles, and 1.5 for the half itself, per row.
+    size_t next_start = 0;  // the first one behind `end`
     while (cuts.back() < nv) {
         const int q = cuts.back();
         int end = std::min(q + kTile, nv);
         if (end < nv || rr.lo[end - 1] != rr.lo[q]) {
-            int cut = end;
-            while (cut > q + 1 && (cut >= nv || rr.lo[cut] == rr.lo[cut - 1])) --cut;  // the last row that begins a new range
+            while (next_start < rr.starts.size() && rr.starts[next_start] <= end) ++next_start;
+            const int cut = next_start > 0 ? rr.starts[next_start - 1] : 0;  // the last row that begins a new range
             const auto per_row = [&](int e) { return (3 + 2 * tiles(rr.hi[e - 1] - rr.lo[q])) / (double)(e - q); };
             if (cut > q + 1 && per_row(cut) < per_row(end)) end = cut;
         }
@@ -312,6 +337,10 @@ void add_units(const RowRanges &rr, int b, int view, bool pairs, bool fill_up, P
 void list_units(const mate_plan_t *pl, const std::vector<RowRanges> &ranges, bool pairs, bool fill_up, ProtoList &out) {
     out.protos.clear();
     out.tiles.clear();
+    size_t rows = 0;
+    for (const RowRanges &rr : ranges) rows += rr.nv;
+    out.protos.reserve(rows / kTile + 2 * ranges.size());
+    out.tiles.reserve(rows / kTile * 8);
     for (int v = 0; v < 2; ++v)
         for (int b = 0; b < pl->B && pl->view[v].n_heads > 0; ++b) add_units(ranges[(size_t)v * pl->B + b], b, v, pairs, fill_up, out);
     sort_protos(out);
@@ -321,8 +350,12 @@ void list_units(const mate_plan_t *pl, const std::vector<RowRanges> &ranges, boo
 // the persistent kernel take work from the head of the list as they become free (a shared counter), so the
 // order is the whole schedule.
 void make_bwd_units(mate_plan_t *pl, const ProtoList &singles, const HeadLists &heads) {
+    size_t n = 0;
+    for (const Proto &pr : singles.protos) n += heads.heads[pr.view].size();
     pl->bwd_units.clear();
     pl->bwd_costs.clear();
+    pl->bwd_units.reserve(n);
+    pl->bwd_costs.reserve(n);
     for (const Proto &pr : singles.protos)
         for (int h : heads.heads[pr.view]) {
             pl->bwd_costs.push_back(pr.cost);
@@ -397,6 +430,7 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
     pl->fwd_units.clear();
     pl->fwd_units.reserve(n_units);
     pl->fwd_costs.clear();
+    pl->fwd_costs.reserve(n_units);
     for (const Entry &e : entries) {
         int k = 0;
         for (int h : heads.heads[e.view]) {
@@ -438,9 +472,7 @@ void build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2]) {
     for (int v = 0; v < 2; ++v)
         for (int b = 0; b < pl->B && pl->view[v].n_heads > 0; ++b) {
             const RowRanges &rr = ranges[(size_t)v * pl->B + b];
-            int64_t c = (int64_t)rr.P * rr.nv + (int64_t)rr.P * (rr.nv - rr.P);
-            for (int t = rr.P; t < rr.nv; ++t) c += rr.hi[t] - rr.lo[t];
-            pl->pairs[(size_t)b * 2 + v] = c;
+            pl->pairs[(size_t)b * 2 + v] = (int64_t)rr.P * rr.nv + (int64_t)rr.P * (rr.nv - rr.P) + rr.own;
         }
 
     const HeadLists heads(pl);

@@ -18,8 +18,9 @@ constexpr int kUnitRows = 256;   // query rows per unit of the tensor-core kerne
 enum { kBoundsOwn = 0, kBoundsBefore = 1, kBoundsAfter = 2 };
 constexpr int kTraceCtas = 256;  // CTAs whose cycle counters a -DMATE_TRACE build keeps
 
-// x / tB for tiles of tB columns (x >= 0); nearly always a shift.
-__host__ __device__ inline int div_tile(int x, int tB) { return tB == kTile ? x >> 7 : x / tB; }
+// x / tB for tiles of tB columns, 0 <= x.  Tiles of fewer than 128 columns come in twos (make_unit), x < 3 tB: a division would
+// be 2.5 KB of code in the forward.
+__host__ __device__ inline int div_tile(int x, int tB) { return tB == kTile ? x >> 7 : (x >= tB) + (x >= 2 * tB); }
 static_assert(kTile == 128, "div_tile");
 
 constexpr int kViewShift = 28;   // of the view in a record's head: no look-up in front of a unit's first loads

@@ -9,12 +9,16 @@
 // attend to key t are the same two ranges; dK/dV therefore need no atomics.
 //
 // A block takes 32 rows of the order against tiles of 64 columns: [0, P), then the union of the rows' other
-// ranges.  256 threads; a thread forms 2 x 4 scores, the 16 lanes of a half warp share two rows from the scores
-// to the results, so only the loads of a tile need the whole block to meet.  The next tile travels to
-// registers under the arithmetic of this one.  Bound by fp32 multiply-adds fed from shared memory (6 to 8
-// 16-byte reads per 32 of them) and, on small tables, by the latency of a handful of tiles.  One warp per
-// row with global reads of every key took 463 us for the forward and 1540 us for the backward of 2 x 512
-// tokens, 12 heads of 64.
+// ranges.  Two groups of 128 threads take the tiles in turn and add up what they have at the end: a table row's block has
+// two or three tiles, one of the global block as many as there are columns, and those are the last to finish.  A
+// thread forms 4 x 4 scores, the 16 lanes of a half warp share four rows from the scores to the results, so only the loads
+// of a tile need the group to meet.  The first matrix of the next tile travels to registers under the second half of this
+// one, the second under the first half.  A warp leaves out the columns that none of its eight rows counts.
+// Bound by fp32 multiply-adds (2048 clk of an SM's units per full tile of the forward, 3072 and 4096 per side of the backward),
+// then by the 16-byte reads of shared memory that feed them (12 clk per 16 clk of multiply-adds), and on small tables by
+// the latency of a tile.
+// 2 x 512 tokens, 12 heads of 64, forward / backward: 29.4 / 62.8 us; with 2 x 4 scores per thread, one group and
+// every column of a tile 37.4 / 70.8; with one warp per row and global reads of every key 463 / 1540.
 #include <cuda_bf16.h>
 
 #include <mutex>
@@ -35,6 +39,7 @@ static __device__ __align__(256) float g_noalloc_rowdot[kNoAllocMaxRows];
 
 constexpr int kMaxD = 128;
 constexpr int kRows = 32, kCols = 64, kThreads = 256;
+constexpr int kGroup = 128, kMine = kRows / (kGroup / 16);  // threads that share a tile, rows of a thread
 constexpr int kPStride = kCols + 4;
 
 __device__ __forceinline__ float4 load4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
@@ -68,11 +73,16 @@ struct Common {
     TensorRows tr;
 };
 
+// First of this thread's rows of the block (both groups have all of them).
+__device__ __forceinline__ int first_row() { return (int)((threadIdx.x % kGroup) >> 4) * kMine; }
+__device__ __forceinline__ void group_sync() { asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / kGroup), "n"(kGroup) : "memory"); }
+
 // The rows of a block and the column tiles they meet.
 struct RowBlock {
     const int32_t *perm;
     size_t bh;
-    int t0, n, P, b_lo, b_hi, n_a, n_tiles, lo[2], hi[2];  // lo, hi: behind the global block, of this thread's two rows
+    int t0, n, P, b_lo, b_hi, n_a, n_tiles, lo[kMine], hi[kMine];  // lo, hi: behind the global block, of this thread's rows
+    int w_lo, w_hi;                                                // all that its warp's rows count there
     __device__ __forceinline__ int orig(int t) const { return perm ? __ldg(perm + t) : t; }
     __device__ __forceinline__ void tile(int i, int &c0, int &w) const {
         c0 = i < n_a ? i * kCols : b_lo + (i - n_a) * kCols;
@@ -81,6 +91,11 @@ struct RowBlock {
     // does column c (of range A or B) count for row j of this thread?
     __device__ __forceinline__ bool counts(int i, int c, int w_end, int j) const {
         return c < w_end && (i < n_a || (c >= lo[j] && c < hi[j]));
+    }
+    // the columns [k0, k1) of the tile (w columns from c0 on) that count for some row of this warp
+    __device__ __forceinline__ void span(int i, int c0, int w, int &k0, int &k1) const {
+        k0 = i < n_a ? 0 : max(w_lo - c0, 0);
+        k1 = i < n_a ? w : min(w_hi - c0, w);
     }
 };
 __device__ __forceinline__ RowBlock row_block(const Common &c, int b, int h, int blk, int *s_range) {
@@ -102,12 +117,19 @@ __device__ __forceinline__ RowBlock row_block(const Common &c, int b, int h, int
             s_range[1] = umax;
         }
     }
+    int w_lo = 0x7fffffff, w_hi = 0;
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int row = min((int)(threadIdx.x >> 4) * 2 + j, max(r.n - 1, 0));
+    for (int j = 0; j < kMine; ++j) {
+        const int row = min(first_row() + j, max(r.n - 1, 0));
         r.lo[j] = r.n > 0 ? max(slo[row], r.P) : 0;
         r.hi[j] = r.n > 0 ? shi[row] : 0;
+        if (r.hi[j] > r.lo[j]) {
+            w_lo = min(w_lo, r.lo[j]);
+            w_hi = max(w_hi, r.hi[j]);
+        }
     }
+    r.w_lo = __reduce_min_sync(0xffffffffu, w_lo);
+    r.w_hi = __reduce_max_sync(0xffffffffu, w_hi);
     __syncthreads();
     r.b_lo = s_range[0];
     r.b_hi = s_range[1];
@@ -116,53 +138,68 @@ __device__ __forceinline__ RowBlock row_block(const Common &c, int b, int h, int
     return r;
 }
 
-// kN rows of a tensor in registers (float4 chunks dealt over the threads), on their way to shared memory.
+// kN rows of a tensor in registers (float4 chunks dealt over the threads of a group), on their way to shared memory.
 template <int kN, int DP>
 struct Chunks {
-    static constexpr int kPer = kN * DP / 4 / kThreads > 0 ? kN * DP / 4 / kThreads : 1;
+    static constexpr int kPer = kN * DP / 4 / kGroup;
+    static_assert(kPer > 0 && kPer * kGroup * 4 == kN * DP, "every thread has the same number of chunks");
     float4 v[kPer];
     template <typename T>
     __device__ __forceinline__ void load(const T *base, const RowBlock &r, int c0, int n, int d) {
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
-            const int c = threadIdx.x + i * kThreads, row = c / (DP / 4), ch = c % (DP / 4);
+            const int c = threadIdx.x % kGroup + i * kGroup, row = c / (DP / 4), ch = c % (DP / 4);
             v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row < kN && ch * 4 < d) v[i] = load4(base + (size_t)r.orig(c0 + min(row, n - 1)) * d + ch * 4);  // rows past n repeat the last
+            if (ch * 4 < d) v[i] = load4(base + (size_t)r.orig(c0 + min(row, n - 1)) * d + ch * 4);  // rows past n repeat the last
         }
     }
     __device__ __forceinline__ void store(float *s) const {
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
-            const int c = threadIdx.x + i * kThreads, row = c / (DP / 4), ch = c % (DP / 4);
-            if (row < kN) *reinterpret_cast<float4 *>(s + row * (DP + 4) + ch * 4) = v[i];
+            const int c = threadIdx.x % kGroup + i * kGroup, row = c / (DP / 4), ch = c % (DP / 4);
+            *reinterpret_cast<float4 *>(s + row * (DP + 4) + ch * 4) = v[i];
         }
     }
 };
 
-// s[2][4] = rows (2 per thread) of A times columns tx, tx + 16, .. of B, both [., DP + 4] in shared memory
-template <int DP>
-__device__ __forceinline__ void scores(float (&s)[2][4], const float *A, const float *B, int row0, int tx) {
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) s[j][c] = 0.f;
-#pragma unroll 4
+// s[.][kQ0 .. kQ0 + kQn) = this thread's rows of A times columns tx + 16 q of B, both [., DP + 4] in shared memory
+template <int DP, int kQ0, int kQn>
+__device__ __forceinline__ void score_cols(float (&s)[kMine][4], const float *A, const float *B, int row0, int tx) {
+#pragma unroll 1
     for (int e = 0; e < DP; e += 4) {
-        float4 a[2], b[4];
+        float4 a[kMine], b[kQn];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) a[j] = *reinterpret_cast<const float4 *>(A + (row0 + j) * (DP + 4) + e);
+        for (int j = 0; j < kMine; ++j) a[j] = *reinterpret_cast<const float4 *>(A + (row0 + j) * (DP + 4) + e);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) b[c] = *reinterpret_cast<const float4 *>(B + (tx + 16 * c) * (DP + 4) + e);
+        for (int c = 0; c < kQn; ++c) b[c] = *reinterpret_cast<const float4 *>(B + (tx + 16 * (kQ0 + c)) * (DP + 4) + e);
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
+        for (int j = 0; j < kMine; ++j)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                s[j][c] = fmaf(a[j].x, b[c].x, s[j][c]);
-                s[j][c] = fmaf(a[j].y, b[c].y, s[j][c]);
-                s[j][c] = fmaf(a[j].z, b[c].z, s[j][c]);
-                s[j][c] = fmaf(a[j].w, b[c].w, s[j][c]);
+            for (int c = 0; c < kQn; ++c) {
+                float &x = s[j][kQ0 + c];
+                x = fmaf(a[j].x, b[c].x, x);
+                x = fmaf(a[j].y, b[c].y, x);
+                x = fmaf(a[j].z, b[c].z, x);
+                x = fmaf(a[j].w, b[c].w, x);
             }
     }
+}
+// All four groups of 16 columns at once, or those that meet [k0, k1) one by one where that is half the multiply-adds
+// or less (the reads of shared memory are as many for two groups alone as for four together).
+template <int DP>
+__device__ __forceinline__ void scores(float (&s)[kMine][4], const float *A, const float *B, int row0, int tx, int k0, int k1) {
+#pragma unroll
+    for (int j = 0; j < kMine; ++j)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[j][c] = 0.f;
+    if (((k1 + 15) >> 4) - (k0 >> 4) > 2) {
+        score_cols<DP, 0, 4>(s, A, B, row0, tx);
+        return;
+    }
+    if (k0 < 16) score_cols<DP, 0, 1>(s, A, B, row0, tx);
+    if (k0 < 32 && k1 > 16) score_cols<DP, 1, 1>(s, A, B, row0, tx);
+    if (k0 < 48 && k1 > 32) score_cols<DP, 2, 1>(s, A, B, row0, tx);
+    if (k1 > 48) score_cols<DP, 3, 1>(s, A, B, row0, tx);
 }
 // The DP / 16 result columns of a thread: groups of kW at tx * kW + g * 16 * kW.
 template <int DP>
@@ -170,15 +207,15 @@ struct Cols {
     static constexpr int kN = DP / 16, kW = kN < 4 ? kN : 4;
     __device__ static __forceinline__ int col(int tx, int i) { return (i / kW) * 16 * kW + tx * kW + i % kW; }
 };
-// acc[2][DP / 16] += rows of X ([., kPStride], 64 columns) times B [64, DP + 4]
+// acc[.][DP / 16] += rows of X ([., kPStride]) times B [64, DP + 4], over the columns [k0, k1) of X
 template <int DP>
-__device__ __forceinline__ void accumulate(float (&acc)[2][DP / 16], const float *X, const float *B, int row0, int tx) {
+__device__ __forceinline__ void accumulate(float (&acc)[kMine][DP / 16], const float *X, const float *B, int row0, int tx, int k0, int k1) {
     constexpr int kN = Cols<DP>::kN;
-#pragma unroll 2
-    for (int k = 0; k < kCols; k += 4) {
-        float4 x[2];
+#pragma unroll 1
+    for (int k = k0 & ~3; k < k1; k += 4) {
+        float4 x[kMine];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) x[j] = *reinterpret_cast<const float4 *>(X + (row0 + j) * kPStride + k);
+        for (int j = 0; j < kMine; ++j) x[j] = *reinterpret_cast<const float4 *>(X + (row0 + j) * kPStride + k);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const float *brow = B + (k + q) * (DP + 4);
@@ -192,7 +229,7 @@ __device__ __forceinline__ void accumulate(float (&acc)[2][DP / 16], const float
                 b[0] = brow[tx];
             }
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < kMine; ++j) {
                 const float xv = q == 0 ? x[j].x : q == 1 ? x[j].y : q == 2 ? x[j].z : x[j].w;
 #pragma unroll
                 for (int i = 0; i < kN; ++i) acc[j][i] = fmaf(xv, b[i], acc[j][i]);
@@ -230,49 +267,57 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
     extern __shared__ __align__(16) float smem[];
     __shared__ int s_range[2];
     ptx::wait_prior_grid();
-    float *sQ = smem, *sK = sQ + kRows * (DP + 4), *sV = sK + kCols * (DP + 4), *sP = sV + kCols * (DP + 4);
+    constexpr int kC = kCols * (DP + 4), kPart = 2 * kC + kRows * kPStride;
+    const int grp = threadIdx.x / kGroup;
+    float *sQ = smem, *part = sQ + kRows * (DP + 4), *sK = part + grp * kPart, *sV = sK + kC, *sP = sV + kC;
     // row blocks vary slowest: the long ones (global block) come first
     const int bh = blockIdx.x % n_bh, b = bh / H, h = bh % H;
     const RowBlock r = row_block(c, b, h, blockIdx.x / n_bh, s_range);
     pad_rows(c, r, b, O, (T *)nullptr, LSE);
     if (r.n <= 0) return;
-    const int tx = threadIdx.x & 15, row0 = (threadIdx.x >> 4) * 2;
-    const T *Qh = Q + r.bh * c.d, *Kh = K + r.bh * c.d, *Vh = V + r.bh * c.d;
+    const int tx = threadIdx.x & 15, row0 = first_row();
+    const T *Kh = K + r.bh * c.d, *Vh = V + r.bh * c.d;
 
-    Chunks<kCols, DP> nk, nv;
-    int c0 = 0, w = 0;
-    if (r.n_tiles > 0) {
-        r.tile(0, c0, w);
-        nk.load(Kh, r, c0, w, c.d);
-        nv.load(Vh, r, c0, w, c.d);
-    }
-    {
+    if (grp == 0) {
         Chunks<kRows, DP> q;
-        q.load(Qh, r, r.t0, r.n, c.d);
+        q.load(Q + r.bh * c.d, r, r.t0, r.n, c.d);
         q.store(sQ);
     }
-    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, acc[2][DP / 16];
+    Chunks<kCols, DP> next;
+    int c0 = 0, w = 0;
+    if (grp < r.n_tiles) {
+        r.tile(grp, c0, w);
+        next.load(Kh, r, c0, w, c.d);
+    }
+    __syncthreads();  // Q is there
+    float m[kMine], l[kMine], acc[kMine][DP / 16];
 #pragma unroll
-    for (int j = 0; j < 2; ++j)
+    for (int j = 0; j < kMine; ++j) {
+        m[j] = -INFINITY;
+        l[j] = 0.f;
 #pragma unroll
         for (int i = 0; i < DP / 16; ++i) acc[j][i] = 0.f;
+    }
 
 #pragma unroll 1
-    for (int i = 0; i < r.n_tiles; ++i) {
+    for (int i = grp; i < r.n_tiles; i += 2) {
         const int t_c0 = c0, t_end = c0 + w;
-        __syncthreads();  // the tile before has been read
-        nk.store(sK);
-        nv.store(sV);
-        __syncthreads();
-        if (i + 1 < r.n_tiles) {
-            r.tile(i + 1, c0, w);
-            nk.load(Kh, r, c0, w, c.d);
-            nv.load(Vh, r, c0, w, c.d);
+        int k0, k1;
+        r.span(i, c0, w, k0, k1);
+        next.store(sK);  // (K of the tile before was read ahead of the group's last meeting)
+        next.load(Vh, r, c0, w, c.d);
+        group_sync();
+        float s[kMine][4];
+        if (k1 > k0) scores<DP>(s, sQ, sK, row0, tx, k0, k1);
+        next.store(sV);
+        if (i + 2 < r.n_tiles) {
+            r.tile(i + 2, c0, w);
+            next.load(Kh, r, c0, w, c.d);
         }
-        float s[2][4];
-        scores<DP>(s, sQ, sK, row0, tx);
+        group_sync();
+        if (k1 <= k0) continue;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
+        for (int j = 0; j < kMine; ++j) {
             float mx = -INFINITY;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -295,11 +340,38 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
             for (int e = 0; e < DP / 16; ++e) acc[j][e] *= alpha;
         }
         __syncwarp();
-        accumulate<DP>(acc, sP, sV, row0, tx);
+        accumulate<DP>(acc, sP, sV, row0, tx, k0, k1);
         __syncwarp();
     }
+    if (r.n_tiles > 1) {  // the second group's part, through its shared memory
+        float *x = part + kPart + threadIdx.x % kGroup;
+        __syncthreads();
+        if (grp == 1) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < kMine; ++j) {
+                *x = m[j], x += kGroup;
+                *x = l[j], x += kGroup;
+#pragma unroll
+                for (int e = 0; e < DP / 16; ++e) *x = acc[j][e], x += kGroup;
+            }
+        }
+        __syncthreads();
+        if (grp == 0) {
+#pragma unroll
+            for (int j = 0; j < kMine; ++j) {
+                const float m1 = *x, m_new = fmaxf(m[j], m1), base = m_new == -INFINITY ? 0.f : m_new;
+                const float f0 = expf(m[j] - base), f1 = expf(m1 - base);
+                x += kGroup;
+                l[j] = l[j] * f0 + *x * f1, x += kGroup;
+                m[j] = m_new;
+#pragma unroll
+                for (int e = 0; e < DP / 16; ++e) acc[j][e] = acc[j][e] * f0 + *x * f1, x += kGroup;
+            }
+        }
+    }
+    if (grp != 0) return;
+#pragma unroll
+    for (int j = 0; j < kMine; ++j) {
         if (row0 + j >= r.n) continue;
         const int k = r.orig(r.t0 + row0 + j);
         // a valid row attends at least to itself, except in the passes of the row-or-column pattern,
@@ -341,8 +413,11 @@ template <typename T, int DP>
 __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(const BwdArgs<T> a) {
     extern __shared__ __align__(16) float smem[];
     __shared__ int s_range[2];
-    constexpr int kR = kRows * (DP + 4), kC = kCols * (DP + 4), kX = kRows * kPStride;
-    float *sRa = smem, *sRb = sRa + kR, *sCa = sRb + kR, *sCb = sCa + kC, *sP = sCb + kC, *sS = sP + kX, *sVec = sS + kX;
+    __shared__ float s_row[2][kRows];  // LSE, D of the rows (query side)
+    constexpr int kR = kRows * (DP + 4), kC = kCols * (DP + 4), kPart = 2 * kC + kRows * kPStride + 2 * kCols;
+    const int grp = threadIdx.x / kGroup, tid = threadIdx.x % kGroup;
+    float *sRa = smem, *sRb = sRa + kR, *part = sRb + kR, *sCa = part + grp * kPart, *sCb = sCa + kC, *sX = sCb + kC,
+          *sVec = sX + kRows * kPStride;
     const Common &c = a.c;
     const bool key_side = (blockIdx.x & 1) == 0;
     const int bh = (blockIdx.x >> 1) % a.n_bh, b = bh / a.H, h = bh % a.H;
@@ -350,76 +425,105 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
     ptx::wait_prior_grid();
     pad_rows(c, r, b, key_side ? a.dK : a.dQ, key_side ? a.dV : (T *)nullptr, (float *)nullptr);
     if (r.n <= 0) return;
-    const int tx = threadIdx.x & 15, row0 = (threadIdx.x >> 4) * 2;
-    const T *Ra = (key_side ? a.K : a.Q) + r.bh * c.d, *Rb = (key_side ? a.V : a.dO) + r.bh * c.d;
+    const int tx = threadIdx.x & 15, row0 = first_row();
     const T *Ca = (key_side ? a.Q : a.K) + r.bh * c.d, *Cb = (key_side ? a.dO : a.V) + r.bh * c.d;
 
-    Chunks<kCols, DP> na, nb;
-    float n_lse = 0.f, n_D = 0.f;  // of column threadIdx.x of the next tile (key side)
+    {
+        Chunks<kRows, DP> x;  // one matrix by each group
+        x.load((grp ? (key_side ? a.V : a.dO) : (key_side ? a.K : a.Q)) + r.bh * c.d, r, r.t0, r.n, c.d);
+        x.store(grp ? sRb : sRa);
+    }
+    Chunks<kCols, DP> next;
+    float n_lse = 0.f, n_D = 0.f;  // of column tid of the next tile (key side)
     int c0 = 0, w = 0;
     auto fetch = [&](int i) {
         r.tile(i, c0, w);
-        na.load(Ca, r, c0, w, c.d);
-        nb.load(Cb, r, c0, w, c.d);
-        if (key_side && threadIdx.x < kCols) {
-            const size_t at = r.bh + r.orig(c0 + min((int)threadIdx.x, w - 1));
+        next.load(Ca, r, c0, w, c.d);
+        if (key_side && tid < kCols) {
+            const size_t at = r.bh + r.orig(c0 + min(tid, w - 1));
             n_lse = a.LSE[at];
             n_D = a.D[at];
         }
     };
-    {
-        Chunks<kRows, DP> x, y;
-        x.load(Ra, r, r.t0, r.n, c.d);
-        y.load(Rb, r, r.t0, r.n, c.d);
-        x.store(sRa);
-        y.store(sRb);
+    if (grp < r.n_tiles) fetch(grp);
+    if (!key_side && threadIdx.x < kRows) {
+        const size_t at = r.bh + r.orig(r.t0 + min((int)threadIdx.x, r.n - 1));
+        s_row[0][threadIdx.x] = a.LSE[at];
+        s_row[1][threadIdx.x] = a.D[at];
     }
-    if (r.n_tiles > 0) fetch(0);
-    float lse[2], D[2], acc0[2][DP / 16], acc1[2][DP / 16];
+    float acc0[kMine][DP / 16], acc1[kMine][DP / 16];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const size_t at = r.bh + r.orig(r.t0 + min(row0 + j, r.n - 1));
-        lse[j] = a.LSE[at];
-        D[j] = a.D[at];
+    for (int j = 0; j < kMine; ++j)
 #pragma unroll
         for (int i = 0; i < DP / 16; ++i) acc0[j][i] = acc1[j][i] = 0.f;
-    }
+    __syncthreads();  // the rows are there
 
 #pragma unroll 1
-    for (int i = 0; i < r.n_tiles; ++i) {
-        const int t_c0 = c0, t_end = c0 + w;
-        __syncthreads();  // the tile before has been read
-        na.store(sCa);
-        nb.store(sCb);
-        if (key_side && threadIdx.x < kCols) {
-            sVec[threadIdx.x] = n_lse;
-            sVec[kCols + threadIdx.x] = n_D;
+    for (int i = grp; i < r.n_tiles; i += 2) {
+        const int t_c0 = c0, t_w = w, t_end = c0 + w;
+        int k0, k1;
+        r.span(i, c0, w, k0, k1);
+        group_sync();  // the tile before has been read
+        next.store(sCa);
+        if (key_side && tid < kCols) {
+            sVec[tid] = n_lse;
+            sVec[kCols + tid] = n_D;
+        }
+        next.load(Cb, r, t_c0, t_w, c.d);
+        group_sync();
+        float s[kMine][4], dp[kMine][4];
+        if (k1 > k0) scores<DP>(s, sRa, sCa, row0, tx, k0, k1);
+        next.store(sCb);
+        group_sync();
+        if (k1 > k0) {
+            scores<DP>(dp, sRb, sCb, row0, tx, k0, k1);
+#pragma unroll
+            for (int j = 0; j < kMine; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int col = tx + 16 * q;
+                    const float lse = key_side ? sVec[col] : s_row[0][row0 + j], D = key_side ? sVec[kCols + col] : s_row[1][row0 + j];
+                    const bool on = r.counts(i, t_c0 + col, t_end, j);
+                    const float p = on ? expf(c.scale * s[j][q] - lse) : 0.f;
+                    s[j][q] = p;
+                    sX[(row0 + j) * kPStride + col] = on ? p * (dp[j][q] - D) : 0.f;
+                }
+        }
+        if (i + 2 < r.n_tiles) fetch(i + 2);  // (no earlier: registers)
+        if (k1 <= k0) continue;
+        __syncwarp();
+        accumulate<DP>(acc0, sX, sCa, row0, tx, k0, k1);
+        __syncwarp();
+        if (key_side) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int j = 0; j < kMine; ++j) sX[(row0 + j) * kPStride + tx + 16 * q] = s[j][q];
+            __syncwarp();
+            accumulate<DP>(acc1, sX, sCb, row0, tx, k0, k1);
+            __syncwarp();
+        }
+    }
+    if (r.n_tiles > 1) {  // the second group's part, through its shared memory
+        float *x = part + kPart + tid;
+        __syncthreads();
+        if (grp == 1) {
+#pragma unroll
+            for (int j = 0; j < kMine; ++j)
+#pragma unroll
+                for (int e = 0; e < DP / 16; ++e, x += 2 * kGroup) x[0] = acc0[j][e], x[kGroup] = acc1[j][e];
         }
         __syncthreads();
-        if (i + 1 < r.n_tiles) fetch(i + 1);
-        float s[2][4], dp[2][4];
-        scores<DP>(s, sRa, sCa, row0, tx);
-        scores<DP>(dp, sRb, sCb, row0, tx);
+        if (grp == 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int col = tx + 16 * q;
-            const float c_lse = key_side ? sVec[col] : 0.f, c_D = key_side ? sVec[kCols + col] : 0.f;
+            for (int j = 0; j < kMine; ++j)
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const bool on = r.counts(i, t_c0 + col, t_end, j);
-                const float p = on ? expf(c.scale * s[j][q] - (key_side ? c_lse : lse[j])) : 0.f;
-                const float ds = on ? p * (dp[j][q] - (key_side ? c_D : D[j])) : 0.f;
-                if (key_side) sP[(row0 + j) * kPStride + col] = p;
-                sS[(row0 + j) * kPStride + col] = ds;
-            }
+                for (int e = 0; e < DP / 16; ++e, x += 2 * kGroup) acc0[j][e] += x[0], acc1[j][e] += x[kGroup];
         }
-        __syncwarp();
-        accumulate<DP>(acc0, sS, sCa, row0, tx);
-        if (key_side) accumulate<DP>(acc1, sP, sCb, row0, tx);
-        __syncwarp();
     }
+    if (grp != 0) return;
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
+    for (int j = 0; j < kMine; ++j) {
         if (row0 + j >= r.n) continue;
         const size_t at = (r.bh + r.orig(r.t0 + row0 + j)) * c.d;
         store_row<T, DP>((key_side ? a.dK : a.dQ) + at, acc0[j], c.scale, tx, c.d);
@@ -448,7 +552,7 @@ template <typename T, int DP>
 int fwd_launch(const mate_plan_t *pl, const void *Q, const void *K, const void *V, int d, float scale, void *O, float *LSE,
                int view_order, cudaStream_t st) {
     static SmemAttrOnce attr;
-    constexpr int bytes = 4 * ((kRows + 2 * kCols) * (DP + 4) + kRows * kPStride);
+    constexpr int bytes = 4 * ((kRows + 4 * kCols) * (DP + 4) + 2 * kRows * kPStride);
     if (attr.ensure((const void *)simt_fwd_kernel<T, DP>, bytes, pl->device) != MATE_OK) return MATE_ERR_CUDA;
     return launch_after(simt_fwd_kernel<T, DP>, dim3((unsigned)n_blocks(pl)), kThreads, bytes, st, (const T *)Q, (const T *)K, (const T *)V,
                         (T *)O, LSE, common(pl, d, scale, view_order), pl->H, pl->B * pl->H) == cudaSuccess
@@ -459,7 +563,7 @@ template <typename T, int DP>
 int bwd_launch(const mate_plan_t *pl, const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
                int d, float scale, void *dQ, void *dK, void *dV, float *D, int pass, cudaStream_t st) {
     static SmemAttrOnce attr;
-    constexpr int bytes = 4 * (2 * (kRows + kCols) * (DP + 4) + 2 * kRows * kPStride + 2 * kCols);
+    constexpr int bytes = 4 * (2 * (kRows + 2 * kCols) * (DP + 4) + 2 * kRows * kPStride + 4 * kCols);
     if (attr.ensure((const void *)simt_bwd_kernel<T, DP>, bytes, pl->device) != MATE_OK) return MATE_ERR_CUDA;
     const size_t rows = pl->n_rows();
     if (pass == 0 && launch_after(simt_rowdot_kernel<T>, dim3((unsigned)((rows + kThreads / 16 - 1) / (kThreads / 16))), kThreads, 0, st,

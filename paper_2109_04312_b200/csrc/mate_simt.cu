@@ -17,8 +17,9 @@
 // Bound by fp32 multiply-adds (2048 clk of an SM's units per full tile of the forward, 3072 and 4096 per side of the backward),
 // then by the 16-byte reads of shared memory that feed them (12 clk per 16 clk of multiply-adds), and on small tables by
 // the latency of a tile.
-// 2 x 512 tokens, 12 heads of 64, forward / backward: 29.4 / 62.8 us; with 2 x 4 scores per thread, one group and
-// every column of a tile 37.4 / 70.8; with one warp per row and global reads of every key 463 / 1540.
+// 2 x 512 tokens, 12 heads of 64, forward / backward: 25.2 / 54.7 us; with the rows' look-ups directly in front of the loads
+// that need them 29.4 / 62.8 (a warp waited 2.2 times as long for global memory as it issued); with 2 x 4 scores per thread,
+// one group and every column of a tile 37.4 / 70.8; with one warp per row and global reads of every key 463 / 1540.
 #include <cuda_bf16.h>
 
 #include <mutex>
@@ -144,13 +145,14 @@ struct Chunks {
     static constexpr int kPer = kN * DP / 4 / kGroup;
     static_assert(kPer > 0 && kPer * kGroup * 4 == kN * DP, "every thread has the same number of chunks");
     float4 v[kPer];
+    // s_at: the rows of the tensor, in shared memory
     template <typename T>
-    __device__ __forceinline__ void load(const T *base, const RowBlock &r, int c0, int n, int d) {
+    __device__ __forceinline__ void load(const T *base, const int *s_at, int d) {
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
             const int c = threadIdx.x % kGroup + i * kGroup, row = c / (DP / 4), ch = c % (DP / 4);
             v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (ch * 4 < d) v[i] = load4(base + (size_t)r.orig(c0 + min(row, n - 1)) * d + ch * 4);  // rows past n repeat the last
+            if (ch * 4 < d) v[i] = load4(base + (size_t)s_at[row] * d + ch * 4);
         }
     }
     __device__ __forceinline__ void store(float *s) const {
@@ -265,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1)
 simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V, T *__restrict__ O,
                 float *__restrict__ LSE, const Common c, int H, int n_bh) {
     extern __shared__ __align__(16) float smem[];
-    __shared__ int s_range[2];
+    __shared__ int s_range[2], s_col[2][kCols], s_own[kRows];  // original rows of each group's tile, of the block
     ptx::wait_prior_grid();
     constexpr int kC = kCols * (DP + 4), kPart = 2 * kC + kRows * kPStride;
     const int grp = threadIdx.x / kGroup;
@@ -278,16 +280,21 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
     const int tx = threadIdx.x & 15, row0 = first_row();
     const T *Kh = K + r.bh * c.d, *Vh = V + r.bh * c.d;
 
-    if (grp == 0) {
-        Chunks<kRows, DP> q;
-        q.load(Q + r.bh * c.d, r, r.t0, r.n, c.d);
-        q.store(sQ);
-    }
-    Chunks<kCols, DP> next;
+    const int tid = threadIdx.x % kGroup;
+    int *at = s_col[grp];
     int c0 = 0, w = 0;
     if (grp < r.n_tiles) {
         r.tile(grp, c0, w);
-        next.load(Kh, r, c0, w, c.d);
+        if (tid < kCols) at[tid] = r.orig(c0 + min(tid, w - 1));
+    }
+    if (tid >= kCols && tid < kCols + kRows && grp == 0) s_own[tid - kCols] = r.orig(r.t0 + min(tid - kCols, r.n - 1));
+    __syncthreads();
+    Chunks<kCols, DP> next;
+    if (grp < r.n_tiles) next.load(Kh, at, c.d);
+    if (grp == 0) {
+        Chunks<kRows, DP> q;
+        q.load(Q + r.bh * c.d, s_own, c.d);
+        q.store(sQ);
     }
     __syncthreads();  // Q is there
     float m[kMine], l[kMine], acc[kMine][DP / 16];
@@ -305,16 +312,19 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
         int k0, k1;
         r.span(i, c0, w, k0, k1);
         next.store(sK);  // (K of the tile before was read ahead of the group's last meeting)
-        next.load(Vh, r, c0, w, c.d);
+        next.load(Vh, at, c.d);
+        int next_at = 0;  // look-ups for the tile after this one, a phase ahead of the loads that need them
+        if (i + 2 < r.n_tiles) {
+            r.tile(i + 2, c0, w);
+            if (tid < kCols) next_at = r.orig(c0 + min(tid, w - 1));
+        }
         group_sync();
         float s[kMine][4];
         if (k1 > k0) scores<DP>(s, sQ, sK, row0, tx, k0, k1);
         next.store(sV);
-        if (i + 2 < r.n_tiles) {
-            r.tile(i + 2, c0, w);
-            next.load(Kh, r, c0, w, c.d);
-        }
+        if (tid < kCols) at[tid] = next_at;
         group_sync();
+        if (i + 2 < r.n_tiles) next.load(Kh, at, c.d);
         if (k1 <= k0) continue;
 #pragma unroll
         for (int j = 0; j < kMine; ++j) {
@@ -373,7 +383,7 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
 #pragma unroll
     for (int j = 0; j < kMine; ++j) {
         if (row0 + j >= r.n) continue;
-        const int k = r.orig(r.t0 + row0 + j);
+        const int k = s_own[row0 + j];
         // a valid row attends at least to itself, except in the passes of the row-or-column pattern,
         // where a row may have no key at all: O = 0, LSE = -inf
         store_row<T, DP>(O + (r.bh + k) * c.d, acc[j], l[j] > 0.f ? 1.f / l[j] : 0.f, tx, c.d);
@@ -412,8 +422,8 @@ struct BwdArgs {
 template <typename T, int DP>
 __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(const BwdArgs<T> a) {
     extern __shared__ __align__(16) float smem[];
-    __shared__ int s_range[2];
-    __shared__ float s_row[2][kRows];  // LSE, D of the rows (query side)
+    __shared__ int s_range[2], s_col[2][kCols], s_own[kRows];  // original rows of each group's tile, of the block
+    __shared__ float s_row[2][kRows];                          // LSE, D of the block's rows (query side)
     constexpr int kR = kRows * (DP + 4), kC = kCols * (DP + 4), kPart = 2 * kC + kRows * kPStride + 2 * kCols;
     const int grp = threadIdx.x / kGroup, tid = threadIdx.x % kGroup;
     float *sRa = smem, *sRb = sRa + kR, *part = sRb + kR, *sCa = part + grp * kPart, *sCb = sCa + kC, *sX = sCb + kC,
@@ -428,28 +438,33 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
     const int tx = threadIdx.x & 15, row0 = first_row();
     const T *Ca = (key_side ? a.Q : a.K) + r.bh * c.d, *Cb = (key_side ? a.dO : a.V) + r.bh * c.d;
 
-    {
-        Chunks<kRows, DP> x;  // one matrix by each group
-        x.load((grp ? (key_side ? a.V : a.dO) : (key_side ? a.K : a.Q)) + r.bh * c.d, r, r.t0, r.n, c.d);
-        x.store(grp ? sRb : sRa);
+    int *at = s_col[grp];
+    int c0 = 0, w = 0, next_at = 0;  // next_at: original row of column tid of the next tile
+    if (grp < r.n_tiles) {
+        r.tile(grp, c0, w);
+        if (tid < kCols) at[tid] = next_at = r.orig(c0 + min(tid, w - 1));
     }
+    if (grp == 0 && tid >= kCols && tid < kCols + kRows) {
+        const int row = tid - kCols, k = r.orig(r.t0 + min(row, r.n - 1));
+        s_own[row] = k;
+        s_row[0][row] = a.LSE[r.bh + k];
+        s_row[1][row] = a.D[r.bh + k];
+    }
+    __syncthreads();
     Chunks<kCols, DP> next;
-    float n_lse = 0.f, n_D = 0.f;  // of column tid of the next tile (key side)
-    int c0 = 0, w = 0;
-    auto fetch = [&](int i) {
-        r.tile(i, c0, w);
-        next.load(Ca, r, c0, w, c.d);
+    float n_lse = 0.f, n_D = 0.f;  // of that row (key side)
+    auto fetch = [&]() {
+        next.load(Ca, at, c.d);
         if (key_side && tid < kCols) {
-            const size_t at = r.bh + r.orig(c0 + min(tid, w - 1));
-            n_lse = a.LSE[at];
-            n_D = a.D[at];
+            n_lse = a.LSE[r.bh + next_at];
+            n_D = a.D[r.bh + next_at];
         }
     };
-    if (grp < r.n_tiles) fetch(grp);
-    if (!key_side && threadIdx.x < kRows) {
-        const size_t at = r.bh + r.orig(r.t0 + min((int)threadIdx.x, r.n - 1));
-        s_row[0][threadIdx.x] = a.LSE[at];
-        s_row[1][threadIdx.x] = a.D[at];
+    if (grp < r.n_tiles) fetch();
+    {
+        Chunks<kRows, DP> x;  // one matrix by each group
+        x.load((grp ? (key_side ? a.V : a.dO) : (key_side ? a.K : a.Q)) + r.bh * c.d, s_own, c.d);
+        x.store(grp ? sRb : sRa);
     }
     float acc0[kMine][DP / 16], acc1[kMine][DP / 16];
 #pragma unroll
@@ -460,7 +475,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
 
 #pragma unroll 1
     for (int i = grp; i < r.n_tiles; i += 2) {
-        const int t_c0 = c0, t_w = w, t_end = c0 + w;
+        const int t_c0 = c0, t_end = c0 + w;
         int k0, k1;
         r.span(i, c0, w, k0, k1);
         group_sync();  // the tile before has been read
@@ -469,11 +484,16 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
             sVec[tid] = n_lse;
             sVec[kCols + tid] = n_D;
         }
-        next.load(Cb, r, t_c0, t_w, c.d);
+        next.load(Cb, at, c.d);
+        if (i + 2 < r.n_tiles) {  // look-ups for the tile after this one, a phase ahead of the loads that need them
+            r.tile(i + 2, c0, w);
+            if (tid < kCols) next_at = r.orig(c0 + min(tid, w - 1));
+        }
         group_sync();
         float s[kMine][4], dp[kMine][4];
         if (k1 > k0) scores<DP>(s, sRa, sCa, row0, tx, k0, k1);
         next.store(sCb);
+        if (tid < kCols) at[tid] = next_at;
         group_sync();
         if (k1 > k0) {
             scores<DP>(dp, sRb, sCb, row0, tx, k0, k1);
@@ -489,7 +509,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
                     sX[(row0 + j) * kPStride + col] = on ? p * (dp[j][q] - D) : 0.f;
                 }
         }
-        if (i + 2 < r.n_tiles) fetch(i + 2);  // (no earlier: registers)
+        if (i + 2 < r.n_tiles) fetch();  // (no earlier: registers)
         if (k1 <= k0) continue;
         __syncwarp();
         accumulate<DP>(acc0, sX, sCa, row0, tx, k0, k1);
@@ -525,9 +545,9 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
 #pragma unroll
     for (int j = 0; j < kMine; ++j) {
         if (row0 + j >= r.n) continue;
-        const size_t at = (r.bh + r.orig(r.t0 + row0 + j)) * c.d;
-        store_row<T, DP>((key_side ? a.dK : a.dQ) + at, acc0[j], c.scale, tx, c.d);
-        if (key_side) store_row<T, DP>(a.dV + at, acc1[j], 1.f, tx, c.d);
+        const size_t o = (r.bh + s_own[row0 + j]) * c.d;
+        store_row<T, DP>((key_side ? a.dK : a.dQ) + o, acc0[j], c.scale, tx, c.d);
+        if (key_side) store_row<T, DP>(a.dV + o, acc1[j], 1.f, tx, c.d);
     }
 }
 

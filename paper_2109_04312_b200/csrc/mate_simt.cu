@@ -14,10 +14,10 @@
 // thread forms 4 x 4 scores, the 16 lanes of a half warp share four rows from the scores to the results, so only the loads
 // of a tile need the group to meet.  The first matrix of the next tile travels to registers under the second half of this
 // one, the second under the first half.  A warp leaves out the columns that none of its eight rows counts.
-// Bound by fp32 multiply-adds (2048 clk of an SM's units per full tile of the forward, 3072 and 4096 per side of the backward),
-// then by the 16-byte reads of shared memory that feed them (12 clk per 16 clk of multiply-adds), and on small tables by
-// the latency of a tile.
-// 2 x 512 tokens, 12 heads of 64, forward / backward: 25.2 / 54.7 us; with the rows' look-ups directly in front of the loads
+// Bound by latency (16 warps per SM at the registers this takes): with 8 x 512 tokens issue slots are 49 % busy, the
+// multiply-add units 26 %, shared memory 32 %; two global loads and three hand-overs per tile are what a warp waits for.
+// 2 x 512 tokens, 12 heads of 64, forward / backward: 24.4 / 53.1 us; with the rows' key ranges in registers
+// (24 of them spilled in the backward) 25.2 / 54.7; with the rows' look-ups directly in front of the loads
 // that need them 29.4 / 62.8 (a warp waited 2.2 times as long for global memory as it issued); with 2 x 4 scores per thread,
 // one group and every column of a tile 37.4 / 70.8; with one warp per row and global reads of every key 463 / 1540.
 #include <cuda_bf16.h>
@@ -78,64 +78,72 @@ struct Common {
 __device__ __forceinline__ int first_row() { return (int)((threadIdx.x % kGroup) >> 4) * kMine; }
 __device__ __forceinline__ void group_sync() { asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / kGroup), "n"(kGroup) : "memory"); }
 
-// The rows of a block and the column tiles they meet.
+// The rows of a block and the column tiles they meet.  What is needed once a tile stays in shared memory (registers
+// are what the backward is short of: of 128 with heads of 64, 24 spilled with the ranges in them, 14 without).
 struct RowBlock {
+    struct Shared {
+        int P, b_lo, b_hi, lo[kRows], hi[kRows];  // lo, hi: behind the global block
+    };
     const int32_t *perm;
+    const Shared *s;
     size_t bh;
-    int t0, n, P, b_lo, b_hi, n_a, n_tiles, lo[kMine], hi[kMine];  // lo, hi: behind the global block, of this thread's rows
-    int w_lo, w_hi;                                                // all that its warp's rows count there
+    int t0, n, n_tiles;
+    int w_lo, w_hi;  // all that the rows of this thread's warp count behind the global block
     __device__ __forceinline__ int orig(int t) const { return perm ? __ldg(perm + t) : t; }
+    __device__ __forceinline__ int n_a() const { return (s->P + kCols - 1) / kCols; }
+    // tile i: w columns from c0 on, of which [k0, k1) count for some row of this warp
     __device__ __forceinline__ void tile(int i, int &c0, int &w) const {
-        c0 = i < n_a ? i * kCols : b_lo + (i - n_a) * kCols;
-        w = min(kCols, (i < n_a ? P : b_hi) - c0);
+        const int na = n_a();
+        c0 = i < na ? i * kCols : s->b_lo + (i - na) * kCols;
+        w = min(kCols, (i < na ? s->P : s->b_hi) - c0);
     }
-    // does column c (of range A or B) count for row j of this thread?
-    __device__ __forceinline__ bool counts(int i, int c, int w_end, int j) const {
-        return c < w_end && (i < n_a || (c >= lo[j] && c < hi[j]));
-    }
-    // the columns [k0, k1) of the tile (w columns from c0 on) that count for some row of this warp
     __device__ __forceinline__ void span(int i, int c0, int w, int &k0, int &k1) const {
-        k0 = i < n_a ? 0 : max(w_lo - c0, 0);
-        k1 = i < n_a ? w : min(w_hi - c0, w);
+        const bool a = i < n_a();
+        k0 = a ? 0 : max(w_lo - c0, 0);
+        k1 = a ? w : min(w_hi - c0, w);
+    }
+    // the columns of tile i that count for a row of the block: [lo, hi)
+    __device__ __forceinline__ void row_span(int i, int c0, int w, int row, int &lo, int &hi) const {
+        const bool a = i < n_a();
+        lo = a ? 0 : s->lo[row] - c0;
+        hi = a ? w : min(s->hi[row] - c0, w);
     }
 };
-__device__ __forceinline__ RowBlock row_block(const Common &c, int b, int h, int blk, int *s_range) {
+__device__ __forceinline__ RowBlock row_block(const Common &c, int b, int h, int blk, RowBlock::Shared *sh) {
     const ViewPlan &vp = c.head_view[h] ? c.colv : c.rowv;
     RowBlock r;
     r.perm = c.view_order ? nullptr : vp.perm + (size_t)b * c.N;
+    r.s = sh;
     r.bh = c.tr.base(b, h);
     r.t0 = blk * kRows;
-    const int nv = c.n_valid[b];
+    const int nv = c.n_valid[b], P = min(c.prefix[b], nv);
     r.n = min(kRows, nv - r.t0);  // valid rows of the block (<= 0: padding only)
-    r.P = min(c.prefix[b], nv);
     const int32_t *slo = vp.seg_lo + (size_t)b * c.N + r.t0, *shi = vp.seg_hi + (size_t)b * c.N + r.t0;
-    if (threadIdx.x < 32) {  // union of the rows' ranges behind the global block
-        const bool on = (int)threadIdx.x < r.n;
-        const int l = on ? max(slo[threadIdx.x], r.P) : 0x7fffffff, u = on ? shi[threadIdx.x] : 0;
+    if (threadIdx.x < kRows) {  // (rows past the last valid one repeat it)
+        const int row = min((int)threadIdx.x, r.n - 1);
+        const int l = r.n > 0 ? max(slo[row], P) : 0, u = r.n > 0 ? shi[row] : 0;
         const int lmin = __reduce_min_sync(0xffffffffu, u > l ? l : 0x7fffffff), umax = __reduce_max_sync(0xffffffffu, u > l ? u : 0);
+        sh->lo[threadIdx.x] = l;
+        sh->hi[threadIdx.x] = u;
         if (threadIdx.x == 0) {
-            s_range[0] = lmin;
-            s_range[1] = umax;
+            sh->P = P;
+            sh->b_lo = lmin;
+            sh->b_hi = umax;
         }
     }
+    __syncthreads();
     int w_lo = 0x7fffffff, w_hi = 0;
 #pragma unroll
     for (int j = 0; j < kMine; ++j) {
-        const int row = min(first_row() + j, max(r.n - 1, 0));
-        r.lo[j] = r.n > 0 ? max(slo[row], r.P) : 0;
-        r.hi[j] = r.n > 0 ? shi[row] : 0;
-        if (r.hi[j] > r.lo[j]) {
-            w_lo = min(w_lo, r.lo[j]);
-            w_hi = max(w_hi, r.hi[j]);
+        const int l = sh->lo[first_row() + j], u = sh->hi[first_row() + j];
+        if (u > l) {
+            w_lo = min(w_lo, l);
+            w_hi = max(w_hi, u);
         }
     }
     r.w_lo = __reduce_min_sync(0xffffffffu, w_lo);
     r.w_hi = __reduce_max_sync(0xffffffffu, w_hi);
-    __syncthreads();
-    r.b_lo = s_range[0];
-    r.b_hi = s_range[1];
-    r.n_a = (r.P + kCols - 1) / kCols;
-    r.n_tiles = r.n_a + (r.b_hi > r.b_lo ? (r.b_hi - r.b_lo + kCols - 1) / kCols : 0);
+    r.n_tiles = r.n_a() + (sh->b_hi > sh->b_lo ? (sh->b_hi - sh->b_lo + kCols - 1) / kCols : 0);
     return r;
 }
 
@@ -167,7 +175,7 @@ struct Chunks {
 // s[.][kQ0 .. kQ0 + kQn) = this thread's rows of A times columns tx + 16 q of B, both [., DP + 4] in shared memory
 template <int DP, int kQ0, int kQn>
 __device__ __forceinline__ void score_cols(float (&s)[kMine][4], const float *A, const float *B, int row0, int tx) {
-#pragma unroll 1
+#pragma unroll (DP > 64 ? 2 : 1)
     for (int e = 0; e < DP; e += 4) {
         float4 a[kMine], b[kQn];
 #pragma unroll
@@ -213,7 +221,7 @@ struct Cols {
 template <int DP>
 __device__ __forceinline__ void accumulate(float (&acc)[kMine][DP / 16], const float *X, const float *B, int row0, int tx, int k0, int k1) {
     constexpr int kN = Cols<DP>::kN;
-#pragma unroll 1
+#pragma unroll 2
     for (int k = k0 & ~3; k < k1; k += 4) {
         float4 x[kMine];
 #pragma unroll
@@ -267,14 +275,15 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1)
 simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V, T *__restrict__ O,
                 float *__restrict__ LSE, const Common c, int H, int n_bh) {
     extern __shared__ __align__(16) float smem[];
-    __shared__ int s_range[2], s_col[2][kCols], s_own[kRows];  // original rows of each group's tile, of the block
+    __shared__ RowBlock::Shared s_rows;
+    __shared__ int s_col[2][kCols], s_own[kRows];  // original rows of each group's tile, of the block
     ptx::wait_prior_grid();
     constexpr int kC = kCols * (DP + 4), kPart = 2 * kC + kRows * kPStride;
     const int grp = threadIdx.x / kGroup;
     float *sQ = smem, *part = sQ + kRows * (DP + 4), *sK = part + grp * kPart, *sV = sK + kC, *sP = sV + kC;
     // row blocks vary slowest: the long ones (global block) come first
     const int bh = blockIdx.x % n_bh, b = bh / H, h = bh % H;
-    const RowBlock r = row_block(c, b, h, blockIdx.x / n_bh, s_range);
+    const RowBlock r = row_block(c, b, h, blockIdx.x / n_bh, &s_rows);
     pad_rows(c, r, b, O, (T *)nullptr, LSE);
     if (r.n <= 0) return;
     const int tx = threadIdx.x & 15, row0 = first_row();
@@ -308,7 +317,7 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
 
 #pragma unroll 1
     for (int i = grp; i < r.n_tiles; i += 2) {
-        const int t_c0 = c0, t_end = c0 + w;
+        const int t_c0 = c0, t_w = w;
         int k0, k1;
         r.span(i, c0, w, k0, k1);
         next.store(sK);  // (K of the tile before was read ahead of the group's last meeting)
@@ -329,9 +338,12 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
 #pragma unroll
         for (int j = 0; j < kMine; ++j) {
             float mx = -INFINITY;
+            int lo, hi;
+            r.row_span(i, t_c0, t_w, row0 + j, lo, hi);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                s[j][q] = r.counts(i, t_c0 + tx + 16 * q, t_end, j) ? c.scale * s[j][q] : -INFINITY;
+                const int col = tx + 16 * q;
+                s[j][q] = col >= lo && col < hi ? c.scale * s[j][q] : -INFINITY;
                 mx = fmaxf(mx, s[j][q]);
             }
             const float m_new = fmaxf(m[j], half_max(mx));
@@ -422,7 +434,8 @@ struct BwdArgs {
 template <typename T, int DP>
 __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(const BwdArgs<T> a) {
     extern __shared__ __align__(16) float smem[];
-    __shared__ int s_range[2], s_col[2][kCols], s_own[kRows];  // original rows of each group's tile, of the block
+    __shared__ RowBlock::Shared s_rows;
+    __shared__ int s_col[2][kCols], s_own[kRows];  // original rows of each group's tile, of the block
     __shared__ float s_row[2][kRows];                          // LSE, D of the block's rows (query side)
     constexpr int kR = kRows * (DP + 4), kC = kCols * (DP + 4), kPart = 2 * kC + kRows * kPStride + 2 * kCols;
     const int grp = threadIdx.x / kGroup, tid = threadIdx.x % kGroup;
@@ -431,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
     const Common &c = a.c;
     const bool key_side = (blockIdx.x & 1) == 0;
     const int bh = (blockIdx.x >> 1) % a.n_bh, b = bh / a.H, h = bh % a.H;
-    const RowBlock r = row_block(c, b, h, (blockIdx.x >> 1) / a.n_bh, s_range);
+    const RowBlock r = row_block(c, b, h, (blockIdx.x >> 1) / a.n_bh, &s_rows);
     ptx::wait_prior_grid();
     pad_rows(c, r, b, key_side ? a.dK : a.dQ, key_side ? a.dV : (T *)nullptr, (float *)nullptr);
     if (r.n <= 0) return;
@@ -475,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
 
 #pragma unroll 1
     for (int i = grp; i < r.n_tiles; i += 2) {
-        const int t_c0 = c0, t_end = c0 + w;
+        const int t_c0 = c0, t_w = w;
         int k0, k1;
         r.span(i, c0, w, k0, k1);
         group_sync();  // the tile before has been read
@@ -498,16 +511,19 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
         if (k1 > k0) {
             scores<DP>(dp, sRb, sCb, row0, tx, k0, k1);
 #pragma unroll
-            for (int j = 0; j < kMine; ++j)
+            for (int j = 0; j < kMine; ++j) {
+                int lo, hi;
+                r.row_span(i, t_c0, t_w, row0 + j, lo, hi);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int col = tx + 16 * q;
                     const float lse = key_side ? sVec[col] : s_row[0][row0 + j], D = key_side ? sVec[kCols + col] : s_row[1][row0 + j];
-                    const bool on = r.counts(i, t_c0 + col, t_end, j);
+                    const bool on = col >= lo && col < hi;
                     const float p = on ? expf(c.scale * s[j][q] - lse) : 0.f;
                     s[j][q] = p;
                     sX[(row0 + j) * kPStride + col] = on ? p * (dp[j][q] - D) : 0.f;
                 }
+            }
         }
         if (i + 2 < r.n_tiles) fetch();  // (no earlier: registers)
         if (k1 <= k0) continue;

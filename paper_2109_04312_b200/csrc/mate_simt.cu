@@ -16,6 +16,8 @@
 // one, the second under the first half.  A warp leaves out the columns that none of its eight rows counts.
 // Bound by latency (16 warps per SM at the registers this takes): with 8 x 512 tokens issue slots are 49 % busy, the
 // multiply-add units 26 %, shared memory 32 %; two global loads and three hand-overs per tile are what a warp waits for.
+// Two blocks per SM (one with heads of more than 64): three of smaller heads fit, but spill (2 x 512 tokens, heads of 32, 16.2 / 31.9 us
+// with two, 19.8 / 41.4 with three; of 16 12.5 / 24.2, 13.3 / 25.9).
 // 2 x 512 tokens, 12 heads of 64, forward / backward: 24.4 / 53.1 us; with the rows' key ranges in registers
 // (24 of them spilled in the backward) 25.2 / 54.7; with the rows' look-ups directly in front of the loads
 // that need them 29.4 / 62.8 (a warp waited 2.2 times as long for global memory as it issued); with 2 x 4 scores per thread,

@@ -46,6 +46,7 @@
 
 #include <type_traits>
 
+#include "load_ring.h"
 #include "mate_internal.h"
 #include "sm100_ptx.cuh"
 #include "tc_tiles.cuh"
@@ -75,6 +76,8 @@ constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
 // CTA is launched with
 constexpr int kRegsCompute = 168, kRegsStore = 48, kRegsMma = 40, kRegsLoad = 56;
 constexpr int kStages = 4;  // ring of column tiles
+using RowRing = LoadRing<2>;
+using ColRing = LoadRing<kStages>;
 constexpr int kSchedDepth = 4;
 constexpr uint32_t kOffR = 0;                                    // [2 buffers] x (Ra: Q or K, Rb: dO or V), 16 KB each
 constexpr uint32_t kOffC = 4 * kTileBytes;                       // [kStages] x (Ca 16 KB, Cb 16 KB)
@@ -83,25 +86,26 @@ constexpr uint32_t kOffMeta = kOffVec + kStages * 1024;          // [2 buffers] 
 constexpr uint32_t kOffStage = kOffMeta + 2 * 5 * kTile * 4;     // [store warps] x 32 rows x 128 bytes
 constexpr uint32_t kOffItem = kOffStage + kStoreWarps * 4096;    // [kSchedDepth] unit records
 constexpr uint32_t kOffBar = kOffItem + kSchedDepth * sizeof(FwdUnit);
-constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024;            // + slack for the 1024-byte alignment
+constexpr uint32_t kSmemBytes = kOffBar + 512 + 1024;            // + slack for the 1024-byte alignment
 static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 // barrier slots (8 bytes each) behind kOffBar
 enum {
-    kBarRFull = 0,    // [2] loaders -> MMA, arithmetic      (count: warps of a team)
-    kBarREmpty = 2,   // [2] MMA commit and arithmetic warps (row data read) -> loaders (count 1 + kComputeWarps + kStoreWarps)
-    kBarCFull = 4,    // [kStages] loaders -> MMA            (count: warps of a team)
-    kBarCEmpty = 8,   // [kStages] MMA commit -> loaders     (count 1)
-    kBarSFull = 12,   // MMA commit -> arithmetic: S and dP of a tile are complete (count 1)
-    kBarAFull = 13,   // arithmetic -> MMA: the bf16 operands of a tile are written (count: one per warp)
-    kBarGDone = 14,   // MMA commit -> arithmetic: the gradient MMAs of a tile are complete (count 1)
-    kBarSchedFull = 16,   // [kSchedDepth] scheduler -> every warp (count 1)
-    kBarSchedEmpty = 20,  // [kSchedDepth] every warp -> scheduler (count kSchedReaders)
-    kBarSTFree = 24,      // arithmetic -> MMA: S and dP of a tile are in registers (count: one per warp)
-    kBarItemDone = 25,    // MMA commit -> store warps: every gradient MMA of an item is complete (count 1)
-    kBarAccFree = 26,     // store warps -> MMA: the gradients of an item are in registers (count: one per warp)
-    kBarFinal = 27,       // [2]
-    kNumBars = 29
+    kBarRFull = 0,                     // [2] loaders -> MMA, arithmetic      (count: warps of a team)
+    kBarREmpty = kBarRFull + 2,        // [4] MMA commit and arithmetic warps (row data read) -> loaders (count 1 + kComputeWarps + kStoreWarps)
+    kBarCFull = kBarREmpty + RowRing::kEmpty,   // [kStages] loaders -> MMA     (count: warps of a team)
+    kBarCEmpty = kBarCFull + kStages,  // [2 kStages] MMA commit -> loaders   (count 1)
+    kBarSFull = kBarCEmpty + ColRing::kEmpty,   // MMA commit -> arithmetic: S and dP of a tile are complete (count 1)
+    kBarAFull,         // arithmetic -> MMA: the bf16 operands of a tile are written (count: one per warp)
+    kBarGDone,         // MMA commit -> arithmetic: the gradient MMAs of a tile are complete (count 1)
+    kBarSTFree,        // arithmetic -> MMA: S and dP of a tile are in registers (count: one per warp)
+    kBarItemDone,      // MMA commit -> store warps: every gradient MMA of an item is complete (count 1)
+    kBarAccFree,       // store warps -> MMA: the gradients of an item are in registers (count: one per warp)
+    kBarSchedFull,                               // [kSchedDepth] scheduler -> every warp (count 1)
+    kBarSchedEmpty = kBarSchedFull + kSchedDepth,  // [kSchedDepth] every warp -> scheduler (count kSchedReaders)
+    kBarFinal = kBarSchedEmpty + kSchedDepth,      // [2]
+    kNumBars = kBarFinal + 2
 };
+static_assert(8 * kNumBars + 8 <= 512, "the barriers and two words behind them");
 constexpr int kSchedReaders = kComputeWarps + kMmaWarps + kStoreWarps + kLoadWarps;
 // tensor memory columns
 constexpr uint32_t kTmS = 0, kTmT = 128, kTmA1 = 256, kTmA2 = 320, kTmAcc1 = 384, kTmAcc2 = 448;
@@ -262,14 +266,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
     if (warp == kLoadWarp0 + 1 && lane < 8) prefetch_tmap(&p.tmQ + lane);  // all eight of them
 
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(bars + 8 * (kBarRFull + i), kTeamWarps);
-            mbar_init(bars + 8 * (kBarREmpty + i), 1 + kComputeWarps + kStoreWarps);
-        }
-        for (int i = 0; i < kStages; ++i) {
-            mbar_init(bars + 8 * (kBarCFull + i), kTeamWarps);
-            mbar_init(bars + 8 * (kBarCEmpty + i), 1);
-        }
+        for (int i = 0; i < 2; ++i) mbar_init(bars + 8 * (kBarRFull + i), kTeamWarps);
+        for (int i = 0; i < RowRing::kEmpty; ++i) mbar_init(bars + 8 * (kBarREmpty + i), 1 + kComputeWarps + kStoreWarps);
+        for (int i = 0; i < kStages; ++i) mbar_init(bars + 8 * (kBarCFull + i), kTeamWarps);
+        for (int i = 0; i < ColRing::kEmpty; ++i) mbar_init(bars + 8 * (kBarCEmpty + i), 1);
         mbar_init(bars + 8 * kBarSFull, 1);
         mbar_init(bars + 8 * kBarAFull, kComputeWarps);
         mbar_init(bars + 8 * kBarSTFree, kComputeWarps);
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             if (!alive) break;
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive(bars + 8 * (kBarREmpty + rb));
+                mbar_arrive(bars + 8 * (kBarREmpty + RowRing::empty(n)));
                 mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
             }
         }
@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             const int r = q4 * 32 + lane;
             const int dst_row = r < rows_h ? (reinterpret_cast<const int32_t *>(sm + kOffMeta) + rb * 5 * kTile)[r] : -1;
             __syncwarp();
-            if (lane == 0) mbar_arrive(bars + 8 * (kBarREmpty + rb));
+            if (lane == 0) mbar_arrive(bars + 8 * (kBarREmpty + RowRing::empty(n)));
             if (any) {
                 if (!wait(bars + 8 * kBarItemDone, units++ & 1)) break;
                 tc_fence_after();
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                         __syncwarp();
                     }
                     if (!alive) break;
-                    if (leader) mma_commit(bars + 8 * (kBarREmpty + rb));  // the row operands are free once these MMAs are done
+                    if (leader) mma_commit(bars + 8 * (kBarREmpty + RowRing::empty(n)));  // the row operands are free once these MMAs are done
                     __syncwarp();
                 } else {
                     constexpr uint32_t idesc = idesc_bf16(128, 64, 0, 1);  // B = 16 rows of the column tile x 64, MN-major
@@ -625,7 +625,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                                 for (int k = 1; k < ks; ++k) mma_ts_lean<1>(tG1, tA1 + 8 * k, a_lo + k * kStep, idesc);
                             }
                             mma_commit(bars + 8 * kBarGDone);
-                            mma_commit(bars + 8 * (kBarCEmpty + st));
+                            mma_commit(bars + 8 * (kBarCEmpty + ColRing::empty(c_cnt)));
                             if (i + 1 == n_tiles) mma_commit(bars + 8 * kBarItemDone);
                         }
                         __syncwarp();
@@ -685,8 +685,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
 #pragma unroll
                 for (int k = 0; k < kPer; ++k) now[k] = (int)bh + __ldg(perm + (i < 0 ? un.q0 + min(r0 + 32 * k, rows_h - 1) : t.pos(min(r0 + 32 * k, t.w - 1))));
                 const uint32_t c = c_cnt + max(i, 0), st = c % kStages;
-                const uint32_t bar_e = bars + 8 * (i < 0 ? kBarREmpty + rb : kBarCEmpty + st), bar_full = bars + 8 * (i < 0 ? kBarRFull + rb : kBarCFull + st);
-                if (!(alive = wait(bar_e, ((i < 0 ? n >> 1 : c / kStages) & 1) ^ 1))) break;
+                const uint32_t bar_e = bars + 8 * (i < 0 ? kBarREmpty + RowRing::wait_empty(n) : kBarCEmpty + ColRing::wait_empty(c)),
+                               bar_full = bars + 8 * (i < 0 ? kBarRFull + rb : kBarCFull + st);
+                if (!(alive = wait(bar_e, i < 0 ? RowRing::wait_parity(n) : ColRing::wait_parity(c)))) break;
                 if (i < 0) {  // row data for the arithmetic threads
 #pragma unroll
                     for (int k = 0; k < kPer; ++k) {

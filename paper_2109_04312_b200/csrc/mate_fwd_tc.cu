@@ -46,6 +46,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include "load_ring.h"
 #include "mate_internal.h"
 #include "sm100_ptx.cuh"
 #include "tc_tiles.cuh"
@@ -72,6 +73,8 @@ constexpr int kTeamWarps = kLoadWarps / kTeams;
 constexpr int kLoadRows = kTile / kTeamWarps;  // rows of a tile a loader warp fetches
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
 constexpr int kStages = 4;                   // K/V ring
+using QRing = LoadRing<2>;
+using KVRing = LoadRing<kStages>;
 // registers per thread after the roles have split: 256 x 176 + 256 x 80 = 65,536 = the 512 x 128 the CTA is
 // launched with
 constexpr int kRegsSoftmax = 176, kRegsOther = 80;
@@ -95,21 +98,21 @@ constexpr float kSumMin = 0x1p-100f, kSumMax = 0x1p60f;      // row sums outside
 
 // barrier slots (8 bytes each) behind kOffBar
 enum {
-    kBarQFull = 0,        // [2] loaders -> MMA, softmax   (count: warps of a team)
-    kBarQEmpty = 2,       // [2] MMA commits and softmax warps (row data read) -> loaders (count kMmaWarps + kSoftmaxWarps)
-    kBarKVFull = 4,       // [kStages] loaders -> MMA      (count: warps of a team)
-    kBarKVEmpty = 8,      // [kStages] MMA -> loaders      (count 2: one per half)
-    kBarSFull = 12,       // [2] MMA commit -> softmax (count 1)
-    kBarSFree = 14,       // [2] softmax -> MMA: S of a tile has been read (count 4: one per warp)
-    kBarPFull = 16,       // [2] softmax -> MMA        (count 4: one per warp)
-    kBarPVDone = 18,      // [2] MMA commit -> softmax: the P V of a tile is complete (count 1)
-    kBarFinal = 20,       // [2]
-    kBarSchedFull = 22,   // [kSchedDepth] scheduler -> every warp that follows the unit list (count 1)
-    kBarSchedEmpty = 26,  // [kSchedDepth] those warps -> scheduler (count kSchedReaders)
-    kNumBars = 30
+    kBarQFull = 0,                             // [2] loaders -> MMA, softmax   (count: warps of a team)
+    kBarQEmpty = kBarQFull + 2,                // [4] MMA commits and softmax warps (row data read) -> loaders (count kMmaWarps + kSoftmaxWarps)
+    kBarKVFull = kBarQEmpty + QRing::kEmpty,   // [kStages] loaders -> MMA      (count: warps of a team)
+    kBarKVEmpty = kBarKVFull + kStages,        // [2 kStages] MMA -> loaders    (count 2: one per half)
+    kBarSFull = kBarKVEmpty + KVRing::kEmpty,  // [2] MMA commit -> softmax (count 1)
+    kBarSFree = kBarSFull + 2,         // [2] softmax -> MMA: S of a tile has been read (count 4: one per warp)
+    kBarPFull = kBarSFree + 2,         // [2] softmax -> MMA        (count 4: one per warp)
+    kBarPVDone = kBarPFull + 2,        // [2] MMA commit -> softmax: the P V of a tile is complete (count 1)
+    kBarFinal = kBarPVDone + 2,        // [2]
+    kBarSchedFull = kBarFinal + 2,                 // [kSchedDepth] scheduler -> every warp that follows the unit list (count 1)
+    kBarSchedEmpty = kBarSchedFull + kSchedDepth,  // [kSchedDepth] those warps -> scheduler (count kSchedReaders)
+    kNumBars = kBarSchedEmpty + kSchedDepth
 };
+static_assert(8 * kNumBars + 16 + 4 * kSchedDepth <= 512, "the barriers and the words behind them");
 constexpr int kSchedReaders = kSoftmaxWarps + kMmaWarps + kLoadWarps;
-static_assert(kStages == 4, "barrier slots");
 
 // kMany: the three passes of a row-or-column plan.  (An instance of its own: the look-ups by pass cost the others up to 1 %,
 // 4 x 2048 tokens 94.4 -> 95.3 us forward and backward.)
@@ -220,17 +223,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
             mbar_init(bars + 8 * (kBarQFull + i), kTeamWarps);
-            mbar_init(bars + 8 * (kBarQEmpty + i), kMmaWarps + kSoftmaxWarps);
             mbar_init(bars + 8 * (kBarSFull + i), 1);
             mbar_init(bars + 8 * (kBarSFree + i), kSoftmaxWarps / 2);
             mbar_init(bars + 8 * (kBarPFull + i), kSoftmaxWarps / 2);
             mbar_init(bars + 8 * (kBarPVDone + i), 1);
             mbar_init(bars + 8 * (kBarFinal + i), 1);
         }
-        for (int i = 0; i < kStages; ++i) {
-            mbar_init(bars + 8 * (kBarKVFull + i), kTeamWarps);
-            mbar_init(bars + 8 * (kBarKVEmpty + i), 2);
-        }
+        for (int i = 0; i < QRing::kEmpty; ++i) mbar_init(bars + 8 * (kBarQEmpty + i), kMmaWarps + kSoftmaxWarps);
+        for (int i = 0; i < kStages; ++i) mbar_init(bars + 8 * (kBarKVFull + i), kTeamWarps);
+        for (int i = 0; i < KVRing::kEmpty; ++i) mbar_init(bars + 8 * (kBarKVEmpty + i), 2);
         for (int i = 0; i < kSchedDepth; ++i) {
             mbar_init(bars + 8 * (kBarSchedFull + i), 1);
             mbar_init(bars + 8 * (kBarSchedEmpty + i), kSchedReaders);
@@ -294,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                        bar_pv = bars + 8 * (kBarPVDone + h), bar_sf = bars + 8 * (kBarSFree + h);
         uint8_t *stage = sm + kOffStage + warp * 2048;
         const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
-        uint32_t ph_s = 0, ph_pv = 0, unit_cnt = 0;
+        uint32_t ph_s = 0, ph_pv = 0;
         bool alive = true;
         wait_prior_grid();
 
@@ -308,13 +309,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             const FwdUnit &un = s_unit[slot];
             if (un.rows == 0) break;
             TR_T0(t_setup);
-            const int qb = unit_cnt & 1;
-            if (!(alive = wait(bars + 8 * (kBarQFull + qb), (unit_cnt >> 1) & 1))) break;
-            ++unit_cnt;
+            const int qb = QRing::buffer(n);
+            if (!(alive = wait(bars + 8 * (kBarQFull + qb), QRing::full_parity(n)))) break;
             auto unit_done = [&]() {
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(bars + 8 * (kBarQEmpty + qb));
+                    mbar_arrive(bars + 8 * (kBarQEmpty + QRing::empty(n)));
                     mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
                 }
             };
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         reg_dealloc<kRegsOther>();
         const bool leader = elect_one();
         const int h = warp - kMmaWarp;
-        uint32_t kv_cnt = 0, unit_cnt = 0, ph_p = 0, ph_sf = 0;
+        uint32_t kv_cnt = 0, ph_p = 0, ph_sf = 0;
         bool alive = true;
         const uint32_t idesc_pv = idesc_bf16(128, 64, 0, 1);
         const uint32_t tSh0 = tmem + h * kTile, tOh = tmem + kTmemO + h * 64, tPh0 = tmem + kTmemP + h * 64;
@@ -633,9 +633,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             if (!next_unit(n, un)) break;
             un.tB &= 0xff;
             const int nA = un.tiles_a(), nB = un.tiles_b(), n_tiles = nA + nB;
-            const int qb = unit_cnt & 1;
+            const int qb = QRing::buffer(n);
             TR_T0(t_qf);
-            if (!(alive = wait(bars + 8 * (kBarQFull + qb), (unit_cnt >> 1) & 1))) break;
+            if (!(alive = wait(bars + 8 * (kBarQFull + qb), QRing::full_parity(n)))) break;
             tc_fence_after();
             TR_ADD(0, t_qf);
             const uint32_t q_lo = smem_desc_lo(base + kOffQ + (qb * 2 + h) * kTileBytes);
@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
 #pragma unroll 1
                         for (int ks = 1; ks < n_ks; ++ks) mma_ts_lean<1>(tOh, tPh + 8 * ks, v_lo + ks * ((16 * kRowBytes) >> 4), idesc_pv);
                         mma_commit(bar_pv);
-                        mma_commit(bars + 8 * (kBarKVEmpty + o_stage));
+                        mma_commit(bars + 8 * (kBarKVEmpty + KVRing::empty(c - 1)));
                     }
                     __syncwarp();
                     acc = true;
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 }
                 if (!visit && i < n_tiles) {  // released by a plain arrival, but not before it has landed
                     if (!(alive = wait(bars + 8 * (kBarKVFull + stage), (c / kStages) & 1))) break;
-                    if (lane == 0) mbar_arrive(bars + 8 * (kBarKVEmpty + stage));
+                    if (lane == 0) mbar_arrive(bars + 8 * (kBarKVEmpty + KVRing::empty(c)));
                 }
                 out = visit;
                 o_c0 = c0;
@@ -713,9 +713,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             }
             kv_cnt += n_tiles;
             if (!alive) break;
-            if (leader) mma_commit(bars + 8 * (kBarQEmpty + qb));
+            if (leader) mma_commit(bars + 8 * (kBarQEmpty + QRing::empty(n)));
             __syncwarp();
-            ++unit_cnt;
         }
         // nothing of this CTA may still run on the tensor pipe when TMEM is freed
         if (leader) mma_commit(bars + 8 * (kBarFinal + h));
@@ -746,7 +745,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         wait_prior_grid();
         const int team = (warp - kLoadWarp0) / kTeamWarps, lw = (warp - kLoadWarp0) % kTeamWarps;
         const bool leader = elect_one();
-        uint32_t kv_cnt = 0, unit_cnt = 0, step = 0;
+        uint32_t kv_cnt = 0, step = 0;
         bool alive = true;
         FwdUnit un;
         uint32_t checked = 0;  // entries of the list that are known to be done
@@ -793,7 +792,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             // instead of 2 x 32 gathers of four rows.  That is the prefix block's full tiles in every unit and, for a
             // row-major table, those of the row view.
             const int ident = !p.bulk ? 0 : p.view_order ? p.N : __ldg(vp.ident + un.b);
-            const int qb = unit_cnt & 1, r0 = kLoadRows * lw;
+            const int qb = QRing::buffer(n), r0 = kLoadRows * lw;
             // This lane's rows r0 + lane and r0 + 32 + lane of a tile, as rows of the tensors (rows behind the last one repeat it).
             int idx[2];
             static_assert(kLoadRows == 64, "rows per lane");
@@ -816,7 +815,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 if ((i ^ first) & 1) continue;
                 const uint32_t c = kv_cnt + max(i, 0), stage = c % kStages;
                 const uint32_t bar_full = bars + 8 * (i < 0 ? kBarQFull + qb : kBarKVFull + stage);
-                if (!(alive = wait(bars + 8 * (i < 0 ? kBarQEmpty + qb : kBarKVEmpty + stage), ((i < 0 ? unit_cnt >> 1 : c / kStages) & 1) ^ 1))) break;
+                if (!(alive = wait(bars + 8 * (i < 0 ? kBarQEmpty + QRing::wait_empty(n) : kBarKVEmpty + KVRing::wait_empty(c)),
+                                   i < 0 ? QRing::wait_parity(n) : KVRing::wait_parity(c)))) break;
                 TR_T0(t_cp);
                 if (i < 0) {
                     // row data for the softmax threads: original position and key range
@@ -867,7 +867,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 else fetch_record(true);
             }
             kv_cnt += n_tiles;
-            ++unit_cnt;
             step += 1 + n_tiles;
         }
     }

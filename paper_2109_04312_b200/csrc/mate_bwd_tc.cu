@@ -10,15 +10,16 @@
 //               -> P^T, dS^T -> dV += P^T dO, dK += dS^T Q
 // so no gradient is accumulated across CTAs and the result does not depend on the schedule.
 //
-// One persistent, warp-specialised CTA per SM (18 of 20 warps in use); work items (unit, side) are handed out through
+// One persistent, warp-specialised CTA per SM; work items (unit, side) are handed out through
 // a counter, longest first.
 //   warps 0-7   arithmetic: two threads (r, r + 128) share row r of the 128-row tile, the lane of
 //               tensor memory; each takes every other chunk of 32 columns.  S and dP (fp32) come out of
 //               tensor memory, P / dS (bf16 pairs) go back into it as MMA operands.
 //   warps 8-11  gradients of a finished item: tensor memory -> the rows' original positions, through a staging area so that
-//               a store covers whole rows; before the first item they zero the gradients of the padding rows
+//               a store covers whole rows
 //   warps 12,13 issue the tcgen05.mma (one elected lane each): S and dP of the tiles / the gradient MMAs, each as soon as
 //               what it needs is there
+//   warps 14,15 zero the gradients of the padding rows
 //   warps 16-19 loaders, in two teams of two that take the loads (row operands, column tiles) in turn: rows by view-order
 //               index, four to a tensor copy (gather4), or a column tile whose rows lie in place in the tensors by one
 //               bulk tensor copy per matrix, into 128-byte swizzled shared memory (row operands double buffered,
@@ -66,7 +67,10 @@ constexpr int kStoreWarp0 = kComputeWarps;
 constexpr int kStoreWarps = 4;
 constexpr int kMmaWarp = kStoreWarp0 + kStoreWarps;
 constexpr int kMmaWarps = 2;  // one for S and dP, one for the gradients
-constexpr int kLoadWarp0 = kMmaWarp + 4;  // (two warps of the MMA warps' group of four have nothing to do)
+constexpr int kPadWarp0 = kMmaWarp + kMmaWarps;
+constexpr int kPadWarps = 2;
+static_assert(kPadRows == 32 * kPadWarps, "a row per lane");
+constexpr int kLoadWarp0 = kPadWarp0 + kPadWarps;
 constexpr int kLoadWarps = 4;
 constexpr int kTeams = 2;                           // of loader warps, which take the steps in turn
 constexpr int kTeamWarps = kLoadWarps / kTeams;
@@ -456,23 +460,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         uint8_t *stage = sm + kOffStage + q4 * 4096;
         uint32_t units = 0;
         wait_prior_grid();
-        // padding rows: zero gradients
-#pragma unroll 1
-        for (int c = blockIdx.x; c < p.n_pads; c += gridDim.x) {
-            const PadChunk pc = p.pads[c];
-            const ViewPlan &vp = p.view[pc.view()];
-#pragma unroll 2
-            for (int i = q4 * 4 + (lane >> 3); i < pc.n; i += 4 * kStoreWarps) {  // eight lanes per row
-                const int orig = __ldg(vp.perm + (size_t)pc.b * p.N + pc.t0 + i);
-                if (p.tr.exists(pc.b, orig)) {
-                    const size_t at = (p.tr.base(pc.b, pc.head()) + orig) * 64 + (lane & 7) * 8;
-                    const int pass = p.pass(pc.view());
-                    *reinterpret_cast<uint4 *>(p.dQ[pass] + at) = make_uint4(0, 0, 0, 0);
-                    *reinterpret_cast<uint4 *>(p.dK[pass] + at) = make_uint4(0, 0, 0, 0);
-                    *reinterpret_cast<uint4 *>(p.dV[pass] + at) = make_uint4(0, 0, 0, 0);
-                }
-            }
-        }
 #pragma unroll 1
         for (uint32_t n = 0;; ++n) {
             const int slot = n % kSchedDepth, rb = n & 1;
@@ -535,7 +522,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             }
         }
     } else if (warp < kLoadWarp0) {
-        // ------------------------------------------------------------------ MMA issuers
+        // ------------------------------------------------------------------ MMA issuers, padding rows
         // One warp issues S and dP of the tiles, the other the gradient MMAs, each as soon as what it needs is there.  The
         // whole warp runs the control flow and one lane issues; votes and shuffles keep conditions and operands
         // warp-uniform (an MMA with other operands takes 51 clk to issue, more than a gradient MMA takes to run).
@@ -636,6 +623,28 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             if (leader) mma_commit(bars + 8 * (kBarFinal + grad));
             __syncwarp();
             mbar_wait_bounded(bars + 8 * (kBarFinal + grad), 0, kWaitLimit);
+        } else {
+            // padding rows: zero gradients.  (Not by the store warps: until a CTA's padding is done they would hold back rows,
+            // records and accumulators.)
+            wait_prior_grid();
+#pragma unroll 1
+            for (int c = blockIdx.x; c < p.n_pads; c += gridDim.x) {
+                const PadChunk pc = p.pads[c];
+                const ViewPlan &vp = p.view[pc.view()];
+                const int pass = p.pass(pc.view()), i = (warp - kPadWarp0) * 32 + lane;
+                int row = i < pc.n ? __ldg(vp.perm + (size_t)pc.b * p.N + pc.t0 + i) : -1;  // one look-up a chunk, a row per lane
+                if (row >= 0 && !p.tr.exists(pc.b, row)) row = -1;
+                const size_t at = p.tr.base(pc.b, pc.head()) * 64 + (lane & 7) * 8;
+#pragma unroll 1
+                for (int k = lane >> 3; k < 32; k += 4) {  // eight lanes per row
+                    const int r = __shfl_sync(0xffffffffu, row, k);
+                    if (r < 0) continue;
+                    const size_t o = at + (size_t)r * 64;
+                    *reinterpret_cast<uint4 *>(p.dQ[pass] + o) = make_uint4(0, 0, 0, 0);
+                    *reinterpret_cast<uint4 *>(p.dK[pass] + o) = make_uint4(0, 0, 0, 0);
+                    *reinterpret_cast<uint4 *>(p.dV[pass] + o) = make_uint4(0, 0, 0, 0);
+                }
+            }
         }
     } else {
         // ------------------------------------------------------------------ loaders

@@ -7,12 +7,10 @@
 //   warps 4-7   softmax of half 1 (rows 128..255)
 //   warps 8, 9  issue the tcgen05.mma of half 0 / half 1 (one elected lane each)
 //   warps 10,11 padding rows
-//   warps 12-15 loaders, in two teams of two that take the loads (Q, key tiles) in turn: rows by view-order index
-//               (the gather of Section 3.1 fused into the loads), four to a tensor copy (gather4), into 128-byte swizzled
-//               shared memory; K/V tiles whose rows lie in place in the tensors come in by one bulk tensor copy each.
-//               The copies complete on the tile's barrier by themselves.  (Four warps with 16-byte cp.async copies of every
-//               tile, in line with waits for them to signal: 80 KB of code instead of 69 then, and forward and backward together
-//               44.7 us for 8 x 512 tokens, 96.0 for 4 x 2048, 161.8 for 2 x 4096; with this form 43.7, 94.0, 158.6.)
+//   warps 12-15 loaders: Q, K, V rows by view-order index (the gather of Section 3.1 fused into the loads) into 128-byte
+//               swizzled shared memory, 16 bytes per lane and copy, 32 rows of every load per warp; K/V tiles whose rows lie
+//               in place in the tensors by one bulk tensor copy each.  Either kind completes on the tile's barrier by
+//               itself, so no warp waits for its copies in order to signal them.
 //
 // Per key tile and half:   S = Q K^T  (tcgen05.mma, M = 128, N <= 128, K = 64, accumulator in TMEM)
 //                          P = exp2(S c - m), row sum
@@ -68,13 +66,11 @@ constexpr int kPadWarp0 = kMmaWarp + kMmaWarps;
 constexpr int kPadWarps = 2;
 constexpr int kLoadWarp0 = kPadWarp0 + kPadWarps;
 constexpr int kLoadWarps = 4;
-constexpr int kTeams = 2;                    // of loader warps, which take the steps in turn
-constexpr int kTeamWarps = kLoadWarps / kTeams;
-constexpr int kLoadRows = kTile / kTeamWarps;  // rows of a tile a loader warp fetches
+static_assert(kTile == 32 * kLoadWarps, "a row of a tile per loader thread");
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
 constexpr int kStages = 4;                   // K/V ring
-using QRing = LoadRing<2>;
-using KVRing = LoadRing<kStages>;
+using QRing = LoadRing<2, 2>;  // every loader warp has a part in every load
+using KVRing = LoadRing<kStages, kStages>;
 // registers per thread after the roles have split: 256 x 176 + 256 x 80 = 65,536 = the 512 x 128 the CTA is
 // launched with
 constexpr int kRegsSoftmax = 176, kRegsOther = 80;
@@ -98,11 +94,11 @@ constexpr float kSumMin = 0x1p-100f, kSumMax = 0x1p60f;      // row sums outside
 
 // barrier slots (8 bytes each) behind kOffBar
 enum {
-    kBarQFull = 0,                             // [2] loaders -> MMA, softmax   (count: warps of a team)
-    kBarQEmpty = kBarQFull + 2,                // [4] MMA commits and softmax warps (row data read) -> loaders (count kMmaWarps + kSoftmaxWarps)
-    kBarKVFull = kBarQEmpty + QRing::kEmpty,   // [kStages] loaders -> MMA      (count: warps of a team)
-    kBarKVEmpty = kBarKVFull + kStages,        // [2 kStages] MMA -> loaders    (count 2: one per half)
-    kBarSFull = kBarKVEmpty + KVRing::kEmpty,  // [2] MMA commit -> softmax (count 1)
+    kBarQFull = 0,                     // [2] loaders -> MMA, softmax   (count kLoadWarps)
+    kBarQEmpty = kBarQFull + 2,        // [2] MMA commits and softmax warps (row data read) -> loaders (count kMmaWarps + kSoftmaxWarps)
+    kBarKVFull = kBarQEmpty + 2,       // [kStages] loaders -> MMA      (count kLoadWarps)
+    kBarKVEmpty = kBarKVFull + kStages,  // [kStages] MMA -> loaders    (count 2: one per half)
+    kBarSFull = kBarKVEmpty + kStages,   // [2] MMA commit -> softmax (count 1)
     kBarSFree = kBarSFull + 2,         // [2] softmax -> MMA: S of a tile has been read (count 4: one per warp)
     kBarPFull = kBarSFree + 2,         // [2] softmax -> MMA        (count 4: one per warp)
     kBarPVDone = kBarPFull + 2,        // [2] MMA commit -> softmax: the P V of a tile is complete (count 1)
@@ -120,11 +116,11 @@ template <bool kMany>
 struct Params {
     static constexpr int kV = kMany ? kViews : 2, kO = kMany ? kPasses : 1;
     __device__ static __forceinline__ int pass(int view) { return kMany ? pass_of(view) : 0; }
-    // 2-D tensor maps over the tensors seen as [B H N rows, 64 columns], 128-byte swizzle: boxes of 128 rows, and of one row
-    // for the gathers
-    CUtensorMap tmK, tmV, tmQ1, tmK1, tmV1;
+    // 2-D tensor maps over K and V seen as [B H N rows, 64 columns]: boxes of 128 rows, 128-byte swizzle
+    CUtensorMap tmK, tmV;
     int bulk;        // 0: every tile is gathered row by row
     int view_order;  // 1: Q, K, V, O and LSE are laid out in each head's own order (no gather, no scatter)
+    const __nv_bfloat16 *Q, *K, *V;
     __nv_bfloat16 *O[kO];
     float *LSE[kO];
     ViewPlan view[kV];
@@ -217,21 +213,23 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         rec = make_int4(0, 0, 0, 0);  // rows = 0: the list is exhausted
         if (u < p.n_units && lane < 4) rec = __ldg(reinterpret_cast<const int4 *>(p.units + u) + lane);
     };
-    if (warp == kLoadWarp0 + 1 && lane < 5) prefetch_tmap(&p.tmK + lane);  // all five of them
+    if (warp == kLoadWarp0 + 1 && lane < 2) prefetch_tmap(&p.tmK + lane);  // both of them
     if (warp == kLoadWarp0) fetch_record(false);  // requested before the set-up below, which takes as long
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bars + 8 * (kBarQFull + i), kTeamWarps);
+            mbar_init(bars + 8 * (kBarQFull + i), kLoadWarps);
+            mbar_init(bars + 8 * (kBarQEmpty + i), kMmaWarps + kSoftmaxWarps);
             mbar_init(bars + 8 * (kBarSFull + i), 1);
             mbar_init(bars + 8 * (kBarSFree + i), kSoftmaxWarps / 2);
             mbar_init(bars + 8 * (kBarPFull + i), kSoftmaxWarps / 2);
             mbar_init(bars + 8 * (kBarPVDone + i), 1);
             mbar_init(bars + 8 * (kBarFinal + i), 1);
         }
-        for (int i = 0; i < QRing::kEmpty; ++i) mbar_init(bars + 8 * (kBarQEmpty + i), kMmaWarps + kSoftmaxWarps);
-        for (int i = 0; i < kStages; ++i) mbar_init(bars + 8 * (kBarKVFull + i), kTeamWarps);
-        for (int i = 0; i < KVRing::kEmpty; ++i) mbar_init(bars + 8 * (kBarKVEmpty + i), 2);
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(bars + 8 * (kBarKVFull + i), kLoadWarps);
+            mbar_init(bars + 8 * (kBarKVEmpty + i), 2);
+        }
         for (int i = 0; i < kSchedDepth; ++i) {
             mbar_init(bars + 8 * (kBarSchedFull + i), 1);
             mbar_init(bars + 8 * (kBarSchedEmpty + i), kSchedReaders);
@@ -314,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             auto unit_done = [&]() {
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(bars + 8 * (kBarQEmpty + QRing::empty(n)));
+                    mbar_arrive(bars + 8 * (kBarQEmpty + qb));
                     mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
                 }
             };
@@ -636,6 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             const int qb = QRing::buffer(n);
             TR_T0(t_qf);
             if (!(alive = wait(bars + 8 * (kBarQFull + qb), QRing::full_parity(n)))) break;
+            fence_proxy_async();  // the copies of 16 bytes come through the generic proxy
             tc_fence_after();
             TR_ADD(0, t_qf);
             const uint32_t q_lo = smem_desc_lo(base + kOffQ + (qb * 2 + h) * kTileBytes);
@@ -648,13 +647,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             for (int i = 0; i <= n_tiles; ++i) {
                 const TileInfo t = tile_info(un, i, nA);
                 const uint32_t c = kv_cnt + i;
-                const int stage = c % kStages;
+                const int stage = KVRing::buffer(c);
                 int c0 = 0, c1 = 0;
                 if (has_rows && i < n_tiles) half_cols(h ? un.lo[1] : un.lo[0], h ? un.hi[1] : un.hi[0], t, c0, c1);
                 const bool visit = c1 > c0;
                 if (visit) {  // the tile has landed
                     TR_T0(t_kv);
-                    if (!(alive = wait(bars + 8 * (kBarKVFull + stage), (c / kStages) & 1))) break;
+                    if (!(alive = wait(bars + 8 * (kBarKVFull + stage), KVRing::full_parity(c)))) break;
+                    fence_proxy_async();
                     TR_ADD(5, t_kv);
                 }
                 if (out) {  // S of the outstanding tile has been read
@@ -696,15 +696,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
 #pragma unroll 1
                         for (int ks = 1; ks < n_ks; ++ks) mma_ts_lean<1>(tOh, tPh + 8 * ks, v_lo + ks * ((16 * kRowBytes) >> 4), idesc_pv);
                         mma_commit(bar_pv);
-                        mma_commit(bars + 8 * (kBarKVEmpty + KVRing::empty(c - 1)));
+                        mma_commit(bars + 8 * (kBarKVEmpty + o_stage));
                     }
                     __syncwarp();
                     acc = true;
                     TR_ADD(3, t_pv);
                 }
                 if (!visit && i < n_tiles) {  // released by a plain arrival, but not before it has landed
-                    if (!(alive = wait(bars + 8 * (kBarKVFull + stage), (c / kStages) & 1))) break;
-                    if (lane == 0) mbar_arrive(bars + 8 * (kBarKVEmpty + KVRing::empty(c)));
+                    if (!(alive = wait(bars + 8 * (kBarKVFull + stage), KVRing::full_parity(c)))) break;
+                    fence_proxy_async();
+                    if (lane == 0) mbar_arrive(bars + 8 * (kBarKVEmpty + stage));
                 }
                 out = visit;
                 o_c0 = c0;
@@ -713,7 +714,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             }
             kv_cnt += n_tiles;
             if (!alive) break;
-            if (leader) mma_commit(bars + 8 * (kBarQEmpty + QRing::empty(n)));
+            if (leader) mma_commit(bars + 8 * (kBarQEmpty + qb));
             __syncwarp();
         }
         // nothing of this CTA may still run on the tensor pipe when TMEM is freed
@@ -743,9 +744,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         // ------------------------------------------------------------------ loaders
         reg_dealloc<kRegsOther>();
         wait_prior_grid();
-        const int team = (warp - kLoadWarp0) / kTeamWarps, lw = (warp - kLoadWarp0) % kTeamWarps;
+        const int lw = warp - kLoadWarp0;
         const bool leader = elect_one();
-        uint32_t kv_cnt = 0, step = 0;
+        uint32_t kv_cnt = 0;
         bool alive = true;
         FwdUnit un;
         uint32_t checked = 0;  // entries of the list that are known to be done
@@ -787,42 +788,34 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             const size_t bn = (size_t)un.b * p.N;
             const int32_t *perm = p.view_order ? nullptr : vp.perm + bn;
             const size_t bh = p.tr.base(un.b, un.head());
+            const uint8_t *Qbh = reinterpret_cast<const uint8_t *>(p.Q + bh * 64), *Kbh = reinterpret_cast<const uint8_t *>(p.K + bh * 64);
+            const int64_t v_off = reinterpret_cast<const uint8_t *>(p.V) - reinterpret_cast<const uint8_t *>(p.K);
             // Rows of the order that sit in place in the tensors ([0, ident)): a K/V tile inside that range
             // (see bulk_tile) is one contiguous [128, 64] box and comes in by one bulk tensor copy per matrix
-            // instead of 2 x 32 gathers of four rows.  That is the prefix block's full tiles in every unit and, for a
+            // instead of 2 x 1024 copies of 16 bytes.  That is the prefix block's full tiles in every unit and, for a
             // row-major table, those of the row view.
             const int ident = !p.bulk ? 0 : p.view_order ? p.N : __ldg(vp.ident + un.b);
-            const int qb = QRing::buffer(n), r0 = kLoadRows * lw;
-            // This lane's rows r0 + lane and r0 + 32 + lane of a tile, as rows of the tensors (rows behind the last one repeat it).
-            int idx[2];
-            static_assert(kLoadRows == 64, "rows per lane");
-            auto look_up = [&](const TileInfo &t) {
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    const int at = t.pos(min(r0 + 32 * k + lane, t.w - 1));
-                    idx[k] = (int)bh + (perm ? __ldg(perm + at) : at);  // no order given: the tensors are in view order
-                }
+            const int qb = QRing::buffer(n);
+            // steps -2, -1: the two Q halves (and the row data of the unit); steps 0 ..: the key tiles
+            auto step_idx = [&](int i) {
+                const TileInfo t = i < 0 ? row_tile(un.row0_of(i + 2), un.rows_of(i + 2)) : tile_info(un, i, nA);
+                return t.w > 0 ? fetch_idx(perm, t, lw, lane) : 0;
             };
-            const int first = (int)((step + team) & 1) - 1;  // of this team's steps
-            // step -1: the two Q halves and the row data of the unit; steps 0 ..: the key tiles
+            int next = step_idx(-2);
 #pragma unroll 1
-            for (int i = -1; i < n_tiles; ++i) {
-                // The number of the next unit travels under the copies.  Claimed in front of the last tile but one of a long
-                // unit, of the last one of a short one: there a claim more tiles ahead ties units to CTAs that are
-                // not the next to be free (4 x 2048 tokens: 33.5 us, 35.1 with all claims early; 1 x 8192: 55.0, 55.9 with
-                // all of them late).
-                if (warp == kLoadWarp0 && i == (n_tiles <= 6 ? n_tiles - 1 : n_tiles - 2) && !redo) claim();
-                if ((i ^ first) & 1) continue;
-                const uint32_t c = kv_cnt + max(i, 0), stage = c % kStages;
+            for (int i = -2; i < n_tiles; ++i) {
+                const int now = next;
+                if (i + 1 < n_tiles) next = step_idx(i + 1);
+                else if (warp == kLoadWarp0 && !redo) claim();  // the number of the next unit travels under the copies
+                const uint32_t c = kv_cnt + max(i, 0), stage = KVRing::buffer(c);
                 const uint32_t bar_full = bars + 8 * (i < 0 ? kBarQFull + qb : kBarKVFull + stage);
-                if (!(alive = wait(bars + 8 * (i < 0 ? kBarQEmpty + QRing::wait_empty(n) : kBarKVEmpty + KVRing::wait_empty(c)),
-                                   i < 0 ? QRing::wait_parity(n) : KVRing::wait_parity(c)))) break;
+                if (i != -1 && !(alive = wait(bars + 8 * (i < 0 ? kBarQEmpty + qb : kBarKVEmpty + stage),
+                                              i < 0 ? QRing::wait_parity(n) : KVRing::wait_parity(c)))) break;
                 TR_T0(t_cp);
-                if (i < 0) {
-                    // row data for the softmax threads: original position and key range
+                if (i == -2) {  // row data for the softmax threads: original position and key range
 #pragma unroll 1
-                    for (int k = 0; k < 4; ++k) {
-                        const int half = k >> 1, rr = r0 + (k & 1) * 32 + lane;
+                    for (int half = 0; half < 2; ++half) {
+                        const int rr = 32 * lw + lane;
                         if (rr < un.rows_of(half)) {
                             const size_t at = bn + un.row0_of(half) + rr;
                             const uint32_t meta = base + kOffMeta + (qb * 3 * kUnitRows + half * kTile + rr) * 4;
@@ -831,34 +824,26 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                             cp_async4(meta + 2 * kUnitRows * 4, vp.seg_hi + at);
                         }
                     }
-                    cp_async_arrive(bar_full);
                 }
-                __syncwarp();
                 const TileInfo t = tile_info(un, max(i, 0), nA);
-                if (i >= 0 && bulk_tile(t, ident)) {
-                    if (leader) {
-                        mbar_arrive_expect_tx(bar_full, lw == 0 ? 2 * kTileBytes : 0);
-                        if (lw == 0) {
-                            const uint32_t dst = base + kOffKV + stage * 2 * kTileBytes;
+                const uint32_t dst = base + (i < 0 ? kOffQ + (qb * 2 + i + 2) * kTileBytes : kOffKV + stage * 2 * kTileBytes);
+                const bool bulk = i >= 0 && bulk_tile(t, ident);
+                // (rows of a Q half past its last one are never looked at: their results are not stored)
+                if (!bulk) gather_rows(dst, i < 0 ? Qbh : Kbh, i >= 0, v_off, now, i < 0 ? un.rows_of(i + 2) : (t.w + 15) & ~15, lw, lane);
+                if (i != -2) {
+                    cp_async_arrive(bar_full);
+                    __syncwarp();
+                    if (bulk && lw == 0) {
+                        if (leader) {
+                            mbar_arrive_expect_tx(bar_full, 2 * kTileBytes);
                             tma_load_2d(dst, &p.tmK, 0, (int)bh + t.first(), bar_full);
                             tma_load_2d(dst + kTileBytes, &p.tmV, 0, (int)bh + t.first(), bar_full);
                         }
-                    }
-                } else {
-                    // (rows of a Q half past its last one are never looked at: their results are not stored)
-                    const auto mine = [&](int rows) { return min(max(rows - r0, 0), kLoadRows); };
-                    const int rows_a = mine(i < 0 ? un.rows_of(0) : (t.w + 15) & ~15), rows_b = i < 0 ? mine(un.rows_of(1)) : rows_a;
-                    if (leader) mbar_arrive_expect_tx(bar_full, gather_bytes(rows_a) + gather_bytes(rows_b));
-#pragma unroll 1
-                    for (int half = 0; half < (i < 0 ? 2 : 1); ++half) {
-                        const int rows = half ? rows_b : rows_a;
-                        if (rows == 0) continue;
-                        look_up(i < 0 ? row_tile(un.row0_of(half), un.rows_of(half)) : t);
-                        gather_rows4<1>(base + (i < 0 ? kOffQ + (qb * 2 + half) * kTileBytes : kOffKV + stage * 2 * kTileBytes),
-                                     i < 0 ? &p.tmQ1 : &p.tmK1, i < 0 ? nullptr : &p.tmV1, idx, r0, rows, leader, bar_full);
+                        __syncwarp();
+                    } else if (lane == 0) {
+                        mbar_arrive(bar_full);
                     }
                 }
-                __syncwarp();
                 TR_ADD(2, t_cp);
                 TR_INC(4);
             }
@@ -867,7 +852,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 else fetch_record(true);
             }
             kv_cnt += n_tiles;
-            step += 1 + n_tiles;
         }
     }
 
@@ -941,10 +925,11 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     const bool want_bulk = !(flags & MATE_FLAG_GATHER_TILES) || (flags & MATE_FLAG_VIEW_ORDER);
     p.bulk = want_bulk ? 1 : 0;
     if (rows >= (size_t(1) << 31)) return MATE_ERR_UNSUPPORTED;
-    if (!make_row_map(&p.tmK, K, rows) || !make_row_map(&p.tmV, V, rows) || !make_row_map(&p.tmQ1, Q, rows, 1) ||
-        !make_row_map(&p.tmK1, K, rows, 1) || !make_row_map(&p.tmV1, V, rows, 1))
-        return MATE_ERR_CUDA;
+    if (!make_row_map(&p.tmK, K, rows) || !make_row_map(&p.tmV, V, rows)) return MATE_ERR_CUDA;
     p.view_order = (flags & MATE_FLAG_VIEW_ORDER) ? 1 : 0;
+    p.Q = (const __nv_bfloat16 *)Q;
+    p.K = (const __nv_bfloat16 *)K;
+    p.V = (const __nv_bfloat16 *)V;
     for (int i = 0; i < p.kO; ++i) {
         p.O[i] = (__nv_bfloat16 *)O[i];
         p.LSE[i] = LSE[i];

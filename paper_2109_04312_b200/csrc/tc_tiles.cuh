@@ -14,6 +14,14 @@ constexpr int kTileBytes = kTile * kRowBytes;  // 16 KB: 128 rows
 // Tensor map over a [rows, 64] bf16 matrix in boxes of box_rows rows (false: no tensor maps to be had).
 bool make_row_map(CUtensorMap *map, const void *base, size_t rows, int box_rows = kTile);
 
+// The loaders copy a tile of up to 128 rows (128 B each), warp w of the four the rows 32 w .. 32 w + 31.
+// A lane looks up the original position of one row (coalesced, one latency for the whole tile, and cheap
+// enough to be done a tile ahead); the copies then run four rows at a time, eight lanes per row, with the
+// positions handed around by shuffle.  Rows behind the last one repeat it.
+__device__ __forceinline__ int fetch_idx(const int32_t *perm, const TileInfo &t, int lw, int lane) {
+    const int at = t.pos(min(32 * lw + lane, t.w - 1));
+    return perm ? __ldg(perm + at) : at;  // no order given: the tensors are in view order
+}
 // n rows from view position q0 on, as a tile
 __device__ __forceinline__ TileInfo row_tile(int q0, int n) {
     TileInfo t;
@@ -31,6 +39,24 @@ __device__ __forceinline__ TileInfo row_tile(int q0, int n) {
 __device__ __forceinline__ bool bulk_tile(const TileInfo &t, int ident) {
     return (t.w & 15) == 0 && t.contiguous() && t.first() + kTile <= ident;
 }
+// Rows [0, n_rows) of one tensor, or of two (`pair`; b_off: bytes from the first one's rows to the second's)
+// -> tiles at s_a and 16 KB behind it, 128-byte swizzle.  (Four rows to a tensor copy, by two teams of two warps that took the
+// loads in turn, kept a warp busy for 3700 to 4400 clk per load; these take 1000.)
+__device__ __forceinline__ void gather_rows(uint32_t s_a, const uint8_t *a_bh, bool pair, int64_t b_off, uint32_t idx, int n_rows,
+                                            int lw, int lane) {
+    if (32 * lw >= n_rows) return;  // (rows past n_rows inside a group of 32 repeat a row that exists)
+    const int sub = lane >> 3;      // row of the group of four
+    a_bh += (lane & 7) * 16;
+    const uint32_t d = s_a + (32 * lw + sub) * kRowBytes + (((lane & 7) ^ sub) << 4);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint8_t *src = a_bh + (size_t)__shfl_sync(0xffffffffu, idx, 4 * i + sub) * kRowBytes;
+        const uint32_t dst = (d ^ ((i & 1) << 6)) + 4 * i * kRowBytes;
+        ptx::cp_async16(dst, src);
+        if (pair) ptx::cp_async16(dst + kTileBytes, src + b_off);
+    }
+}
+
 // Tile rows r0 .. r0 + n_rows - 1 (at most 64; up to a multiple of four) of two tensors, by index: -> tiles at s_a and 16 KB
 // behind it, 128-byte swizzle, four rows per copy.  idx: the tensors' rows for tile rows r0 + lane and r0 + 32 + lane.  The
 // whole warp takes part, its leader issues; the copies count on `bar` (gather_bytes per tensor).

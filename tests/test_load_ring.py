@@ -1,4 +1,4 @@
-"""The barriers between the loader teams of the tensor-core kernels and the readers of what they load (csrc/load_ring.h), as a
+"""The barriers between the loader warps of the tensor-core kernels and the readers of what they load (csrc/load_ring.h), as a
 model on the CPU (tests/load_ring_model.cpp): no wait passes before the phase it is for is over, whatever
 the order in which the roles get on, and no run stands still."""
 import ctypes
@@ -31,6 +31,6 @@ def test_no_wait_passes_early(model, kernel, most):
 
 
 @pytest.mark.parametrize("kernel", ["forward", "backward"])
-def test_one_barrier_per_buffer_is_not_enough(model, kernel):
-    early, _ = early_and_stuck(model.one_barrier, kernel == "backward", 2500, 2, 11)
+def test_one_barrier_per_buffer_is_not_enough_for_teams(model, kernel):
+    early, _ = early_and_stuck(model.teams, kernel == "backward", 2500, 2, 11)
     assert early > 0

@@ -20,10 +20,10 @@
 //   warps 12,13 issue the tcgen05.mma (one elected lane each): S and dP of the tiles / the gradient MMAs, each as soon as
 //               what it needs is there
 //   warps 14,15 zero the gradients of the padding rows
-//   warps 16-19 loaders, in two teams of two that take the loads (row operands, column tiles) in turn: rows by view-order
-//               index, four to a tensor copy (gather4), or a column tile whose rows lie in place in the tensors by one
-//               bulk tensor copy per matrix, into 128-byte swizzled shared memory (row operands double buffered,
-//               column tiles in a ring of 4)
+//   warps 16-19 loaders: rows by view-order index, 16 bytes per lane and copy, 32 rows of every load per warp, or a column
+//               tile whose rows lie in place in the tensors by one bulk tensor copy per matrix, into 128-byte swizzled shared
+//               memory (row operands double buffered, column tiles in a ring of 4).  Either kind completes on the
+//               tile's barrier by itself, so no warp waits for its copies in order to signal them.
 // What bounds it.  The exponentials take 1024 clk per 128 x 128 tile and side (16 per clock and SM); what is left is the
 // chain S complete -> registers -> arithmetic -> operands -> next S, about 2050 clk per tile when all pairs count, and on
 // tables the loads and the cost per item.  Hence:
@@ -72,9 +72,7 @@ constexpr int kPadWarps = 2;
 static_assert(kPadRows == 32 * kPadWarps, "a row per lane");
 constexpr int kLoadWarp0 = kPadWarp0 + kPadWarps;
 constexpr int kLoadWarps = 4;
-constexpr int kTeams = 2;                           // of loader warps, which take the steps in turn
-constexpr int kTeamWarps = kLoadWarps / kTeams;
-constexpr int kLoadRows = kTile / kTeamWarps;       // rows of a tile a loader warp fetches
+static_assert(kTile == 32 * kLoadWarps, "a row of a tile per loader thread");
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
 // registers per thread after the roles have split: 256 x 168 + 128 x 48 + 128 x 40 + 128 x 56 = 61,440 = the 640 x 96 the
 // CTA is launched with
@@ -94,11 +92,11 @@ constexpr uint32_t kSmemBytes = kOffBar + 512 + 1024;            // + slack for 
 static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 // barrier slots (8 bytes each) behind kOffBar
 enum {
-    kBarRFull = 0,                     // [2] loaders -> MMA, arithmetic      (count: warps of a team)
-    kBarREmpty = kBarRFull + 2,        // [4] MMA commit and arithmetic warps (row data read) -> loaders (count 1 + kComputeWarps + kStoreWarps)
-    kBarCFull = kBarREmpty + RowRing::kEmpty,   // [kStages] loaders -> MMA     (count: warps of a team)
-    kBarCEmpty = kBarCFull + kStages,  // [2 kStages] MMA commit -> loaders   (count 1)
-    kBarSFull = kBarCEmpty + ColRing::kEmpty,   // MMA commit -> arithmetic: S and dP of a tile are complete (count 1)
+    kBarRFull = 0,                     // [2] loaders -> MMA, arithmetic      (count kLoadWarps)
+    kBarREmpty = kBarRFull + 2,        // [2] MMA commit and arithmetic warps (row data read) -> loaders (count 1 + kComputeWarps + kStoreWarps)
+    kBarCFull = kBarREmpty + 2,        // [kStages] loaders -> MMA            (count kLoadWarps)
+    kBarCEmpty = kBarCFull + kStages,  // [kStages] MMA commit -> loaders     (count 1)
+    kBarSFull = kBarCEmpty + kStages,  // MMA commit -> arithmetic: S and dP of a tile are complete (count 1)
     kBarAFull,         // arithmetic -> MMA: the bf16 operands of a tile are written (count: one per warp)
     kBarGDone,         // MMA commit -> arithmetic: the gradient MMAs of a tile are complete (count 1)
     kBarSTFree,        // arithmetic -> MMA: S and dP of a tile are in registers (count: one per warp)
@@ -121,8 +119,8 @@ template <bool kMany>
 struct Params {
     static constexpr int kV = kMany ? kViews : 2, kO = kMany ? kPasses : 1;
     __device__ static __forceinline__ int pass(int view) { return kMany ? pass_of(view) : 0; }
-    CUtensorMap tmQ, tmK, tmV, tmdO;      // boxes of 128 rows, 128-byte swizzle
-    CUtensorMap tmQ1, tmK1, tmV1, tmdO1;  // of one row, for the gathers
+    CUtensorMap tmQ, tmK, tmV, tmdO;  // boxes of 128 rows, 128-byte swizzle
+    const __nv_bfloat16 *Q, *K, *V, *dO;
     const float *nlse, *D;  // per row, original order: -LSE log2 e, D
     __nv_bfloat16 *dQ[kO], *dK[kO], *dV[kO];
     ViewPlan view[kV];
@@ -267,13 +265,17 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         }
     };
     if (warp == kLoadWarp0) fetch_record(false);
-    if (warp == kLoadWarp0 + 1 && lane < 8) prefetch_tmap(&p.tmQ + lane);  // all eight of them
+    if (warp == kLoadWarp0 + 1 && lane < 4) prefetch_tmap(&p.tmQ + lane);  // all four of them
 
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) mbar_init(bars + 8 * (kBarRFull + i), kTeamWarps);
-        for (int i = 0; i < RowRing::kEmpty; ++i) mbar_init(bars + 8 * (kBarREmpty + i), 1 + kComputeWarps + kStoreWarps);
-        for (int i = 0; i < kStages; ++i) mbar_init(bars + 8 * (kBarCFull + i), kTeamWarps);
-        for (int i = 0; i < ColRing::kEmpty; ++i) mbar_init(bars + 8 * (kBarCEmpty + i), 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bars + 8 * (kBarRFull + i), kLoadWarps);
+            mbar_init(bars + 8 * (kBarREmpty + i), 1 + kComputeWarps + kStoreWarps);
+        }
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(bars + 8 * (kBarCFull + i), kLoadWarps);
+            mbar_init(bars + 8 * (kBarCEmpty + i), 1);
+        }
         mbar_init(bars + 8 * kBarSFull, 1);
         mbar_init(bars + 8 * kBarAFull, kComputeWarps);
         mbar_init(bars + 8 * kBarSTFree, kComputeWarps);
@@ -332,7 +334,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
 
 #pragma unroll 1
         for (uint32_t n = 0; alive; ++n) {
-            const int slot = n % kSchedDepth, rb = n & 1;
+            const int slot = n % kSchedDepth, rb = RowRing::buffer(n);
             if (!wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) break;
             // The record and the row data stay in shared memory until the item's last tile: what is needed of them is
             // read where it is needed (registers are what this role is short of).
@@ -340,7 +342,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             if (un.rows == 0) break;
             const bool key_side = un.ws_off == 0;
             const ItemTiles tiles(un);
-            if (!(alive = wait(bars + 8 * (kBarRFull + rb), (n >> 1) & 1))) break;
+            if (!(alive = wait(bars + 8 * (kBarRFull + rb), RowRing::full_parity(n)))) break;
             // this row's data (rows past the end shadow the last one)
             const uint32_t meta = base + kOffMeta + (rb * 5 * kTile + min(r, un.rows_of(0) - 1)) * 4;
             const int w_lo_max = __reduce_max_sync(0xffffffffu, ld_shared_s32(meta + kTile * 4)),
@@ -359,7 +361,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
 #pragma unroll 1
                 for (int i = 0; i < tiles.n; ++i) {
                     const bool full = t.w == kTile && (t.pre == kTile || (w_lo_max - t.k0 <= t.pre && w_hi_min - t.k0 >= kTile));
-                    const uint32_t vec = base + kOffVec + (c_cnt % kStages) * 1024;
+                    const uint32_t vec = base + kOffVec + ColRing::buffer(c_cnt) * 1024;
                     TR_T0(t_ws);
                     if (!(alive = wait(bars + 8 * kBarSFull, c_cnt & 1))) break;
                     tc_fence_after();
@@ -447,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             if (!alive) break;
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive(bars + 8 * (kBarREmpty + RowRing::empty(n)));
+                mbar_arrive(bars + 8 * (kBarREmpty + rb));
                 mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
             }
         }
@@ -462,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         wait_prior_grid();
 #pragma unroll 1
         for (uint32_t n = 0;; ++n) {
-            const int slot = n % kSchedDepth, rb = n & 1;
+            const int slot = n % kSchedDepth, rb = RowRing::buffer(n);
             if (!wait(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) break;
             const FwdUnit &un = s_item[slot];
             if (un.rows == 0) break;
@@ -471,11 +473,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             const size_t at = p.tr.base(un.b, un.head()) * 64;
             __syncwarp();
             if (lane == 0) mbar_arrive(bars + 8 * (kBarSchedEmpty + slot));
-            if (!wait(bars + 8 * (kBarRFull + rb), (n >> 1) & 1)) break;
+            if (!wait(bars + 8 * (kBarRFull + rb), RowRing::full_parity(n))) break;
             const int r = q4 * 32 + lane;
             const int dst_row = r < rows_h ? (reinterpret_cast<const int32_t *>(sm + kOffMeta) + rb * 5 * kTile)[r] : -1;
             __syncwarp();
-            if (lane == 0) mbar_arrive(bars + 8 * (kBarREmpty + RowRing::empty(n)));
+            if (lane == 0) mbar_arrive(bars + 8 * (kBarREmpty + rb));
             if (any) {
                 if (!wait(bars + 8 * kBarItemDone, units++ & 1)) break;
                 tc_fence_after();
@@ -544,7 +546,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             bool alive = true;
 #pragma unroll 1
             for (uint32_t n = 0; alive; ++n) {
-                const int slot = n % kSchedDepth, rb = n & 1;
+                const int slot = n % kSchedDepth, rb = RowRing::buffer(n);
                 if (!wait_u(bars + 8 * (kBarSchedFull + slot), (n / kSchedDepth) & 1)) break;
                 const FwdUnit &un = s_item[slot];
                 auto uniform = [&](int x) { return __shfl_sync(0xffffffffu, x, 0); };
@@ -556,15 +558,17 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                 const int nA = (len_a + kTile - 1) / kTile, n_tiles = nA + (len_b + kTile - 1) / kTile;
                 auto steps = [&](int i) { return (min(i < nA ? len_a - i * kTile : len_b - (i - nA) * kTile, kTile) + 15) >> 4; };  // of 16 columns
                 if (!grad) {
-                    if (!(alive = wait_u(bars + 8 * (kBarRFull + rb), (n >> 1) & 1))) break;
+                    if (!(alive = wait_u(bars + 8 * (kBarRFull + rb), RowRing::full_parity(n)))) break;
+                    fence_proxy_async();
                     const uint32_t ra = smem_desc_lo(base + kOffR) + rb * ((2 * kTileBytes) >> 4), rbb = ra + (kTileBytes >> 4);
 #pragma unroll 1
                     for (int i = 0; i < n_tiles; ++i, ++c_cnt) {
-                        const uint32_t st = c_cnt % kStages;
+                        const uint32_t st = ColRing::buffer(c_cnt);
                         const uint32_t idesc = idesc_bf16(128, 0, 0, 0) | (uint32_t)steps(i) << 18;  // N = 16 columns per step
                         const uint32_t ca = smem_desc_lo(base + kOffC) + st * ((2 * kTileBytes) >> 4), cb = ca + (kTileBytes >> 4);
                         const uint32_t tS = tmem + kTmS, tT = tmem + kTmT;
-                        if (!(alive = wait_u(bars + 8 * (kBarCFull + st), (c_cnt / kStages) & 1))) break;  // the tile has landed
+                        if (!(alive = wait_u(bars + 8 * (kBarCFull + st), ColRing::full_parity(c_cnt)))) break;  // the tile has landed
+                        fence_proxy_async();  // the copies of 16 bytes come through the generic proxy
                         // the tile before sits in registers (parity 1 of a barrier without a phase behind it: at once)
                         if (!(alive = wait_u(bars + 8 * kBarSTFree, (c_cnt - 1) & 1))) break;
                         tc_fence_after();
@@ -582,7 +586,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                         __syncwarp();
                     }
                     if (!alive) break;
-                    if (leader) mma_commit(bars + 8 * (kBarREmpty + RowRing::empty(n)));  // the row operands are free once these MMAs are done
+                    if (leader) mma_commit(bars + 8 * (kBarREmpty + rb));  // the row operands are free once these MMAs are done
                     __syncwarp();
                 } else {
                     constexpr uint32_t idesc = idesc_bf16(128, 64, 0, 1);  // B = 16 rows of the column tile x 64, MN-major
@@ -592,7 +596,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                     const uint32_t tA1 = tmem + kTmA1, tA2 = tmem + kTmA2, tG1 = tmem + kTmAcc1, tG2 = tmem + kTmAcc2;
 #pragma unroll 1
                     for (int i = 0; i < n_tiles; ++i, ++c_cnt) {
-                        const uint32_t st = c_cnt % kStages;
+                        const uint32_t st = ColRing::buffer(c_cnt);
                         const int ks = steps(i);
                         const uint32_t a_lo = smem_desc_lo(base + kOffC) + st * ((2 * kTileBytes) >> 4), b_lo = a_lo + (kTileBytes >> 4);
                         if (!(alive = wait_u(bars + 8 * kBarAFull, c_cnt & 1))) break;
@@ -612,7 +616,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                                 for (int k = 1; k < ks; ++k) mma_ts_lean<1>(tG1, tA1 + 8 * k, a_lo + k * kStep, idesc);
                             }
                             mma_commit(bars + 8 * kBarGDone);
-                            mma_commit(bars + 8 * (kBarCEmpty + ColRing::empty(c_cnt)));
+                            mma_commit(bars + 8 * (kBarCEmpty + st));
                             if (i + 1 == n_tiles) mma_commit(bars + 8 * kBarItemDone);
                         }
                         __syncwarp();
@@ -650,14 +654,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         // ------------------------------------------------------------------ loaders
         reg_dealloc<kRegsLoad>();
         wait_prior_grid();
-        const int team = (warp - kLoadWarp0) / kTeamWarps, lw = (warp - kLoadWarp0) % kTeamWarps;
-        uint32_t step = 0;
+        const int lw = warp - kLoadWarp0;
         const bool leader = elect_one();
         uint32_t c_cnt = 0;
         bool alive = true;
 #pragma unroll 1
         for (uint32_t n = 0; alive; ++n) {
-            const int slot = n % kSchedDepth, rb = n & 1;
+            const int slot = n % kSchedDepth, rb = RowRing::buffer(n);
             if (warp == kLoadWarp0) {
                 if (!wait(bars + 8 * (kBarSchedEmpty + slot), ((n / kSchedDepth) & 1) ^ 1)) break;
                 if (lane < 4) reinterpret_cast<int4 *>(s_item + slot)[lane] = rec;
@@ -678,72 +681,64 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             const size_t bh = p.tr.base(un.b, un.head());
             // column tiles inside [0, ident) of the order are contiguous in the tensors (see bulk_tile)
             const int ident = __ldg(vp.ident + un.b);
-            const int r0 = kLoadRows * lw + lane;  // this lane's rows of a tile: r0, r0 + 32, .. (rows behind the last one repeat it)
-
             // step -1: the row operands and row data; steps 0 ..: the column tiles
-            constexpr int kPer = kLoadRows / 32;
-            const int first = (int)((step + team) & 1) - 1;  // of this team's steps
+            const int rr = 32 * lw + lane;  // this lane's row of a tile
+            auto step_idx = [&](int i) {  // as a row of the tensors
+                const TileInfo t = tiles.tile(max(i, 0));
+                return (uint32_t)bh + (uint32_t)__ldg(perm + (i < 0 ? un.q0 + min(rr, rows_h - 1) : t.pos(min(rr, t.w - 1))));
+            };
+            uint32_t next = step_idx(-1);
 #pragma unroll 1
             for (int i = -1; i < tiles.n; ++i) {
                 // the next item's number and then its record travel under the copies
                 if (warp == kLoadWarp0 && i == max(tiles.n - 2, -1)) claim();
                 if (warp == kLoadWarp0 && i + 1 == tiles.n) fetch_record();
-                if ((i ^ first) & 1) continue;
+                const uint32_t now = next;
+                if (i + 1 < tiles.n) next = step_idx(i + 1);
                 const TileInfo t = tiles.tile(max(i, 0));
-                int now[kPer];  // rows of the tensors
-#pragma unroll
-                for (int k = 0; k < kPer; ++k) now[k] = (int)bh + __ldg(perm + (i < 0 ? un.q0 + min(r0 + 32 * k, rows_h - 1) : t.pos(min(r0 + 32 * k, t.w - 1))));
-                const uint32_t c = c_cnt + max(i, 0), st = c % kStages;
-                const uint32_t bar_e = bars + 8 * (i < 0 ? kBarREmpty + RowRing::wait_empty(n) : kBarCEmpty + ColRing::wait_empty(c)),
-                               bar_full = bars + 8 * (i < 0 ? kBarRFull + rb : kBarCFull + st);
-                if (!(alive = wait(bar_e, i < 0 ? RowRing::wait_parity(n) : ColRing::wait_parity(c)))) break;
+                const uint32_t c = c_cnt + max(i, 0), st = ColRing::buffer(c);
+                const uint32_t bar_full = bars + 8 * (i < 0 ? kBarRFull + rb : kBarCFull + st);
+                if (!(alive = wait(bars + 8 * (i < 0 ? kBarREmpty + rb : kBarCEmpty + st),
+                                   i < 0 ? RowRing::wait_parity(n) : ColRing::wait_parity(c)))) break;
                 if (i < 0) {  // row data for the arithmetic threads
-#pragma unroll
-                    for (int k = 0; k < kPer; ++k) {
-                        const int rr = r0 + 32 * k;
+                    if (rr < rows_h) {
                         const uint32_t meta = base + kOffMeta + rb * 5 * kTile * 4 + rr * 4;
-                        if (rr < rows_h) {
-                            const size_t at = bn + un.q0 + rr;
-                            cp_async4(meta, vp.perm + at);
-                            cp_async4(meta + kTile * 4, vp.seg_lo + at);
-                            cp_async4(meta + 2 * kTile * 4, vp.seg_hi + at);
-                            if (!key_side) {
-                                cp_async4(meta + 3 * kTile * 4, p.nlse + now[k]);
-                                cp_async4(meta + 4 * kTile * 4, p.D + now[k]);
-                            }
+                        const size_t at = bn + un.q0 + rr;
+                        cp_async4(meta, vp.perm + at);
+                        cp_async4(meta + kTile * 4, vp.seg_lo + at);
+                        cp_async4(meta + 2 * kTile * 4, vp.seg_hi + at);
+                        if (!key_side) {
+                            cp_async4(meta + 3 * kTile * 4, p.nlse + now);
+                            cp_async4(meta + 4 * kTile * 4, p.D + now);
                         }
                     }
-                    cp_async_arrive(bar_full);
                 } else if (key_side) {  // column data
-#pragma unroll
-                    for (int k = 0; k < kPer; ++k) {
-                        const uint32_t vec = base + kOffVec + st * 1024 + (r0 + 32 * k) * 4;
-                        cp_async4(vec, p.nlse + now[k]);
-                        cp_async4(vec + 512, p.D + now[k]);
-                    }
-                    cp_async_arrive(bar_full);
+                    const uint32_t vec = base + kOffVec + st * 1024 + rr * 4;
+                    cp_async4(vec, p.nlse + now);
+                    cp_async4(vec + 512, p.D + now);
                 }
-                __syncwarp();
                 const uint32_t dst = base + (i < 0 ? kOffR + rb * 2 * kTileBytes : kOffC + st * 2 * kTileBytes);
                 const bool kv = (i < 0) == key_side;  // K and V, or Q and dO
-                if (i >= 0 && bulk_tile(t, ident)) {
-                    if (leader) {
-                        mbar_arrive_expect_tx(bar_full, lw == 0 ? 2 * kTileBytes : 0);
-                        if (lw == 0) {
-                            tma_load_2d(dst, kv ? &p.tmK : &p.tmQ, 0, (int)bh + t.first(), bar_full);
-                            tma_load_2d(dst + kTileBytes, kv ? &p.tmV : &p.tmdO, 0, (int)bh + t.first(), bar_full);
-                        }
-                    }
-                } else {
-                    // (the row operands' rows past the last one are never looked at: their results are not stored)
-                    const int n_rows = min(max((i < 0 ? rows_h : (t.w + 15) & ~15) - kLoadRows * lw, 0), kLoadRows);
-                    if (leader) mbar_arrive_expect_tx(bar_full, 2 * gather_bytes(n_rows));
-                    gather_rows4<2>(dst, kv ? &p.tmK1 : &p.tmQ1, kv ? &p.tmV1 : &p.tmdO1, now, r0 - lane, n_rows, leader, bar_full);
+                const bool bulk = i >= 0 && bulk_tile(t, ident);
+                // (the row operands' rows past the last one are never looked at: their results are not stored)
+                if (!bulk) {
+                    const uint8_t *a = reinterpret_cast<const uint8_t *>(kv ? p.K : p.Q), *b = reinterpret_cast<const uint8_t *>(kv ? p.V : p.dO);
+                    gather_rows(dst, a, true, b - a, now, i < 0 ? rows_h : (t.w + 15) & ~15, lw, lane);
                 }
+                cp_async_arrive(bar_full);
                 __syncwarp();
+                if (bulk && lw == 0) {
+                    if (leader) {
+                        mbar_arrive_expect_tx(bar_full, 2 * kTileBytes);
+                        tma_load_2d(dst, kv ? &p.tmK : &p.tmQ, 0, (int)bh + t.first(), bar_full);
+                        tma_load_2d(dst + kTileBytes, kv ? &p.tmV : &p.tmdO, 0, (int)bh + t.first(), bar_full);
+                    }
+                    __syncwarp();
+                } else if (lane == 0) {
+                    mbar_arrive(bar_full);
+                }
             }
             c_cnt += tiles.n;
-            step += 1 + tiles.n;
         }
     }
 
@@ -786,13 +781,13 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     float *D = (float *)(ws + 256);
     float *nlse = D + align256((size_t)plan->B * plan->H * plan->N * sizeof(float)) / sizeof(float);
     Params<kMany> p;
-    struct {
-        CUtensorMap *box, *row;
-        const void *x;
-    } maps[] = {{&p.tmQ, &p.tmQ1, Q}, {&p.tmK, &p.tmK1, K}, {&p.tmV, &p.tmV1, V}, {&p.tmdO, &p.tmdO1, dO}};
     if (rows >= (size_t(1) << 31)) return MATE_ERR_UNSUPPORTED;
-    for (const auto &m : maps)
-        if (!make_row_map(m.box, m.x, rows) || !make_row_map(m.row, m.x, rows, 1)) return MATE_ERR_CUDA;
+    if (!make_row_map(&p.tmQ, Q, rows) || !make_row_map(&p.tmK, K, rows) || !make_row_map(&p.tmV, V, rows) || !make_row_map(&p.tmdO, dO, rows))
+        return MATE_ERR_CUDA;
+    p.Q = (const __nv_bfloat16 *)Q;
+    p.K = (const __nv_bfloat16 *)K;
+    p.V = (const __nv_bfloat16 *)V;
+    p.dO = (const __nv_bfloat16 *)dO;
     p.nlse = nlse;
     p.D = D;
     for (int i = 0; i < p.kO; ++i) {

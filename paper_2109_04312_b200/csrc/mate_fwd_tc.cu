@@ -69,8 +69,8 @@ constexpr int kLoadWarps = 4;
 static_assert(kTile == 32 * kLoadWarps, "a row of a tile per loader thread");
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
 constexpr int kStages = 4;                   // K/V ring
-using QRing = LoadRing<2, 2>;  // every loader warp has a part in every load
-using KVRing = LoadRing<kStages, kStages>;
+using QRing = LoadRing<2>;
+using KVRing = LoadRing<kStages>;
 // registers per thread after the roles have split: 256 x 176 + 256 x 80 = 65,536 = the 512 x 128 the CTA is
 // launched with
 constexpr int kRegsSoftmax = 176, kRegsOther = 80;
@@ -891,14 +891,14 @@ EncodeTiledFn encode_tiled_fn() {
 
 }  // namespace
 
-// Map over a [rows, 64] bf16 matrix (row = 128 bytes): boxes of box_rows rows, written to shared memory in
+// Map over a [rows, 64] bf16 matrix (row = 128 bytes): boxes of 128 rows, written to shared memory in
 // the 128-byte swizzle the tensor-core descriptors expect (16-byte chunk index XOR row & 7).
-bool make_row_map(CUtensorMap *map, const void *base, size_t rows, int box_rows) {
+bool make_row_map(CUtensorMap *map, const void *base, size_t rows) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {64, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {kRowBytes};
-    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+    const cuuint32_t box[2] = {64, kTile};
     const cuuint32_t elem[2] = {1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, elem,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,

@@ -11,8 +11,8 @@ namespace mate {
 constexpr int kRowBytes = 128;                 // 64 bf16
 constexpr int kTileBytes = kTile * kRowBytes;  // 16 KB: 128 rows
 
-// Tensor map over a [rows, 64] bf16 matrix in boxes of box_rows rows (false: no tensor maps to be had).
-bool make_row_map(CUtensorMap *map, const void *base, size_t rows, int box_rows = kTile);
+// Tensor map over a [rows, 64] bf16 matrix in boxes of 128 rows (false: no tensor maps to be had).
+bool make_row_map(CUtensorMap *map, const void *base, size_t rows);
 
 // The loaders copy a tile of up to 128 rows (128 B each), warp w of the four the rows 32 w .. 32 w + 31.
 // A lane looks up the original position of one row (coalesced, one latency for the whole tile, and cheap
@@ -54,26 +54,6 @@ __device__ __forceinline__ void gather_rows(uint32_t s_a, const uint8_t *a_bh, b
         const uint32_t dst = (d ^ ((i & 1) << 6)) + 4 * i * kRowBytes;
         ptx::cp_async16(dst, src);
         if (pair) ptx::cp_async16(dst + kTileBytes, src + b_off);
-    }
-}
-
-// Tile rows r0 .. r0 + n_rows - 1 (at most 64; up to a multiple of four) of two tensors, by index: -> tiles at s_a and 16 KB
-// behind it, 128-byte swizzle, four rows per copy.  idx: the tensors' rows for tile rows r0 + lane and r0 + 32 + lane.  The
-// whole warp takes part, its leader issues; the copies count on `bar` (gather_bytes per tensor).
-__device__ __forceinline__ uint32_t gather_bytes(int n_rows) { return (uint32_t)((n_rows + 3) >> 2) * 4 * kRowBytes; }
-template <int kUnroll>
-__device__ __forceinline__ void gather_rows4(uint32_t s_a, const CUtensorMap *map_a, const CUtensorMap *map_b, const int (&idx)[2], int r0,
-                                             int n_rows, bool leader, uint32_t bar) {
-    s_a += r0 * kRowBytes;
-#pragma unroll kUnroll
-    for (int g = 0; 4 * g < n_rows; ++g, s_a += 4 * kRowBytes) {
-        const int v = g < 8 ? idx[0] : idx[1], l = 4 * (g & 7);
-        const int y0 = __shfl_sync(0xffffffffu, v, l), y1 = __shfl_sync(0xffffffffu, v, l + 1), y2 = __shfl_sync(0xffffffffu, v, l + 2),
-                  y3 = __shfl_sync(0xffffffffu, v, l + 3);
-        if (leader) {
-            ptx::tma_gather4(s_a, map_a, y0, y1, y2, y3, bar);
-            if (map_b) ptx::tma_gather4(s_a + kTileBytes, map_b, y0, y1, y2, y3, bar);
-        }
     }
 }
 

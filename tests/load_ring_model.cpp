@@ -12,6 +12,8 @@
 namespace {
 
 constexpr uint32_t kTileBufs = 4, kRecords = 4, kLoadWarps = 4;
+using Rows = mate::LoadRing<2>;
+using Tiles = mate::LoadRing<kTileBufs>;
 
 struct Barrier {
     int count = 1, pending = 1;
@@ -82,7 +84,7 @@ struct Model {
 };
 
 // Loaders: the rows of every item, then its tiles, in turn by kTeams teams of warps; warp 0 also publishes the records.
-template <class Rows, class Tiles, uint32_t kTeams>
+template <uint32_t kTeams>
 void loaders(Model &m, const std::vector<int> &tiles, const std::vector<int> &sched_full, const std::vector<int> &sched_empty,
              const std::vector<int> &row_full, const std::vector<int> &row_empty, const std::vector<int> &tile_full,
              const std::vector<int> &tile_empty) {
@@ -100,10 +102,8 @@ void loaders(Model &m, const std::vector<int> &tiles, const std::vector<int> &sc
             for (int i = -1; i < tiles[n]; ++i, ++step) {
                 if (step % kTeams == w * kTeams / kLoadWarps) {
                     const uint32_t load = i < 0 ? n : c;
-                    const int64_t before = i < 0 ? (int64_t)n - 2 : (int64_t)c - kTileBufs;  // the load whose release is awaited
-                    const uint32_t bars = i < 0 ? Rows::kEmpty : Tiles::kEmpty;
-                    ops.push_back({Op::kWait, i < 0 ? row_empty[Rows::wait_empty(load)] : tile_empty[Tiles::wait_empty(load)],
-                                   i < 0 ? Rows::wait_parity(load) : Tiles::wait_parity(load), before < 0 ? 0 : before / bars + 1});
+                    ops.push_back({Op::kWait, i < 0 ? row_empty[Rows::buffer(load)] : tile_empty[Tiles::buffer(load)],
+                                   i < 0 ? Rows::wait_parity(load) : Tiles::wait_parity(load), load / (i < 0 ? 2 : kTileBufs)});
                     ops.push_back({Op::kLater, i < 0 ? row_full[Rows::buffer(load)] : tile_full[Tiles::buffer(load)]});
                 }
                 if (i >= 0) ++c;
@@ -113,15 +113,15 @@ void loaders(Model &m, const std::vector<int> &tiles, const std::vector<int> &sc
     }
 }
 
-template <class Rows, class Tiles, uint32_t kTeams>
+template <uint32_t kTeams>
 Model backward(const std::vector<int> &tiles) {
     Model m;
     const int n_math = 2, n_store = 2, readers = n_math + n_store + 2 + kLoadWarps, parts = kLoadWarps / kTeams;
     const auto sched_full = m.add(kRecords, 1), sched_empty = m.add(kRecords, readers), row_full = m.add(2, parts),
-               row_empty = m.add(Rows::kEmpty, 1 + n_math + n_store), tile_full = m.add(kTileBufs, parts),
-               tile_empty = m.add(Tiles::kEmpty, 1);
+               row_empty = m.add(2, 1 + n_math + n_store), tile_full = m.add(kTileBufs, parts),
+               tile_empty = m.add(kTileBufs, 1);
     const int s_full = m.add(1), a_full = m.add(n_math), g_done = m.add(1), st_free = m.add(n_math), item_done = m.add(1), acc_free = m.add(n_store);
-    loaders<Rows, Tiles, kTeams>(m, tiles, sched_full, sched_empty, row_full, row_empty, tile_full, tile_empty);
+    loaders<kTeams>(m, tiles, sched_full, sched_empty, row_full, row_empty, tile_full, tile_empty);
     const uint32_t N = (uint32_t)tiles.size();
     const auto record = [&](std::vector<Op> &o, uint32_t n) { o.push_back(wait(sched_full[n % kRecords], n / kRecords)); };
     const auto rows = [&](std::vector<Op> &o, uint32_t n) { o.push_back({Op::kWait, row_full[Rows::buffer(n)], Rows::full_parity(n), n / 2 + 1}); };
@@ -132,7 +132,7 @@ Model backward(const std::vector<int> &tiles) {
         for (auto *o : {&store, &s, &g}) o->push_back({Op::kArrive, sched_empty[n % kRecords]});
         if (n == N) break;
         for (auto *o : {&math, &store, &s}) rows(*o, n);
-        store.push_back({Op::kArrive, row_empty[Rows::empty(n)]});
+        store.push_back({Op::kArrive, row_empty[Rows::buffer(n)]});
         if (tiles[n] > 0) {
             g.push_back(wait(acc_free, (int64_t)with_tiles - 1));
             store.push_back(wait(item_done, with_tiles));
@@ -149,11 +149,11 @@ Model backward(const std::vector<int> &tiles) {
             math.push_back({Op::kArrive, a_full});
             g.push_back(wait(a_full, c));
             g.push_back({Op::kLater, g_done});
-            g.push_back({Op::kLater, tile_empty[Tiles::empty(c)]});
+            g.push_back({Op::kLater, tile_empty[Tiles::buffer(c)]});
             if (i + 1 == tiles[n]) g.push_back({Op::kLater, item_done});
         }
-        s.push_back({Op::kLater, row_empty[Rows::empty(n)]});
-        math.push_back({Op::kArrive, row_empty[Rows::empty(n)]});
+        s.push_back({Op::kLater, row_empty[Rows::buffer(n)]});
+        math.push_back({Op::kArrive, row_empty[Rows::buffer(n)]});
         math.push_back({Op::kArrive, sched_empty[n % kRecords]});
     }
     m.roles.insert(m.roles.end(), {math, math, store, store, s, g});
@@ -161,13 +161,13 @@ Model backward(const std::vector<int> &tiles) {
 }
 
 // visits[n][h]: bit i set where half h visits tile i of item n
-template <class Rows, class Tiles, uint32_t kTeams>
+template <uint32_t kTeams>
 Model forward(const std::vector<int> &tiles, const std::vector<uint32_t> (&visits)[2]) {
     Model m;
     const int readers = 2 + 2 + kLoadWarps, parts = kLoadWarps / kTeams;
     const auto sched_full = m.add(kRecords, 1), sched_empty = m.add(kRecords, readers), row_full = m.add(2, parts),
-               row_empty = m.add(Rows::kEmpty, 2 + 2), tile_full = m.add(kTileBufs, parts), tile_empty = m.add(Tiles::kEmpty, 2);
-    loaders<Rows, Tiles, kTeams>(m, tiles, sched_full, sched_empty, row_full, row_empty, tile_full, tile_empty);
+               row_empty = m.add(2, 2 + 2), tile_full = m.add(kTileBufs, parts), tile_empty = m.add(kTileBufs, 2);
+    loaders<kTeams>(m, tiles, sched_full, sched_empty, row_full, row_empty, tile_full, tile_empty);
     const uint32_t N = (uint32_t)tiles.size();
     for (int h = 0; h < 2; ++h) {
         const int s_full = m.add(1), s_free = m.add(1), p_full = m.add(1), pv_done = m.add(1);
@@ -191,11 +191,11 @@ Model forward(const std::vector<int> &tiles, const std::vector<uint32_t> (&visit
                 if (out) {
                     mma.push_back(wait(p_full, (int64_t)seen - 1));
                     mma.push_back({Op::kLater, pv_done});
-                    mma.push_back({Op::kLater, tile_empty[Tiles::empty(c + i - 1)]});
+                    mma.push_back({Op::kLater, tile_empty[Tiles::buffer(c + i - 1)]});
                 }
                 if (!visit && i < tiles[n]) {
                     mma.push_back({Op::kWait, tile_full[Tiles::buffer(c + i)], Tiles::full_parity(c + i), (c + i) / kTileBufs + 1});
-                    mma.push_back({Op::kArrive, tile_empty[Tiles::empty(c + i)]});
+                    mma.push_back({Op::kArrive, tile_empty[Tiles::buffer(c + i)]});
                 }
                 if (visit) {
                     soft.push_back(wait(s_full, seen));
@@ -208,8 +208,8 @@ Model forward(const std::vector<int> &tiles, const std::vector<uint32_t> (&visit
             }
             if (in_unit > 0) soft.push_back(wait(pv_done, (int64_t)seen - 1));
             c += tiles[n];
-            mma.push_back({Op::kLater, row_empty[Rows::empty(n)]});
-            soft.push_back({Op::kArrive, row_empty[Rows::empty(n)]});
+            mma.push_back({Op::kLater, row_empty[Rows::buffer(n)]});
+            soft.push_back({Op::kArrive, row_empty[Rows::buffer(n)]});
             soft.push_back({Op::kArrive, sched_empty[n % kRecords]});
         }
         m.roles.push_back(mma);
@@ -220,7 +220,7 @@ Model forward(const std::vector<int> &tiles, const std::vector<uint32_t> (&visit
 
 // Random lists of up to 14 items of up to `most` tiles, half of them longest first: runs with an early wait in out[0], runs
 // that stand still in out[1].
-template <class Rows, class Tiles, uint32_t kTeams>
+template <uint32_t kTeams>
 void lists(bool bwd, int runs, int most, uint32_t seed, int *out) {
     std::mt19937 rng(seed);
     out[0] = out[1] = 0;
@@ -231,7 +231,7 @@ void lists(bool bwd, int runs, int most, uint32_t seed, int *out) {
         std::vector<uint32_t> visits[2];
         for (auto &v : visits)
             for (size_t n = 0; n < tiles.size(); ++n) v.push_back(rng() % 4 ? (rng() % 2 ? ~0u : (uint32_t)rng()) : 0);
-        Model m = bwd ? backward<Rows, Tiles, kTeams>(tiles) : forward<Rows, Tiles, kTeams>(tiles, visits);
+        Model m = bwd ? backward<kTeams>(tiles) : forward<kTeams>(tiles, visits);
         const int what = m.run(rng);
         if (what) ++out[what - 1];
     }
@@ -239,14 +239,6 @@ void lists(bool bwd, int runs, int most, uint32_t seed, int *out) {
 
 }  // namespace
 
-using OneRows = mate::LoadRing<2, 2>;
-using OneTiles = mate::LoadRing<kTileBufs, kTileBufs>;
-
-extern "C" void as_built(int bwd, int runs, int most, unsigned seed, int *out) {
-    if (bwd) lists<mate::LoadRing<2>, mate::LoadRing<kTileBufs>, 2>(true, runs, most, seed, out);
-    else lists<OneRows, OneTiles, 1>(false, runs, most, seed, out);
-}
-// loads by two teams in turn, one barrier per buffer
-extern "C" void teams(int bwd, int runs, int most, unsigned seed, int *out) {
-    lists<OneRows, OneTiles, 2>(bwd != 0, runs, most, seed, out);
-}
+extern "C" void as_built(int bwd, int runs, int most, unsigned seed, int *out) { lists<1>(bwd != 0, runs, most, seed, out); }
+// loads by two teams of warps in turn
+extern "C" void teams(int bwd, int runs, int most, unsigned seed, int *out) { lists<2>(bwd != 0, runs, most, seed, out); }

@@ -196,8 +196,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = tid & 31;
 
     // The first loader warp hands out the units; its lanes 0-3 hold the record of the next one.  The first unit of
-    // a CTA is its own index, later ones come from the shared counter, each claimed when the loaders
-    // reach the last tile of the unit before it; the number and then the record travel under the copies.  Every CTA's last claim fails, so the claims of a
+    // a CTA is its own index, later ones come from the shared counter, each claimed under the last tiles of the unit
+    // before it.  Every CTA's last claim fails, so the claims of a
     // launch number n_units: the one that draws the last number puts the counter back to zero for the next launch.
     int4 rec = make_int4(0, 0, 0, 0);
     int u_next = blockIdx.x;  // lane 0
@@ -806,7 +806,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
             for (int i = -2; i < n_tiles; ++i) {
                 const int now = next;
                 if (i + 1 < n_tiles) next = step_idx(i + 1);
-                else if (warp == kLoadWarp0 && !redo) claim();  // the number of the next unit travels under the copies
                 const uint32_t c = kv_cnt + max(i, 0), stage = KVRing::buffer(c);
                 const uint32_t bar_full = bars + 8 * (i < 0 ? kBarQFull + qb : kBarKVFull + stage);
                 if (i != -1 && !(alive = wait(bars + 8 * (i < 0 ? kBarQEmpty + qb : kBarKVEmpty + stage),
@@ -848,8 +847,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                 TR_INC(4);
             }
             if (warp == kLoadWarp0 && alive) {
-                if (redo) rec = held_back;
-                else fetch_record(true);
+                if (redo) {
+                    rec = held_back;
+                } else {
+                    // The next unit is claimed when the fourth tile from the end has been read (the first tile, of a shorter unit).
+                    // Claimed before that it goes to a CTA that is not the next to be free, claimed much later its loads are late.
+                    // As soon as every load is under way / so / at the second tile from the end, forward alone: 8 x 512
+                    // tokens 15.9 / 15.3 / 15.4 us, 4 x 2048 30.2 / 29.6 / 30.0, 1 x 8192 53.2 / 49.7 / 51.1, 2 x 4096 51.7 / 51.4 /
+                    // 54.3.  Units of one tile do not wait: nothing would be left to hide the claim behind.
+                    const uint32_t c = kv_cnt + max(n_tiles - 4, 0);
+                    if (n_tiles > 1 && !(alive = wait(bars + 8 * (kBarKVEmpty + KVRing::buffer(c)), KVRing::wait_parity(c + kStages)))) break;
+                    claim();
+                    fetch_record(true);
+                }
             }
             kv_cnt += n_tiles;
         }

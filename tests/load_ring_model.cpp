@@ -83,11 +83,12 @@ struct Model {
     }
 };
 
-// Loaders: the rows of every item, then its tiles, in turn by kTeams teams of warps; warp 0 also publishes the records.
+// Loaders: the rows of every item, then its tiles, in turn by kTeams teams of warps; warp 0 also publishes the records, in the
+// forward (`claims`) not before the fourth tile from the end of the item before has been read.
 template <uint32_t kTeams>
 void loaders(Model &m, const std::vector<int> &tiles, const std::vector<int> &sched_full, const std::vector<int> &sched_empty,
              const std::vector<int> &row_full, const std::vector<int> &row_empty, const std::vector<int> &tile_full,
-             const std::vector<int> &tile_empty) {
+             const std::vector<int> &tile_empty, bool claims) {
     for (uint32_t w = 0; w < kLoadWarps; ++w) {
         std::vector<Op> ops;
         uint32_t step = 0, c = 0;
@@ -108,6 +109,10 @@ void loaders(Model &m, const std::vector<int> &tiles, const std::vector<int> &sc
                 }
                 if (i >= 0) ++c;
             }
+            if (claims && w == 0 && tiles[n] > 1) {
+                const uint32_t read = c - std::min(tiles[n], 4);
+                ops.push_back({Op::kWait, tile_empty[Tiles::buffer(read)], Tiles::wait_parity(read + kTileBufs), read / kTileBufs + 1});
+            }
         }
         m.roles.push_back(ops);
     }
@@ -121,7 +126,7 @@ Model backward(const std::vector<int> &tiles) {
                row_empty = m.add(2, 1 + n_math + n_store), tile_full = m.add(kTileBufs, parts),
                tile_empty = m.add(kTileBufs, 1);
     const int s_full = m.add(1), a_full = m.add(n_math), g_done = m.add(1), st_free = m.add(n_math), item_done = m.add(1), acc_free = m.add(n_store);
-    loaders<kTeams>(m, tiles, sched_full, sched_empty, row_full, row_empty, tile_full, tile_empty);
+    loaders<kTeams>(m, tiles, sched_full, sched_empty, row_full, row_empty, tile_full, tile_empty, false);
     const uint32_t N = (uint32_t)tiles.size();
     const auto record = [&](std::vector<Op> &o, uint32_t n) { o.push_back(wait(sched_full[n % kRecords], n / kRecords)); };
     const auto rows = [&](std::vector<Op> &o, uint32_t n) { o.push_back({Op::kWait, row_full[Rows::buffer(n)], Rows::full_parity(n), n / 2 + 1}); };
@@ -167,7 +172,7 @@ Model forward(const std::vector<int> &tiles, const std::vector<uint32_t> (&visit
     const int readers = 2 + 2 + kLoadWarps, parts = kLoadWarps / kTeams;
     const auto sched_full = m.add(kRecords, 1), sched_empty = m.add(kRecords, readers), row_full = m.add(2, parts),
                row_empty = m.add(2, 2 + 2), tile_full = m.add(kTileBufs, parts), tile_empty = m.add(kTileBufs, 2);
-    loaders<kTeams>(m, tiles, sched_full, sched_empty, row_full, row_empty, tile_full, tile_empty);
+    loaders<kTeams>(m, tiles, sched_full, sched_empty, row_full, row_empty, tile_full, tile_empty, true);
     const uint32_t N = (uint32_t)tiles.size();
     for (int h = 0; h < 2; ++h) {
         const int s_full = m.add(1), s_free = m.add(1), p_full = m.add(1), pv_done = m.add(1);

@@ -32,9 +32,9 @@
 //   - Two threads per row (four warps per scheduler) hide the latencies as well, but the control flow of twice
 //     the warps takes more issue slots than that gains.
 //   - The instruction cache is about 32 KB for all roles of the CTA; straight-line code that misses it issues
-//     at a third of the rate, from L2 at a sixth.  Rarely taken paths are rolled, there is one path for exact units, and
-//     the padding rows' loop is not unrolled (it was 8 of 69 KB): 59 KB.  8 x 512 tokens 17.9 -> 17.7 us, 4 x 2048 33.6 -> 33.0,
-//     2 x 4096 54.9 -> 54.5, packed 37.9 -> 37.3.
+//     at a third of the rate, from L2 at a sixth.  Rarely taken paths are rolled, and
+//     the padding rows' loop is not unrolled (it was 8 KB).  Exact units have the path of full tiles all the same: on large
+//     scores 4 x 2048 tokens take 60.0 us with it and 72.6 without, 1 x 8192 99.7 and 121.8, others the same.
 // Key tiles of range B are visited by a half only where they meet the segments of its rows, and inside
 // a tile a warp evaluates only the 32-column chunks that meet the segments of its 32 rows.  The scatter
 // back to the original token order is fused into the epilogue.
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                         tmem_st8(tO + c2 * 8, o);
                     }
                 };
-                if (!exact && (j < fa || (j >= fb0 && j < fb1))) {
+                if (j < fa || (j >= fb0 && j < fb1)) {
                     uint32_t v[4][32];
 #pragma unroll
                     for (int ch = 0; ch < 4; ++ch) tmem_ld32(tS + ch * 32, v[ch]);
@@ -399,12 +399,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                     for (int ch = 0; ch < 4; ++ch) reg_fence(v[ch]);
                     tc_fence_before();  // S may be overwritten
                     if (lane == 0) mbar_arrive(bar_sf);
-                    if (j == 0) {  // base of the row: the max over its first tile
+                    if (j == 0 || exact) {  // base of the row: the max over its first tile, or, exactly, over every tile
                         float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
                         for (int ch = 0; ch < 4; ++ch) chunk_max(v[ch], tm);
-                        const float t2 = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2;
-                        m2 = t2 == -INFINITY ? 0.f : t2;
+                        new_base(fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2);
                     }
                     const uint64_t neg_m2 = pack_f32x2(-m2, -m2);
 #pragma unroll

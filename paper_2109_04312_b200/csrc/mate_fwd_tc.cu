@@ -385,6 +385,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                         uint32_t o[8];
                         tmem_ld8(tO + c2 * 8, o);
                         tc_wait_ld();
+                        reg_fence(o);
 #pragma unroll
                         for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
                         tmem_st8(tO + c2 * 8, o);
@@ -512,6 +513,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                     if (n_visit > 0) {
                         tmem_ld16(tO + c2 * 16, o);
                         tc_wait_ld();
+                        reg_fence(o);
                     } else {
 #pragma unroll
                         for (int e = 0; e < 16; ++e) o[e] = 0u;

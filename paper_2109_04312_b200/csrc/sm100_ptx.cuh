@@ -239,6 +239,12 @@ __device__ __forceinline__ void reg_fence(uint32_t (&v)[16]) {
                  :
                  : "memory");
 }
+__device__ __forceinline__ void reg_fence(uint32_t (&v)[8]) {
+    asm volatile(""
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
+                 :
+                 : "memory");
+}
 
 // 32 lanes x 16 consecutive 32-bit columns: thread i of the warp gets lane (base_lane + i)
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {

@@ -360,7 +360,7 @@ void make_bwd_units(mate_plan_t *pl, const ProtoList &singles, const HeadLists &
         for (int h : heads.heads[pr.view]) {
             pl->bwd_costs.push_back(pr.cost);
             pl->bwd_units.push_back(pr.u);
-            pl->bwd_units.back().hv = h | pr.view << mate::kViewShift;
+            pl->bwd_units.back().hv = mate::pack_hv(h, pr.view);
         }
     pl->n_bwd_units = (int)pl->bwd_units.size();
     pl->bwd_grid = std::min(std::max(pl->n_ctas, 1), std::max(2 * pl->n_bwd_units, pl->n_pads));
@@ -437,7 +437,7 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
             pl->fwd_costs.push_back(e.cost);
             pl->fwd_units.push_back(e.u);
             FwdUnit &u = pl->fwd_units.back();
-            u.hv = h | e.view << mate::kViewShift;
+            u.hv = mate::pack_hv(h, e.view);
             if (u.n_parts() > 1) {
                 u.ctr += k;
                 u.ws_off += (int32_t)((k * u.n_parts() * mate::kPartialBytes) >> 10);
@@ -451,7 +451,7 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
     pl->pads.clear();
     for (int b = 0; b < pl->B; ++b)
         for (int t0 = pl->n_valid[b]; t0 < pl->N; t0 += mate::kPadRows)
-            for (int h = 0; h < pl->H; ++h) pl->pads.push_back({b, h | pl->head_view[h] << mate::kViewShift, t0, std::min(mate::kPadRows, pl->N - t0)});
+            for (int h = 0; h < pl->H; ++h) pl->pads.push_back({b, mate::pack_hv(h, pl->head_view[h]), t0, std::min(mate::kPadRows, pl->N - t0)});
     pl->n_pads = (int)pl->pads.size();
     pl->fwd_grid = std::min(n_ctas, std::max(pl->n_fwd_units, pl->n_pads));
     if (getenv("MATE_LOG"))
@@ -504,7 +504,7 @@ void join_units(mate_plan_t *pl) {
     };
     for (int s = 0; s < 2; ++s) {
         mate_plan_t *sub = pl->sub[s];
-        const auto view = [s](int hv) { return (hv & ((1 << mate::kViewShift) - 1)) | (2 + s) << mate::kViewShift; };
+        const auto view = [s](int32_t hv) { return mate::pack_hv(mate::head_of(hv), 2 + s); };
         for (FwdUnit u : sub->fwd_units) {
             u.hv = view(u.hv);
             if (u.n_parts() > 1) {

@@ -23,7 +23,11 @@ constexpr int kTraceCtas = 256;  // CTAs whose cycle counters a -DMATE_TRACE bui
 __host__ __device__ inline int div_tile(int x, int tB) { return tB == kTile ? x >> 7 : (x >= tB) + (x >= 2 * tB); }
 static_assert(kTile == 128, "div_tile");
 
-constexpr int kViewShift = 28;   // of the view in a record's head: no look-up in front of a unit's first loads
+// A record's head and view in one word: no look-up in front of a unit's first loads.  (The kernels' grids end at 2^30 heads too.)
+constexpr int kViewShift = 30;
+__host__ __device__ inline int32_t pack_hv(int head, int view) { return (int32_t)((uint32_t)head | (uint32_t)view << kViewShift); }
+__host__ __device__ inline int head_of(int32_t hv) { return hv & ((1 << kViewShift) - 1); }
+__host__ __device__ inline int view_of(int32_t hv) { return (int)((uint32_t)hv >> kViewShift); }
 // Views of a work-list: row, column, and the two further passes of a row-or-column plan, which have outputs of their own.
 constexpr int kViews = 4, kPasses = 3;
 __host__ __device__ inline int pass_of(int view) { return view < 2 ? 0 : view - 1; }
@@ -42,7 +46,7 @@ __host__ __device__ inline int pass_of(int view) { return view < 2 ? 0 : view - 
 // partial result to the workspace at ws_off (KiB); per group of 32 rows the part that finishes
 // last (counted in counters[kSchedWords + 8 * ctr + row / 32]) combines them.
 struct alignas(16) FwdUnit {  // (copied as four 16-byte words)
-    int32_t b, hv;             // hv = head | view << kViewShift
+    int32_t b, hv;             // hv = pack_hv(head, view)
     int32_t q0, rows;          // rows = n0 | n1 << 8 | kP << 16; 0 ends a list
     int32_t kA0, kA_end;
     int32_t kB0, kB_end;
@@ -50,8 +54,8 @@ struct alignas(16) FwdUnit {  // (copied as four 16-byte words)
     int32_t tB, parts;         // parts = n_parts | part << 16 (tB: the forward keeps flags above bit 7 on its way)
     int32_t ws_off, ctr;
 
-    __host__ __device__ int head() const { return hv & ((1 << kViewShift) - 1); }
-    __host__ __device__ int view() const { return hv >> kViewShift; }
+    __host__ __device__ int head() const { return head_of(hv); }
+    __host__ __device__ int view() const { return view_of(hv); }
     __host__ __device__ int rows_of(int half) const { return half ? (rows >> 8) & 0xff : rows & 0xff; }
     __host__ __device__ int row0_of(int half) const { return half ? q0 + (rows & 0xff) : q0; }
     __host__ __device__ int kP() const { return rows >> 16; }
@@ -98,8 +102,8 @@ constexpr size_t kPartialBytes = (size_t)kUnitRows * (64 + 4) * sizeof(float);
 constexpr int kPadRows = 64;
 struct PadChunk {
     int32_t b, hv, t0, n;
-    __host__ __device__ int head() const { return hv & ((1 << kViewShift) - 1); }
-    __host__ __device__ int view() const { return hv >> kViewShift; }
+    __host__ __device__ int head() const { return head_of(hv); }
+    __host__ __device__ int view() const { return view_of(hv); }
 };
 
 // Where the rows of example b, head h start in the caller's tensors (in rows of d elements), and how

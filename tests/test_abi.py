@@ -56,6 +56,15 @@ def test_null_arguments_are_rejected_without_a_gpu(lib):
     assert lib.mate_attn_workspace_bytes(None, 64, 0, 0, ctypes.byref(f), ctypes.byref(f)) == -1
 
 
+@pytest.mark.parametrize("H", [1 << 20, 1 << 28, (1 << 29) + 1])
+def test_number_of_heads_is_no_reason_to_refuse(lib, H):
+    # the check of the views comes last: a bad one at the end says that nothing else was refused
+    views = (ctypes.c_uint8 * H)()
+    views[H - 1] = 2
+    ids, out = (ctypes.c_int32 * 1)(), ctypes.c_void_p()
+    assert lib.mate_plan(ids, ids, 1, 1, 0, views, H, 1, 1, None, ctypes.byref(out)) == -1
+
+
 def test_binding_fails_loudly_without_the_library(monkeypatch):
     from paper_2109_04312_b200 import api
     monkeypatch.setattr(api, "_lib", None)

@@ -406,7 +406,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
                         for (int ch = 0; ch < 4; ++ch) chunk_max(v[ch], tm);
                         new_base(fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * p.scale_log2);
                     }
-                    const uint64_t neg_m2 = pack_f32x2(-m2, -m2);
+                    const float neg_m = m2 == -INFINITY ? 0.f : -m2;  // (exact units: no score above -inf so far)
+                    const uint64_t neg_m2 = pack_f32x2(neg_m, neg_m);
 #pragma unroll
                     for (int ch = 0; ch < 4; ++ch) {
                         uint32_t packed[16];

@@ -64,3 +64,15 @@ def test_large_random_scores(value_scale, scale):
     vals = tables.make_values(cfg, info["N"], 77)
     for impl in impls_for(cfg):
         run_case(cfg, rows, cols, vals, impl, backward=(value_scale < 3.0), scale=scale, unit_grads=True)
+
+
+def test_a_whole_tile_out_of_range_in_an_exact_unit():
+    # Row 5 (of the global block: every tile counts in full but for the last) has products of -2^200 with the whole first tile,
+    # -inf in fp32 and a weight of zero; its later scores, standard deviation 50, send the unit through once more
+    cfg, rows, cols, vals = custom_case(300, [(r, 1, 30) for r in range(1, 8)], 520, H=4)
+    rng = np.random.default_rng(6)
+    Q, K = vals["Q"].copy(), vals["K"].copy()
+    Q[:, :, 5] = 12.5 * rng.choice([-1.0, 1.0], size=Q[:, :, 5].shape)
+    Q[..., 0], K[..., 0] = 0.0, 0.0
+    Q[:, :, 5, 0], K[:, :, :128, 0] = 2.0 ** 100, -2.0 ** 100
+    run_case(cfg, rows, cols, dict(vals, Q=Q, K=K), mate().IMPL_TCGEN05, backward=False, scale=1.0)

@@ -120,6 +120,7 @@ struct Params {
     static constexpr int kV = kMany ? kViews : 2, kO = kMany ? kPasses : 1;
     __device__ static __forceinline__ int pass(int view) { return kMany ? pass_of(view) : 0; }
     CUtensorMap tmQ, tmK, tmV, tmdO;  // boxes of 128 rows, 128-byte swizzle
+    int bulk;                         // 0: there are none, every tile is gathered row by row
     const __nv_bfloat16 *Q, *K, *V, *dO;
     const float *nlse, *D;  // per row, original order: -LSE log2 e, D
     __nv_bfloat16 *dQ[kO], *dK[kO], *dV[kO];
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         }
     };
     if (warp == kLoadWarp0) fetch_record(false);
-    if (warp == kLoadWarp0 + 1 && lane < 4) prefetch_tmap(&p.tmQ + lane);  // all four of them
+    if (warp == kLoadWarp0 + 1 && lane < 4) prefetch_tmap(&p.tmQ + lane, p.bulk);  // all four of them
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -683,7 +684,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
             const int32_t *perm = vp.perm + bn;
             const size_t bh = p.tr.base(un.b, un.head());
             // column tiles inside [0, ident) of the order are contiguous in the tensors (see bulk_tile)
-            const int ident = __ldg(vp.ident + un.b);
+            const int ident = p.bulk ? __ldg(vp.ident + un.b) : 0;
             // step -1: the row operands and row data; steps 0 ..: the column tiles
             const int rr = 32 * lw + lane;  // this lane's row of a tile
             auto step_idx = [&](int i) {  // as a row of the tensors
@@ -785,9 +786,8 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     float *D = (float *)(ws + 256);
     float *nlse = D + align256((size_t)plan->B * plan->H * plan->N * sizeof(float)) / sizeof(float);
     Params<kMany> p;
-    if (rows >= (size_t(1) << 31)) return MATE_ERR_UNSUPPORTED;
-    if (!make_row_map(&p.tmQ, Q, rows) || !make_row_map(&p.tmK, K, rows) || !make_row_map(&p.tmV, V, rows) || !make_row_map(&p.tmdO, dO, rows))
-        return MATE_ERR_CUDA;
+    p.bulk = rows < (size_t(1) << 31) && make_row_map(&p.tmQ, Q, rows) && make_row_map(&p.tmK, K, rows) &&
+             make_row_map(&p.tmV, V, rows) && make_row_map(&p.tmdO, dO, rows);
     p.Q = (const __nv_bfloat16 *)Q;
     p.K = (const __nv_bfloat16 *)K;
     p.V = (const __nv_bfloat16 *)V;

@@ -118,7 +118,7 @@ struct Params {
     __device__ static __forceinline__ int pass(int view) { return kMany ? pass_of(view) : 0; }
     // 2-D tensor maps over K and V seen as [B H N rows, 64 columns]: boxes of 128 rows, 128-byte swizzle
     CUtensorMap tmK, tmV;
-    int bulk;        // 0: every tile is gathered row by row
+    int bulk;        // 0: every tile is gathered row by row (the maps may be missing)
     int view_order;  // 1: Q, K, V, O and LSE are laid out in each head's own order (no gather, no scatter)
     const __nv_bfloat16 *Q, *K, *V;
     __nv_bfloat16 *O[kO];
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fwd_kernel(const __grid_consta
         rec = make_int4(0, 0, 0, 0);  // rows = 0: the list is exhausted
         if (u < p.n_units && lane < 4) rec = __ldg(reinterpret_cast<const int4 *>(p.units + u) + lane);
     };
-    if (warp == kLoadWarp0 + 1 && lane < 2) prefetch_tmap(&p.tmK + lane);  // both of them
+    if (warp == kLoadWarp0 + 1 && lane < 2) prefetch_tmap(&p.tmK + lane, p.bulk);  // both of them
     if (warp == kLoadWarp0) fetch_record(false);  // requested before the set-up below, which takes as long
 
     if (tid == 0) {
@@ -932,12 +932,10 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     Params<kMany> p;
     const size_t rows = plan->n_rows();
     // Bulk tensor copies for the K/V tiles that are contiguous in the caller's tensors (see bulk_tile), unless the
-    // caller asks for gathers; tensors in view order always take them.  Bulk copies against gathers, back to back:
+    // caller asks for gathers or there are no maps to be had; tensors in view order always take them.  Bulk copies against gathers, back to back:
     // 4 x 2048 tokens 32.3 us against 32.7, 8 x 512 17.9 and 17.9, 2 x 4096 55.5 and 55.4, 1 x 8192 54.8 and 54.5.
     const bool want_bulk = !(flags & MATE_FLAG_GATHER_TILES) || (flags & MATE_FLAG_VIEW_ORDER);
-    p.bulk = want_bulk ? 1 : 0;
-    if (rows >= (size_t(1) << 31)) return MATE_ERR_UNSUPPORTED;
-    if (!make_row_map(&p.tmK, K, rows) || !make_row_map(&p.tmV, V, rows)) return MATE_ERR_CUDA;
+    p.bulk = want_bulk && rows < (size_t(1) << 31) && make_row_map(&p.tmK, K, rows) && make_row_map(&p.tmV, V, rows);
     p.view_order = (flags & MATE_FLAG_VIEW_ORDER) ? 1 : 0;
     p.Q = (const __nv_bfloat16 *)Q;
     p.K = (const __nv_bfloat16 *)K;

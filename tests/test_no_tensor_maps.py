@@ -1,0 +1,30 @@
+"""A driver that hands out no tensor maps is no reason to refuse a call: the tensor-core kernels then gather every tile row by
+row.  Their host side on a CUDA runtime of host functions (tests/launch_on_fake_cuda.cpp).  No GPU."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2109_04312_b200", "csrc")
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    so = str(tmp_path_factory.mktemp("launch") / "launch.so")
+    # device code as PTX only: none of it is run
+    subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "-shared", "-Xcompiler", "-fPIC",
+                    "-Xlinker", "-Bsymbolic", "-cudart", "none", "-I", CSRC, "-I", os.path.join(ROOT, "include"), "-o", so,
+                    os.path.join(CSRC, "mate_fwd_tc.cu"), os.path.join(CSRC, "mate_bwd_tc.cu"),
+                    os.path.join(ROOT, "tests", "launch_on_fake_cuda.cpp")], check=True)
+    return ctypes.CDLL(so)
+
+
+@pytest.mark.parametrize("backward,launches", [(0, 1), (1, 2)])
+def test_calls_go_through_without_maps(lib, backward, launches):
+    n, bulk = ctypes.c_int(), ctypes.c_int()
+    assert lib.call(backward, ctypes.byref(n), ctypes.byref(bulk)) == 0
+    assert (n.value, bulk.value) == (launches, 0)

@@ -349,16 +349,14 @@ void list_units(const mate_plan_t *pl, const std::vector<RowRanges> &ranges, boo
 // Backward: single halves, none split; its work items are the units, once per side.  Longest first: the CTAs of
 // the persistent kernel take work from the head of the list as they become free (a shared counter), so the
 // order is the whole schedule.
-void make_bwd_units(mate_plan_t *pl, const ProtoList &singles, const HeadLists &heads) {
+void make_bwd_units(mate_plan_t *pl, const ProtoList &singles, const HeadLists &heads, bool costs) {
     size_t n = 0;
     for (const Proto &pr : singles.protos) n += heads.heads[pr.view].size();
     pl->bwd_units.clear();
-    pl->bwd_costs.clear();
     pl->bwd_units.reserve(n);
-    pl->bwd_costs.reserve(n);
     for (const Proto &pr : singles.protos)
         for (int h : heads.heads[pr.view]) {
-            pl->bwd_costs.push_back(pr.cost);
+            if (costs) pl->bwd_costs.push_back(pr.cost);
             pl->bwd_units.push_back(pr.u);
             pl->bwd_units.back().hv = mate::pack_hv(h, pr.view);
         }
@@ -380,7 +378,7 @@ FwdUnit slice_unit(const FwdUnit &u, int i0, int i1) {
 
 // Forward.  A unit of more than 1.3 of a CTA's share of the clocks is cut between tiles into parts of about
 // 0.75 of it (never less than four tiles), to be combined in the kernel; longest first, as for the backward.
-void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const HeadLists &heads) {
+void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const HeadLists &heads, bool costs) {
     const int n_ctas = std::max(pl->n_ctas, 1);
     ProtoList list;
     list_units(pl, ranges, true, false, list);
@@ -429,12 +427,10 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
     std::stable_sort(entries.begin(), entries.end(), [](const Entry &a, const Entry &b) { return a.cost > b.cost; });
     pl->fwd_units.clear();
     pl->fwd_units.reserve(n_units);
-    pl->fwd_costs.clear();
-    pl->fwd_costs.reserve(n_units);
     for (const Entry &e : entries) {
         int k = 0;
         for (int h : heads.heads[e.view]) {
-            pl->fwd_costs.push_back(e.cost);
+            if (costs) pl->fwd_costs.push_back(e.cost);
             pl->fwd_units.push_back(e.u);
             FwdUnit &u = pl->fwd_units.back();
             u.hv = mate::pack_hv(h, e.view);
@@ -461,7 +457,8 @@ void make_fwd_units(mate_plan_t *pl, const std::vector<RowRanges> &ranges, const
                 entries.empty() ? 0ll : (long long)entries.front().cost, pl->fwd_ws_bytes, pl->n_pads);
 }
 
-void build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2]) {
+// costs: the lists are to be joined with others (join_units).
+void build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2], bool costs) {
     static_assert(mate::kPartialBytes % 1024 == 0, "ws_off counts KiB");
     std::vector<RowRanges> ranges((size_t)2 * pl->B);
     for (int v = 0; v < 2; ++v)
@@ -476,13 +473,13 @@ void build_units(mate_plan_t *pl, const int32_t *const (&seg_off_host)[2]) {
         }
 
     const HeadLists heads(pl);
-    make_fwd_units(pl, ranges, heads);
+    make_fwd_units(pl, ranges, heads, costs);
     size_t n_halves = 0;
     for (int v = 0; v < 2; ++v)
         for (int b = 0; b < pl->B; ++b) n_halves += heads.heads[v].size() * ceil_div(ranges[(size_t)v * pl->B + b].nv, kTile);
     ProtoList singles;
     list_units(pl, ranges, false, n_halves > (size_t)std::max(pl->n_ctas, 1), singles);
-    make_bwd_units(pl, singles, heads);
+    make_bwd_units(pl, singles, heads, costs);
 }
 
 // Row-or-column plan: the lists of the two further passes join this plan's, longest first again, so that one launch
@@ -528,6 +525,7 @@ void join_units(mate_plan_t *pl) {
     }
     by_cost(pl->fwd_units, pl->fwd_costs);
     by_cost(pl->bwd_units, pl->bwd_costs);
+    for (mate_plan_t *x : {pl, pl->sub[0], pl->sub[1]}) x->fwd_costs = x->bwd_costs = {};
     pl->n_fwd_slots = slots;
     pl->n_fwd_units = (int)pl->fwd_units.size();
     pl->n_bwd_units = (int)pl->bwd_units.size();
@@ -799,7 +797,7 @@ static int fill_plan(mate_plan_t *pl, mate::Staging &host, const int32_t *row_id
     if (out_host(pl->status_dev)[0] != 0) return MATE_ERR_INVALID_ARG;
     pl->n_valid.assign(out_host(pl->n_valid_dev), out_host(pl->n_valid_dev) + B);
     const int32_t *seg_off_host[2] = {out_host(pl->view[0].seg_off), out_host(pl->view[1].seg_off)};
-    build_units(pl, seg_off_host);
+    build_units(pl, seg_off_host, !upload);
     return upload ? upload_units(pl, st) : MATE_OK;
 }
 

@@ -75,8 +75,7 @@ enum { MATE_IMPL_AUTO = 0, MATE_IMPL_SIMT = 1, MATE_IMPL_TCGEN05 = 2 };
  *                instead of row-by-row gathers.  Same results bit for bit.  This is the default wherever
  *                the driver provides tensor maps, so the bit only states it.
  *   GATHER_TILES every K/V tile is gathered row by row.  (Timed back to back on sequences of 512 to
- *                8192 positions, bulk copies are 1 % faster on one workload and within 0.6 % on the
- *                others.)  Both bits together: MATE_ERR_INVALID_ARG. */
+ *                8192 positions, bulk copies are up to 0.7 % faster.)  Both bits together: MATE_ERR_INVALID_ARG. */
 enum { MATE_FLAG_VIEW_ORDER = 4, MATE_FLAG_BULK_TILES = 8, MATE_FLAG_GATHER_TILES = 16 };
 
 const char *mate_status_string(int status);

@@ -32,16 +32,16 @@
 //     first chunk's arithmetic.
 //   - The arithmetic warps have no part in an item's end: the store warps wait for its last gradient MMAs (700 clk
 //     behind the last operands) and take the gradients out of tensor memory under the next item's first tile.
-//   - A load costs a warp about 1700 clk of look-up, waiting and issuing (its instructions queue behind the exponentials),
-//     with a position's latency in it; two teams keep two loads under way.  The copies complete on the
-//     tile's barrier by themselves, so no warp waits for them to signal.
-//   - All roles share an instruction cache of about 32 KB: waits and rare paths are rolled, gathers are a loop of 15
-//     instructions.  (With the gathers and waits unrolled, 68 KB of code instead of 54, the same kernel takes 92 us for
-//     4 x 2048 tokens: a warp waits for instructions 3.9 times as long as it issues, instead of 0.7.)
+//   - All loader warps take part in every load, with the look-ups a tile ahead of the copies.  (Tensor copies of four rows by
+//     teams of two warps that take the loads in turn: 1 x 512 tokens 10.5 us, 4 x 2048 58.3, 1 x 8192 108.3 against 10.0, 56.1,
+//     104.9.)
+//   - All roles share an instruction cache of about 32 KB: waits and rare paths are rolled.  (An earlier form with gathers and
+//     waits unrolled, 14 KB more, took 92 us for 4 x 2048 tokens: a warp waited for instructions 3.9 times as long as it
+//     issued, instead of 0.7.)
 //   - The tensor maps are fetched ahead of the first copy (4 x 2048 tokens, forward and backward, 99.4 us without, 98.0 with).
-// With one warp for all MMAs, cp.async gathers by four warps and the epilogue in the arithmetic warps, forward and backward
-// back to back took 47.7 us for 8 x 512 tokens, 101.8 for 4 x 2048, 176.0 for 1 x 8192 and 172.9 for 2 x 4096; with this form
-// 46.4, 98.1, 165.6 and 162.7.
+// Forward and backward back to back, 8 x 512 tokens / 4 x 2048 / 1 x 8192 / 2 x 4096: one warp for all MMAs and the epilogue in the
+// arithmetic warps 47.7 / 101.8 / 176.0 / 172.9 us; with store warps and two MMA warps, gathers by tensor copies 46.4 / 98.1 /
+// 165.6 / 162.7 (backward alone 23.0 / 59.6 / 107.7 / 102.1); this form 41.1 / 86.9 / 160.1 / 155.6 (22.3 / 57.8 / 104.2 / 100.0).
 #include <cuda.h>
 #include <cuda_bf16.h>
 

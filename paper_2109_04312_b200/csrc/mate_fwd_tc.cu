@@ -933,7 +933,7 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     const size_t rows = plan->n_rows();
     // Bulk tensor copies for the K/V tiles that are contiguous in the caller's tensors (see bulk_tile), unless the
     // caller asks for gathers or there are no maps to be had; tensors in view order always take them.  Bulk copies against gathers, back to back:
-    // 4 x 2048 tokens 32.3 us against 32.7, 8 x 512 17.9 and 17.9, 2 x 4096 55.5 and 55.4, 1 x 8192 54.8 and 54.5.
+    // 4 x 2048 tokens 29.4 us against 29.5, 8 x 512 15.5 and 15.5, 2 x 4096 51.1 and 51.5, 1 x 8192 48.6 and 48.8.
     const bool want_bulk = !(flags & MATE_FLAG_GATHER_TILES) || (flags & MATE_FLAG_VIEW_ORDER);
     p.bulk = want_bulk && rows < (size_t(1) << 31) && make_row_map(&p.tmK, K, rows) && make_row_map(&p.tmV, V, rows);
     p.view_order = (flags & MATE_FLAG_VIEW_ORDER) ? 1 : 0;

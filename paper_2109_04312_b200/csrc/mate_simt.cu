@@ -14,8 +14,10 @@
 // thread forms 4 x 4 scores, the 16 lanes of a half warp share four rows from the scores to the results, so only the loads
 // of a tile need the group to meet.  The first matrix of the next tile travels to registers under the second half of this
 // one, the second under the first half.  A warp leaves out the columns that none of its eight rows counts.
-// Bound by latency (16 warps per SM at the registers this takes): with 8 x 512 tokens issue slots are 49 % busy, the
-// multiply-add units 26 %, shared memory 32 %; two global loads and three hand-overs per tile are what a warp waits for.
+// With 8 x 512 tokens (16 warps per SM at the registers this takes) the data pipe that serves shared memory is 66 % busy in the
+// forward and 71 % in the backward, issue slots 59 and 56 %, the multiply-add units 36 %; what a warp waits for is shared
+// memory (1.2 and 1.7 cycles per instruction), its turn (1.2, 0.9) and the group (1.0; two hand-overs per tile in the forward, three
+// in the backward), hardly global memory any more (0.3, 0.7).
 // Two blocks per SM (one with heads of more than 64): three of smaller heads fit, but spill (2 x 512 tokens, heads of 32, 16.2 / 31.9 us
 // with two, 19.8 / 41.4 with three; of 16 12.5 / 24.2, 13.3 / 25.9).
 // 2 x 512 tokens, 12 heads of 64, forward / backward: 24.4 / 53.1 us; with the rows' key ranges in registers

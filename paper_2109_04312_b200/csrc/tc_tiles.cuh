@@ -35,7 +35,7 @@ __device__ __forceinline__ TileInfo row_tile(int q0, int n) {
 // whole groups of 16 rows, so a tile that ends inside a group is gathered: behind its last row the box holds
 // padding or another example's tokens, whose values must not take part (the weight 0 of a masked column does not
 // undo a NaN or an Inf), while a gather repeats a row of the tile.  Against bulk copies of every such tile, forward
-// and backward: 8 x 512 tokens 47.8 -> 48.3 us, 4 x 2048 104.4 -> 103.8, 1 x 8192 177.3 -> 177.9.
+// and backward, with earlier kernels: 8 x 512 tokens 47.8 -> 48.3 us, 4 x 2048 104.4 -> 103.8, 1 x 8192 177.3 -> 177.9.
 __device__ __forceinline__ bool bulk_tile(const TileInfo &t, int ident) {
     return (t.w & 15) == 0 && t.contiguous() && t.first() + kTile <= ident;
 }

@@ -111,7 +111,6 @@ static_assert(8 * kNumBars + 8 <= 512, "the barriers and two words behind them")
 constexpr int kSchedReaders = kComputeWarps + kMmaWarps + kStoreWarps + kLoadWarps;
 // tensor memory columns
 constexpr uint32_t kTmS = 0, kTmT = 128, kTmA1 = 256, kTmA2 = 320, kTmAcc1 = 384, kTmAcc2 = 448;
-constexpr uint32_t kWaitLimit = 4096;  // tries (about 5 us each) before a wait gives up
 
 // kMany: the three passes of a row-or-column plan.  (An instance of its own: the look-ups by pass cost the others up to 1 %,
 // 4 x 2048 tokens 94.4 -> 95.3 us forward and backward.)

@@ -88,7 +88,6 @@ static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kTmemO = 256;
 constexpr uint32_t kTmemP = 384;
-constexpr uint32_t kWaitLimit = 4096;        // tries (about 5 us each) before a wait gives up
 constexpr float kRescale = 8.f;                              // exact units: log2 units before the base moves
 constexpr float kSumMin = 0x1p-100f, kSumMax = 0x1p60f;      // row sums outside: the unit is done once more, exactly
 

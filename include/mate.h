@@ -213,7 +213,7 @@ int mate_attn_workspace_bytes(const mate_plan_t *plan, int d, int dtype, unsigne
  *   workspace device scratch of at least fwd_bytes (may be null when that is 0), 256-byte aligned;
  *             contents are undefined afterwards; concurrent calls need separate workspaces AND
  *             separate plans (see mate_plan)
- *   scale     any finite value.  The tensor-core kernels need scale > 0; with MATE_IMPL_AUTO other
+ *   scale     any finite value.  The tensor-core forward needs scale > 0; with MATE_IMPL_AUTO other
  *             values run on the SIMT kernels, with MATE_IMPL_TCGEN05 they give MATE_ERR_UNSUPPORTED
  * d must be a multiple of 8 and at most 128.  Asynchronous on `stream`. */
 int mate_attn_fwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, int d,

@@ -24,8 +24,13 @@
 //               tile whose rows lie in place in the tensors by one bulk tensor copy per matrix, into 128-byte swizzled shared
 //               memory (row operands double buffered, column tiles in a ring of 4).  Either kind completes on the
 //               tile's barrier by itself, so no warp waits for its copies in order to signal them.
+// On the key side -LSE and D belong to the columns.  Read from shared memory by every arithmetic thread (32 loads of 16 bytes per
+// tile) they cost 340 clk of the shared-memory pipe, and the registers they went through spilled.  They come in with the MMAs
+// instead: S and dP get one more K step, ones x (-LSE / scale) and ones x (-D), each number as the sum of three bf16, which is
+// exact.  Errors against 64 bits (2-norm, 1 x 2048 to 1 x 8192 tokens, scores up to 30 times as large) are those of the loads to
+// three digits: dK 2.364e-3 and 2.364e-3, dV 2.328e-3 and 2.328e-3 on 2 x 512 tokens.
 // What bounds it.  The exponentials take 1024 clk per 128 x 128 tile and side (16 per clock and SM); what is left is the
-// chain S complete -> registers -> arithmetic -> operands -> next S, about 2050 clk per tile when all pairs count, and on
+// chain S complete -> registers -> arithmetic -> operands -> next S, about 1600 clk per tile when all pairs count, and on
 // tables the loads and the cost per item.  Hence:
 //   - A tile that counts in full is taken into registers whole (64 columns of S and of dP per thread), which frees S
 //     and dP for the next tile's MMAs before the arithmetic begins; the operand columns are waited for behind the
@@ -41,10 +46,13 @@
 //   - The tensor maps are fetched ahead of the first copy (4 x 2048 tokens, forward and backward, 99.4 us without, 98.0 with).
 // Forward and backward back to back, 8 x 512 tokens / 4 x 2048 / 1 x 8192 / 2 x 4096: one warp for all MMAs and the epilogue in the
 // arithmetic warps 47.7 / 101.8 / 176.0 / 172.9 us; with store warps and two MMA warps, gathers by tensor copies 46.4 / 98.1 /
-// 165.6 / 162.7 (backward alone 23.0 / 59.6 / 107.7 / 102.1); this form 41.1 / 86.9 / 160.1 / 155.6 (22.3 / 57.8 / 104.2 / 100.0).
+// 165.6 / 162.7 (backward alone 23.0 / 59.6 / 107.7 / 102.1); by 16-byte copies 41.1 / 86.9 / 160.1 / 155.6 (22.1 / 57.8 / 104.3 / 99.9);
+// waits without a hint 21.4 / 56.3 / 101.2 / 97.2 alone; this form, with the row dots in one wave, 21.4 / 54.6 / 98.0 / 96.6.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "load_ring.h"
@@ -74,19 +82,21 @@ constexpr int kLoadWarp0 = kPadWarp0 + kPadWarps;
 constexpr int kLoadWarps = 4;
 static_assert(kTile == 32 * kLoadWarps, "a row of a tile per loader thread");
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
-// registers per thread after the roles have split: 256 x 168 + 128 x 48 + 128 x 40 + 128 x 56 = 61,440 = the 640 x 96 the
+// registers per thread after the roles have split: 256 x 160 + 128 x 56 + 128 x 40 + 128 x 64 = 61,440 = the 640 x 96 the
 // CTA is launched with
-constexpr int kRegsCompute = 168, kRegsStore = 48, kRegsMma = 40, kRegsLoad = 56;
+constexpr int kRegsCompute = 160, kRegsStore = 56, kRegsMma = 40, kRegsLoad = 64;
 constexpr int kStages = 4;  // ring of column tiles
 using RowRing = LoadRing<2>;
 using ColRing = LoadRing<kStages>;
 constexpr int kSchedDepth = 4;
 constexpr uint32_t kOffR = 0;                                    // [2 buffers] x (Ra: Q or K, Rb: dO or V), 16 KB each
 constexpr uint32_t kOffC = 4 * kTileBytes;                       // [kStages] x (Ca 16 KB, Cb 16 KB)
-constexpr uint32_t kOffVec = kOffC + kStages * 2 * kTileBytes;   // [kStages] x 128 x (-LSE log2 e), 128 x D
-constexpr uint32_t kOffMeta = kOffVec + kStages * 1024;          // [2 buffers] x (perm, seg_lo, seg_hi, -LSE log2 e, D) of 128 rows
-constexpr uint32_t kOffStage = kOffMeta + 2 * 5 * kTile * 4;     // [store warps] x 32 rows x 128 bytes
-constexpr uint32_t kOffItem = kOffStage + kStoreWarps * 4096;    // [kSchedDepth] unit records
+constexpr uint32_t kOffExt = kOffC + kStages * 2 * kTileBytes;   // [kStages] x 128 rows x 16 bytes of -LSE / scale, then of -D (key side)
+constexpr uint32_t kOffOnes = kOffExt + kStages * 4096;          // 128 rows x (1, 1, 1, 0, 0, 0, 0, 0)
+constexpr uint32_t kOffZero = kOffOnes + 2048;                   // 128 rows x 16 bytes of zeros
+constexpr uint32_t kOffMeta = kOffZero + 2048;                   // [2 buffers] x (perm, seg_lo, seg_hi, -LSE log2 e, D) of 128 rows
+constexpr uint32_t kOffStage = kOffMeta + 2 * 5 * kTile * 4;     // [store warps] x 32 rows x 64 bytes
+constexpr uint32_t kOffItem = kOffStage + kStoreWarps * 2048;    // [kSchedDepth] unit records
 constexpr uint32_t kOffBar = kOffItem + kSchedDepth * sizeof(FwdUnit);
 constexpr uint32_t kSmemBytes = kOffBar + 512 + 1024;            // + slack for the 1024-byte alignment
 static_assert(kSmemBytes <= 232448, "shared memory per CTA");
@@ -122,6 +132,7 @@ struct Params {
     int bulk;                         // 0: there are none, every tile is gathered row by row
     const __nv_bfloat16 *Q, *K, *V, *dO;
     const float *nlse, *D;  // per row, original order: -LSE log2 e, D
+    const uint4 *ext;       // per row: -LSE / scale and -D, each as the sum of three bf16 (and five zeros)
     __nv_bfloat16 *dQ[kO], *dK[kO], *dV[kO];
     ViewPlan view[kV];
     const FwdUnit *units;  // one half each; item = 2 unit + (0 key side, 1 query side)
@@ -134,21 +145,35 @@ struct Params {
     int32_t *counter;      // next work item (zeroed before the launch)
 };
 
-// D_k = sum_e dO_ke O_ke and -LSE_k log2 e per row (original order), d = 64: eight threads per row, 16 bytes
-// of each tensor per thread, two rows per thread in flight.  HBM-bound.  The first block also clears the
+// A number as the sum of three bf16, exactly (24 bits of mantissa, 8 each): the first three of eight in a row of 16 bytes.
+__device__ __forceinline__ uint4 split_bf16(float x) {
+    const uint32_t h = __float_as_uint(x) & 0xffff0000u;
+    float left = x - __uint_as_float(h);
+    if (!(fabsf(x) <= 3.4028235e38f)) left = 0.f;  // inf and NaN as they are
+    const uint32_t m = __float_as_uint(left) & 0xffff0000u;
+    const uint32_t l = __float_as_uint(left - __uint_as_float(m));
+    return make_uint4(h >> 16 | m, l >> 16, 0u, 0u);
+}
+// D_k = sum_e dO_ke O_ke and -LSE_k log2 e per row (original order), and what the MMAs of the key side add to their
+// accumulators (ext), d = 64: eight threads per row, 16 bytes
+// of each tensor and row per thread, all rows of a thread in flight.  HBM- or L2-bound, and in front of every backward: blocks
+// of a second wave, and a row's LSE fetched behind its sum, cost 1.0 to 1.3 us at 4 x 2048 to 1 x 8192 tokens (55.9 -> 54.7 and
+// 99.3 -> 98.0 us with four rows per thread instead of two), four rows where two fit 0.6 us at 8 x 512.  The first block also clears the
 // work-item counter of the kernel that follows (and the rest of its 256 bytes).
-constexpr int kRowdotRows = 64;  // per block
+// kRows: rows of a group of eight threads, 32 groups to a block.
+template <int kRows>
 __global__ void __launch_bounds__(256) rowdot_kernel(const __nv_bfloat16 *__restrict__ dO, const __nv_bfloat16 *__restrict__ O,
                                                      const float *__restrict__ LSE, float *__restrict__ D,
-                                                     float *__restrict__ nlse, size_t rows, int32_t *counter) {
+                                                     float *__restrict__ nlse, uint4 *__restrict__ ext, float scale,
+                                                     size_t rows, int32_t *counter) {
     launch_dependents();
     wait_prior_grid();
     if (blockIdx.x == 0 && threadIdx.x < 64) counter[threadIdx.x] = 0;
     const int part = threadIdx.x & 7;
-    const size_t r0 = (size_t)blockIdx.x * kRowdotRows + (threadIdx.x >> 3);
-    uint4 a[2], b[2];
+    const size_t r0 = (size_t)blockIdx.x * (32 * kRows) + (threadIdx.x >> 3), own = r0 + 32 * part;  // own: the row this thread finishes
+    uint4 a[kRows], b[kRows];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < kRows; ++q) {
         const size_t r = r0 + 32 * q;
         a[q] = b[q] = make_uint4(0, 0, 0, 0);
         if (r < rows) {
@@ -156,9 +181,11 @@ __global__ void __launch_bounds__(256) rowdot_kernel(const __nv_bfloat16 *__rest
             b[q] = __ldg(reinterpret_cast<const uint4 *>(O + r * 64) + part);
         }
     }
+    const bool finish = part < kRows && own < rows;
+    const float lse = finish ? __ldg(LSE + own) : 0.f;
+    float dot = 0.f;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const size_t r = r0 + 32 * q;
+    for (int q = 0; q < kRows; ++q) {
         const uint32_t aw[4] = {a[q].x, a[q].y, a[q].z, a[q].w}, bw[4] = {b[q].x, b[q].y, b[q].z, b[q].w};
         float acc = 0.f;
 #pragma unroll
@@ -170,44 +197,36 @@ __global__ void __launch_bounds__(256) rowdot_kernel(const __nv_bfloat16 *__rest
         }
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (part == 0 && r < rows) {
-            D[r] = acc;
-            nlse[r] = LSE[r] * -1.4426950408889634f;
-        }
+        if (part == q) dot = acc;
+    }
+    if (finish) {
+        D[own] = dot;
+        nlse[own] = lse * -1.4426950408889634f;
+        // (a row without keys counts nowhere: nothing that is not a number may come from it)
+        ext[2 * own] = split_bf16(lse == -INFINITY ? 0.f : -lse / scale);
+        ext[2 * own + 1] = split_bf16(-dot);
     }
 }
 
 // P and dS of 32 columns, as bf16 pairs (even column in the low half): p = exp2(s * scale2 + nlse), dS = p (dP - D).
-// kKeySide: nlse and D are per column (in shared memory at vec and 512 bytes behind), otherwise per row.  Columns whose bit of
+// Query side: nlse and D are the row's.  Key side: the accumulators hold s - LSE / scale and dP - D already.  Columns whose bit of
 // `on` is clear do not count (kMask).  Two columns per instruction except for the exponential.
 template <bool kKeySide, bool kMask>
 __device__ __forceinline__ void math32(const uint32_t (&sv)[32], const uint32_t (&tv)[32], uint64_t scale2, uint64_t row_nlse2,
-                                       uint64_t row_D2, uint32_t vec, uint32_t on,
-                                       uint32_t (&pk_p)[16], uint32_t (&pk_ds)[16]) {
+                                       uint64_t row_D2, uint32_t on, uint32_t (&pk_p)[16], uint32_t (&pk_ds)[16]) {
 #pragma unroll
-    for (int e = 0; e < 32; e += 4) {
-        uint64_t nl[2] = {row_nlse2, row_nlse2}, Dv[2] = {row_D2, row_D2};
-        if (kKeySide) {
-            const float4 a = ld_shared_f4(vec + 4 * e), d4 = ld_shared_f4(vec + 512 + 4 * e);
-            nl[0] = pack_f32x2(a.x, a.y);
-            nl[1] = pack_f32x2(a.z, a.w);
-            Dv[0] = pack_f32x2(d4.x, d4.y);
-            Dv[1] = pack_f32x2(d4.z, d4.w);
+    for (int k = 0; k < 32; k += 2) {
+        const uint64_t s = pack_f32x2(sv[k], sv[k + 1]), t = pack_f32x2(tv[k], tv[k + 1]);
+        float x0, x1, d0, d1;
+        unpack_f32x2(kKeySide ? mul_f32x2(s, scale2) : fma_f32x2(s, scale2, row_nlse2), x0, x1);
+        float p0 = ex2(x0), p1 = ex2(x1);
+        if (kMask) {
+            if (!(on & (1u << k))) p0 = 0.f;
+            if (!(on & (2u << k))) p1 = 0.f;
         }
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int k = e + 2 * q;
-            float x0, x1, d0, d1;
-            unpack_f32x2(fma_f32x2(pack_f32x2(sv[k], sv[k + 1]), scale2, nl[q]), x0, x1);
-            float p0 = ex2(x0), p1 = ex2(x1);
-            if (kMask) {
-                if (!(on & (1u << k))) p0 = 0.f;
-                if (!(on & (2u << k))) p1 = 0.f;
-            }
-            unpack_f32x2(mul_f32x2(pack_f32x2(p0, p1), sub_f32x2(pack_f32x2(tv[k], tv[k + 1]), Dv[q])), d0, d1);
-            if (kKeySide) pk_p[k >> 1] = cvt_bf16x2(p0, p1);
-            pk_ds[k >> 1] = cvt_bf16x2(d0, d1);
-        }
+        unpack_f32x2(mul_f32x2(pack_f32x2(p0, p1), kKeySide ? t : sub_f32x2(t, row_D2)), d0, d1);
+        if (kKeySide) pk_p[k >> 1] = cvt_bf16x2(p0, p1);
+        pk_ds[k >> 1] = cvt_bf16x2(d0, d1);
     }
 }
 // Tiles of an item: nA of range A, then those of range B (all of them kTile columns wide but for the last of either).
@@ -293,6 +312,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         *s_abort = 0;
         fence_mbar_init();
     }
+    if (tid < 256) {  // (1, 1, 1, 0 ..) and zeros: the parts of the additional K step that do not change
+        *reinterpret_cast<uint4 *>(sm + kOffOnes + 16 * tid) = tid < 128 ? make_uint4(0x3f803f80u, 0x3f80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+        fence_proxy_async();
+    }
     if (warp == kMmaWarp) {
         tmem_alloc(smem_u32((const void *)tmem_slot), 512);
         tmem_relinquish();
@@ -364,7 +387,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
 #pragma unroll 1
                 for (int i = 0; i < tiles.n; ++i) {
                     const bool full = t.w == kTile && (t.pre == kTile || (w_lo_max - t.k0 <= t.pre && w_hi_min - t.k0 >= kTile));
-                    const uint32_t vec = base + kOffVec + ColRing::buffer(c_cnt) * 1024;
                     TR_T0(t_ws);
                     if (!(alive = wait(bars + 8 * kBarSFull, c_cnt & 1))) break;
                     tc_fence_after();
@@ -390,13 +412,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                         }
                         release_st();
                         TR_ADD(4, t_cmp);
-                        math32<kKeySide, false>(sv[0], tv[0], scale2, row_nlse2, row_D2, vec + cq * 128, 0u, pk_p, pk_ds);
+                        math32<kKeySide, false>(sv[0], tv[0], scale2, row_nlse2, row_D2, 0u, pk_p, pk_ds);
                         TR_T0(t_wa);
                         gradients_done();  // of the tile before: the operand columns are free
                         TR_ADD(1, t_wa);
                         if (kKeySide) tmem_st16(tm + kTmA1 + cq * 16, pk_p);
                         tmem_st16(tm + (kKeySide ? kTmA2 : kTmA1) + cq * 16, pk_ds);
-                        math32<kKeySide, false>(sv[1], tv[1], scale2, row_nlse2, row_D2, vec + 256 + cq * 128, 0u, pk_p, pk_ds);
+                        math32<kKeySide, false>(sv[1], tv[1], scale2, row_nlse2, row_D2, 0u, pk_p, pk_ds);
                         if (kKeySide) tmem_st16(tm + kTmA1 + cq * 16 + 32, pk_p);
                         tmem_st16(tm + (kKeySide ? kTmA2 : kTmA1) + cq * 16 + 32, pk_ds);
                     } else {
@@ -422,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                                     release_st();
                                     held = false;
                                 }
-                                math32<kKeySide, true>(sv, tv, scale2, row_nlse2, row_D2, vec + 4 * cb,
+                                math32<kKeySide, true>(sv, tv, scale2, row_nlse2, row_D2,
                                                        bits_below(t.pre - cb) | (bits_below(r_hi - cb) & ~bits_below(r_lo - cb)), pk_p, pk_ds);
                             }
                             if (!a_free) gradients_done();
@@ -462,7 +484,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         const int q4 = warp - kStoreWarp0;  // rows 32 q4 .. of the tile = lanes of tensor memory this warp can read
         static_assert(kStoreWarp0 % 4 == 0, "warp w reads the lanes 32 (w % 4) ..");
         const uint32_t acc = tmem + ((uint32_t)(q4 * 32) << 16) + kTmAcc1;
-        uint8_t *stage = sm + kOffStage + q4 * 4096;
+        uint8_t *stage = sm + kOffStage + q4 * 2048;
         uint32_t units = 0;
         wait_prior_grid();
 #pragma unroll 1
@@ -485,42 +507,40 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                 if (!wait(bars + 8 * kBarItemDone, units++ & 1)) break;
                 tc_fence_after();
             }
-            // key side: dV, dK; query side: dQ.  64 columns at a time through the staging area, so that a store writes
-            // whole rows of 128 bytes.
+            // key side: dV, dK; query side: dQ.  32 columns at a time through the staging area, so that a store writes
+            // 64 consecutive bytes of eight rows.
+            const int n_c = key_side ? 4 : 2;
 #pragma unroll 1
-            for (int c = 0; c < (key_side ? 2 : 1); ++c) {
-                const float mul = key_side && c == 0 ? 1.f : p.scale;
-#pragma unroll 1
-                for (int half = 0; half < 2; ++half) {
-                    uint32_t o[32];
-                    if (any) {
-                        tmem_ld32(acc + c * 64 + half * 32, o);
-                        tc_wait_ld();
-                        reg_fence(o);
-                    } else {  // rows without any pair (possible in the passes of the row-or-column pattern)
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) o[e] = 0u;
-                    }
-                    if (any && half == 1 && c == (key_side ? 1 : 0)) {  // read for the last time
+            for (int c = 0; c < n_c; ++c) {
+                const float mul = key_side && c < 2 ? 1.f : p.scale;
+                uint32_t o[32];
+                if (any) {
+                    tmem_ld32(acc + c * 32, o);
+                    tc_wait_ld();
+                    reg_fence(o);
+                    if (c + 1 == n_c) {  // read for the last time
                         tc_fence_before();
                         if (lane == 0) mbar_arrive(bars + 8 * kBarAccFree);
                     }
+                } else {  // rows without any pair (possible in the passes of the row-or-column pattern)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        uint32_t w4[4];
+                    for (int e = 0; e < 32; ++e) o[e] = 0u;
+                }
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            w4[e] = cvt_bf16x2(__uint_as_float(o[8 * j + 2 * e]) * mul, __uint_as_float(o[8 * j + 2 * e + 1]) * mul);
-                        *reinterpret_cast<uint4 *>(stage + lane * 128 + (((half * 4 + j) ^ (lane & 7)) << 4)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-                    }
+                for (int j = 0; j < 4; ++j) {
+                    uint32_t w4[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        w4[e] = cvt_bf16x2(__uint_as_float(o[8 * j + 2 * e]) * mul, __uint_as_float(o[8 * j + 2 * e + 1]) * mul);
+                    *reinterpret_cast<uint4 *>(stage + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
                 }
                 __syncwarp();
-                __nv_bfloat16 *out = (key_side ? (c ? p.dK[pass] : p.dV[pass]) : p.dQ[pass]) + at;
+                __nv_bfloat16 *out = (key_side ? (c < 2 ? p.dV[pass] : p.dK[pass]) : p.dQ[pass]) + at + (c & 1) * 32;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int row = 4 * i + (lane >> 3), j = lane & 7;
+                for (int i = 0; i < 4; ++i) {
+                    const int row = 8 * i + (lane >> 2), j = lane & 3;
                     const int dr = __shfl_sync(0xffffffffu, dst_row, row);
-                    const uint4 x = *reinterpret_cast<const uint4 *>(stage + row * 128 + ((j ^ (row & 7)) << 4));
+                    const uint4 x = *reinterpret_cast<const uint4 *>(stage + row * 64 + ((j ^ ((row >> 1) & 3)) << 4));
                     if (dr >= 0) *reinterpret_cast<uint4 *>(out + (size_t)dr * 64 + j * 8) = x;
                 }
                 __syncwarp();
@@ -564,12 +584,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                     if (!(alive = wait_u(bars + 8 * (kBarRFull + rb), RowRing::full_parity(n)))) break;
                     fence_proxy_async();
                     const uint32_t ra = smem_desc_lo(base + kOffR) + rb * ((2 * kTileBytes) >> 4), rbb = ra + (kTileBytes >> 4);
+                    const uint32_t ones = smem_desc_lo_rows16(base + kOffOnes, base + kOffZero);
 #pragma unroll 1
                     for (int i = 0; i < n_tiles; ++i, ++c_cnt) {
                         const uint32_t st = ColRing::buffer(c_cnt);
                         const uint32_t idesc = idesc_bf16(128, 0, 0, 0) | (uint32_t)steps(i) << 18;  // N = 16 columns per step
                         const uint32_t ca = smem_desc_lo(base + kOffC) + st * ((2 * kTileBytes) >> 4), cb = ca + (kTileBytes >> 4);
-                        const uint32_t tS = tmem + kTmS, tT = tmem + kTmT;
+                        const uint32_t tS = tmem + kTmS, tT = tmem + kTmT, ext = base + kOffExt + st * 4096;
                         if (!(alive = wait_u(bars + 8 * (kBarCFull + st), ColRing::full_parity(c_cnt)))) break;  // the tile has landed
                         fence_proxy_async();  // the copies of 16 bytes come through the generic proxy
                         // the tile before sits in registers (parity 1 of a barrier without a phase behind it: at once)
@@ -584,6 +605,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                             mma_ss_lean<1>(tT, rbb + 2, cb + 2, idesc);
                             mma_ss_lean<1>(tT, rbb + 4, cb + 4, idesc);
                             mma_ss_lean<1>(tT, rbb + 6, cb + 6, idesc);
+                            if (key_side) {  // - LSE / scale and - D of the columns: ones x (three bf16 per column)
+                                mma_ss_rows16(tS, ones, smem_desc_lo_rows16(ext, base + kOffZero), idesc);
+                                mma_ss_rows16(tT, ones, smem_desc_lo_rows16(ext + 2048, base + kOffZero), idesc);
+                            }
                             mma_commit(bars + 8 * kBarSFull);
                         }
                         __syncwarp();
@@ -713,9 +738,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                         }
                     }
                 } else if (key_side) {  // column data
-                    const uint32_t vec = base + kOffVec + st * 1024 + rr * 4;
-                    cp_async4(vec, p.nlse + now);
-                    cp_async4(vec + 512, p.D + now);
+                    const uint32_t ext = base + kOffExt + st * 4096 + rr * 16;
+                    cp_async16(ext, p.ext + 2 * (size_t)now);
+                    cp_async16(ext + 2048, p.ext + 2 * (size_t)now + 1);
                 }
                 const uint32_t dst = base + (i < 0 ? kOffR + rb * 2 * kTileBytes : kOffC + st * 2 * kTileBytes);
                 const bool kv = (i < 0) == key_side;  // K and V, or Q and dO
@@ -767,10 +792,12 @@ inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 }  // namespace
 
-// workspace: [256 B counters][D: B*H*N floats][-LSE log2 e: as many]
+// workspace: [256 B counters][D: B*H*N floats][-LSE log2 e: as many][the key side's column data: 32 B per row]
 size_t tc_bwd_workspace(const mate_plan_t *plan) {
-    return 256 + 2 * align256((size_t)plan->B * plan->H * plan->N * sizeof(float));
+    const size_t rows = (size_t)plan->B * plan->H * plan->N;
+    return 256 + 2 * align256(rows * sizeof(float)) + rows * 32;
 }
+bool tc_bwd_scale(float scale) { return fabsf(scale) >= 0x1p-100f && fabsf(scale) <= 0x1p100f; }
 
 namespace {
 template <bool kMany>
@@ -783,7 +810,9 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     const size_t rows = plan->n_rows();
     uint8_t *ws = (uint8_t *)workspace;
     float *D = (float *)(ws + 256);
-    float *nlse = D + align256((size_t)plan->B * plan->H * plan->N * sizeof(float)) / sizeof(float);
+    const size_t row_floats = align256((size_t)plan->B * plan->H * plan->N * sizeof(float)) / sizeof(float);
+    float *nlse = D + row_floats;
+    uint4 *ext = (uint4 *)(nlse + row_floats);
     Params<kMany> p;
     p.bulk = rows < (size_t(1) << 31) && make_row_map(&p.tmQ, Q, rows) && make_row_map(&p.tmK, K, rows) &&
              make_row_map(&p.tmV, V, rows) && make_row_map(&p.tmdO, dO, rows);
@@ -793,6 +822,7 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.dO = (const __nv_bfloat16 *)dO;
     p.nlse = nlse;
     p.D = D;
+    p.ext = ext;
     for (int i = 0; i < p.kO; ++i) {
         p.dQ[i] = (__nv_bfloat16 *)dQ[i];
         p.dK[i] = (__nv_bfloat16 *)dK[i];
@@ -811,8 +841,15 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     p.status = plan->status_dev;
     p.counter = (int32_t *)ws;
 
-    if (launch_after(rowdot_kernel, dim3((unsigned)((rows + kRowdotRows - 1) / kRowdotRows)), 256, 0, stream, (const __nv_bfloat16 *)dO,
-                                  (const __nv_bfloat16 *)O, LSE, D, nlse, rows, (int32_t *)ws) != cudaSuccess)
+    const auto rowdot = [&](auto n) {
+        constexpr int kRows = decltype(n)::value;
+        return launch_after(rowdot_kernel<kRows>, dim3((unsigned)((rows + 32 * kRows - 1) / (32 * kRows))), 256, 0, stream, (const __nv_bfloat16 *)dO,
+                            (const __nv_bfloat16 *)O, LSE, D, nlse, ext, scale, rows, (int32_t *)ws);
+    };
+    // As few rows per thread as bring all blocks onto the GPU at once (six to an SM).
+    const size_t at_once = (size_t)std::max(plan->n_ctas, 1) * 6 * 32;
+    if ((rows <= at_once ? rowdot(std::integral_constant<int, 1>{}) : rows <= 2 * at_once ? rowdot(std::integral_constant<int, 2>{})
+                                                                                          : rowdot(std::integral_constant<int, 4>{})) != cudaSuccess)
         return MATE_ERR_CUDA;
     return launch_after(tc_bwd_kernel<kMany>, dim3((unsigned)plan->bwd_grid), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }

@@ -148,6 +148,23 @@ __device__ __forceinline__ void mma_ss_lean(uint32_t d_tmem, uint32_t a_lo, uint
         : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "n"(kAcc), "n"(kDescHiSw128)
         : "memory");
 }
+// The same with both operands one K step of rows of 16 bytes and no swizzle: eight rows make a block of 128 bytes, the blocks
+// follow one another, and the second half of the step (bytes 16 to 31 of a row) lies `leading byte offset` behind.
+constexpr uint32_t kDescHiRows16 = (128u >> 4) | (1u << 14);
+__device__ __forceinline__ uint32_t smem_desc_lo_rows16(uint32_t saddr, uint32_t second_half) {
+    return ((saddr & 0x3FFFFu) >> 4) | ((second_half - saddr) >> 4) << 16;
+}
+__device__ __forceinline__ void mma_ss_rows16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {  // D += A B
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, 1, 0;\n\t"
+        "mov.b64 da, {%1, %4};\n\t"
+        "mov.b64 db, {%2, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}"
+        :
+        : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "n"(kDescHiRows16)
+        : "memory");
+}
 template <int kAcc>
 __device__ __forceinline__ void mma_ts_lean(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc) {
     asm volatile(

@@ -67,6 +67,29 @@ def test_tensor_core_units_that_are_cut_and_a_busy_grid():
     _check(rows, cols, 70, [0, 1] * 26, 64, "bf16", 9)
 
 
+@pytest.mark.parametrize("H", [768, 769, 1536, 1537])  # x 37 positions: around one and two rows per thread on 148 SMs
+def test_row_dots_of_every_size(H):
+    rows, cols = _structure(5, 31, 4, 3, 11)
+    _check(rows, cols, 5, [0, 1, 0] * (H // 3) + [1] * (H % 3), 64, "bf16", 12, 1)
+
+
+@pytest.mark.parametrize("scale", [0.0, -0.125, 2.0 ** -101, 2.0 ** -99, 1.5])  # the backward divides by some of them
+def test_backward_takes_every_scale(scale):
+    import paper_2109_04312_b200 as m
+    rows, cols = _structure(20, 300, 30, 4, 13)
+    hv, rng = np.array([0, 1], np.uint8), np.random.default_rng(14)
+    vals = {n: tables.round_to_bf16((rng.standard_normal((1, 2, 320, 64)) * 0.5).astype(np.float32)) for n in ("Q", "K", "V", "dO")}
+    plan = m.mate_plan(torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda(), 20, hv)
+    Q, K, V, dO = (hp.to_dev(vals[n], "bf16") for n in ("Q", "K", "V", "dO"))
+    O, LSE = m.mate_attn_fwd(plan, Q, K, V, scale)
+    grads = m.mate_attn_bwd(plan, Q, K, V, O, LSE, dO, scale)
+    plan.status()
+    want = oracle.bwd(vals["Q"], vals["K"], vals["V"], vals["dO"], rows, cols, 20, hv, scale)
+    atol, rtol = hp.tol("bf16")
+    for name, g, o in zip(("dQ", "dK", "dV"), grads, want):
+        hp.assert_close(hp.to_np(g), o, atol, rtol, name)
+
+
 def _poisoned(t, where):
     """A copy of t whose rows `where` (a mask over its rows) hold NaN, Inf and -Inf in turn."""
     x = t.clone().view(-1, t.shape[-1])

@@ -442,6 +442,10 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
     __shared__ int s_col[2][kCols], s_own[kRows];  // original rows of each group's tile, of the block
     __shared__ float s_row[2][kRows];                          // LSE, D of the block's rows (query side)
     constexpr int kR = kRows * (DP + 4), kC = kCols * (DP + 4), kPart = 2 * kC + kRows * kPStride + 2 * kCols;
+    // P waits in shared memory for dP where it would not fit into the registers: with heads of 64, 24 to 44 of which were spilled, 2 x
+    // 512 / 8 x 512 tokens 52.5 / 195 us with P in registers, 50.0 / 187 with it in shared memory; heads of 16, 32 and 128, which do
+    // not spill, 22.4, 30.6 and 90.6 us and 23.5, 31.3 and 91.2.
+    constexpr bool kPShared = DP == 64;
     const int grp = threadIdx.x / kGroup, tid = threadIdx.x % kGroup;
     float *sRa = smem, *sRb = sRa + kR, *part = sRb + kR, *sCa = part + grp * kPart, *sCb = sCa + kC, *sX = sCb + kC,
           *sVec = sX + kRows * kPStride;
@@ -507,25 +511,66 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
             if (tid < kCols) next_at = r.orig(c0 + min(tid, w - 1));
         }
         group_sync();
-        float s[kMine][4], dp[kMine][4];
-        if (k1 > k0) scores<DP>(s, sRa, sCa, row0, tx, k0, k1);
-        next.store(sCb);
-        if (tid < kCols) at[tid] = next_at;
-        group_sync();
-        if (k1 > k0) {
-            scores<DP>(dp, sRb, sCb, row0, tx, k0, k1);
+        float s[kMine][4];
+        if constexpr (kPShared) {
+            if (k1 > k0) {
+                scores<DP>(s, sRa, sCa, row0, tx, k0, k1);
 #pragma unroll
-            for (int j = 0; j < kMine; ++j) {
-                int lo, hi;
-                r.row_span(i, t_c0, t_w, row0 + j, lo, hi);
+                for (int j = 0; j < kMine; ++j) {
+                    int lo, hi;
+                    r.row_span(i, t_c0, t_w, row0 + j, lo, hi);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int col = tx + 16 * q;
-                    const float lse = key_side ? sVec[col] : s_row[0][row0 + j], D = key_side ? sVec[kCols + col] : s_row[1][row0 + j];
-                    const bool on = col >= lo && col < hi;
-                    const float p = on ? expf(c.scale * s[j][q] - lse) : 0.f;
-                    s[j][q] = p;
-                    sX[(row0 + j) * kPStride + col] = on ? p * (dp[j][q] - D) : 0.f;
+                    for (int q = 0; q < 4; ++q) {
+                        const int col = tx + 16 * q;
+                        const float lse = key_side ? sVec[col] : s_row[0][row0 + j];
+                        sX[(row0 + j) * kPStride + col] = col >= lo && col < hi ? expf(c.scale * s[j][q] - lse) : 0.f;
+                    }
+                }
+            }
+            next.store(sCb);
+            if (tid < kCols) at[tid] = next_at;
+            group_sync();
+            if (k1 > k0) {
+                if (key_side) {
+                    __syncwarp();
+                    accumulate<DP>(acc1, sX, sCb, row0, tx, k0, k1);
+                }
+                scores<DP>(s, sRb, sCb, row0, tx, k0, k1);
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < kMine; ++j) {
+                    int lo, hi;
+                    r.row_span(i, t_c0, t_w, row0 + j, lo, hi);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int col = tx + 16 * q;
+                        const float D = key_side ? sVec[kCols + col] : s_row[1][row0 + j];
+                        float &x = sX[(row0 + j) * kPStride + col];
+                        x = col >= lo && col < hi ? x * (s[j][q] - D) : 0.f;
+                    }
+                }
+            }
+        } else {
+            float dp[kMine][4];
+            if (k1 > k0) scores<DP>(s, sRa, sCa, row0, tx, k0, k1);
+            next.store(sCb);
+            if (tid < kCols) at[tid] = next_at;
+            group_sync();
+            if (k1 > k0) {
+                scores<DP>(dp, sRb, sCb, row0, tx, k0, k1);
+#pragma unroll
+                for (int j = 0; j < kMine; ++j) {
+                    int lo, hi;
+                    r.row_span(i, t_c0, t_w, row0 + j, lo, hi);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int col = tx + 16 * q;
+                        const float lse = key_side ? sVec[col] : s_row[0][row0 + j], D = key_side ? sVec[kCols + col] : s_row[1][row0 + j];
+                        const bool on = col >= lo && col < hi;
+                        const float p = on ? expf(c.scale * s[j][q] - lse) : 0.f;
+                        s[j][q] = p;
+                        sX[(row0 + j) * kPStride + col] = on ? p * (dp[j][q] - D) : 0.f;
+                    }
                 }
             }
         }
@@ -534,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
         __syncwarp();
         accumulate<DP>(acc0, sX, sCa, row0, tx, k0, k1);
         __syncwarp();
-        if (key_side) {
+        if (!kPShared && key_side) {
 #pragma unroll
             for (int q = 0; q < 4; ++q)
 #pragma unroll

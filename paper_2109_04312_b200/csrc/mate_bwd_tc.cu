@@ -202,8 +202,9 @@ __global__ void __launch_bounds__(256) rowdot_kernel(const __nv_bfloat16 *__rest
     if (finish) {
         D[own] = dot;
         nlse[own] = lse * -1.4426950408889634f;
-        // (a row without keys counts nowhere: nothing that is not a number may come from it)
-        ext[2 * own] = split_bf16(lse == -INFINITY ? 0.f : -lse / scale);
+        // (LSE = -inf: a padding row, which is no column of any tile, or a query all of whose scores are -inf, whose weights are not
+        // numbers: -inf + inf)
+        ext[2 * own] = split_bf16(-lse / scale);
         ext[2 * own + 1] = split_bf16(-dot);
     }
 }

@@ -90,6 +90,38 @@ def test_backward_takes_every_scale(scale):
         hp.assert_close(hp.to_np(g), o, atol, rtol, name)
 
 
+@pytest.mark.parametrize("at", [[130], [5, 130]])  # a row of the table; one of the prefix too, which every other row meets
+@pytest.mark.parametrize("kind", ["exact", "sat"])
+def test_a_query_without_a_finite_score(kind, at):
+    # All scores of some valid queries are -inf (products of -2^200), so their LSE is -inf as well: their weights are not numbers
+    # on either side of the backward, whichever kernels run.  A row that is padding has that LSE too, and reaches nothing.
+    import paper_2109_04312_b200 as m
+    rows, cols = (np.concatenate([x, np.full((1, 40), -1, np.int32)], 1) for x in _structure(20, 300, 30, 4, 13))
+    r, c = torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda()
+    plan = m.mate_plan_sat(r, c, 20, 2) if kind == "sat" else m.mate_plan(r, c, 20, [0, 1])
+    gen = torch.Generator(device="cuda").manual_seed(15)
+    Q, K, V, dO = ((torch.randn(1, 2, 360, 64, device="cuda", generator=gen) * 0.5).bfloat16() for _ in range(4))
+    Q[..., 0], K[..., 0] = 0.0, -2.0 ** 100
+    Q[:, :, at, 0] = 2.0 ** 100
+    mask = {}
+    for impl in (m.IMPL_TCGEN05, m.IMPL_SIMT):
+        O, LSE = m.mate_attn_fwd(plan, Q, K, V, None, impl)
+        assert torch.equal(torch.isneginf(LSE[0, 0]).nonzero().flatten().cpu(), torch.tensor(at + list(range(320, 360))))
+        mask[impl] = [torch.isnan(x) for x in m.mate_attn_bwd(plan, Q, K, V, O, LSE, dO, None, impl)]
+    plan.status()
+    ids = [rows[0, :320], cols[0, :320]]
+    for name, tc, simt in zip(("dQ", "dK", "dV"), mask[m.IMPL_TCGEN05], mask[m.IMPL_SIMT]):
+        assert torch.equal(tc, simt), name
+        for h in range(2):
+            met = np.zeros(360, bool)
+            for k in at:
+                same = (ids[0] == ids[0][k]) | (ids[1] == ids[1][k]) if kind == "sat" else ids[h] == ids[h][k]
+                met[:320] |= same | (np.arange(320) < 20) | (k < 20)
+            if name == "dQ":
+                met = np.isin(np.arange(360), at)
+            assert np.array_equal(tc[0, h].any(-1).cpu().numpy(), met), (name, h)
+
+
 def _poisoned(t, where):
     """A copy of t whose rows `where` (a mask over its rows) hold NaN, Inf and -Inf in turn."""
     x = t.clone().view(-1, t.shape[-1])

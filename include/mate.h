@@ -223,7 +223,7 @@ int mate_attn_fwd(const mate_plan_t *plan, const void *Q, const void *K, const v
 /* Backward of mate_attn_fwd (derived from the Section 3 head formula; the paper states no
  * backward): given O and LSE of the forward call and dO, writes dQ, dK, dV (fully overwritten,
  * no accumulation into previous contents).  Same layouts, types and rules as the forward, except that
- * every finite scale is taken: beyond 2^+-100 in magnitude (0 among them) on the SIMT kernels. */
+ * the tensor-core backward takes every finite scale. */
 int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
                   const void *O, const float *LSE, const void *dO, int d, int dtype, float scale,
                   void *dQ, void *dK, void *dV, void *workspace, size_t workspace_bytes,

@@ -999,7 +999,6 @@ int mate_attn_bwd(const mate_plan_t *plan, const void *Q, const void *K, const v
     const void *ptrs[] = {Q, K, V, O, LSE, dO, dQ, dK, dV};
     for (const void *p : ptrs)
         if (!aligned16(p)) return MATE_ERR_ALIGNMENT;
-    use_tc = use_tc && mate::tc_bwd_scale(scale);
     size_t need = 0;
     mate_attn_workspace_bytes(plan, d, dtype, use_tc ? MATE_IMPL_TCGEN05 : MATE_IMPL_SIMT, nullptr, &need);
     if (!workspace || workspace_bytes < need) return MATE_ERR_WORKSPACE;

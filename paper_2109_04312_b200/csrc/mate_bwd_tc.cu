@@ -26,8 +26,8 @@
 //               tile's barrier by itself, so no warp waits for its copies in order to signal them.
 // On the key side -LSE and D belong to the columns.  Read from shared memory by every arithmetic thread (32 loads of 16 bytes per
 // tile) they cost 340 clk of the shared-memory pipe, and the registers they went through spilled.  They come in with the MMAs
-// instead: S and dP get one more K step, ones x (-LSE / scale) and ones x (-D), each number as the sum of three bf16, which is
-// exact.  Errors against 64 bits (2-norm, 1 x 2048 to 1 x 8192 tokens, scores up to 30 times as large) are those of the loads to
+// instead, wherever the scale can be divided by (divides): S and dP get one more K step, ones x (-LSE / scale) and ones x (-D), each
+// number as the sum of three bf16, which is exact.  Errors against 64 bits (2-norm, 1 x 2048 to 1 x 8192 tokens, scores up to 30 times as large) are those of the loads to
 // three digits: dK 2.364e-3 and 2.364e-3, dV 2.328e-3 and 2.328e-3 on 2 x 512 tokens.
 // What bounds it.  The exponentials take 1024 clk per 128 x 128 tile and side (16 per clock and SM); what is left is the
 // chain S complete -> registers -> arithmetic -> operands -> next S, about 1600 clk per tile when all pairs count, and on
@@ -91,7 +91,8 @@ using ColRing = LoadRing<kStages>;
 constexpr int kSchedDepth = 4;
 constexpr uint32_t kOffR = 0;                                    // [2 buffers] x (Ra: Q or K, Rb: dO or V), 16 KB each
 constexpr uint32_t kOffC = 4 * kTileBytes;                       // [kStages] x (Ca 16 KB, Cb 16 KB)
-constexpr uint32_t kOffExt = kOffC + kStages * 2 * kTileBytes;   // [kStages] x 128 rows x 16 bytes of -LSE / scale, then of -D (key side)
+constexpr uint32_t kOffExt = kOffC + kStages * 2 * kTileBytes;   // [kStages] x 128 rows x 16 bytes of -LSE / scale, then of -D (key side;
+                                                                 // !kByMma: 128 x (-LSE log2 e), 128 x D)
 constexpr uint32_t kOffOnes = kOffExt + kStages * 4096;          // 128 rows x (1, 1, 1, 0, 0, 0, 0, 0)
 constexpr uint32_t kOffZero = kOffOnes + 2048;                   // 128 rows x 16 bytes of zeros
 constexpr uint32_t kOffMeta = kOffZero + 2048;                   // [2 buffers] x (perm, seg_lo, seg_hi, -LSE log2 e, D) of 128 rows
@@ -210,22 +211,30 @@ __global__ void __launch_bounds__(256) rowdot_kernel(const __nv_bfloat16 *__rest
 }
 
 // P and dS of 32 columns, as bf16 pairs (even column in the low half): p = exp2(s * scale2 + nlse), dS = p (dP - D).
-// Query side: nlse and D are the row's.  Key side: the accumulators hold s - LSE / scale and dP - D already.  Columns whose bit of
+// Query side: nlse and D are the row's.  Key side: they are the columns', and the accumulators hold s - LSE / scale and dP - D
+// already (kByMma), or they are in shared memory, at vec and 512 bytes behind.  Columns whose bit of
 // `on` is clear do not count (kMask).  Two columns per instruction except for the exponential.
-template <bool kKeySide, bool kMask>
+template <bool kKeySide, bool kMask, bool kByMma>
 __device__ __forceinline__ void math32(const uint32_t (&sv)[32], const uint32_t (&tv)[32], uint64_t scale2, uint64_t row_nlse2,
-                                       uint64_t row_D2, uint32_t on, uint32_t (&pk_p)[16], uint32_t (&pk_ds)[16]) {
+                                       uint64_t row_D2, uint32_t vec, uint32_t on, uint32_t (&pk_p)[16], uint32_t (&pk_ds)[16]) {
+    uint64_t nlse2[2] = {row_nlse2, row_nlse2}, D2[2] = {row_D2, row_D2};
 #pragma unroll
     for (int k = 0; k < 32; k += 2) {
+        if (kKeySide && !kByMma && k % 4 == 0) {
+            const float4 a = ld_shared_f4(vec + 4 * k), b = ld_shared_f4(vec + 512 + 4 * k);
+            nlse2[0] = pack_f32x2(a.x, a.y), nlse2[1] = pack_f32x2(a.z, a.w);
+            D2[0] = pack_f32x2(b.x, b.y), D2[1] = pack_f32x2(b.z, b.w);
+        }
         const uint64_t s = pack_f32x2(sv[k], sv[k + 1]), t = pack_f32x2(tv[k], tv[k + 1]);
+        const int q = k / 2 % 2;
         float x0, x1, d0, d1;
-        unpack_f32x2(kKeySide ? mul_f32x2(s, scale2) : fma_f32x2(s, scale2, row_nlse2), x0, x1);
+        unpack_f32x2(kKeySide && kByMma ? mul_f32x2(s, scale2) : fma_f32x2(s, scale2, nlse2[q]), x0, x1);
         float p0 = ex2(x0), p1 = ex2(x1);
         if (kMask) {
             if (!(on & (1u << k))) p0 = 0.f;
             if (!(on & (2u << k))) p1 = 0.f;
         }
-        unpack_f32x2(mul_f32x2(pack_f32x2(p0, p1), kKeySide ? t : sub_f32x2(t, row_D2)), d0, d1);
+        unpack_f32x2(mul_f32x2(pack_f32x2(p0, p1), kKeySide && kByMma ? t : sub_f32x2(t, D2[q])), d0, d1);
         if (kKeySide) pk_p[k >> 1] = cvt_bf16x2(p0, p1);
         pk_ds[k >> 1] = cvt_bf16x2(d0, d1);
     }
@@ -255,7 +264,9 @@ struct ItemTiles {
 };
 __device__ __forceinline__ uint32_t bits_below(int n) { return n <= 0 ? 0u : n >= 32 ? 0xffffffffu : (1u << n) - 1u; }
 
-template <bool kMany>
+// kByMma: the key side's column data come in with the MMAs, which takes a scale that can be divided by (divides); otherwise
+// every thread reads them from shared memory.
+template <bool kMany, bool kByMma>
 __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_constant__ Params<kMany> p) {
     launch_dependents();
     extern __shared__ uint8_t smem_raw[];
@@ -388,6 +399,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
 #pragma unroll 1
                 for (int i = 0; i < tiles.n; ++i) {
                     const bool full = t.w == kTile && (t.pre == kTile || (w_lo_max - t.k0 <= t.pre && w_hi_min - t.k0 >= kTile));
+                    const uint32_t vec = base + kOffExt + ColRing::buffer(c_cnt) * 4096;
                     TR_T0(t_ws);
                     if (!(alive = wait(bars + 8 * kBarSFull, c_cnt & 1))) break;
                     tc_fence_after();
@@ -413,13 +425,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                         }
                         release_st();
                         TR_ADD(4, t_cmp);
-                        math32<kKeySide, false>(sv[0], tv[0], scale2, row_nlse2, row_D2, 0u, pk_p, pk_ds);
+                        math32<kKeySide, false, kByMma>(sv[0], tv[0], scale2, row_nlse2, row_D2, vec + cq * 128, 0u, pk_p, pk_ds);
                         TR_T0(t_wa);
                         gradients_done();  // of the tile before: the operand columns are free
                         TR_ADD(1, t_wa);
                         if (kKeySide) tmem_st16(tm + kTmA1 + cq * 16, pk_p);
                         tmem_st16(tm + (kKeySide ? kTmA2 : kTmA1) + cq * 16, pk_ds);
-                        math32<kKeySide, false>(sv[1], tv[1], scale2, row_nlse2, row_D2, 0u, pk_p, pk_ds);
+                        math32<kKeySide, false, kByMma>(sv[1], tv[1], scale2, row_nlse2, row_D2, vec + 256 + cq * 128, 0u, pk_p, pk_ds);
                         if (kKeySide) tmem_st16(tm + kTmA1 + cq * 16 + 32, pk_p);
                         tmem_st16(tm + (kKeySide ? kTmA2 : kTmA1) + cq * 16 + 32, pk_ds);
                     } else {
@@ -445,8 +457,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                                     release_st();
                                     held = false;
                                 }
-                                math32<kKeySide, true>(sv, tv, scale2, row_nlse2, row_D2,
-                                                       bits_below(t.pre - cb) | (bits_below(r_hi - cb) & ~bits_below(r_lo - cb)), pk_p, pk_ds);
+                                math32<kKeySide, true, kByMma>(sv, tv, scale2, row_nlse2, row_D2, vec + 4 * cb,
+                                                               bits_below(t.pre - cb) | (bits_below(r_hi - cb) & ~bits_below(r_lo - cb)), pk_p, pk_ds);
                             }
                             if (!a_free) gradients_done();
                             a_free = true;
@@ -606,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                             mma_ss_lean<1>(tT, rbb + 2, cb + 2, idesc);
                             mma_ss_lean<1>(tT, rbb + 4, cb + 4, idesc);
                             mma_ss_lean<1>(tT, rbb + 6, cb + 6, idesc);
-                            if (key_side) {  // - LSE / scale and - D of the columns: ones x (three bf16 per column)
+                            if (kByMma && key_side) {  // - LSE / scale and - D of the columns: ones x (three bf16 per column)
                                 mma_ss_rows16(tS, ones, smem_desc_lo_rows16(ext, base + kOffZero), idesc);
                                 mma_ss_rows16(tT, ones, smem_desc_lo_rows16(ext + 2048, base + kOffZero), idesc);
                             }
@@ -739,9 +751,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
                         }
                     }
                 } else if (key_side) {  // column data
-                    const uint32_t ext = base + kOffExt + st * 4096 + rr * 16;
-                    cp_async16(ext, p.ext + 2 * (size_t)now);
-                    cp_async16(ext + 2048, p.ext + 2 * (size_t)now + 1);
+                    const uint32_t ext = base + kOffExt + st * 4096;
+                    if (kByMma) {
+                        cp_async16(ext + rr * 16, p.ext + 2 * (size_t)now);
+                        cp_async16(ext + 2048 + rr * 16, p.ext + 2 * (size_t)now + 1);
+                    } else {
+                        cp_async4(ext + rr * 4, p.nlse + now);
+                        cp_async4(ext + 512 + rr * 4, p.D + now);
+                    }
                 }
                 const uint32_t dst = base + (i < 0 ? kOffR + rb * 2 * kTileBytes : kOffC + st * 2 * kTileBytes);
                 const bool kv = (i < 0) == key_side;  // K and V, or Q and dO
@@ -798,16 +815,19 @@ size_t tc_bwd_workspace(const mate_plan_t *plan) {
     const size_t rows = (size_t)plan->B * plan->H * plan->N;
     return 256 + 2 * align256(rows * sizeof(float)) + rows * 32;
 }
-bool tc_bwd_scale(float scale) { return fabsf(scale) >= 0x1p-100f && fabsf(scale) <= 0x1p100f; }
 
 namespace {
-template <bool kMany>
+// Whether -LSE / scale is a number that three bf16 hold: with smaller scales (0 among them) it overflows, with larger ones the lowest
+// of the three comes close to the smallest bf16, 2^-133.  Any other scale takes the kernel that does not divide.
+bool divides(float scale) { return fabsf(scale) >= 0x1p-100f && fabsf(scale) <= 0x1p100f; }
+
+template <bool kMany, bool kByMma>
 int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V, const void *O,
            const float *LSE, const void *dO, float scale, void *const (&dQ)[kPasses], void *const (&dK)[kPasses],
            void *const (&dV)[kPasses], void *workspace, cudaStream_t stream) {
     static SmemAttrOnce attr;
     if (plan->bwd_grid == 0) return MATE_OK;
-    if (attr.ensure((const void *)tc_bwd_kernel<kMany>, (int)kSmemBytes, plan->device) != MATE_OK) return MATE_ERR_CUDA;
+    if (attr.ensure((const void *)tc_bwd_kernel<kMany, kByMma>, (int)kSmemBytes, plan->device) != MATE_OK) return MATE_ERR_CUDA;
     const size_t rows = plan->n_rows();
     uint8_t *ws = (uint8_t *)workspace;
     float *D = (float *)(ws + 256);
@@ -852,7 +872,7 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     if ((rows <= at_once ? rowdot(std::integral_constant<int, 1>{}) : rows <= 2 * at_once ? rowdot(std::integral_constant<int, 2>{})
                                                                                           : rowdot(std::integral_constant<int, 4>{})) != cudaSuccess)
         return MATE_ERR_CUDA;
-    return launch_after(tc_bwd_kernel<kMany>, dim3((unsigned)plan->bwd_grid), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
+    return launch_after(tc_bwd_kernel<kMany, kByMma>, dim3((unsigned)plan->bwd_grid), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MATE_OK : MATE_ERR_CUDA;
 }
 
 }  // namespace
@@ -860,8 +880,12 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
 int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, const void *O,
            const float *LSE, const void *dO, float scale, void *const (&dQ)[kPasses], void *const (&dK)[kPasses],
            void *const (&dV)[kPasses], void *workspace, cudaStream_t stream) {
-    return plan->sub[0] ? launch<true>(plan, Q, K, V, O, LSE, dO, scale, dQ, dK, dV, workspace, stream)
-                        : launch<false>(plan, Q, K, V, O, LSE, dO, scale, dQ, dK, dV, workspace, stream);
+    const auto run = [&](auto many, auto by_mma) {
+        return launch<many(), by_mma()>(plan, Q, K, V, O, LSE, dO, scale, dQ, dK, dV, workspace, stream);
+    };
+    const std::true_type yes;
+    const std::false_type no;
+    return plan->sub[0] ? (divides(scale) ? run(yes, yes) : run(yes, no)) : (divides(scale) ? run(no, yes) : run(no, no));
 }
 
 }  // namespace mate

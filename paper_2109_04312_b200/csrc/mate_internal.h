@@ -298,7 +298,6 @@ int simt_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *
 bool tc_supported(int d, int dtype);
 size_t tc_fwd_workspace(const mate_plan_t *plan, int d);
 size_t tc_bwd_workspace(const mate_plan_t *plan);
-bool tc_bwd_scale(float scale);  // whether the tensor-core backward takes it (it divides by it)
 // (outputs: one set per pass; an ordinary plan has one)
 int tc_bwd(const mate_plan_t *plan, const void *Q, const void *K, const void *V, const void *O,
            const float *LSE, const void *dO, float scale, void *const (&dQ)[kPasses], void *const (&dK)[kPasses],

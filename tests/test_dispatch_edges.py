@@ -73,21 +73,33 @@ def test_row_dots_of_every_size(H):
     _check(rows, cols, 5, [0, 1, 0] * (H // 3) + [1] * (H % 3), 64, "bf16", 12, 1)
 
 
-@pytest.mark.parametrize("scale", [0.0, -0.125, 2.0 ** -101, 2.0 ** -99, 1.5])  # the backward divides by some of them
-def test_backward_takes_every_scale(scale):
+# On both sides of where the tensor-core backward stops dividing by the scale, and the scales in use.  Q and K are scaled by powers of two so
+# that the scores stay what they are, and the gradients are compared by 2-norm, so that those of a tiny scale count as much.
+# Bound: P, dS (or O in D) and the result rounded to bf16, 2^-9 each and independent of one another; row or column: two more, the
+# gradients of the passes and their sum.
+@pytest.mark.parametrize("kind", ["exact", "sat"])
+@pytest.mark.parametrize("scale", [0.0, 2.0 ** -120, 2.0 ** -101, 2.0 ** -99, -2.0 ** -101, -0.125, 1.5, 2.0 ** 99, 2.0 ** 101])
+def test_backward_takes_every_scale(scale, kind):
     import paper_2109_04312_b200 as m
     rows, cols = _structure(20, 300, 30, 4, 13)
-    hv, rng = np.array([0, 1], np.uint8), np.random.default_rng(14)
+    hv, rng = np.array([2, 2] if kind == "sat" else [0, 1], np.uint8), np.random.default_rng(14)
     vals = {n: tables.round_to_bf16((rng.standard_normal((1, 2, 320, 64)) * 0.5).astype(np.float32)) for n in ("Q", "K", "V", "dO")}
-    plan = m.mate_plan(torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda(), 20, hv)
+    e = -3 - int(np.floor(np.log2(abs(scale)))) if scale else 0
+    vals["Q"], vals["K"] = np.ldexp(vals["Q"], e // 2), np.ldexp(vals["K"], e - e // 2)
+    r, c = torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda()
+    plan = m.mate_plan_sat(r, c, 20, 2) if kind == "sat" else m.mate_plan(r, c, 20, hv)
     Q, K, V, dO = (hp.to_dev(vals[n], "bf16") for n in ("Q", "K", "V", "dO"))
     O, LSE = m.mate_attn_fwd(plan, Q, K, V, scale)
-    grads = m.mate_attn_bwd(plan, Q, K, V, O, LSE, dO, scale)
+    auto, forced, simt = (m.mate_attn_bwd(plan, Q, K, V, O, LSE, dO, scale, i) for i in (m.IMPL_AUTO, m.IMPL_TCGEN05, m.IMPL_SIMT))
     plan.status()
     want = oracle.bwd(vals["Q"], vals["K"], vals["V"], vals["dO"], rows, cols, 20, hv, scale)
-    atol, rtol = hp.tol("bf16")
-    for name, g, o in zip(("dQ", "dK", "dV"), grads, want):
-        hp.assert_close(hp.to_np(g), o, atol, rtol, name)
+    bound = (5 if kind == "sat" else 3) ** 0.5 * 2.0 ** -9
+    for name, a, f, s, w in zip(("dQ", "dK", "dV"), auto, forced, simt, want):
+        assert torch.equal(a, f), name
+        for g in (f, s):
+            assert np.linalg.norm(hp.to_np(g) - w) <= bound * np.linalg.norm(w), name
+        # P and dS are rounded on the tensor cores only: the implementation that was asked for has run
+        assert not np.any(w) or not torch.equal(f, s), name
 
 
 @pytest.mark.parametrize("at", [[130], [5, 130]])  # a row of the table; one of the prefix too, which every other row meets

@@ -150,8 +150,8 @@ int mate_plan_varlen(const int32_t *row_ids, const int32_t *col_ids, int B, int 
  * [B + 1], cu_seqlens[0] = 0, non-decreasing, cu_seqlens[B] = T; prefix_len: HOST int32 [B],
  * 0 <= prefix_len[b] <= length of example b.  Negative ids inside an example still mark padding.
  * With such a plan every tensor of mate_attn_fwd / mate_attn_bwd / mate_attn_bwd_noalloc is
- * [H, T, d] (LSE [H, T]) in place of [B, H, N, d] ([B, H, N]); the plan's N (mate_plan_get,
- * mate_attn_workspace_bytes) is the longest example.  The exact pattern only; MATE_FLAG_VIEW_ORDER
+ * [H, T, d] (LSE [H, T]) in place of [B, H, N, d] ([B, H, N]); the plan's N (mate_plan_get)
+ * is the longest example.  The exact pattern only; MATE_FLAG_VIEW_ORDER
  * and mate_cell_mean return MATE_ERR_UNSUPPORTED.  Ownership and errors as for mate_plan. */
 int mate_plan_packed(const int32_t *row_ids, const int32_t *col_ids, int B, const int32_t *cu_seqlens,
                      const int32_t *prefix_len, const uint8_t *head_view, int H, int max_row_id, int max_col_id,

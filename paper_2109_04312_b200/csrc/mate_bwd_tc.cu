@@ -810,9 +810,9 @@ inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 }  // namespace
 
-// workspace: [256 B counters][D: B*H*N floats][-LSE log2 e: as many][the key side's column data: 32 B per row]
+// workspace, by rows of the tensors: [256 B counters][D: a float each][-LSE log2 e: a float][the key side's column data: 32 B]
 size_t tc_bwd_workspace(const mate_plan_t *plan) {
-    const size_t rows = (size_t)plan->B * plan->H * plan->N;
+    const size_t rows = plan->n_rows();
     return 256 + 2 * align256(rows * sizeof(float)) + rows * 32;
 }
 
@@ -831,7 +831,7 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     const size_t rows = plan->n_rows();
     uint8_t *ws = (uint8_t *)workspace;
     float *D = (float *)(ws + 256);
-    const size_t row_floats = align256((size_t)plan->B * plan->H * plan->N * sizeof(float)) / sizeof(float);
+    const size_t row_floats = align256(rows * sizeof(float)) / sizeof(float);
     float *nlse = D + row_floats;
     uint4 *ext = (uint4 *)(nlse + row_floats);
     Params<kMany> p;

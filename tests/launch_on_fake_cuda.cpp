@@ -52,4 +52,11 @@ int call(int backward, int *launches, int *bulk) {
     return rc;
 }
 
+// what the backward of a plan asks for (T: tokens of a packed one, N its longest example)
+size_t backward_workspace(int B, int H, int N, int T) {
+    mate_plan_s plan;
+    plan.B = B, plan.H = H, plan.N = N, plan.T = T;
+    return mate::tc_bwd_workspace(&plan);
+}
+
 }  // extern "C"

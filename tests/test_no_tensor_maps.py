@@ -28,3 +28,11 @@ def test_calls_go_through_without_maps(lib, backward, launches):
     n, bulk = ctypes.c_int(), ctypes.c_int()
     assert lib.call(backward, ctypes.byref(n), ctypes.byref(bulk)) == 0
     assert (n.value, bulk.value) == (launches, 0)
+
+
+@pytest.mark.parametrize("B,H,N,T", [(1, 12, 8192, 0), (4, 12, 2047, 0), (64, 12, 8192, 8192 + 63 * 128), (3, 1, 5, 7)])
+def test_backward_workspace_goes_by_rows_of_the_tensors(lib, B, H, N, T):
+    # 40 bytes a row; one long example among short ones does not make a packed batch as long as so many of them
+    lib.backward_workspace.restype = ctypes.c_size_t
+    rows = H * T if T else B * H * N
+    assert 40 * rows <= lib.backward_workspace(B, H, N, T) <= 40 * rows + 1024

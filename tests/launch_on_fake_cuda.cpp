@@ -6,6 +6,7 @@
 
 namespace {
 int n_launches = 0;
+unsigned first_grid = 0;  // of a call's first launch
 size_t word_at = 0;  // of the last launch's parameters
 int word = -1;
 }  // namespace
@@ -28,8 +29,8 @@ cudaError_t cudaGetDriverEntryPoint(const char *, void **fn, unsigned long long,
     *res = cudaDriverEntryPointSymbolNotFound;
     return cudaErrorInvalidValue;
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *, const void *, void **args) {
-    ++n_launches;
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *config, const void *, void **args) {
+    if (++n_launches == 1) first_grid = config->gridDim.x;
     if (word_at) memcpy(&word, static_cast<const char *>(args[0]) + word_at, sizeof word);
     return cudaSuccess;
 }
@@ -50,6 +51,18 @@ int call(int backward, int *launches, int *bulk) {
     *launches = n_launches;
     *bulk = word;
     return rc;
+}
+
+// blocks of the row dots of H heads of N rows on a GPU of n_ctas SMs
+int rowdot_grid(int H, int N, int n_ctas) {
+    static char mem[256];
+    mate_plan_s plan;
+    plan.B = 1, plan.H = H, plan.N = N;
+    plan.n_ctas = n_ctas;
+    plan.bwd_grid = 1;
+    void *t[mate::kPasses] = {mem, nullptr, nullptr};
+    n_launches = word_at = 0;
+    return mate::tc_bwd(&plan, mem, mem, mem, mem, (float *)mem, mem, 0.125f, t, t, t, mem, nullptr) == 0 ? (int)first_grid : -1;
 }
 
 // what the backward of a plan asks for (T: tokens of a packed one, N its longest example)

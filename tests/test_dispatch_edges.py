@@ -67,7 +67,8 @@ def test_tensor_core_units_that_are_cut_and_a_busy_grid():
     _check(rows, cols, 70, [0, 1] * 26, 64, "bf16", 9)
 
 
-@pytest.mark.parametrize("H", [768, 769, 1536, 1537])  # x 37 positions: around one and two rows per thread on 148 SMs
+# x 37 positions: around one and two rows per thread on 148 SMs, with six and with eight blocks to an SM
+@pytest.mark.parametrize("H", [768, 769, 1024, 1025, 1536, 1537, 2048, 2049])
 def test_row_dots_of_every_size(H):
     rows, cols = _structure(5, 31, 4, 3, 11)
     _check(rows, cols, 5, [0, 1, 0] * (H // 3) + [1] * (H % 3), 64, "bf16", 12, 1)

@@ -30,6 +30,14 @@ def test_calls_go_through_without_maps(lib, backward, launches):
     assert (n.value, bulk.value) == (launches, 0)
 
 
+@pytest.mark.parametrize("n_ctas", [132, 148])
+def test_row_dots_go_in_one_wave_with_as_few_rows_per_thread_as_can_be(lib, n_ctas):
+    # blocks of 32 rows and 8 to an SM, of 64 and 8, of 128 (and 6, from where one wave no longer holds them)
+    one, two = n_ctas * 8 * 32, n_ctas * 8 * 64
+    for rows, per_block in ((1, 32), (n_ctas * 6 * 32 + 1, 32), (one, 32), (one + 1, 64), (n_ctas * 6 * 64 + 1, 64), (two, 64), (two + 1, 128)):
+        assert lib.rowdot_grid(1, rows, n_ctas) == -(-rows // per_block), rows
+
+
 @pytest.mark.parametrize("B,H,N,T", [(1, 12, 8192, 0), (4, 12, 2047, 0), (64, 12, 8192, 8192 + 63 * 128), (3, 1, 5, 7)])
 def test_backward_workspace_goes_by_rows_of_the_tensors(lib, B, H, N, T):
     # 40 bytes a row; one long example among short ones does not make a packed batch as long as so many of them

@@ -103,6 +103,36 @@ def test_backward_takes_every_scale(scale, kind):
         assert not np.any(w) or not torch.equal(f, s), name
 
 
+@pytest.mark.parametrize("q0,v0", [(0.0, 0.0), (8192.0, 0.0), (0.0, 64.0), (8192.0, 64.0)])
+@pytest.mark.parametrize("P,n_table,row_len", [(20, 300, 30), (130, 254, 254)])
+def test_key_side_keeps_the_low_bits_of_lse_and_d(P, n_table, row_len, q0, v0):
+    # A component of its own takes LSE / scale to 8192 (LSE to 1024) or D to 4096 in front of scores and differences dP - D of a few
+    # units.  dK and dV against 64 bits given the same O and LSE: 2.3e-3 to 2.4e-3 of their norm, 1.3e-2 to 2.3e-2 where the last 8 of the
+    # 24 bits of either are left out.  Bound: P (or dS) and the result rounded to bf16, 2^-9 each, and as much for S and dP, whose
+    # last bits are 2^-10 in fp32.
+    import paper_2109_04312_b200 as m
+    rows, cols = _structure(P, n_table, row_len, 4, 16)
+    r, c = torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda()
+    plan, scale, n = m.mate_plan(r, c, P, [0, 1]), 0.125, P + n_table
+    gen = torch.Generator(device="cuda").manual_seed(17)
+    Q, K, V, dO = ((torch.randn(1, 2, n, 64, device="cuda", generator=gen) * 0.5).bfloat16() for _ in range(4))
+    if q0:
+        Q[..., 0], K[..., 0] = q0, 1.0
+    if v0:
+        V[..., 0], dO[..., 0] = v0, v0
+    O, LSE = m.mate_attn_fwd(plan, Q, K, V, scale, m.IMPL_TCGEN05)
+    _, dK, dV = m.mate_attn_bwd(plan, Q, K, V, O, LSE, dO, scale, m.IMPL_TCGEN05)
+    plan.status()
+    ids, pre = torch.stack([r[0], c[0]]), torch.arange(n, device="cuda") < P
+    on = pre[:, None] | pre[None, :] | (ids[:, :, None] == ids[:, None, :])
+    Q, K, V, dO, O = (x[0].double() for x in (Q, K, V, dO, O))
+    p = torch.exp(scale * Q @ K.transpose(1, 2) - LSE[0].double()[..., None]) * on
+    ds = p * (dO @ V.transpose(1, 2) - (dO * O).sum(-1, keepdim=True))
+    for name, g, w in (("dK", dK, scale * ds.transpose(1, 2) @ Q), ("dV", dV, p.transpose(1, 2) @ dO)):
+        g, w = g[0, :, :, 1:].double(), w[:, :, 1:]  # (without the component that is as large as that)
+        assert (g - w).norm() <= 3.0 ** 0.5 * 2.0 ** -9 * w.norm(), (name, float((g - w).norm() / w.norm()))
+
+
 @pytest.mark.parametrize("at", [[130], [5, 130]])  # a row of the table; one of the prefix too, which every other row meets
 @pytest.mark.parametrize("kind", ["exact", "sat"])
 def test_a_query_without_a_finite_score(kind, at):

@@ -162,9 +162,11 @@ __device__ __forceinline__ uint4 split_bf16(float x) {
 // 99.3 -> 98.0 us with four rows per thread instead of two), four rows where two fit 0.6 us at 8 x 512.  The first block also clears the
 // work-item counter of the kernel that follows (and the rest of its 256 bytes).
 // kRows: rows of a group of eight threads, 32 groups to a block.
-constexpr int rowdot_blocks(int n_rows) { return n_rows < 4 ? 8 : 6; }  // of an SM (26, 32 and 40 registers)
+constexpr int kRowdotBlocks = 8;  // of an SM, with one or two rows (26 and 32 registers)
+// (Four rows take 48 registers with all their loads in flight.  With 40, for six blocks to an SM, backward of 4 x 2048 / 2 x 4096 tokens
+// 54.9 / 95.6 us instead of 54.4 / 95.4, with 34 54.7 / 96.7.)
 template <int kRows>
-__global__ void __launch_bounds__(256, rowdot_blocks(kRows)) rowdot_kernel(const __nv_bfloat16 *__restrict__ dO, const __nv_bfloat16 *__restrict__ O,
+__global__ void __launch_bounds__(256, kRows < 4 ? kRowdotBlocks : 1) rowdot_kernel(const __nv_bfloat16 *__restrict__ dO, const __nv_bfloat16 *__restrict__ O,
                                                      const float *__restrict__ LSE, float *__restrict__ D,
                                                      float *__restrict__ nlse, uint4 *__restrict__ ext, float scale,
                                                      size_t rows, int32_t *counter) {
@@ -870,7 +872,7 @@ int launch(const mate_plan_t *plan, const void *Q, const void *K, const void *V,
     };
     // As few rows per thread as bring all blocks onto the GPU at once.  (Twice as many between 28,416 and 37,888 and between 56,832
     // and 75,776 rows, as for six blocks of each kind to an SM: backward of 4 x 680 tokens 19.1 us, 18.4 by this rule, 4 x 1400 32.1, 30.9.)
-    const auto at_once = [&](int n) { return rows <= (size_t)std::max(plan->n_ctas, 1) * rowdot_blocks(n) * 32 * n; };
+    const auto at_once = [&](int n) { return rows <= (size_t)std::max(plan->n_ctas, 1) * kRowdotBlocks * 32 * n; };
     if ((at_once(1) ? rowdot(std::integral_constant<int, 1>{}) : at_once(2) ? rowdot(std::integral_constant<int, 2>{})
                                                                             : rowdot(std::integral_constant<int, 4>{})) != cudaSuccess)
         return MATE_ERR_CUDA;

@@ -192,7 +192,7 @@ int mate_plan_useful_pairs(const mate_plan_t *plan, int64_t *pairs);
 int mate_plan_status(const mate_plan_t *plan, void *stream);
 
 /* Test hook (the paper has no counterpart): launches a one-thread kernel that waits, with the
- * bounded helper the attention kernels use and a limit of a few tries (a few microseconds each), on a
+ * bounded helper the attention kernels use and a limit of a few tries (1.4 microseconds each), on a
  * barrier that nothing arrives on; the wait gives up, the kernel raises the plan's time-out word as
  * the attention kernels would, and returns.  The next mate_plan_status on the plan then reports
  * MATE_ERR_TIMEOUT once, and the plan stays usable.  Lets the time-out path be exercised without

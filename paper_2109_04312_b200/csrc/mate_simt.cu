@@ -15,13 +15,13 @@
 // of a tile need the group to meet.  The first matrix of the next tile travels to registers under the second half of this
 // one, the second under the first half.  A warp leaves out the columns that none of its eight rows counts.
 // With 8 x 512 tokens (16 warps per SM at the registers this takes) the data pipe that serves shared memory is 66 % busy in the
-// forward and 71 % in the backward, issue slots 59 and 56 %, the multiply-add units 36 %; what a warp waits for is shared
-// memory (1.2 and 1.7 cycles per instruction), its turn (1.2, 0.9) and the group (1.0; two hand-overs per tile in the forward, three
-// in the backward), hardly global memory any more (0.3, 0.7).
+// forward and 70 % in the backward, issue slots 59 and 58 %, the multiply-add units 36 and 37 %; what a warp waits for is shared
+// memory (1.2 and 1.8 cycles per instruction), its turn (1.2, 1.0) and the group (1.0; two hand-overs per tile in the forward, three
+// in the backward), hardly global memory (0.3).
 // Two blocks per SM (one with heads of more than 64): three of smaller heads fit, but spill (2 x 512 tokens, heads of 32, 16.2 / 31.9 us
 // with two, 19.8 / 41.4 with three; of 16 12.5 / 24.2, 13.3 / 25.9).
-// 2 x 512 tokens, 12 heads of 64, forward / backward: 24.4 / 53.1 us; with the rows' key ranges in registers
-// (24 of them spilled in the backward) 25.2 / 54.7; with the rows' look-ups directly in front of the loads
+// 2 x 512 tokens, 12 heads of 64, forward / backward: 23.7 / 50.0 us, 23.7 / 52.5 with P of the backward in registers.  The forms before, as
+// timed then: 24.4 / 53.1; with the rows' key ranges in registers 25.2 / 54.7; with the rows' look-ups directly in front of the loads
 // that need them 29.4 / 62.8 (a warp waited 2.2 times as long for global memory as it issued); with 2 x 4 scores per thread,
 // one group and every column of a tile 37.4 / 70.8; with one warp per row and global reads of every key 463 / 1540.
 #include <cuda_bf16.h>
@@ -82,8 +82,9 @@ struct Common {
 __device__ __forceinline__ int first_row() { return (int)((threadIdx.x % kGroup) >> 4) * kMine; }
 __device__ __forceinline__ void group_sync() { asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / kGroup), "n"(kGroup) : "memory"); }
 
-// The rows of a block and the column tiles they meet.  What is needed once a tile stays in shared memory (registers
-// are what the backward is short of: of 128 with heads of 64, 24 spilled with the ranges in them, 14 without).
+// The rows of a block and the column tiles they meet.  What is needed once a tile stays in shared memory: registers are what the
+// kernels are short of (128 with heads of 64, bytes spilled and read back: forward 8 / 8 with fp32 tensors and 20 / 16 with bf16,
+// backward 4 / 4 with either).
 struct RowBlock {
     struct Shared {
         int P, b_lo, b_hi, lo[kRows], hi[kRows];  // lo, hi: behind the global block
@@ -442,9 +443,9 @@ __global__ void __launch_bounds__(kThreads, DP <= 64 ? 2 : 1) simt_bwd_kernel(co
     __shared__ int s_col[2][kCols], s_own[kRows];  // original rows of each group's tile, of the block
     __shared__ float s_row[2][kRows];                          // LSE, D of the block's rows (query side)
     constexpr int kR = kRows * (DP + 4), kC = kCols * (DP + 4), kPart = 2 * kC + kRows * kPStride + 2 * kCols;
-    // P waits in shared memory for dP where it would not fit into the registers: with heads of 64, 24 to 44 of which were spilled, 2 x
-    // 512 / 8 x 512 tokens 52.5 / 195 us with P in registers, 50.0 / 187 with it in shared memory; heads of 16, 32 and 128, which do
-    // not spill, 22.4, 30.6 and 90.6 us and 23.5, 31.3 and 91.2.
+    // P waits in shared memory for dP where it would not fit into the registers: with heads of 64 and P in registers 144 / 104 bytes are
+    // spilled and read back (bf16 tensors 176 / 96) instead of 4 / 4, and 2 x 512 / 8 x 512 tokens take 52.5 / 195 us instead of 50.0 / 186;
+    // heads of 16, 32 and 128, which do not spill, 22.4, 30.6 and 90.6 us with P in registers and 23.5, 31.3 and 91.2 in shared memory.
     constexpr bool kPShared = DP == 64;
     const int grp = threadIdx.x / kGroup, tid = threadIdx.x % kGroup;
     float *sRa = smem, *sRb = sRa + kR, *part = sRb + kR, *sCa = part + grp * kPart, *sCb = sCa + kC, *sX = sCb + kC,

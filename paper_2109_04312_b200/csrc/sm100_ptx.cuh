@@ -60,8 +60,8 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const void *tmap,
 }
 
 // Brings a tensor map of the kernel's parameters, where there is one, to where the copies look for it (about 0.5 us on first
-// use).  (A branch around it changes how the compiler deals out the registers of the whole backward: 80 bytes of spills read
-// back instead of 16, 1 x 8192 tokens 112.4 us instead of 104.2.)
+// use).  (A branch around it changed how the compiler dealt out the registers of the whole backward, when that still spilled: 80
+// bytes read back instead of 16, 1 x 8192 tokens 112.4 us instead of 104.2.)
 __device__ __forceinline__ void prefetch_tmap(const void *tmap, int there_is_one) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t@p prefetch.tensormap [%0];\n\t}" ::"l"(tmap), "r"(there_is_one)
                  : "memory");

@@ -1,5 +1,5 @@
 // The host side of the tensor-core kernels (csrc/mate_fwd_tc.cu, csrc/mate_bwd_tc.cu) on a CUDA runtime of plain host functions:
-// a driver without tensor maps, launches that are only counted.
+// a driver without tensor maps, launches that are only counted and looked at.
 #include <cstring>
 
 #include "mate_internal.h"

@@ -1,5 +1,6 @@
-"""A driver that hands out no tensor maps is no reason to refuse a call: the tensor-core kernels then gather every tile row by
-row.  Their host side on a CUDA runtime of host functions (tests/launch_on_fake_cuda.cpp).  No GPU."""
+"""The host side of the tensor-core kernels on a CUDA runtime of host functions (tests/launch_on_fake_cuda.cpp): a driver that hands
+out no tensor maps is no reason to refuse a call (every tile is then gathered row by row); the row dots' grid; the backward's
+workspace.  No GPU."""
 import ctypes
 import os
 import shutil
@@ -32,7 +33,7 @@ def test_calls_go_through_without_maps(lib, backward, launches):
 
 @pytest.mark.parametrize("n_ctas", [132, 148])
 def test_row_dots_go_in_one_wave_with_as_few_rows_per_thread_as_can_be(lib, n_ctas):
-    # blocks of 32 rows and 8 to an SM, of 64 and 8, of 128 (and 6, from where one wave no longer holds them)
+    # blocks of 32 or 64 rows where eight of them to an SM are enough, of 128 for more
     one, two = n_ctas * 8 * 32, n_ctas * 8 * 64
     for rows, per_block in ((1, 32), (n_ctas * 6 * 32 + 1, 32), (one, 32), (one + 1, 64), (n_ctas * 6 * 64 + 1, 64), (two, 64), (two + 1, 128)):
         assert lib.rowdot_grid(1, rows, n_ctas) == -(-rows // per_block), rows

@@ -84,8 +84,13 @@ constexpr int kLoadWarps = 4;
 static_assert(kTile == 32 * kLoadWarps, "a row of a tile per loader thread");
 constexpr int kThreads = 32 * (kLoadWarp0 + kLoadWarps);
 // registers per thread after the roles have split: 256 x 160 + 128 x 56 + 128 x 40 + 128 x 64 = 61,440 = the 640 x 96 the
-// CTA is launched with
-constexpr int kRegsCompute = 160, kRegsStore = 56, kRegsMma = 40, kRegsLoad = 64;
+// CTA is launched with; 256 x 168 + 128 x 48 + 128 x 40 + 128 x 56, as many, where the arithmetic warps read the columns' data
+// (!kByMma, which spills 36 bytes and reads back 80 so, 72 and 176 with the other split: 1 x 8192 tokens 108.2 instead of 116.4 us)
+template <bool kByMma>
+struct Regs {
+    static constexpr int kCompute = kByMma ? 160 : 168, kStore = kByMma ? 56 : 48, kMma = 40, kLoad = kByMma ? 64 : 56;
+    static_assert(2 * kCompute + kStore + kMma + kLoad == 480, "what the CTA is launched with");
+};
 constexpr int kStages = 4;  // ring of column tiles
 using RowRing = LoadRing<2>;
 using ColRing = LoadRing<kStages>;
@@ -361,7 +366,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
     };
     if (warp < kComputeWarps) {
         // ------------------------------------------------------------------ arithmetic + epilogue
-        reg_alloc<kRegsCompute>();
+        reg_alloc<Regs<kByMma>::kCompute>();
         const int r = tid & 127;   // row of the tile = lane of tensor memory
         const int cq = warp >> 2;  // takes the chunks cq and cq + 2 of a column tile
         const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
@@ -497,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         }
     } else if (warp < kMmaWarp) {
         // ------------------------------------------------------------------ gradients: tensor memory -> original positions
-        reg_dealloc<kRegsStore>();
+        reg_dealloc<Regs<kByMma>::kStore>();
         const int q4 = warp - kStoreWarp0;  // rows 32 q4 .. of the tile = lanes of tensor memory this warp can read
         static_assert(kStoreWarp0 % 4 == 0, "warp w reads the lanes 32 (w % 4) ..");
         const uint32_t acc = tmem + ((uint32_t)(q4 * 32) << 16) + kTmAcc1;
@@ -568,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         // One warp issues S and dP of the tiles, the other the gradient MMAs, each as soon as what it needs is there.  The
         // whole warp runs the control flow and one lane issues; votes and shuffles keep conditions and operands
         // warp-uniform (an MMA with other operands takes 51 clk to issue, more than a gradient MMA takes to run).
-        reg_dealloc<kRegsMma>();
+        reg_dealloc<Regs<kByMma>::kMma>();
         if (warp < kMmaWarp + kMmaWarps) {
             const bool leader = elect_one();
             const bool grad = warp != kMmaWarp;
@@ -697,7 +702,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_bwd_kernel(const __grid_consta
         }
     } else {
         // ------------------------------------------------------------------ loaders
-        reg_dealloc<kRegsLoad>();
+        reg_dealloc<Regs<kByMma>::kLoad>();
         wait_prior_grid();
         const int lw = warp - kLoadWarp0;
         const bool leader = elect_one();
